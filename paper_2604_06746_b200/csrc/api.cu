@@ -1,5 +1,6 @@
 // C ABI of libstructkv: argument validation, context and workspace bookkeeping, dispatch to
 // the kernels, and the host-side pivot rule (Eq. 7-9).
+#include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -28,7 +29,7 @@ static bool config_supported(const structkv_config& cfg) {
 }
 
 static int rows_pad_of(const structkv_config& cfg) {
-  const int rows_pg = (cfg.n_q_heads / cfg.n_kv_heads) * cfg.window;
+  const int rows_pg = (cfg.n_q_heads / cfg.n_kv_heads) * tc_window_pad(cfg.window);
   return cfg.n_kv_heads * (int)align_up((size_t)rows_pg, kRowBlock);
 }
 
@@ -44,15 +45,19 @@ Workspace carve_workspace(const structkv_config& cfg, void* base) {
   const size_t rows_pad = (size_t)rows_pad_of(cfg);
   const size_t n_pad = align_up((size_t)cfg.max_seq, kKeyTile);
   w.status = (int*)take(256);
-  w.row_part = (float4*)take((size_t)kMaxParts * rows_pad * sizeof(float4));
+  w.ctl = (int*)take(kCtlInts * sizeof(int));                  // follows the status block: one memset
+  w.row_part = (float4*)take(std::max((size_t)kSimtParts * rows_pad * sizeof(float4),
+                                      tc_part_tasks(cfg, 1, false) * kRowBlock * sizeof(float2)));
   w.row_lse2 = (float*)take(rows_pad * sizeof(float));
   w.row_ent = (float*)take(rows_pad * sizeof(float));
   w.cols = (float*)take((size_t)cfg.n_q_heads * n_pad * sizeof(float));
   w.head_part = (float*)take((size_t)kMaxStatLayers * cfg.n_q_heads * 4 * sizeof(float));
-  w.queue = (unsigned long long*)take((size_t)kMaxBatch * kQueueUnits * sizeof(unsigned long long));
   w.bytes = off;
   return w;
 }
+
+// the status block and the control block behind it start from zero
+constexpr size_t kZeroBytes = 256 + kCtlInts * sizeof(int);
 
 }  // namespace skv
 
@@ -94,13 +99,13 @@ structkv_status structkv_create(structkv_ctx** ctx_out, const structkv_config* c
   c.cfg = *cfg;
   c.ws = carve_workspace(*cfg, workspace_dev);
   c.rows = cfg->n_q_heads * cfg->window;
+  c.w_pad = tc_window_pad(cfg->window);
   c.rows_pad = rows_pad_of(*cfg);
   c.n_pad = (int)align_up((size_t)cfg->max_seq, kKeyTile);
   c.tc = nullptr;
   if (cudaGetDevice(&c.device) != cudaSuccess ||
       cudaDeviceGetAttribute(&c.sm_count, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess ||
-      cudaMemset(c.ws.status, 0, 256) != cudaSuccess ||
-      cudaMemset(c.ws.queue, 0, (size_t)kMaxBatch * kQueueUnits * sizeof(unsigned long long)) != cudaSuccess ||
+      cudaMemset(c.ws.status, 0, kZeroBytes) != cudaSuccess ||
       cudaDeviceSynchronize() != cudaSuccess) {
     delete ctx;
     return STRUCTKV_ERR_CUDA;
@@ -140,35 +145,26 @@ structkv_status structkv_score_layer(structkv_ctx* ctx, const void* q_window, co
     return STRUCTKV_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
 
-  ScoreArgs a;
-  a.q = q_window; a.k = k;
-  a.k_stride_head = k_stride_head; a.k_stride_token = k_stride_token;
-  a.n_keys = n_keys; a.scale = scale;
-  a.batch = 1; a.total_keys = n_keys; a.cu_seqlens = nullptr;
-  a.inputs_ready = (flags & STRUCTKV_FLAG_INPUTS_READY) != 0;
-  a.cols = head_cols_out ? head_cols_out : c.ws.cols;
-  a.col_stride = head_cols_out ? (long long)n_keys : (long long)c.n_pad;
-
-  const bool use_tc = cfg.dtype == STRUCTKV_BF16 && !(flags & STRUCTKV_FLAG_FORCE_SIMT) &&
-                      tc_supported(c, a);
-  int parts = 0;
-  cudaError_t e;
-  e = use_tc ? launch_score_tc(c, a, &parts, 1, st) : launch_score_simt(c, a, &parts, 1, st);
-  if (e != cudaSuccess) return STRUCTKV_ERR_CUDA;
-  if (!use_tc) {
-    e = launch_finalize_rows(c, parts, st);
-    if (e != cudaSuccess) return STRUCTKV_ERR_CUDA;
+  float* cols = head_cols_out ? head_cols_out : c.ws.cols;
+  const long long col_stride = head_cols_out ? (long long)n_keys : (long long)c.n_pad;
+  if (cfg.dtype == STRUCTKV_BF16 && !(flags & STRUCTKV_FLAG_FORCE_SIMT) && tc_supported(c, k_stride_head, k_stride_token)) {
+    const TcCall a{1, &q_window, &k, &scale, nullptr, k_stride_head, k_stride_token, n_keys, cols, 0, col_stride,
+                   (float2*)c.ws.row_part, c.ws.row_lse2, c.ws.row_ent};
+    if (launch_score_tc(c, a, st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
+  } else {
+    const ScoreArgs a{q_window, k, k_stride_head, k_stride_token, n_keys, scale, cols, col_stride};
+    int parts = 0;
+    if (launch_score_simt(c, a, &parts, 1, st) != cudaSuccess || launch_finalize_rows(c, parts, st) != cudaSuccess ||
+        launch_score_simt(c, a, &parts, 2, st) != cudaSuccess)
+      return STRUCTKV_ERR_CUDA;
   }
-  e = use_tc ? launch_score_tc(c, a, &parts, 2, st) : launch_score_simt(c, a, &parts, 2, st);
-  if (e != cudaSuccess) return STRUCTKV_ERR_CUDA;
-  e = launch_reduce_finish(c, a.cols, a.col_stride, n_keys, lambda, s_out, c_inout,
-                           !(flags & STRUCTKV_FLAG_NO_HEAD_STATS), metrics_out, st);
-  return e == cudaSuccess ? STRUCTKV_OK : STRUCTKV_ERR_CUDA;
+  return launch_reduce_finish(c, cols, col_stride, n_keys, lambda, s_out, c_inout, !(flags & STRUCTKV_FLAG_NO_HEAD_STATS),
+                              metrics_out, st) == cudaSuccess ? STRUCTKV_OK : STRUCTKV_ERR_CUDA;
 }
 
 // ---- batches of prompts of different lengths (packed along the token axis) ------------------
 namespace skv {
-struct BatchWs { float4* row_part; float* row_ent; float* cols; float* head_part; size_t bytes; };
+struct BatchWs { float2* row_part; float* nlse; float* row_ent; float* cols; float* head_part; size_t bytes; };
 static BatchWs carve_batch(const structkv_config& cfg, int max_batch, long long max_total, void* base) {
   BatchWs w{};
   char* p = (char*)base;
@@ -180,7 +176,8 @@ static BatchWs carve_batch(const structkv_config& cfg, int max_batch, long long 
   };
   const size_t rows_all = (size_t)max_batch * rows_pad_of(cfg);
   const size_t t_pad = align_up((size_t)max_total, kKeyTile);
-  w.row_part = (float4*)take((size_t)kMaxParts * rows_all * sizeof(float4));
+  w.row_part = (float2*)take(tc_part_tasks(cfg, max_batch, true) * kRowBlock * sizeof(float2));
+  w.nlse = (float*)take(rows_all * sizeof(float));
   w.row_ent = (float*)take(rows_all * sizeof(float));
   w.cols = (float*)take((size_t)cfg.n_q_heads * t_pad * sizeof(float));
   w.head_part = (float*)take((size_t)max_batch * cfg.n_q_heads * 4 * sizeof(float));
@@ -223,33 +220,20 @@ structkv_status structkv_score_layer_batch(structkv_ctx* ctx, const void* q_wind
   cudaStream_t st = (cudaStream_t)stream;
   const BatchWs bw = carve_batch(cfg, batch, total, batch_workspace);
 
-  Ctx view = c;                       // same device, tensor-map encoder and status word; batch-sized scratch
-  view.ws.row_part = bw.row_part;
-  view.ws.row_ent = bw.row_ent;
-  view.ws.cols = bw.cols;
-  view.ws.head_part = bw.head_part;
-  // the ticket counters stay the context's own (its workspace is known to be initialised)
-  ScoreArgs a;
-  a.q = q_window; a.k = k;
-  a.k_stride_head = k_stride_head; a.k_stride_token = k_stride_token;
-  a.n_keys = 0; a.batch = batch; a.total_keys = total; a.cu_seqlens = cu_seqlens;
-  a.scale = scale;
-  a.inputs_ready = (flags & STRUCTKV_FLAG_INPUTS_READY) != 0;
-  a.cols = head_cols_out ? head_cols_out : bw.cols;
-  a.col_stride = head_cols_out ? (long long)total : (long long)align_up((size_t)total, kKeyTile);
   // only the tensor-core scorer handles packed batches
-  if (cfg.dtype != STRUCTKV_BF16 || !tc_supported(view, a)) return STRUCTKV_ERR_UNSUPPORTED;
-  int parts = 0;
-  if (launch_score_tc(view, a, &parts, 1, st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
-  if (launch_score_tc(view, a, &parts, 2, st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
-  std::memcpy(c.queue_period, view.queue_period, sizeof(c.queue_period));   // the launches updated the view's copy
+  if (cfg.dtype != STRUCTKV_BF16 || !tc_supported(c, k_stride_head, k_stride_token)) return STRUCTKV_ERR_UNSUPPORTED;
+  float* cols = head_cols_out ? head_cols_out : bw.cols;
+  const long long col_stride = head_cols_out ? (long long)total : (long long)align_up((size_t)total, kKeyTile);
+  const TcCall a{batch, &q_window, &k, &scale, cu_seqlens, k_stride_head, k_stride_token, 0, cols, 0, col_stride,
+                 bw.row_part, bw.nlse, bw.row_ent};
+  if (launch_score_tc(c, a, st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
   // per sequence: S = sum over heads, C <- lambda C + S, and the sequence's metric triple
   for (int b = 0; b < batch; ++b) {
     const int key0 = cu_seqlens[b], n_b = cu_seqlens[b + 1] - key0;
-    Ctx one = view;
+    Ctx one = c;
     one.ws.row_ent = bw.row_ent + (size_t)b * c.rows_pad;
     one.ws.head_part = bw.head_part + (size_t)b * cfg.n_q_heads * 4;
-    if (launch_reduce_finish(one, a.cols + key0, a.col_stride, n_b, lambda, s_out + key0,
+    if (launch_reduce_finish(one, cols + key0, col_stride, n_b, lambda, s_out + key0,
                              c_inout ? c_inout + key0 : nullptr, !(flags & STRUCTKV_FLAG_NO_HEAD_STATS),
                              metrics_out + 3 * b, st) != cudaSuccess)
       return STRUCTKV_ERR_CUDA;
@@ -259,7 +243,7 @@ structkv_status structkv_score_layer_batch(structkv_ctx* ctx, const void* q_wind
 
 // ---- several resident layers in one call, the passes of neighbouring layers interleaved ---------
 namespace skv {
-struct LayersWs { float4* row_part[2]; float* row_ent; unsigned int* done; unsigned long long* queue; size_t bytes; };
+struct LayersWs { float2* row_part; float* nlse; float* row_ent; size_t bytes; };
 static LayersWs carve_layers(const structkv_config& cfg, int max_layers, void* base) {
   LayersWs w{};
   char* p = (char*)base;
@@ -270,9 +254,8 @@ static LayersWs carve_layers(const structkv_config& cfg, int max_layers, void* b
     return r;
   };
   const size_t rows_pad = (size_t)rows_pad_of(cfg);
-  w.done = (unsigned int*)take(256);
-  w.queue = (unsigned long long*)take((size_t)max_layers * kQueueUnits * sizeof(unsigned long long));   // follows `done`: one memset
-  for (int i = 0; i < 2; ++i) w.row_part[i] = (float4*)take((size_t)kMaxParts * rows_pad * sizeof(float4));
+  w.row_part = (float2*)take(tc_part_tasks(cfg, max_layers, false) * kRowBlock * sizeof(float2));
+  w.nlse = (float*)take((size_t)std::min(max_layers, kMaxBatch) * rows_pad * sizeof(float));
   w.row_ent = (float*)take((size_t)max_layers * rows_pad * sizeof(float));
   w.bytes = off;
   return w;
@@ -311,18 +294,7 @@ structkv_status structkv_score_layers(structkv_ctx* ctx, int n_layers, const voi
       return STRUCTKV_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
 
-  auto args_of = [&](int l) {
-    ScoreArgs a;
-    a.q = q_windows[l]; a.k = ks[l];
-    a.k_stride_head = k_stride_head; a.k_stride_token = k_stride_token;
-    a.n_keys = n_keys; a.scale = scales[l];
-    a.batch = 1; a.total_keys = n_keys; a.cu_seqlens = nullptr;
-    a.cols = head_cols_out + (size_t)l * head_cols_layer_stride;
-    a.col_stride = n_keys;
-    return a;
-  };
-  ScoreArgs probe = args_of(0);
-  if (cfg.dtype != STRUCTKV_BF16 || !tc_supported(c, probe)) {
+  if (cfg.dtype != STRUCTKV_BF16 || !tc_supported(c, k_stride_head, k_stride_token)) {
     // the CUDA-core scorer has no interleaved form: one layer after the other, same results
     for (int l = 0; l < n_layers; ++l) {
       const structkv_status s = structkv_score_layer(
@@ -337,32 +309,9 @@ structkv_status structkv_score_layers(structkv_ctx* ctx, int n_layers, const voi
   if (!layers_workspace || layers_workspace_bytes < need || ((uintptr_t)layers_workspace % 256) != 0)
     return STRUCTKV_ERR_WORKSPACE;
   const LayersWs lw = carve_layers(cfg, n_layers, layers_workspace);
-  // completion counters and every layer's own ticket counters start from zero
-  if (cudaMemsetAsync(lw.done, 0, 256 + (size_t)n_layers * kQueueUnits * sizeof(unsigned long long), st) != cudaSuccess)
-    return STRUCTKV_ERR_CUDA;
-
-  // Stream order: P1(0), then for every layer l: P1(l + 1), P2(l).  P2(l) waits for the completion
-  // counter of P1(l), which finished while P1(l + 1) ran, instead of for the whole kernel before it;
-  // P1(l + 2) overwrites the row statistics P2(l) reads only after P2(l), the kernel before it in
-  // the stream, has completed.  Two statistics buffers and two counters alternate.
-  Ctx view = c;
-  auto launch = [&](int l, int pass) {
-    view.ws.row_part = lw.row_part[l & 1];
-    view.ws.row_ent = lw.row_ent + (size_t)l * c.rows_pad;
-    ScoreArgs a = args_of(l);
-    a.inputs_ready = true;
-    a.done = lw.done + (l & 1);
-    a.done_round = l / 2 + 1;
-    a.queue = lw.queue + (size_t)l * kQueueUnits;
-    int parts = 0;
-    return launch_score_tc(view, a, &parts, pass, st) == cudaSuccess;
-  };
-  bool ok = launch(0, 1);
-  for (int l = 0; ok && l < n_layers; ++l) {
-    if (l + 1 < n_layers) ok = launch(l + 1, 1);
-    ok = ok && launch(l, 2);
-  }
-  if (!ok) return STRUCTKV_ERR_CUDA;
+  const TcCall a{n_layers, q_windows, ks, scales, nullptr, k_stride_head, k_stride_token, n_keys, head_cols_out,
+                 head_cols_layer_stride, n_keys, lw.row_part, lw.nlse, lw.row_ent};
+  if (launch_score_tc(c, a, st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
   return launch_reduce_layers(c, head_cols_out, head_cols_layer_stride, n_keys, n_keys, n_layers, lambda, s_out,
                               s_layer_stride, c_inout, lw.row_ent, metrics_out, st) == cudaSuccess
              ? STRUCTKV_OK
@@ -554,13 +503,9 @@ structkv_status structkv_poll_device_status(structkv_ctx* ctx, void* stream) {
       cudaStreamSynchronize(st) != cudaSuccess)
     return STRUCTKV_ERR_CUDA;
   if (word != 0) {
-    // a scorer launch that gave up may have left its ticket counters short of what the host
-    // expects: start them over together with the status word
-    if (cudaMemsetAsync(ctx->c.ws.status, 0, sizeof(int), st) != cudaSuccess ||
-        cudaMemsetAsync(ctx->c.ws.queue, 0, (size_t)kMaxBatch * kQueueUnits * sizeof(unsigned long long), st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
+    // a scorer launch that gave up may have left its counters behind: start them over as well
+    if (cudaMemsetAsync(ctx->c.ws.status, 0, kZeroBytes, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
       return STRUCTKV_ERR_CUDA;
-    std::memset(ctx->c.queue_period, 0, sizeof(ctx->c.queue_period));
   }
   if (word < 0 || word > (int)STRUCTKV_ERR_TIMEOUT) return STRUCTKV_ERR_CUDA;
   return (structkv_status)word;
@@ -632,15 +577,12 @@ extern "C" structkv_status structkv_score_layer_static(
   c.device = dev;
   c.sm_count = slot->sm_count;
   c.rows = cfg->n_q_heads * cfg->window;
+  c.w_pad = tc_window_pad(cfg->window);
   c.rows_pad = rows_pad_of(*cfg);
   c.n_pad = (int)align_up((size_t)cfg->max_seq, kKeyTile);
   c.tc = cfg->dtype == STRUCTKV_BF16 ? slot->tc : nullptr;
-  // The scratch keeps the previous call's contents; the status word must start from zero.
-  if (cudaMemsetAsync(c.ws.status, 0, 256, (cudaStream_t)stream) != cudaSuccess) return STRUCTKV_ERR_CUDA;
-  // the per-call context starts its ticket counters from zero as well
-  if (cudaMemsetAsync(c.ws.queue, 0, (size_t)kMaxBatch * kQueueUnits * sizeof(unsigned long long), (cudaStream_t)stream) !=
-      cudaSuccess)
-    return STRUCTKV_ERR_CUDA;
+  // The scratch keeps the previous call's contents; the status word and the scorer's counters start from zero.
+  if (cudaMemsetAsync(c.ws.status, 0, kZeroBytes, (cudaStream_t)stream) != cudaSuccess) return STRUCTKV_ERR_CUDA;
   return structkv_score_layer(&tmp, q_window, k, k_stride_head, k_stride_token, n_keys, scale, lambda,
                               s_out, c_inout, head_cols_out, metrics_out, flags, stream);
 }

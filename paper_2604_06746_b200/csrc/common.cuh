@@ -10,30 +10,27 @@
 namespace skv {
 
 constexpr int kKeyTile = 128;        // keys per tile in every scorer
-constexpr int kMaxParts = 160;       // upper bound on key segments per score row
+constexpr int kMaxSms = 160;          // SMs a scorer launch uses at most (bounds its pass-1 tasks)
+constexpr int kSimtParts = 64;        // key segments per score row of the CUDA-core scorer
 constexpr int kRowBlock = 256;       // score rows (head, window row) per tensor-core row block
 constexpr int kMaxBatch = 32;        // sequences one batched scoring call may hold
 constexpr int kMaxStatLayers = 128;   // layers one batched head-statistics call may cover
 constexpr int kMaxGatherLayers = 128; // layers one multi-layer gather may cover (their pointers are a kernel argument)
-constexpr int kQueueUnits = 256;      // (KV group, row block) units of one sequence the scorer's work queue can hold
+constexpr int kQueueUnits = 256;      // (KV group, row block) units of one problem the tensor-core scorer can hold
+constexpr int kCtlInts = 64 + 2 * kMaxBatch * kQueueUnits;   // its control block: tickets, arrivals, ready flags
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
 // Device status word values are structkv_status codes; 0 = nothing recorded.
 struct Workspace {
   int* status;          // [64] ints, word 0 is the status
-  float4* row_part;     // [kMaxParts][rows_pad] (m2, Z, U, unused) partial softmax statistics
-  float* row_lse2;      // [rows_pad] log2-domain log-sum-exp of each score row
-  float* row_ent;       // [rows_pad] entropy of each score row (nats)
+  int* ctl;             // [kCtlInts], follows the status block; zero between scorer launches (a launch leaves it zero)
+  float4* row_part;     // partial softmax statistics: CUDA cores [kSimtParts][rows_pad] (m2, Z, U, -), tensor cores
+                        // float2 [pass-1 task][kRowBlock]
+  float* row_lse2;      // [rows_pad] log2-domain log-sum-exp of each score row (tensor cores: negated)
+  float* row_ent;       // [rows_pad] entropy of each score row (nats), 0 where there is no row
   float* cols;          // [H][n_pad] pooled per-head attention when the caller passes none
   float* head_part;     // [kMaxStatLayers][H][4] per-(layer, head) {sum of squared deviations from 1/n, top-k mass}
-  // [kMaxBatch][kQueueUnits] ticket counters of the tensor-core scorer's second pass, one per
-  // (sequence slot of a call, KV group, row block); zero when the context is created.  A launch
-  // draws exactly T = tiles + CTAs-of-the-unit tickets from a unit's counter and reads a ticket
-  // modulo T, so launches of one shape follow each other with no reset and no per-launch host
-  // state (a captured launch can be replayed); the host zeroes a slot only when its T changes
-  // (queue_period in Ctx)
-  unsigned long long* queue;
   size_t bytes;
 };
 
@@ -43,12 +40,10 @@ struct Ctx {
   int device;
   int sm_count;
   int rows;             // H * w
-  int rows_pad;         // rows per KV group padded to kRowBlock, times H_kv
+  int w_pad;            // rows a head occupies in the tensor-core scorer's blocks: w up to a power of two, at least 8
+  int rows_pad;         // rows per KV group (heads at w_pad rows) padded to kRowBlock, times H_kv
   int n_pad;            // max_seq rounded up to kKeyTile
-  void* tc;             // tensor-core scorer state (tensor maps), owned by score_tc.cu
-  // tickets per launch (T) the counters of a sequence slot were last used with: [0] for the units
-  // on full row blocks, [1] for the units on a KV group's last row block; 0 = counters are zero
-  unsigned int queue_period[kMaxBatch][2] = {};
+  void* tc;             // tensor-core scorer state (tensor-map encoder), owned by score_tc.cu
 };
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -61,18 +56,8 @@ struct ScoreArgs {
   const void* q;            // [H, w, d]
   const void* k;
   long long k_stride_head, k_stride_token;   // elements
-  int n_keys;               // keys of the sequence (a plain call), unused for a batch
-  int batch;                // sequences in the call (1 for a plain call)
-  int total_keys;           // rows of K along the token axis: n_keys, or cu_seqlens[batch]
-  const int* cu_seqlens;    // host, [batch + 1] first key of every sequence in the packed K; NULL = plain call
+  int n_keys;
   float scale;
-  bool inputs_ready = false; // q and k are complete and visible: nothing in flight on the stream writes them
-  // completion counter of pass 1 (device, or NULL) and how many pass-1 launches, this one included,
-  // have used it since it was zeroed: pass 2 of the same layer waits for done_round * grid
-  unsigned int* done = nullptr;
-  int done_round = 0;
-  // ticket counters for this launch alone ([kQueueUnits], zero), or NULL for the context's shared ones
-  unsigned long long* queue = nullptr;
   float* cols;              // [H][col_stride] pooled per-head attention (output of pass 2)
   long long col_stride;
 };
@@ -81,18 +66,35 @@ struct ScoreArgs {
 cudaError_t launch_score_simt(const Ctx& ctx, const ScoreArgs& a, int* parts_out, int pass,
                               cudaStream_t st);
 
-// Tensor-core (tcgen05) two-pass scorer for bf16 storage.
-bool tc_supported(const Ctx& ctx, const ScoreArgs& a);
+// Tensor-core (tcgen05) scorer for bf16 storage: both passes over `n` problems (layers of one shape, or
+// the sequences of a packed batch), one launch per kMaxBatch layers.
+struct TcCall {
+  int n;                          // layers, or sequences
+  const void* const* q;           // layers: [n]; batch: one tensor [n, H, w, d]
+  const void* const* k;           // layers: [n]; batch: one packed tensor
+  const float* scale;             // layers: [n]; batch: one
+  const int* cu_seqlens;          // batch: host, [n + 1]; NULL for layers
+  long long k_stride_head, k_stride_token;   // elements
+  int n_keys;                     // keys of a layer
+  float* cols;                    // layer l at cols + l * cols_layer_stride; sequence b at column cu_seqlens[b]
+  long long cols_layer_stride, col_stride;
+  float2* part;                   // tc_part_tasks(...) * kRowBlock entries
+  float* nlse;                    // [min(n, kMaxBatch)][rows_pad]
+  float* row_ent;                 // [n][rows_pad]
+};
+bool tc_supported(const Ctx& ctx, long long k_stride_head, long long k_stride_token);
+int tc_window_pad(int window);
+// pass-1 tasks (partial statistics of kRowBlock rows) a launch over n problems needs room for
+size_t tc_part_tasks(const structkv_config& cfg, int n, bool batch);
 structkv_status tc_create(Ctx& ctx);
 void tc_destroy(Ctx& ctx);
-cudaError_t launch_score_tc(Ctx& ctx, const ScoreArgs& a, int* parts_out, int pass, cudaStream_t st);
+cudaError_t launch_score_tc(const Ctx& ctx, const TcCall& a, cudaStream_t st);
 
 // One thread waits (bounded by limit_cycles) on a barrier nobody arrives on, then records
 // STRUCTKV_ERR_TIMEOUT in *status.
 cudaError_t launch_wait_probe(unsigned long long limit_cycles, int* status, cudaStream_t st);
 
-// Merges the per-segment softmax statistics of every row into row_lse2 / row_ent (used by the
-// CUDA-core scorer; the tensor-core scorer does this at the start of its second pass).
+// Merges the per-segment softmax statistics of every row into row_lse2 / row_ent (CUDA-core scorer).
 cudaError_t launch_finalize_rows(const Ctx& ctx, int parts, cudaStream_t st);
 
 // S_j = sum_h cols[h][j]; optional C <- lambda C + S; then the layer's metrics: metrics[0] from

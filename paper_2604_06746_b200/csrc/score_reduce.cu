@@ -78,7 +78,7 @@ template <int VEC>
 __global__ void __launch_bounds__(kRcThreads)
 reduce_finish(const float* __restrict__ cols, long long col_stride, int H, int n, float lambda,
               float* __restrict__ s_out, float* __restrict__ c_inout, const float* __restrict__ row_ent,
-              int rows_pad, int rows_pg_pad, int rows_pg, int n_valid, const float* __restrict__ head_part,
+              int rows_pad, int n_valid, const float* __restrict__ head_part,
               int with_head_stats, float* __restrict__ metrics) {
   __shared__ float red[33];
   pdl_trigger();
@@ -123,8 +123,7 @@ reduce_finish(const float* __restrict__ cols, long long col_stride, int H, int n
   }
   if (blockIdx.x != 0) return;
   float ent = 0.f;
-  for (int r = threadIdx.x; r < rows_pad; r += kRcThreads)
-    if ((r % rows_pg_pad) < rows_pg) ent += row_ent[r];
+  for (int r = threadIdx.x; r < rows_pad; r += kRcThreads) ent += row_ent[r];
   const float tot = block_sum_1024(ent, red);
   if (threadIdx.x != 0) return;
   metrics[0] = tot / (float)n_valid;
@@ -151,8 +150,8 @@ template <int VEC>
 __global__ void __launch_bounds__(kRcThreads)
 reduce_layers(const float* __restrict__ cols, long long layer_stride, long long col_stride, int H, int n,
               int n_layers, float lambda, float* __restrict__ s_out, long long s_stride,
-              float* __restrict__ c_inout, const float* __restrict__ row_ent, int rows_pad, int rows_pg_pad,
-              int rows_pg, int n_valid, float* __restrict__ metrics) {
+              float* __restrict__ c_inout, const float* __restrict__ row_ent, int rows_pad,
+              int n_valid, float* __restrict__ metrics) {
   __shared__ float red[33];
   pdl_trigger();
   pdl_wait();
@@ -203,8 +202,7 @@ reduce_layers(const float* __restrict__ cols, long long layer_stride, long long 
   // blocks walk over the layers for the entropies (there may be fewer blocks than layers)
   for (int l = blockIdx.x; l < n_layers; l += gridDim.x) {
     float ent = 0.f;
-    for (int r = threadIdx.x; r < rows_pad; r += kRcThreads)
-      if ((r % rows_pg_pad) < rows_pg) ent += row_ent[(size_t)l * rows_pad + r];
+    for (int r = threadIdx.x; r < rows_pad; r += kRcThreads) ent += row_ent[(size_t)l * rows_pad + r];
     const float tot = block_sum_1024(ent, red);
     if (threadIdx.x == 0) {
       metrics[l * 3 + 0] = tot / (float)n_valid;
@@ -457,17 +455,15 @@ cudaError_t launch_reduce_layers(const Ctx& ctx, const float* cols, long long la
                                  int n, int n_layers, float lambda, float* s_out, long long s_stride,
                                  float* c_inout, const float* row_ent, float* metrics, cudaStream_t st) {
   const int H = ctx.cfg.n_q_heads;
-  const int rows_pg_pad = ctx.rows_pad / ctx.cfg.n_kv_heads;
-  const int rows_pg = (H / ctx.cfg.n_kv_heads) * ctx.cfg.window;
   const bool vec = n % 4 == 0 && col_stride % 4 == 0 && layer_stride % 4 == 0 && s_stride % 4 == 0 &&
                    ((uintptr_t)cols % 16) == 0 && ((uintptr_t)s_out % 16) == 0 && ((uintptr_t)c_inout % 16) == 0;
   if (vec)
     return launch_pdl(reduce_layers<4>, dim3((n / 4 + 63) / 64), dim3(kRcThreads), 0, st, cols, layer_stride,
                       col_stride, H, n, n_layers, lambda, s_out, s_stride, c_inout, row_ent, ctx.rows_pad,
-                      rows_pg_pad, rows_pg, ctx.rows, metrics);
+                      ctx.rows, metrics);
   return launch_pdl(reduce_layers<1>, dim3((n + kRcThreads - 1) / kRcThreads), dim3(kRcThreads), 0, st, cols,
                     layer_stride, col_stride, H, n, n_layers, lambda, s_out, s_stride, c_inout, row_ent,
-                    ctx.rows_pad, rows_pg_pad, rows_pg, ctx.rows, metrics);
+                    ctx.rows_pad, ctx.rows, metrics);
 }
 
 cudaError_t launch_reduce_finish(const Ctx& ctx, const float* cols, long long col_stride, int n, float lambda,
@@ -478,18 +474,16 @@ cudaError_t launch_reduce_finish(const Ctx& ctx, const float* cols, long long co
     const cudaError_t e = launch_head_stats(cols, 0, col_stride, 1, H, n, ctx.ws.head_part, ctx.sm_count, st);
     if (e != cudaSuccess) return e;
   }
-  const int rows_pg_pad = ctx.rows_pad / ctx.cfg.n_kv_heads;
-  const int rows_pg = (H / ctx.cfg.n_kv_heads) * ctx.cfg.window;
   const bool vec = n % 4 == 0 && col_stride % 4 == 0 && ((uintptr_t)cols % 16) == 0 &&
                    ((uintptr_t)s_out % 16) == 0 && ((uintptr_t)c_inout % 16) == 0;
   if (vec)
     return launch_pdl(reduce_finish<4>, dim3((n / 4 + 63) / 64), dim3(kRcThreads), 0, st, cols,
                       col_stride, H, n, lambda, s_out, c_inout, (const float*)ctx.ws.row_ent, ctx.rows_pad,
-                      rows_pg_pad, rows_pg, ctx.rows, (const float*)ctx.ws.head_part, with_head_stats ? 1 : 0,
+                      ctx.rows, (const float*)ctx.ws.head_part, with_head_stats ? 1 : 0,
                       metrics);
   return launch_pdl(reduce_finish<1>, dim3((n + kRcThreads - 1) / kRcThreads), dim3(kRcThreads), 0, st, cols,
                     col_stride, H, n, lambda, s_out, c_inout, (const float*)ctx.ws.row_ent, ctx.rows_pad,
-                    rows_pg_pad, rows_pg, ctx.rows, (const float*)ctx.ws.head_part, with_head_stats ? 1 : 0,
+                    ctx.rows, (const float*)ctx.ws.head_part, with_head_stats ? 1 : 0,
                     metrics);
 }
 

@@ -160,7 +160,7 @@ cudaError_t launch_typed(const Ctx& ctx, const ScoreArgs& a, int* parts_out, int
   const float c2 = a.scale * kLog2e;
   if (pass == 1) {
     const int n_chunks = (N + kP1Keys - 1) / kP1Keys;
-    int parts = n_chunks < 64 ? n_chunks : 64;
+    int parts = n_chunks < kSimtParts ? n_chunks : kSimtParts;
     *parts_out = parts;
     const size_t smem = ((size_t)w * D + kP1Keys * (D + 1) + 3 * (size_t)w) * sizeof(float);
     cudaError_t e = cudaFuncSetAttribute(simt_pass1<T, D>,

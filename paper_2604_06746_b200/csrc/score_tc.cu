@@ -1,964 +1,16 @@
-// Tensor-core scorer for bf16 storage on sm_100a: TMA-staged K tiles, tcgen05.mma with fp32
-// accumulators in tensor memory, softmax statistics / column sums computed straight out of
-// tensor memory.  Two kernels share one skeleton:
-//
-//   pass 1  D[rows, keys] = Q K^T     lane = score row  -> per-row (ref, Z, U) over a key segment
-//   pass 2  D[keys, rows] = K Q^T     lane = key        -> per-head column sums for every key
-//
-// so both reductions are loops inside one thread (no shuffles).  Both passes issue M128 x N256
-// MMAs: pass 1 multiplies one 128-row half of the Q block with a PAIR of 128-key tiles (two
-// neighbouring stages of the K ring form one 256-key operand), pass 2 one 128-key tile with the
-// whole 256-row Q block.  (An N128 MMA reads as many operand bytes from shared memory per clock
-// as the SM can deliver, and slows down as soon as anything else touches shared memory.)
-// A work unit is (KV group g, row block rb of up to 256 score rows), served by `segs` CTAs.  In
-// pass 1 each of them owns a fixed, equal share of the unit's key-tile pairs (its partial row
-// statistics must not depend on timing); in pass 2 they draw key tiles from the unit's ticket
-// counter, so that all of them finish within one tile of each other whenever they started.
-// Warp roles: warp 0 = TMA producer (and ticket taker), warp 1 = MMA issuer (owns the
-// tensor-memory allocation), warps 2..17 = compute (four per scheduler, so that one warp's
-// tensor-memory load latency hides behind the others' arithmetic).  Which item a K stage or an
-// accumulator holds travels with it through shared memory; an end mark follows the last item.
-// Pass 2 starts by merging the pass-1 CTAs' row statistics into each row's log-sum-exp (and, in
-// segment 0, its entropy).
-// Every wait is bounded; on expiry the CTA records STRUCTKV_ERR_TIMEOUT and stops issuing work;
-// it then waits (with a fresh bound that ignores the abort flag) for its own copies and MMAs in
-// flight, and frees tensor memory only if those MMAs are known to have retired.
-#include <cuda.h>
-#include <cudaTypedefs.h>
+// Host side of the tensor-core scorer (score_tc.cuh): tensor maps, how a call's work is cut into
+// tasks and in which order they are drawn.
+#include "score_tc.cuh"
 
-#include "common.cuh"
+#include <algorithm>
+#include <cmath>
 
 namespace skv {
 namespace {
 
-constexpr int kStages = 4;             // K tile ring
-constexpr int kAccStages = 2;          // accumulator ring in tensor memory (256 columns each)
-constexpr int kComputeWarps = 16;
-constexpr int kComputeThreads = kComputeWarps * 32;
-constexpr int kTcThreads = 64 + kComputeThreads;   // TMA warp, MMA warp, compute warps
-constexpr unsigned long long kWaitCycles = 1000000000ull;   // about 0.5 s at the maximum SM clock
-constexpr float kMasked = -1.0e30f;    // stands for -inf: 2^x flushes to 0 and 0 * x stays finite
-
-// One sequence of a call: its keys are rows [key0, key0 + n_keys) of the packed K.  Every full
-// row block of a KV group is worked on by `segs` CTAs and the group's last row block by
-// `segs_last` (fewer when it holds only one 128-row half), so a group takes
-// (n_rb - 1) * segs + segs_last consecutive CTAs from cta0 on.  A plain call is a batch of one.
-struct SeqDesc {
-  int key0, n_keys, cta0, segs, segs_last;
-  unsigned int period, period_last;   // pass 2: tickets one launch draws from a unit's counter (tiles + CTAs of the unit)
-};
-
-struct TcParams {
-  int window, group, rows_pg, rows_pg_pad, rows_pad, n_rb;
-  int n_seq;                           // sequences in this launch
-  int q_rows;                          // score rows of one sequence in the Q tensor (H * w)
-  long long rows_all;                  // n_seq * rows_pad: stride between segments in row_part
-  SeqDesc seq[kMaxBatch];
-  float c2;                            // scale * log2(e)
-  float inv_c2;                        // 1 / c2, or 0 when the fold of -lse into the MMA is off
-  int fold;                            // pass 2: the accumulator already holds q.k - lse / c2
-  int inputs_ready;                    // pass 1: Q and K are complete and visible, no kernel in flight writes them
-  // Work queue of pass 2: one ticket counter per (sequence, KV group, row block); a CTA draws
-  // key tiles of its unit from it until the unit has none left.  The counters only ever grow;
-  // a ticket is read modulo the number of tickets one launch draws (SeqDesc::period).
-  unsigned long long* queue;
-  int use_tickets;                     // pass 2: draw tiles from the counters (else a fixed split like pass 1's)
-  // Completion counter of pass 1 (or NULL): every pass-1 CTA adds one once its row statistics are
-  // stored; pass 2 then waits for `done_target` instead of for the kernel before it in the stream,
-  // which lets a caller put the NEXT layer's pass 1 between the two passes of a layer.
-  unsigned int* done;
-  unsigned int done_target;
-  float4* row_part;                    // pass 1 out, pass 2 in: [segs][n_seq][rows_pad] (ref, Z, U, -)
-  float* row_ent;                      // pass 2 out (segment 0 only): [n_seq][rows_pad] entropy of each score row, nats
-  float* cols;                         // pass 2 out [H][col_stride], sequence b at column key0_b
-  long long col_stride;
-  int* status;
-};
-
 struct TcState {
   PFN_cuTensorMapEncodeTiled_v12000 encode;
 };
-
-// ---- PTX wrappers ----------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-  return ok != 0;
-}
-// Same test, letting the hardware suspend the thread for up to `ns` nanoseconds while the phase
-// is incomplete: a waiting producer then issues (almost) no instructions on its scheduler.
-#ifndef SKV_WAIT_HINT_NS
-#define SKV_WAIT_HINT_NS 1000
-#endif
-__device__ __forceinline__ bool mbar_try_suspend(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
-      "selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok) : "r"(bar), "r"(parity), "r"((uint32_t)SKV_WAIT_HINT_NS) : "memory");
-  return ok != 0;
-}
-// Bounded wait of a producer (TMA / MMA warp): long, rarely latency critical.
-__device__ __forceinline__ bool mbar_wait_producer(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                                   unsigned long long limit) {
-  if (mbar_try(bar, parity)) return true;
-  const long long t0 = clock64();
-  for (;;) {
-#pragma unroll 1
-    for (int i = 0; i < 16; ++i)
-      if (SKV_WAIT_HINT_NS > 0 ? mbar_try_suspend(bar, parity) : mbar_try(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if ((unsigned long long)(clock64() - t0) > limit) { *abort_flag = 1; return false; }
-  }
-}
-// Bounded wait.  Returns false if the barrier did not flip within `limit` cycles or the CTA is
-// aborting; the first waiter whose bound expires raises the CTA's abort flag.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                          unsigned long long limit = kWaitCycles) {
-  if (mbar_try(bar, parity)) return true;
-  const long long t0 = clock64();
-  for (;;) {
-#pragma unroll 1
-    for (int i = 0; i < 256; ++i)
-      if (mbar_try(bar, parity)) return true;
-    if (*abort_flag) return false;
-    if ((unsigned long long)(clock64() - t0) > limit) { *abort_flag = 1; return false; }
-  }
-}
-// Bounded wait for work this thread itself put in flight (copies, MMAs): runs after an abort as
-// well, so it ignores the abort flag and starts its own timer.  False = still in flight.
-__device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                           unsigned long long limit = kWaitCycles) {
-  if (mbar_try(bar, parity)) return true;
-  const long long t0 = clock64();
-  for (;;) {
-#pragma unroll 1
-    for (int i = 0; i < 256; ++i)
-      if (mbar_try(bar, parity)) return true;
-    if ((unsigned long long)(clock64() - t0) > limit) { *abort_flag = 1; return false; }
-  }
-}
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0,
-                                            int c1, int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-      ::"r"(dst), "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
-}
-// The same copy with an L2 eviction-priority hint for the lines it brings in.
-__device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0,
-                                                 int c1, int c2, uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint "
-      "[%0], [%1, {%3, %4, %5}], [%2], %6;"
-      ::"r"(dst), "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1), "r"(c2), "l"(policy) : "memory");
-}
-__device__ __forceinline__ uint64_t l2_policy_evict_last() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ uint64_t l2_policy_evict_first() {
-  uint64_t p;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
-  return p;
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0,
-                                            int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-      ::"r"(dst), "l"((uint64_t)map), "r"(bar), "r"(c0), "r"(c1) : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                            uint32_t accumulate) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-      ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-// 32 lanes x 32 consecutive fp32 columns: thread l of the warp receives row (lane base + l).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-// Waits for the thread's outstanding tensor-memory loads.  The loaded registers are operands,
-// so no use of them can be scheduled ahead of the wait.
-__device__ __forceinline__ void tmem_ld_wait(float (&v)[32]) {
-  uint32_t* r = reinterpret_cast<uint32_t*>(v);
-  asm volatile(
-      "tcgen05.wait::ld.sync.aligned;"
-      : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-        "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
-        "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
-        "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-      :: "memory");
-}
-
-// Two fp32 values in one 64-bit register, for the packed fp32 instructions of sm_100
-// (one issue slot for two results).
-__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t r, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(r));
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-
-// 2^x for a pair, on the FMA pipe, x in [-125, 126]: round-to-nearest split x = n + f with the
-// 1.5 * 2^23 trick (n lands in the low mantissa bits of t), a degree-3 minimax polynomial
-// for 2^f on [-0.5, 0.5] (relative error 7.5e-5), and n added into the exponent field.
-__device__ __forceinline__ uint64_t exp2_poly2(uint64_t x) {
-  const uint64_t magic = pack2(12582912.0f, 12582912.0f);
-  const uint64_t t = add2(x, magic);
-  const uint64_t f = sub2(x, sub2(t, magic));
-  uint64_t p = fma2(pack2(0.0551716685f, 0.0551716685f), f, pack2(0.2426111251f, 0.2426111251f));
-  p = fma2(p, f, pack2(0.6932609677f, 0.6932609677f));
-  p = fma2(p, f, pack2(0.9999280572f, 0.9999280572f));
-  float t0, t1, p0, p1;
-  unpack2(t, t0, t1);
-  unpack2(p, p0, p1);
-  return pack2(__int_as_float(__float_as_int(p0) + (__float_as_int(t0) << 23)),
-               __int_as_float(__float_as_int(p1) + (__float_as_int(t1) << 23)));
-}
-// 2^x for a pair on the special-function unit.
-__device__ __forceinline__ uint64_t exp2_sfu2(uint64_t x) {
-  float x0, x1;
-  unpack2(x, x0, x1);
-  return pack2(fast_exp2(x0), fast_exp2(x1));
-}
-// In pass 1, of every 8 consecutive element pairs the first kPoly1 take the polynomial.
-#ifndef SKV_POLY1
-#define SKV_POLY1 1
-#endif
-// Pass 2: subtract lse inside the MMA (one extra K-step) instead of loading it from shared memory.
-#ifndef SKV_FOLD
-#define SKV_FOLD 1
-#endif
-// Percentage of a pass-1 segment (its end) that L2 is asked to keep for pass 2; 0 = no hints.
-#ifndef SKV_L2_KEEP_PCT
-#define SKV_L2_KEEP_PCT 20
-#endif
-constexpr int kPoly1 = SKV_POLY1;
-// In pass 2, of every 8 consecutive element pairs the first kPoly2 take the polynomial, the
-// rest the special-function unit: the two pipes work side by side (2 of 8 measured best).
-#ifndef SKV_POLY2
-#define SKV_POLY2 2
-#endif
-constexpr int kPoly2 = SKV_POLY2;
-
-// Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of 128 bytes, 8-row
-// groups 1024 bytes apart (the layout TMA writes with CU_TENSOR_MAP_SWIZZLE_128B).
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr >> 4) & 0x3fffu);          // start address, 16-byte units
-  d |= (uint64_t)1 << 16;                          // leading-dimension byte offset (unused for swizzled K-major)
-  d |= (uint64_t)(1024 >> 4) << 32;                // stride between 8-row groups
-  d |= (uint64_t)1 << 46;                          // descriptor version of this architecture
-  d |= (uint64_t)2 << 61;                          // 128-byte swizzle
-  return d;
-}
-// Shared-memory matrix descriptor of an unswizzled K-major operand of 16 columns (one MMA
-// K-step): 8-row x 16-byte core matrices of 128 contiguous bytes, the two K halves of a row
-// group 128 bytes apart, row groups 256 bytes apart.  Element (row, k) therefore sits at
-// (row / 8) * 256 + (k / 8) * 128 + (row % 8) * 16 + (k % 8) * 2.
-__device__ __forceinline__ uint64_t smem_desc_k16(uint32_t addr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((addr >> 4) & 0x3fffu);
-  d |= (uint64_t)(128 >> 4) << 16;                 // between the core matrices of one row group (K direction)
-  d |= (uint64_t)(256 >> 4) << 32;                 // between row groups
-  d |= (uint64_t)1 << 46;
-  return d;
-}
-__device__ __forceinline__ uint32_t k16_offset(int row, int k) {
-  return (uint32_t)((row >> 3) * 256 + (k >> 3) * 128 + (row & 7) * 16 + (k & 7) * 2);
-}
-// Instruction descriptor: bf16 x bf16 -> fp32, both operands K-major, tile M x N.
-__host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-// ---- shared memory layout ----------------------------------------------------------------
-template <int D>
-struct Smem {
-  static constexpr int kSub = D / 64;                      // 64-column (128-byte) sub-tiles per operand
-  static constexpr int kQBytes = kRowBlock * 128 * kSub;   // Q block: 256 rows
-  static constexpr int kKSub = kKeyTile * 128;             // one sub-tile of one K stage: 128 keys x 128 bytes
-  static constexpr int kKBytes = kKSub * kSub;             // bytes TMA delivers per stage
-  static constexpr int kQOff = 0;
-  // K ring, sub-tile major: sub-tile c of stage s sits at kKOff + (c * kStages + s) * kKSub, so the
-  // same sub-tile of stages s and s + 1 is one contiguous 256-key operand
-  static constexpr int kKOff = kQBytes;
-  static constexpr int kLseOff = kKOff + kStages * kKBytes;          // 256 floats
-  // pass 1: [4 column groups][256 rows] (ref, Z, U); pass 2: 256 x (M, Z, X) for the merge
-  static constexpr int kMergeOff = kLseOff + kRowBlock * 4;
-  static constexpr int kBarOff = kMergeOff + 4 * kRowBlock * 16;
-  static constexpr int kBytes = kBarOff + 256;
-  static constexpr int kAlloc = kBytes + 1024;             // slack to align the base to 1024 bytes
-  static_assert(kAlloc <= 227 * 1024, "shared memory of one CTA");
-};
-
-// Barrier slots (8 bytes each) inside the barrier area.
-enum { kBarFull = 0, kBarEmpty = kStages, kBarQ = 2 * kStages, kBarAccFull = 2 * kStages + 1,
-       kBarAccEmpty = kBarAccFull + kAccStages, kBarDrain = kBarAccEmpty + kAccStages,
-       kBarExt = kBarDrain + 1, kBarCount = kBarExt + 1 };
-
-template <int D, int PASS, int W>
-__global__ void __launch_bounds__(kTcThreads, 1)
-tc_score(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
-         const __grid_constant__ TcParams p) {
-  using L = Smem<D>;
-  extern __shared__ unsigned char smem_raw[];
-  const uint32_t raw = smem_u32(smem_raw);
-  const uint32_t base = (raw + 1023u) & ~1023u;
-  unsigned char* sm = smem_raw + (base - raw);
-  const uint32_t bars = base + L::kBarOff;
-  float* lse_s = reinterpret_cast<float*>(sm + L::kLseOff);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(sm + L::kBarOff + 8 * kBarCount);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + L::kBarOff + 8 * kBarCount + 8);
-  volatile int* mma_in_flight = reinterpret_cast<volatile int*>(sm + L::kBarOff + 8 * kBarCount + 16);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int sq = 0;                                                // the sequence this CTA works on
-  while (sq + 1 < p.n_seq && (int)blockIdx.x >= p.seq[sq + 1].cta0) ++sq;
-  const int n_keys = p.seq[sq].n_keys, key0 = p.seq[sq].key0;
-  const int cta = (int)blockIdx.x - p.seq[sq].cta0;
-  const int per_group = (p.n_rb - 1) * p.seq[sq].segs + p.seq[sq].segs_last;
-  const int g = cta / per_group, in_group = cta - g * per_group;
-  const int rb = min(in_group / p.seq[sq].segs, p.n_rb - 1);
-  const int seg = in_group - rb * p.seq[sq].segs;
-  const int segs = rb == p.n_rb - 1 ? p.seq[sq].segs_last : p.seq[sq].segs;
-  const int unit = g * p.n_rb + rb;
-  const size_t row_base = (size_t)sq * p.rows_pad + (size_t)g * p.rows_pg_pad + rb * kRowBlock;
-  // Pass 1 works on pairs of key tiles (256 keys per MMA), pass 2 on single tiles.
-  // Pass 1: CTA `seg` of a unit owns a fixed, contiguous range of pairs.  Its row statistics are
-  // partial sums over exactly that range, so the result does not depend on timing (the same
-  // inputs give the same bits).
-  // Pass 2: a tile's column sums do not depend on who computes them, so the CTAs of a unit draw
-  // tiles from the unit's ticket counter: one that starts late or runs slowly simply takes fewer,
-  // and all CTAs of a unit finish within one tile of each other.  Tiles are handed out from the
-  // end of the sequence: the tiles pass 1 touched last are the ones still in L2.
-  const int n_tiles = (n_keys + kKeyTile - 1) / kKeyTile;
-  const int n_items = PASS == 1 ? (n_tiles + 1) / 2 : n_tiles;
-  const int t_lo = (int)((long long)seg * n_items / segs);          // fixed split: first item of this CTA
-  const int n_static = (int)((long long)(seg + 1) * n_items / segs) - t_lo;
-  const int units_per_seq = p.n_rb * (p.rows_pad / p.rows_pg_pad);
-  unsigned long long* const ticket = p.queue + (size_t)sq * kQueueUnits + unit;
-  int* item_s = reinterpret_cast<int*>(sm + L::kBarOff + 8 * kBarCount + 32);      // producer -> MMA issuer, per K slot
-  volatile int* unit_item = reinterpret_cast<volatile int*>(sm + L::kBarOff + 8 * kBarCount + 48);   // MMA issuer -> compute warps, per accumulator stage
-  const int rows_here = min(kRowBlock, p.rows_pg - rb * kRowBlock);     // valid score rows in this block
-  const int n_half = (rows_here + 127) / 128;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) { mbar_init(bars + 8 * (kBarFull + s), 1); mbar_init(bars + 8 * (kBarEmpty + s), 1); }
-    mbar_init(bars + 8 * kBarQ, 1);
-    for (int a = 0; a < kAccStages; ++a) {
-      mbar_init(bars + 8 * (kBarAccFull + a), 1);
-      mbar_init(bars + 8 * (kBarAccEmpty + a), kComputeWarps);   // one arrival per compute warp
-    }
-    mbar_init(bars + 8 * kBarDrain, 1);
-    mbar_init(bars + 8 * kBarExt, 1);
-    *abort_flag = 0;
-    *mma_in_flight = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  // Pass 1 reads tensors an earlier kernel may have produced and overwrites statistics the
-  // previous layer still reads: it waits for that kernel first and only then lets pass 2 begin,
-  // so pass 2 (whose producer warps read K and Q without waiting) never runs ahead of the
-  // kernel that precedes pass 1.  In pass 2 only the compute warps depend on pass 1 (the row
-  // statistics): the loads of K and Q and the MMAs start at once.
-  // Where the caller vouches for Q and K (inputs_ready), pass 1 starts at once as well and only
-  // its stores of the row statistics wait for the kernels before it; pass 2 still cannot begin
-  // its own stores before those kernels are done, because pass 1 cannot complete earlier.
-  if (PASS == 1 && !p.inputs_ready) pdl_wait();
-  pdl_trigger();
-
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      // first ticket at once: its latency hides behind the Q load
-      const bool tickets = PASS == 2 && p.use_tickets;
-      unsigned long long tk = tickets ? atomicAdd(ticket, 1ull) : 0ull;
-      mbar_expect_tx(bars + 8 * kBarQ, L::kQBytes);
-      const int q_row0 = sq * p.q_rows + g * p.rows_pg + rb * kRowBlock;
-      for (int s = 0; s < L::kSub; ++s)
-        tma_load_2d(base + L::kQOff + s * (L::kQBytes / L::kSub), &map_q, bars + 8 * kBarQ, s * 64, q_row0);
-      int issued = 0;                                      // 128-key tiles requested so far
-      bool end_marked = false;
-      // Pass 2 meets first the tiles pass 1 read last: pass 1 asks L2 to keep the last
-      // SKV_L2_KEEP_PCT percent of the sequence's keys and lets the rest stream through; pass 2
-      // never needs a line again.
-      const uint64_t pol_keep = l2_policy_evict_last(), pol_stream = l2_policy_evict_first();
-      const int keep_from = PASS == 1 ? n_items - (n_items * SKV_L2_KEEP_PCT) / 100 : n_items;
-      constexpr int kPerItem = PASS == 1 ? 2 : 1;          // K stages one item occupies
-      for (int it = 0;; ++it) {
-        int item;
-        if (!tickets) {
-          // pass 1 ascending; pass 2 descending, from the end of its share
-          item = it < n_static ? (PASS == 1 ? t_lo + it : t_lo + n_static - 1 - it) : -1;
-        } else {
-          const int idx = (int)(tk % (unsigned long long)(rb == p.n_rb - 1 ? p.seq[sq].period_last : p.seq[sq].period));
-          item = idx < n_items ? n_items - 1 - idx : -1;
-          if (item >= 0) tk = atomicAdd(ticket, 1ull);     // the next ticket travels while this tile is loaded
-        }
-        const int s0 = (kPerItem * it) % kStages;
-        const uint32_t ph = (uint32_t)((kPerItem * it) / kStages) & 1u;
-        if (!mbar_wait_producer(bars + 8 * (kBarEmpty + s0), ph ^ 1u, abort_flag, kWaitCycles)) break;
-        item_s[s0 / kPerItem] = item;                      // read by the MMA issuer once the stage is full
-        if (item < 0) {                                    // nothing left: an empty "full" stage says so
-          mbar_arrive(bars + 8 * (kBarFull + s0));
-          end_marked = true;
-          break;
-        }
-        bool ok = true;
-#pragma unroll
-        for (int half = 0; half < kPerItem && ok; ++half) {
-          const int s = s0 + half;
-          if (half > 0) ok = mbar_wait_producer(bars + 8 * (kBarEmpty + s), ph ^ 1u, abort_flag, kWaitCycles);
-          if (!ok) break;
-          mbar_expect_tx(bars + 8 * (kBarFull + s), L::kKBytes);
-          // a tile may reach beyond the sequence's last key (into zero fill, or into the next
-          // sequence of a packed batch): the causal mask discards those keys
-          const int tile = kPerItem * item + half;
-          for (int c = 0; c < L::kSub; ++c) {
-            if (SKV_L2_KEEP_PCT > 0)
-              tma_load_3d_hint(base + L::kKOff + (c * kStages + s) * L::kKSub, &map_k, bars + 8 * (kBarFull + s),
-                               c * 64, key0 + tile * kKeyTile, g, item >= keep_from ? pol_keep : pol_stream);
-            else
-              tma_load_3d(base + L::kKOff + (c * kStages + s) * L::kKSub, &map_k, bars + 8 * (kBarFull + s),
-                          c * 64, key0 + tile * kKeyTile, g);
-          }
-          ++issued;
-        }
-        if (!ok) break;
-      }
-      // drain: every copy this thread issued must have landed before the CTA may exit.  The end
-      // mark went into the stage of copy (issued - kStages): that copy was seen consumed before the
-      // mark was placed, and its barrier has moved on by two phases, so it is not waited for.
-      mbar_drain(bars + 8 * kBarQ, 0, abort_flag);
-      for (int t = max(0, issued - kStages + (end_marked ? 1 : 0)); t < issued; ++t)
-        mbar_drain(bars + 8 * (kBarFull + t % kStages), (uint32_t)(t / kStages) & 1u, abort_flag);
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      constexpr uint32_t idesc = instr_desc(128, 256);
-      const uint64_t q_desc0 = smem_desc(base + L::kQOff), k_desc0 = smem_desc(base + L::kKOff);
-      bool ok = mbar_wait_producer(bars + 8 * kBarQ, 0, abort_flag, kWaitCycles);
-      // Tells the compute warps through accumulator stage `a` of unit `u` that no unit follows.
-      auto announce_end = [&](int u) {
-        const int a = u % kAccStages;
-        if (!mbar_wait_producer(bars + 8 * (kBarAccEmpty + a), ((uint32_t)(u / kAccStages) & 1u) ^ 1u, abort_flag, kWaitCycles))
-          return;
-        unit_item[a] = -1;
-        mbar_arrive(bars + 8 * (kBarAccFull + a));
-      };
-      // descriptors differ only in the start-address field (16-byte units, no carry out of it)
-      if (PASS == 1) {
-        // unit u = (pair, row half): A = one 128-row half of Q, B = the pair's 256 keys
-        for (int t = 0, u = 0; ok; ++t) {
-          const int s0 = (2 * t) % kStages;
-          const uint32_t ph = (uint32_t)((2 * t) / kStages) & 1u;
-          if (!mbar_wait_producer(bars + 8 * (kBarFull + s0), ph, abort_flag, kWaitCycles)) break;
-          const int item = item_s[s0 / 2];
-          if (item < 0) { announce_end(u); break; }
-          if (!mbar_wait_producer(bars + 8 * (kBarFull + s0 + 1), ph, abort_flag, kWaitCycles)) break;
-          const uint64_t kd = k_desc0 + (uint64_t)((s0 * L::kKSub) >> 4);
-          for (int hf = 0; hf < n_half; ++hf, ++u) {
-            const int a = u % kAccStages;
-            if (!mbar_wait_producer(bars + 8 * (kBarAccEmpty + a), ((uint32_t)(u / kAccStages) & 1u) ^ 1u, abort_flag, kWaitCycles)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-              const uint32_t qo = (kk / 4) * (L::kQBytes / L::kSub) + hf * (128 * 128) + (kk % 4) * 32;
-              const uint32_t ko = (kk / 4) * (kStages * L::kKSub) + (kk % 4) * 32;
-              tc_mma_bf16(tmem + a * 256, q_desc0 + (qo >> 4), kd + (ko >> 4), idesc, kk > 0);
-            }
-            *mma_in_flight = 1;
-            unit_item[a] = item;                       // which pair the accumulator holds
-            __threadfence_block();
-            tc_commit(bars + 8 * (kBarAccFull + a));   // accumulator ready for the compute warps
-          }
-          if (!ok) break;
-          tc_commit(bars + 8 * (kBarEmpty + s0));      // both K stages reusable once these MMAs have read them
-          tc_commit(bars + 8 * (kBarEmpty + s0 + 1));
-        }
-      } else {
-        for (int t = 0; ok; ++t) {
-          const int s = t % kStages, a = t % kAccStages;
-          if (!mbar_wait_producer(bars + 8 * (kBarFull + s), (uint32_t)(t / kStages) & 1u, abort_flag, kWaitCycles)) break;
-          const int item = item_s[s];
-          if (item < 0) { announce_end(t); break; }
-          if (!mbar_wait_producer(bars + 8 * (kBarAccEmpty + a), ((uint32_t)(t / kAccStages) & 1u) ^ 1u, abort_flag, kWaitCycles)) break;
-          tc_fence_after();
-          const uint64_t kd = k_desc0 + (uint64_t)((s * L::kKSub) >> 4);
-#pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk) {
-            const uint32_t ko = (kk / 4) * (kStages * L::kKSub) + (kk % 4) * 32;
-            const uint32_t qo = (kk / 4) * (L::kQBytes / L::kSub) + (kk % 4) * 32;
-            tc_mma_bf16(tmem + a * 256, kd + (ko >> 4), q_desc0 + (qo >> 4), idesc, kk > 0);
-          }
-          *mma_in_flight = 1;
-          if (p.fold) {
-            // one more K-step adds -lse / c2 of every row: ones (key side) x three bf16 pieces of
-            // the value (row side), written by the compute warps once pass 1 has completed
-            if (t == 0 && !mbar_wait_producer(bars + 8 * kBarExt, 0, abort_flag, kWaitCycles)) break;
-            tc_mma_bf16(tmem + a * 256, smem_desc_k16(base + L::kMergeOff + 4096),
-                        smem_desc_k16(base + L::kMergeOff + 8192), idesc, 1);
-          }
-          unit_item[a] = item;                         // which tile the accumulator holds
-          __threadfence_block();
-          tc_commit(bars + 8 * (kBarEmpty + s));       // K stage reusable once these MMAs have read it
-          tc_commit(bars + 8 * (kBarAccFull + a));     // accumulator ready for the compute warps
-        }
-      }
-      // drain: all issued MMAs must retire before tensor memory is freed
-      if (*mma_in_flight) {
-        tc_commit(bars + 8 * kBarDrain);
-        if (mbar_drain(bars + 8 * kBarDrain, 0, abort_flag)) *mma_in_flight = 0;
-      }
-    }
-  } else {
-    // ---------------- compute warps ----------------
-    const int cw = warp - 2;                 // 0..15
-    const int quarter = warp & 3;            // tensor-memory lane quarter this warp may read
-    const int sub = cw >> 2;                 // which 64 accumulator columns of a tile this warp reads
-    const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-    // a tile is "plain" when all of its keys are visible to every window row (j0 + 127 <= N - w);
-    // the first (N - w + 1) / 128 tiles are
-    const int first_tail_tile = (n_keys - p.window + 1) / kKeyTile;
-    float v[32];
-    // lane 0 polls the barrier for its warp (bounded) and reads which item the accumulator
-    // holds; the outcome is broadcast: the item, -1 when the unit has no item left, -2 after an
-    // expired wait
-    auto acc_full = [&](int t) {
-      int item = -2;
-      if (lane == 0 && mbar_wait(bars + 8 * (kBarAccFull + t % kAccStages), (uint32_t)(t / kAccStages) & 1u, abort_flag))
-        item = unit_item[t % kAccStages];
-      item = __shfl_sync(0xffffffffu, item, 0);
-      tc_fence_after();
-      return item;
-    };
-    // all of this warp's loads of the tile have landed: one arrival per warp frees the accumulator
-    auto acc_release = [&](int t) {
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bars + 8 * (kBarAccEmpty + t % kAccStages));
-    };
-
-    if (PASS == 1) {
-      // A unit's accumulator holds one 128-row half of the block x the pair's 256 keys.  This
-      // thread owns row (quarter * 32 + lane) of BOTH halves (units alternate between them) and
-      // the 64 keys [sub * 64, sub * 64 + 64) of every pair.
-      struct RowStat { float ref, Z, U; };
-      RowStat st[2] = {{-INFINITY, 0.f, 0.f}, {-INFINITY, 0.f, 0.f}};
-      const uint64_t c22 = pack2(p.c2, p.c2);
-      const int row_lo = quarter * 32 + lane;
-      const int i_win = row_lo % p.window;          // window row of this thread's rows (the window divides 128)
-      const int t_pos = n_keys - p.window + i_win;                     // their position: they see keys <= t_pos
-      const int last_open_key = n_keys - p.window;               // the last key every window row sees
-      // Z += 2^(x - ref), U += 2^(x - ref) (x - ref) over one chunk whose keys are all visible;
-      // of every 8 elements the first kPoly1 are exponentiated on the FMA pipe
-      auto accumulate = [&](RowStat& r) {
-        // packed fp32: one instruction for two elements wherever the operation is not the exponential
-        const uint64_t nref2 = pack2(-r.ref, -r.ref);
-        uint64_t Z2 = pack2(r.Z, 0.f), U2 = pack2(r.U, 0.f);
-#pragma unroll
-        for (int pr = 0; pr < 16; ++pr) {
-          const uint64_t x2 = fma2(pack2(v[2 * pr], v[2 * pr + 1]), c22, nref2);
-          uint64_t p2;
-          if ((pr & 7) < kPoly1) {
-            float x0, x1;
-            unpack2(x2, x0, x1);
-            p2 = exp2_poly2(pack2(fminf(fmaxf(x0, -125.f), 126.f), fminf(fmaxf(x1, -125.f), 126.f)));
-          } else {
-            p2 = exp2_sfu2(x2);
-          }
-          Z2 = add2(Z2, p2);
-          U2 = fma2(p2, x2, U2);
-        }
-        float a, b;
-        unpack2(Z2, a, b);
-        r.Z = a + b;
-        unpack2(U2, a, b);
-        r.U = a + b;
-      };
-      // same with the causal mask, moving the reference up to the chunk maximum first
-      // (v[0] is key jb); works from registers, so the accumulator is not needed again
-      auto accumulate_careful = [&](RowStat& r, int jb) {
-        float mx = -INFINITY;
-#pragma unroll
-        for (int e = 0; e < 32; ++e)
-          if (jb + e <= t_pos) mx = fmaxf(mx, v[e] * p.c2);
-        if (mx > r.ref) {
-          if (r.ref != -INFINITY) {
-            const float dm = r.ref - mx, f = fast_exp2(dm);
-            r.U = f * fmaf(dm, r.Z, r.U);
-            r.Z = f * r.Z;
-          }
-          r.ref = mx;
-        }
-        const float ref_use = (r.ref == -INFINITY) ? 0.f : r.ref;  // row has seen no key yet: all masked
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          const float x = (jb + e <= t_pos) ? fmaf(v[e], p.c2, -ref_use) : kMasked;
-          const float pr = fast_exp2(x);
-          r.Z += pr;
-          r.U = fmaf(pr, x, r.U);
-        }
-      };
-      // `fast` is warp-uniform: the keys are unmasked and the reference already exists
-      auto chunk = [&](RowStat& r, int jb, bool fast) {
-        if (fast) {
-          const float Z0 = r.Z, U0 = r.U;
-          accumulate(r);
-          // a logit far above the reference overflowed (or was clamped at 2^126): redo the chunk
-          const bool ovf = !(r.Z < 4.0e37f) || !(fabsf(r.U) < 3.0e38f);
-          if (__any_sync(0xffffffffu, ovf)) { r.Z = Z0; r.U = U0; accumulate_careful(r, jb); }
-        } else {
-          accumulate_careful(r, jb);
-        }
-      };
-      bool live = true;
-      for (int t = 0, u = 0; live; ++t) {
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          if (hf < n_half && live) {
-            const int item = acc_full(u);                 // the same pair for both row halves
-            if (item < 0) { live = false; continue; }
-            const int jb = item * (2 * kKeyTile) + sub * 64;
-            // a 32-key chunk takes the plain path when every window row sees all of its keys; of
-            // the sequence's last pair only the chunks that hold window keys (or lie beyond the
-            // sequence) take the masked one
-            const bool plain0 = jb + 31 <= last_open_key, plain1 = jb + 63 <= last_open_key;
-            const bool warp_active = (hf * 128 + quarter * 32) < rows_here;
-            const uint32_t taddr = tmem + lane_base + (uint32_t)((u % kAccStages) * 256 + sub * 64);
-            if (warp_active) {
-              tmem_ld32(taddr, v);
-              tmem_ld_wait(v);
-              chunk(st[hf], jb, plain0 && t > 0);         // the first pair gives the rows their reference
-              tmem_ld32(taddr + 32, v);
-              tmem_ld_wait(v);
-            }
-            acc_release(u);
-            if (warp_active) chunk(st[hf], jb + 32, plain1);
-            ++u;
-          }
-        }
-      }
-      // The four column groups of a row fold into ONE partial per (row, segment): re-reference
-      // each to the largest reference M, Z = sum_c 2^(ref_c - M) Z_c,
-      // U = sum_c 2^(ref_c - M) (U_c + (ref_c - M) Z_c).
-      float4* part_s = reinterpret_cast<float4*>(sm + L::kMergeOff);
-      // the previous layer's pass 2 may still be reading the row statistics this pass overwrites
-      if (p.inputs_ready) pdl_wait();
-#pragma unroll
-      for (int hf = 0; hf < 2; ++hf)
-        part_s[sub * kRowBlock + hf * 128 + row_lo] = make_float4(st[hf].ref, st[hf].Z, st[hf].U, 0.f);
-      asm volatile("bar.sync 1, %0;" ::"n"(kComputeThreads) : "memory");
-      if (sub == 0) {
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          const int row_in_block = hf * 128 + row_lo;
-          if (row_in_block < rows_here) {
-            float4 c[4];
-            float M = -INFINITY;
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              c[k] = part_s[k * kRowBlock + row_in_block];
-              if (c[k].y > 0.f) M = fmaxf(M, c[k].x);
-            }
-            float Z = 0.f, U = 0.f;
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-              if (c[k].y > 0.f) {
-                const float dm = c[k].x - M, f = fast_exp2(dm);
-                Z = fmaf(f, c[k].y, Z);
-                U = fmaf(f, fmaf(dm, c[k].y, c[k].z), U);
-              }
-            p.row_part[(size_t)seg * p.rows_all + row_base + row_in_block] =
-                make_float4(M, Z, U, 0.f);
-          }
-        }
-      }
-      if (p.done) {
-        // the statistics are visible device-wide before the counter moves
-        __threadfence();
-        asm volatile("bar.sync 1, %0;" ::"n"(kComputeThreads) : "memory");
-        if (threadIdx.x == 64) atomicAdd(p.done, 1u);
-      }
-    } else {
-      // pass 2.  First the compute threads merge the partial statistics of this block's rows,
-      // two threads per row (each takes every other partial, loads batched), then one of them
-      // folds the two.  With l_s = ref_s + log2 Z_s (a partial's log-sum-exp), a running maximum
-      // M, Zt = sum_s 2^(l_s - M) and Xt = sum_s 2^(l_s - M) (ref_s - M + U_s / Z_s):
-      //   lse2 = M + log2 Zt,   entropy = ln2 (log2 Zt - Xt / Zt)                (Eq. 4, one row)
-      // lse_s holds -lse2; padded rows get -inf so that they contribute 2^(-inf) = 0.
-      {
-        const int ct = (int)threadIdx.x - 64;
-        if (p.fold) {
-          // operands of the extra K-step: zero both, then 1.0 in the first three K columns of the
-          // key-side operand (the row side is written after the merge below)
-          uint4* ext = reinterpret_cast<uint4*>(sm + L::kMergeOff + 4096);
-          for (int i = ct; i < (4096 + 8192) / 16; i += kComputeThreads) ext[i] = make_uint4(0u, 0u, 0u, 0u);
-          asm volatile("bar.sync 1, %0;" ::"n"(kComputeThreads) : "memory");
-          if (ct < kKeyTile) {
-            unsigned char* ax = sm + L::kMergeOff + 4096;
-#pragma unroll
-            for (int k = 0; k < 3; ++k)
-              *reinterpret_cast<__nv_bfloat16*>(ax + k16_offset(ct, k)) = __float2bfloat16_rn(1.0f);
-          }
-        }
-        if (p.done) {
-          // pass 1 of this layer is an earlier launch of the stream: all of its CTAs have started
-          // by the time this kernel runs, so the bounded wait below cannot be a wait for work
-          // that is not scheduled yet
-          if (ct == 0) {
-            const long long t0 = clock64();
-            for (;;) {
-              unsigned int seen;
-              asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(p.done) : "memory");
-              if (seen >= p.done_target || *abort_flag) break;
-              if ((unsigned long long)(clock64() - t0) > kWaitCycles) { *abort_flag = 1; break; }
-              __nanosleep(200);
-            }
-          }
-          asm volatile("bar.sync 1, %0;" ::"n"(kComputeThreads) : "memory");
-        } else {
-          pdl_wait();
-        }
-        const int r = ct & (kRowBlock - 1), hp = ct >> 8;
-        const size_t row = row_base + r;
-        const int parts = segs;
-        float M = -INFINITY, Zt = 0.f, Xt = 0.f;
-        auto fold = [&](float ref_s, float Z_s, float X_s) {     // X_s = sum 2^(..)(.. - ref_s), relative to ref_s
-          if (!(Z_s > 0.f)) return;
-          const float l = ref_s + log2f(Z_s);
-          if (l > M) {
-            if (M != -INFINITY) {
-              const float d = M - l, f = fast_exp2(d);
-              Xt = f * fmaf(d, Zt, Xt);
-              Zt = f * Zt;
-            }
-            M = l;
-          }
-          const float wgt = fast_exp2(l - M);
-          Zt += wgt;
-          Xt = fmaf(wgt, (ref_s - M) + X_s / Z_s, Xt);
-        };
-        if (r < rows_here) {
-          constexpr int kBatch = 9;                      // 18 segments (one per SM share of a KV group): one round of loads
-          for (int s0 = hp; s0 < parts; s0 += 2 * kBatch) {
-            float4 pv[kBatch];
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-              const int sidx = s0 + 2 * b;
-              pv[b] = sidx < parts ? __ldcg(&p.row_part[(size_t)sidx * p.rows_all + row])
-                                   : make_float4(-INFINITY, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int b = 0; b < kBatch; ++b) fold(pv[b].x, pv[b].y, pv[b].z);
-          }
-        }
-        float4* merge_s = reinterpret_cast<float4*>(sm + L::kMergeOff);
-        if (hp == 1) merge_s[r] = make_float4(M, Zt, Xt, 0.f);
-        asm volatile("bar.sync 1, %0;" ::"n"(kComputeThreads) : "memory");
-        if (hp == 0) {
-          // the other thread's result is one more partial: (reference M', sum Zt', Xt' relative to M')
-          const float4 o = merge_s[r];
-          if (o.y > 0.f) {
-            // its log-sum-exp is M' + log2 Zt'; fold() expects (ref, Z, X) with X relative to ref
-            fold(o.x, o.y, o.z);
-          }
-          float nlse = -INFINITY, ent = 0.f;
-          if (r < rows_here && Zt > 0.f) {
-            const float lz = log2f(Zt);
-            nlse = -(M + lz);
-            ent = kLn2 * (lz - Xt / Zt);
-          }
-          if (r < rows_here && seg == 0) p.row_ent[row] = ent;
-          lse_s[r] = nlse;
-          if (p.fold) {
-            // -lse / c2 as hi + mid + lo (bf16 each: 24 bits together); padded rows get a huge
-            // negative value so that their 2^x is 0
-            const float Lv = nlse == -INFINITY ? -1.0e30f : nlse * p.inv_c2;
-            const __nv_bfloat16 hi = __float2bfloat16_rn(Lv);
-            const float r1 = Lv - __bfloat162float(hi);
-            const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-            const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-            unsigned char* bx = sm + L::kMergeOff + 8192;
-            *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 0)) = hi;
-            *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 1)) = mid;
-            *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 2)) = lo;
-          }
-        }
-        if (p.fold) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
-        asm volatile("bar.sync 1, %0;" ::"n"(kComputeThreads) : "memory");
-        if (p.fold && ct == 0) mbar_arrive(bars + 8 * kBarExt);
-      }
-      // This thread owns key (tile * 128 + quarter * 32 + lane).  Rows: for W <= 64 the block's
-      // rows [sub * 64, sub * 64 + 64) of every tile (two heads at W = 32, one at W = 64); for
-      // W = 128 the 128 rows of head (sub & 1) on every other tile, tiles alternating between the
-      // warps with sub >> 1 = 0 and 1, so that a head's column sum never spans two warps.
-      constexpr int kChunks = (W == 128) ? 4 : 2;
-      const int col0 = (W == 128) ? (sub & 1) * 128 : sub * 64;   // first accumulator column = local row
-      const float inv_w = 1.0f / (float)p.window;
-      const int row0 = rb * kRowBlock + col0;                // first score row (within the group) of this thread
-      const bool warp_active = col0 < rows_here;
-      const int h0 = g * p.group + row0 / p.window;          // (first) head of this thread
-      // sum over the chunk's 32 rows of 2^(x - lse) for this thread's key, all rows visible
-      // (packed arithmetic; lse_s holds -lse)
-      auto pair_sum = [&](uint64_t s2, int pr, uint64_t x2) {
-        uint64_t p2;
-        if ((pr & 7) < kPoly2) {
-          float x0, x1;
-          unpack2(x2, x0, x1);
-          p2 = exp2_poly2(pack2(fminf(fmaxf(x0, -125.f), 126.f), fminf(fmaxf(x1, -125.f), 126.f)));
-        } else {
-          p2 = exp2_sfu2(x2);
-        }
-        return add2(s2, p2);
-      };
-      // the same sum when the MMA has already subtracted lse / c2: x = c2 * accumulator
-      auto colsum_folded = [&]() {
-        const uint64_t c22 = pack2(p.c2, p.c2), zero2 = pack2(0.f, 0.f);
-        uint64_t s2 = zero2;
-#pragma unroll
-        for (int pr = 0; pr < 16; ++pr) s2 = pair_sum(s2, pr, fma2(pack2(v[2 * pr], v[2 * pr + 1]), c22, zero2));
-        float a, b;
-        unpack2(s2, a, b);
-        return a + b;
-      };
-      auto colsum = [&](int c) {
-        if (p.fold) return colsum_folded();
-        const ulonglong2* l2 = reinterpret_cast<const ulonglong2*>(lse_s + col0 + c * 32);
-        const uint64_t c22 = pack2(p.c2, p.c2);
-        uint64_t s2 = pack2(0.f, 0.f);
-#pragma unroll
-        for (int e4 = 0; e4 < 8; ++e4) {
-          const ulonglong2 l = l2[e4];                      // -lse of rows 4 e4 .. 4 e4 + 3
-#pragma unroll
-          for (int q = 0; q < 2; ++q) {
-            const int pr = 2 * e4 + q;
-            s2 = pair_sum(s2, pr, fma2(pack2(v[2 * pr], v[2 * pr + 1]), c22, q == 0 ? l.x : l.y));
-          }
-        }
-        float a, b;
-        unpack2(s2, a, b);
-        return a + b;
-      };
-      // same for a tile that holds window keys: window row i sees key j only if i >= i_min
-      auto colsum_masked = [&](int c, int i_min) {
-        float s = 0.f;
-#pragma unroll
-        for (int e = 0; e < 32; ++e) {
-          const int i = (row0 + c * 32 + e) % p.window;
-          const float x = fmaf(v[e], p.c2, p.fold ? 0.f : lse_s[col0 + c * 32 + e]);
-          s += (i >= i_min) ? fast_exp2(x) : 0.f;
-        }
-        return s;
-      };
-      for (int t = 0;; ++t) {
-        const int tile = acc_full(t);
-        if (tile < 0) break;
-        const int j = tile * kKeyTile + quarter * 32 + lane;
-        const bool plain = tile < first_tail_tile;
-        const int i_min = j - (n_keys - p.window);        // window rows i < i_min do not see key j
-        const uint32_t taddr = tmem + lane_base + (uint32_t)((t % kAccStages) * 256 + col0);
-        const bool mine = warp_active && (W != 128 || (t & 1) == (sub >> 1));
-        float sc[kChunks];
-#pragma unroll
-        for (int c = 0; c < kChunks; ++c) {
-          sc[c] = 0.f;
-          if (mine) {
-            tmem_ld32(taddr + c * 32, v);
-            tmem_ld_wait(v);
-          }
-          if (c == kChunks - 1) acc_release(t);             // every load of the tile has landed
-          if (mine) sc[c] = plain ? colsum(c) : colsum_masked(c, i_min);
-        }
-        if (mine && j < n_keys) {
-          if (W == 32) {
-            p.cols[(size_t)h0 * p.col_stride + key0 + j] = sc[0] * inv_w;
-            if (row0 + 32 < p.rows_pg) p.cols[(size_t)(h0 + 1) * p.col_stride + key0 + j] = sc[1] * inv_w;
-          } else {
-            float tot = 0.f;
-#pragma unroll
-            for (int c = 0; c < kChunks; ++c) tot += sc[c];
-            p.cols[(size_t)h0 * p.col_stride + key0 + j] = tot * inv_w;
-          }
-        }
-      }
-    }
-    tmem_ld_wait();
-  }
-
-  // ---------------- teardown ----------------
-  tc_fence_before();
-  __syncthreads();
-  if (*abort_flag && threadIdx.x == 0) atomicCAS(p.status, 0, (int)STRUCTKV_ERR_TIMEOUT);
-  // tensor memory is freed only when no MMA of this CTA can still write to it
-  if (warp == 1 && !*mma_in_flight) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
-  }
-}
 
 // Self-test of the bounded wait: one thread waits, with the scorer's own helper, on a barrier
 // that nothing will ever arrive on.  No copy, MMA or tensor-memory allocation is involved, so
@@ -975,51 +27,134 @@ __global__ void wait_expiry_probe(unsigned long long limit_cycles, int* status) 
   }
 }
 
-template <int D, int PASS, int W>
-cudaError_t launch_one(const CUtensorMap& mq, const CUtensorMap& mk, const TcParams& p, int grid,
-                       cudaStream_t st) {
-  auto kern = tc_score<D, PASS, W>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D>::kAlloc);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(grid), dim3(kTcThreads), Smem<D>::kAlloc, st, mq, mk, p);
+bool encode3(const Ctx& ctx, CUtensorMap* m, const void* base, cuuint64_t d1, cuuint64_t d2, cuuint64_t s1,
+             cuuint64_t s2, cuuint32_t b1, cuuint32_t b2) {
+  const cuuint64_t dims[3] = {(cuuint64_t)ctx.cfg.head_dim, d1, d2};
+  const cuuint64_t strides[2] = {s1, s2};
+  const cuuint32_t box[3] = {64, b1, b2}, estr[3] = {1, 1, 1};
+  return ((TcState*)ctx.tc)->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
+                                    estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, int PASS>
-cudaError_t launch_w(int w, const CUtensorMap& mq, const CUtensorMap& mk, const TcParams& p, int grid,
-                     cudaStream_t st) {
-  switch (w) {
-    case 32: return launch_one<D, PASS, 32>(mq, mk, p, grid, st);
-    case 64: return launch_one<D, PASS, 64>(mq, mk, p, grid, st);
-    case 128: return launch_one<D, PASS, 128>(mq, mk, p, grid, st);
+// How a configuration's score rows are laid out and weighted.
+struct Layout {
+  int group, rows_pg, n_rb, units, shape, unit_rows, w_last, w_group, w_total;
+};
+Layout layout_of(const structkv_config& cfg) {
+  Layout l;
+  const int w_pad = tc_window_pad(cfg.window);
+  l.group = cfg.n_q_heads / cfg.n_kv_heads;
+  l.rows_pg = l.group * w_pad;
+  if (l.rows_pg <= 64) {
+    // up to 64 rows the wide layout would leave at least half of the lanes to padding
+    l.unit_rows = l.rows_pg <= 32 ? 32 : 64;
+    l.shape = l.rows_pg <= 32 ? kNarrow32 : kNarrow64;
+  } else {
+    l.unit_rows = kRowBlock;
+    l.shape = w_pad <= 16 ? kWide16 : w_pad == 32 ? kWide32 : w_pad == 64 ? kWide64 : w_pad == 128 ? kWide128 : kWide256;
   }
-  return cudaErrorInvalidValue;
+  l.n_rb = (l.rows_pg + l.unit_rows - 1) / l.unit_rows;
+  l.units = cfg.n_kv_heads * l.n_rb;
+  // equal units need no weights
+  l.w_last = l.n_rb > 1 && l.rows_pg - (l.n_rb - 1) * kRowBlock <= 128 ? 13 : kFullWeight;
+  l.w_group = (l.n_rb - 1) * kFullWeight + l.w_last;
+  l.w_total = cfg.n_kv_heads * l.w_group;
+  return l;
+}
+// Tasks of one pass: about `target`, at least one for every unit, and no more than one per item of a
+// unit.
+int clamp_tasks(const Layout& l, int target, int items) {
+  const int lo = (l.w_total + l.w_last - 1) / l.w_last;
+  const int hi = std::max(lo, (int)std::min(60000ll, (long long)items * l.w_total / kFullWeight));
+  return std::min(std::max(target, lo), hi);
 }
 
-bool encode_maps(const Ctx& ctx, const ScoreArgs& a, CUtensorMap* mq, CUtensorMap* mk) {
-  TcState* s = (TcState*)ctx.tc;
-  const int d = ctx.cfg.head_dim;
-  {
-    cuuint64_t dims[2] = {(cuuint64_t)d, (cuuint64_t)a.batch * ctx.cfg.n_q_heads * ctx.cfg.window};
-    cuuint64_t strides[1] = {(cuuint64_t)d * 2};
-    cuuint32_t box[2] = {64, (cuuint32_t)kRowBlock};
-    cuuint32_t estr[2] = {1, 1};
-    if (s->encode(mq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(a.q), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return false;
+template <int MAXP>
+cudaError_t launch_problems(const Ctx& ctx, const TcCall& a, int first, int n, cudaStream_t st) {
+  TcParams<MAXP> p;
+  const structkv_config& cfg = ctx.cfg;
+  const Layout l = layout_of(cfg);
+  const bool batch = a.cu_seqlens != nullptr;
+  const int sms = std::min(ctx.sm_count, kMaxSms);
+  const int total_keys = batch ? a.cu_seqlens[n] : a.n_keys;
+  const int box_rows = l.unit_rows == kRowBlock ? kRowBlock / 2 : l.unit_rows;    // Q is loaded in halves of a wide block
+  const cuuint64_t row = (cuuint64_t)cfg.head_dim * 2;
+  const int n_maps = batch ? 1 : n;
+  for (int i = 0; i < n_maps; ++i) {
+    if (!encode3(ctx, &p.map_q[i], a.q[first + i], cfg.window, (cuuint64_t)cfg.n_q_heads * (batch ? n : 1), row,
+                 row * cfg.window, std::min(ctx.w_pad, box_rows), std::max(1, box_rows / ctx.w_pad)))
+      return cudaErrorInvalidValue;
+    const cuuint64_t s_tok = (cuuint64_t)a.k_stride_token * 2;
+    const cuuint64_t s_head = cfg.n_kv_heads == 1 ? s_tok * (cuuint64_t)total_keys : (cuuint64_t)a.k_stride_head * 2;
+    if (!encode3(ctx, &p.map_k[i], a.k[first + i], total_keys, cfg.n_kv_heads, s_tok, s_head, kKeyTile, 1))
+      return cudaErrorInvalidValue;
   }
-  {
-    cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)a.total_keys, (cuuint64_t)ctx.cfg.n_kv_heads};
-    cuuint64_t strides[2] = {(cuuint64_t)a.k_stride_token * 2, (cuuint64_t)a.k_stride_head * 2};
-    cuuint32_t box[3] = {64, (cuuint32_t)kKeyTile, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    if (ctx.cfg.n_kv_heads == 1) strides[1] = strides[0] * (cuuint64_t)a.total_keys;
-    if (s->encode(mk, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(a.k), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return false;
+  int part0 = 0;
+  for (int i = 0; i < n; ++i) {
+    TcProblem& pb = p.prob[i];
+    pb.key0 = batch ? a.cu_seqlens[i] : 0;
+    pb.n_keys = batch ? a.cu_seqlens[i + 1] - pb.key0 : a.n_keys;
+    pb.map = batch ? 0 : i;
+    pb.head0 = batch ? i * cfg.n_q_heads : 0;
+    pb.cols = a.cols + (batch ? (size_t)pb.key0 : (size_t)(first + i) * a.cols_layer_stride);
+    const float c2 = (batch ? a.scale[0] : a.scale[first + i]) * kLog2e;
+    pb.negate = c2 < 0.f;
+    pb.c2 = std::max(std::fabs(c2), 1e-30f);
+    pb.inv_c2 = 1.f / pb.c2;
+    pb.v_min = -125.f / pb.c2;
+    const int tiles = (pb.n_keys + kKeyTile - 1) / kKeyTile;
+    // One task per SM and pass, shared out over the sequences of a batch by their lengths; in pass 1 at
+    // least two pairs of tiles a task, which carries 1.5 us of hand-over whatever its size.
+    const int share = batch ? std::max(1, (int)((long long)sms * pb.n_keys / total_keys)) : sms;
+    pb.t1 = clamp_tasks(l, share, (tiles + 3) / 4);
+    // Pass 2 leaves no partial results, so the pass nothing follows is cut finer: its tasks end
+    // closer together.
+    const bool last = batch || i == n - 1;
+    pb.t2 = last ? clamp_tasks(l, 2 * share, tiles) : clamp_tasks(l, share, (tiles + 3) / 4);
+    pb.part0 = part0;
+    part0 += pb.t1;
   }
-  return true;
+  // ticket order
+  int n_ph = 0, tickets = 0;
+  auto phase = [&](int i, int pass) {
+    p.phase[n_ph++] = TcPhase{tickets, 0, (unsigned char)i, (unsigned char)pass};
+    tickets += pass == 1 ? p.prob[i].t1 : p.prob[i].t2;
+  };
+  if (batch) {
+    for (int pass = 1; pass <= 2; ++pass)
+      for (int i = 0; i < n; ++i) phase(i, pass);
+  } else {
+    // Pass 1 runs `ahead` layers in front of pass 2, far enough to cover the way from a unit's last
+    // pass-1 task to its merged statistics (10 to 15 us) with other work: one layer where a layer's
+    // pass 1 is at least eight pairs of key tiles (1.2 us each) per SM, more for shorter sequences.
+    const long long pairs = (long long)l.units * ((p.prob[0].n_keys + 2 * kKeyTile - 1) / (2 * kKeyTile));
+    const int ahead = (int)std::min<long long>(std::min(n - 1, 12), std::max(1ll, (8ll * sms + pairs - 1) / pairs));
+    for (int i = 0; i < n + ahead; ++i) {
+      if (i < n) phase(i, 1);
+      if (i >= ahead) phase(i - ahead, 2);
+    }
+  }
+  p.phase[n_ph] = TcPhase{tickets, 0, 0, 0};
+  p.n_phase = n_ph;
+  p.n_prob = n;
+  p.window = cfg.window;
+  p.w_pad = ctx.w_pad;
+  p.group = l.group;
+  p.rows_pg = l.rows_pg;
+  p.n_rb = l.n_rb;
+  p.n_units = l.units;
+  p.w_group = l.w_group;
+  p.w_total = l.w_total;
+  p.w_last = l.w_last;
+  p.ctl = ctx.ws.ctl;
+  p.part = a.part;
+  p.nlse = a.nlse;
+  p.row_ent = a.row_ent + (size_t)first * ctx.rows_pad;
+  p.col_stride = a.col_stride;
+  p.status = ctx.ws.status;
+  const int grid = std::min(sms, tickets);
+  return cfg.head_dim == 128 ? tc_launch_128(l.shape, p, grid, ctx.device, st) : tc_launch_64(l.shape, p, grid, ctx.device, st);
 }
 
 }  // namespace
@@ -1029,17 +164,25 @@ cudaError_t launch_wait_probe(unsigned long long limit_cycles, int* status, cuda
   return cudaGetLastError();
 }
 
-bool tc_supported(const Ctx& ctx, const ScoreArgs& a) {
+int tc_window_pad(int window) {
+  int w = 8;
+  while (w < window) w *= 2;
+  return w;
+}
+
+size_t tc_part_tasks(const structkv_config& cfg, int n, bool batch) {
+  const size_t units = (size_t)layout_of(cfg).units;
+  const size_t m = (size_t)std::min(n, kMaxBatch);
+  return batch ? kMaxSms + 2 * units * m : (kMaxSms + 2 * units) * m;
+}
+
+bool tc_supported(const Ctx& ctx, long long k_stride_head, long long k_stride_token) {
   if (!ctx.tc || ctx.cfg.dtype != STRUCTKV_BF16) return false;
-  const int w = ctx.cfg.window;
-  if (w != 32 && w != 64 && w != 128) return false;
   if (ctx.cfg.head_dim != 64 && ctx.cfg.head_dim != 128) return false;
   // tensor-map limits: strides below 2^40 bytes, multiples of 16 bytes (checked by the caller)
-  if (a.k_stride_token * 2 >= (1ll << 40) || a.k_stride_head * 2 >= (1ll << 40)) return false;
-  if (ctx.cfg.n_kv_heads > 1 && a.k_stride_head == 0) return false;
-  const int rows_pg = (ctx.cfg.n_q_heads / ctx.cfg.n_kv_heads) * w;
-  if (ctx.cfg.n_kv_heads * ((rows_pg + kRowBlock - 1) / kRowBlock) > kQueueUnits) return false;   // work-queue slots
-  return true;
+  if (k_stride_token * 2 >= (1ll << 40) || k_stride_head * 2 >= (1ll << 40)) return false;
+  if (ctx.cfg.n_kv_heads > 1 && k_stride_head == 0) return false;
+  return layout_of(ctx.cfg).units <= kQueueUnits;
 }
 
 structkv_status tc_create(Ctx& ctx) {
@@ -1059,82 +202,14 @@ void tc_destroy(Ctx& ctx) {
   ctx.tc = nullptr;
 }
 
-cudaError_t launch_score_tc(Ctx& ctx, const ScoreArgs& a, int* parts_out, int pass, cudaStream_t st) {
-  CUtensorMap mq, mk;
-  if (!encode_maps(ctx, a, &mq, &mk)) return cudaErrorInvalidValue;
-  TcParams p;
-  p.window = ctx.cfg.window;
-  p.group = ctx.cfg.n_q_heads / ctx.cfg.n_kv_heads;
-  p.rows_pg = p.group * p.window;
-  p.rows_pg_pad = ctx.rows_pad / ctx.cfg.n_kv_heads;
-  p.rows_pad = ctx.rows_pad;
-  p.n_rb = (p.rows_pg + kRowBlock - 1) / kRowBlock;
-  p.n_seq = a.batch;
-  p.q_rows = ctx.cfg.n_q_heads * ctx.cfg.window;
-  p.rows_all = (long long)a.batch * ctx.rows_pad;
-  // The CTAs of the grid (about one per SM) are shared out over the sequences in proportion to
-  // their lengths, and inside a KV group over its row blocks in proportion to their cost: a last
-  // block that holds a single 128-row half costs half a full block per key tile in pass 1 and
-  // between a half and three quarters in pass 2 (fewer warps share its exponentials), 0.65 over
-  // both.  Every unit gets at least one key segment and at most one per pair of key tiles.
-  const int halves_last = (p.rows_pg - (p.n_rb - 1) * kRowBlock + 127) / 128;       // 1 or 2
-  const double weight_last = halves_last == 2 ? 1.0 : 0.65;
-  const double group_weight = (double)(p.n_rb - 1) + weight_last;
-  int grid = 0, max_segs = 0;
-  for (int b = 0; b < a.batch; ++b) {
-    const int key0 = a.cu_seqlens ? a.cu_seqlens[b] : 0;
-    const int n_b = a.cu_seqlens ? a.cu_seqlens[b + 1] - key0 : a.n_keys;
-    const int n_pairs = ((n_b + kKeyTile - 1) / kKeyTile + 1) / 2;
-    const double per_group = (double)ctx.sm_count * n_b / ((double)a.total_keys * ctx.cfg.n_kv_heads);
-    auto clamp_segs = [&](int v) { return v < 1 ? 1 : (v > n_pairs ? n_pairs : (v > kMaxParts ? kMaxParts : v)); };
-    // pass 1 leaves one partial statistic per segment, hence the bound kMaxParts
-    const int segs = clamp_segs((int)(per_group / group_weight));
-    const int segs_last = p.n_rb == 1 ? segs : clamp_segs((int)(weight_last * segs + 0.5));
-    const unsigned int n_tiles_b = (unsigned int)((n_b + kKeyTile - 1) / kKeyTile);
-    p.seq[b] = SeqDesc{key0, n_b, grid, segs, segs_last, n_tiles_b + (unsigned int)segs, n_tiles_b + (unsigned int)segs_last};
-    grid += ctx.cfg.n_kv_heads * ((p.n_rb - 1) * segs + segs_last);
-    if (segs > max_segs) max_segs = segs;
-    if (segs_last > max_segs) max_segs = segs_last;
+cudaError_t launch_score_tc(const Ctx& ctx, const TcCall& a, cudaStream_t st) {
+  if (a.cu_seqlens) return a.n == 1 ? launch_problems<1>(ctx, a, 0, 1, st) : launch_problems<kMaxBatch>(ctx, a, 0, a.n, st);
+  for (int l = 0; l < a.n; l += kMaxBatch) {
+    const int n = std::min(kMaxBatch, a.n - l);
+    const cudaError_t e = n == 1 ? launch_problems<1>(ctx, a, l, 1, st) : launch_problems<kMaxBatch>(ctx, a, l, n, st);
+    if (e != cudaSuccess) return e;
   }
-  p.c2 = a.scale * kLog2e;
-  // the fold needs a finite lse / c2 (a zero scale keeps the plain form)
-  p.fold = (SKV_FOLD != 0) && pass == 2 && fabsf(p.c2) > 1e-20f ? 1 : 0;
-  p.inputs_ready = a.inputs_ready ? 1 : 0;
-  // tickets of pass 2: a unit's counter advances, per launch, by its tiles plus one failed draw per
-  // CTA of the unit, and tickets are read modulo that number.  A slot whose number changes (another
-  // sequence length) starts again from zero; this is settled before pass 1, so that nothing comes
-  // between the two passes.
-  p.queue = a.queue ? a.queue : ctx.ws.queue;
-  // Two launches must never draw from the same counters at the same time.  With the caller's word
-  // that the inputs are ready, the next layer's kernels may start before this layer's pass 2 has
-  // finished, so the shared counters are used only without that word; a caller that interleaves
-  // layers brings counters of its own for every launch.
-  p.use_tickets = (a.queue != nullptr || !a.inputs_ready) ? 1 : 0;
-  p.done = a.done;
-  p.done_target = (unsigned int)(a.done_round * grid);   // every earlier use of the counter added one per CTA of this grid
-  if (pass == 1 && !a.queue)
-    for (int b = 0; b < a.batch; ++b) {
-      const unsigned int want[2] = {p.seq[b].period, p.seq[b].period_last};
-      const bool stale = (ctx.queue_period[b][0] != 0 && ctx.queue_period[b][0] != want[0]) ||
-                         (ctx.queue_period[b][1] != 0 && ctx.queue_period[b][1] != want[1]);
-      if (stale && cudaMemsetAsync(ctx.ws.queue + (size_t)b * kQueueUnits, 0,
-                                   (size_t)kQueueUnits * sizeof(unsigned long long), st) != cudaSuccess)
-        return cudaErrorUnknown;
-      ctx.queue_period[b][0] = want[0];
-      ctx.queue_period[b][1] = want[1];
-    }
-  p.inv_c2 = p.fold ? 1.0f / p.c2 : 0.f;
-  p.row_part = ctx.ws.row_part;
-  p.row_ent = ctx.ws.row_ent;
-  p.cols = a.cols;
-  p.col_stride = a.col_stride;
-  p.status = ctx.ws.status;
-  *parts_out = max_segs;
-  const int d = ctx.cfg.head_dim, w = ctx.cfg.window;
-  cudaError_t e;
-  if (d == 128) e = pass == 1 ? launch_w<128, 1>(w, mq, mk, p, grid, st) : launch_w<128, 2>(w, mq, mk, p, grid, st);
-  else e = pass == 1 ? launch_w<64, 1>(w, mq, mk, p, grid, st) : launch_w<64, 2>(w, mq, mk, p, grid, st);
-  return e;
+  return cudaSuccess;
 }
 
 }  // namespace skv

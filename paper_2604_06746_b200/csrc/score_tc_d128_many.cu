@@ -1,0 +1,8 @@
+// Tensor-core scorer, head dimension 128, several problems (layers, sequences) per launch.
+#include "score_tc_inst.cuh"
+
+namespace skv {
+cudaError_t tc_launch_128(int shape, const TcParams<kMaxBatch>& p, int grid, int device, cudaStream_t st) {
+  return tc_dispatch<128, kMaxBatch>(shape, p, grid, device, st);
+}
+}  // namespace skv
