@@ -330,15 +330,9 @@ structkv_status structkv_select_batch(structkv_ctx* ctx, const float* scores, co
   }
   cudaStream_t st = (cudaStream_t)stream;
   // padding entries read -1: no prompt ever addresses a batch-mate's tokens
-  if (cudaMemsetAsync(idx_out, 0xff, (size_t)batch * idx_stride * sizeof(int), st) != cudaSuccess)
-    return STRUCTKV_ERR_CUDA;
-  for (int b = 0; b < batch; ++b) {
-    const int key0 = cu_seqlens[b], n_b = cu_seqlens[b + 1] - key0;
-    if (launch_select(scores + key0, 0, 1, n_b, budgets[b], window, idx_out + (size_t)b * idx_stride, st) !=
-        cudaSuccess)
-      return STRUCTKV_ERR_CUDA;
-  }
-  return STRUCTKV_OK;
+  return launch_select_packed(scores, cu_seqlens, budgets, batch, window, idx_out, idx_stride, st) == cudaSuccess
+             ? STRUCTKV_OK
+             : STRUCTKV_ERR_CUDA;
 }
 
 structkv_status structkv_head_stats(structkv_ctx* ctx, const float* head_cols, long long layer_stride,

@@ -118,6 +118,9 @@ cudaError_t launch_accumulate(const float* s_hist, long long row_stride, int piv
 
 cudaError_t launch_select(const float* scores, long long row_stride, int batch, int n, int budget,
                           int window, int* idx_out, cudaStream_t st);
+// The same for packed sequences of different lengths and budgets; rows are padded with -1.
+cudaError_t launch_select_packed(const float* scores, const int* cu_seqlens, const int* budgets, int batch, int window,
+                                 int* idx_out, long long idx_stride, cudaStream_t st);
 
 cudaError_t launch_block_scores(const float* scores, long long row_stride, int batch, int n, int block_size,
                                 float* out, cudaStream_t st);

@@ -1,210 +1,214 @@
 // Budgeted token selection (top-k of the prefix, ties to the lower index, output in position
-// order, window appended).  A cluster of kSelCluster CTAs shares one score vector, each CTA
-// owning a contiguous slice of the prefix.  Three counting sweeps over order-preserving 32-bit
-// keys (11 + 11 + 10 bits) find the k-th largest key exactly: every CTA counts its slice in
-// shared memory (each bin kept kSelCopies times so that a warp's hits on one bin spread), the
-// counts are merged in CTA 0 through distributed shared memory with integer atomics, and every
-// CTA reads the merged counts.  One counting sweep then gives each CTA its output offset and
-// one ordered sweep writes the indices.
-#include <cooperative_groups.h>
+// order, window appended), exact: four eight-bit levels find the k-th largest key (radix.cuh), then every
+// kept token's place in the output follows from ballots and one scan of the counts per (group of
+// 1024 tokens, warp).  A cluster of CL CTAs shares one vector, each CTA a contiguous slice that it
+// holds in registers (up to ITEMS tokens a thread; a longer slice is read again per level).
+//
+// Bound by the chain of barriers, not by memory.  One CTA up to 16384 tokens (no exchange between
+// CTAs), a cluster of eight beyond.
+#include <atomic>
 
-#include "common.cuh"
-
-namespace cg = cooperative_groups;
+#include "radix.cuh"
 
 namespace skv {
 namespace {
 
-constexpr int kSelCluster = 8;
-constexpr int kSelThreads = 1024;
-constexpr int kSelBins = 2048;
-constexpr int kSelCopies = 8;
-constexpr int kSelItems = 4;     // consecutive elements per thread in the output sweep
-constexpr int kSelBatch = 8;     // loads in flight per thread in the counting sweeps
+struct SelectArgs {
+  const float* scores;
+  int* out;
+  long long row_stride, out_stride;    // between the vectors of a uniform call; rows of `out`
+  int n, budget, window, batch;
+  // packed sequences: vector b is scores[cu[b] .. cu[b + 1]) with its own budget; the row's remainder reads -1
+  int packed;
+  int cu[kMaxBatch + 1], budgets[kMaxBatch];
+};
 
-// Larger float -> larger unsigned; -0 is folded onto +0.
-__device__ __forceinline__ unsigned order_key(float v) {
-  const unsigned b = __float_as_uint(v + 0.0f);
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-
-// Shared memory (dynamic): hist[kSelBins][kSelCopies] | merged[3][kSelBins] (one per level).
-__global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kSelThreads)
-select_topk(const float* __restrict__ scores, long long row_stride, int n, int budget, int window,
-            int* __restrict__ idx_out) {
-  extern __shared__ unsigned sel_smem[];
-  unsigned* hist = sel_smem;
-  unsigned* merged = sel_smem + kSelBins * kSelCopies;
-  __shared__ unsigned warp_tot[33];
-  __shared__ unsigned cta_gt[kSelCluster], cta_eq[kSelCluster];
-  __shared__ unsigned sel_bin, sel_rem;
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int vec = blockIdx.x / kSelCluster;
-  const float* s = scores + (size_t)vec * row_stride;
-  int* out = idx_out + (size_t)vec * budget;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, copy = tid & (kSelCopies - 1);
-  const int prefix_len = n - window;
-  const int k = budget - window;
-
-  if (rank == 0)
-    for (int i = tid; i < window; i += kSelThreads) out[k + i] = prefix_len + i;
+template <int CL, int ITEMS>
+__global__ void __launch_bounds__(kRxThreads, ITEMS <= 8 ? 2 : 1) select_topk(const __grid_constant__ SelectArgs a) {
+  extern __shared__ __align__(16) unsigned char sel_smem[];
+  RadixShared<CL>& s = *reinterpret_cast<RadixShared<CL>*>(sel_smem);
+  __shared__ unsigned cta_tot[2][CL];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int rank = CL > 1 ? (int)cg::this_cluster().block_rank() : 0;
+  const int vec = blockIdx.x / CL;
+  pdl_trigger();
+  radix_clear(s, 0);
+  cluster_barrier<CL>();                             // all CTAs of the cluster run before any remote access
+  pdl_wait();
+  const float* x = a.scores + (a.packed ? (size_t)a.cu[vec] : (size_t)vec * a.row_stride);
+  const int n = a.packed ? a.cu[vec + 1] - a.cu[vec] : a.n, budget = a.packed ? a.budgets[vec] : a.budget;
+  int* out = a.out + (size_t)vec * a.out_stride;
+  const int prefix_len = n - a.window, k = budget - a.window;
+  if (rank == 0) {
+    for (int i = tid; i < a.window; i += kRxThreads) out[k + i] = prefix_len + i;
+    if (a.packed)
+      for (long long i = budget + tid; i < a.out_stride; i += kRxThreads) out[i] = -1;
+  }
   if (k <= 0) return;                                // the same decision in every CTA of the cluster
 
-  const int per = (prefix_len + kSelCluster - 1) / kSelCluster;
+  const int per = (prefix_len + CL - 1) / CL;
   const int lo = min(prefix_len, rank * per), hi = min(prefix_len, lo + per);
-  unsigned* merged0 = cluster.map_shared_rank(merged, 0);
-  cluster.sync();                                    // all CTAs of the cluster run before any remote access
-
-  unsigned thr = 0, need_eq = 0xffffffffu;           // threshold key; how many keys equal to it are taken
-  const bool keep_all = k >= prefix_len;             // every prefix token is kept
-  if (!keep_all) {
-    unsigned prefix = 0, prefix_mask = 0, remaining = (unsigned)k;
-    const int shifts[3] = {21, 10, 0};
-    const int widths[3] = {11, 11, 10};
-    for (int b = tid; b < 3 * kSelBins; b += kSelThreads) merged[b] = 0;
-    cluster.sync();                                  // every merged[] is zero before anyone pushes
-    for (int pass = 0; pass < 3; ++pass) {
-      for (int b = tid; b < kSelBins * kSelCopies; b += kSelThreads) hist[b] = 0;
-      __syncthreads();
-      const unsigned bmask = (1u << widths[pass]) - 1u;
-      for (int j0 = lo + tid; j0 < hi; j0 += kSelThreads * kSelBatch) {
-        float val[kSelBatch];
+  constexpr int kChunk = kRxThreads * ITEMS;
+  const int chunks = (per + kChunk - 1) / kChunk;    // more than one: the slice does not fit the registers
+  unsigned key[ITEMS];
+  // token of item e: base + e * 1024 + tid
+  auto load = [&](int c) {
+    const int base = lo + c * kChunk;
+    float v[ITEMS];
 #pragma unroll
-        for (int e = 0; e < kSelBatch; ++e) {
-          const int j = j0 + e * kSelThreads;
-          val[e] = j < hi ? s[j] : 0.f;
-        }
-#pragma unroll
-        for (int e = 0; e < kSelBatch; ++e) {
-          const unsigned u = order_key(val[e]);
-          if (j0 + e * kSelThreads < hi && (u & prefix_mask) == prefix)
-            atomicAdd(&hist[((u >> shifts[pass]) & bmask) * kSelCopies + copy], 1u);
-        }
-      }
-      __syncthreads();
-      unsigned* mlevel = merged + pass * kSelBins;   // bins above 2^width stay zero at the last level
-      for (int b = tid; b < kSelBins; b += kSelThreads) {
-        unsigned c = 0;
-#pragma unroll
-        for (int q = 0; q < kSelCopies; ++q) c += hist[b * kSelCopies + q];
-        if (c) atomicAdd(&merged0[pass * kSelBins + b], c);
-      }
-      cluster.sync();
-      // copy the cluster-wide counts into this CTA (remote reads in parallel), then pick locally
-      if (rank != 0)
-        for (int b = tid; b < kSelBins; b += kSelThreads) mlevel[b] = merged0[pass * kSelBins + b];
-      __syncthreads();
-      block_pick_from_top(mlevel, remaining, warp_tot, &sel_bin, &sel_rem);
-      prefix |= sel_bin << shifts[pass];
-      prefix_mask |= bmask << shifts[pass];
-      remaining = sel_rem;
+    for (int e = 0; e < ITEMS; ++e) {
+      const int j = base + e * kRxThreads + tid;
+      v[e] = j < hi ? x[j] : 0.f;
     }
-    thr = prefix;
-    need_eq = remaining;
+#pragma unroll
+    for (int e = 0; e < ITEMS; ++e) key[e] = order_key(v[e]);
+  };
+  auto valid = [&](int c, int e) { return lo + c * kChunk + e * kRxThreads + tid < hi; };
+
+  if (chunks == 1) load(0);
+  // kept: every key >= ge, and the first need_eq of the keys equal to thr
+  unsigned ge = 0, thr = 0, need_eq = 0;
+  if (k < prefix_len) {
+    unsigned remaining = (unsigned)k;
+    int level = 0;
+#pragma unroll 1
+    for (; level < kRxLevels; ++level) {
+      const int shift = 24 - 8 * level;
+      const unsigned mask = level == 0 ? 0u : 0xffffffffu << (shift + 8);
+      for (int c = 0; c < chunks; ++c) {
+        if (chunks > 1) load(c);
+#pragma unroll
+        for (int e = 0; e < ITEMS; ++e)
+          if (valid(c, e) && (key[e] & mask) == thr) radix_count(s, level & 1, (key[e] >> shift) & 255u);
+      }
+      unsigned digit, in;
+      radix_pick(s, level & 1, remaining, digit, in);
+      thr |= digit << shift;
+      if (in == remaining) break;                    // all keys of the digit are kept: no need to look inside
+    }
+    ge = level < kRxLevels ? thr : thr + 1;
+    need_eq = level < kRxLevels ? 0 : remaining;
   }
 
-  // keys greater than / equal to the threshold in this CTA's slice -> offsets of the slice
-  unsigned my_gt = 0, my_eq = 0;
-  for (int j0 = lo + tid; j0 < hi; j0 += kSelThreads * kSelBatch) {
-    float val[kSelBatch];
-#pragma unroll
-    for (int e = 0; e < kSelBatch; ++e) {
-      const int j = j0 + e * kSelThreads;
-      val[e] = j < hi ? s[j] : 0.f;
-    }
-#pragma unroll
-    for (int e = 0; e < kSelBatch; ++e) {
-      const unsigned u = order_key(val[e]);
-      const bool in = j0 + e * kSelThreads < hi;
-      my_gt += (in && (keep_all || u > thr)) ? 1u : 0u;
-      my_eq += (in && !keep_all && u == thr) ? 1u : 0u;
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    my_gt += __shfl_xor_sync(0xffffffffu, my_gt, o);
-    my_eq += __shfl_xor_sync(0xffffffffu, my_eq, o);
-  }
-  if (lane == 0) warp_tot[warp] = my_gt;
-  __syncthreads();
-  unsigned blk_gt = 0;
-  for (int wv = 0; wv < kSelThreads / 32; ++wv) blk_gt += warp_tot[wv];
-  __syncthreads();
-  if (lane == 0) warp_tot[warp] = my_eq;
-  __syncthreads();
-  unsigned blk_eq = 0;
-  for (int wv = 0; wv < kSelThreads / 32; ++wv) blk_eq += warp_tot[wv];
-  if (tid == 0) {
-    for (int r = 0; r < kSelCluster; ++r) {          // every CTA gets every CTA's totals
-      cluster.map_shared_rank(cta_gt, r)[rank] = blk_gt;
-      cluster.map_shared_rank(cta_eq, r)[rank] = blk_eq;
-    }
-  }
-  cluster.sync();
+  // keys kept outright / equal to the threshold in this CTA's slice -> where the slice starts
   unsigned gt_run = 0, eq_run = 0;
-  for (int r = 0; r < rank; ++r) { gt_run += cta_gt[r]; eq_run += cta_eq[r]; }
-
-  // Ordered sweep.  Position of token j in the output =
-  //   (#keys > thr before j) + min(#keys == thr before j, need_eq).
-  const int chunk = kSelThreads * kSelItems;
-  for (int base = lo; base < hi; base += chunk) {
-    const int j0 = base + tid * kSelItems;
-    unsigned key[kSelItems];
-    unsigned packed = 0;                   // (#gt << 16) | #eq among this thread's items
+  if (CL > 1) {
+    unsigned my_gt = 0, my_eq = 0;
+    for (int c = 0; c < chunks; ++c) {
+      if (chunks > 1) load(c);
 #pragma unroll
-    for (int e = 0; e < kSelItems; ++e) {
-      const int j = j0 + e;
-      const bool in = j < hi;
-      key[e] = in ? order_key(s[j]) : 0u;
-      if (in) packed += (keep_all || key[e] > thr) ? 0x10000u : ((key[e] == thr) ? 1u : 0u);
+      for (int e = 0; e < ITEMS; ++e) {
+        my_gt += valid(c, e) && key[e] >= ge ? 1u : 0u;
+        my_eq += valid(c, e) && key[e] < ge && key[e] == thr ? 1u : 0u;
+      }
     }
-    unsigned incl = packed;
+    my_gt = __reduce_add_sync(0xffffffffu, my_gt);
+    my_eq = __reduce_add_sync(0xffffffffu, my_eq);
+    if (lane == 0) { s.scratch[warp] = my_gt; s.scratch[32 + warp] = my_eq; }
+    __syncthreads();
+    if (warp < 2) {
+      const unsigned t = __reduce_add_sync(0xffffffffu, s.scratch[warp * 32 + lane]);
+      if (lane < CL) cg::this_cluster().map_shared_rank(&cta_tot[0][0], lane)[warp * CL + rank] = t;
+    }
+    cluster_barrier<CL>();
+    for (int r = 0; r < rank; ++r) { gt_run += cta_tot[0][r]; eq_run += cta_tot[1][r]; }
+  }
+
+  // Place of token j in the output = (#kept outright before j) + min(#equal before j, need_eq).
+  unsigned* const cnt = s.scratch;                   // [ITEMS][32 warps] (#outright << 16) | #equal, then exclusive sums
+  unsigned* const tot = s.scratch + kRxThreads;      // [ITEMS]
+  const unsigned below = (1u << lane) - 1u;
+  for (int c = 0; c < chunks; ++c) {
+    if (chunks > 1) load(c);
+    __syncthreads();                                 // scratch is free
+#pragma unroll
+    for (int e = 0; e < ITEMS; ++e) {
+      const bool in = valid(c, e), gt = in && key[e] >= ge, eq = in && !gt && key[e] == thr;
+      const unsigned bg = __ballot_sync(0xffffffffu, gt), be = __ballot_sync(0xffffffffu, eq);
+      if (lane == 0) cnt[e * 32 + warp] = (unsigned)__popc(bg) << 16 | (unsigned)__popc(be);
+    }
+    __syncthreads();
+    if (tid < ITEMS * 32) {                          // warp e scans the warps of item e
+      const unsigned v = cnt[tid];
+      unsigned incl = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      cnt[tid] = incl - v;
+      if (lane == 31) tot[warp] = incl;
+    }
+    __syncthreads();
+    unsigned t_incl = lane < ITEMS ? tot[lane] : 0u;
+    const unsigned t_own = t_incl;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
+      const unsigned t = __shfl_up_sync(0xffffffffu, t_incl, o);
+      if (lane >= o) t_incl += t;
     }
-    __syncthreads();                       // warp_tot reuse across chunks
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    unsigned warp_before = 0, chunk_tot = 0;
-    for (int wv = 0; wv < kSelThreads / 32; ++wv) {
-      const unsigned t = warp_tot[wv];
-      if (wv < warp) warp_before += t;
-      chunk_tot += t;
-    }
-    const unsigned excl = warp_before + incl - packed;
-    unsigned gt_before = gt_run + (excl >> 16), eq_before = eq_run + (excl & 0xffffu);
 #pragma unroll
-    for (int e = 0; e < kSelItems; ++e) {
-      const int j = j0 + e;
-      if (j < hi) {
-        const bool gt = keep_all || key[e] > thr;
-        const bool eq = !gt && key[e] == thr;
-        if (gt || (eq && eq_before < need_eq)) {
-          const unsigned pos = gt_before + (eq_before < need_eq ? eq_before : need_eq);
-          out[pos] = j;
-        }
-        gt_before += gt ? 1u : 0u;
-        eq_before += eq ? 1u : 0u;
-      }
+    for (int e = 0; e < ITEMS; ++e) {
+      const bool in = valid(c, e), gt = in && key[e] >= ge, eq = in && !gt && key[e] == thr;
+      const unsigned bg = __ballot_sync(0xffffffffu, gt), be = __ballot_sync(0xffffffffu, eq);
+      const unsigned before = __shfl_sync(0xffffffffu, t_incl - t_own, e) + cnt[e * 32 + warp];
+      const unsigned gt_before = gt_run + (before >> 16) + __popc(bg & below);
+      const unsigned eq_before = eq_run + (before & 0xffffu) + __popc(be & below);
+      if (gt || (eq && eq_before < need_eq))
+        out[gt_before + min(eq_before, need_eq)] = lo + c * kChunk + e * kRxThreads + tid;
     }
-    gt_run += chunk_tot >> 16;
-    eq_run += chunk_tot & 0xffffu;
+    const unsigned all = __shfl_sync(0xffffffffu, t_incl, 31);
+    gt_run += all >> 16;
+    eq_run += all & 0xffffu;
   }
+}
+
+template <int CL, int ITEMS>
+cudaError_t launch(const SelectArgs& a, cudaStream_t st) {
+  static std::atomic<unsigned long long> ready{0};        // devices whose shared-memory limit has been raised
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (!(ready.load(std::memory_order_acquire) & bit)) {
+    e = cudaFuncSetAttribute(select_topk<CL, ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RadixShared<CL>));
+    if (e != cudaSuccess) return e;
+    ready.fetch_or(bit, std::memory_order_release);
+  }
+  return launch_cluster<CL>(select_topk<CL, ITEMS>, a.batch * CL, sizeof(RadixShared<CL>), st, a);
+}
+
+// Fewest items per thread that hold a slice; beyond 16 x 8192 tokens a slice takes several rounds.
+cudaError_t dispatch(const SelectArgs& a, int longest, cudaStream_t st) {
+  if (longest <= 4 * kRxThreads) return launch<1, 4>(a, st);
+  if (longest <= 16 * kRxThreads) return launch<1, 16>(a, st);
+  if (longest <= 8 * 8 * kRxThreads) return launch<8, 8>(a, st);
+  return launch<8, 16>(a, st);
 }
 
 }  // namespace
 
-cudaError_t launch_select(const float* scores, long long row_stride, int batch, int n, int budget,
-                          int window, int* idx_out, cudaStream_t st) {
-  const int smem = (kSelBins * kSelCopies + 3 * kSelBins) * (int)sizeof(unsigned);
-  cudaError_t e = cudaFuncSetAttribute(select_topk, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
-  select_topk<<<batch * kSelCluster, kSelThreads, smem, st>>>(scores, row_stride, n, budget, window,
-                                                             idx_out);
-  return cudaGetLastError();
+cudaError_t launch_select(const float* scores, long long row_stride, int batch, int n, int budget, int window,
+                          int* idx_out, cudaStream_t st) {
+  SelectArgs a;
+  a.scores = scores; a.out = idx_out; a.row_stride = row_stride; a.out_stride = budget;
+  a.n = n; a.budget = budget; a.window = window; a.batch = batch; a.packed = 0;
+  return dispatch(a, n - window, st);
+}
+
+cudaError_t launch_select_packed(const float* scores, const int* cu_seqlens, const int* budgets, int batch, int window,
+                                 int* idx_out, long long idx_stride, cudaStream_t st) {
+  SelectArgs a;
+  a.scores = scores; a.out = idx_out; a.row_stride = 0; a.out_stride = idx_stride;
+  a.n = a.budget = 0; a.window = window; a.batch = batch; a.packed = 1;
+  int longest = 0;
+  a.cu[0] = cu_seqlens[0];
+  for (int b = 0; b < batch; ++b) {
+    a.cu[b + 1] = cu_seqlens[b + 1];
+    a.budgets[b] = budgets[b];
+    longest = cu_seqlens[b + 1] - cu_seqlens[b] - window > longest ? cu_seqlens[b + 1] - cu_seqlens[b] - window : longest;
+  }
+  return dispatch(a, longest, st);
 }
 
 }  // namespace skv
