@@ -45,7 +45,11 @@ Workspace carve_workspace(const structkv_config& cfg, void* base) {
   const size_t rows_pad = (size_t)rows_pad_of(cfg);
   const size_t n_pad = align_up((size_t)cfg.max_seq, kKeyTile);
   w.status = (int*)take(256);
-  w.ctl = (int*)take(kCtlInts * sizeof(int));                  // follows the status block: one memset
+  // everything that starts from zero comes first: one memset
+  w.ctl = (int*)take(kCtlInts * sizeof(int));
+  w.stat_ctr = (int*)take(kMaxStatLayers * sizeof(int));
+  w.chunk_ctr = (int*)take(n_pad / kKeyTile * sizeof(int));
+  w.zero_bytes = off;
   w.row_part = (float4*)take(std::max((size_t)kSimtParts * rows_pad * sizeof(float4),
                                       tc_part_tasks(cfg, 1, false) * kRowBlock * sizeof(float2)));
   w.row_lse2 = (float*)take(rows_pad * sizeof(float));
@@ -55,9 +59,6 @@ Workspace carve_workspace(const structkv_config& cfg, void* base) {
   w.bytes = off;
   return w;
 }
-
-// the status block and the control block behind it start from zero
-constexpr size_t kZeroBytes = 256 + kCtlInts * sizeof(int);
 
 }  // namespace skv
 
@@ -105,7 +106,7 @@ structkv_status structkv_create(structkv_ctx** ctx_out, const structkv_config* c
   c.tc = nullptr;
   if (cudaGetDevice(&c.device) != cudaSuccess ||
       cudaDeviceGetAttribute(&c.sm_count, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess ||
-      cudaMemset(c.ws.status, 0, kZeroBytes) != cudaSuccess ||
+      cudaMemset(c.ws.status, 0, c.ws.zero_bytes) != cudaSuccess ||
       cudaDeviceSynchronize() != cudaSuccess) {
     delete ctx;
     return STRUCTKV_ERR_CUDA;
@@ -158,8 +159,8 @@ structkv_status structkv_score_layer(structkv_ctx* ctx, const void* q_window, co
         launch_score_simt(c, a, &parts, 2, st) != cudaSuccess)
       return STRUCTKV_ERR_CUDA;
   }
-  return launch_reduce_finish(c, cols, col_stride, n_keys, lambda, s_out, c_inout, !(flags & STRUCTKV_FLAG_NO_HEAD_STATS),
-                              metrics_out, st) == cudaSuccess ? STRUCTKV_OK : STRUCTKV_ERR_CUDA;
+  return launch_finish_layers(c, cols, 0, col_stride, n_keys, 1, lambda, s_out, 0, c_inout, c.ws.row_ent,
+                              !(flags & STRUCTKV_FLAG_NO_HEAD_STATS), metrics_out, st) == cudaSuccess ? STRUCTKV_OK : STRUCTKV_ERR_CUDA;
 }
 
 // ---- batches of prompts of different lengths (packed along the token axis) ------------------
@@ -227,18 +228,10 @@ structkv_status structkv_score_layer_batch(structkv_ctx* ctx, const void* q_wind
   const TcCall a{batch, &q_window, &k, &scale, cu_seqlens, k_stride_head, k_stride_token, 0, cols, 0, col_stride,
                  bw.row_part, bw.nlse, bw.row_ent};
   if (launch_score_tc(c, a, st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
-  // per sequence: S = sum over heads, C <- lambda C + S, and the sequence's metric triple
-  for (int b = 0; b < batch; ++b) {
-    const int key0 = cu_seqlens[b], n_b = cu_seqlens[b + 1] - key0;
-    Ctx one = c;
-    one.ws.row_ent = bw.row_ent + (size_t)b * c.rows_pad;
-    one.ws.head_part = bw.head_part + (size_t)b * cfg.n_q_heads * 4;
-    if (launch_reduce_finish(one, cols + key0, col_stride, n_b, lambda, s_out + key0,
-                             c_inout ? c_inout + key0 : nullptr, !(flags & STRUCTKV_FLAG_NO_HEAD_STATS),
-                             metrics_out + 3 * b, st) != cudaSuccess)
-      return STRUCTKV_ERR_CUDA;
-  }
-  return STRUCTKV_OK;
+  return launch_finish_packed(c, cols, col_stride, cu_seqlens, batch, lambda, s_out, c_inout, bw.row_ent, bw.head_part,
+                              !(flags & STRUCTKV_FLAG_NO_HEAD_STATS), metrics_out, st) == cudaSuccess
+             ? STRUCTKV_OK
+             : STRUCTKV_ERR_CUDA;
 }
 
 // ---- several resident layers in one call, the passes of neighbouring layers interleaved ---------
@@ -312,8 +305,8 @@ structkv_status structkv_score_layers(structkv_ctx* ctx, int n_layers, const voi
   const TcCall a{n_layers, q_windows, ks, scales, nullptr, k_stride_head, k_stride_token, n_keys, head_cols_out,
                  head_cols_layer_stride, n_keys, lw.row_part, lw.nlse, lw.row_ent};
   if (launch_score_tc(c, a, st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
-  return launch_reduce_layers(c, head_cols_out, head_cols_layer_stride, n_keys, n_keys, n_layers, lambda, s_out,
-                              s_layer_stride, c_inout, lw.row_ent, metrics_out, st) == cudaSuccess
+  return launch_finish_layers(c, head_cols_out, head_cols_layer_stride, n_keys, n_keys, n_layers, lambda, s_out,
+                              s_layer_stride, c_inout, lw.row_ent, false, metrics_out, st) == cudaSuccess
              ? STRUCTKV_OK
              : STRUCTKV_ERR_CUDA;
 }
@@ -498,7 +491,7 @@ structkv_status structkv_poll_device_status(structkv_ctx* ctx, void* stream) {
     return STRUCTKV_ERR_CUDA;
   if (word != 0) {
     // a scorer launch that gave up may have left its counters behind: start them over as well
-    if (cudaMemsetAsync(ctx->c.ws.status, 0, kZeroBytes, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
+    if (cudaMemsetAsync(ctx->c.ws.status, 0, ctx->c.ws.zero_bytes, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
       return STRUCTKV_ERR_CUDA;
   }
   if (word < 0 || word > (int)STRUCTKV_ERR_TIMEOUT) return STRUCTKV_ERR_CUDA;
@@ -576,7 +569,7 @@ extern "C" structkv_status structkv_score_layer_static(
   c.n_pad = (int)align_up((size_t)cfg->max_seq, kKeyTile);
   c.tc = cfg->dtype == STRUCTKV_BF16 ? slot->tc : nullptr;
   // The scratch keeps the previous call's contents; the status word and the scorer's counters start from zero.
-  if (cudaMemsetAsync(c.ws.status, 0, kZeroBytes, (cudaStream_t)stream) != cudaSuccess) return STRUCTKV_ERR_CUDA;
+  if (cudaMemsetAsync(c.ws.status, 0, c.ws.zero_bytes, (cudaStream_t)stream) != cudaSuccess) return STRUCTKV_ERR_CUDA;
   return structkv_score_layer(&tmp, q_window, k, k_stride_head, k_stride_token, n_keys, scale, lambda,
                               s_out, c_inout, head_cols_out, metrics_out, flags, stream);
 }

@@ -31,6 +31,9 @@ struct Workspace {
   float* row_ent;       // [rows_pad] entropy of each score row (nats), 0 where there is no row
   float* cols;          // [H][n_pad] pooled per-head attention when the caller passes none
   float* head_part;     // [kMaxStatLayers][H][4] per-(layer, head) {sum of squared deviations from 1/n, top-k mass}
+  int* stat_ctr;        // [kMaxStatLayers] and, behind it, chunk_ctr [n_pad / kKeyTile]: zero between launches
+  int* chunk_ctr;
+  size_t zero_bytes;    // from `status` on: what starts from zero
   size_t bytes;
 };
 
@@ -97,17 +100,16 @@ cudaError_t launch_wait_probe(unsigned long long limit_cycles, int* status, cuda
 // Merges the per-segment softmax statistics of every row into row_lse2 / row_ent (CUDA-core scorer).
 cudaError_t launch_finalize_rows(const Ctx& ctx, int parts, cudaStream_t st);
 
-// S_j = sum_h cols[h][j]; optional C <- lambda C + S; then the layer's metrics: metrics[0] from
-// row_ent (Eq. 4); metrics[1..2] from the pooled per-head attention (Eq. 5-6, computed here when
-// with_head_stats), or NaN.
-cudaError_t launch_reduce_finish(const Ctx& ctx, const float* cols, long long col_stride, int n, float lambda,
-                                 float* s_out, float* c_inout, bool with_head_stats, float* metrics,
-                                 cudaStream_t st);
-// The same for n_layers layers in one launch: S^(l) rows s_stride apart, C carried from layer to
-// layer, entropies from row_ent[l][rows_pad]; metrics [n_layers][3] with NaN for sparsity / variance.
-cudaError_t launch_reduce_layers(const Ctx& ctx, const float* cols, long long layer_stride, long long col_stride,
-                                 int n, int n_layers, float lambda, float* s_out, long long s_stride,
-                                 float* c_inout, const float* row_ent, float* metrics, cudaStream_t st);
+// After the scorer passes of n_layers layers: S^(l)_j = sum_h cols[l][h][j] (rows s_stride apart), C <-
+// lambda C + S^(l) carried from layer to layer if c_inout, metrics[l][0] from row_ent[l][rows_pad] (Eq. 4) and
+// metrics[l][1..2] from the pooled per-head attention (Eq. 5-6) or NaN.
+cudaError_t launch_finish_layers(const Ctx& ctx, const float* cols, long long layer_stride, long long col_stride, int n,
+                                 int n_layers, float lambda, float* s_out, long long s_stride, float* c_inout,
+                                 const float* row_ent, bool with_head_stats, float* metrics, cudaStream_t st);
+// The same for the sequences of a packed batch (sequence b at column cu_seqlens[b] of cols, s_out and c_inout).
+cudaError_t launch_finish_packed(const Ctx& ctx, const float* cols, long long col_stride, const int* cu_seqlens, int batch,
+                                 float lambda, float* s_out, float* c_inout, const float* row_ent, float* head_part,
+                                 bool with_head_stats, float* metrics, cudaStream_t st);
 
 // Eq. 5-6 for n_layers layers at once from their pooled per-head attention: writes metrics[l][1..2].
 cudaError_t launch_head_stats_batch(const Ctx& ctx, const float* cols, long long layer_stride, long long col_stride,
@@ -166,33 +168,6 @@ __device__ __forceinline__ float fast_exp2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-
-// Called by all threads of a 1024-thread block after a histogram pass over `nb` = 2048 bins.
-// Walks the bins from the top and finds the bin holding the `remaining`-th largest candidate;
-// writes that bin and the rank still wanted inside it.  `scratch` holds 33 words.
-__device__ __forceinline__ void block_pick_from_top(const unsigned* hist, unsigned remaining,
-                                                    unsigned* scratch, unsigned* sel_bin, unsigned* sel_rem) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int b_hi = 2047 - 2 * tid, b_lo = b_hi - 1;        // this thread's two bins, higher first
-  const unsigned c_hi = hist[b_hi], c_lo = hist[b_lo];
-  const unsigned mine = c_hi + c_lo;
-  unsigned incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  __syncthreads();
-  if (lane == 31) scratch[warp] = incl;
-  __syncthreads();
-  unsigned before = incl - mine;
-  for (int w = 0; w < warp; ++w) before += scratch[w];
-  if (before < remaining && remaining <= before + mine) {
-    if (before + c_hi >= remaining) { *sel_bin = (unsigned)b_hi; *sel_rem = remaining - before; }
-    else { *sel_bin = (unsigned)b_lo; *sel_rem = remaining - before - c_hi; }
-  }
-  __syncthreads();
 }
 
 }  // namespace skv

@@ -1,31 +1,12 @@
-// Small deterministic reductions around the scorers: row finalisation (log-sum-exp, entropy),
-// column reduction over heads with the centrality update, per-head sparsity / variance, and
+// Small deterministic reductions around the scorers: row finalisation (CUDA-core scorer), the sum
+// over heads with the centrality update, per-head sparsity / variance with the layer's metrics, and
 // the closed-form centrality re-accumulation.
-#include <cooperative_groups.h>
+#include <atomic>
 
-#include "common.cuh"
-
-namespace cg = cooperative_groups;
+#include "radix.cuh"
 
 namespace skv {
 namespace {
-
-__device__ __forceinline__ float block_sum_1024(float v, float* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  if (warp == 0) {
-    float x = (lane < (int)(blockDim.x >> 5)) ? red[lane] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    if (lane == 0) red[32] = x;
-  }
-  __syncthreads();
-  return red[32];
-}
 
 // One thread per score row.  Row r of group g is valid iff its index inside the group is
 // < rows_pg.  Each of the `parts` key segments left (ref, Z, U) for the row: Z = sum 2^(x - ref),
@@ -66,173 +47,279 @@ finalize_rows(const float4* __restrict__ row_part, int parts, int rows_pad, int 
   row_ent[r] = ent;
 }
 
-// S_j = sum over heads (fixed order) of cols[h][j];  C_j <- lambda C_j + S_j  (Eq. 2, Eq. 3).
-// Four keys per thread where the layout allows 16-byte accesses.  NOTE: the order in which heads
-// are added differs between the two instantiations (grouped vs. sequential).  Block 0 also finishes the
-// layer's metrics: metrics[0] = mean entropy of the valid score rows (Eq. 4); metrics[1] = mean
-// over heads of the top-mass (Eq. 5), metrics[2] = mean over heads of (sum of squared deviations
-// from 1/n) / n (Eq. 6), both from head_part, or NaN when head statistics are not computed here.
-// Fixed summation order throughout.
-constexpr int kRcThreads = 256;
-template <int VEC>
-__global__ void __launch_bounds__(kRcThreads)
-reduce_finish(const float* __restrict__ cols, long long col_stride, int H, int n, float lambda,
-              float* __restrict__ s_out, float* __restrict__ c_inout, const float* __restrict__ row_ent,
-              int rows_pad, int n_valid, const float* __restrict__ head_part,
-              int with_head_stats, float* __restrict__ metrics) {
-  __shared__ float red[33];
-  pdl_trigger();
-  pdl_wait();
-  if (VEC == 4) {
-    // 64 threads along the keys (four keys each) x 4 groups of heads: four times the loads in
-    // flight; the groups' partial sums are added in group order (fixed order, deterministic)
-    __shared__ float4 part[3][64];
-    const int lane_j = threadIdx.x & 63, grp = threadIdx.x >> 6;
-    const int j4 = (blockIdx.x * 64 + lane_j) * 4;
-    const int h_per = (H + 3) / 4, h_lo = grp * h_per, h_hi = min(H, h_lo + h_per);
-    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (j4 < n) {                                  // n is a multiple of 4 in this instantiation
-#pragma unroll 4
-      for (int h = h_lo; h < h_hi; ++h) {
-        const float4 v = *reinterpret_cast<const float4*>(cols + (size_t)h * col_stride + j4);
-        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-      }
-    }
-    if (grp > 0) part[grp - 1][lane_j] = s;
-    __syncthreads();
-    if (grp == 0 && j4 < n) {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const float4 o = part[k][lane_j];
-        s.x += o.x; s.y += o.y; s.z += o.z; s.w += o.w;
-      }
-      *reinterpret_cast<float4*>(s_out + j4) = s;
-      if (c_inout) {
-        float4 c = *reinterpret_cast<const float4*>(c_inout + j4);
-        c.x = fmaf(lambda, c.x, s.x); c.y = fmaf(lambda, c.y, s.y);
-        c.z = fmaf(lambda, c.z, s.z); c.w = fmaf(lambda, c.w, s.w);
-        *reinterpret_cast<float4*>(c_inout + j4) = c;
-      }
-    }
-  } else if (blockIdx.x * kRcThreads + threadIdx.x < n) {
-    const int j = blockIdx.x * kRcThreads + threadIdx.x;
-    float s = 0.f;
-    for (int h = 0; h < H; ++h) s += cols[(size_t)h * col_stride + j];
-    s_out[j] = s;
-    if (c_inout) c_inout[j] = fmaf(lambda, c_inout[j], s);
-  }
-  if (blockIdx.x != 0) return;
-  float ent = 0.f;
-  for (int r = threadIdx.x; r < rows_pad; r += kRcThreads) ent += row_ent[r];
-  const float tot = block_sum_1024(ent, red);
-  if (threadIdx.x != 0) return;
-  metrics[0] = tot / (float)n_valid;
-  if (!with_head_stats) {
-    metrics[1] = __int_as_float(0x7fc00000);
-    metrics[2] = __int_as_float(0x7fc00000);
-    return;
-  }
-  float rho = 0.f, var = 0.f;
-  const float inv_n = 1.f / (float)n;
-  for (int h = 0; h < H; ++h) {
-    rho += head_part[h * 4 + 1];
-    var += head_part[h * 4 + 0] * inv_n;
-  }
-  metrics[1] = rho / (float)H;
-  metrics[2] = var / (float)H;
+// ---- what follows the scorer passes of a layer, of several layers or of a packed batch ----------
+// One launch: CTAs of clusters first (one cluster per (problem, head) vector, Eq. 5-6), then blocks
+// that sum 128 x VEC keys over the heads (Eq. 2) and carry the centrality (Eq. 3).  Every sum has a
+// fixed order.
+struct FinishArgs {
+  const float* cols;                   // problem p, head h, key j at cols + p * layer_stride + h * col_stride + j
+  long long layer_stride, col_stride;
+  int H, n, n_prob;
+  float lambda;
+  float* s_out;                        // problem p at s_out + p * s_stride
+  long long s_stride;
+  float* c_inout;                      // layers: one vector carried through them; packed: at s_out's offsets
+  const float* row_ent;                // [n_prob][rows_pad], or NULL: no entropy, no sums
+  int rows_pad, n_valid;
+  float* metrics;                      // [n_prob][3]
+  float* head_part;                    // [n_prob][H][4]
+  int with_stats, n_stat_ctas, chunks; // chunks: key ranges a problem's sum is cut into
+  int* stat_ctr;                       // [n_prob] heads done; zero between launches
+  int* chunk_ctr;                      // [chunks] layers done; zero between launches
+  int packed;                          // sequences of one layer: problem p owns columns [cu[p], cu[p + 1])
+  int cu[kMaxBatch + 1];
+};
+constexpr int kSumLanes = 128, kSumGroups = 8;
+
+struct Problem { const float* cols; float* s; int n; };
+__device__ __forceinline__ Problem problem_of(const FinishArgs& a, int p) {
+  if (a.packed) return {a.cols + a.cu[p], a.s_out + a.cu[p], a.cu[p + 1] - a.cu[p]};
+  return {a.cols + (size_t)p * a.layer_stride, a.s_out + (size_t)p * a.s_stride, a.n};
 }
 
-// reduce_finish for several layers at once (the layers' scorer passes have all run): per layer l
-// S^(l) = sum over heads, in reduce_finish's order, C <- lambda C + S^(l) carried in registers from
-// layer to layer, and, in block l, the layer's entropy; sparsity and variance are left as NaN
-// (they come from head_stats).  Every bit equals what a chain of reduce_finish launches gives.
-template <int VEC>
-__global__ void __launch_bounds__(kRcThreads)
-reduce_layers(const float* __restrict__ cols, long long layer_stride, long long col_stride, int H, int n,
-              int n_layers, float lambda, float* __restrict__ s_out, long long s_stride,
-              float* __restrict__ c_inout, const float* __restrict__ row_ent, int rows_pad,
-              int n_valid, float* __restrict__ metrics) {
-  __shared__ float red[33];
-  pdl_trigger();
-  pdl_wait();
-  if (VEC == 4) {
-    __shared__ float4 part[3][64];
-    const int lane_j = threadIdx.x & 63, grp = threadIdx.x >> 6;
-    const int j4 = (blockIdx.x * 64 + lane_j) * 4;
-    const int h_per = (H + 3) / 4, h_lo = grp * h_per, h_hi = min(H, h_lo + h_per);
-    float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (grp == 0 && j4 < n && c_inout) c = *reinterpret_cast<const float4*>(c_inout + j4);
-    for (int l = 0; l < n_layers; ++l) {
-      const float* cl = cols + (size_t)l * layer_stride;
-      float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (j4 < n) {
+// Sum of v over the block, in every thread of warp 0 (fixed order).
+__device__ __forceinline__ float block_total(float v, float* red) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) red[warp] = v;
+  __syncthreads();
+  if (warp == 0) {
+    v = red[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  }
+  return v;
+}
+
+template <int VEC> struct Keys;
+template <> struct Keys<4> { using T = float4; };
+template <> struct Keys<1> { using T = float; };
+__device__ __forceinline__ void add_to(float4& s, const float4& v) { s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
+__device__ __forceinline__ void add_to(float& s, float v) { s += v; }
+__device__ __forceinline__ float4 decay(float l, const float4& c, const float4& s) {
+  return make_float4(fmaf(l, c.x, s.x), fmaf(l, c.y, s.y), fmaf(l, c.z, s.z), fmaf(l, c.w, s.w));
+}
+__device__ __forceinline__ float decay(float l, float c, float s) { return fmaf(l, c, s); }
+
+// Keys [chunk * 128 * VEC, ...) of problem p: eight groups of heads side by side (one chain of H loads
+// took 9 us), their sums added in group order.  The centrality of several layers is a recursion over
+// them: the block that completes a key range takes all of its layers.
+// THREADS: each row of 128 threads takes kSumGroups * 128 / THREADS of the groups.
+template <int VEC, int THREADS>
+__device__ __forceinline__ void sum_block(const FinishArgs& a, int p, int chunk) {
+  using T = typename Keys<VEC>::T;
+  __shared__ T part[kSumGroups - 1][kSumLanes];
+  __shared__ float red[32];
+  __shared__ int last;
+  const Problem pb = problem_of(a, p);
+  constexpr int kRows = THREADS / kSumLanes, kMine = kSumGroups / kRows;
+  const int lane_j = threadIdx.x & (kSumLanes - 1), grp = threadIdx.x / kSumLanes;
+  const int j = (chunk * kSumLanes + lane_j) * VEC;    // VEC 4: every problem's n is a multiple of 4
+  const int h_per = (a.H + kSumGroups - 1) / kSumGroups;
+  T s{};
+#pragma unroll
+  for (int m = 0; m < kMine; ++m) {
+    const int gr = grp + m * kRows, h_lo = min(a.H, gr * h_per), h_hi = min(a.H, h_lo + h_per);
+    T t{};
+    if (j < pb.n) {
 #pragma unroll 4
-        for (int h = h_lo; h < h_hi; ++h) {
-          const float4 v = *reinterpret_cast<const float4*>(cl + (size_t)h * col_stride + j4);
-          s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-        }
-      }
-      if (grp > 0) part[grp - 1][lane_j] = s;
+      for (int h = h_lo; h < h_hi; ++h) add_to(t, *reinterpret_cast<const T*>(pb.cols + (size_t)h * a.col_stride + j));
+    }
+    if (gr == 0) s = t;
+    else part[gr - 1][lane_j] = t;
+  }
+  __syncthreads();
+  if (grp == 0 && j < pb.n) {
+#pragma unroll
+    for (int k = 0; k < kSumGroups - 1; ++k) add_to(s, part[k][lane_j]);
+    *reinterpret_cast<T*>(pb.s + j) = s;
+  }
+  if (a.c_inout) {
+    const bool chained = !a.packed && a.n_prob > 1;
+    T* c = reinterpret_cast<T*>(a.c_inout + (a.packed ? a.cu[p] : 0) + j);
+    if (!chained) {
+      if (grp == 0 && j < pb.n) *c = decay(a.lambda, *c, s);
+    } else {
+      __threadfence();
       __syncthreads();
-      if (grp == 0 && j4 < n) {
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const float4 o = part[k][lane_j];
-          s.x += o.x; s.y += o.y; s.z += o.z; s.w += o.w;
+      if (threadIdx.x == 0) last = atomicAdd(&a.chunk_ctr[chunk], 1) == a.n_prob - 1;
+      __syncthreads();
+      if (last) {
+        __threadfence();
+        if (grp == 0 && j < pb.n) {
+          T acc = *c;
+#pragma unroll 8
+          for (int l = 0; l < a.n_prob; ++l)
+            acc = decay(a.lambda, acc, __ldcg(reinterpret_cast<const T*>(a.s_out + (size_t)l * a.s_stride + j)));
+          *c = acc;
         }
-        *reinterpret_cast<float4*>(s_out + (size_t)l * s_stride + j4) = s;
-        c.x = fmaf(lambda, c.x, s.x); c.y = fmaf(lambda, c.y, s.y);
-        c.z = fmaf(lambda, c.z, s.z); c.w = fmaf(lambda, c.w, s.w);
+        if (threadIdx.x == 0) a.chunk_ctr[chunk] = 0;
       }
-      __syncthreads();                               // part[] is reused by the next layer
     }
-    if (grp == 0 && j4 < n && c_inout) *reinterpret_cast<float4*>(c_inout + j4) = c;
-  } else if (blockIdx.x * kRcThreads + threadIdx.x < n) {
-    const int j = blockIdx.x * kRcThreads + threadIdx.x;
-    float c = c_inout ? c_inout[j] : 0.f;
-    for (int l = 0; l < n_layers; ++l) {
-      const float* cl = cols + (size_t)l * layer_stride;
-      float s = 0.f;
-      for (int h = 0; h < H; ++h) s += cl[(size_t)h * col_stride + j];
-      s_out[(size_t)l * s_stride + j] = s;
-      c = fmaf(lambda, c, s);
-    }
-    if (c_inout) c_inout[j] = c;
   }
-  // blocks walk over the layers for the entropies (there may be fewer blocks than layers)
-  for (int l = blockIdx.x; l < n_layers; l += gridDim.x) {
-    float ent = 0.f;
-    for (int r = threadIdx.x; r < rows_pad; r += kRcThreads) ent += row_ent[(size_t)l * rows_pad + r];
-    const float tot = block_sum_1024(ent, red);
-    if (threadIdx.x == 0) {
-      metrics[l * 3 + 0] = tot / (float)n_valid;
-      metrics[l * 3 + 1] = __int_as_float(0x7fc00000);
-      metrics[l * 3 + 2] = __int_as_float(0x7fc00000);
-    }
-    __syncthreads();
+  if (chunk != 0) return;
+  // the problem's entropy (Eq. 4); rows that do not exist hold 0
+  float ent = 0.f;
+  // (the same partial sums whatever the block size: thread t of 1024 takes rows t, t + 1024, ...)
+  for (int t = threadIdx.x; t < kRxThreads; t += THREADS) {
+    float e = 0.f;
+    for (int r = t; r < a.rows_pad; r += kRxThreads) e += a.row_ent[(size_t)p * a.rows_pad + r];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if ((t & 31) == 0) red[t >> 5] = e;
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    ent = red[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ent += __shfl_xor_sync(0xffffffffu, ent, o);
+  }
+  if (threadIdx.x == 0) {
+    a.metrics[p * 3] = ent / (float)a.n_valid;
+    if (!a.with_stats) a.metrics[p * 3 + 1] = a.metrics[p * 3 + 2] = __int_as_float(0x7fc00000);
   }
 }
 
-// Per head: sum of squared deviations from 1/n (Eq. 6: the pooled vector sums to 1, so 1/n is its
-// mean; summing deviations instead of squares keeps near-uniform attention from cancelling) and
-// the mass of the k_rho largest entries (Eq. 5) of the pooled attention vector.  A cluster of
-// CL CTAs shares one head; each CTA owns a slice of the keys.  All entries are >= 0, so the
-// unsigned order of the fp32 bit patterns is the order of the values.  Two counting sweeps locate the k_rho-th largest value to 22 bits
-// (histograms are merged in CTA 0 of the cluster through distributed shared memory with
-// integer atomics, so the result does not depend on arrival order):
+// Eq. 5 and 6 of one (problem, head) vector, by a cluster: the sum of squared deviations from 1/n (the
+// pooled vector sums to 1, so 1/n is its mean; summing deviations instead of squares keeps
+// near-uniform attention from cancelling) and the mass of the floor(n / 10) largest entries.  Three
+// radix levels give the threshold to 24 bits; of the entries that share them, the ones still wanted
+// count with their average.  All entries are >= 0: the order of the bit patterns is theirs.
+template <int CL, int ITEMS>
+__device__ __forceinline__ void stats_cta(const FinishArgs& a, RadixShared<CL>& s, int vec) {
+  const int tid = threadIdx.x;
+  const int rank = CL > 1 ? (int)cg::this_cluster().block_rank() : 0;
+  const int p = vec / a.H;
+  const Problem pb = problem_of(a, p);
+  const float* x = pb.cols + (size_t)(vec - p * a.H) * a.col_stride;
+  const int n = pb.n, per = (n + CL - 1) / CL, lo = min(n, rank * per), hi = min(n, lo + per);
+  constexpr int kChunk = kRxThreads * ITEMS;
+  const int chunks = (per + kChunk - 1) / kChunk;
+  unsigned key[ITEMS];
+  auto load = [&](int c) {
+#pragma unroll
+    for (int e = 0; e < ITEMS; ++e) {
+      const int j = lo + c * kChunk + e * kRxThreads + tid;
+      key[e] = j < hi ? __float_as_uint(x[j] + 0.f) : 0x80000000u;   // sign bit: no entry (-0 becomes +0)
+    }
+  };
+  const float mean = 1.f / (float)n;
+  float sq = 0.f;
+  unsigned remaining = (unsigned)max(1, n / 10), thr = 0, in = 0;
+#pragma unroll 1
+  for (int level = 0; level < 3; ++level) {
+    const int shift = 24 - 8 * level;
+    const unsigned mask = level == 0 ? 0x80000000u : 0xffffffffu << (shift + 8);
+    for (int c = 0; c < chunks; ++c) {
+      if (chunks > 1 || level == 0) load(c);
+#pragma unroll
+      for (int e = 0; e < ITEMS; ++e) {
+        if (level == 0 && !(key[e] >> 31)) {
+          const float dv = __uint_as_float(key[e]) - mean;
+          sq = fmaf(dv, dv, sq);
+        }
+        if ((key[e] & mask) == thr) radix_count(s, level & 1, (key[e] >> shift) & 255u);
+      }
+    }
+    unsigned digit;
+    radix_pick(s, level & 1, remaining, digit, in);
+    thr |= digit << shift;
+  }
+  float above = 0.f, inside = 0.f;
+  for (int c = 0; c < chunks; ++c) {
+    if (chunks > 1) load(c);
+#pragma unroll
+    for (int e = 0; e < ITEMS; ++e) {
+      const unsigned top = key[e] & 0xffffff00u;
+      if (!(key[e] >> 31)) {
+        if (top > thr) above += __uint_as_float(key[e]);
+        else if (top == thr) inside += __uint_as_float(key[e]);
+      }
+    }
+  }
+  sq = block_total(sq, s.red[0]);
+  above = block_total(above, s.red[1]);
+  inside = block_total(inside, s.red[2]);
+  __shared__ float slots[3 * CL];
+  if (CL > 1) {
+    if (tid == 0) {
+      float* to = cg::this_cluster().map_shared_rank(slots, 0);
+      to[3 * rank] = sq; to[3 * rank + 1] = above; to[3 * rank + 2] = inside;
+    }
+    cluster_barrier<CL>();
+    if (rank != 0) return;
+  }
+  if (tid >= 32) return;
+  int last = 0;
+  if (tid == 0) {
+    if (CL > 1) {
+      sq = above = inside = 0.f;
+      for (int r = 0; r < CL; ++r) { sq += slots[3 * r]; above += slots[3 * r + 1]; inside += slots[3 * r + 2]; }
+    }
+    float* hp = a.head_part + (size_t)vec * 4;
+    __stcg(hp, sq);
+    __stcg(hp + 1, above + (float)remaining * (inside / (float)in));
+    __threadfence();
+    last = atomicAdd(&a.stat_ctr[p], 1) == a.H - 1;
+  }
+  if (!__shfl_sync(0xffffffffu, last, 0)) return;
+  // the last head of the problem averages all of them (fixed order)
+  __threadfence();
+  float rho = 0.f, var = 0.f;
+  for (int h = tid; h < a.H; h += 32) {
+    const float* hp = a.head_part + ((size_t)p * a.H + h) * 4;
+    var += __ldcg(hp) * mean;
+    rho += __ldcg(hp + 1);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    rho += __shfl_xor_sync(0xffffffffu, rho, o);
+    var += __shfl_xor_sync(0xffffffffu, var, o);
+  }
+  if (tid == 0) {
+    a.metrics[p * 3 + 1] = rho / (float)a.H;
+    a.metrics[p * 3 + 2] = var / (float)a.H;
+    a.stat_ctr[p] = 0;
+  }
+}
+
+template <int CL, int ITEMS, int VEC>
+__global__ void __launch_bounds__(kRxThreads, ITEMS <= 8 ? 2 : 1) finish(const __grid_constant__ FinishArgs a) {
+  extern __shared__ __align__(16) unsigned char fin_smem[];
+  RadixShared<CL>& s = *reinterpret_cast<RadixShared<CL>*>(fin_smem);
+  const bool stats = (int)blockIdx.x < a.n_stat_ctas;
+  pdl_trigger();
+  if (stats) {
+    radix_clear(s, 0);
+    cluster_barrier<CL>();                           // all CTAs of the cluster run before any remote access
+  }
+  pdl_wait();
+  if (stats) {
+    stats_cta<CL, ITEMS>(a, s, blockIdx.x / CL);
+  } else {
+    const int b = blockIdx.x - a.n_stat_ctas, p = b / a.chunks;
+    if (p < a.n_prob) sum_block<VEC, kRxThreads>(a, p, b - p * a.chunks);
+  }
+}
+constexpr int kSumThreads = 256;     // many short blocks: 16 loads in flight per thread
+template <int VEC>
+__global__ void __launch_bounds__(kSumThreads) sum_layers(const __grid_constant__ FinishArgs a) {
+  pdl_trigger();
+  pdl_wait();
+  sum_block<VEC, kSumThreads>(a, blockIdx.x / a.chunks, blockIdx.x % a.chunks);
+}
+
+// ---- Eq. 5-6 of many long vectors: one CTA per vector, two sweeps over memory --------------------
+// With more vectors than the clusters above could run side by side (32 layers of 131072 keys: 1024
+// vectors, 231 us in two sweeps of 537 MB; clusters of eight 1630 us).  Counting sweeps locate the
+// k-th largest value to 22 bits:
 //   sweep 1: histogram of bits 30..20 (exponent + 3 mantissa bits); sum of squared deviations
-//   sweep 2: exact sum of the entries above the threshold bin (fixed order) and a histogram of
-//            bits 19..9 of the entries inside it
-// The entries inside the threshold bin are then summed as count x bin midpoint: bins of the
-// second level are 2^-14 wide relative to their value, far inside the metric's tolerance.
-constexpr int kHsCluster = 8;      // CTAs per (layer, head) when few vectors are in flight (one layer at a time)
-constexpr int kHsThreads = 1024;
-constexpr int kHsBins = 2048;
-// each bin is kept several times (lane & (copies - 1)) so that a warp's hits on one bin spread: 8 copies
-// where a cluster shares a vector (two CTAs per SM), 16 where one CTA sweeps a whole vector (a lane
-// then shares its banks with one other lane only)
-__host__ __device__ constexpr int hs_copies(int cl) { return cl == 1 ? 16 : 8; }
-constexpr int kHsItems = 16;      // entries per thread kept in registers between the sweeps
+//   sweep 2: exact sum of the entries above the threshold bin and a histogram of bits 19..9 inside it
+// The entries inside the threshold bin are then summed as count x bin midpoint: bins of the second
+// level are 2^-14 wide relative to their value, far inside the metric's tolerance.
+constexpr int kHsThreads = 1024, kHsBins = 2048;
+constexpr int kHsCopies = 16;      // copies of a bin, so that a warp's hits on one bin spread
 
 // Applies f to a[lo .. hi) once each, kHsThreads threads together: 16-byte loads, four of them in
 // flight per thread, scalar accesses only for the unaligned ends.  The order in which a thread
@@ -261,120 +348,99 @@ __device__ __forceinline__ void sweep_from_memory(const float* __restrict__ a, i
   if (t0 + tid < hi) f(a[t0 + tid]);
 }
 
-// Shared memory of head_stats: hist[kHsBins][copies] | merged[2][kHsBins] (dynamic, 80 or 144 KB).
-template <int CL>     // CTAs that share one (layer, head) vector: kHsCluster, or 1 when a batch of layers fills the GPU
+// Called by all threads of a 1024-thread block after a histogram pass over `nb` = 2048 bins.
+// Walks the bins from the top and finds the bin holding the `remaining`-th largest candidate;
+// writes that bin and the rank still wanted inside it.  `scratch` holds 33 words.
+__device__ __forceinline__ void block_pick_from_top(const unsigned* hist, unsigned remaining,
+                                                    unsigned* scratch, unsigned* sel_bin, unsigned* sel_rem) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b_hi = 2047 - 2 * tid, b_lo = b_hi - 1;        // this thread's two bins, higher first
+  const unsigned c_hi = hist[b_hi], c_lo = hist[b_lo];
+  const unsigned mine = c_hi + c_lo;
+  unsigned incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  __syncthreads();
+  if (lane == 31) scratch[warp] = incl;
+  __syncthreads();
+  unsigned before = incl - mine;
+  for (int w = 0; w < warp; ++w) before += scratch[w];
+  if (before < remaining && remaining <= before + mine) {
+    if (before + c_hi >= remaining) { *sel_bin = (unsigned)b_hi; *sel_rem = remaining - before; }
+    else { *sel_bin = (unsigned)b_lo; *sel_rem = remaining - before - c_hi; }
+  }
+  __syncthreads();
+}
+
+// Shared memory: hist[kHsBins][kHsCopies] | merged[2][kHsBins] (dynamic, 144 KB).
 __global__ void __launch_bounds__(kHsThreads)
-head_stats(const float* __restrict__ cols, long long layer_stride, long long col_stride, int H, int n,
-           int k_rho, float* __restrict__ head_part) {
+head_stats(const float* __restrict__ cols, long long layer_stride, long long col_stride, int H, int n, int k_rho,
+           float* __restrict__ head_part) {
   extern __shared__ unsigned hs_smem[];
-  constexpr int kHsCopies = hs_copies(CL);
-  unsigned* hist = hs_smem;                          // this CTA's counts, kHsCopies per bin
-  unsigned* merged = hs_smem + kHsBins * kHsCopies;  // cluster-wide counts of the two levels (CTA 0's copy counts)
-  __shared__ float red[33];
+  unsigned* hist = hs_smem;
+  unsigned* merged = hs_smem + kHsBins * kHsCopies;
+  __shared__ float red[3][33];
   __shared__ unsigned scan_tmp[33];
-  __shared__ float slots[2 * kHsCluster];            // CTA 0: per-CTA {sum of squared deviations, mass above}
   __shared__ unsigned sel_bin, sel_rem;
-  cg::cluster_group cluster = cg::this_cluster();
-  const int rank = (int)cluster.block_rank();
-  const int head = blockIdx.x / CL;                  // (layer, head) pair: one cluster each
+  const int head = blockIdx.x;                       // (layer, head) pair
   const float* a = cols + (size_t)(head / H) * layer_stride + (size_t)(head % H) * col_stride;
   const int tid = threadIdx.x, copy = tid & (kHsCopies - 1);
-  const int per = (n + CL - 1) / CL;
-  const int lo = rank * per, hi = min(n, lo + per);
-  const bool in_regs = per <= kHsItems * kHsThreads;  // otherwise the second sweep reads memory again
-  unsigned* merged0 = cluster.map_shared_rank(merged, 0);
-
   auto clear_local = [&]() {
     for (int b = tid; b < kHsBins * kHsCopies; b += kHsThreads) hist[b] = 0;
   };
-  auto push = [&](int level) {                       // this CTA's counts into CTA 0's merged[level]
+  auto push = [&](int level) {                       // sum of a bin's copies
     for (int b = tid; b < kHsBins; b += kHsThreads) {
       unsigned c = 0;
 #pragma unroll
       for (int k = 0; k < kHsCopies; ++k) c += hist[b * kHsCopies + ((k + tid) & (kHsCopies - 1))];   // rotated: no bank conflicts
-      if (c) atomicAdd(&merged0[level * kHsBins + b], c);
+      merged[level * kHsBins + b] = c;
     }
   };
-
   pdl_trigger();
   clear_local();
-  for (int b = tid; b < 2 * kHsBins; b += kHsThreads) merged[b] = 0;
   pdl_wait();                                        // the pooled columns come from the kernels before
-  float reg[kHsItems];
-#pragma unroll
-  for (int e = 0; e < kHsItems; ++e) {
-    const int j = lo + e * kHsThreads + tid;
-    reg[e] = (in_regs && j < hi) ? a[j] : -1.f;      // -1 marks "no entry" (real entries are >= 0)
-  }
-  cluster.sync();                                    // every merged[] is zero before anyone pushes
+  __syncthreads();
   float sq = 0.f;
   const float mean = 1.f / (float)n;
-  if (in_regs) {
-#pragma unroll
-    for (int e = 0; e < kHsItems; ++e)
-      if (reg[e] >= 0.f) {
-        const float dv = reg[e] - mean;
-        sq = fmaf(dv, dv, sq);
-        atomicAdd(&hist[((__float_as_uint(reg[e]) >> 20) & 0x7ffu) * kHsCopies + copy], 1u);
-      }
-  } else {
-    sweep_from_memory(a, lo, hi, tid, [&](float v) {
-      const float dv = v - mean;
-      sq = fmaf(dv, dv, sq);
-      atomicAdd(&hist[((__float_as_uint(v) >> 20) & 0x7ffu) * kHsCopies + copy], 1u);
-    });
-  }
+  sweep_from_memory(a, 0, n, tid, [&](float v) {
+    const float dv = v - mean;
+    sq = fmaf(dv, dv, sq);
+    atomicAdd(&hist[((__float_as_uint(v) >> 20) & 0x7ffu) * kHsCopies + copy], 1u);
+  });
   __syncthreads();
   push(0);
-  cluster.sync();
-  // level-1 counts of the whole head: copy them here (remote reads in parallel), pick the bin
-  if (rank != 0)
-    for (int b = tid; b < kHsBins; b += kHsThreads) merged[b] = merged0[b];
-  clear_local();
   __syncthreads();
+  clear_local();
   block_pick_from_top(merged, (unsigned)k_rho, scan_tmp, &sel_bin, &sel_rem);
   const unsigned b1 = sel_bin, rem1 = sel_rem;
   float mass = 0.f;
-  auto second = [&](float v) {
+  sweep_from_memory(a, 0, n, tid, [&](float v) {
     const unsigned u = __float_as_uint(v), top = (u >> 20) & 0x7ffu;
     if (top > b1) mass += v;
     else if (top == b1) atomicAdd(&hist[((u >> 9) & 0x7ffu) * kHsCopies + copy], 1u);
-  };
-  if (in_regs) {
-#pragma unroll
-    for (int e = 0; e < kHsItems; ++e)
-      if (reg[e] >= 0.f) second(reg[e]);
-  } else {
-    sweep_from_memory(a, lo, hi, tid, second);
-  }
+  });
   __syncthreads();
   push(1);
-  const float tot_sq = block_sum_1024(sq, red);
-  const float tot_mass = block_sum_1024(mass, red);
-  if (tid == 0) {
-    float* slots0 = cluster.map_shared_rank(slots, 0);
-    slots0[2 * rank] = tot_sq;
-    slots0[2 * rank + 1] = tot_mass;
+  __syncthreads();
+  const unsigned* m2 = merged + kHsBins;
+  block_pick_from_top(m2, rem1, scan_tmp, &sel_bin, &sel_rem);
+  const unsigned b2 = sel_bin, rem2 = sel_rem;
+  // entries of the threshold bin above sub-bin b2, and rem2 entries of sub-bin b2 itself
+  float in_bin = 0.f;
+  for (int b = tid; b < kHsBins; b += kHsThreads) {
+    const float mid = __uint_as_float((b1 << 20) | ((unsigned)b << 9) | 0x100u);
+    const unsigned cnt = (unsigned)b > b2 ? m2[b] : ((unsigned)b == b2 ? rem2 : 0u);
+    in_bin = fmaf((float)cnt, mid, in_bin);
   }
-  cluster.sync();
-  if (rank == 0) {
-    const unsigned* m2 = merged + kHsBins;
-    block_pick_from_top(m2, rem1, scan_tmp, &sel_bin, &sel_rem);
-    const unsigned b2 = sel_bin, rem2 = sel_rem;
-    // entries of the threshold bin above sub-bin b2, and rem2 entries of sub-bin b2 itself
-    float in_bin = 0.f;
-    for (int b = tid; b < kHsBins; b += kHsThreads) {
-      const float mid = __uint_as_float((b1 << 20) | ((unsigned)b << 9) | 0x100u);
-      const unsigned cnt = (unsigned)b > b2 ? m2[b] : ((unsigned)b == b2 ? rem2 : 0u);
-      in_bin = fmaf((float)cnt, mid, in_bin);
-    }
-    const float tot_in_bin = block_sum_1024(in_bin, red);
-    if (tid == 0) {
-      float s2 = 0.f, m = 0.f;
-      for (int r = 0; r < CL; ++r) { s2 += slots[2 * r]; m += slots[2 * r + 1]; }
-      head_part[head * 4 + 0] = s2;
-      head_part[head * 4 + 1] = m + tot_in_bin;
-    }
+  sq = block_total(sq, red[0]);
+  mass = block_total(mass, red[1]);
+  in_bin = block_total(in_bin, red[2]);
+  if (tid == 0) {
+    head_part[head * 4 + 0] = sq;
+    head_part[head * 4 + 1] = mass + in_bin;
   }
 }
 
@@ -416,84 +482,99 @@ cudaError_t launch_finalize_rows(const Ctx& ctx, int parts, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <int CL>
-static cudaError_t launch_head_stats_cl(const float* cols, long long layer_stride, long long col_stride,
-                                        int n_layers, int H, int n, int k_rho, float* head_part, cudaStream_t st) {
-  const int smem = (kHsBins * hs_copies(CL) + 2 * kHsBins) * (int)sizeof(unsigned);
-  cudaError_t e = cudaFuncSetAttribute(head_stats<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+// Raises a kernel's shared-memory limit once per device.
+template <typename K>
+static cudaError_t allow_smem(K* kernel, int bytes, std::atomic<unsigned long long>& ready) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(n_layers * H * CL);
-  cfg.blockDim = dim3(kHsThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = CL;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, head_stats<CL>, cols, layer_stride, col_stride, H, n, k_rho, head_part);
+  const unsigned long long bit = 1ull << (dev & 63);
+  if (ready.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess) ready.fetch_or(bit, std::memory_order_release);
+  return e;
 }
 
-// One layer at a time the vectors are few and the kernel is a chain of latencies: a cluster of
-// CTAs per vector shortens it.  A batch of layers brings enough vectors to fill the GPU with one
-// CTA each, which avoids the cluster barriers and remote merges altogether.
-static cudaError_t launch_head_stats(const float* cols, long long layer_stride, long long col_stride, int n_layers,
-                                     int H, int n, float* head_part, int sm_count, cudaStream_t st) {
-  int k_rho = n / 10;
-  if (k_rho < 1) k_rho = 1;
-  if ((long long)n_layers * H >= 2ll * sm_count)
-    return launch_head_stats_cl<1>(cols, layer_stride, col_stride, n_layers, H, n, k_rho, head_part, st);
-  return launch_head_stats_cl<kHsCluster>(cols, layer_stride, col_stride, n_layers, H, n, k_rho, head_part, st);
+template <int CL, int ITEMS, int VEC>
+static cudaError_t launch_finish_as(FinishArgs& a, int sums, cudaStream_t st) {
+  static std::atomic<unsigned long long> ready{0};
+  const cudaError_t e = allow_smem(finish<CL, ITEMS, VEC>, (int)sizeof(RadixShared<CL>), ready);
+  if (e != cudaSuccess) return e;
+  a.n_stat_ctas = a.n_prob * a.H * CL;
+  return launch_cluster<CL>(finish<CL, ITEMS, VEC>, (a.n_stat_ctas + sums + CL - 1) / CL * CL, sizeof(RadixShared<CL>), st, a);
+}
+template <int VEC>
+static cudaError_t launch_finish(FinishArgs& a, int longest, cudaStream_t st) {
+  a.chunks = (longest + kSumLanes * VEC - 1) / (kSumLanes * VEC);
+  const int sums = a.row_ent ? a.n_prob * a.chunks : 0;
+  if (!a.with_stats) return launch_pdl(sum_layers<VEC>, dim3(sums), dim3(kSumThreads), 0, st, a);
+  // one CTA per vector while its registers hold it (no exchange between CTAs), else the smallest
+  // cluster that does
+  if (longest <= 4 * kRxThreads) return launch_finish_as<1, 4, VEC>(a, sums, st);
+  if (longest <= 8 * kRxThreads) return launch_finish_as<1, 8, VEC>(a, sums, st);
+  if (longest <= 16 * kRxThreads) return launch_finish_as<1, 16, VEC>(a, sums, st);
+  if (longest <= 32 * kRxThreads) return launch_finish_as<2, 16, VEC>(a, sums, st);
+  if (longest <= 64 * kRxThreads) return launch_finish_as<4, 16, VEC>(a, sums, st);
+  return launch_finish_as<4, 32, VEC>(a, sums, st);
 }
 
-cudaError_t launch_reduce_layers(const Ctx& ctx, const float* cols, long long layer_stride, long long col_stride,
-                                 int n, int n_layers, float lambda, float* s_out, long long s_stride,
-                                 float* c_inout, const float* row_ent, float* metrics, cudaStream_t st) {
-  const int H = ctx.cfg.n_q_heads;
+static FinishArgs finish_args(const Ctx& ctx, const float* cols, long long col_stride, int n, float* metrics) {
+  FinishArgs a = {};
+  a.cols = cols; a.col_stride = col_stride;
+  a.H = ctx.cfg.n_q_heads; a.n = n; a.n_prob = 1;
+  a.rows_pad = ctx.rows_pad; a.n_valid = ctx.rows;
+  a.metrics = metrics;
+  a.head_part = ctx.ws.head_part; a.stat_ctr = ctx.ws.stat_ctr; a.chunk_ctr = ctx.ws.chunk_ctr;
+  return a;
+}
+
+cudaError_t launch_finish_layers(const Ctx& ctx, const float* cols, long long layer_stride, long long col_stride, int n,
+                                 int n_layers, float lambda, float* s_out, long long s_stride, float* c_inout,
+                                 const float* row_ent, bool with_head_stats, float* metrics, cudaStream_t st) {
+  FinishArgs a = finish_args(ctx, cols, col_stride, n, metrics);
+  a.layer_stride = layer_stride; a.n_prob = n_layers; a.lambda = lambda;
+  a.s_out = s_out; a.s_stride = s_stride; a.c_inout = c_inout; a.row_ent = row_ent;
+  a.with_stats = with_head_stats;
   const bool vec = n % 4 == 0 && col_stride % 4 == 0 && layer_stride % 4 == 0 && s_stride % 4 == 0 &&
                    ((uintptr_t)cols % 16) == 0 && ((uintptr_t)s_out % 16) == 0 && ((uintptr_t)c_inout % 16) == 0;
-  if (vec)
-    return launch_pdl(reduce_layers<4>, dim3((n / 4 + 63) / 64), dim3(kRcThreads), 0, st, cols, layer_stride,
-                      col_stride, H, n, n_layers, lambda, s_out, s_stride, c_inout, row_ent, ctx.rows_pad,
-                      ctx.rows, metrics);
-  return launch_pdl(reduce_layers<1>, dim3((n + kRcThreads - 1) / kRcThreads), dim3(kRcThreads), 0, st, cols,
-                    layer_stride, col_stride, H, n, n_layers, lambda, s_out, s_stride, c_inout, row_ent,
-                    ctx.rows_pad, ctx.rows, metrics);
+  return vec ? launch_finish<4>(a, n, st) : launch_finish<1>(a, n, st);
 }
 
-cudaError_t launch_reduce_finish(const Ctx& ctx, const float* cols, long long col_stride, int n, float lambda,
-                                 float* s_out, float* c_inout, bool with_head_stats, float* metrics,
-                                 cudaStream_t st) {
-  const int H = ctx.cfg.n_q_heads;
-  if (with_head_stats) {
-    const cudaError_t e = launch_head_stats(cols, 0, col_stride, 1, H, n, ctx.ws.head_part, ctx.sm_count, st);
-    if (e != cudaSuccess) return e;
+cudaError_t launch_finish_packed(const Ctx& ctx, const float* cols, long long col_stride, const int* cu_seqlens, int batch,
+                                 float lambda, float* s_out, float* c_inout, const float* row_ent, float* head_part,
+                                 bool with_head_stats, float* metrics, cudaStream_t st) {
+  FinishArgs a = finish_args(ctx, cols, col_stride, 0, metrics);
+  a.n_prob = batch; a.lambda = lambda; a.s_out = s_out; a.c_inout = c_inout; a.row_ent = row_ent;
+  a.head_part = head_part; a.with_stats = with_head_stats; a.packed = 1;
+  int longest = 0;
+  bool vec = col_stride % 4 == 0 && ((uintptr_t)cols % 16) == 0 && ((uintptr_t)s_out % 16) == 0 && ((uintptr_t)c_inout % 16) == 0;
+  for (int b = 0; b <= batch; ++b) {
+    a.cu[b] = cu_seqlens[b];
+    vec = vec && cu_seqlens[b] % 4 == 0;
+    if (b > 0) longest = cu_seqlens[b] - cu_seqlens[b - 1] > longest ? cu_seqlens[b] - cu_seqlens[b - 1] : longest;
   }
-  const bool vec = n % 4 == 0 && col_stride % 4 == 0 && ((uintptr_t)cols % 16) == 0 &&
-                   ((uintptr_t)s_out % 16) == 0 && ((uintptr_t)c_inout % 16) == 0;
-  if (vec)
-    return launch_pdl(reduce_finish<4>, dim3((n / 4 + 63) / 64), dim3(kRcThreads), 0, st, cols,
-                      col_stride, H, n, lambda, s_out, c_inout, (const float*)ctx.ws.row_ent, ctx.rows_pad,
-                      ctx.rows, (const float*)ctx.ws.head_part, with_head_stats ? 1 : 0,
-                      metrics);
-  return launch_pdl(reduce_finish<1>, dim3((n + kRcThreads - 1) / kRcThreads), dim3(kRcThreads), 0, st, cols,
-                    col_stride, H, n, lambda, s_out, c_inout, (const float*)ctx.ws.row_ent, ctx.rows_pad,
-                    ctx.rows, (const float*)ctx.ws.head_part, with_head_stats ? 1 : 0,
-                    metrics);
+  return vec ? launch_finish<4>(a, longest, st) : launch_finish<1>(a, longest, st);
 }
 
 cudaError_t launch_head_stats_batch(const Ctx& ctx, const float* cols, long long layer_stride, long long col_stride,
                                     int n_layers, int n, float* metrics, cudaStream_t st) {
   const int H = ctx.cfg.n_q_heads;
-  cudaError_t e = launch_head_stats(cols, layer_stride, col_stride, n_layers, H, n, ctx.ws.head_part, ctx.sm_count, st);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(head_metrics, dim3((n_layers + 63) / 64), dim3(64), 0, st, (const float*)ctx.ws.head_part,
-                    n_layers, H, n, metrics);
+  // Two sweeps per vector where the vectors fill the GPU several times over and are long: with 1024
+  // vectors 85 / 115 / 231 us at 16000 / 32768 / 131072 keys, the register form 91 / 140 / > 500.
+  if ((long long)n_layers * H >= 2ll * ctx.sm_count && n > 8 * kRxThreads) {
+    static std::atomic<unsigned long long> ready{0};
+    const int smem = (kHsBins * kHsCopies + 2 * kHsBins) * (int)sizeof(unsigned);
+    cudaError_t e = allow_smem(head_stats, smem, ready);
+    if (e != cudaSuccess) return e;
+    e = launch_pdl(head_stats, dim3(n_layers * H), dim3(kHsThreads), smem, st, cols, layer_stride, col_stride, H, n,
+                   n / 10 < 1 ? 1 : n / 10, ctx.ws.head_part);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(head_metrics, dim3((n_layers + 63) / 64), dim3(64), 0, st, (const float*)ctx.ws.head_part, n_layers,
+                      H, n, metrics);
+  }
+  FinishArgs a = finish_args(ctx, cols, col_stride, n, metrics);
+  a.layer_stride = layer_stride; a.n_prob = n_layers; a.with_stats = 1;
+  return launch_finish<1>(a, n, st);
 }
 
 cudaError_t launch_accumulate(const float* s_hist, long long row_stride, int pivot, int n,

@@ -4,8 +4,7 @@
 // 1024 tokens, warp).  A cluster of CL CTAs shares one vector, each CTA a contiguous slice that it
 // holds in registers (up to ITEMS tokens a thread; a longer slice is read again per level).
 //
-// Bound by the chain of barriers, not by memory.  One CTA up to 16384 tokens (no exchange between
-// CTAs), a cluster of eight beyond.
+// Bound by the chain of barriers, not by memory: one CTA up to 16384 tokens (no exchange between CTAs).
 #include <atomic>
 
 #include "radix.cuh"
@@ -178,12 +177,21 @@ cudaError_t launch(const SelectArgs& a, cudaStream_t st) {
   return launch_cluster<CL>(select_topk<CL, ITEMS>, a.batch * CL, sizeof(RadixShared<CL>), st, a);
 }
 
-// Fewest items per thread that hold a slice; beyond 16 x 8192 tokens a slice takes several rounds.
+// The smallest cluster and the fewest items per thread that hold a vector, as measured (us for 1 / 32
+// vectors): 1777 tokens 5.8 / 7.7 with 1 x 4 items, 5003 9.6 / 11.5 with 1 x 8, 12000 12.6 / 15.0 with
+// 1 x 16 (14.0 / 19.6 with a cluster of 2), 32768 17.3 / 20.3 with 2 x 16 (20.6 / 23.5 with 1 x 32, 19.3 /
+// 41.9 with 8 x 8), 65536 19.2 / 22.8 with 4 x 16.  At 131072 eight CTAs of 16 items take 23.1 us for one
+// vector but 69.1 for 32, whose 256 CTAs no longer run side by side; four of 32 take 28.6 / 33.0.
 cudaError_t dispatch(const SelectArgs& a, int longest, cudaStream_t st) {
   if (longest <= 4 * kRxThreads) return launch<1, 4>(a, st);
+  if (longest <= 8 * kRxThreads) return launch<1, 8>(a, st);
   if (longest <= 16 * kRxThreads) return launch<1, 16>(a, st);
-  if (longest <= 8 * 8 * kRxThreads) return launch<8, 8>(a, st);
-  return launch<8, 16>(a, st);
+  if (longest <= 32 * kRxThreads) return launch<2, 16>(a, st);
+  if (longest <= 64 * kRxThreads) return launch<4, 16>(a, st);
+  const bool room = a.batch <= 16;                   // eight CTAs a vector, one per SM
+  if (!room) return launch<4, 32>(a, st);
+  if (longest <= 128 * kRxThreads) return launch<8, 16>(a, st);
+  return launch<8, 32>(a, st);                       // beyond 262144 tokens the slices are read again per level
 }
 
 }  // namespace

@@ -1,0 +1,73 @@
+"""Selection and head statistics at the sizes where their split over CTAs changes (one CTA with 4, 8 or 16
+entries a thread, clusters of two, four and eight, slices that do not fit the registers), against the
+oracle: selection exact with ties, statistics within the metric tolerance."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import structkv_oracle as O
+from tests import parity as P
+
+pytestmark = pytest.mark.gpu
+EDGES = [1024, 4096, 8192, 16384, 32768, 65536, 131072, 262144]
+
+
+@pytest.fixture(scope="module")
+def ctx(cuda_device):
+    from paper_2604_06746_b200 import binding
+    c = binding.Context(4, 2, 128, 64, 1 << 19, torch.bfloat16, cuda_device)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("batch", [1, 17])
+@pytest.mark.parametrize("edge", EDGES)
+def test_select_around_the_edges(ctx, edge, batch):
+    rng = np.random.default_rng(edge + batch)
+    for n in (edge + 63, edge + 64, edge + 65):              # prefix of edge - 1, edge, edge + 1 tokens
+        sc = (rng.random((batch, n)) ** 3).astype(np.float32)
+        sc[:, ::3] = np.float32(0.125)                       # a third of the tokens tie
+        k = 64 + int(0.6 * n) if n % 2 else 64 + n // 50     # the threshold inside the ties, and above them
+        out = torch.zeros((batch, k), dtype=torch.int32, device="cuda")
+        ctx.select(torch.from_numpy(sc).cuda(), k, 64, out)
+        got = out.cpu().numpy()
+        for b in {0, batch - 1}:
+            assert np.array_equal(got[b], O.select(sc[b], k, 64)), (n, b)
+
+
+def test_select_beyond_the_registers_of_a_cluster(ctx):
+    rng = np.random.default_rng(9)
+    n, k = 300001, 40000
+    sc = rng.integers(0, 1000, size=n).astype(np.float32)
+    out = torch.zeros((1, k), dtype=torch.int32, device="cuda")
+    ctx.select(torch.from_numpy(sc).cuda(), k, 64, out)
+    assert np.array_equal(out[0].cpu().numpy(), O.select(sc, k, 64))
+
+
+def test_packed_selection_of_unequal_prompts(ctx):
+    rng = np.random.default_rng(10)
+    lens, budgets = (70, 5000, 64, 40001, 900), (66, 5000, 64, 3000, 64)
+    cu = np.concatenate([[0], np.cumsum(lens)]).tolist()
+    sc = rng.integers(-50, 50, size=cu[-1]).astype(np.float32)
+    out = torch.zeros((len(lens), 6000), dtype=torch.int32, device="cuda")
+    ctx.select_batch(torch.from_numpy(sc).cuda(), cu, budgets, 64, out)
+    got = out.cpu().numpy()
+    for b, k in enumerate(budgets):
+        assert np.array_equal(got[b, :k], O.select(sc[cu[b]:cu[b + 1]], k, 64)), b
+        assert np.all(got[b, k:] == -1)
+
+
+@pytest.mark.parametrize("edge", EDGES[1:-1])
+def test_head_statistics_around_the_edges(ctx, edge):
+    rng = np.random.default_rng(edge)
+    for n in (edge, edge + 1):
+        x = rng.random((1, 4, n)) ** 4
+        x[:, :, ::5] = 0.0
+        x[:, :2, 1::5] = 0.3                                 # ties across the threshold
+        x[:, 3, 7] += 0.1 * n
+        x32 = (x / x.sum(axis=2, keepdims=True)).astype(np.float32)
+        m = torch.zeros((1, 3), device="cuda")
+        ctx.head_stats(torch.from_numpy(x32).cuda(), m)
+        rho, var = O.head_statistics(x32[0].astype(np.float64))
+        P.assert_metric_close(m[0, 1].item(), rho, f"sparsity at {n}")
+        P.assert_metric_close(m[0, 2].item(), var, f"variance at {n}")
