@@ -105,13 +105,17 @@ cudaError_t launch_problems(const Ctx& ctx, const TcCall& a, int first, int n, c
     pb.v_min = -125.f / pb.c2;
     const int tiles = (pb.n_keys + kKeyTile - 1) / kKeyTile;
     // One task per SM and pass, shared out over the sequences of a batch by their lengths; in pass 1 at
-    // least two pairs of tiles a task, which carries 1.5 us of hand-over whatever its size.
+    // least two pairs of tiles a task, which carries 1.5 us of hand-over whatever its size, unless all
+    // of them run at once anyway.
     const int share = batch ? std::max(1, (int)((long long)sms * pb.n_keys / total_keys)) : sms;
-    pb.t1 = clamp_tasks(l, share, (tiles + 3) / 4);
+    const int pairs = (tiles + 1) / 2;
+    pb.t1 = clamp_tasks(l, share, (long long)l.units * pairs <= sms ? pairs : (pairs + 1) / 2);
     // Pass 2 leaves no partial results, so the pass nothing follows is cut finer: its tasks end
     // closer together.
+    // (Not below eight tiles a task, each of which merges its unit's statistics first.)
     const bool last = batch || i == n - 1;
-    pb.t2 = last ? clamp_tasks(l, 2 * share, tiles) : clamp_tasks(l, share, (tiles + 3) / 4);
+    if (!last) pb.t2 = clamp_tasks(l, share, (tiles + 3) / 4);
+    else pb.t2 = clamp_tasks(l, (long long)l.units * tiles >= 16ll * share ? 2 * share : share, tiles);
     pb.part0 = part0;
     part0 += pb.t1;
   }
@@ -153,6 +157,7 @@ cudaError_t launch_problems(const Ctx& ctx, const TcCall& a, int first, int n, c
   p.row_ent = a.row_ent + (size_t)first * ctx.rows_pad;
   p.col_stride = a.col_stride;
   p.status = ctx.ws.status;
+  p.hurry = n == 1 || batch;
   const int grid = std::min(sms, tickets);
   return cfg.head_dim == 128 ? tc_launch_128(l.shape, p, grid, ctx.device, st) : tc_launch_64(l.shape, p, grid, ctx.device, st);
 }

@@ -60,6 +60,7 @@ constexpr int kTcThreads = (kHelperWarps + kComputeWarps) * 32;   // 20 warps: t
 constexpr unsigned long long kWaitCycles = 1000000000ull;   // about 0.5 s at the maximum SM clock
 constexpr float kMasked = -1.0e30f;    // exponent standing for -inf: 2^x flushes to 0 and 0 * x stays finite
 constexpr float kMaskedAcc = -3.0e38f; // the same for an accumulator, before the scaling by c2 >= 1e-30
+constexpr int kMergeGroup = 6;         // partials of a row merged together
 constexpr int kFullWeight = 20;        // weight of a full row block when key ranges are dealt out (see tc_deal)
 
 // Layout classes of the kernel (template argument).
@@ -91,6 +92,11 @@ struct alignas(64) TcParams {
   float* row_ent;                      // [problem][unit][256] entropy of a row, nats (0: no row)
   long long col_stride;
   int* status;
+  // Pass 2 has nothing to do but wait for pass 1 (one layer, a batch): the compute warps fold and merge the
+  // row statistics themselves, all 512 threads at once, instead of leaving it to one helper warp
+  // beside them (at 8192 keys 2 + 2 us instead of 3 + 6).  With layers to interleave the helpers'
+  // time is hidden and the compute warps' is not.
+  int hurry;
 };
 constexpr int kCtlTicket = 0, kCtlExit = 1, kCtlArrive = 64, kCtlReady = 64 + kMaxBatch * kQueueUnits;
 static_assert(kCtlInts == 64 + 2 * kMaxBatch * kQueueUnits, "control block");
@@ -391,7 +397,7 @@ struct TcTask { int pass, prob, g, rb, lo, hi, part, part0, n_part; };   // pass
 // Barrier slots (8 bytes each) inside the barrier area.
 enum { kBarFull = 0, kBarEmpty = kBarFull + kStages, kBarTaskFull = kBarEmpty + kStages,
        kBarTaskEmpty = kBarTaskFull + kTaskRing, kBarQFull = kBarTaskEmpty + kTaskRing, kBarQEmpty = kBarQFull + 2,
-       kBarExtFull = kBarQEmpty + 2, kBarExtEmpty, kBarPartFull, kBarPartEmpty, kBarDrain, kBarAccFull,
+       kBarExtFull = kBarQEmpty + 2, kBarExtEmpty, kBarSync, kBarPartFull, kBarPartEmpty, kBarDrain, kBarAccFull,
        kBarAccEmpty = kBarAccFull + 8, kBarCount = kBarAccEmpty + 8 };
 constexpr int kTaskConsumers = 3 + kComputeWarps;          // MMA, lse hand-over, fold, compute warps
 
@@ -424,6 +430,43 @@ __device__ __forceinline__ void merge_partials(float& M, float& W, float& X, con
     const float e = pv[b].x == -INFINITY ? -200.f : pv[b].x - top, w = fast_exp2(e);
     W += w;
     X = fmaf(w, pv[b].y - e, X);
+  }
+}
+// The four column groups (wide) or lane quarters (narrow) of a row fold into one partial.
+template <int R>
+__device__ __forceinline__ float2 fold_row(const float2* part_s, int r) {
+  float2 c[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) c[k] = part_s[k * R + r];
+  float M = -INFINITY, W = 0.f, X = 0.f;
+  merge_partials(M, W, X, c);
+  const float lw = __log2f(W);
+  return W > 0.f ? make_float2(M + lw, lw + __fdividef(X, W)) : make_float2(-INFINITY, 0.f);
+}
+// Merges a unit's partials for the rows lane, lane + 32, ... of one warp, four rows (24 loads) at a time;
+// done(row, -lse, entropy) with (-inf, 0) for rows that saw no key.
+template <int R, typename F>
+__device__ __forceinline__ void merge_unit(const float2* part, int n_part, int lane, F done) {
+  constexpr int kRowsAt = R < 128 ? R / 32 : 4, kBatch = kMergeGroup;
+  for (int r0 = lane; r0 < R; r0 += 32 * kRowsAt) {
+    float M[kRowsAt], W[kRowsAt], X[kRowsAt];
+#pragma unroll
+    for (int q = 0; q < kRowsAt; ++q) { M[q] = -INFINITY; W[q] = X[q] = 0.f; }
+    for (int s0 = 0; s0 < n_part; s0 += kBatch) {
+      float2 pv[kRowsAt][kBatch];
+#pragma unroll
+      for (int b = 0; b < kBatch; ++b)
+#pragma unroll
+        for (int q = 0; q < kRowsAt; ++q)
+          pv[q][b] = s0 + b < n_part ? __ldcg(part + (size_t)(s0 + b) * kRowBlock + r0 + 32 * q) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+      for (int q = 0; q < kRowsAt; ++q) merge_partials(M[q], W[q], X[q], pv[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kRowsAt; ++q) {
+      const float lz = __log2f(W[q]);
+      done(r0 + 32 * q, W[q] > 0.f ? -(M[q] + lz) : -INFINITY, W[q] > 0.f ? kLn2 * (lz + X[q] / W[q]) : 0.f);
+    }
   }
 }
 // Adds one chunk of 32 keys to a row's statistics, all keys visible.  False: a logit far above the
@@ -519,6 +562,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     for (int s = 0; s < kTaskRing; ++s) { mbar_init(bar(kBarTaskFull + s), 1); mbar_init(bar(kBarTaskEmpty + s), kTaskConsumers); }
     for (int b = kBarQFull; b <= kBarExtEmpty; ++b) mbar_init(bar(b), 1);
     mbar_init(bar(kBarPartFull), kComputeWarps);
+    mbar_init(bar(kBarSync), kComputeWarps);
     mbar_init(bar(kBarPartEmpty), 1);
     mbar_init(bar(kBarDrain), 1);
     for (int a = 0; a < S::kAcc; ++a) { mbar_init(bar(kBarAccFull + a), 1); mbar_init(bar(kBarAccEmpty + a), kComputeWarps); }
@@ -556,6 +600,20 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     if (lane == 0) mbar_arrive(bar(kBarTaskEmpty + k));
     return t.pass != 0;
   };
+  // -lse / c2 of a row as hi + mid + lo (bf16 each: 24 bits together) into the extra K-step's operand; rows
+  // that do not exist get a huge negative value so that their 2^x is 0.
+  auto put_lse = [&](int r, float nlse, float inv_c2) {
+    const float Lv = nlse == -INFINITY ? kMaskedAcc : nlse * inv_c2;
+    const __nv_bfloat16 hi = __float2bfloat16_rn(Lv);
+    const float r1 = Lv - __bfloat162float(hi);
+    const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
+    const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
+    unsigned char* bx = sm + L::kExtOff;
+    *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 0)) = hi;
+    *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 1)) = mid;
+    *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 2)) = lo;
+  };
+  auto is_row = [&](int row) { return row < p.rows_pg && row % p.w_pad < p.window; };   // row of the KV group, padding excluded
   // Tiles of item `it` of a task: pass 1 ascends, pass 2 descends; half 1 may be missing at the end.
   auto tile_of = [](const TcTask& t, int it, int half) { return t.pass == 1 ? t.lo + 2 * it + half : t.hi - 1 - 2 * it - half; };
   auto present = [](const TcTask& t, int tile) { return tile >= t.lo && tile < t.hi; };
@@ -586,19 +644,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
           t.rb = min((w_at - t.g * p.w_group) / kFullWeight, p.n_rb - 1);
           const int w0 = t.g * p.w_group + t.rb * kFullWeight;
           const int i0 = tc_deal(w0, tasks, p.w_total);
-          t.n_part = tc_deal(w0 + (t.rb == p.n_rb - 1 ? p.w_last : kFullWeight), tasks, p.w_total) - i0;
+          const int w_unit = t.rb == p.n_rb - 1 ? p.w_last : kFullWeight;
+          const int n_seg = tc_deal(w0 + w_unit, tasks, p.w_total) - i0;
           const int seg = i - i0, n_tiles = (pb.n_keys + kKeyTile - 1) / kKeyTile;
           if (t.pass == 1) {
             const int n_pairs = (n_tiles + 1) / 2;
-            t.lo = 2 * (int)((long long)seg * n_pairs / t.n_part);
-            t.hi = 2 * (int)((long long)(seg + 1) * n_pairs / t.n_part);
+            t.lo = 2 * (int)((long long)seg * n_pairs / n_seg);
+            t.hi = 2 * (int)((long long)(seg + 1) * n_pairs / n_seg);
             if (S::kNarrow) t.hi = min(t.hi, n_tiles);     // a wide accumulator takes a pair: the odd tile's partner is masked
           } else {
-            t.lo = (int)((long long)seg * n_tiles / t.n_part);
-            t.hi = (int)((long long)(seg + 1) * n_tiles / t.n_part);
+            t.lo = (int)((long long)seg * n_tiles / n_seg);
+            t.hi = (int)((long long)(seg + 1) * n_tiles / n_seg);
           }
           t.part = pb.part0 + i;
-          t.part0 = pb.part0 + i0;
+          // the unit's partials: pass 1 deals its own number of tasks
+          const int p0 = tc_deal(w0, pb.t1, p.w_total);
+          t.n_part = tc_deal(w0 + w_unit, pb.t1, p.w_total) - p0;
+          t.part0 = pb.part0 + p0;
           tk = atomicAdd(ticket, 1);                       // travels while this task is loaded
         }
         const int k = n % kTaskRing;
@@ -759,7 +821,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     int n_ext = 0;
     TcTask t;
     for (int n = 0; next_task(n, t); ++n) {
-      if (t.pass != 2 || t.lo == t.hi) continue;
+      if (p.hurry || t.pass != 2 || t.lo == t.hi) continue;
       int ok = 1;
       const int unit = t.g * p.n_rb + t.rb;
       if (lane == 0) {
@@ -773,28 +835,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
           if (seen != 0) break;
           if (*abort_flag) ok = 0;
           else if ((unsigned long long)(clock64() - t0) > kWaitCycles) { *abort_flag = 1; ok = 0; }
-          else __nanosleep(100);
+          else __nanosleep(50);
         }
       }
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
-      const float* nl = p.nlse + ((size_t)t.prob * p.n_units + unit) * kRowBlock;
+      const size_t at0 = ((size_t)t.prob * p.n_units + unit) * kRowBlock;
       const float inv_c2 = p.prob[t.prob].inv_c2;
 #pragma unroll
-      for (int i = 0; i < R / 32; ++i) {
-        const int r = i * 32 + lane;
-        // -lse / c2 as hi + mid + lo (bf16 each: 24 bits together); rows that do not exist get a huge
-        // negative value so that their 2^x is 0
-        const float nlse = __ldcg(nl + r);
-        const float Lv = nlse == -INFINITY ? kMaskedAcc : nlse * inv_c2;
-        const __nv_bfloat16 hi = __float2bfloat16_rn(Lv);
-        const float r1 = Lv - __bfloat162float(hi);
-        const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-        unsigned char* bx = sm + L::kExtOff;
-        *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 0)) = hi;
-        *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 1)) = mid;
-        *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 2)) = lo;
-      }
+      for (int i = 0; i < R / 32; ++i) put_lse(i * 32 + lane, __ldcg(p.nlse + at0 + i * 32 + lane), inv_c2);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(kBarExtFull));
@@ -806,21 +854,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     int n_p1 = 0;
     TcTask t;
     for (int n = 0; next_task(n, t); ++n) {
-      if (t.pass != 1) continue;
+      if (p.hurry || t.pass != 1) continue;
       int ok = 1;
       if (lane == 0) ok = mbar_wait_producer(bar(kBarPartFull), (uint32_t)n_p1 & 1u, abort_flag, kWaitCycles) ? 1 : 0;
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
       ++n_p1;
-      // the four column groups (wide) or lane quarters (narrow) of a row fold into one partial per task
 #pragma unroll 4
       for (int r = lane; r < R; r += 32) {
-        float2 c[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) c[k] = part_s[k * R + r];
-        float M = -INFINITY, W = 0.f, X = 0.f;
-        merge_partials(M, W, X, c);
-        const float lw = __log2f(W);
-        __stcg(&p.part[(size_t)t.part * kRowBlock + r], W > 0.f ? make_float2(M + lw, lw + __fdividef(X, W)) : make_float2(-INFINITY, 0.f));
+        __stcg(&p.part[(size_t)t.part * kRowBlock + r], fold_row<R>(part_s, r));
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(kBarPartEmpty));
@@ -832,36 +873,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
       if (!__shfl_sync(0xffffffffu, last, 0)) continue;
       __threadfence();
       // this task completes the unit: merge its partials into each row's log-sum-exp and entropy
-      const float2* part = p.part + (size_t)t.part0 * kRowBlock;
       const size_t at0 = ((size_t)t.prob * p.n_units + unit) * kRowBlock;
-      constexpr int kRowsAt = R < 128 ? R / 32 : 4, kBatch = 6;
-      for (int r0 = lane; r0 < R; r0 += 32 * kRowsAt) {
-        float M[kRowsAt], W[kRowsAt], X[kRowsAt];
-#pragma unroll
-        for (int q = 0; q < kRowsAt; ++q) { M[q] = -INFINITY; W[q] = X[q] = 0.f; }
-        for (int s0 = 0; s0 < t.n_part; s0 += kBatch) {
-          float2 pv[kRowsAt][kBatch];
-#pragma unroll
-          for (int b = 0; b < kBatch; ++b)
-#pragma unroll
-            for (int q = 0; q < kRowsAt; ++q)
-              pv[q][b] = s0 + b < t.n_part ? __ldcg(part + (size_t)(s0 + b) * kRowBlock + r0 + 32 * q) : make_float2(-INFINITY, 0.f);
-#pragma unroll
-          for (int q = 0; q < kRowsAt; ++q) merge_partials(M[q], W[q], X[q], pv[q]);
-        }
-#pragma unroll
-        for (int q = 0; q < kRowsAt; ++q) {
-          const int r = r0 + 32 * q, row = t.rb * R + r;
-          float nlse = -INFINITY, ent = 0.f;
-          if (row < p.rows_pg && row % p.w_pad < p.window && W[q] > 0.f) {
-            const float lz = __log2f(W[q]);
-            nlse = -(M[q] + lz);
-            ent = kLn2 * (lz + X[q] / W[q]);
-          }
-          __stcg(p.nlse + at0 + r, nlse);
-          p.row_ent[at0 + r] = ent;
-        }
-      }
+      merge_unit<R>(p.part + (size_t)t.part0 * kRowBlock, t.n_part, lane, [&](int r, float nlse, float ent) {
+        const bool row = is_row(t.rb * R + r);
+        __stcg(p.nlse + at0 + r, row ? nlse : -INFINITY);
+        p.row_ent[at0 + r] = row ? ent : 0.f;
+      });
       for (int r = R + lane; r < kRowBlock; r += 32) p.row_ent[at0 + r] = 0.f;   // rows of the block the unit does not have
       __threadfence();
       __syncwarp();
@@ -874,7 +891,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     const int sub = (warp - kHelperWarps) >> 2;   // which quarter of an accumulator's columns (or of the tiles) it takes
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
     float2* part_s = reinterpret_cast<float2*>(sm + L::kPartOff);
-    int u = 0, n_p1 = 0;
+    int u = 0, n_p1 = 0, n_sync = 0, n_ext = 0;
     // Every lane polls: a barrier that has already flipped costs one test, no divergence, no broadcast
     // (with four chunks of arithmetic per accumulator and scheduler each instruction here shows).
     auto acc_full = [&]() {
@@ -897,10 +914,74 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
       if (lane == 0) ok = mbar_wait(bar(kBarPartEmpty), ((uint32_t)n_p1 & 1u) ^ 1u, abort_flag) ? 1 : 0;
       return __shfl_sync(0xffffffffu, ok, 0) != 0;
     };
-    auto part_done = [&]() {
+    // Bounded barrier of the compute warps.
+    auto sync_all = [&]() {
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(kBarPartFull));
-      ++n_p1;
+      if (lane == 0) mbar_arrive(bar(kBarSync));
+      const bool ok = mbar_wait(bar(kBarSync), (uint32_t)n_sync++ & 1u, abort_flag);
+      return __all_sync(0xffffffffu, ok) != 0;
+    };
+    const int ct = (int)threadIdx.x - kHelperWarps * 32;
+    // The task's statistics are in shared memory: the fold warp takes them from here, or, in a hurry,
+    // the compute warps themselves.
+    auto part_done = [&](const TcTask& t) {
+      if (!p.hurry) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kBarPartFull));
+        ++n_p1;
+        return true;
+      }
+      if (!sync_all()) return false;
+      if (ct < R) __stcg(&p.part[(size_t)t.part * kRowBlock + ct], fold_row<R>(part_s, ct));
+      __threadfence();
+      if (!sync_all()) return false;
+      if (ct == 0) atomicAdd(p.ctl + kCtlArrive + t.prob * kQueueUnits + t.g * p.n_rb + t.rb, 1);
+      return true;
+    };
+    // In a hurry: the compute warps wait for the unit's partials and merge them, a thread per row, into the
+    // extra K-step's operand (the task that holds key 0 leaves the entropies).
+    auto merge_now = [&](const TcTask& t) {
+      const int unit = t.g * p.n_rb + t.rb;
+      if (ct == 0) {
+        bool ok = mbar_wait(bar(kBarExtEmpty), ((uint32_t)n_ext & 1u) ^ 1u, abort_flag);
+        const int* count = p.ctl + kCtlArrive + t.prob * kQueueUnits + unit;
+        const long long t0 = clock64();
+        while (ok) {
+          int seen;
+          asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
+          if (seen >= t.n_part) break;
+          if (*abort_flag) ok = false;
+          else if ((unsigned long long)(clock64() - t0) > kWaitCycles) { *abort_flag = 1; ok = false; }
+        }
+      }
+      if (!sync_all() || *abort_flag) return false;
+      if (ct < R) {
+        const float2* part = p.part + (size_t)t.part0 * kRowBlock + ct;
+        float M = -INFINITY, W = 0.f, X = 0.f;
+        // all partials of a row in one round of loads (148 SMs, 8 units: 18 or 19), merged in the helper
+        // warp's groups: the bits must not depend on who merges
+        constexpr int kRounds = 4;
+        for (int s0 = 0; s0 < t.n_part; s0 += kRounds * kMergeGroup) {
+          float2 pv[kRounds][kMergeGroup];
+#pragma unroll
+          for (int b = 0; b < kRounds * kMergeGroup; ++b)
+            pv[b / kMergeGroup][b % kMergeGroup] =
+                s0 + b < t.n_part ? __ldcg(part + (size_t)(s0 + b) * kRowBlock) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+          for (int k = 0; k < kRounds; ++k) merge_partials(M, W, X, pv[k]);
+        }
+        const bool row = is_row(t.rb * R + ct) && W > 0.f;
+        const float lz = __log2f(W);
+        put_lse(ct, row ? -(M + lz) : -INFINITY, p.prob[t.prob].inv_c2);
+        if (t.lo == 0) p.row_ent[((size_t)t.prob * p.n_units + unit) * kRowBlock + ct] = row ? kLn2 * (lz + X / W) : 0.f;
+      } else if (t.lo == 0 && ct < kRowBlock) {
+        p.row_ent[((size_t)t.prob * p.n_units + unit) * kRowBlock + ct] = 0.f;   // rows of the block the unit does not have
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
+      if (!sync_all()) return false;
+      if (ct == 0) mbar_arrive(bar(kBarExtFull));
+      ++n_ext;
+      return true;
     };
     TcTask t;
     bool live = true;
@@ -960,10 +1041,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
           }
           ++u;
         }
-        if (!live || !part_free()) break;
+        if (!live || (!p.hurry && !part_free())) break;
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) part_s[sub * R + hf * 128 + row_lo] = stat_partial(rs[hf]);
-        part_done();
+        if (!part_done(t)) break;
       } else if (t.pass == 1) {
         if constexpr (S::kNarrow) {
           // Lane = key, RT rows per thread; every lane keeps its own reference per row.
@@ -1005,7 +1086,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
               U[e] = fmaf(pe, x, U[e]);
             }
           }
-          if (!live || !part_free()) break;
+          if (!live || (!p.hurry && !part_free())) break;
 #pragma unroll
           for (int e = 0; e < RT; ++e) {
             float M = Z[e] > 0.f ? ref[e] : -INFINITY;
@@ -1020,10 +1101,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
             }
             if (lane == e) part_s[quarter * R + sub * RT + e] = stat_partial(RowStat{M, Ze, Ue});
           }
-          part_done();
+          if (!part_done(t)) break;
         }
       } else {
         // Pass 2: this thread owns key (tile * 128 + quarter * 32 + lane); x = c2 * accumulator.
+        if (p.hurry && t.hi > t.lo && !merge_now(t)) break;
         const float v_min = pb.v_min, inv_w = 1.0f / (float)p.window;
         // Columns (rows of the block) this warp sums: a quarter of them on every tile, or, where a
         // head spans more, the head's rows on every second or fourth tile, so that a head's column
