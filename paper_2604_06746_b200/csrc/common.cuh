@@ -163,6 +163,9 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
+__device__ __forceinline__ void add_to(float4& s, const float4& v) { s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
+__device__ __forceinline__ void add_to(float& s, float v) { s += v; }
+
 // 2^x on the special-function unit (relative error about 2^-22; denormal results flush to 0).
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;

@@ -41,6 +41,8 @@ gather_rows(const char* __restrict__ src, long long slab_stride, long long row_s
             int units_per_row, int n_slabs, int n_rows_src, const int* __restrict__ idx,
             long long idx_slab_stride, int n_idx,
             char* __restrict__ dst, int* __restrict__ status) {
+  pdl_trigger();
+  pdl_wait();
   const long long total = (long long)n_slabs * n_idx * units_per_row;
   const long long stride = (long long)gridDim.x * kCpThreads;
   for (long long u0 = (long long)blockIdx.x * kCpThreads + threadIdx.x; u0 < total;
@@ -83,6 +85,8 @@ gather_rows_layers(const __grid_constant__ LayerPtrs srcs, long long slab_stride
                    int units_per_row, int n_slabs, int n_rows_src, const int* __restrict__ idx,
                    long long idx_layer_stride, int n_idx, char* __restrict__ dst, long long dst_layer_stride,
                    int* __restrict__ status) {
+  pdl_trigger();
+  pdl_wait();
   const int layer = blockIdx.y;
   const char* __restrict__ src = srcs.src[layer];
   const int* __restrict__ my_idx = idx + (long long)layer * idx_layer_stride;
@@ -144,17 +148,9 @@ cudaError_t launch_compact_layers(const void* const* srcs, int n_layers, long lo
   if (blocks < 1) blocks = 1;
   const dim3 grid((unsigned)blocks, (unsigned)n_layers);
   char* d = (char*)dst;
-  if (unit == 16)
-    gather_rows_layers<uint4><<<grid, kCpThreads, 0, st>>>(lp, slab_stride, row_stride, upr, n_slabs, n_rows_src, idx,
-                                                          idx_layer_stride, n_idx, d, dst_layer_stride, status);
-  else if (unit == 4)
-    gather_rows_layers<unsigned><<<grid, kCpThreads, 0, st>>>(lp, slab_stride, row_stride, upr, n_slabs, n_rows_src,
-                                                             idx, idx_layer_stride, n_idx, d, dst_layer_stride, status);
-  else
-    gather_rows_layers<unsigned char><<<grid, kCpThreads, 0, st>>>(lp, slab_stride, row_stride, upr, n_slabs,
-                                                                  n_rows_src, idx, idx_layer_stride, n_idx, d,
-                                                                  dst_layer_stride, status);
-  return cudaGetLastError();
+  const auto kernel = unit == 16 ? gather_rows_layers<uint4> : unit == 4 ? gather_rows_layers<unsigned> : gather_rows_layers<unsigned char>;
+  return launch_pdl(kernel, grid, dim3(kCpThreads), 0, st, lp, slab_stride, row_stride, upr, n_slabs, n_rows_src, idx,
+                    idx_layer_stride, n_idx, d, dst_layer_stride, status);
 }
 
 cudaError_t launch_compact(const void* src, long long slab_stride, long long row_stride,
@@ -175,16 +171,9 @@ cudaError_t launch_compact(const void* src, long long slab_stride, long long row
   if (blocks < 1) blocks = 1;
   const char* s = (const char*)src;
   char* d = (char*)dst;
-  if (unit == 16)
-    gather_rows<uint4><<<(int)blocks, kCpThreads, 0, st>>>(s, slab_stride, row_stride, upr, n_slabs,
-                                                          n_rows_src, idx, idx_slab_stride, n_idx, d, status);
-  else if (unit == 4)
-    gather_rows<unsigned><<<(int)blocks, kCpThreads, 0, st>>>(s, slab_stride, row_stride, upr, n_slabs,
-                                                             n_rows_src, idx, idx_slab_stride, n_idx, d, status);
-  else
-    gather_rows<unsigned char><<<(int)blocks, kCpThreads, 0, st>>>(s, slab_stride, row_stride, upr,
-                                                                  n_slabs, n_rows_src, idx, idx_slab_stride, n_idx, d, status);
-  return cudaGetLastError();
+  const auto kernel = unit == 16 ? gather_rows<uint4> : unit == 4 ? gather_rows<unsigned> : gather_rows<unsigned char>;
+  return launch_pdl(kernel, dim3((unsigned)blocks), dim3(kCpThreads), 0, st, s, slab_stride, row_stride, upr, n_slabs,
+                    n_rows_src, idx, idx_slab_stride, n_idx, d, status);
 }
 
 }  // namespace skv

@@ -95,8 +95,6 @@ __device__ __forceinline__ float block_total(float v, float* red) {
 template <int VEC> struct Keys;
 template <> struct Keys<4> { using T = float4; };
 template <> struct Keys<1> { using T = float; };
-__device__ __forceinline__ void add_to(float4& s, const float4& v) { s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
-__device__ __forceinline__ void add_to(float& s, float v) { s += v; }
 __device__ __forceinline__ float4 decay(float l, const float4& c, const float4& s) {
   return make_float4(fmaf(l, c.x, s.x), fmaf(l, c.y, s.y), fmaf(l, c.z, s.z), fmaf(l, c.w, s.w));
 }
@@ -461,14 +459,20 @@ __global__ void head_metrics(const float* __restrict__ head_part, int n_layers, 
   metrics[l * 3 + 2] = var / (float)H;
 }
 
-// c_out[j] = sum_{l <= pivot} lambda^(pivot - l) s_hist[l][j], as the recursion c = lambda c + s.
-__global__ void accumulate(const float* __restrict__ s_hist, long long row_stride, int pivot, int n,
-                           float lambda, float* __restrict__ c_out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+// c_out[j] = sum_{l <= pivot} lambda^(pivot - l) s_hist[l][j], as the recursion c = lambda c + s; the loads of
+// eight layers are in flight together.
+template <int VEC>
+__global__ void __launch_bounds__(128) accumulate(const float* __restrict__ s_hist, long long row_stride, int pivot, int n,
+                                                  float lambda, float* __restrict__ c_out) {
+  using T = typename Keys<VEC>::T;
+  pdl_trigger();
+  pdl_wait();
+  const int j = (blockIdx.x * blockDim.x + threadIdx.x) * VEC;
   if (j >= n) return;
-  float c = 0.f;
-  for (int l = 0; l <= pivot; ++l) c = fmaf(lambda, c, s_hist[(size_t)l * row_stride + j]);
-  c_out[j] = c;
+  T c{};
+#pragma unroll 8
+  for (int l = 0; l <= pivot; ++l) c = decay(lambda, c, *reinterpret_cast<const T*>(s_hist + (size_t)l * row_stride + j));
+  *reinterpret_cast<T*>(c_out + j) = c;
 }
 
 }  // namespace
@@ -579,8 +583,9 @@ cudaError_t launch_head_stats_batch(const Ctx& ctx, const float* cols, long long
 
 cudaError_t launch_accumulate(const float* s_hist, long long row_stride, int pivot, int n,
                               float lambda, float* c_out, cudaStream_t st) {
-  accumulate<<<(n + 255) / 256, 256, 0, st>>>(s_hist, row_stride, pivot, n, lambda, c_out);
-  return cudaGetLastError();
+  if (n % 4 == 0 && row_stride % 4 == 0 && (uintptr_t)s_hist % 16 == 0 && (uintptr_t)c_out % 16 == 0)
+    return launch_pdl(accumulate<4>, dim3((n / 4 + 127) / 128), dim3(128), 0, st, s_hist, row_stride, pivot, n, lambda, c_out);
+  return launch_pdl(accumulate<1>, dim3((n + 127) / 128), dim3(128), 0, st, s_hist, row_stride, pivot, n, lambda, c_out);
 }
 
 }  // namespace skv

@@ -180,8 +180,11 @@ class Prefill:
         if last <= first:
             return
         self.ctx.select(self.s_red[first:last], self.kv_budget, self.w, self.i_red[first:last])
-        for l in range(first, last):
-            self.ctx.compact(self.pos_out[None, :, None], self.i_red[l], self.i_kv_pos[l][None, :, None])
+        # every layer gathers from the same position ids: one launch for (up to 128 of) them
+        pos = self.pos_out[None, :, None]
+        for lo in range(first, last, 128):
+            hi = min(last, lo + 128)
+            self.ctx.compact_layers([pos] * (hi - lo), self.i_red[lo:hi], self.i_kv_pos[lo:hi, None, :, None])
 
     def run(self, layers: Sequence[Dict[str, torch.Tensor]], hidden: Optional[torch.Tensor] = None,
             positions: Optional[torch.Tensor] = None) -> int:
