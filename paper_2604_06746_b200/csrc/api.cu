@@ -50,8 +50,7 @@ Workspace carve_workspace(const structkv_config& cfg, void* base) {
   w.stat_ctr = (int*)take(kMaxStatLayers * sizeof(int));
   w.chunk_ctr = (int*)take(n_pad / kKeyTile * sizeof(int));
   w.zero_bytes = off;
-  w.row_part = (float4*)take(std::max((size_t)kSimtParts * rows_pad * sizeof(float4),
-                                      tc_part_tasks(cfg, 1, false) * kRowBlock * sizeof(float2)));
+  w.row_part = (float2*)take(std::max(simt_part_entries(cfg, 1), tc_part_tasks(cfg, 1, false) * kRowBlock) * sizeof(float2));
   w.row_lse2 = (float*)take(rows_pad * sizeof(float));
   w.row_ent = (float*)take(rows_pad * sizeof(float));
   w.cols = (float*)take((size_t)cfg.n_q_heads * n_pad * sizeof(float));
@@ -148,17 +147,10 @@ structkv_status structkv_score_layer(structkv_ctx* ctx, const void* q_window, co
 
   float* cols = head_cols_out ? head_cols_out : c.ws.cols;
   const long long col_stride = head_cols_out ? (long long)n_keys : (long long)c.n_pad;
-  if (cfg.dtype == STRUCTKV_BF16 && !(flags & STRUCTKV_FLAG_FORCE_SIMT) && tc_supported(c, k_stride_head, k_stride_token)) {
-    const TcCall a{1, &q_window, &k, &scale, nullptr, k_stride_head, k_stride_token, n_keys, cols, 0, col_stride,
-                   (float2*)c.ws.row_part, c.ws.row_lse2, c.ws.row_ent};
-    if (launch_score_tc(c, a, st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
-  } else {
-    const ScoreArgs a{q_window, k, k_stride_head, k_stride_token, n_keys, scale, cols, col_stride};
-    int parts = 0;
-    if (launch_score_simt(c, a, &parts, 1, st) != cudaSuccess || launch_finalize_rows(c, parts, st) != cudaSuccess ||
-        launch_score_simt(c, a, &parts, 2, st) != cudaSuccess)
-      return STRUCTKV_ERR_CUDA;
-  }
+  const ScoreCall a{1, &q_window, &k, &scale, nullptr, k_stride_head, k_stride_token, n_keys, cols, 0, col_stride,
+                    c.ws.row_part, c.ws.row_lse2, c.ws.row_ent};
+  const bool use_tc = !(flags & STRUCTKV_FLAG_FORCE_SIMT) && tc_supported(c, k_stride_head, k_stride_token);
+  if ((use_tc ? launch_score_tc(c, a, st) : launch_score_simt(c, a, st)) != cudaSuccess) return STRUCTKV_ERR_CUDA;
   return launch_finish_layers(c, cols, 0, col_stride, n_keys, 1, lambda, s_out, 0, c_inout, c.ws.row_ent,
                               !(flags & STRUCTKV_FLAG_NO_HEAD_STATS), metrics_out, st) == cudaSuccess ? STRUCTKV_OK : STRUCTKV_ERR_CUDA;
 }
@@ -225,7 +217,7 @@ structkv_status structkv_score_layer_batch(structkv_ctx* ctx, const void* q_wind
   if (cfg.dtype != STRUCTKV_BF16 || !tc_supported(c, k_stride_head, k_stride_token)) return STRUCTKV_ERR_UNSUPPORTED;
   float* cols = head_cols_out ? head_cols_out : bw.cols;
   const long long col_stride = head_cols_out ? (long long)total : (long long)align_up((size_t)total, kKeyTile);
-  const TcCall a{batch, &q_window, &k, &scale, cu_seqlens, k_stride_head, k_stride_token, 0, cols, 0, col_stride,
+  const ScoreCall a{batch, &q_window, &k, &scale, cu_seqlens, k_stride_head, k_stride_token, 0, cols, 0, col_stride,
                  bw.row_part, bw.nlse, bw.row_ent};
   if (launch_score_tc(c, a, st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
   return launch_finish_packed(c, cols, col_stride, cu_seqlens, batch, lambda, s_out, c_inout, bw.row_ent, bw.head_part,
@@ -247,7 +239,9 @@ static LayersWs carve_layers(const structkv_config& cfg, int max_layers, void* b
     return r;
   };
   const size_t rows_pad = (size_t)rows_pad_of(cfg);
-  w.row_part = (float2*)take(tc_part_tasks(cfg, max_layers, false) * kRowBlock * sizeof(float2));
+  // (fp32 storage never runs on the tensor cores, bf16 storage on the CUDA cores layer after layer)
+  w.row_part = (float2*)take((cfg.dtype == STRUCTKV_FP32 ? simt_part_entries(cfg, max_layers)
+                                                         : tc_part_tasks(cfg, max_layers, false) * kRowBlock) * sizeof(float2));
   w.nlse = (float*)take((size_t)std::min(max_layers, kMaxBatch) * rows_pad * sizeof(float));
   w.row_ent = (float*)take((size_t)max_layers * rows_pad * sizeof(float));
   w.bytes = off;
@@ -287,8 +281,9 @@ structkv_status structkv_score_layers(structkv_ctx* ctx, int n_layers, const voi
       return STRUCTKV_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
 
-  if (cfg.dtype != STRUCTKV_BF16 || !tc_supported(c, k_stride_head, k_stride_token)) {
-    // the CUDA-core scorer has no interleaved form: one layer after the other, same results
+  const bool use_tc = tc_supported(c, k_stride_head, k_stride_token);
+  if (!use_tc && (cfg.dtype == STRUCTKV_BF16 || !layers_workspace)) {
+    // bf16 layers the tensor cores do not take: one after the other, same results
     for (int l = 0; l < n_layers; ++l) {
       const structkv_status s = structkv_score_layer(
           ctx, q_windows[l], ks[l], k_stride_head, k_stride_token, n_keys, scales[l], lambda,
@@ -302,9 +297,9 @@ structkv_status structkv_score_layers(structkv_ctx* ctx, int n_layers, const voi
   if (!layers_workspace || layers_workspace_bytes < need || ((uintptr_t)layers_workspace % 256) != 0)
     return STRUCTKV_ERR_WORKSPACE;
   const LayersWs lw = carve_layers(cfg, n_layers, layers_workspace);
-  const TcCall a{n_layers, q_windows, ks, scales, nullptr, k_stride_head, k_stride_token, n_keys, head_cols_out,
+  const ScoreCall a{n_layers, q_windows, ks, scales, nullptr, k_stride_head, k_stride_token, n_keys, head_cols_out,
                  head_cols_layer_stride, n_keys, lw.row_part, lw.nlse, lw.row_ent};
-  if (launch_score_tc(c, a, st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
+  if ((use_tc ? launch_score_tc(c, a, st) : launch_score_simt(c, a, st)) != cudaSuccess) return STRUCTKV_ERR_CUDA;
   return launch_finish_layers(c, head_cols_out, head_cols_layer_stride, n_keys, n_keys, n_layers, lambda, s_out,
                               s_layer_stride, c_inout, lw.row_ent, false, metrics_out, st) == cudaSuccess
              ? STRUCTKV_OK

@@ -18,6 +18,7 @@ constexpr int kMaxStatLayers = 128;   // layers one batched head-statistics call
 constexpr int kMaxGatherLayers = 128; // layers one multi-layer gather may cover (their pointers are a kernel argument)
 constexpr int kQueueUnits = 256;      // (KV group, row block) units of one problem the tensor-core scorer can hold
 constexpr int kCtlInts = 64 + 2 * kMaxBatch * kQueueUnits;   // its control block: tickets, arrivals, ready flags
+constexpr int kMergeGroup = 6;         // partials of a row merged together
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 
@@ -25,9 +26,9 @@ constexpr float kLn2 = 0.6931471805599453f;
 struct Workspace {
   int* status;          // [64] ints, word 0 is the status
   int* ctl;             // [kCtlInts], follows the status block; zero between scorer launches (a launch leaves it zero)
-  float4* row_part;     // partial softmax statistics: CUDA cores [kSimtParts][rows_pad] (m2, Z, U, -), tensor cores
-                        // float2 [pass-1 task][kRowBlock]
-  float* row_lse2;      // [rows_pad] log2-domain log-sum-exp of each score row (tensor cores: negated)
+  float2* row_part;     // partial softmax statistics of score rows: CUDA cores [kSimtParts][rows_pad], tensor cores
+                        // [pass-1 task][kRowBlock]
+  float* row_lse2;      // [rows_pad] negated log2-domain log-sum-exp of each score row (tensor cores)
   float* row_ent;       // [rows_pad] entropy of each score row (nats), 0 where there is no row
   float* cols;          // [H][n_pad] pooled per-head attention when the caller passes none
   float* head_part;     // [kMaxStatLayers][H][4] per-(layer, head) {sum of squared deviations from 1/n, top-k mass}
@@ -43,7 +44,7 @@ struct Ctx {
   int device;
   int sm_count;
   int rows;             // H * w
-  int w_pad;            // rows a head occupies in the tensor-core scorer's blocks: w up to a power of two, at least 8
+  int w_pad;            // rows a head occupies in a scorer's row blocks: w up to a power of two, at least 8
   int rows_pad;         // rows per KV group (heads at w_pad rows) padded to kRowBlock, times H_kv
   int n_pad;            // max_seq rounded up to kKeyTile
   void* tc;             // tensor-core scorer state (tensor-map encoder), owned by score_tc.cu
@@ -55,23 +56,9 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 Workspace carve_workspace(const structkv_config& cfg, void* base);
 
 // ---- launchers (each returns cudaGetLastError() of its launches) -------------------------
-struct ScoreArgs {
-  const void* q;            // [H, w, d]
-  const void* k;
-  long long k_stride_head, k_stride_token;   // elements
-  int n_keys;
-  float scale;
-  float* cols;              // [H][col_stride] pooled per-head attention (output of pass 2)
-  long long col_stride;
-};
-
-// CUDA-core two-pass scorer (fp32 or bf16 storage).  parts_out = key segments per row.
-cudaError_t launch_score_simt(const Ctx& ctx, const ScoreArgs& a, int* parts_out, int pass,
-                              cudaStream_t st);
-
-// Tensor-core (tcgen05) scorer for bf16 storage: both passes over `n` problems (layers of one shape, or
-// the sequences of a packed batch), one launch per kMaxBatch layers.
-struct TcCall {
+// Both scorer passes over `n` problems: layers of one shape, or (tensor cores only) the sequences of a
+// packed batch.
+struct ScoreCall {
   int n;                          // layers, or sequences
   const void* const* q;           // layers: [n]; batch: one tensor [n, H, w, d]
   const void* const* k;           // layers: [n]; batch: one packed tensor
@@ -81,24 +68,25 @@ struct TcCall {
   int n_keys;                     // keys of a layer
   float* cols;                    // layer l at cols + l * cols_layer_stride; sequence b at column cu_seqlens[b]
   long long cols_layer_stride, col_stride;
-  float2* part;                   // tc_part_tasks(...) * kRowBlock entries
-  float* nlse;                    // [min(n, kMaxBatch)][rows_pad]
+  float2* part;                   // tensor cores: tc_part_tasks(...) * kRowBlock entries; CUDA cores: simt_part_entries(...)
+  float* nlse;                    // tensor cores: [min(n, kMaxBatch)][rows_pad]
   float* row_ent;                 // [n][rows_pad]
 };
+// CUDA cores: fp32 storage, and what the tensor-core scorer does not take.
+size_t simt_part_entries(const structkv_config& cfg, int n);
+cudaError_t launch_score_simt(const Ctx& ctx, const ScoreCall& a, cudaStream_t st);
+// Tensor cores (tcgen05): bf16 storage; one launch per kMaxBatch layers.
 bool tc_supported(const Ctx& ctx, long long k_stride_head, long long k_stride_token);
 int tc_window_pad(int window);
 // pass-1 tasks (partial statistics of kRowBlock rows) a launch over n problems needs room for
 size_t tc_part_tasks(const structkv_config& cfg, int n, bool batch);
 structkv_status tc_create(Ctx& ctx);
 void tc_destroy(Ctx& ctx);
-cudaError_t launch_score_tc(const Ctx& ctx, const TcCall& a, cudaStream_t st);
+cudaError_t launch_score_tc(const Ctx& ctx, const ScoreCall& a, cudaStream_t st);
 
 // One thread waits (bounded by limit_cycles) on a barrier nobody arrives on, then records
 // STRUCTKV_ERR_TIMEOUT in *status.
 cudaError_t launch_wait_probe(unsigned long long limit_cycles, int* status, cudaStream_t st);
-
-// Merges the per-segment softmax statistics of every row into row_lse2 / row_ent (CUDA-core scorer).
-cudaError_t launch_finalize_rows(const Ctx& ctx, int parts, cudaStream_t st);
 
 // After the scorer passes of n_layers layers: S^(l)_j = sum_h cols[l][h][j] (rows s_stride apart), C <-
 // lambda C + S^(l) carried from layer to layer if c_inout, metrics[l][0] from row_ent[l][rows_pad] (Eq. 4) and
@@ -173,4 +161,35 @@ __device__ __forceinline__ float fast_exp2(float x) {
   return y;
 }
 
+// One row's softmax statistics over some keys: Z = sum 2^(x - ref), U = sum 2^(x - ref) (x - ref).
+struct RowStat { float ref, Z, U; };
+
+// A row's partial as it is stored: (l, h), its log-sum-exp l = ref + log2 Z and the entropy of the
+// softmax over its keys alone, h = log2 Z - U / Z (both in bits); (-inf, 0) where it saw no key of the
+// row.  Over a row's partials, lse = log2 sum 2^l and with w = 2^(l - lse) the row's entropy is
+// sum w (h + lse - l)  (Eq. 4, one row).  The compute warps take the logarithm and the division, and
+// loads of four rows are in flight together: merging is one warp's work beside sixteen busy ones,
+// and pass 2 waits for it (18 partials of 256 rows: 35 us with one row and one logarithm at a time).
+__device__ __forceinline__ float2 stat_partial(const RowStat& r) {
+  const float lz = __log2f(r.Z);
+  return r.Z > 0.f ? make_float2(r.ref + lz, lz - __fdividef(r.U, r.Z)) : make_float2(-INFINITY, 0.f);
+}
+// Adds partials to (M, W, X): lse so far = M + log2 W, X = sum 2^(l - M) (h - l + M).
+template <int N>
+__device__ __forceinline__ void merge_partials(float& M, float& W, float& X, const float2 (&pv)[N]) {
+  float top = M;
+#pragma unroll
+  for (int b = 0; b < N; ++b) top = fmaxf(top, pv[b].x);
+  if (top == -INFINITY) return;
+  const float d = M == -INFINITY ? 0.f : M - top, f = fast_exp2(d);
+  X = f * fmaf(-d, W, X);
+  W *= f;
+  M = top;
+#pragma unroll
+  for (int b = 0; b < N; ++b) {
+    const float e = pv[b].x == -INFINITY ? -200.f : pv[b].x - top, w = fast_exp2(e);
+    W += w;
+    X = fmaf(w, pv[b].y - e, X);
+  }
+}
 }  // namespace skv

@@ -1,4 +1,4 @@
-// Small deterministic reductions around the scorers: row finalisation (CUDA-core scorer), the sum
+// Small deterministic reductions after the scorers: the sum
 // over heads with the centrality update, per-head sparsity / variance with the layer's metrics, and
 // the closed-form centrality re-accumulation.
 #include <atomic>
@@ -7,45 +7,6 @@
 
 namespace skv {
 namespace {
-
-// One thread per score row.  Row r of group g is valid iff its index inside the group is
-// < rows_pg.  Each of the `parts` key segments left (ref, Z, U) for the row: Z = sum 2^(x - ref),
-// U = sum 2^(x - ref) (x - ref), x = logit * log2(e); ref is any reference the segment chose.
-// With l_p = ref_p + log2 Z_p (the segment's log-sum-exp) and M = max_p l_p:
-//   lse2 = M + log2 sum_p 2^(l_p - M)
-//   mean of (x - M) under the row's softmax = sum_p 2^(l_p - M) (ref_p - M + U_p / Z_p) / sum_p 2^(l_p - M)
-//   entropy = ln2 * (lse2 - M - that mean)                                   (Eq. 4, one row)
-__global__ void __launch_bounds__(256)
-finalize_rows(const float4* __restrict__ row_part, int parts, int rows_pad, int rows_pg_pad,
-              int rows_pg, float* __restrict__ row_lse2, float* __restrict__ row_ent) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= rows_pad) return;
-  const bool valid = (r % rows_pg_pad) < rows_pg;
-  float lse2 = INFINITY, ent = 0.f;        // padded rows: 2^(x - inf) = 0 in pass 2
-  if (valid) {
-    float M = -INFINITY;
-    for (int p = 0; p < parts; ++p) {
-      const float4 v = row_part[(size_t)p * rows_pad + r];
-      if (v.y > 0.f) M = fmaxf(M, v.x + log2f(v.y));
-    }
-    if (M != -INFINITY) {
-      float Zt = 0.f, Xt = 0.f;
-      for (int p = 0; p < parts; ++p) {
-        const float4 v = row_part[(size_t)p * rows_pad + r];
-        if (v.y > 0.f) {
-          const float wgt = fast_exp2(v.x + log2f(v.y) - M);
-          Zt += wgt;
-          Xt = fmaf(wgt, (v.x - M) + v.z / v.y, Xt);
-        }
-      }
-      const float lz = log2f(Zt);
-      lse2 = M + lz;
-      ent = kLn2 * (lz - Xt / Zt);
-    }
-  }
-  row_lse2[r] = lse2;
-  row_ent[r] = ent;
-}
 
 // ---- what follows the scorer passes of a layer, of several layers or of a packed batch ----------
 // One launch: CTAs of clusters first (one cluster per (problem, head) vector, Eq. 5-6), then blocks
@@ -476,15 +437,6 @@ __global__ void __launch_bounds__(128) accumulate(const float* __restrict__ s_hi
 }
 
 }  // namespace
-
-cudaError_t launch_finalize_rows(const Ctx& ctx, int parts, cudaStream_t st) {
-  const int rows_pg_pad = ctx.rows_pad / ctx.cfg.n_kv_heads;
-  const int rows_pg = (ctx.cfg.n_q_heads / ctx.cfg.n_kv_heads) * ctx.cfg.window;
-  finalize_rows<<<(ctx.rows_pad + 255) / 256, 256, 0, st>>>(ctx.ws.row_part, parts, ctx.rows_pad,
-                                                           rows_pg_pad, rows_pg, ctx.ws.row_lse2,
-                                                           ctx.ws.row_ent);
-  return cudaGetLastError();
-}
 
 // Raises a kernel's shared-memory limit once per device.
 template <typename K>

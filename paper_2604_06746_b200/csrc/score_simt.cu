@@ -1,197 +1,289 @@
-// CUDA-core two-pass scorer: window logits, row softmax statistics (pass 1) and pooled
-// per-head attention columns (pass 2).  Serves fp32 storage and any shape the tensor-core
-// scorer does not take.  Everything is fp32 arithmetic in the log2 domain.
+// CUDA-core two-pass scorer: window logits, row softmax statistics (pass 1) and pooled per-head
+// attention columns (pass 2), all layers of a call in one launch per pass.  Serves fp32 storage and
+// what the tensor-core scorer does not take.  Everything is fp32 arithmetic in the log2 domain.
 //
-// Row numbering (shared with the tensor-core scorer and the finalize kernel): score row
-// (h, i) of KV group g = h / G lives at  g * rows_per_group_pad + (h % G) * w + i.
+// Score rows are numbered as in the tensor-core scorer: row (h, i) of KV group g = h / G lives at
+// g * rows_pg_pad + (h % G) * w_pad + i.  A block multiplies 128 rows with 64 keys, 8 x 4 per thread,
+// both operands in shared memory with the head dimension outermost: 32 multiply-adds for three
+// 16-byte loads.  Bound by the FMA pipe on long sequences and by latency on short ones (8 heads,
+// window 32, head dim 64, 2048 keys: a layer took 15 + 21 + 18 us with one dot product per lane, a
+// pass that merged the partials and one key per thread; four layers now take 10 us together).
+#include <algorithm>
+#include <atomic>
+
 #include "common.cuh"
 
 namespace skv {
 namespace {
 
-constexpr int kP1Keys = 64;      // keys per pass-1 chunk
-constexpr int kP1Threads = 256;
-constexpr int kP2Threads = 128;  // one key per thread in pass 2
+constexpr int kSmRows = 128, kSmKeys = 64, kSmThreads = 256;
+constexpr int kSmLayers = 32;              // layers per launch (their pointers are a kernel argument)
 
-template <typename T> __device__ __forceinline__ float to_f32(T v);
-template <> __device__ __forceinline__ float to_f32<float>(float v) { return v; }
-template <> __device__ __forceinline__ float to_f32<__nv_bfloat16>(__nv_bfloat16 v) {
-  return __bfloat162float(v);
+struct SimtArgs {
+  const void *q[kSmLayers], *k[kSmLayers];
+  float c2[kSmLayers];
+  long long sh, st;
+  int N, w, w_pad, group, rows_pg, rows_pg_pad, rows_pad, n_rt, parts, n_keys_tiles;
+  float2* part;                            // [layer][parts][rows_pad]
+  float* row_ent;                          // [layer][rows_pad]
+  float* cols;
+  long long cols_layer_stride, col_stride;
+};
+
+__device__ __forceinline__ float4 load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  const uint2 u = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u), __uint_as_float(u.y << 16),
+                     __uint_as_float(u.y & 0xffff0000u));
 }
 
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
+template <int D>
+struct SimtShared {
+  float q[D][kSmRows + 4];                 // [column][row]
+  float k[D][kSmKeys + 4];
+  union {
+    float lse[kSmRows];                    // pass 2: -log2-sum-exp of the tile's rows
+    float2 half[kSmRows];
+  };
+  float col[kSmRows / 8][kSmKeys];         // pass 2: sums over eight rows
+};
 
-// Pass 1.  grid = (parts, H).  Each block sweeps its key segment in chunks of kP1Keys keys;
-// a warp owns window rows i = warp, warp + 8, ... and its lanes own the keys of the chunk.
-// Per row it keeps (m2, Z, U): running max of x = logit*log2e, Z = sum 2^(x-m2),
-// U = sum 2^(x-m2) (x-m2).
+// Stages 128 score rows (tile rt of group g) with the head dimension outermost; padding is zero.
 template <typename T, int D>
-__global__ void __launch_bounds__(kP1Threads)
-simt_pass1(const T* __restrict__ q, const T* __restrict__ k, long long sh, long long st, int N,
-           int w, int G, float c2, int parts, int rows_pg_pad, int rows_pad,
-           float4* __restrict__ row_part) {
-  extern __shared__ float smem[];
-  float* qs = smem;                         // [w][D]
-  float* ks = qs + (size_t)w * D;           // [kP1Keys][D + 1]
-  float* sm = ks + kP1Keys * (D + 1);       // [w] m2
-  float* sz = sm + w;                       // [w] Z
-  float* su = sz + w;                       // [w] U
-  const int h = blockIdx.y, g = h / G, part = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-  for (int x = tid; x < w * D; x += kP1Threads) qs[x] = to_f32<T>(q[(size_t)h * w * D + x]);
-  for (int x = tid; x < w; x += kP1Threads) { sm[x] = -INFINITY; sz[x] = 0.f; su[x] = 0.f; }
-
-  const int n_chunks = (N + kP1Keys - 1) / kP1Keys;
-  const int c_lo = (int)((long long)part * n_chunks / parts);
-  const int c_hi = (int)((long long)(part + 1) * n_chunks / parts);
-  const T* kg = k + (size_t)g * sh;
-
-  for (int c = c_lo; c < c_hi; ++c) {
-    const int j0 = c * kP1Keys;
-    __syncthreads();
-    for (int x = tid; x < kP1Keys * D; x += kP1Threads) {
-      const int key = x / D, col = x - key * D, j = j0 + key;
-      ks[key * (D + 1) + col] = (j < N) ? to_f32<T>(kg[(size_t)j * st + col]) : 0.f;
-    }
-    __syncthreads();
-    for (int i = warp; i < w; i += kP1Threads / 32) {
-      const int t = N - w + i;
-      const float* qi = qs + (size_t)i * D;
-      float xs[kP1Keys / 32];
-      float mx = -INFINITY;
+__device__ __forceinline__ void stage_rows(const SimtArgs& a, const T* q, int g, int rt, float (*dst)[kSmRows + 4]) {
+  for (int x = threadIdx.x; x < kSmRows * (D / 4); x += kSmThreads) {
+    const int r = x % kSmRows, c = x / kSmRows * 4, row = rt * kSmRows + r, i = row % a.w_pad;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (row < a.rows_pg && i < a.w) v = load4(q + ((size_t)(g * a.group + row / a.w_pad) * a.w + i) * D + c);
+    dst[c][r] = v.x; dst[c + 1][r] = v.y; dst[c + 2][r] = v.z; dst[c + 3][r] = v.w;
+  }
+}
+template <typename T, int D>
+__device__ __forceinline__ void stage_keys(const SimtArgs& a, const T* k, int j0, float (*dst)[kSmKeys + 4]) {
+  for (int x = threadIdx.x; x < kSmKeys * (D / 4); x += kSmThreads) {
+    const int r = x % kSmKeys, c = x / kSmKeys * 4;
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (j0 + r < a.N) v = load4(k + (size_t)(j0 + r) * a.st + c);
+    dst[c][r] = v.x; dst[c + 1][r] = v.y; dst[c + 2][r] = v.z; dst[c + 3][r] = v.w;
+  }
+}
+// acc[r][c] = q(row tr * 8 + r) . k(key tc * 4 + c)
+template <int D>
+__device__ __forceinline__ void multiply(const SimtShared<D>& s, int tr, int tc, float (&acc)[8][4]) {
 #pragma unroll
-      for (int kk = 0; kk < kP1Keys / 32; ++kk) {
-        const int key = lane + 32 * kk;
-        const float* kr = ks + key * (D + 1);
-        float s = 0.f;
+  for (int r = 0; r < 8; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
 #pragma unroll 8
-        for (int col = 0; col < D; ++col) s = fmaf(qi[col], kr[col], s);
-        xs[kk] = (j0 + key <= t) ? s * c2 : -INFINITY;
-        mx = fmaxf(mx, xs[kk]);
-      }
-      mx = warp_max(mx);
-      if (mx == -INFINITY) continue;        // the whole chunk is masked for this row
-      const float m_old = sm[i];
-      const float m_new = fmaxf(m_old, mx);
-      float zs = 0.f, us = 0.f;
+  for (int d = 0; d < D; ++d) {
+    const float4 q0 = *reinterpret_cast<const float4*>(&s.q[d][tr * 8]), q1 = *reinterpret_cast<const float4*>(&s.q[d][tr * 8 + 4]);
+    const float4 kv = *reinterpret_cast<const float4*>(&s.k[d][tc * 4]);
+    const float qr[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w}, kc[4] = {kv.x, kv.y, kv.z, kv.w};
 #pragma unroll
-      for (int kk = 0; kk < kP1Keys / 32; ++kk) {
-        if (xs[kk] != -INFINITY) {
-          const float dx = xs[kk] - m_new;
-          const float p = fast_exp2(dx);
-          zs += p;
-          us = fmaf(p, dx, us);
-        }
-      }
-      zs = warp_sum(zs);
-      us = warp_sum(us);
-      if (lane == 0) {
-        float Z = sz[i], U = su[i];
-        if (m_old != -INFINITY) {
-          const float dm = m_old - m_new, f = fast_exp2(dm);
-          U = f * fmaf(dm, Z, U);
-          Z = f * Z;
-        }
-        sm[i] = m_new; sz[i] = Z + zs; su[i] = U + us;
-      }
-      __syncwarp();
-    }
-  }
-  __syncthreads();
-  for (int i = tid; i < w; i += kP1Threads) {
-    const int r = g * rows_pg_pad + (h % G) * w + i;
-    row_part[(size_t)part * rows_pad + r] = make_float4(sm[i], sz[i], su[i], 0.f);
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(qr[r], kc[c], acc[r][c]);
   }
 }
 
-// Pass 2.  grid = (ceil(N / 128), H); thread = key.  cols[h][j] = (1/w) sum_i 2^(x_ij - lse2_i).
+// Pass 1.  grid = (parts, row tiles x groups, layers): statistics of 128 rows over one key segment.
 template <typename T, int D>
-__global__ void __launch_bounds__(kP2Threads)
-simt_pass2(const T* __restrict__ q, const T* __restrict__ k, long long sh, long long st, int N,
-           int w, int G, float c2, int rows_pg_pad, const float* __restrict__ row_lse2,
-           float* __restrict__ cols, long long col_stride) {
-  extern __shared__ float smem[];
-  float* qs = smem;                         // [w][D]
-  float* ls = qs + (size_t)w * D;           // [w]
-  const int h = blockIdx.y, g = h / G, tid = threadIdx.x;
-  for (int x = tid; x < w * D; x += kP2Threads) qs[x] = to_f32<T>(q[(size_t)h * w * D + x]);
-  for (int x = tid; x < w; x += kP2Threads) ls[x] = row_lse2[g * rows_pg_pad + (h % G) * w + x];
-  __syncthreads();
-  const int j = blockIdx.x * kP2Threads + tid;
-  if (j >= N) return;
-  float kr[D];
-  const T* kp = k + (size_t)g * sh + (size_t)j * st;
+__global__ void __launch_bounds__(kSmThreads) simt_pass1(const __grid_constant__ SimtArgs a) {
+  extern __shared__ __align__(16) unsigned char simt_smem[];
+  SimtShared<D>& s = *reinterpret_cast<SimtShared<D>*>(simt_smem);
+  pdl_trigger();
+  pdl_wait();
+  const int part = blockIdx.x, g = blockIdx.y / a.n_rt, rt = blockIdx.y - g * a.n_rt, layer = blockIdx.z;
+  const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;
+  const T* kg = (const T*)a.k[layer] + (size_t)g * a.sh;
+  const float c2 = a.c2[layer];
+  stage_rows<T, D>(a, (const T*)a.q[layer], g, rt, s.q);
+  RowStat st[8];
 #pragma unroll
-  for (int col = 0; col < D; ++col) kr[col] = to_f32<T>(kp[col]);
-  float acc = 0.f;
-  const int i_first = max(0, j - (N - w));   // rows i < i_first do not see key j
-  for (int i = i_first; i < w; ++i) {
-    const float4* qi = reinterpret_cast<const float4*>(qs + (size_t)i * D);
-    float s0 = 0.f, s1 = 0.f;
+  for (int r = 0; r < 8; ++r) st[r] = RowStat{-INFINITY, 0.f, 0.f};
+  const int t_lo = (int)((long long)part * a.n_keys_tiles / a.parts), t_hi = (int)((long long)(part + 1) * a.n_keys_tiles / a.parts);
+  for (int t = t_lo; t < t_hi; ++t) {
+    const int j0 = t * kSmKeys;
+    stage_keys<T, D>(a, kg, j0, s.k);
+    __syncthreads();
+    float acc[8][4];
+    multiply<D>(s, tr, tc, acc);
+    __syncthreads();
 #pragma unroll
-    for (int c4 = 0; c4 < D / 4; c4 += 2) {
-      const float4 a = qi[c4], b = qi[c4 + 1];
-      s0 = fmaf(a.x, kr[4 * c4 + 0], s0); s0 = fmaf(a.y, kr[4 * c4 + 1], s0);
-      s0 = fmaf(a.z, kr[4 * c4 + 2], s0); s0 = fmaf(a.w, kr[4 * c4 + 3], s0);
-      s1 = fmaf(b.x, kr[4 * c4 + 4], s1); s1 = fmaf(b.y, kr[4 * c4 + 5], s1);
-      s1 = fmaf(b.z, kr[4 * c4 + 6], s1); s1 = fmaf(b.w, kr[4 * c4 + 7], s1);
+    for (int r = 0; r < 8; ++r) {
+      const int t_pos = a.N - a.w + (rt * kSmRows + tr * 8 + r) % a.w_pad;      // the row's position: it sees keys <= t_pos
+      float x[4], mx = -INFINITY;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        x[c] = j0 + tc * 4 + c <= t_pos && j0 + tc * 4 + c < a.N ? acc[r][c] * c2 : -INFINITY;
+        mx = fmaxf(mx, x[c]);
+      }
+      if (mx > st[r].ref) {
+        if (st[r].ref != -INFINITY) {
+          const float dm = st[r].ref - mx, f = fast_exp2(dm);
+          st[r].U = f * fmaf(dm, st[r].Z, st[r].U);
+          st[r].Z *= f;
+        }
+        st[r].ref = mx;
+      }
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (x[c] != -INFINITY) {
+          const float dx = x[c] - st[r].ref, pe = fast_exp2(dx);
+          st[r].Z += pe;
+          st[r].U = fmaf(pe, dx, st[r].U);
+        }
     }
-    acc += fast_exp2(fmaf(s0 + s1, c2, -ls[i]));
   }
-  cols[(size_t)h * col_stride + j] = acc / (float)w;
+  // the 16 threads of a row fold into one partial
+#pragma unroll
+  for (int r = 0; r < 8; ++r) {
+    float M = st[r].ref;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
+    const float dm = st[r].ref == -INFINITY ? 0.f : st[r].ref - M, f = fast_exp2(dm);
+    float Z = f * st[r].Z, U = f * fmaf(dm, st[r].Z, st[r].U);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      Z += __shfl_xor_sync(0xffffffffu, Z, o);
+      U += __shfl_xor_sync(0xffffffffu, U, o);
+    }
+    const int row = rt * kSmRows + tr * 8 + r;
+    if (tc == r && row < a.rows_pg_pad)
+      a.part[((size_t)layer * a.parts + part) * a.rows_pad + g * a.rows_pg_pad + row] = stat_partial(RowStat{M, Z, U});
+  }
+}
+
+// Pass 2.  grid = (key tiles, row tiles x groups, layers): merges the rows' partials, then
+// cols[h][j] = (1/w) sum_i 2^(x_ij - lse_i) for the heads of 128 rows (a head of 256 rows takes two tiles).
+template <typename T, int D>
+__global__ void __launch_bounds__(kSmThreads) simt_pass2(const __grid_constant__ SimtArgs a) {
+  extern __shared__ __align__(16) unsigned char simt_smem[];
+  SimtShared<D>& s = *reinterpret_cast<SimtShared<D>*>(simt_smem);
+  pdl_trigger();
+  const int span = a.w_pad > kSmRows ? a.w_pad / kSmRows : 1, n_rs = a.n_rt / span;   // row tiles a block takes
+  const int j0 = blockIdx.x * kSmKeys, g = blockIdx.y / n_rs, rs = blockIdx.y - g * n_rs, layer = blockIdx.z;
+  const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;
+  const float c2 = a.c2[layer];
+  pdl_wait();
+  if (j0 == 0 && rs == n_rs - 1)                        // rows of the group's last block that no tile holds
+    for (int row = a.n_rt * kSmRows + threadIdx.x; row < a.rows_pg_pad; row += kSmThreads)
+      a.row_ent[(size_t)layer * a.rows_pad + g * a.rows_pg_pad + row] = 0.f;
+  stage_keys<T, D>(a, (const T*)a.k[layer] + (size_t)g * a.sh, j0, s.k);
+  float total = 0.f;                                   // heads longer than a tile
+  for (int m = 0; m < span; ++m) {
+    const int rt = rs * span + m;
+    stage_rows<T, D>(a, (const T*)a.q[layer], g, rt, s.q);
+    // two threads per row, each half of the partials
+    const int r = threadIdx.x & (kSmRows - 1), hp = threadIdx.x / kSmRows, row = rt * kSmRows + r;
+    const int p_lo = hp * a.parts / 2, p_hi = (hp + 1) * a.parts / 2;
+    float M = -INFINITY, W = 0.f, X = 0.f;
+    const bool valid = row < a.rows_pg && row % a.w_pad < a.w;
+    if (valid) {
+      constexpr int kBatch = 8;
+      for (int p0 = p_lo; p0 < p_hi; p0 += kBatch) {
+        float2 pv[kBatch];
+#pragma unroll
+        for (int b = 0; b < kBatch; ++b)
+          pv[b] = p0 + b < p_hi ? __ldcg(a.part + ((size_t)layer * a.parts + p0 + b) * a.rows_pad + g * a.rows_pg_pad + row)
+                                : make_float2(-INFINITY, 0.f);
+        merge_partials(M, W, X, pv);
+      }
+    }
+    const float lw = __log2f(W);
+    if (hp == 1) s.half[r] = W > 0.f ? make_float2(M + lw, lw + X / W) : make_float2(-INFINITY, 0.f);
+    __syncthreads();
+    float lse = INFINITY;                              // rows that do not exist: 2^(x - inf) = 0
+    if (hp == 0) {
+      const float2 o[1] = {s.half[r]};
+      merge_partials(M, W, X, o);
+      const float lz = __log2f(W);
+      if (valid && W > 0.f) lse = M + lz;
+      if (j0 == 0 && row < a.rows_pg_pad)
+        a.row_ent[(size_t)layer * a.rows_pad + g * a.rows_pg_pad + row] = valid && W > 0.f ? kLn2 * (lz + X / W) : 0.f;
+    }
+    __syncthreads();
+    if (hp == 0) s.lse[r] = lse;
+    __syncthreads();
+    float acc[8][4], sum[4] = {0.f, 0.f, 0.f, 0.f};
+    multiply<D>(s, tr, tc, acc);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int i = (rt * kSmRows + tr * 8 + q) % a.w_pad, t_pos = a.N - a.w + i;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float pe = fast_exp2(fmaf(acc[q][c], c2, -s.lse[tr * 8 + q]));
+        sum[c] += j0 + tc * 4 + c <= t_pos ? pe : 0.f;
+      }
+    }
+    *reinterpret_cast<float4*>(&s.col[tr][tc * 4]) = make_float4(sum[0], sum[1], sum[2], sum[3]);
+    __syncthreads();
+    // sums over a head's groups of eight rows
+    const int per_head = min(a.w_pad, kSmRows) / 8, heads = kSmRows / 8 / per_head;
+    for (int x = threadIdx.x; x < heads * kSmKeys; x += kSmThreads) {
+      const int hh = x / kSmKeys, j = x % kSmKeys;
+      float t = 0.f;
+      for (int e = 0; e < per_head; ++e) t += s.col[hh * per_head + e][j];
+      total += t;
+      const int head = (rt * kSmRows) / a.w_pad + hh;
+      if (m == span - 1 && head < a.group && j0 + j < a.N)
+        a.cols[(size_t)layer * a.cols_layer_stride + (size_t)(g * a.group + head) * a.col_stride + j0 + j] =
+            (span > 1 ? total : t) / (float)a.w;
+    }
+    __syncthreads();
+  }
 }
 
 template <typename T, int D>
-cudaError_t launch_typed(const Ctx& ctx, const ScoreArgs& a, int* parts_out, int pass,
-                         cudaStream_t st) {
-  const int H = ctx.cfg.n_q_heads, G = H / ctx.cfg.n_kv_heads, w = ctx.cfg.window;
-  const int N = a.n_keys;
-  const int rows_pg_pad = ctx.rows_pad / ctx.cfg.n_kv_heads;
-  const float c2 = a.scale * kLog2e;
-  if (pass == 1) {
-    const int n_chunks = (N + kP1Keys - 1) / kP1Keys;
-    int parts = n_chunks < kSimtParts ? n_chunks : kSimtParts;
-    *parts_out = parts;
-    const size_t smem = ((size_t)w * D + kP1Keys * (D + 1) + 3 * (size_t)w) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(simt_pass1<T, D>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+cudaError_t launch_typed(const Ctx& ctx, const SimtArgs& a, int layers, cudaStream_t st) {
+  static std::atomic<unsigned long long> ready{0};        // devices whose shared-memory limit has been raised
+  const unsigned long long bit = 1ull << (ctx.device & 63);
+  const int smem = (int)sizeof(SimtShared<D>);
+  if (!(ready.load(std::memory_order_acquire) & bit)) {
+    cudaError_t e = cudaFuncSetAttribute(simt_pass1<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(simt_pass2<T, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    simt_pass1<T, D><<<dim3(parts, H), kP1Threads, smem, st>>>(
-        (const T*)a.q, (const T*)a.k, a.k_stride_head, a.k_stride_token, N, w, G, c2, parts,
-        rows_pg_pad, ctx.rows_pad, ctx.ws.row_part);
-  } else {
-    const size_t smem = ((size_t)w * D + (size_t)w) * sizeof(float);
-    cudaError_t e = cudaFuncSetAttribute(simt_pass2<T, D>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    simt_pass2<T, D><<<dim3((N + kP2Threads - 1) / kP2Threads, H), kP2Threads, smem, st>>>(
-        (const T*)a.q, (const T*)a.k, a.k_stride_head, a.k_stride_token, N, w, G, c2,
-        rows_pg_pad, ctx.ws.row_lse2, a.cols, a.col_stride);
+    ready.fetch_or(bit, std::memory_order_release);
   }
-  return cudaGetLastError();
+  const int G = ctx.cfg.n_kv_heads, span = a.w_pad > kSmRows ? a.w_pad / kSmRows : 1;
+  const cudaError_t e = launch_pdl(simt_pass1<T, D>, dim3(a.parts, a.n_rt * G, layers), dim3(kSmThreads), smem, st, a);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(simt_pass2<T, D>, dim3(a.n_keys_tiles, a.n_rt / span * G, layers), dim3(kSmThreads), smem, st, a);
 }
 
 }  // namespace
 
-cudaError_t launch_score_simt(const Ctx& ctx, const ScoreArgs& a, int* parts_out, int pass,
-                              cudaStream_t st) {
-  const bool f32 = ctx.cfg.dtype == STRUCTKV_FP32;
-  const int d = ctx.cfg.head_dim;
-  if (f32 && d == 64) return launch_typed<float, 64>(ctx, a, parts_out, pass, st);
-  if (f32 && d == 128) return launch_typed<float, 128>(ctx, a, parts_out, pass, st);
-  if (!f32 && d == 64) return launch_typed<__nv_bfloat16, 64>(ctx, a, parts_out, pass, st);
-  if (!f32 && d == 128) return launch_typed<__nv_bfloat16, 128>(ctx, a, parts_out, pass, st);
-  return cudaErrorInvalidValue;
+size_t simt_part_entries(const structkv_config& cfg, int n) {
+  const size_t rows = align_up((size_t)(cfg.n_q_heads / cfg.n_kv_heads) * tc_window_pad(cfg.window), kRowBlock) * cfg.n_kv_heads;
+  return (size_t)std::min(n, kSmLayers) * kSimtParts * rows;
+}
+
+cudaError_t launch_score_simt(const Ctx& ctx, const ScoreCall& c, cudaStream_t st) {
+  SimtArgs a = {};
+  a.sh = c.k_stride_head; a.st = c.k_stride_token;
+  a.N = c.n_keys; a.w = ctx.cfg.window; a.w_pad = ctx.w_pad;
+  a.group = ctx.cfg.n_q_heads / ctx.cfg.n_kv_heads;
+  a.rows_pg = a.group * a.w_pad; a.rows_pg_pad = ctx.rows_pad / ctx.cfg.n_kv_heads; a.rows_pad = ctx.rows_pad;
+  // row tiles that hold rows, an even number where a head takes two
+  a.n_rt = (a.rows_pg + kSmRows - 1) / kSmRows;
+  a.n_keys_tiles = (a.N + kSmKeys - 1) / kSmKeys;
+  a.parts = std::min(a.n_keys_tiles, kSimtParts);
+  a.part = c.part; a.col_stride = c.col_stride; a.cols_layer_stride = c.cols_layer_stride;
+  for (int l0 = 0; l0 < c.n; l0 += kSmLayers) {
+    const int layers = std::min(kSmLayers, c.n - l0);
+    for (int l = 0; l < layers; ++l) {
+      a.q[l] = c.q[l0 + l]; a.k[l] = c.k[l0 + l];
+      a.c2[l] = c.scale[l0 + l] * kLog2e;
+    }
+    a.row_ent = c.row_ent + (size_t)l0 * ctx.rows_pad;
+    a.cols = c.cols + (size_t)l0 * c.cols_layer_stride;
+    const bool f32 = ctx.cfg.dtype == STRUCTKV_FP32;
+    cudaError_t e = cudaErrorInvalidValue;
+    if (ctx.cfg.head_dim == 64) e = f32 ? launch_typed<float, 64>(ctx, a, layers, st) : launch_typed<__nv_bfloat16, 64>(ctx, a, layers, st);
+    if (ctx.cfg.head_dim == 128) e = f32 ? launch_typed<float, 128>(ctx, a, layers, st) : launch_typed<__nv_bfloat16, 128>(ctx, a, layers, st);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace skv

@@ -71,7 +71,7 @@ int clamp_tasks(const Layout& l, int target, int items) {
 }
 
 template <int MAXP>
-cudaError_t launch_problems(const Ctx& ctx, const TcCall& a, int first, int n, cudaStream_t st) {
+cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n, cudaStream_t st) {
   TcParams<MAXP> p;
   const structkv_config& cfg = ctx.cfg;
   const Layout l = layout_of(cfg);
@@ -207,7 +207,7 @@ void tc_destroy(Ctx& ctx) {
   ctx.tc = nullptr;
 }
 
-cudaError_t launch_score_tc(const Ctx& ctx, const TcCall& a, cudaStream_t st) {
+cudaError_t launch_score_tc(const Ctx& ctx, const ScoreCall& a, cudaStream_t st) {
   if (a.cu_seqlens) return a.n == 1 ? launch_problems<1>(ctx, a, 0, 1, st) : launch_problems<kMaxBatch>(ctx, a, 0, a.n, st);
   for (int l = 0; l < a.n; l += kMaxBatch) {
     const int n = std::min(kMaxBatch, a.n - l);

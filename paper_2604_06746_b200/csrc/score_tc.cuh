@@ -60,7 +60,6 @@ constexpr int kTcThreads = (kHelperWarps + kComputeWarps) * 32;   // 20 warps: t
 constexpr unsigned long long kWaitCycles = 1000000000ull;   // about 0.5 s at the maximum SM clock
 constexpr float kMasked = -1.0e30f;    // exponent standing for -inf: 2^x flushes to 0 and 0 * x stays finite
 constexpr float kMaskedAcc = -3.0e38f; // the same for an accumulator, before the scaling by c2 >= 1e-30
-constexpr int kMergeGroup = 6;         // partials of a row merged together
 constexpr int kFullWeight = 20;        // weight of a full row block when key ranges are dealt out (see tc_deal)
 
 // Layout classes of the kernel (template argument).
@@ -401,37 +400,6 @@ enum { kBarFull = 0, kBarEmpty = kBarFull + kStages, kBarTaskFull = kBarEmpty + 
        kBarAccEmpty = kBarAccFull + 8, kBarCount = kBarAccEmpty + 8 };
 constexpr int kTaskConsumers = 3 + kComputeWarps;          // MMA, lse hand-over, fold, compute warps
 
-// One row's softmax statistics over some keys: Z = sum 2^(x - ref), U = sum 2^(x - ref) (x - ref).
-struct RowStat { float ref, Z, U; };
-
-// A row's partial as it is stored: (l, h), its log-sum-exp l = ref + log2 Z and the entropy of the
-// softmax over its keys alone, h = log2 Z - U / Z (both in bits); (-inf, 0) where it saw no key of the
-// row.  Over a row's partials, lse = log2 sum 2^l and with w = 2^(l - lse) the row's entropy is
-// sum w (h + lse - l)  (Eq. 4, one row).  The compute warps take the logarithm and the division, and
-// loads of four rows are in flight together: merging is one warp's work beside sixteen busy ones,
-// and pass 2 waits for it (18 partials of 256 rows: 35 us with one row and one logarithm at a time).
-__device__ __forceinline__ float2 stat_partial(const RowStat& r) {
-  const float lz = __log2f(r.Z);
-  return r.Z > 0.f ? make_float2(r.ref + lz, lz - __fdividef(r.U, r.Z)) : make_float2(-INFINITY, 0.f);
-}
-// Adds partials to (M, W, X): lse so far = M + log2 W, X = sum 2^(l - M) (h - l + M).
-template <int N>
-__device__ __forceinline__ void merge_partials(float& M, float& W, float& X, const float2 (&pv)[N]) {
-  float top = M;
-#pragma unroll
-  for (int b = 0; b < N; ++b) top = fmaxf(top, pv[b].x);
-  if (top == -INFINITY) return;
-  const float d = M == -INFINITY ? 0.f : M - top, f = fast_exp2(d);
-  X = f * fmaf(-d, W, X);
-  W *= f;
-  M = top;
-#pragma unroll
-  for (int b = 0; b < N; ++b) {
-    const float e = pv[b].x == -INFINITY ? -200.f : pv[b].x - top, w = fast_exp2(e);
-    W += w;
-    X = fmaf(w, pv[b].y - e, X);
-  }
-}
 // The four column groups (wide) or lane quarters (narrow) of a row fold into one partial.
 template <int R>
 __device__ __forceinline__ float2 fold_row(const float2* part_s, int r) {
