@@ -311,6 +311,70 @@ structkv_status structkv_select(structkv_ctx* ctx, const float* scores, long lon
                                 void* stream);
 
 /*
+ * structkv_pivot, structkv_accumulate and structkv_select (for the layers and for the centrality) in one
+ * call: Eq. 7-9, Eq. 3 at the pivot, Eq. 10 and Eq. 13, in that order, without a host round trip between
+ * them: the pivot is found on the device (same arithmetic, double precision), the host waits only for
+ * its value.  Results are those of the separate calls.
+ *   s_hist    device, [n_layers] rows of n fp32 scores, row_stride elements apart.
+ *   metrics_dev, weights, l_limit, pivot_out, t_out   as for structkv_pivot (t_out may be NULL).
+ *   c_star    device, [n] fp32: the centrality at the pivot.
+ *   i_kv      device, [n_layers, kv_budget] int32;  i_struct  device, [struct_budget] int32.
+ * Returns once the pivot is known; the selections may still be running on `stream`.  Cannot be
+ * captured into a graph.  Errors: INVALID_ARG, CUDA.
+ */
+structkv_status structkv_pivot_select(structkv_ctx* ctx, const float* s_hist, long long row_stride, int n_layers,
+                                      int n, const float* metrics_dev, const float* weights, int l_limit,
+                                      float lambda, int window, int kv_budget, int* i_kv, int struct_budget,
+                                      float* c_star, int* i_struct, int* pivot_out, float* t_out, void* stream);
+
+/*
+ * The whole of Algorithm 1 over one prompt whose layers are resident: structkv_score_layers (C starting
+ * from zero), structkv_head_stats, structkv_pivot_select, structkv_compact_layers for K/V and structkv_compact
+ * for hidden states and position ids, enqueued by one call.  Every field means what the argument of
+ * that name means there.  kv_srcs, hidden and positions may be NULL (that gather is left out).
+ * Returns once the pivot is known; selections and gathers may still be running on `stream`.  Results are
+ * those of the separate calls.  Errors: INVALID_ARG, WORKSPACE, CUDA.
+ */
+typedef struct {
+  int n_layers;                             /* 1 .. 128 */
+  const void* const* q_windows;             /* host arrays of device pointers, [n_layers] */
+  const void* const* ks;
+  const float* scales;                      /* host, [n_layers] */
+  long long k_stride_head, k_stride_token;
+  int n_keys;
+  float lambda;
+  float* s_out;                             /* [n_layers] rows s_layer_stride apart */
+  long long s_layer_stride;
+  float* c_out;                             /* [n_keys]: C over all layers */
+  float* head_cols;                         /* [n_layers, H, n_keys] */
+  long long head_cols_layer_stride;
+  float* metrics;                           /* [n_layers, 3] */
+  void* layers_workspace;
+  size_t layers_workspace_bytes;
+  float weights[3];
+  int l_limit;
+  int window, kv_budget, struct_budget;
+  int* i_kv;
+  int* i_struct;
+  float* c_star;
+  const void* const* kv_srcs;               /* as srcs of structkv_compact_layers; index lists are i_kv */
+  long long kv_slab_stride_bytes, kv_row_stride_bytes;
+  int kv_row_bytes, kv_slabs, kv_rows;
+  void* kv_dst;
+  long long kv_dst_layer_stride_bytes;
+  const void* hidden;                       /* [n_keys] rows of hidden_row_bytes, hidden_row_stride_bytes apart */
+  long long hidden_row_stride_bytes;
+  int hidden_row_bytes;
+  void* hidden_dst;
+  const void* positions;                    /* the same for position ids */
+  long long position_row_stride_bytes;
+  int position_row_bytes;
+  void* positions_dst;
+} structkv_prefill_args;
+structkv_status structkv_prefill(structkv_ctx* ctx, const structkv_prefill_args* args, int* pivot_out, float* t_out,
+                                 void* stream);
+
+/*
  * Row gather / compaction.  Paper: Algorithm 1 line 17 (cache K, V at I_KV), line 13 and
  * Eq. 11-12 (hidden states and position ids at I_struct).  For every slab s and output row r:
  * dst[s, r, 0:row_bytes] = src[s*slab_stride_bytes + idx[r]*row_stride_bytes + 0:row_bytes],

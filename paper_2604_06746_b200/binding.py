@@ -86,6 +86,28 @@ lib.structkv_block_scores.restype = _i
 lib.structkv_block_scores.argtypes = [_vp, _vp, _ll, _i, _i, _i, _vp, _vp]
 lib.structkv_mass_recovery.restype = _i
 lib.structkv_mass_recovery.argtypes = [_vp, _vp, _ll, _i, _i, _vp, _i, _vp, _vp]
+lib.structkv_pivot_select.restype = _i
+lib.structkv_pivot_select.argtypes = [_vp, _vp, _ll, _i, _i, _vp, ctypes.POINTER(_f), _i, _f, _i, _i, _vp, _i, _vp, _vp,
+                                      ctypes.POINTER(_i), ctypes.POINTER(_f), _vp]
+
+
+class PrefillArgs(ctypes.Structure):
+    """structkv_prefill_args."""
+    _fields_ = [("n_layers", _i), ("q_windows", ctypes.POINTER(_vp)), ("ks", ctypes.POINTER(_vp)),
+                ("scales", ctypes.POINTER(_f)), ("k_stride_head", _ll), ("k_stride_token", _ll), ("n_keys", _i),
+                ("lam", _f), ("s_out", _vp), ("s_layer_stride", _ll), ("c_out", _vp), ("head_cols", _vp),
+                ("head_cols_layer_stride", _ll), ("metrics", _vp), ("layers_workspace", _vp),
+                ("layers_workspace_bytes", ctypes.c_size_t), ("weights", _f * 3), ("l_limit", _i), ("window", _i),
+                ("kv_budget", _i), ("struct_budget", _i), ("i_kv", _vp), ("i_struct", _vp), ("c_star", _vp),
+                ("kv_srcs", ctypes.POINTER(_vp)), ("kv_slab_stride_bytes", _ll), ("kv_row_stride_bytes", _ll),
+                ("kv_row_bytes", _i), ("kv_slabs", _i), ("kv_rows", _i), ("kv_dst", _vp),
+                ("kv_dst_layer_stride_bytes", _ll), ("hidden", _vp), ("hidden_row_stride_bytes", _ll),
+                ("hidden_row_bytes", _i), ("hidden_dst", _vp), ("positions", _vp), ("position_row_stride_bytes", _ll),
+                ("position_row_bytes", _i), ("positions_dst", _vp)]
+
+
+lib.structkv_prefill.restype = _i
+lib.structkv_prefill.argtypes = [_vp, ctypes.POINTER(PrefillArgs), ctypes.POINTER(_i), ctypes.POINTER(_f), _vp]
 lib.structkv_selftest_wait_expiry.restype = _i
 lib.structkv_selftest_wait_expiry.argtypes = [_vp, ctypes.c_ulonglong, _vp]
 lib.structkv_poll_device_status.restype = _i
@@ -108,8 +130,8 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream(stream: Optional[torch.cuda.Stream]) -> int:
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    # the raw handle: building a Stream object costs more than a kernel launch
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
 
 
 def version() -> int:
@@ -286,6 +308,29 @@ class Context:
         T = (_f * L)()
         _check(lib.structkv_pivot(self._h, metrics.data_ptr(), L, w, l_limit, ctypes.byref(piv), T,
                                   _stream(stream)), "structkv_pivot")
+        return piv.value, list(T)
+
+    def pivot_select(self, s_hist: torch.Tensor, metrics: torch.Tensor, weights: Sequence[float], l_limit: int, lam: float,
+                     window: int, kv_budget: int, i_kv: torch.Tensor, struct_budget: int, c_star: torch.Tensor,
+                     i_struct: torch.Tensor, stream: Optional[torch.cuda.Stream] = None) -> Tuple[int, list]:
+        """structkv_pivot_select over ``s_hist [L, n]`` and ``metrics [L, 3]``: ``c_star [n]``, ``i_kv [L, kv_budget]`` and
+        ``i_struct [struct_budget]`` are written; returns ``(L*, T)`` while the selections may still be running."""
+        L, n = s_hist.shape
+        assert s_hist.stride(1) == 1 and s_hist.dtype == torch.float32 and metrics.is_contiguous()
+        assert metrics.shape == (L, 3) and metrics.dtype == torch.float32 and c_star.is_contiguous() and c_star.numel() == n
+        assert i_kv.dtype == i_struct.dtype == torch.int32 and i_kv.is_contiguous() and i_struct.is_contiguous()
+        assert i_kv.numel() == L * kv_budget and i_struct.numel() == struct_budget
+        piv, T = _i(0), (_f * L)()
+        _check(lib.structkv_pivot_select(self._h, s_hist.data_ptr(), s_hist.stride(0), L, n, metrics.data_ptr(),
+                                         (_f * 3)(*weights), l_limit, lam, window, kv_budget, i_kv.data_ptr(),
+                                         struct_budget, c_star.data_ptr(), i_struct.data_ptr(), ctypes.byref(piv), T,
+                                         _stream(stream)), "structkv_pivot_select")
+        return piv.value, list(T)
+
+    def prefill(self, args: PrefillArgs, stream: Optional[torch.cuda.Stream] = None) -> Tuple[int, list]:
+        """structkv_prefill on a prepared argument block; returns ``(L*, T)``."""
+        piv, T = _i(0), (_f * args.n_layers)()
+        _check(lib.structkv_prefill(self._h, ctypes.byref(args), ctypes.byref(piv), T, _stream(stream)), "structkv_prefill")
         return piv.value, list(T)
 
     def accumulate(self, s_hist: torch.Tensor, pivot: int, lam: float, c_out: torch.Tensor,

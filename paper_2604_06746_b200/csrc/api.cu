@@ -1,6 +1,7 @@
 // C ABI of libstructkv: argument validation, context and workspace bookkeeping, dispatch to
 // the kernels, and the host-side pivot rule (Eq. 7-9).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
@@ -58,6 +59,45 @@ Workspace carve_workspace(const structkv_config& cfg, void* base) {
   w.bytes = off;
   return w;
 }
+
+// ---- host words the device writes for the host: one page-locked block per process, a slot per context --
+struct HostSlot {
+  int* mem;                              // [kSlotInts], mapped
+  unsigned seq;                          // calls so far: tags the answers
+};
+namespace {
+constexpr int kSlots = 64, kSlotInts = 256;
+static_assert(kSlotInts > kMaxStatLayers, "a slot holds the pivot and every T_l");
+std::mutex g_slot_mutex;
+int* g_slot_mem = nullptr;
+bool g_slot_used[kSlots];
+
+// A slot for the context, or NULL: none left, or no page-locked memory (the caller then copies).
+HostSlot* take_slot() {
+  std::lock_guard<std::mutex> lock(g_slot_mutex);
+  if (!g_slot_mem &&
+      cudaHostAlloc((void**)&g_slot_mem, sizeof(int) * kSlots * kSlotInts, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+    g_slot_mem = nullptr;
+    cudaGetLastError();
+    return nullptr;
+  }
+  for (int i = 0; i < kSlots; ++i)
+    if (!g_slot_used[i]) {
+      HostSlot* s = new (std::nothrow) HostSlot{g_slot_mem + i * kSlotInts, 0};
+      if (!s) return nullptr;
+      g_slot_used[i] = true;
+      s->mem[0] = 0;
+      return s;
+    }
+  return nullptr;
+}
+void give_back(HostSlot* s) {
+  if (!s) return;
+  std::lock_guard<std::mutex> lock(g_slot_mutex);
+  g_slot_used[(s->mem - g_slot_mem) / kSlotInts] = false;
+  delete s;
+}
+}  // namespace
 
 }  // namespace skv
 
@@ -121,6 +161,7 @@ structkv_status structkv_create(structkv_ctx** ctx_out, const structkv_config* c
 void structkv_destroy(structkv_ctx* ctx) {
   if (!ctx) return;
   tc_destroy(ctx->c);
+  give_back(ctx->c.slot);
   delete ctx;
 }
 
@@ -254,13 +295,13 @@ size_t structkv_layers_workspace_bytes(const structkv_config* cfg, int max_layer
   return carve_layers(*cfg, max_layers, nullptr).bytes;
 }
 
-structkv_status structkv_score_layers(structkv_ctx* ctx, int n_layers, const void* const* q_windows,
+static structkv_status score_layers(structkv_ctx* ctx, int n_layers, const void* const* q_windows,
                                       const void* const* ks, long long k_stride_head,
                                       long long k_stride_token, int n_keys, const float* scales, float lambda,
                                       float* s_out, long long s_layer_stride, float* c_inout,
                                       float* head_cols_out, long long head_cols_layer_stride,
                                       float* metrics_out, void* layers_workspace,
-                                      size_t layers_workspace_bytes, void* stream) {
+                                      size_t layers_workspace_bytes, void* stream, bool c_from_zero, bool with_stats) {
   if (!ctx || !q_windows || !ks || !scales || !s_out || !head_cols_out || !metrics_out)
     return STRUCTKV_ERR_INVALID_ARG;
   if (n_layers < 1 || n_layers > 65536) return STRUCTKV_ERR_INVALID_ARG;
@@ -284,11 +325,12 @@ structkv_status structkv_score_layers(structkv_ctx* ctx, int n_layers, const voi
   const bool use_tc = tc_supported(c, k_stride_head, k_stride_token);
   if (!use_tc && (cfg.dtype == STRUCTKV_BF16 || !layers_workspace)) {
     // bf16 layers the tensor cores do not take: one after the other, same results
+    if (c_from_zero && cudaMemsetAsync(c_inout, 0, (size_t)n_keys * sizeof(float), st) != cudaSuccess) return STRUCTKV_ERR_CUDA;
     for (int l = 0; l < n_layers; ++l) {
       const structkv_status s = structkv_score_layer(
           ctx, q_windows[l], ks[l], k_stride_head, k_stride_token, n_keys, scales[l], lambda,
           s_out + (size_t)l * s_layer_stride, c_inout, head_cols_out + (size_t)l * head_cols_layer_stride,
-          metrics_out + 3 * l, STRUCTKV_FLAG_NO_HEAD_STATS, stream);
+          metrics_out + 3 * l, with_stats ? 0u : STRUCTKV_FLAG_NO_HEAD_STATS, stream);
       if (s != STRUCTKV_OK) return s;
     }
     return STRUCTKV_OK;
@@ -300,10 +342,26 @@ structkv_status structkv_score_layers(structkv_ctx* ctx, int n_layers, const voi
   const ScoreCall a{n_layers, q_windows, ks, scales, nullptr, k_stride_head, k_stride_token, n_keys, head_cols_out,
                  head_cols_layer_stride, n_keys, lw.row_part, lw.nlse, lw.row_ent};
   if ((use_tc ? launch_score_tc(c, a, st) : launch_score_simt(c, a, st)) != cudaSuccess) return STRUCTKV_ERR_CUDA;
-  return launch_finish_layers(c, head_cols_out, head_cols_layer_stride, n_keys, n_keys, n_layers, lambda, s_out,
-                              s_layer_stride, c_inout, lw.row_ent, false, metrics_out, st) == cudaSuccess
-             ? STRUCTKV_OK
-             : STRUCTKV_ERR_CUDA;
+  const bool ride = with_stats && head_stats_ride_along(c, n_layers, n_keys);
+  if (launch_finish_layers(c, head_cols_out, head_cols_layer_stride, n_keys, n_keys, n_layers, lambda, s_out, s_layer_stride,
+                           c_inout, lw.row_ent, ride, metrics_out, st, c_from_zero) != cudaSuccess)
+    return STRUCTKV_ERR_CUDA;
+  if (with_stats && !ride &&
+      launch_head_stats_batch(c, head_cols_out, head_cols_layer_stride, n_keys, n_layers, n_keys, metrics_out, st) != cudaSuccess)
+    return STRUCTKV_ERR_CUDA;
+  return STRUCTKV_OK;
+}
+
+structkv_status structkv_score_layers(structkv_ctx* ctx, int n_layers, const void* const* q_windows,
+                                      const void* const* ks, long long k_stride_head,
+                                      long long k_stride_token, int n_keys, const float* scales, float lambda,
+                                      float* s_out, long long s_layer_stride, float* c_inout,
+                                      float* head_cols_out, long long head_cols_layer_stride,
+                                      float* metrics_out, void* layers_workspace,
+                                      size_t layers_workspace_bytes, void* stream) {
+  return score_layers(ctx, n_layers, q_windows, ks, k_stride_head, k_stride_token, n_keys, scales, lambda, s_out,
+                      s_layer_stride, c_inout, head_cols_out, head_cols_layer_stride, metrics_out, layers_workspace,
+                      layers_workspace_bytes, stream, false, false);
 }
 
 structkv_status structkv_select_batch(structkv_ctx* ctx, const float* scores, const int* cu_seqlens,
@@ -394,6 +452,107 @@ structkv_status structkv_select(structkv_ctx* ctx, const float* scores, long lon
                  cudaSuccess
              ? STRUCTKV_OK
              : STRUCTKV_ERR_CUDA;
+}
+
+// Enqueues pivot, centrality and selections; false: not possible in this form (no slot, too many layers).
+static bool can_pivot_on_device(Ctx& c, int n_layers) {
+  if (n_layers > kMaxStatLayers) return false;
+  if (!c.slot) c.slot = take_slot();
+  return c.slot != nullptr;
+}
+static structkv_status enqueue_pivot_select(Ctx& c, const float* s_hist, long long row_stride, int n_layers, int n,
+                                            const float* metrics, const float* weights, int l_limit, float lambda, int window,
+                                            int kv_budget, int* i_kv, int struct_budget, float* c_star, int* i_struct,
+                                            cudaStream_t st) {
+  const int tag = (int)(++c.slot->seq << 8);
+  if (launch_accumulate_at_pivot(s_hist, row_stride, n_layers, n, lambda, metrics, weights, l_limit, c_star, c.slot->mem,
+                                 tag, st) != cudaSuccess)
+    return STRUCTKV_ERR_CUDA;
+  const SelectExtra extra{c_star, struct_budget, i_struct};
+  return launch_select(s_hist, row_stride, n_layers, n, kv_budget, window, i_kv, st, &extra) == cudaSuccess ? STRUCTKV_OK
+                                                                                                            : STRUCTKV_ERR_CUDA;
+}
+// Waits for the word enqueue_pivot_select asked for.
+static structkv_status await_pivot(Ctx& c, int n_layers, int* pivot_out, float* t_out, cudaStream_t st) {
+  volatile int* mem = c.slot->mem;
+  const unsigned tag = c.slot->seq << 8;
+  for (unsigned spins = 1; ((unsigned)mem[0] & ~255u) != tag; ++spins) {
+    if (spins % 100000 != 0) continue;                 // tens of microseconds
+    const cudaError_t e = cudaStreamQuery(st);
+    if (e == cudaErrorNotReady) continue;
+    if (e != cudaSuccess || ((unsigned)mem[0] & ~255u) != tag) return STRUCTKV_ERR_CUDA;   // done, and no word
+  }
+  std::atomic_thread_fence(std::memory_order_acquire);
+  *pivot_out = mem[0] & 255;
+  if (t_out)
+    for (int l = 0; l < n_layers; ++l) {
+      const int bits = mem[1 + l];
+      std::memcpy(&t_out[l], &bits, sizeof(float));
+    }
+  return STRUCTKV_OK;
+}
+static bool pivot_select_args_ok(const float* s_hist, long long row_stride, int n_layers, int n, const float* metrics,
+                                 const float* weights, float lambda, int window, int kv_budget, const int* i_kv,
+                                 int struct_budget, const float* c_star, const int* i_struct, const int* pivot_out) {
+  return s_hist && metrics && weights && i_kv && c_star && i_struct && pivot_out && n_layers >= 1 && n_layers <= 65536 && n >= 1 &&
+         row_stride >= n && std::isfinite(lambda) && window >= 0 && window <= kv_budget && kv_budget <= n &&
+         window <= struct_budget && struct_budget <= n;
+}
+
+structkv_status structkv_pivot_select(structkv_ctx* ctx, const float* s_hist, long long row_stride, int n_layers,
+                                      int n, const float* metrics_dev, const float* weights, int l_limit,
+                                      float lambda, int window, int kv_budget, int* i_kv, int struct_budget,
+                                      float* c_star, int* i_struct, int* pivot_out, float* t_out, void* stream) {
+  if (!ctx || !pivot_select_args_ok(s_hist, row_stride, n_layers, n, metrics_dev, weights, lambda, window, kv_budget, i_kv,
+                                    struct_budget, c_star, i_struct, pivot_out))
+    return STRUCTKV_ERR_INVALID_ARG;
+  cudaStream_t st = (cudaStream_t)stream;
+  if (!can_pivot_on_device(ctx->c, n_layers)) {
+    structkv_status s = structkv_pivot(ctx, metrics_dev, n_layers, weights, l_limit, pivot_out, t_out, stream);
+    if (s == STRUCTKV_OK) s = structkv_accumulate(ctx, s_hist, row_stride, *pivot_out, n, lambda, c_star, stream);
+    if (s == STRUCTKV_OK) s = structkv_select(ctx, s_hist, row_stride, n_layers, n, kv_budget, window, i_kv, stream);
+    if (s == STRUCTKV_OK) s = structkv_select(ctx, c_star, n, 1, n, struct_budget, window, i_struct, stream);
+    return s;
+  }
+  const structkv_status s = enqueue_pivot_select(ctx->c, s_hist, row_stride, n_layers, n, metrics_dev, weights, l_limit, lambda,
+                                                 window, kv_budget, i_kv, struct_budget, c_star, i_struct, st);
+  return s == STRUCTKV_OK ? await_pivot(ctx->c, n_layers, pivot_out, t_out, st) : s;
+}
+
+structkv_status structkv_prefill(structkv_ctx* ctx, const structkv_prefill_args* p, int* pivot_out, float* t_out,
+                                 void* stream) {
+  if (!ctx || !p || !p->c_out || p->n_layers < 1 || p->n_layers > kMaxStatLayers ||
+      !pivot_select_args_ok(p->s_out, p->s_layer_stride, p->n_layers, p->n_keys, p->metrics, p->weights, p->lambda, p->window,
+                            p->kv_budget, p->i_kv, p->struct_budget, p->c_star, p->i_struct, pivot_out))
+    return STRUCTKV_ERR_INVALID_ARG;
+  cudaStream_t st = (cudaStream_t)stream;
+  structkv_status s = score_layers(ctx, p->n_layers, p->q_windows, p->ks, p->k_stride_head, p->k_stride_token, p->n_keys,
+                                   p->scales, p->lambda, p->s_out, p->s_layer_stride, p->c_out, p->head_cols,
+                                   p->head_cols_layer_stride, p->metrics, p->layers_workspace, p->layers_workspace_bytes,
+                                   stream, true, true);
+  if (s != STRUCTKV_OK) return s;
+  const bool on_device = can_pivot_on_device(ctx->c, p->n_layers);
+  s = on_device ? enqueue_pivot_select(ctx->c, p->s_out, p->s_layer_stride, p->n_layers, p->n_keys, p->metrics, p->weights,
+                                       p->l_limit, p->lambda, p->window, p->kv_budget, p->i_kv, p->struct_budget, p->c_star,
+                                       p->i_struct, st)
+                : structkv_pivot_select(ctx, p->s_out, p->s_layer_stride, p->n_layers, p->n_keys, p->metrics, p->weights,
+                                        p->l_limit, p->lambda, p->window, p->kv_budget, p->i_kv, p->struct_budget, p->c_star,
+                                        p->i_struct, pivot_out, t_out, stream);
+  if (s == STRUCTKV_OK && p->kv_srcs)
+    s = structkv_compact_layers(ctx, p->kv_srcs, p->n_layers, p->kv_slab_stride_bytes, p->kv_row_stride_bytes, p->kv_row_bytes,
+                                p->kv_slabs, p->kv_rows, p->i_kv, p->kv_budget, p->kv_budget, p->kv_dst,
+                                p->kv_dst_layer_stride_bytes, stream);
+  if (s == STRUCTKV_OK && p->hidden)
+    s = structkv_compact(ctx, p->hidden, 0, p->hidden_row_stride_bytes, p->hidden_row_bytes, 1, p->n_keys, p->i_struct,
+                         p->struct_budget, p->hidden_dst, stream);
+  if (s == STRUCTKV_OK && p->positions)
+    s = structkv_compact(ctx, p->positions, 0, p->position_row_stride_bytes, p->position_row_bytes, 1, p->n_keys, p->i_struct,
+                         p->struct_budget, p->positions_dst, stream);
+  if (on_device) {
+    const structkv_status w = await_pivot(ctx->c, p->n_layers, pivot_out, t_out, st);   // also after an error: the word is on its way
+    if (s == STRUCTKV_OK) s = w;
+  }
+  return s;
 }
 
 structkv_status structkv_compact(structkv_ctx* ctx, const void* src, long long slab_stride_bytes,

@@ -48,6 +48,7 @@ struct Ctx {
   int rows_pad;         // rows per KV group (heads at w_pad rows) padded to kRowBlock, times H_kv
   int n_pad;            // max_seq rounded up to kKeyTile
   void* tc;             // tensor-core scorer state (tensor-map encoder), owned by score_tc.cu
+  struct HostSlot* slot = nullptr;   // where the device leaves the pivot for the host (api.cu), taken at first use
 };
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -93,7 +94,10 @@ cudaError_t launch_wait_probe(unsigned long long limit_cycles, int* status, cuda
 // metrics[l][1..2] from the pooled per-head attention (Eq. 5-6) or NaN.
 cudaError_t launch_finish_layers(const Ctx& ctx, const float* cols, long long layer_stride, long long col_stride, int n,
                                  int n_layers, float lambda, float* s_out, long long s_stride, float* c_inout,
-                                 const float* row_ent, bool with_head_stats, float* metrics, cudaStream_t st);
+                                 const float* row_ent, bool with_head_stats, float* metrics, cudaStream_t st,
+                                 bool c_from_zero = false);
+// whether Eq. 5-6 of so many vectors of n entries are best taken in that launch
+bool head_stats_ride_along(const Ctx& ctx, int n_layers, int n);
 // The same for the sequences of a packed batch (sequence b at column cu_seqlens[b] of cols, s_out and c_inout).
 cudaError_t launch_finish_packed(const Ctx& ctx, const float* cols, long long col_stride, const int* cu_seqlens, int batch,
                                  float lambda, float* s_out, float* c_inout, const float* row_ent, float* head_part,
@@ -106,8 +110,16 @@ cudaError_t launch_head_stats_batch(const Ctx& ctx, const float* cols, long long
 cudaError_t launch_accumulate(const float* s_hist, long long row_stride, int pivot, int n,
                               float lambda, float* c_out, cudaStream_t st);
 
+// Eq. 7-9 on the device (n_layers <= kMaxStatLayers), then launch_accumulate at that pivot.  `host` (mapped
+// memory) receives T_l [n_layers] from word 1 on and then, in word 0, tag | pivot (the tag's low byte is 0).
+cudaError_t launch_accumulate_at_pivot(const float* s_hist, long long row_stride, int n_layers, int n, float lambda,
+                                       const float* metrics, const float* weights, int l_limit, float* c_out, int* host,
+                                       int tag, cudaStream_t st);
+
+// One more vector of a selection, with its own budget and output.
+struct SelectExtra { const float* scores; int budget; int* idx_out; };
 cudaError_t launch_select(const float* scores, long long row_stride, int batch, int n, int budget,
-                          int window, int* idx_out, cudaStream_t st);
+                          int window, int* idx_out, cudaStream_t st, const SelectExtra* extra = nullptr);
 // The same for packed sequences of different lengths and budgets; rows are padded with -1.
 cudaError_t launch_select_packed(const float* scores, const int* cu_seqlens, const int* budgets, int batch, int window,
                                  int* idx_out, long long idx_stride, cudaStream_t st);

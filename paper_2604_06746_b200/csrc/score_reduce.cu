@@ -20,6 +20,7 @@ struct FinishArgs {
   float* s_out;                        // problem p at s_out + p * s_stride
   long long s_stride;
   float* c_inout;                      // layers: one vector carried through them; packed: at s_out's offsets
+  int c_from_zero;                     // its old contents count as 0
   const float* row_ent;                // [n_prob][rows_pad], or NULL: no entropy, no sums
   int rows_pad, n_valid;
   float* metrics;                      // [n_prob][3]
@@ -98,7 +99,7 @@ __device__ __forceinline__ void sum_block(const FinishArgs& a, int p, int chunk)
     const bool chained = !a.packed && a.n_prob > 1;
     T* c = reinterpret_cast<T*>(a.c_inout + (a.packed ? a.cu[p] : 0) + j);
     if (!chained) {
-      if (grp == 0 && j < pb.n) *c = decay(a.lambda, *c, s);
+      if (grp == 0 && j < pb.n) *c = a.c_from_zero ? s : decay(a.lambda, *c, s);
     } else {
       __threadfence();
       __syncthreads();
@@ -107,7 +108,8 @@ __device__ __forceinline__ void sum_block(const FinishArgs& a, int p, int chunk)
       if (last) {
         __threadfence();
         if (grp == 0 && j < pb.n) {
-          T acc = *c;
+          T acc{};
+          if (!a.c_from_zero) acc = *c;
 #pragma unroll 8
           for (int l = 0; l < a.n_prob; ++l)
             acc = decay(a.lambda, acc, __ldcg(reinterpret_cast<const T*>(a.s_out + (size_t)l * a.s_stride + j)));
@@ -436,6 +438,89 @@ __global__ void __launch_bounds__(128) accumulate(const float* __restrict__ s_hi
   *reinterpret_cast<T*>(c_out + j) = c;
 }
 
+// Eq. 7-9, then the same recursion.  Every block finds the pivot for itself (one warp, 2 us), so that no
+// launch and no host round trip comes between the metrics and the centrality.
+template <int VEC>
+__global__ void __launch_bounds__(128)
+accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int n_layers, int n, float lambda,
+                    const float* __restrict__ metrics, float3 weights, int l_limit, float* __restrict__ c_out,
+                    volatile int* host, int tag) {
+  using T = typename Keys<VEC>::T;
+  __shared__ int pivot_s;
+  pdl_trigger();
+  pdl_wait();
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    constexpr int kPer = kMaxStatLayers / 32;
+    double Tl[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) Tl[k] = 0.0;
+    for (int col = 0; col < 3; ++col) {
+      const double sign = col == 0 ? -1.0 : 1.0, w = col == 0 ? weights.x : col == 1 ? weights.y : weights.z;
+      double d[kPer], lo = INFINITY, hi = -INFINITY;
+      int nan = 0;
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        const int l = lane + 32 * k;
+        if (l < n_layers) {
+          const float m = metrics[l * 3 + col], before = l > 0 ? metrics[(l - 1) * 3 + col] : 0.f;
+          nan |= isnan(m);
+          d[k] = sign * ((double)m - (double)before);
+          if (l > 0) { lo = d[k] < lo ? d[k] : lo; hi = d[k] > hi ? d[k] : hi; }
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double a = __shfl_xor_sync(0xffffffffu, lo, o), b = __shfl_xor_sync(0xffffffffu, hi, o);
+        lo = a < lo ? a : lo;
+        hi = b > hi ? b : hi;
+      }
+      if (__any_sync(0xffffffffu, nan) || !(hi > lo)) continue;
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) {
+        const int l = lane + 32 * k;
+        if (l > 0 && l < n_layers)
+          Tl[k] = __dadd_rn(Tl[k], __ddiv_rn(__dmul_rn(w, __dsub_rn(d[k], lo)), __dsub_rn(hi, lo)));
+      }
+    }
+    double best = -INFINITY;
+    int at = kMaxStatLayers;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const int l = lane + 32 * k;
+      if (l > 0 && l < n_layers && Tl[k] > best) { best = Tl[k]; at = l; }
+      if (blockIdx.x == 0 && l < n_layers) {
+        host[1 + l] = __float_as_int((float)Tl[k]);
+        __threadfence_system();
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double b = __shfl_xor_sync(0xffffffffu, best, o);
+      const int i = __shfl_xor_sync(0xffffffffu, at, o);
+      if (b > best || (b == best && i < at)) { best = b; at = i; }
+    }
+    if (at == kMaxStatLayers) at = n_layers >= 2 ? 1 : 0;   // one layer, or nothing compares
+    if (n_layers >= 2 && l_limit >= 0 && at > l_limit) at = l_limit;
+    __syncwarp();
+    if (lane == 0) {
+      pivot_s = at;
+      if (blockIdx.x == 0) {                           // last: the host polls this word
+        __threadfence_system();
+        host[0] = tag | at;
+      }
+    }
+  }
+  __syncthreads();
+  const int pivot = pivot_s;
+  const int j = (blockIdx.x * blockDim.x + threadIdx.x) * VEC;
+  if (j >= n) return;
+  T c{};
+#pragma unroll 8
+  for (int l = 0; l <= pivot; ++l) c = decay(lambda, c, *reinterpret_cast<const T*>(s_hist + (size_t)l * row_stride + j));
+  *reinterpret_cast<T*>(c_out + j) = c;
+}
+
 }  // namespace
 
 // Raises a kernel's shared-memory limit once per device.
@@ -486,9 +571,10 @@ static FinishArgs finish_args(const Ctx& ctx, const float* cols, long long col_s
 
 cudaError_t launch_finish_layers(const Ctx& ctx, const float* cols, long long layer_stride, long long col_stride, int n,
                                  int n_layers, float lambda, float* s_out, long long s_stride, float* c_inout,
-                                 const float* row_ent, bool with_head_stats, float* metrics, cudaStream_t st) {
+                                 const float* row_ent, bool with_head_stats, float* metrics, cudaStream_t st,
+                                 bool c_from_zero) {
   FinishArgs a = finish_args(ctx, cols, col_stride, n, metrics);
-  a.layer_stride = layer_stride; a.n_prob = n_layers; a.lambda = lambda;
+  a.layer_stride = layer_stride; a.n_prob = n_layers; a.lambda = lambda; a.c_from_zero = c_from_zero;
   a.s_out = s_out; a.s_stride = s_stride; a.c_inout = c_inout; a.row_ent = row_ent;
   a.with_stats = with_head_stats;
   const bool vec = n % 4 == 0 && col_stride % 4 == 0 && layer_stride % 4 == 0 && s_stride % 4 == 0 &&
@@ -512,12 +598,16 @@ cudaError_t launch_finish_packed(const Ctx& ctx, const float* cols, long long co
   return vec ? launch_finish<4>(a, longest, st) : launch_finish<1>(a, longest, st);
 }
 
+// Two sweeps per vector where the vectors fill the GPU several times over and are long: with 1024
+// vectors 85 / 115 / 231 us at 16000 / 32768 / 131072 keys, the register form 91 / 140 / > 500.
+bool head_stats_ride_along(const Ctx& ctx, int n_layers, int n) {
+  return (long long)n_layers * ctx.cfg.n_q_heads < 2ll * ctx.sm_count || n <= 8 * kRxThreads;
+}
+
 cudaError_t launch_head_stats_batch(const Ctx& ctx, const float* cols, long long layer_stride, long long col_stride,
                                     int n_layers, int n, float* metrics, cudaStream_t st) {
   const int H = ctx.cfg.n_q_heads;
-  // Two sweeps per vector where the vectors fill the GPU several times over and are long: with 1024
-  // vectors 85 / 115 / 231 us at 16000 / 32768 / 131072 keys, the register form 91 / 140 / > 500.
-  if ((long long)n_layers * H >= 2ll * ctx.sm_count && n > 8 * kRxThreads) {
+  if (!head_stats_ride_along(ctx, n_layers, n)) {
     static std::atomic<unsigned long long> ready{0};
     const int smem = (kHsBins * kHsCopies + 2 * kHsBins) * (int)sizeof(unsigned);
     cudaError_t e = allow_smem(head_stats, smem, ready);
@@ -538,6 +628,17 @@ cudaError_t launch_accumulate(const float* s_hist, long long row_stride, int piv
   if (n % 4 == 0 && row_stride % 4 == 0 && (uintptr_t)s_hist % 16 == 0 && (uintptr_t)c_out % 16 == 0)
     return launch_pdl(accumulate<4>, dim3((n / 4 + 127) / 128), dim3(128), 0, st, s_hist, row_stride, pivot, n, lambda, c_out);
   return launch_pdl(accumulate<1>, dim3((n + 127) / 128), dim3(128), 0, st, s_hist, row_stride, pivot, n, lambda, c_out);
+}
+
+cudaError_t launch_accumulate_at_pivot(const float* s_hist, long long row_stride, int n_layers, int n, float lambda,
+                                       const float* metrics, const float* weights, int l_limit, float* c_out, int* host,
+                                       int tag, cudaStream_t st) {
+  const float3 w = make_float3(weights[0], weights[1], weights[2]);
+  if (n % 4 == 0 && row_stride % 4 == 0 && (uintptr_t)s_hist % 16 == 0 && (uintptr_t)c_out % 16 == 0)
+    return launch_pdl(accumulate_at_pivot<4>, dim3((n / 4 + 127) / 128), dim3(128), 0, st, s_hist, row_stride, n_layers, n,
+                      lambda, metrics, w, l_limit, c_out, (volatile int*)host, tag);
+  return launch_pdl(accumulate_at_pivot<1>, dim3((n + 127) / 128), dim3(128), 0, st, s_hist, row_stride, n_layers, n, lambda,
+                    metrics, w, l_limit, c_out, (volatile int*)host, tag);
 }
 
 }  // namespace skv

@@ -20,6 +20,7 @@ struct SelectArgs {
   // packed sequences: vector b is scores[cu[b] .. cu[b + 1]) with its own budget; the row's remainder reads -1
   int packed;
   int cu[kMaxBatch + 1], budgets[kMaxBatch];
+  SelectExtra extra;                   // vector `batch` of a uniform call, if it has scores
 };
 
 template <int CL, int ITEMS>
@@ -34,9 +35,10 @@ __global__ void __launch_bounds__(kRxThreads, ITEMS <= 8 ? 2 : 1) select_topk(co
   radix_clear(s, 0);
   cluster_barrier<CL>();                             // all CTAs of the cluster run before any remote access
   pdl_wait();
-  const float* x = a.scores + (a.packed ? (size_t)a.cu[vec] : (size_t)vec * a.row_stride);
-  const int n = a.packed ? a.cu[vec + 1] - a.cu[vec] : a.n, budget = a.packed ? a.budgets[vec] : a.budget;
-  int* out = a.out + (size_t)vec * a.out_stride;
+  const bool own = !a.packed && vec == a.batch;      // the extra vector
+  const float* x = own ? a.extra.scores : a.scores + (a.packed ? (size_t)a.cu[vec] : (size_t)vec * a.row_stride);
+  const int n = a.packed ? a.cu[vec + 1] - a.cu[vec] : a.n, budget = own ? a.extra.budget : a.packed ? a.budgets[vec] : a.budget;
+  int* out = own ? a.extra.idx_out : a.out + (size_t)vec * a.out_stride;
   const int prefix_len = n - a.window, k = budget - a.window;
   if (rank == 0) {
     for (int i = tid; i < a.window; i += kRxThreads) out[k + i] = prefix_len + i;
@@ -174,7 +176,7 @@ cudaError_t launch(const SelectArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     ready.fetch_or(bit, std::memory_order_release);
   }
-  return launch_cluster<CL>(select_topk<CL, ITEMS>, a.batch * CL, sizeof(RadixShared<CL>), st, a);
+  return launch_cluster<CL>(select_topk<CL, ITEMS>, (a.batch + (a.extra.scores ? 1 : 0)) * CL, sizeof(RadixShared<CL>), st, a);
 }
 
 // The smallest cluster and the fewest items per thread that hold a vector, as measured (us for 1 / 32
@@ -197,8 +199,9 @@ cudaError_t dispatch(const SelectArgs& a, int longest, cudaStream_t st) {
 }  // namespace
 
 cudaError_t launch_select(const float* scores, long long row_stride, int batch, int n, int budget, int window,
-                          int* idx_out, cudaStream_t st) {
+                          int* idx_out, cudaStream_t st, const SelectExtra* extra) {
   SelectArgs a;
+  a.extra = extra ? *extra : SelectExtra{nullptr, 0, nullptr};
   a.scores = scores; a.out = idx_out; a.row_stride = row_stride; a.out_stride = budget;
   a.n = n; a.budget = budget; a.window = window; a.batch = batch; a.packed = 0;
   return dispatch(a, n - window, st);
@@ -207,6 +210,7 @@ cudaError_t launch_select(const float* scores, long long row_stride, int batch, 
 cudaError_t launch_select_packed(const float* scores, const int* cu_seqlens, const int* budgets, int batch, int window,
                                  int* idx_out, long long idx_stride, cudaStream_t st) {
   SelectArgs a;
+  a.extra = SelectExtra{nullptr, 0, nullptr};
   a.scores = scores; a.out = idx_out; a.row_stride = 0; a.out_stride = idx_stride;
   a.n = a.budget = 0; a.window = window; a.batch = batch; a.packed = 1;
   int longest = 0;

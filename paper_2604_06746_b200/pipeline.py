@@ -53,8 +53,8 @@ class Prefill:
         self.head_cols = (torch.empty((n_layers, n_q_heads, seq), dtype=f32, device=dev) if self.defer else None)
         self._stats_done = 0
         self._layers_ws = None
-        self._side = None
         self._kv_sources = None
+        self._plan = None
 
     # -- Algorithm 1 lines 3-6 for one layer
     def score(self, layer: int, q_win: torch.Tensor, k: torch.Tensor, scale: float,
@@ -104,19 +104,9 @@ class Prefill:
     def detect_and_select(self, n_scored: Optional[int] = None) -> int:
         L = self.L if n_scored is None else n_scored
         self.finish_scores(L)
-        # The per-layer selections (Eq. 13) do not depend on the pivot: they are enqueued first, and the
-        # metric table travels to the host on a side stream meanwhile, so the device is not idle while
-        # the host evaluates Eq. 7-9.
-        main = torch.cuda.current_stream(self.device)
-        if self._side is None:
-            self._side = torch.cuda.Stream(device=self.device)
-        ready = torch.cuda.Event()
-        ready.record(main)
-        self._side.wait_event(ready)
-        self.ctx.select(self.s_hist[:L], self.kv_budget, self.w, self.i_kv[:L])
-        self.pivot, self.transition = self.ctx.pivot(self.metrics[:L], self.weights, self.l_limit, stream=self._side)
-        self.ctx.accumulate(self.s_hist, self.pivot, self.lam, self.c_star)
-        self.ctx.select(self.c_star, self.struct_budget, self.w, self.i_struct)
+        self.pivot, self.transition = self.ctx.pivot_select(
+            self.s_hist[:L], self.metrics[:L], self.weights, self.l_limit, self.lam, self.w, self.kv_budget, self.i_kv[:L],
+            self.struct_budget, self.c_star, self.i_struct)
         return self.pivot
 
     # -- Algorithm 1 line 17 for one layer
@@ -188,10 +178,77 @@ class Prefill:
 
     def run(self, layers: Sequence[Dict[str, torch.Tensor]], hidden: Optional[torch.Tensor] = None,
             positions: Optional[torch.Tensor] = None) -> int:
-        """Whole path over resident per-layer tensors (dicts with q_win, k, v, scale)."""
+        """Whole path over resident per-layer tensors (dicts with q_win, k, v, scale): one library call where every
+        layer keeps K and V in one joint allocation and all share one layout, otherwise step by step."""
+        args = self._prefill_args(layers, hidden, positions)
+        if args is not None:
+            self.pivot, self.transition = self.ctx.prefill(args)
+            self._stats_done = self.L
+            return self.pivot
         self.score_all(layers)
         self.detect_and_select(len(layers))
         self.compact_all_kv(layers)
         if hidden is not None:
             self.compact_hidden(hidden, positions)
         return self.pivot
+
+    def _prefill_args(self, layers, hidden, positions) -> Optional[binding.PrefillArgs]:
+        """The argument block of the one-call path, laid out once per set of tensors (None: not in that form).
+        A block is used again only for the very same tensors at the same addresses."""
+        plan = self._plan
+        if plan is not None and len(layers) == len(plan["layers"]) and hidden is plan["hidden"] and positions is plan["positions"]:
+            for t, (q, k, kv, scale, qp, kp, kvp) in zip(layers, plan["layers"]):
+                if not (t["q_win"] is q and t["k"] is k and t.get("kv") is kv and t["scale"] == scale and q.data_ptr() == qp
+                        and k.data_ptr() == kp and kv.data_ptr() == kvp):
+                    break
+            else:
+                if hidden is None or (hidden.data_ptr(), positions.data_ptr()) == plan["rows"]:
+                    return plan["args"]
+        L = len(layers)
+        if not (self.defer and self.keep_kv and L == self.L and L <= 128 and all("kv" in t for t in layers)
+                and self.flags in (0, binding.FLAG_INPUTS_READY)):
+            return None
+        k0, kv0 = layers[0]["k"], layers[0]["kv"]
+        if not all(t["k"].shape == k0.shape and t["k"].stride() == k0.stride() and t["kv"].shape == kv0.shape
+                   and t["kv"].stride() == kv0.stride() and t["k"].dtype == t["q_win"].dtype == t["kv"].dtype == self.dtype
+                   and t["q_win"].is_contiguous() for t in layers):
+            return None
+        if k0.stride(2) != 1 or k0.shape[1] != self.N or kv0.shape != (2, self.Hkv, self.N, self.d):
+            return None
+        if hidden is not None and not (self.hidden_out is not None and hidden.dim() == 2 and hidden.stride(1) == 1
+                                       and hidden.shape == (self.N, self.hidden_out.shape[1])
+                                       and hidden.dtype == self.hidden_out.dtype and positions.dim() == 1
+                                       and positions.shape[0] == self.N and positions.dtype == self.pos_out.dtype):
+            return None
+        src = self.ctx.layer_sources([t["kv"].view(2 * self.Hkv, self.N, self.d) for t in layers])
+        if self._layers_ws is None:
+            self._layers_ws = self.ctx.layers_workspace(self.L)
+        vp, f = binding._vp, binding._f
+        a = binding.PrefillArgs()
+        a.n_layers, a.n_keys, a.lam, a.l_limit, a.window = L, self.N, self.lam, self.l_limit, self.w
+        a.q_windows = (vp * L)(*[t["q_win"].data_ptr() for t in layers])
+        a.ks = (vp * L)(*[t["k"].data_ptr() for t in layers])
+        a.scales = (f * L)(*[t["scale"] for t in layers])
+        a.k_stride_head, a.k_stride_token = k0.stride(0), k0.stride(1)
+        a.s_out, a.s_layer_stride, a.c_out = self.s_hist.data_ptr(), self.s_hist.stride(0), self.c_running.data_ptr()
+        a.head_cols, a.head_cols_layer_stride = self.head_cols.data_ptr(), self.head_cols.stride(0)
+        a.metrics = self.metrics.data_ptr()
+        a.layers_workspace, a.layers_workspace_bytes = self._layers_ws.data_ptr(), self._layers_ws.numel()
+        a.weights = (f * 3)(*self.weights)
+        a.kv_budget, a.struct_budget = self.kv_budget, self.struct_budget
+        a.i_kv, a.i_struct, a.c_star = self.i_kv.data_ptr(), self.i_struct.data_ptr(), self.c_star.data_ptr()
+        a.kv_srcs = src.ptrs
+        a.kv_slab_stride_bytes, a.kv_row_stride_bytes = src.slab_stride_bytes, src.row_stride_bytes
+        a.kv_row_bytes, a.kv_slabs, a.kv_rows = src.row_bytes, src.n_slabs, src.n_rows
+        a.kv_dst, a.kv_dst_layer_stride_bytes = self.kv_out.data_ptr(), self.kv_out.stride(0) * self.kv_out.element_size()
+        if hidden is not None:
+            es, ps = hidden.element_size(), positions.element_size()
+            a.hidden, a.hidden_row_stride_bytes, a.hidden_row_bytes = hidden.data_ptr(), hidden.stride(0) * es, hidden.shape[1] * es
+            a.hidden_dst = self.hidden_out.data_ptr()
+            a.positions, a.position_row_stride_bytes, a.position_row_bytes = positions.data_ptr(), positions.stride(0) * ps, ps
+            a.positions_dst = self.pos_out.data_ptr()
+        self._plan = {"args": a, "src": src, "hidden": hidden, "positions": positions,
+                      "rows": None if hidden is None else (hidden.data_ptr(), positions.data_ptr()),
+                      "layers": [(t["q_win"], t["k"], t["kv"], t["scale"], t["q_win"].data_ptr(), t["k"].data_ptr(),
+                                  t["kv"].data_ptr()) for t in layers]}
+        return a

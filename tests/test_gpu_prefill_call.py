@@ -1,0 +1,82 @@
+"""structkv_pivot_select and structkv_prefill against the separate calls they stand for: the same bits, the
+same pivot and transition scores, also with a cap, without hidden states, with one layer, and when the
+tensors change from call to call."""
+import pytest
+import torch
+
+from paper_2604_06746_b200 import synth
+
+pytestmark = pytest.mark.gpu
+OUT = ("s_hist", "metrics", "c_running", "c_star", "i_kv", "i_struct", "kv_out")
+
+
+def step_by_step(pf, layers, hidden, positions):
+    """The separate entry points, pivot on the host."""
+    pf.score_all(layers)
+    pf.finish_scores(len(layers))
+    pf.pivot, pf.transition = pf.ctx.pivot(pf.metrics, pf.weights, pf.l_limit)
+    pf.ctx.accumulate(pf.s_hist, pf.pivot, pf.lam, pf.c_star)
+    pf.ctx.select(pf.s_hist, pf.kv_budget, pf.w, pf.i_kv)
+    pf.ctx.select(pf.c_star, pf.struct_budget, pf.w, pf.i_struct)
+    pf.compact_all_kv(layers)
+    if hidden is not None:
+        pf.compact_hidden(hidden, positions)
+
+
+@pytest.mark.parametrize("name,seq,n_layers,budget,l_limit,with_hidden", [
+    ("llama32k", 3000 + 1, 6, 300, -1, True), ("llama32k", 20000, 5, 1000, 2, True), ("tiny", 2048, 4, 256, -1, True),
+    ("qwen64k", 1500, 3, 200, 1, False), ("llama32k", 900, 1, 100, -1, True)])
+def test_one_call_equals_the_separate_calls(cuda_device, name, seq, n_layers, budget, l_limit, with_hidden):
+    from paper_2604_06746_b200 import binding, pipeline
+    wl = synth.WORKLOADS[name].scaled(seq, n_layers=n_layers, n_hubs=6, budgets=(budget,))
+    pl = synth.plan(wl)
+    dt = synth.torch_dtype(wl.dtype)
+    sets = []
+    for shift in (0, 1):                                  # two prompts: a reused context must not mix them up
+        ls = [synth.make_layer(wl, pl, (l + shift) % n_layers, device=cuda_device) for l in range(n_layers)]
+        hid = torch.randn((seq, 96), device=cuda_device).to(torch.bfloat16) if with_hidden else None
+        pos = torch.arange(seq, device=cuda_device, dtype=torch.int32) + shift if with_hidden else None
+        sets.append((ls, hid, pos))
+    make = lambda: pipeline.Prefill(wl.n_layers, wl.n_q_heads, wl.n_kv_heads, wl.head_dim, wl.window, wl.seq, budget,
+                                    wl.struct_budget(), dt, hidden_dim=96 if with_hidden else 0, device=cuda_device,
+                                    l_limit=l_limit)
+    one, ref = make(), make()
+    one.c_running.fill_(7.0)                              # C starts from zero whatever the buffer holds
+    for ls, hid, pos in (sets[0], sets[1], sets[1], sets[0]):
+        one.run(ls, hid, pos)
+        assert one._plan is not None
+        step_by_step(ref, ls, hid, pos)
+        torch.cuda.synchronize()
+        assert one.pivot == ref.pivot and one.transition == ref.transition
+        for key in OUT + (("hidden_out", "pos_out") if with_hidden else ()):
+            assert torch.equal(getattr(one, key), getattr(ref, key)), key
+    assert one.ctx.poll_device_status() == binding.OK
+
+
+def test_pivot_on_the_device_equals_the_host_rule(cuda_device):
+    """Ties, constant columns, NaN columns (head statistics switched off), many layers."""
+    from paper_2604_06746_b200 import binding
+    n, w = 200, 8
+    ctx = binding.Context(8, 2, 64, w, n, torch.float32, cuda_device)
+    g = torch.Generator().manual_seed(1)
+    for L in (1, 2, 3, 33, 128, 131):                     # 131: beyond the device form
+        for kind in range(4):
+            m = torch.rand((L, 3), generator=g)
+            if kind == 1:
+                m[:, 1] = 0.25                            # zero range
+            if kind == 2:
+                m[:, 1:] = float("nan")
+            if kind == 3:
+                m = torch.round(m * 2) / 2                # tied transitions: the first maximum wins
+            m = m.to(cuda_device)
+            s = torch.rand((L, n), device=cuda_device)
+            c1, c2 = torch.zeros(n, device=cuda_device), torch.zeros(n, device=cuda_device)
+            i_kv = torch.zeros((L, 50), dtype=torch.int32, device=cuda_device)
+            i_st = torch.zeros(90, dtype=torch.int32, device=cuda_device)
+            for limit in (-1, 1):
+                got = ctx.pivot_select(s, m, (0.2, 0.3, 0.5), limit, 0.9, w, 50, i_kv, 90, c1, i_st)
+                want = ctx.pivot(m, (0.2, 0.3, 0.5), limit)
+                assert got == want, (L, kind, limit)
+                ctx.accumulate(s, want[0], 0.9, c2)
+                assert torch.equal(c1, c2)
+    ctx.close()
