@@ -1,7 +1,9 @@
 // Small deterministic reductions after the scorers: the sum
 // over heads with the centrality update, per-head sparsity / variance with the layer's metrics, and
 // the closed-form centrality re-accumulation.
+#include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "radix.cuh"
 
@@ -47,7 +49,7 @@ __device__ __forceinline__ float block_total(float v, float* red) {
   if (lane == 0) red[warp] = v;
   __syncthreads();
   if (warp == 0) {
-    v = red[lane];
+    v = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.f;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   }
@@ -62,16 +64,22 @@ __device__ __forceinline__ float4 decay(float l, const float4& c, const float4& 
 }
 __device__ __forceinline__ float decay(float l, float c, float s) { return fmaf(l, c, s); }
 
+template <int VEC>
+struct SumShared {
+  typename Keys<VEC>::T part[kSumGroups - 1][kSumLanes];
+  float red[32];
+  int last;
+};
 // Keys [chunk * 128 * VEC, ...) of problem p: eight groups of heads side by side (one chain of H loads
 // took 9 us), their sums added in group order.  The centrality of several layers is a recursion over
 // them: the block that completes a key range takes all of its layers.
 // THREADS: each row of 128 threads takes kSumGroups * 128 / THREADS of the groups.
 template <int VEC, int THREADS>
-__device__ __forceinline__ void sum_block(const FinishArgs& a, int p, int chunk) {
+__device__ __forceinline__ void sum_block(const FinishArgs& a, SumShared<VEC>& sh, int p, int chunk) {
   using T = typename Keys<VEC>::T;
-  __shared__ T part[kSumGroups - 1][kSumLanes];
-  __shared__ float red[32];
-  __shared__ int last;
+  auto& part = sh.part;
+  float* const red = sh.red;
+  int& last = sh.last;
   const Problem pb = problem_of(a, p);
   constexpr int kRows = THREADS / kSumLanes, kMine = kSumGroups / kRows;
   const int lane_j = threadIdx.x & (kSumLanes - 1), grp = threadIdx.x / kSumLanes;
@@ -142,32 +150,39 @@ __device__ __forceinline__ void sum_block(const FinishArgs& a, int p, int chunk)
   }
 }
 
-// Eq. 5 and 6 of one (problem, head) vector, by a cluster: the sum of squared deviations from 1/n (the
-// pooled vector sums to 1, so 1/n is its mean; summing deviations instead of squares keeps
-// near-uniform attention from cancelling) and the mass of the floor(n / 10) largest entries.  Three
-// radix levels give the threshold to 24 bits; of the entries that share them, the ones still wanted
-// count with their average.  All entries are >= 0: the order of the bit patterns is theirs.
-template <int CL, int ITEMS>
-__device__ __forceinline__ void stats_cta(const FinishArgs& a, RadixShared<CL>& s, int vec) {
+// Eq. 5 and 6 of one (problem, head) vector, by a cluster or by one CTA: the sum of squared deviations
+// from 1/n (the pooled vector sums to 1, so 1/n is its mean; summing deviations instead of squares
+// keeps near-uniform attention from cancelling) and the mass of the floor(n / 10) largest entries.
+// Three radix levels give the threshold to 24 bits; of the entries that share them, the ones still
+// wanted count with their average; a level that settles it is the last.  All entries are >= 0: the
+// order of the bit patterns is theirs.
+template <int ITEMS, typename S>
+__device__ __forceinline__ void stats_cta(const FinishArgs& a, S& s, float* vec_s, int vec) {
+  constexpr int CL = S::CL;
+  constexpr bool RESIDENT = std::is_same_v<S, RadixResident>;
   const int tid = threadIdx.x;
   const int rank = CL > 1 ? (int)cg::this_cluster().block_rank() : 0;
   const int p = vec / a.H;
   const Problem pb = problem_of(a, p);
   const float* x = pb.cols + (size_t)(vec - p * a.H) * a.col_stride;
   const int n = pb.n, per = (n + CL - 1) / CL, lo = min(n, rank * per), hi = min(n, lo + per);
-  constexpr int kChunk = kRxThreads * ITEMS;
+  constexpr int kChunk = S::THREADS * ITEMS;
   const int chunks = (per + kChunk - 1) / kChunk;
   unsigned key[ITEMS];
   auto load = [&](int c) {
 #pragma unroll
     for (int e = 0; e < ITEMS; ++e) {
-      const int j = lo + c * kChunk + e * kRxThreads + tid;
-      key[e] = j < hi ? __float_as_uint(x[j] + 0.f) : 0x80000000u;   // sign bit: no entry (-0 becomes +0)
+      const int j = lo + c * kChunk + e * S::THREADS + tid;
+      key[e] = j < hi ? __float_as_uint((RESIDENT ? vec_s[j] : x[j]) + 0.f) : 0x80000000u;   // sign bit: no entry (-0 becomes +0)
     }
   };
+  if (RESIDENT) {
+    stage_vector(vec_s, x, n);
+    __syncthreads();
+  }
   const float mean = 1.f / (float)n;
   float sq = 0.f;
-  unsigned remaining = (unsigned)max(1, n / 10), thr = 0, in = 0;
+  unsigned remaining = (unsigned)max(1, n / 10), thr = 0, in = 0, known = 0;   // known: mask of the bits found so far
 #pragma unroll 1
   for (int level = 0; level < 3; ++level) {
     const int shift = 24 - 8 * level;
@@ -186,13 +201,15 @@ __device__ __forceinline__ void stats_cta(const FinishArgs& a, RadixShared<CL>& 
     unsigned digit;
     radix_pick(s, level & 1, remaining, digit, in);
     thr |= digit << shift;
+    known = 0xffffffffu << shift;
+    if (in == remaining) break;                      // all entries that share these bits count
   }
   float above = 0.f, inside = 0.f;
   for (int c = 0; c < chunks; ++c) {
     if (chunks > 1) load(c);
 #pragma unroll
     for (int e = 0; e < ITEMS; ++e) {
-      const unsigned top = key[e] & 0xffffff00u;
+      const unsigned top = key[e] & known;
       if (!(key[e] >> 31)) {
         if (top > thr) above += __uint_as_float(key[e]);
         else if (top == thr) inside += __uint_as_float(key[e]);
@@ -245,30 +262,33 @@ __device__ __forceinline__ void stats_cta(const FinishArgs& a, RadixShared<CL>& 
   }
 }
 
-template <int CL, int ITEMS, int VEC>
-__global__ void __launch_bounds__(kRxThreads, ITEMS <= 8 ? 2 : 1) finish(const __grid_constant__ FinishArgs a) {
+template <int ITEMS, int VEC, typename S>
+__global__ void
+__launch_bounds__(S::THREADS, S::THREADS < kRxThreads ? 4 : ITEMS <= 8 && !std::is_same_v<S, RadixResident> ? 2 : 1)
+finish(const __grid_constant__ FinishArgs a) {
   extern __shared__ __align__(16) unsigned char fin_smem[];
-  RadixShared<CL>& s = *reinterpret_cast<RadixShared<CL>*>(fin_smem);
+  S& s = *reinterpret_cast<S*>(fin_smem);
   const bool stats = (int)blockIdx.x < a.n_stat_ctas;
   pdl_trigger();
   if (stats) {
     radix_clear(s, 0);
-    cluster_barrier<CL>();                           // all CTAs of the cluster run before any remote access
+    cluster_barrier<S::CL>();                        // all CTAs of the cluster run before any remote access
   }
   pdl_wait();
   if (stats) {
-    stats_cta<CL, ITEMS>(a, s, blockIdx.x / CL);
+    stats_cta<ITEMS>(a, s, reinterpret_cast<float*>(fin_smem + (sizeof(S) + 15) / 16 * 16), blockIdx.x / S::CL);
   } else {
     const int b = blockIdx.x - a.n_stat_ctas, p = b / a.chunks;
-    if (p < a.n_prob) sum_block<VEC, kRxThreads>(a, p, b - p * a.chunks);
+    if (p < a.n_prob) sum_block<VEC, S::THREADS>(a, *reinterpret_cast<SumShared<VEC>*>(fin_smem), p, b - p * a.chunks);
   }
 }
 constexpr int kSumThreads = 256;     // many short blocks: 16 loads in flight per thread
 template <int VEC>
 __global__ void __launch_bounds__(kSumThreads) sum_layers(const __grid_constant__ FinishArgs a) {
+  __shared__ SumShared<VEC> sh;
   pdl_trigger();
   pdl_wait();
-  sum_block<VEC, kSumThreads>(a, blockIdx.x / a.chunks, blockIdx.x % a.chunks);
+  sum_block<VEC, kSumThreads>(a, sh, blockIdx.x / a.chunks, blockIdx.x % a.chunks);
 }
 
 // ---- Eq. 5-6 of many long vectors: one CTA per vector, two sweeps over memory --------------------
@@ -536,19 +556,36 @@ static cudaError_t allow_smem(K* kernel, int bytes, std::atomic<unsigned long lo
   return e;
 }
 
-template <int CL, int ITEMS, int VEC>
+template <int CL, int ITEMS, int VEC, typename S = RadixShared<CL>>
 static cudaError_t launch_finish_as(FinishArgs& a, int sums, cudaStream_t st) {
   static std::atomic<unsigned long long> ready{0};
-  const cudaError_t e = allow_smem(finish<CL, ITEMS, VEC>, (int)sizeof(RadixShared<CL>), ready);
+  constexpr int smem = std::is_same_v<S, RadixResident> ? kResidentBytes : (int)std::max(sizeof(S), sizeof(SumShared<VEC>));
+  const cudaError_t e = allow_smem(finish<ITEMS, VEC, S>, smem, ready);
   if (e != cudaSuccess) return e;
   a.n_stat_ctas = a.n_prob * a.H * CL;
-  return launch_cluster<CL>(finish<CL, ITEMS, VEC>, (a.n_stat_ctas + sums + CL - 1) / CL * CL, sizeof(RadixShared<CL>), st, a);
+  return launch_cluster<CL, S::THREADS>(finish<ITEMS, VEC, S>, (a.n_stat_ctas + sums + CL - 1) / CL * CL, smem, st, a);
 }
 template <int VEC>
-static cudaError_t launch_finish(FinishArgs& a, int longest, cudaStream_t st) {
+static cudaError_t launch_finish(FinishArgs& a, int longest, int sms, cudaStream_t st) {
   a.chunks = (longest + kSumLanes * VEC - 1) / (kSumLanes * VEC);
   const int sums = a.row_ent ? a.n_prob * a.chunks : 0;
   if (!a.with_stats) return launch_pdl(sum_layers<VEC>, dim3(sums), dim3(kSumThreads), 0, st, a);
+  // More vectors than SMs: four small CTAs share an SM, where those of 1024 threads ran one or two at a time
+  // (1024 vectors of 600 / 1777 / 5003 / 8192 keys: 37.6 / 41.3 / 49.0 / 52.6 us before, 21.4 / 23.5 / 33.2 /
+  // 36.5 now).  Longer vectors do not fit their registers.
+  const int vecs = a.n_prob * a.H;
+  if (vecs > sms && longest <= 32 * RadixSmall::THREADS) {
+    if (longest <= 8 * RadixSmall::THREADS) return launch_finish_as<1, 8, VEC, RadixSmall>(a, sums, st);
+    if (longest <= 16 * RadixSmall::THREADS) return launch_finish_as<1, 16, VEC, RadixSmall>(a, sums, st);
+    return launch_finish_as<1, 32, VEC, RadixSmall>(a, sums, st);
+  }
+  // About one vector per SM: the vector in shared memory.  Clusters would leave some of them for a second
+  // wave, and half an SM holds fewer loads in flight (128 vectors of 1777 / 5003 / 20000 / 50000 keys: 13.6 /
+  // 15.6 / 30.4 / 67.4 us before, 10.7 / 11.3 / 17.3 / 29.2 now; at 12000 14.2 against the 12.9 of 16 items).
+  // With 32 vectors the clusters' extra SMs count for more: 20.7 against 16.5 us at 32768 keys.
+  if (2 * vecs > sms && vecs <= sms && longest <= kResidentMax &&
+      (longest <= 8 * kRxThreads || longest > 16 * kRxThreads))
+    return launch_finish_as<1, 8, VEC, RadixResident>(a, sums, st);
   // one CTA per vector while its registers hold it (no exchange between CTAs), else the smallest
   // cluster that does
   if (longest <= 4 * kRxThreads) return launch_finish_as<1, 4, VEC>(a, sums, st);
@@ -579,7 +616,7 @@ cudaError_t launch_finish_layers(const Ctx& ctx, const float* cols, long long la
   a.with_stats = with_head_stats;
   const bool vec = n % 4 == 0 && col_stride % 4 == 0 && layer_stride % 4 == 0 && s_stride % 4 == 0 &&
                    ((uintptr_t)cols % 16) == 0 && ((uintptr_t)s_out % 16) == 0 && ((uintptr_t)c_inout % 16) == 0;
-  return vec ? launch_finish<4>(a, n, st) : launch_finish<1>(a, n, st);
+  return vec ? launch_finish<4>(a, n, ctx.sm_count, st) : launch_finish<1>(a, n, ctx.sm_count, st);
 }
 
 cudaError_t launch_finish_packed(const Ctx& ctx, const float* cols, long long col_stride, const int* cu_seqlens, int batch,
@@ -595,7 +632,7 @@ cudaError_t launch_finish_packed(const Ctx& ctx, const float* cols, long long co
     vec = vec && cu_seqlens[b] % 4 == 0;
     if (b > 0) longest = cu_seqlens[b] - cu_seqlens[b - 1] > longest ? cu_seqlens[b] - cu_seqlens[b - 1] : longest;
   }
-  return vec ? launch_finish<4>(a, longest, st) : launch_finish<1>(a, longest, st);
+  return vec ? launch_finish<4>(a, longest, ctx.sm_count, st) : launch_finish<1>(a, longest, ctx.sm_count, st);
 }
 
 // Two sweeps per vector where the vectors fill the GPU several times over and are long: with 1024
@@ -620,7 +657,7 @@ cudaError_t launch_head_stats_batch(const Ctx& ctx, const float* cols, long long
   }
   FinishArgs a = finish_args(ctx, cols, col_stride, n, metrics);
   a.layer_stride = layer_stride; a.n_prob = n_layers; a.with_stats = 1;
-  return launch_finish<1>(a, n, st);
+  return launch_finish<1>(a, n, ctx.sm_count, st);
 }
 
 cudaError_t launch_accumulate(const float* s_hist, long long row_stride, int pivot, int n,
