@@ -144,6 +144,8 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
   p.n_prob = n;
   p.window = cfg.window;
   p.w_pad = ctx.w_pad;
+  p.w_shift = 0;
+  while ((1 << p.w_shift) < ctx.w_pad) ++p.w_shift;
   p.group = l.group;
   p.rows_pg = l.rows_pg;
   p.n_rb = l.n_rb;
@@ -157,8 +159,7 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
   p.row_ent = a.row_ent + (size_t)first * ctx.rows_pad;
   p.col_stride = a.col_stride;
   p.status = ctx.ws.status;
-  // (and with many short layers, whose passes are over before the helper is: 315 -> 304 us for 32 of 5003 keys)
-  p.hurry = n == 1 || batch || (long long)l.units * ((p.prob[0].n_keys + 255) / 256) <= 2ll * sms;
+  p.hurry = n == 1 || batch;
   const int grid = std::min(sms, tickets);
   return cfg.head_dim == 128 ? tc_launch_128(l.shape, p, grid, ctx.device, st) : tc_launch_64(l.shape, p, grid, ctx.device, st);
 }

@@ -35,9 +35,11 @@
 // power cap: at 131072 keys the clock settles near 1.6 GHz.
 //
 // Warp roles: warp 0 = ticket taker and TMA producer, warp 1 = MMA issuer (owns the tensor-memory
-// allocation), warp 2 = hands a unit's log-sum-exps to pass 2, warp 3 = folds and stores row
-// statistics (the CTA whose task completes a unit merges its partials), warps 4-19 = compute (four
-// per scheduler).  Tasks reach the consumers through a ring of descriptors in shared memory.
+// allocation), warp 2 = hands a unit's log-sum-exps to pass 2, warp 3 = counts finished
+// pass-1 tasks (the CTA whose task completes a unit merges its partials), warps 4-19 = compute (four
+// per scheduler).  Tasks reach the consumers through a ring of descriptors in shared memory that holds
+// all they need (indexing the launch's parameters by problem cost 1500 clocks of constant-cache misses
+// a task).
 // Every wait is bounded; on expiry the CTA records STRUCTKV_ERR_TIMEOUT and stops issuing work;
 // it then waits (with a fresh bound that ignores the abort flag) for its own copies and MMAs in
 // flight, and frees tensor memory only if those MMAs are known to have retired.
@@ -84,6 +86,7 @@ struct alignas(64) TcParams {
   TcPhase phase[4 * MAXP + 1];         // the last one only carries the ticket count
   int n_phase, n_prob;
   int window, w_pad, group, rows_pg, n_rb, n_units;    // w_pad: rows a head occupies; rows_pg = group * w_pad
+  int w_shift;                         // log2(w_pad)
   int w_group, w_total, w_last;        // weights of a KV group, of all, of a group's last row block
   int* ctl;                            // ticket, exits; then arrivals and ready flags [kMaxBatch][kQueueUnits]
   float2* part;                        // [pass-1 task][256] (log-sum-exp, entropy) in bits
@@ -91,10 +94,10 @@ struct alignas(64) TcParams {
   float* row_ent;                      // [problem][unit][256] entropy of a row, nats (0: no row)
   long long col_stride;
   int* status;
-  // Pass 2 has nothing to do but wait for pass 1 (one layer, a batch): the compute warps fold and merge the
-  // row statistics themselves, all 512 threads at once, instead of leaving it to one helper warp
-  // beside them (at 8192 keys 2 + 2 us instead of 3 + 6).  With layers to interleave the helpers'
-  // time is hidden and the compute warps' is not.
+  // Pass 2 has nothing to do but wait for pass 1 (one layer, a batch): the compute warps count their arrivals
+  // and merge the row statistics themselves, a thread per row, instead of leaving it to one helper
+  // warp beside them (at 8192 keys 2 us instead of 6).  With layers to interleave the helpers' time is
+  // hidden and the compute warps' is not (32 layers of 5003 keys: 317 us in a hurry, 300 without).
   int hurry;
 };
 constexpr int kCtlTicket = 0, kCtlExit = 1, kCtlArrive = 64, kCtlReady = 64 + kMaxBatch * kQueueUnits;
@@ -216,24 +219,6 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, ui
 }
 // 32 lanes x N consecutive fp32 columns: thread l of the warp receives row (lane base + l).  The
 // loaded registers are operands of the wait, so no use of them can be scheduled ahead of it.
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-               : "r"(taddr) : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])
-               :: "memory");
-}
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[16]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
-                 "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
-               : "r"(taddr) : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
-                 "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15])
-               :: "memory");
-}
 __device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[32]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
                "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
@@ -250,6 +235,70 @@ __device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&v)[32]) {
                  "+f"(v[23]), "+f"(v[24]), "+f"(v[25]), "+f"(v[26]), "+f"(v[27]), "+f"(v[28]), "+f"(v[29]),
                  "+f"(v[30]), "+f"(v[31])
                :: "memory");
+}
+// The load and its wait apart: several accumulators' loads travel together.
+template <int RT>
+__device__ __forceinline__ void tmem_ld_issue(uint32_t taddr, float* v) {
+  if constexpr (RT == 8)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "r"(taddr) : "memory");
+  else
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]),
+                   "=f"(v[8]), "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+                 : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait(float (&v)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
+                 "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15])
+               :: "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait(float (&v)[32]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]),
+                 "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]),
+                 "+f"(v[16]), "+f"(v[17]), "+f"(v[18]), "+f"(v[19]), "+f"(v[20]), "+f"(v[21]), "+f"(v[22]),
+                 "+f"(v[23]), "+f"(v[24]), "+f"(v[25]), "+f"(v[26]), "+f"(v[27]), "+f"(v[28]), "+f"(v[29]),
+                 "+f"(v[30]), "+f"(v[31])
+               :: "memory");
+}
+// Largest value of a warp, in every lane.
+__device__ __forceinline__ float warp_max(float x) {
+  float m;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(x));
+  return m;
+}
+// Sums x[0 .. N) over the warp; lane l ends with the total of element l / (32 / N).  N + 4 - log2 N shuffles
+// instead of 5 N: each halving leaves a lane half as many elements.
+template <int N, int O = 16>
+__device__ __forceinline__ float warp_sum_scatter(const float (&x)[N], int lane) {
+  if constexpr (N == 1) {
+    float t = x[0];
+#pragma unroll
+    for (int o = O; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+  } else {
+    float y[N / 2];
+    const bool up = lane & O;
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i)
+      y[i] = (up ? x[i + N / 2] : x[i]) + __shfl_xor_sync(0xffffffffu, up ? x[i] : x[i + N / 2], O);
+    return warp_sum_scatter<N / 2, O / 2>(y, lane);
+  }
+}
+// Element l / (32 / N) of x for lane l.
+template <int N, int O = 16>
+__device__ __forceinline__ float lane_element(const float (&x)[N], int lane) {
+  if constexpr (N == 1) {
+    return x[0];
+  } else {
+    float y[N / 2];
+#pragma unroll
+    for (int i = 0; i < N / 2; ++i) y[i] = lane & O ? x[i + N / 2] : x[i];
+    return lane_element<N / 2, O / 2>(y, lane);
+  }
 }
 
 // Two fp32 values in one 64-bit register, for the packed fp32 instructions of sm_100
@@ -362,13 +411,28 @@ __host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
 }
 
 // ---- shared memory layout ----------------------------------------------------------------
+// What a task's consumers need to know, in one piece of shared memory: parameters of the launch indexed by
+// problem would be constant-memory misses on the way from one task to the next.
+struct alignas(16) TcTask {
+  int pass, unit, lo, hi;              // pass 0: no task left; key tiles [lo, hi)
+  int n_keys, rows, row0, slot;        // score rows of the KV group from the unit's first on; that row; (problem, unit)
+  float c2, v_min, inv_c2;
+  int negate;
+  float* cols;                         // pass 2: output of the KV group's first head
+  int prob, group;
+  int part, part0, n_part, pad;        // pass 1: where its statistics go; the unit's partials
+};
+constexpr int kTaskBytes = 96;
+static_assert(sizeof(TcTask) <= kTaskBytes && sizeof(TcTask) % 16 == 0, "task slot");
 template <int SH>
 struct Shape {
   static constexpr bool kNarrow = SH >= kNarrow32;
   static constexpr int kRows = SH == kNarrow32 ? 32 : SH == kNarrow64 ? 64 : kRowBlock;   // score rows of a unit
   static constexpr int kW = SH == kWide16 ? 16 : SH == kWide32 ? 32 : SH == kWide64 ? 64 : SH == kWide128 ? 128 : 256;
   static constexpr int kQHalves = kNarrow ? 1 : 2;         // parts the Q block is loaded in
+  static constexpr int kQBufs = kNarrow ? 2 : 1;           // Q blocks held (of wide ones two do not fit)
   static constexpr int kAcc = kNarrow ? 8 : 2;             // accumulator ring in tensor memory
+  static constexpr int kFoldWarps = kNarrow ? 4 : 8;       // compute warps that store a pass-1 task's statistics
   static constexpr int kAccCols = 512 / kAcc;
 };
 template <int D, int SH>
@@ -381,31 +445,31 @@ struct Smem {
   static constexpr int kKBytes = kKSub * kSub;             // bytes TMA delivers per stage
   // K ring, sub-tile major: sub-tile c of stage s sits at kKOff + (c * kStages + s) * kKSub, so the
   // same sub-tile of stages s and s + 1 is one contiguous 256-key operand
-  static constexpr int kKOff = kQBytes;
+  static constexpr int kKOff = kQBytes * Shape<SH>::kQBufs;
   static constexpr int kOnesOff = kKOff + kStages * kKBytes;       // extra K-step, key side: 128 x 16 bf16
-  static constexpr int kExtOff = kOnesOff + kKeyTile * 32;         // extra K-step, row side: kRows x 16 bf16
-  static constexpr int kPartOff = kExtOff + kRows * 32;            // [4][kRows] partials (log-sum-exp, entropy)
-  static constexpr int kTaskOff = kPartOff + 4 * kRows * 8;        // task ring, 64 bytes a slot
-  static constexpr int kBarOff = kTaskOff + kTaskRing * 64;
+  static constexpr int kExtOff = kOnesOff + kKeyTile * 32;         // extra K-step, row side: [2][kRows x 16] bf16
+  static constexpr int kPartOff = kExtOff + 2 * kRows * 32;        // [2][3][kRows] partials (log-sum-exp, entropy)
+  static constexpr int kTaskOff = kPartOff + 2 * 3 * kRows * 8;    // task ring
+  static constexpr int kBarOff = kTaskOff + kTaskRing * kTaskBytes;
   static constexpr int kBytes = kBarOff + 512;
   static constexpr int kAlloc = kBytes + 1024;             // slack to align the base to 1024 bytes
   static_assert(kAlloc <= 227 * 1024, "shared memory of one CTA");
 };
-struct TcTask { int pass, prob, g, rb, lo, hi, part, part0, n_part; };   // pass 0: no task left
 
 // Barrier slots (8 bytes each) inside the barrier area.
 enum { kBarFull = 0, kBarEmpty = kBarFull + kStages, kBarTaskFull = kBarEmpty + kStages,
        kBarTaskEmpty = kBarTaskFull + kTaskRing, kBarQFull = kBarTaskEmpty + kTaskRing, kBarQEmpty = kBarQFull + 2,
-       kBarExtFull = kBarQEmpty + 2, kBarExtEmpty, kBarSync, kBarPartFull, kBarPartEmpty, kBarDrain, kBarAccFull,
+       kBarExtFull = kBarQEmpty + 2, kBarExtEmpty = kBarExtFull + 2, kBarFold = kBarExtEmpty + 2,
+       kBarPartFull = kBarFold + 4, kBarPartEmpty, kBarDrain, kBarAccFull,
        kBarAccEmpty = kBarAccFull + 8, kBarCount = kBarAccEmpty + 8 };
 constexpr int kTaskConsumers = 3 + kComputeWarps;          // MMA, lse hand-over, fold, compute warps
 
-// The four column groups (wide) or lane quarters (narrow) of a row fold into one partial.
-template <int R>
-__device__ __forceinline__ float2 fold_row(const float2* part_s, int r) {
+// The four column groups (wide) or lane quarters (narrow) of a row fold into one partial, in this order; the
+// thread that folds holds the own-th of them.
+__device__ __forceinline__ float2 fold_row(const float2* part_s, int stride, float2 mine, int own) {
   float2 c[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) c[k] = part_s[k * R + r];
+  for (int k = 0; k < 4; ++k) c[k] = k == own ? mine : part_s[(k < own ? k : k - 1) * stride];
   float M = -INFINITY, W = 0.f, X = 0.f;
   merge_partials(M, W, X, c);
   const float lw = __log2f(W);
@@ -426,7 +490,7 @@ __device__ __forceinline__ void merge_unit(const float2* part, int n_part, int l
       for (int b = 0; b < kBatch; ++b)
 #pragma unroll
         for (int q = 0; q < kRowsAt; ++q)
-          pv[q][b] = s0 + b < n_part ? __ldcg(part + (size_t)(s0 + b) * kRowBlock + r0 + 32 * q) : make_float2(-INFINITY, 0.f);
+          pv[q][b] = s0 + b < n_part ? __ldcg(part + (size_t)(s0 + b) * R + r0 + 32 * q) : make_float2(-INFINITY, 0.f);
 #pragma unroll
       for (int q = 0; q < kRowsAt; ++q) merge_partials(M[q], W[q], X[q], pv[q]);
     }
@@ -522,15 +586,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sm + L::kBarOff + 8 * kBarCount + 8);
   volatile int* mma_in_flight = reinterpret_cast<volatile int*>(sm + L::kBarOff + 8 * kBarCount + 16);
   volatile int* last_flag = reinterpret_cast<volatile int*>(sm + L::kBarOff + 8 * kBarCount + 24);
-  auto task_slot = [&](int k) { return reinterpret_cast<volatile int*>(sm + L::kTaskOff + k * 64); };
+  auto task_slot = [&](int k) { return reinterpret_cast<TcTask*>(sm + L::kTaskOff + k * kTaskBytes); };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) { mbar_init(bar(kBarFull + s), 1); mbar_init(bar(kBarEmpty + s), 1); }
     for (int s = 0; s < kTaskRing; ++s) { mbar_init(bar(kBarTaskFull + s), 1); mbar_init(bar(kBarTaskEmpty + s), kTaskConsumers); }
-    for (int b = kBarQFull; b <= kBarExtEmpty; ++b) mbar_init(bar(b), 1);
-    mbar_init(bar(kBarPartFull), kComputeWarps);
-    mbar_init(bar(kBarSync), kComputeWarps);
+    for (int b = kBarQFull; b < kBarFold; ++b)
+      mbar_init(bar(b), p.hurry && b >= kBarExtFull && b < kBarExtEmpty ? R / 32 : 1);
+    for (int b = 0; b < 4; ++b) mbar_init(bar(kBarFold + b), 4);
+    mbar_init(bar(kBarPartFull), S::kFoldWarps);
     mbar_init(bar(kBarPartEmpty), 1);
     mbar_init(bar(kBarDrain), 1);
     for (int a = 0; a < S::kAcc; ++a) { mbar_init(bar(kBarAccFull + a), 1); mbar_init(bar(kBarAccEmpty + a), kComputeWarps); }
@@ -543,7 +608,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   // operands of pass 2's extra K-step: 1.0 in the first three K columns on the key side, zeros elsewhere
-  for (int i = threadIdx.x; i < (kKeyTile + R) * 32 / 16; i += kTcThreads)
+  for (int i = threadIdx.x; i < (kKeyTile + 2 * R) * 32 / 16; i += kTcThreads)
     reinterpret_cast<uint4*>(sm + L::kOnesOff)[i] =
         i < kKeyTile * 2 && (i & 8) == 0 ? make_uint4(0x3f803f80u, 0x00003f80u, 0u, 0u) : make_uint4(0u, 0u, 0u, 0u);
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -562,26 +627,31 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     if (lane == 0)
       ok = mbar_wait_producer(bar(kBarTaskFull + k), (uint32_t)(n / kTaskRing) & 1u, abort_flag, kWaitCycles) ? 1 : 0;
     if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
-    volatile int* s = task_slot(k);
-    t = TcTask{s[0], s[1], s[2], s[3], s[4], s[5], s[6], s[7], s[8]};
+    asm volatile("" ::: "memory");
+    t = *task_slot(k);
+    asm volatile("" ::: "memory");
     __syncwarp();
     if (lane == 0) mbar_arrive(bar(kBarTaskEmpty + k));
     return t.pass != 0;
   };
   // -lse / c2 of a row as hi + mid + lo (bf16 each: 24 bits together) into the extra K-step's operand; rows
   // that do not exist get a huge negative value so that their 2^x is 0.
-  auto put_lse = [&](int r, float nlse, float inv_c2) {
+  auto put_lse = [&](int buf, int r, float nlse, float inv_c2) {
     const float Lv = nlse == -INFINITY ? kMaskedAcc : nlse * inv_c2;
     const __nv_bfloat16 hi = __float2bfloat16_rn(Lv);
     const float r1 = Lv - __bfloat162float(hi);
     const __nv_bfloat16 mid = __float2bfloat16_rn(r1);
     const __nv_bfloat16 lo = __float2bfloat16_rn(r1 - __bfloat162float(mid));
-    unsigned char* bx = sm + L::kExtOff;
+    unsigned char* bx = sm + L::kExtOff + buf * (R * 32);
     *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 0)) = hi;
     *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 1)) = mid;
     *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 2)) = lo;
   };
-  auto is_row = [&](int row) { return row < p.rows_pg && row % p.w_pad < p.window; };   // row of the KV group, padding excluded
+  auto is_row = [&](int row) { return row < p.rows_pg && (row & (p.w_pad - 1)) < p.window; };   // row of the KV group, padding excluded
+  // The n-th Q block: wide ones come in halves with a barrier each, narrow ones alternate between two buffers.
+  auto q_bar = [](int n, int half) { return S::kQBufs == 2 ? n & 1 : half; };
+  auto q_parity = [](int n) { return (uint32_t)(S::kQBufs == 2 ? n >> 1 : n) & 1u; };
+  auto q_buf = [](int n) { return S::kQBufs == 2 ? (n & 1) * L::kQBytes : 0; };
   // Tiles of item `it` of a task: pass 1 ascends, pass 2 descends; half 1 may be missing at the end.
   auto tile_of = [](const TcTask& t, int it, int half) { return t.pass == 1 ? t.lo + 2 * it + half : t.hi - 1 - 2 * it - half; };
   auto present = [](const TcTask& t, int tile) { return tile >= t.lo && tile < t.hi; };
@@ -594,25 +664,28 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
       int* const ticket = p.ctl + kCtlTicket;
       const int n_tickets = p.phase[p.n_phase].first;
       int tk = atomicAdd(ticket, 1), ph = 0;
-      int st = 0, n_q = 0, q_loads = 0;                    // K stages used, Q blocks loaded, halves of Q requested so far
+      int st = 0, n_q = 0;                                 // K stages used, Q blocks loaded so far
+      unsigned q_uses[2] = {0, 0};                         // copies behind each Q barrier
       unsigned real = 0;                                   // stages whose last use was a copy
       for (int n = 0;; ++n) {
         TcTask t{};
+        int g = 0, rb = 0;
         if (tk < n_tickets) {
           while (tk >= p.phase[ph + 1].first) ++ph;
           t.pass = p.phase[ph].pass;
           t.prob = p.phase[ph].prob;
+          t.group = p.group;
           const TcProblem& pb = p.prob[t.prob];
           const int tasks = t.pass == 1 ? pb.t1 : pb.t2;
           int i = p.phase[ph].task0 + tk - p.phase[ph].first;
           if (t.pass == 2) i = tasks - 1 - i;              // pass 2 starts with the keys pass 1 touched last
           // the unit whose share [tc_deal(W), tc_deal(W + w)) holds task i
           const int w_at = ((i + 1) * p.w_total - 1) / tasks;
-          t.g = w_at / p.w_group;
-          t.rb = min((w_at - t.g * p.w_group) / kFullWeight, p.n_rb - 1);
-          const int w0 = t.g * p.w_group + t.rb * kFullWeight;
+          g = w_at / p.w_group;
+          rb = min((w_at - g * p.w_group) / kFullWeight, p.n_rb - 1);
+          const int w0 = g * p.w_group + rb * kFullWeight;
           const int i0 = tc_deal(w0, tasks, p.w_total);
-          const int w_unit = t.rb == p.n_rb - 1 ? p.w_last : kFullWeight;
+          const int w_unit = rb == p.n_rb - 1 ? p.w_last : kFullWeight;
           const int n_seg = tc_deal(w0 + w_unit, tasks, p.w_total) - i0;
           const int seg = i - i0, n_tiles = (pb.n_keys + kKeyTile - 1) / kKeyTile;
           if (t.pass == 1) {
@@ -629,13 +702,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
           const int p0 = tc_deal(w0, pb.t1, p.w_total);
           t.n_part = tc_deal(w0 + w_unit, pb.t1, p.w_total) - p0;
           t.part0 = pb.part0 + p0;
+          t.unit = g * p.n_rb + rb;
+          t.slot = t.prob * p.n_units + t.unit;
+          t.n_keys = pb.n_keys;
+          t.row0 = rb * R;
+          t.rows = p.rows_pg - rb * R;
+          t.c2 = pb.c2; t.v_min = pb.v_min; t.inv_c2 = pb.inv_c2; t.negate = pb.negate;
+          t.cols = pb.cols + (size_t)g * p.group * p.col_stride;
           tk = atomicAdd(ticket, 1);                       // travels while this task is loaded
         }
         const int k = n % kTaskRing;
         if (!mbar_wait_producer(bar(kBarTaskEmpty + k), ((uint32_t)(n / kTaskRing) & 1u) ^ 1u, abort_flag, kWaitCycles)) break;
-        volatile int* s = task_slot(k);
-        s[0] = t.pass; s[1] = t.prob; s[2] = t.g; s[3] = t.rb; s[4] = t.lo; s[5] = t.hi;
-        s[6] = t.part; s[7] = t.part0; s[8] = t.n_part;
+        *task_slot(k) = t;
         mbar_arrive(bar(kBarTaskFull + k));
         if (t.pass == 0) break;
         const TcProblem& pb = p.prob[t.prob];
@@ -658,21 +736,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
             // sequence of a packed batch): the causal mask discards those keys
             for (int c = 0; c < L::kSub; ++c)
               tma_load_3d_hint(base + L::kKOff + (c * kStages + sg) * L::kKSub, &p.map_k[pb.map], bar(kBarFull + sg),
-                               c * 64, pb.key0 + tile * kKeyTile, t.g, tile >= keep_from ? pol_keep : pol_stream);
+                               c * 64, pb.key0 + tile * kKeyTile, g, tile >= keep_from ? pol_keep : pol_stream);
           }
           if (it == 0 && ok) {
             // The Q block, behind the first keys, in halves: each waits for the previous task's MMAs on it,
             // and pass 1 is done with the first half an accumulator earlier.
-            const int head = pb.head0 + t.g * p.group + t.rb * (R / p.w_pad);
+            const int head = pb.head0 + g * p.group + rb * (R / p.w_pad);
             for (int hq = 0; hq < kQHalves && ok; ++hq) {
-              ok = mbar_wait_producer(bar(kBarQEmpty + hq), ((uint32_t)n_q & 1u) ^ 1u, abort_flag, kWaitCycles);
+              const int qb = q_bar(n_q, hq);
+              ok = mbar_wait_producer(bar(kBarQEmpty + qb), q_parity(n_q) ^ 1u, abort_flag, kWaitCycles);
               if (!ok) break;
-              mbar_expect_tx(bar(kBarQFull + hq), L::kQBytes / kQHalves);
+              mbar_expect_tx(bar(kBarQFull + qb), L::kQBytes / kQHalves);
               const int row = hq * (R / kQHalves);
               for (int c = 0; c < L::kSub; ++c)
-                tma_load_3d_hint(base + c * L::kQSub + row * 128, &p.map_q[pb.map], bar(kBarQFull + hq), c * 64,
+                tma_load_3d_hint(base + q_buf(n_q) + c * L::kQSub + row * 128, &p.map_q[pb.map], bar(kBarQFull + qb), c * 64,
                                  row % p.w_pad, head + row / p.w_pad, pol_keep);
-              q_loads = kQHalves * n_q + hq + 1;
+              ++q_uses[qb];
             }
             if (ok) ++n_q;
           }
@@ -681,8 +760,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
       }
       // every copy this thread issued must have landed before the CTA may exit (they have, unless
       // the CTA is aborting: an MMA consumed each of them)
-      for (int hq = 0; hq < kQHalves; ++hq)
-        if (q_loads > hq) mbar_drain(bar(kBarQFull + hq), (uint32_t)((q_loads - 1 - hq) / kQHalves) & 1u, abort_flag);
+      for (int qb = 0; qb < 2; ++qb)
+        if (q_uses[qb]) mbar_drain(bar(kBarQFull + qb), (q_uses[qb] - 1u) & 1u, abort_flag);
       for (int u = max(0, st - kStages); u < st; ++u)
         if (real >> (u % kStages) & 1u) mbar_drain(bar(kBarFull + u % kStages), (uint32_t)(u / kStages) & 1u, abort_flag);
     }
@@ -690,12 +769,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
       constexpr uint32_t idesc_ext = instr_desc(128, R);   // wide pass 1 has N = 256 = R as well
-      const uint64_t q_desc0 = smem_desc(base), k_desc0 = smem_desc(base + L::kKOff);
+      const uint64_t q_desc_at = smem_desc(base), k_desc0 = smem_desc(base + L::kKOff);
       const uint64_t ones_desc = smem_desc_k16(base + L::kOnesOff), ext_desc = smem_desc_k16(base + L::kExtOff);
       int st = 0, n_q = 0, n_ext = 0, u = 0;               // K stages, tasks with items, pass-2 tasks, accumulators so far
       bool ok = true;
       auto full = [&](int s) { return mbar_wait_producer(bar(kBarFull + s % kStages), (uint32_t)(s / kStages) & 1u, abort_flag, kWaitCycles); };
-      auto q_full = [&](int hq) { return mbar_wait_producer(bar(kBarQFull + hq), (uint32_t)n_q & 1u, abort_flag, kWaitCycles); };
+      auto q_full = [&](int hq) { return mbar_wait_producer(bar(kBarQFull + q_bar(n_q, hq)), q_parity(n_q), abort_flag, kWaitCycles); };
       auto acc_free = [&]() {
         const bool r = mbar_wait_producer(bar(kBarAccEmpty + u % S::kAcc), ((uint32_t)(u / S::kAcc) & 1u) ^ 1u, abort_flag, kWaitCycles);
         tc_fence_after();
@@ -704,15 +783,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
       for (int n = 0; ok; ++n) {
         const int k = n % kTaskRing;
         if (!mbar_wait_producer(bar(kBarTaskFull + k), (uint32_t)(n / kTaskRing) & 1u, abort_flag, kWaitCycles)) break;
-        volatile int* s = task_slot(k);
-        TcTask t{};
-        t.pass = s[0]; t.prob = s[1]; t.rb = s[3]; t.lo = s[4]; t.hi = s[5];
+        asm volatile("" ::: "memory");
+        const TcTask t = *task_slot(k);
+        asm volatile("" ::: "memory");
         mbar_arrive(bar(kBarTaskEmpty + k));
         if (t.pass == 0) break;
         const int items = items_of(t);
         if (items == 0) continue;
-        const int n_half = min(R, p.rows_pg - t.rb * R) > 128 ? 2 : 1;
-        const uint32_t idesc = idesc_ext | (p.prob[t.prob].negate ? 1u << 13 : 0u);
+        const int n_half = min(R, t.rows) > 128 ? 2 : 1;
+        const uint32_t idesc = idesc_ext | (t.negate ? 1u << 13 : 0u);
+        const uint64_t q_desc0 = q_desc_at + (uint64_t)(q_buf(n_q) >> 4);
         for (int it = 0; it < items && ok; ++it, st += 2) {
           // descriptors differ only in the start-address field (16-byte units, no carry out of it)
           if (!S::kNarrow && t.pass == 1) {
@@ -758,8 +838,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
                 // one more K-step adds -lse / c2 of every row: ones (key side) x three bf16 pieces of
                 // the value (row side)
                 if (it == 0 && half == 0 &&
-                    !(ok = mbar_wait_producer(bar(kBarExtFull), (uint32_t)n_ext & 1u, abort_flag, kWaitCycles))) break;
-                tc_mma_bf16(acc, ones_desc, ext_desc, idesc_ext, 1);
+                    !(ok = mbar_wait_producer(bar(kBarExtFull + (n_ext & 1)), (uint32_t)(n_ext >> 1) & 1u, abort_flag, kWaitCycles))) break;
+                tc_mma_bf16(acc, ones_desc, ext_desc + (uint64_t)((n_ext & 1) * (R * 32) >> 4), idesc_ext, 1);
               }
               tc_commit(bar(kBarEmpty + sg));              // K stage reusable once these MMAs have read it
               tc_commit(bar(kBarAccFull + u % S::kAcc));   // accumulator ready for the compute warps
@@ -770,13 +850,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         if (!ok) break;
         // hand Q back (wide pass 1 did so half by half; a block of one half never used the second)
         if (S::kNarrow || t.pass == 2) {
-          for (int hq = 0; hq < kQHalves; ++hq) tc_commit(bar(kBarQEmpty + hq));
+          for (int hq = 0; hq < kQHalves; ++hq) tc_commit(bar(kBarQEmpty + q_bar(n_q, hq)));
         } else if (n_half == 1) {
           if (!(ok = q_full(1))) break;
           tc_commit(bar(kBarQEmpty + 1));
         }
         ++n_q;
-        if (t.pass == 2) { tc_commit(bar(kBarExtEmpty)); ++n_ext; }
+        if (t.pass == 2) { tc_commit(bar(kBarExtEmpty + (n_ext & 1))); ++n_ext; }
       }
       // drain: all issued MMAs must retire before tensor memory is freed
       if (*mma_in_flight) {
@@ -791,11 +871,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     for (int n = 0; next_task(n, t); ++n) {
       if (p.hurry || t.pass != 2 || t.lo == t.hi) continue;
       int ok = 1;
-      const int unit = t.g * p.n_rb + t.rb;
       if (lane == 0) {
-        // the previous pass-2 task's MMAs have read the operand; this unit's statistics are merged
-        ok = mbar_wait_producer(bar(kBarExtEmpty), ((uint32_t)n_ext & 1u) ^ 1u, abort_flag, kWaitCycles) ? 1 : 0;
-        const int* flag = p.ctl + kCtlReady + t.prob * kQueueUnits + unit;
+        // the MMAs of the last task but one have read the operand; this unit's statistics are merged
+        ok = mbar_wait_producer(bar(kBarExtEmpty + (n_ext & 1)), ((uint32_t)(n_ext >> 1) & 1u) ^ 1u, abort_flag, kWaitCycles) ? 1 : 0;
+        const int* flag = p.ctl + kCtlReady + t.prob * kQueueUnits + t.unit;
         const long long t0 = clock64();
         while (ok) {
           int seen;
@@ -807,43 +886,38 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         }
       }
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
-      const size_t at0 = ((size_t)t.prob * p.n_units + unit) * kRowBlock;
-      const float inv_c2 = p.prob[t.prob].inv_c2;
+      const size_t at0 = (size_t)t.slot * kRowBlock;
 #pragma unroll
-      for (int i = 0; i < R / 32; ++i) put_lse(i * 32 + lane, __ldcg(p.nlse + at0 + i * 32 + lane), inv_c2);
+      for (int i = 0; i < R / 32; ++i) put_lse(n_ext & 1, i * 32 + lane, __ldcg(p.nlse + at0 + i * 32 + lane), t.inv_c2);
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(kBarExtFull));
+      if (lane == 0) mbar_arrive(bar(kBarExtFull + (n_ext & 1)));
       ++n_ext;
     }
   } else if (warp == 3) {
     // ---------------- row statistics of pass-1 tasks ----------------
-    const float2* part_s = reinterpret_cast<const float2*>(sm + L::kPartOff);
     int n_p1 = 0;
     TcTask t;
     for (int n = 0; next_task(n, t); ++n) {
       if (p.hurry || t.pass != 1) continue;
-      int ok = 1;
-      if (lane == 0) ok = mbar_wait_producer(bar(kBarPartFull), (uint32_t)n_p1 & 1u, abort_flag, kWaitCycles) ? 1 : 0;
+      int last = 0, ok = 1;
+      if (lane == 0) {
+        // the compute warps have stored the task's statistics
+        ok = mbar_wait_producer(bar(kBarPartFull), (uint32_t)n_p1 & 1u, abort_flag, kWaitCycles) ? 1 : 0;
+        if (ok) {
+          mbar_arrive(bar(kBarPartEmpty));
+          __threadfence();
+          last = atomicAdd(p.ctl + kCtlArrive + t.prob * kQueueUnits + t.unit, 1) == t.n_part - 1;
+        }
+      }
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
       ++n_p1;
-#pragma unroll 4
-      for (int r = lane; r < R; r += 32) {
-        __stcg(&p.part[(size_t)t.part * kRowBlock + r], fold_row<R>(part_s, r));
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(bar(kBarPartEmpty));
-      __threadfence();
-      __syncwarp();
-      const int unit = t.g * p.n_rb + t.rb;
-      int last = 0;
-      if (lane == 0) last = atomicAdd(p.ctl + kCtlArrive + t.prob * kQueueUnits + unit, 1) == t.n_part - 1;
       if (!__shfl_sync(0xffffffffu, last, 0)) continue;
       __threadfence();
       // this task completes the unit: merge its partials into each row's log-sum-exp and entropy
-      const size_t at0 = ((size_t)t.prob * p.n_units + unit) * kRowBlock;
-      merge_unit<R>(p.part + (size_t)t.part0 * kRowBlock, t.n_part, lane, [&](int r, float nlse, float ent) {
-        const bool row = is_row(t.rb * R + r);
+      const size_t at0 = (size_t)t.slot * kRowBlock;
+      merge_unit<R>(p.part + (size_t)t.part0 * R, t.n_part, lane, [&](int r, float nlse, float ent) {
+        const bool row = is_row(t.row0 + r);
         __stcg(p.nlse + at0 + r, row ? nlse : -INFINITY);
         p.row_ent[at0 + r] = row ? ent : 0.f;
       });
@@ -851,7 +925,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
       __threadfence();
       __syncwarp();
       if (lane == 0)
-        asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p.ctl + kCtlReady + t.prob * kQueueUnits + unit), "r"(1) : "memory");
+        asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(p.ctl + kCtlReady + t.prob * kQueueUnits + t.unit), "r"(1) : "memory");
     }
   } else {
     // ---------------- compute warps ----------------
@@ -859,16 +933,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     const int sub = (warp - kHelperWarps) >> 2;   // which quarter of an accumulator's columns (or of the tiles) it takes
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
     float2* part_s = reinterpret_cast<float2*>(sm + L::kPartOff);
-    int u = 0, n_p1 = 0, n_sync = 0, n_ext = 0;
+    int u = 0, n_p1 = 0, n_ext = 0;
     // Every lane polls: a barrier that has already flipped costs one test, no divergence, no broadcast
     // (with four chunks of arithmetic per accumulator and scheduler each instruction here shows).
-    auto acc_full = [&]() {
+    auto acc_full_at = [&](int u) {
       const uint32_t b = bar(kBarAccFull + u % S::kAcc), parity = (uint32_t)(u / S::kAcc) & 1u;
       bool ok = mbar_try(b, parity);
       if (!__all_sync(0xffffffffu, ok)) ok = __all_sync(0xffffffffu, mbar_wait(b, parity, abort_flag)) != 0;
       tc_fence_after();
       return ok;
     };
+    auto acc_full = [&]() { return acc_full_at(u); };
     // all of this warp's loads of the accumulator have landed: one arrival per warp frees it
     auto acc_release = [&]() {
       tc_fence_before();
@@ -876,55 +951,51 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
       if (lane == 0) mbar_arrive(bar(kBarAccEmpty + u % S::kAcc));
     };
     auto acc_addr = [&]() { return tmem + lane_base + (uint32_t)((u % S::kAcc) * S::kAccCols); };
-    // the fold warp has read the previous task's statistics
-    auto part_free = [&]() {
-      int ok = 1;
-      if (lane == 0) ok = mbar_wait(bar(kBarPartEmpty), ((uint32_t)n_p1 & 1u) ^ 1u, abort_flag) ? 1 : 0;
-      return __shfl_sync(0xffffffffu, ok, 0) != 0;
-    };
-    // Bounded barrier of the compute warps.
-    auto sync_all = [&]() {
+    const int ct = (int)threadIdx.x - kHelperWarps * 32;
+    // Statistics of a pass-1 task: the four warps that hold parts of the same rows (wide: one lane quarter, four
+    // column groups; narrow: one set of rows, four lane quarters) leave them in shared memory, meet, and one or
+    // two of them fold and store them.  Two buffers: whoever writes one again has met the readers of
+    // the other since.  The helper that counts the task's arrival works beside the next task.
+    auto part_buf = [&](int k) { return part_s + ((n_p1 & 1) * 3 + k) * R; };
+    auto fold_meet = [&](int set) {
       __syncwarp();
-      if (lane == 0) mbar_arrive(bar(kBarSync));
-      const bool ok = mbar_wait(bar(kBarSync), (uint32_t)n_sync++ & 1u, abort_flag);
+      if (lane == 0) mbar_arrive(bar(kBarFold + set));
+      const bool ok = mbar_wait(bar(kBarFold + set), (uint32_t)n_p1 & 1u, abort_flag);
       return __all_sync(0xffffffffu, ok) != 0;
     };
-    const int ct = (int)threadIdx.x - kHelperWarps * 32;
-    // The task's statistics are in shared memory: the fold warp takes them from here, or, in a hurry,
-    // the compute warps themselves.
-    auto part_done = [&](const TcTask& t) {
-      if (!p.hurry) {
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(kBarPartFull));
-        ++n_p1;
-        return true;
+    auto part_stored = [&](const TcTask& t) {
+      __syncwarp();
+      bool ok = true;
+      if (lane == 0) {
+        if (p.hurry) {                                     // each storing warp counts for itself
+          __threadfence();
+          atomicAdd(p.ctl + kCtlArrive + t.prob * kQueueUnits + t.unit, 1);
+        } else {                                           // the helper has seen the previous task's
+          ok = mbar_wait(bar(kBarPartEmpty), ((uint32_t)n_p1 & 1u) ^ 1u, abort_flag);
+          if (ok) mbar_arrive(bar(kBarPartFull));
+        }
       }
-      if (!sync_all()) return false;
-      if (ct < R) __stcg(&p.part[(size_t)t.part * kRowBlock + ct], fold_row<R>(part_s, ct));
-      __threadfence();
-      if (!sync_all()) return false;
-      if (ct == 0) atomicAdd(p.ctl + kCtlArrive + t.prob * kQueueUnits + t.g * p.n_rb + t.rb, 1);
-      return true;
+      return __shfl_sync(0xffffffffu, ok, 0);
     };
-    // In a hurry: the compute warps wait for the unit's partials and merge them, a thread per row, into the
-    // extra K-step's operand (the task that holds key 0 leaves the entropies).
+    // In a hurry: R / 32 of the compute warps wait for the unit's partials and merge them, a thread per row, into
+    // the extra K-step's operand (the task that holds key 0 leaves the entropies).
     auto merge_now = [&](const TcTask& t) {
-      const int unit = t.g * p.n_rb + t.rb;
-      if (ct == 0) {
-        bool ok = mbar_wait(bar(kBarExtEmpty), ((uint32_t)n_ext & 1u) ^ 1u, abort_flag);
-        const int* count = p.ctl + kCtlArrive + t.prob * kQueueUnits + unit;
+      bool ok = true;
+      if (lane == 0 && ct < R) {
+        ok = mbar_wait(bar(kBarExtEmpty + (n_ext & 1)), ((uint32_t)(n_ext >> 1) & 1u) ^ 1u, abort_flag);
+        const int* count = p.ctl + kCtlArrive + t.prob * kQueueUnits + t.unit;
         const long long t0 = clock64();
         while (ok) {
           int seen;
           asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
-          if (seen >= t.n_part) break;
+          if (seen >= t.n_part * S::kFoldWarps) break;
           if (*abort_flag) ok = false;
           else if ((unsigned long long)(clock64() - t0) > kWaitCycles) { *abort_flag = 1; ok = false; }
         }
       }
-      if (!sync_all() || *abort_flag) return false;
+      if (!__shfl_sync(0xffffffffu, ok, 0)) return false;
       if (ct < R) {
-        const float2* part = p.part + (size_t)t.part0 * kRowBlock + ct;
+        const float2* part = p.part + (size_t)t.part0 * R + ct;
         float M = -INFINITY, W = 0.f, X = 0.f;
         // all partials of a row in one round of loads (148 SMs, 8 units: 18 or 19), merged in the helper
         // warp's groups: the bits must not depend on who merges
@@ -934,29 +1005,30 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
 #pragma unroll
           for (int b = 0; b < kRounds * kMergeGroup; ++b)
             pv[b / kMergeGroup][b % kMergeGroup] =
-                s0 + b < t.n_part ? __ldcg(part + (size_t)(s0 + b) * kRowBlock) : make_float2(-INFINITY, 0.f);
+                s0 + b < t.n_part ? __ldcg(part + (size_t)(s0 + b) * R) : make_float2(-INFINITY, 0.f);
 #pragma unroll
           for (int k = 0; k < kRounds; ++k) merge_partials(M, W, X, pv[k]);
         }
-        const bool row = is_row(t.rb * R + ct) && W > 0.f;
+        const bool row = is_row(t.row0 + ct) && W > 0.f;
         const float lz = __log2f(W);
-        put_lse(ct, row ? -(M + lz) : -INFINITY, p.prob[t.prob].inv_c2);
-        if (t.lo == 0) p.row_ent[((size_t)t.prob * p.n_units + unit) * kRowBlock + ct] = row ? kLn2 * (lz + X / W) : 0.f;
+        put_lse(n_ext & 1, ct, row ? -(M + lz) : -INFINITY, t.inv_c2);
+        if (t.lo == 0) p.row_ent[(size_t)t.slot * kRowBlock + ct] = row ? kLn2 * (lz + X / W) : 0.f;
       } else if (t.lo == 0 && ct < kRowBlock) {
-        p.row_ent[((size_t)t.prob * p.n_units + unit) * kRowBlock + ct] = 0.f;   // rows of the block the unit does not have
+        p.row_ent[(size_t)t.slot * kRowBlock + ct] = 0.f;   // rows of the block the unit does not have
       }
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
-      if (!sync_all()) return false;
-      if (ct == 0) mbar_arrive(bar(kBarExtFull));
+      if (ct < R) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // visible to the tensor core
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kBarExtFull + (n_ext & 1)));
+      }
       ++n_ext;
       return true;
     };
     TcTask t;
     bool live = true;
     for (int n = 0; live && next_task(n, t); ++n) {
-      const TcProblem& pb = p.prob[t.prob];
-      const int n_keys = pb.n_keys, items = items_of(t);
-      const float c2 = pb.c2;
+      const int n_keys = t.n_keys, items = items_of(t);
+      const float c2 = t.c2;
       const uint64_t c22 = pack2(c2, c2);
       const int last_open_key = n_keys - p.window;         // the last key every window row sees
       // a tile is "plain" when all of its keys are visible to every window row (j0 + 127 <= N - w);
@@ -969,7 +1041,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         float v[32] = {};
         RowStat rs[2] = {{-INFINITY, 0.f, 0.f}, {-INFINITY, 0.f, 0.f}};
         const int row_lo = quarter * 32 + lane;
-        const int rows_here = min(R, p.rows_pg - t.rb * R), n_half = rows_here > 128 ? 2 : 1;
+        const int rows_here = min(R, t.rows), n_half = rows_here > 128 ? 2 : 1;
         auto chunk = [&](RowStat& r, int jb, bool first, int hf) {
           // of the last pair only the chunks that hold window keys (or lie beyond the sequence) are masked
           bool careful = jb + 31 > last_open_key;
@@ -1009,72 +1081,132 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
           }
           ++u;
         }
-        if (!live || (!p.hurry && !part_free())) break;
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) part_s[sub * R + hf * 128 + row_lo] = stat_partial(rs[hf]);
-        if (!part_done(t)) break;
+        if (!live) break;
+        // column group 0 folds the rows of the first half, column group 1 those of the second
+        const float2 part0 = stat_partial(rs[0]), part1 = stat_partial(rs[1]);
+        if (sub != 0) part_buf(sub - 1)[row_lo] = part0;
+        if (sub != 1) part_buf(sub == 0 ? 0 : sub - 1)[128 + row_lo] = part1;
+        if (!fold_meet(quarter)) break;
+        if (sub < 2) {
+          const int r = sub * 128 + row_lo;
+          __stcg(&p.part[(size_t)t.part * R + r], fold_row(part_buf(0) + r, R, sub == 0 ? part0 : part1, sub));
+          if (!part_stored(t)) break;
+        }
+        ++n_p1;
       } else if (t.pass == 1) {
         if constexpr (S::kNarrow) {
-          // Lane = key, RT rows per thread; every lane keeps its own reference per row.
-          constexpr int RT = R / 4;
-          float v[RT], ref[RT], Z[RT], U[RT];
+          // Lane = key, RT rows per thread, T tiles at a time: their waits and loads overlap (a tile by
+          // itself left 500 clocks of latency bare).  A row's reference is the warp's, so that the lanes'
+          // sums add up without rescaling and, scattered over the lanes, in 2 RT shuffles: with a
+          // reference per lane the end of a task took 4500 clocks.  28 layers of 8192 keys, window 8:
+          // 281 us before, 179 now; of 32768 keys 21.2 us a layer before, 20.8 now (the reading of K).
+          constexpr int RT = R / 4, T = RT == 8 ? 4 : 1, kLanes = 32 / RT;
+          float v[T * RT];
+          const float masked = fmaxf(kMasked * t.inv_c2, kMaskedAcc);   // times c2: finite, and 2^x flushes to 0
+          uint64_t nref2[RT / 2], Z2[RT / 2], U2[RT / 2];  // pairs of rows: -reference, Z, U
 #pragma unroll
-          for (int e = 0; e < RT; ++e) ref[e] = Z[e] = U[e] = 0.f;
-          bool first = true;
-          for (int tile = t.lo; tile < t.hi; ++tile) {
-            if (!acc_full()) { live = false; break; }
-            tmem_ld(acc_addr() + sub * RT, v);
-            acc_release();
-            ++u;
-            const int over = tile * kKeyTile + quarter * 32 + lane - last_open_key;   // rows i < over do not see this key
-            const bool plain = tile < first_tail_tile;
+          for (int e = 0; e < RT / 2; ++e) nref2[e] = Z2[e] = U2[e] = 0;
+          for (int tile0 = t.lo; tile0 < t.hi; tile0 += T) {
+            const int n_here = min(T, t.hi - tile0);
+            for (int k = 0; k < n_here; ++k) live = live && acc_full_at(u + k);
+            if (!live) break;
+#pragma unroll
+            for (int k = 0; k < T; ++k)
+              tmem_ld_issue<RT>(tmem + lane_base + (uint32_t)(((u + min(k, n_here - 1)) % S::kAcc) * S::kAccCols) + sub * RT, v + k * RT);
+            tmem_ld_wait(v);
+            tc_fence_before();
+            __syncwarp();
+            if (lane < n_here) mbar_arrive(bar(kBarAccEmpty + (u + lane) % S::kAcc));
+            u += n_here;
+            const bool plain = tile0 + n_here <= first_tail_tile && n_here == T;
+            if (!plain) {
+#pragma unroll
+              for (int k = 0; k < T; ++k) {
+                const int over = k < n_here ? (tile0 + k) * kKeyTile + quarter * 32 + lane - last_open_key : 0x7fffffff;
+#pragma unroll
+                for (int e = 0; e < RT; ++e)         // rows i < over do not see this key
+                  if (((sub * RT + e) & (p.w_pad - 1)) < over) v[k * RT + e] = masked;
+              }
+            }
+            // largest logit of rows 2 e and 2 e + 1 over the warp's keys of these tiles
+            auto row_max = [&](int e, float& m0, float& m1) {
+              m0 = v[2 * e];
+              m1 = v[2 * e + 1];
+#pragma unroll
+              for (int k = 1; k < T; ++k) {
+                m0 = fmaxf(m0, v[k * RT + 2 * e]);
+                m1 = fmaxf(m1, v[k * RT + 2 * e + 1]);
+              }
+              m0 = warp_max(m0) * c2;
+              m1 = warp_max(m1) * c2;
+            };
+            if (tile0 == t.lo) {                           // the references: where a task starts, unless masked
+#pragma unroll
+              for (int e = 0; e < RT / 2; ++e) {
+                float m0, m1;
+                row_max(e, m0, m1);
+                nref2[e] = pack2(m0 > 0.5f * masked * c2 ? -m0 : 0.f, m1 > 0.5f * masked * c2 ? -m1 : 0.f);
+              }
+            }
             float top = -INFINITY;
 #pragma unroll
-            for (int e = 0; e < RT; ++e) {
-              v[e] *= c2;
-              if (!plain && ((sub * RT + e) & (p.w_pad - 1)) < over) v[e] = kMasked;
-              if (first && v[e] > 0.5f * kMasked) ref[e] = v[e];
-              top = fmaxf(top, v[e] - ref[e]);
+            for (int i = 0; i < T * RT / 2; ++i) {
+              const uint64_t x2 = fma2(pack2(v[2 * i], v[2 * i + 1]), c22, nref2[i % (RT / 2)]);
+              float x0, x1;
+              unpack2(x2, x0, x1);
+              top = fmaxf(top, fmaxf(x0, x1));
             }
-            first = false;
-            if (__any_sync(0xffffffffu, top > 60.f)) {
+            if (__any_sync(0xffffffffu, top > 60.f)) {     // far above the references: they move up
 #pragma unroll
-              for (int e = 0; e < RT; ++e)
-                if (v[e] > ref[e]) {
-                  const float dm = ref[e] - v[e], f = fast_exp2(dm);
-                  U[e] = f * fmaf(dm, Z[e], U[e]);
-                  Z[e] *= f;
-                  ref[e] = v[e];
-                }
+              for (int e = 0; e < RT / 2; ++e) {
+                float m[2], r[2], z[2], w[2];
+                row_max(e, m[0], m[1]);
+                unpack2(nref2[e], r[0], r[1]);
+                unpack2(Z2[e], z[0], z[1]);
+                unpack2(U2[e], w[0], w[1]);
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                  if (m[h] > -r[h]) {
+                    const float dm = -r[h] - m[h], f = fast_exp2(dm);
+                    w[h] = f * fmaf(dm, z[h], w[h]);
+                    z[h] *= f;
+                    r[h] = -m[h];
+                  }
+                nref2[e] = pack2(r[0], r[1]);
+                Z2[e] = pack2(z[0], z[1]);
+                U2[e] = pack2(w[0], w[1]);
+              }
             }
 #pragma unroll
-            for (int e = 0; e < RT; ++e) {
-              const float x = v[e] - ref[e], pe = fast_exp2(x);
-              Z[e] += pe;
-              U[e] = fmaf(pe, x, U[e]);
+            for (int i = 0; i < T * RT / 2; ++i) {
+              const uint64_t x2 = fma2(pack2(v[2 * i], v[2 * i + 1]), c22, nref2[i % (RT / 2)]), p2 = exp2_sfu2(x2);
+              Z2[i % (RT / 2)] = add2(Z2[i % (RT / 2)], p2);
+              U2[i % (RT / 2)] = fma2(p2, x2, U2[i % (RT / 2)]);
             }
           }
-          if (!live || (!p.hurry && !part_free())) break;
+          if (!live) break;
+          float ref[RT], Z[RT], U[RT];
 #pragma unroll
-          for (int e = 0; e < RT; ++e) {
-            float M = Z[e] > 0.f ? ref[e] : -INFINITY;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-            const float dm = Z[e] > 0.f ? ref[e] - M : 0.f, f = fast_exp2(dm);
-            float Ze = f * Z[e], Ue = f * fmaf(dm, Z[e], U[e]);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-              Ze += __shfl_xor_sync(0xffffffffu, Ze, o);
-              Ue += __shfl_xor_sync(0xffffffffu, Ue, o);
-            }
-            if (lane == e) part_s[quarter * R + sub * RT + e] = stat_partial(RowStat{M, Ze, Ue});
+          for (int e = 0; e < RT / 2; ++e) {
+            unpack2(nref2[e], ref[2 * e], ref[2 * e + 1]);
+            unpack2(Z2[e], Z[2 * e], Z[2 * e + 1]);
+            unpack2(U2[e], U[2 * e], U[2 * e + 1]);
           }
-          if (!part_done(t)) break;
+          const float ref_l = -lane_element(ref, lane), Z_l = warp_sum_scatter(Z, lane), U_l = warp_sum_scatter(U, lane);
+          const float2 part = stat_partial(RowStat{Z_l > 0.f ? ref_l : -INFINITY, Z_l, U_l});
+          const int r = sub * RT + lane / kLanes;
+          if (quarter != 0 && lane % kLanes == 0) part_buf(quarter - 1)[r] = part;
+          if (!fold_meet(sub)) break;
+          if (quarter == 0) {
+            if (lane % kLanes == 0) __stcg(&p.part[(size_t)t.part * R + r], fold_row(part_buf(0) + r, R, part, 0));
+            if (!part_stored(t)) break;
+          }
+          ++n_p1;
         }
       } else {
         // Pass 2: this thread owns key (tile * 128 + quarter * 32 + lane); x = c2 * accumulator.
         if (p.hurry && t.hi > t.lo && !merge_now(t)) break;
-        const float v_min = pb.v_min, inv_w = 1.0f / (float)p.window;
+        const float v_min = t.v_min, inv_w = 1.0f / (float)p.window;
         // Columns (rows of the block) this warp sums: a quarter of them on every tile, or, where a
         // head spans more, the head's rows on every second or fourth tile, so that a head's column
         // sum never spans two warps.  Narrow blocks: all rows on every fourth tile.
@@ -1084,9 +1216,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         const int turn = S::kNarrow || kW == 256 ? 3 : kW == 128 ? 1 : 0;
         const int col0 = S::kNarrow || kW == 256 ? 0 : kW == 128 ? (sub & 1) * 128 : sub * 64;
         const int my_turn = kW == 128 && !S::kNarrow ? sub >> 1 : sub;
-        const int row0 = t.rb * R + col0;                   // first score row (within the group) of this warp
-        const bool warp_active = row0 < p.rows_pg;
-        const int h0 = t.g * p.group + row0 / p.w_pad, h_end = (t.g + 1) * p.group;
+        const bool warp_active = col0 < t.rows;
+        const int h0 = (t.row0 + col0) >> p.w_shift, h_end = t.group;   // heads within the KV group
         for (int i = 0; i < t.hi - t.lo; ++i) {
           if (!acc_full()) { live = false; break; }
           const int tile = t.hi - 1 - i;
@@ -1110,7 +1241,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
                 if (((col0 + c + e) & (p.w_pad - 1)) < i_min) v[e] = kMaskedAcc;
             }
             auto finish_head = [&]() {
-              if (head < h_end && j < n_keys) pb.cols[(size_t)head * p.col_stride + j] = tot * inv_w;
+              if (head < h_end && j < n_keys) t.cols[(size_t)head * p.col_stride + j] = tot * inv_w;
               ++head;
               tot = 0.f;
             };

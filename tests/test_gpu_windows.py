@@ -57,11 +57,14 @@ def test_unusual_scales(cuda_device, w, scale):
     score(cuda_device, 32, 8, 128, w, 3000, scale)
 
 
-def test_more_layers_than_one_launch_takes(cuda_device):
-    """structkv_score_layers beyond the problems one launch holds, with a sequence short enough for the
-    first pass to run several layers ahead: the bits of the layer-by-layer calls."""
+@pytest.mark.parametrize("L,H,Hkv,d,w,N", [
+    (37, 8, 2, 64, 32, 700), (9, 32, 8, 128, 8, 1281), (5, 8, 2, 128, 16, 24577), (40, 6, 2, 64, 5, 513),
+    (4, 4, 4, 64, 64, 131), (3, 32, 8, 128, 64, 2000),
+])
+def test_layers_of_one_launch(cuda_device, L, H, Hkv, d, w, N):
+    """structkv_score_layers, also beyond the problems one launch holds and with sequences short enough for
+    the first pass to run several layers ahead: the bits of the layer-by-layer calls."""
     from paper_2604_06746_b200 import binding
-    L, H, Hkv, d, w, N = 37, 8, 2, 64, 32, 700
     g = torch.Generator(device=cuda_device)
     g.manual_seed(3)
     qs = [torch.randn((H, w, d), generator=g, device=cuda_device).bfloat16() for _ in range(L)]
