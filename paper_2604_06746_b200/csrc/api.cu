@@ -342,12 +342,8 @@ static structkv_status score_layers(structkv_ctx* ctx, int n_layers, const void*
   const ScoreCall a{n_layers, q_windows, ks, scales, nullptr, k_stride_head, k_stride_token, n_keys, head_cols_out,
                  head_cols_layer_stride, n_keys, lw.row_part, lw.nlse, lw.row_ent};
   if ((use_tc ? launch_score_tc(c, a, st) : launch_score_simt(c, a, st)) != cudaSuccess) return STRUCTKV_ERR_CUDA;
-  const bool ride = with_stats && head_stats_ride_along(c, n_layers, n_keys);
   if (launch_finish_layers(c, head_cols_out, head_cols_layer_stride, n_keys, n_keys, n_layers, lambda, s_out, s_layer_stride,
-                           c_inout, lw.row_ent, ride, metrics_out, st, c_from_zero) != cudaSuccess)
-    return STRUCTKV_ERR_CUDA;
-  if (with_stats && !ride &&
-      launch_head_stats_batch(c, head_cols_out, head_cols_layer_stride, n_keys, n_layers, n_keys, metrics_out, st) != cudaSuccess)
+                           c_inout, lw.row_ent, with_stats, metrics_out, st, c_from_zero) != cudaSuccess)
     return STRUCTKV_ERR_CUDA;
   return STRUCTKV_OK;
 }

@@ -96,8 +96,6 @@ cudaError_t launch_finish_layers(const Ctx& ctx, const float* cols, long long la
                                  int n_layers, float lambda, float* s_out, long long s_stride, float* c_inout,
                                  const float* row_ent, bool with_head_stats, float* metrics, cudaStream_t st,
                                  bool c_from_zero = false);
-// whether Eq. 5-6 of so many vectors of n entries are best taken in that launch
-bool head_stats_ride_along(const Ctx& ctx, int n_layers, int n);
 // The same for the sequences of a packed batch (sequence b at column cu_seqlens[b] of cols, s_out and c_inout).
 cudaError_t launch_finish_packed(const Ctx& ctx, const float* cols, long long col_stride, const int* cu_seqlens, int batch,
                                  float lambda, float* s_out, float* c_inout, const float* row_ent, float* head_part,

@@ -20,27 +20,23 @@ namespace cg = cooperative_groups;
 constexpr int kRxThreads = 1024;
 constexpr int kRxLevels = 4;
 
-// COPIES of a bin; BUFFERS: two alternate from level to level, one costs a barrier more; THREADS of a CTA.
-template <int CL_, int COPIES_ = 32, int BUFFERS_ = 2, int THREADS_ = kRxThreads>
+template <int CL>
 struct RadixShared {
-  static constexpr int CL = CL_, COPIES = COPIES_, BUFFERS = BUFFERS_, THREADS = THREADS_;
-  unsigned hist[BUFFERS][256 * COPIES];
+  unsigned hist[2][256 * 32];          // levels alternate
   unsigned cnt[2][CL][256];            // counts of every CTA of the cluster
   unsigned mine[256];                  // this CTA's, before the exchange
-  unsigned scratch[THREADS + 64];      // block reductions, output offsets
+  unsigned scratch[2 * kRxThreads];    // block reductions, output offsets
   float red[4][33];
 };
-using RadixResident = RadixShared<1, 16, 1>;      // leaves shared memory for the vector itself
-using RadixSmall = RadixShared<1, 16, 1, 256>;    // short vectors, many of them: several CTAs on an SM
 
-template <typename S>
-__device__ __forceinline__ void radix_clear(S& s, int buf) {
-  uint4* h = reinterpret_cast<uint4*>(s.hist[buf % S::BUFFERS]);
-  for (int i = threadIdx.x; i < 256 * S::COPIES / 4; i += S::THREADS) h[i] = make_uint4(0u, 0u, 0u, 0u);
+template <int CL>
+__device__ __forceinline__ void radix_clear(RadixShared<CL>& s, int buf) {
+  uint4* h = reinterpret_cast<uint4*>(s.hist[buf]);
+  for (int i = threadIdx.x; i < 256 * 32 / 4; i += kRxThreads) h[i] = make_uint4(0u, 0u, 0u, 0u);
 }
-template <typename S>
-__device__ __forceinline__ void radix_count(S& s, int buf, unsigned digit) {
-  atomicAdd(&s.hist[buf % S::BUFFERS][digit * S::COPIES + (threadIdx.x & (S::COPIES - 1))], 1u);
+template <int CL>
+__device__ __forceinline__ void radix_count(RadixShared<CL>& s, int buf, unsigned digit) {
+  atomicAdd(&s.hist[buf][digit * 32 + (threadIdx.x & 31)], 1u);
 }
 template <int CL>
 __device__ __forceinline__ void cluster_barrier() {
@@ -48,30 +44,19 @@ __device__ __forceinline__ void cluster_barrier() {
   else __syncthreads();
 }
 // After a level's counting (no barrier needed before): finds the digit that holds the `remaining`-th
-// largest key, the rank still wanted inside it and how many keys share it.  The histogram of the next
-// level is clear when it returns.
-template <typename S>
-__device__ __forceinline__ void radix_pick(S& s, int buf, unsigned& remaining, unsigned& digit, unsigned& in_digit) {
-  constexpr int CL = S::CL, COPIES = S::COPIES;
+// largest key, the rank still wanted inside it and how many keys share it.  The other histogram
+// buffer is clear when it returns, ready for the next level.
+template <int CL>
+__device__ __forceinline__ void radix_pick(RadixShared<CL>& s, int buf, unsigned& remaining, unsigned& digit, unsigned& in_digit) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned* const h = s.hist[buf % S::BUFFERS];
-  unsigned* const to_cnt = CL > 1 ? s.mine : s.cnt[buf][0];
   __syncthreads();
-  constexpr int kAt = 32 / COPIES;                   // bins a warp sums side by side
-  constexpr int kBins = 256 / (S::THREADS / 32);     // bins of a warp
-#pragma unroll 8
-  for (int b = 0; b < kBins; b += kAt) {
-    unsigned c = h[(warp * kBins + b) * COPIES + lane];
-    if (COPIES == 32) {
-      c = __reduce_add_sync(0xffffffffu, c);
-    } else {
 #pragma unroll
-      for (int o = COPIES / 2; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    if (lane % COPIES == 0) to_cnt[warp * kBins + b + lane / COPIES] = c;
+  for (int b = 0; b < 8; ++b) {
+    const int bin = warp * 8 + b;
+    const unsigned c = __reduce_add_sync(0xffffffffu, s.hist[buf][bin * 32 + lane]);
+    if (lane == 0) (CL > 1 ? s.mine : s.cnt[buf][0])[bin] = c;
   }
-  if (S::BUFFERS == 1) __syncthreads();
-  radix_clear(s, buf + 1);
+  radix_clear(s, buf ^ 1);
   __syncthreads();
   if (CL > 1) {
     const int rank = (int)cg::this_cluster().block_rank();
@@ -117,28 +102,6 @@ __device__ __forceinline__ void radix_pick(S& s, int buf, unsigned& remaining, u
   remaining = __shfl_sync(0xffffffffu, rem, src);
 }
 
-// Copies x[0 .. n) to shared memory (dst 16-byte aligned), 16 bytes at a time.
-__device__ __forceinline__ void stage_vector(float* dst, const float* __restrict__ x, int n) {
-  const int head = min(n, (int)((4 - ((uintptr_t)x >> 2 & 3)) & 3)), n4 = (n - head) / 4;
-  if ((int)threadIdx.x < head) dst[threadIdx.x] = x[threadIdx.x];
-  const float4* x4 = reinterpret_cast<const float4*>(x + head);
-#pragma unroll 4
-  for (int i = threadIdx.x; i < n4; i += kRxThreads) {
-    const float4 v = x4[i];
-    if (head == 0) {
-      reinterpret_cast<float4*>(dst)[i] = v;
-    } else {
-      float* d = dst + head + 4 * i;
-      d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
-    }
-  }
-  for (int i = head + 4 * n4 + threadIdx.x; i < n; i += kRxThreads) dst[i] = x[i];
-}
-// The longest vector one CTA holds in shared memory beside a RadixResident.
-constexpr int kResidentMax = 50 * 1024;
-constexpr int kResidentBytes = (int)(sizeof(RadixResident) + 15) / 16 * 16 + kResidentMax * 4;
-static_assert(kResidentBytes + 1024 <= 227 * 1024, "shared memory of one CTA");
-
 // Larger float -> larger unsigned; -0 is folded onto +0.
 __device__ __forceinline__ unsigned order_key(float v) {
   const unsigned b = __float_as_uint(v + 0.0f);
@@ -146,11 +109,11 @@ __device__ __forceinline__ unsigned order_key(float v) {
 }
 
 // Kernel launch with a cluster of CL CTAs and early start.
-template <int CL, int THREADS = kRxThreads, typename... KArgs, typename... Args>
+template <int CL, typename... KArgs, typename... Args>
 inline cudaError_t launch_cluster(void (*kernel)(KArgs...), int grid, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(THREADS);
+  cfg.blockDim = dim3(kRxThreads);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];

@@ -1,19 +1,14 @@
 // Small deterministic reductions after the scorers: the sum
 // over heads with the centrality update, per-head sparsity / variance with the layer's metrics, and
 // the closed-form centrality re-accumulation.
-#include <algorithm>
-#include <atomic>
-#include <type_traits>
-
-#include "radix.cuh"
+#include "common.cuh"
 
 namespace skv {
 namespace {
 
 // ---- what follows the scorer passes of a layer, of several layers or of a packed batch ----------
-// One launch: CTAs of clusters first (one cluster per (problem, head) vector, Eq. 5-6), then blocks
-// that sum 128 x VEC keys over the heads (Eq. 2) and carry the centrality (Eq. 3).  Every sum has a
-// fixed order.
+// One launch: one CTA per (problem, head) vector first (Eq. 5-6), then blocks that sum 128 x VEC keys over
+// the heads (Eq. 2) and carry the centrality (Eq. 3).  Every sum has a fixed order.
 struct FinishArgs {
   const float* cols;                   // problem p, head h, key j at cols + p * layer_stride + h * col_stride + j
   long long layer_stride, col_stride;
@@ -34,26 +29,12 @@ struct FinishArgs {
   int cu[kMaxBatch + 1];
 };
 constexpr int kSumLanes = 128, kSumGroups = 8;
+constexpr int kEntThreads = 1024;      // partial sums of a problem's entropy
 
 struct Problem { const float* cols; float* s; int n; };
 __device__ __forceinline__ Problem problem_of(const FinishArgs& a, int p) {
   if (a.packed) return {a.cols + a.cu[p], a.s_out + a.cu[p], a.cu[p + 1] - a.cu[p]};
   return {a.cols + (size_t)p * a.layer_stride, a.s_out + (size_t)p * a.s_stride, a.n};
-}
-
-// Sum of v over the block, in every thread of warp 0 (fixed order).
-__device__ __forceinline__ float block_total(float v, float* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  if (warp == 0) {
-    v = lane < (int)(blockDim.x >> 5) ? red[lane] : 0.f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  }
-  return v;
 }
 
 template <int VEC> struct Keys;
@@ -131,9 +112,9 @@ __device__ __forceinline__ void sum_block(const FinishArgs& a, SumShared<VEC>& s
   // the problem's entropy (Eq. 4); rows that do not exist hold 0
   float ent = 0.f;
   // (the same partial sums whatever the block size: thread t of 1024 takes rows t, t + 1024, ...)
-  for (int t = threadIdx.x; t < kRxThreads; t += THREADS) {
+  for (int t = threadIdx.x; t < kEntThreads; t += THREADS) {
     float e = 0.f;
-    for (int r = t; r < a.rows_pad; r += kRxThreads) e += a.row_ent[(size_t)p * a.rows_pad + r];
+    for (int r = t; r < a.rows_pad; r += kEntThreads) e += a.row_ent[(size_t)p * a.rows_pad + r];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
     if ((t & 31) == 0) red[t >> 5] = e;
@@ -150,99 +131,19 @@ __device__ __forceinline__ void sum_block(const FinishArgs& a, SumShared<VEC>& s
   }
 }
 
-// Eq. 5 and 6 of one (problem, head) vector, by a cluster or by one CTA: the sum of squared deviations
-// from 1/n (the pooled vector sums to 1, so 1/n is its mean; summing deviations instead of squares
-// keeps near-uniform attention from cancelling) and the mass of the floor(n / 10) largest entries.
-// Three radix levels give the threshold to 24 bits; of the entries that share them, the ones still
-// wanted count with their average; a level that settles it is the last.  All entries are >= 0: the
-// order of the bit patterns is theirs.
-template <int ITEMS, typename S>
-__device__ __forceinline__ void stats_cta(const FinishArgs& a, S& s, float* vec_s, int vec) {
-  constexpr int CL = S::CL;
-  constexpr bool RESIDENT = std::is_same_v<S, RadixResident>;
-  const int tid = threadIdx.x;
-  const int rank = CL > 1 ? (int)cg::this_cluster().block_rank() : 0;
-  const int p = vec / a.H;
-  const Problem pb = problem_of(a, p);
-  const float* x = pb.cols + (size_t)(vec - p * a.H) * a.col_stride;
-  const int n = pb.n, per = (n + CL - 1) / CL, lo = min(n, rank * per), hi = min(n, lo + per);
-  constexpr int kChunk = S::THREADS * ITEMS;
-  const int chunks = (per + kChunk - 1) / kChunk;
-  unsigned key[ITEMS];
-  auto load = [&](int c) {
-#pragma unroll
-    for (int e = 0; e < ITEMS; ++e) {
-      const int j = lo + c * kChunk + e * S::THREADS + tid;
-      key[e] = j < hi ? __float_as_uint((RESIDENT ? vec_s[j] : x[j]) + 0.f) : 0x80000000u;   // sign bit: no entry (-0 becomes +0)
-    }
-  };
-  if (RESIDENT) {
-    stage_vector(vec_s, x, n);
-    __syncthreads();
-  }
-  const float mean = 1.f / (float)n;
-  float sq = 0.f;
-  unsigned remaining = (unsigned)max(1, n / 10), thr = 0, in = 0, known = 0;   // known: mask of the bits found so far
-#pragma unroll 1
-  for (int level = 0; level < 3; ++level) {
-    const int shift = 24 - 8 * level;
-    const unsigned mask = level == 0 ? 0x80000000u : 0xffffffffu << (shift + 8);
-    for (int c = 0; c < chunks; ++c) {
-      if (chunks > 1 || level == 0) load(c);
-#pragma unroll
-      for (int e = 0; e < ITEMS; ++e) {
-        if (level == 0 && !(key[e] >> 31)) {
-          const float dv = __uint_as_float(key[e]) - mean;
-          sq = fmaf(dv, dv, sq);
-        }
-        if ((key[e] & mask) == thr) radix_count(s, level & 1, (key[e] >> shift) & 255u);
-      }
-    }
-    unsigned digit;
-    radix_pick(s, level & 1, remaining, digit, in);
-    thr |= digit << shift;
-    known = 0xffffffffu << shift;
-    if (in == remaining) break;                      // all entries that share these bits count
-  }
-  float above = 0.f, inside = 0.f;
-  for (int c = 0; c < chunks; ++c) {
-    if (chunks > 1) load(c);
-#pragma unroll
-    for (int e = 0; e < ITEMS; ++e) {
-      const unsigned top = key[e] & known;
-      if (!(key[e] >> 31)) {
-        if (top > thr) above += __uint_as_float(key[e]);
-        else if (top == thr) inside += __uint_as_float(key[e]);
-      }
-    }
-  }
-  sq = block_total(sq, s.red[0]);
-  above = block_total(above, s.red[1]);
-  inside = block_total(inside, s.red[2]);
-  __shared__ float slots[3 * CL];
-  if (CL > 1) {
-    if (tid == 0) {
-      float* to = cg::this_cluster().map_shared_rank(slots, 0);
-      to[3 * rank] = sq; to[3 * rank + 1] = above; to[3 * rank + 2] = inside;
-    }
-    cluster_barrier<CL>();
-    if (rank != 0) return;
-  }
-  if (tid >= 32) return;
+// A vector's sums are known (to thread 0; one warp calls): the last head of a problem averages all of them,
+// in a fixed order.
+__device__ __forceinline__ void head_done(const FinishArgs& a, int vec, float mean, float sq, float mass) {
+  const int tid = threadIdx.x, p = vec / a.H;
   int last = 0;
   if (tid == 0) {
-    if (CL > 1) {
-      sq = above = inside = 0.f;
-      for (int r = 0; r < CL; ++r) { sq += slots[3 * r]; above += slots[3 * r + 1]; inside += slots[3 * r + 2]; }
-    }
     float* hp = a.head_part + (size_t)vec * 4;
     __stcg(hp, sq);
-    __stcg(hp + 1, above + (float)remaining * (inside / (float)in));
+    __stcg(hp + 1, mass);
     __threadfence();
     last = atomicAdd(&a.stat_ctr[p], 1) == a.H - 1;
   }
   if (!__shfl_sync(0xffffffffu, last, 0)) return;
-  // the last head of the problem averages all of them (fixed order)
   __threadfence();
   float rho = 0.f, var = 0.f;
   for (int h = tid; h < a.H; h += 32) {
@@ -262,24 +163,150 @@ __device__ __forceinline__ void stats_cta(const FinishArgs& a, S& s, float* vec_
   }
 }
 
-template <int ITEMS, int VEC, typename S>
-__global__ void
-__launch_bounds__(S::THREADS, S::THREADS < kRxThreads ? 4 : ITEMS <= 8 && !std::is_same_v<S, RadixResident> ? 2 : 1)
-finish(const __grid_constant__ FinishArgs a) {
-  extern __shared__ __align__(16) unsigned char fin_smem[];
-  S& s = *reinterpret_cast<S*>(fin_smem);
+// Eq. 5 and 6 of one (problem, head) vector by one CTA, in two sweeps over memory: the sum of squared
+// deviations from 1/n (the pooled vector sums to 1, so 1/n is its mean; summing deviations instead of
+// squares keeps near-uniform attention from cancelling) and the mass of the floor(n / 10) largest entries.
+// Counting sweeps locate the k-th largest value to 22 bits (all entries are >= 0: the order of the bit
+// patterns is theirs):
+//   sweep 1: histogram of bits 30..20 (exponent + 3 mantissa bits); sum of squared deviations
+//   sweep 2: exact sum of the entries above the threshold bin and a histogram of bits 19..9 inside it
+// The entries inside the threshold bin are then summed as count x bin midpoint: bins of the second
+// level are 2^-14 wide relative to their value, far inside the metric's tolerance.
+//
+// Bound by latency up to some 100 vectors, then by the shared-memory atomics and, where the vectors exceed
+// L2 together, by reading them twice (1024 vectors of 131072 keys: 2 x 537 MB, 164 us).  One histogram,
+// without copies for the lanes: same-address hits cost less than clearing and summing copies, whether the
+// values concentrate or not (1024 vectors of 5003 / 32768 keys: 41 / 85 us with four, 20 / 59 with one).
+// Eight-bit rank searches over keys in registers, by one CTA or a cluster, took four barriers more and ran
+// in waves (32 vectors of 5003 / 32768 keys 11 / 17 us, now 8 / 12; 128 of 131072 89, now 28).
+constexpr int kSwBins = 2048;
+struct SweepShared {
+  unsigned hist[2][kSwBins];
+  float red[3][33];
+  unsigned scan[33], bin, rem;
+};
+// The bits of a vector's sums must depend neither on how many threads work on it nor on its alignment: entry j
+// belongs to accumulator j mod 1024, and 512 threads have two each (k = 0 and 1).
+template <int T> constexpr int kStandFor = 1024 / T;
+// Applies f(entry, k) to a[0 .. n) once each, 48 or 64 KB of loads in flight on an SM.
+template <int T, class F>
+__device__ __forceinline__ void sweep_from_memory(const float* __restrict__ a, int n, F f) {
+  constexpr int kAt = T == 1024 ? 16 : 8, odd = kStandFor<T> - 1;
+  int j = threadIdx.x;
+  float v[kAt];
+  for (; j - (int)threadIdx.x + kAt * T <= n; j += kAt * T) {
+#pragma unroll
+    for (int u = 0; u < kAt; ++u) v[u] = a[j + u * T];
+#pragma unroll
+    for (int u = 0; u < kAt; ++u) f(v[u], u & odd);
+  }
+#pragma unroll
+  for (int u = 0; u < kAt; ++u)
+    if (j + u * T < n) v[u] = a[j + u * T];
+#pragma unroll
+  for (int u = 0; u < kAt; ++u)
+    if (j + u * T < n) f(v[u], u & odd);
+}
+// Sum of the accumulators over the block, in every thread of warp 0 (fixed order).
+template <int T>
+__device__ __forceinline__ float block_total(const float (&v)[kStandFor<T>], float* red) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < kStandFor<T>; ++k) {
+    float s = v[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) red[k * (T / 32) + warp] = s;
+  }
+  __syncthreads();
+  float s = 0.f;
+  if (warp == 0) {
+    s = red[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  }
+  return s;
+}
+// Walks the bins of a histogram from the top: s.bin holds the `remaining`-th largest candidate, s.rem is the
+// rank still wanted inside it.
+template <int T>
+__device__ __forceinline__ void sweep_pick(SweepShared& s, const unsigned* hist, unsigned remaining) {
+  constexpr int kPer = kSwBins / T;                        // bins of a thread, higher first
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, top = kSwBins - 1 - kPer * tid;
+  unsigned c[kPer], mine = 0;
+  __syncthreads();
+#pragma unroll
+  for (int b = 0; b < kPer; ++b) mine += c[b] = hist[top - b];
+  unsigned incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) s.scan[warp] = incl;
+  __syncthreads();
+  unsigned before = incl - mine;
+  for (int w = 0; w < warp; ++w) before += s.scan[w];
+  if (before < remaining && remaining <= before + mine) {
+#pragma unroll
+    for (int b = 0; b < kPer; ++b) {
+      if (before < remaining && remaining <= before + c[b]) {
+        s.bin = (unsigned)(top - b);
+        s.rem = remaining - before;
+      }
+      before += c[b];
+    }
+  }
+  __syncthreads();
+}
+template <int T>
+__device__ __forceinline__ void sweep_cta(const FinishArgs& a, SweepShared& s, int vec) {
+  const int tid = threadIdx.x, p = vec / a.H;
+  const Problem pb = problem_of(a, p);
+  const float* x = pb.cols + (size_t)(vec - p * a.H) * a.col_stride;
+  const int n = pb.n;
+  const float mean = 1.f / (float)n;
+  float sq[kStandFor<T>] = {}, mass[kStandFor<T>] = {}, in_bin[kStandFor<T>] = {};
+  sweep_from_memory<T>(x, n, [&](float v, int k) {
+    const float dv = v - mean;
+    sq[k] = fmaf(dv, dv, sq[k]);
+    atomicAdd(&s.hist[0][(__float_as_uint(v) >> 20) & 0x7ffu], 1u);
+  });
+  sweep_pick<T>(s, s.hist[0], (unsigned)max(1, n / 10));
+  const unsigned b1 = s.bin, rem1 = s.rem;
+  sweep_from_memory<T>(x, n, [&](float v, int k) {
+    const unsigned u = __float_as_uint(v), top = (u >> 20) & 0x7ffu;
+    if (top > b1) mass[k] += v;
+    else if (top == b1) atomicAdd(&s.hist[1][(u >> 9) & 0x7ffu], 1u);
+  });
+  sweep_pick<T>(s, s.hist[1], rem1);
+  // entries of the threshold bin above sub-bin b2, and rem2 entries of sub-bin b2 itself
+  const unsigned b2 = s.bin, rem2 = s.rem;
+#pragma unroll
+  for (int q = 0; q < kSwBins / T; ++q) {
+    const int b = q * T + tid;
+    const float mid = __uint_as_float((b1 << 20) | ((unsigned)b << 9) | 0x100u);
+    const unsigned cnt = (unsigned)b > b2 ? s.hist[1][b] : ((unsigned)b == b2 ? rem2 : 0u);
+    float& to = in_bin[q & (kStandFor<T> - 1)];
+    to = fmaf((float)cnt, mid, to);
+  }
+  const float sq_t = block_total<T>(sq, s.red[0]), mass_t = block_total<T>(mass, s.red[1]), in_t = block_total<T>(in_bin, s.red[2]);
+  if (tid < 32) head_done(a, vec, mean, sq_t, mass_t + in_t);
+}
+template <int VEC, int T>
+__global__ void __launch_bounds__(T, T == 512 ? 3 : 1) finish(const __grid_constant__ FinishArgs a) {
+  __shared__ union { SweepShared stats; SumShared<VEC> sum; } sh;
   const bool stats = (int)blockIdx.x < a.n_stat_ctas;
   pdl_trigger();
-  if (stats) {
-    radix_clear(s, 0);
-    cluster_barrier<S::CL>();                        // all CTAs of the cluster run before any remote access
-  }
+  if (stats)
+    for (int b = threadIdx.x; b < 2 * kSwBins; b += T) sh.stats.hist[0][b] = 0;
   pdl_wait();
+  __syncthreads();
   if (stats) {
-    stats_cta<ITEMS>(a, s, reinterpret_cast<float*>(fin_smem + (sizeof(S) + 15) / 16 * 16), blockIdx.x / S::CL);
+    sweep_cta<T>(a, sh.stats, blockIdx.x);
   } else {
     const int b = blockIdx.x - a.n_stat_ctas, p = b / a.chunks;
-    if (p < a.n_prob) sum_block<VEC, S::THREADS>(a, *reinterpret_cast<SumShared<VEC>*>(fin_smem), p, b - p * a.chunks);
+    sum_block<VEC, T>(a, sh.sum, p, b - p * a.chunks);
   }
 }
 constexpr int kSumThreads = 256;     // many short blocks: 16 loads in flight per thread
@@ -289,157 +316,6 @@ __global__ void __launch_bounds__(kSumThreads) sum_layers(const __grid_constant_
   pdl_trigger();
   pdl_wait();
   sum_block<VEC, kSumThreads>(a, sh, blockIdx.x / a.chunks, blockIdx.x % a.chunks);
-}
-
-// ---- Eq. 5-6 of many long vectors: one CTA per vector, two sweeps over memory --------------------
-// With more vectors than the clusters above could run side by side (32 layers of 131072 keys: 1024
-// vectors, 231 us in two sweeps of 537 MB; clusters of eight 1630 us).  Counting sweeps locate the
-// k-th largest value to 22 bits:
-//   sweep 1: histogram of bits 30..20 (exponent + 3 mantissa bits); sum of squared deviations
-//   sweep 2: exact sum of the entries above the threshold bin and a histogram of bits 19..9 inside it
-// The entries inside the threshold bin are then summed as count x bin midpoint: bins of the second
-// level are 2^-14 wide relative to their value, far inside the metric's tolerance.
-constexpr int kHsThreads = 1024, kHsBins = 2048;
-constexpr int kHsCopies = 16;      // copies of a bin, so that a warp's hits on one bin spread
-
-// Applies f to a[lo .. hi) once each, kHsThreads threads together: 16-byte loads, four of them in
-// flight per thread, scalar accesses only for the unaligned ends.  The order in which a thread
-// meets its entries is fixed.
-template <class F>
-__device__ __forceinline__ void sweep_from_memory(const float* __restrict__ a, int lo, int hi, int tid, F f) {
-  const int mis = (int)((reinterpret_cast<uintptr_t>(a + lo) >> 2) & 3u);
-  const int n_head = min(hi - lo, (4 - mis) & 3);
-  if (tid < n_head) f(a[lo + tid]);
-  const int b0 = lo + n_head;
-  const int n4 = (hi - b0) >> 2;
-  const float4* a4 = reinterpret_cast<const float4*>(a + b0);
-  int i = tid;
-  for (; i + 3 * kHsThreads < n4; i += 4 * kHsThreads) {
-    const float4 v0 = a4[i], v1 = a4[i + kHsThreads], v2 = a4[i + 2 * kHsThreads], v3 = a4[i + 3 * kHsThreads];
-    f(v0.x); f(v0.y); f(v0.z); f(v0.w);
-    f(v1.x); f(v1.y); f(v1.z); f(v1.w);
-    f(v2.x); f(v2.y); f(v2.z); f(v2.w);
-    f(v3.x); f(v3.y); f(v3.z); f(v3.w);
-  }
-  for (; i < n4; i += kHsThreads) {
-    const float4 v = a4[i];
-    f(v.x); f(v.y); f(v.z); f(v.w);
-  }
-  const int t0 = b0 + 4 * n4;
-  if (t0 + tid < hi) f(a[t0 + tid]);
-}
-
-// Called by all threads of a 1024-thread block after a histogram pass over `nb` = 2048 bins.
-// Walks the bins from the top and finds the bin holding the `remaining`-th largest candidate;
-// writes that bin and the rank still wanted inside it.  `scratch` holds 33 words.
-__device__ __forceinline__ void block_pick_from_top(const unsigned* hist, unsigned remaining,
-                                                    unsigned* scratch, unsigned* sel_bin, unsigned* sel_rem) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int b_hi = 2047 - 2 * tid, b_lo = b_hi - 1;        // this thread's two bins, higher first
-  const unsigned c_hi = hist[b_hi], c_lo = hist[b_lo];
-  const unsigned mine = c_hi + c_lo;
-  unsigned incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  __syncthreads();
-  if (lane == 31) scratch[warp] = incl;
-  __syncthreads();
-  unsigned before = incl - mine;
-  for (int w = 0; w < warp; ++w) before += scratch[w];
-  if (before < remaining && remaining <= before + mine) {
-    if (before + c_hi >= remaining) { *sel_bin = (unsigned)b_hi; *sel_rem = remaining - before; }
-    else { *sel_bin = (unsigned)b_lo; *sel_rem = remaining - before - c_hi; }
-  }
-  __syncthreads();
-}
-
-// Shared memory: hist[kHsBins][kHsCopies] | merged[2][kHsBins] (dynamic, 144 KB).
-__global__ void __launch_bounds__(kHsThreads)
-head_stats(const float* __restrict__ cols, long long layer_stride, long long col_stride, int H, int n, int k_rho,
-           float* __restrict__ head_part) {
-  extern __shared__ unsigned hs_smem[];
-  unsigned* hist = hs_smem;
-  unsigned* merged = hs_smem + kHsBins * kHsCopies;
-  __shared__ float red[3][33];
-  __shared__ unsigned scan_tmp[33];
-  __shared__ unsigned sel_bin, sel_rem;
-  const int head = blockIdx.x;                       // (layer, head) pair
-  const float* a = cols + (size_t)(head / H) * layer_stride + (size_t)(head % H) * col_stride;
-  const int tid = threadIdx.x, copy = tid & (kHsCopies - 1);
-  auto clear_local = [&]() {
-    for (int b = tid; b < kHsBins * kHsCopies; b += kHsThreads) hist[b] = 0;
-  };
-  auto push = [&](int level) {                       // sum of a bin's copies
-    for (int b = tid; b < kHsBins; b += kHsThreads) {
-      unsigned c = 0;
-#pragma unroll
-      for (int k = 0; k < kHsCopies; ++k) c += hist[b * kHsCopies + ((k + tid) & (kHsCopies - 1))];   // rotated: no bank conflicts
-      merged[level * kHsBins + b] = c;
-    }
-  };
-  pdl_trigger();
-  clear_local();
-  pdl_wait();                                        // the pooled columns come from the kernels before
-  __syncthreads();
-  float sq = 0.f;
-  const float mean = 1.f / (float)n;
-  sweep_from_memory(a, 0, n, tid, [&](float v) {
-    const float dv = v - mean;
-    sq = fmaf(dv, dv, sq);
-    atomicAdd(&hist[((__float_as_uint(v) >> 20) & 0x7ffu) * kHsCopies + copy], 1u);
-  });
-  __syncthreads();
-  push(0);
-  __syncthreads();
-  clear_local();
-  block_pick_from_top(merged, (unsigned)k_rho, scan_tmp, &sel_bin, &sel_rem);
-  const unsigned b1 = sel_bin, rem1 = sel_rem;
-  float mass = 0.f;
-  sweep_from_memory(a, 0, n, tid, [&](float v) {
-    const unsigned u = __float_as_uint(v), top = (u >> 20) & 0x7ffu;
-    if (top > b1) mass += v;
-    else if (top == b1) atomicAdd(&hist[((u >> 9) & 0x7ffu) * kHsCopies + copy], 1u);
-  });
-  __syncthreads();
-  push(1);
-  __syncthreads();
-  const unsigned* m2 = merged + kHsBins;
-  block_pick_from_top(m2, rem1, scan_tmp, &sel_bin, &sel_rem);
-  const unsigned b2 = sel_bin, rem2 = sel_rem;
-  // entries of the threshold bin above sub-bin b2, and rem2 entries of sub-bin b2 itself
-  float in_bin = 0.f;
-  for (int b = tid; b < kHsBins; b += kHsThreads) {
-    const float mid = __uint_as_float((b1 << 20) | ((unsigned)b << 9) | 0x100u);
-    const unsigned cnt = (unsigned)b > b2 ? m2[b] : ((unsigned)b == b2 ? rem2 : 0u);
-    in_bin = fmaf((float)cnt, mid, in_bin);
-  }
-  sq = block_total(sq, red[0]);
-  mass = block_total(mass, red[1]);
-  in_bin = block_total(in_bin, red[2]);
-  if (tid == 0) {
-    head_part[head * 4 + 0] = sq;
-    head_part[head * 4 + 1] = mass + in_bin;
-  }
-}
-
-// Eq. 5-6 of a batch of layers from their per-head parts: one thread per layer.
-__global__ void head_metrics(const float* __restrict__ head_part, int n_layers, int H, int n,
-                             float* __restrict__ metrics) {
-  pdl_trigger();
-  pdl_wait();
-  const int l = blockIdx.x * blockDim.x + threadIdx.x;
-  if (l >= n_layers) return;
-  float rho = 0.f, var = 0.f;
-  const float inv_n = 1.f / (float)n;
-  for (int h = 0; h < H; ++h) {
-    rho += head_part[((size_t)l * H + h) * 4 + 1];
-    var += head_part[((size_t)l * H + h) * 4 + 0] * inv_n;
-  }
-  metrics[l * 3 + 1] = rho / (float)H;
-  metrics[l * 3 + 2] = var / (float)H;
 }
 
 // c_out[j] = sum_{l <= pivot} lambda^(pivot - l) s_hist[l][j], as the recursion c = lambda c + s; the loads of
@@ -543,57 +419,18 @@ accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int 
 
 }  // namespace
 
-// Raises a kernel's shared-memory limit once per device.
-template <typename K>
-static cudaError_t allow_smem(K* kernel, int bytes, std::atomic<unsigned long long>& ready) {
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  const unsigned long long bit = 1ull << (dev & 63);
-  if (ready.load(std::memory_order_acquire) & bit) return cudaSuccess;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) ready.fetch_or(bit, std::memory_order_release);
-  return e;
-}
-
-template <int CL, int ITEMS, int VEC, typename S = RadixShared<CL>>
-static cudaError_t launch_finish_as(FinishArgs& a, int sums, cudaStream_t st) {
-  static std::atomic<unsigned long long> ready{0};
-  constexpr int smem = std::is_same_v<S, RadixResident> ? kResidentBytes : (int)std::max(sizeof(S), sizeof(SumShared<VEC>));
-  const cudaError_t e = allow_smem(finish<ITEMS, VEC, S>, smem, ready);
-  if (e != cudaSuccess) return e;
-  a.n_stat_ctas = a.n_prob * a.H * CL;
-  return launch_cluster<CL, S::THREADS>(finish<ITEMS, VEC, S>, (a.n_stat_ctas + sums + CL - 1) / CL * CL, smem, st, a);
-}
 template <int VEC>
 static cudaError_t launch_finish(FinishArgs& a, int longest, int sms, cudaStream_t st) {
   a.chunks = (longest + kSumLanes * VEC - 1) / (kSumLanes * VEC);
   const int sums = a.row_ent ? a.n_prob * a.chunks : 0;
   if (!a.with_stats) return launch_pdl(sum_layers<VEC>, dim3(sums), dim3(kSumThreads), 0, st, a);
-  // More vectors than SMs: four small CTAs share an SM, where those of 1024 threads ran one or two at a time
-  // (1024 vectors of 600 / 1777 / 5003 / 8192 keys: 37.6 / 41.3 / 49.0 / 52.6 us before, 21.4 / 23.5 / 33.2 /
-  // 36.5 now).  Longer vectors do not fit their registers.
-  const int vecs = a.n_prob * a.H;
-  if (vecs > sms && longest <= 32 * RadixSmall::THREADS) {
-    if (longest <= 8 * RadixSmall::THREADS) return launch_finish_as<1, 8, VEC, RadixSmall>(a, sums, st);
-    if (longest <= 16 * RadixSmall::THREADS) return launch_finish_as<1, 16, VEC, RadixSmall>(a, sums, st);
-    return launch_finish_as<1, 32, VEC, RadixSmall>(a, sums, st);
-  }
-  // About one vector per SM: the vector in shared memory.  Clusters would leave some of them for a second
-  // wave, and half an SM holds fewer loads in flight (128 vectors of 1777 / 5003 / 20000 / 50000 keys: 13.6 /
-  // 15.6 / 30.4 / 67.4 us before, 10.7 / 11.3 / 17.3 / 29.2 now; at 12000 14.2 against the 12.9 of 16 items).
-  // With 32 vectors the clusters' extra SMs count for more: 20.7 against 16.5 us at 32768 keys.
-  if (2 * vecs > sms && vecs <= sms && longest <= kResidentMax &&
-      (longest <= 8 * kRxThreads || longest > 16 * kRxThreads))
-    return launch_finish_as<1, 8, VEC, RadixResident>(a, sums, st);
-  // one CTA per vector while its registers hold it (no exchange between CTAs), else the smallest
-  // cluster that does
-  if (longest <= 4 * kRxThreads) return launch_finish_as<1, 4, VEC>(a, sums, st);
-  if (longest <= 8 * kRxThreads) return launch_finish_as<1, 8, VEC>(a, sums, st);
-  if (longest <= 16 * kRxThreads) return launch_finish_as<1, 16, VEC>(a, sums, st);
-  if (longest <= 32 * kRxThreads) return launch_finish_as<2, 16, VEC>(a, sums, st);
-  if (longest <= 64 * kRxThreads) return launch_finish_as<4, 16, VEC>(a, sums, st);
-  return launch_finish_as<4, 32, VEC>(a, sums, st);
+  // An SM per vector: as many threads as a CTA can have.  More vectors than SMs: three CTAs an SM fill each
+  // other's gaps between barriers (512 vectors of 5003 / 32768 keys: 26 / 41 us with one of 1024 threads an
+  // SM, 15 / 31 with three of 512).
+  a.n_stat_ctas = a.n_prob * a.H;
+  const dim3 grid(a.n_stat_ctas + sums);
+  if (a.n_stat_ctas <= sms) return launch_pdl(finish<VEC, 1024>, grid, dim3(1024), 0, st, a);
+  return launch_pdl(finish<VEC, 512>, grid, dim3(512), 0, st, a);
 }
 
 static FinishArgs finish_args(const Ctx& ctx, const float* cols, long long col_stride, int n, float* metrics) {
@@ -635,26 +472,8 @@ cudaError_t launch_finish_packed(const Ctx& ctx, const float* cols, long long co
   return vec ? launch_finish<4>(a, longest, ctx.sm_count, st) : launch_finish<1>(a, longest, ctx.sm_count, st);
 }
 
-// Two sweeps per vector where the vectors fill the GPU several times over and are long: with 1024
-// vectors 85 / 115 / 231 us at 16000 / 32768 / 131072 keys, the register form 91 / 140 / > 500.
-bool head_stats_ride_along(const Ctx& ctx, int n_layers, int n) {
-  return (long long)n_layers * ctx.cfg.n_q_heads < 2ll * ctx.sm_count || n <= 8 * kRxThreads;
-}
-
 cudaError_t launch_head_stats_batch(const Ctx& ctx, const float* cols, long long layer_stride, long long col_stride,
                                     int n_layers, int n, float* metrics, cudaStream_t st) {
-  const int H = ctx.cfg.n_q_heads;
-  if (!head_stats_ride_along(ctx, n_layers, n)) {
-    static std::atomic<unsigned long long> ready{0};
-    const int smem = (kHsBins * kHsCopies + 2 * kHsBins) * (int)sizeof(unsigned);
-    cudaError_t e = allow_smem(head_stats, smem, ready);
-    if (e != cudaSuccess) return e;
-    e = launch_pdl(head_stats, dim3(n_layers * H), dim3(kHsThreads), smem, st, cols, layer_stride, col_stride, H, n,
-                   n / 10 < 1 ? 1 : n / 10, ctx.ws.head_part);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(head_metrics, dim3((n_layers + 63) / 64), dim3(64), 0, st, (const float*)ctx.ws.head_part, n_layers,
-                      H, n, metrics);
-  }
   FinishArgs a = finish_args(ctx, cols, col_stride, n, metrics);
   a.layer_stride = layer_stride; a.n_prob = n_layers; a.with_stats = 1;
   return launch_finish<1>(a, n, ctx.sm_count, st);

@@ -76,7 +76,7 @@ def test_head_statistics_around_the_edges(ctx, edge):
 @pytest.mark.parametrize("layers", [20, 40])
 @pytest.mark.parametrize("n", [7, 601, 2048, 2049, 4097, 8192, 8193, 16385, 50000, 51200, 51201])
 def test_head_statistics_of_many_vectors(ctx, layers, n):
-    """About one vector per SM, and more vectors than SMs (small CTAs, vectors held in shared memory)."""
+    """An SM per vector, and more vectors than SMs: within the tolerance, and the bits of a layer by itself."""
     rng = np.random.default_rng(n + layers)
     buf = torch.zeros((layers, 4, n + 1), device="cuda")     # odd strides: every alignment of a vector
     x = rng.random((layers, 4, n)) ** 4
@@ -85,7 +85,10 @@ def test_head_statistics_of_many_vectors(ctx, layers, n):
     buf[:, :, 1:] = torch.from_numpy(x32).cuda()
     m = torch.zeros((layers, 3), device="cuda")
     ctx.head_stats(buf[:, :, 1:], m)
+    one = torch.zeros((1, 3), device="cuda")
     for l in {0, 1, layers - 1}:
+        ctx.head_stats(buf[l:l + 1, :, 1:], one)
+        assert torch.equal(m[l], one[0])
         rho, var = O.head_statistics(x32[l].astype(np.float64))
         P.assert_metric_close(m[l, 1].item(), rho, f"sparsity at {n}")
         P.assert_metric_close(m[l, 2].item(), var, f"variance at {n}")
