@@ -104,20 +104,26 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
     pb.inv_c2 = 1.f / pb.c2;
     pb.v_min = -125.f / pb.c2;
     const int tiles = (pb.n_keys + kKeyTile - 1) / kKeyTile;
-    // One task per SM and pass, shared out over the sequences of a batch by their lengths; in pass 1 at
-    // least two pairs of tiles a task, which carries 1.5 us of hand-over whatever its size, unless all
-    // of them run at once anyway.
+    // Pass 1 leaves one partial per key segment: as many segments as SMs, shared out over the sequences of a
+    // batch by their lengths, of at least two pairs of tiles unless all of them run at once anyway.
+    // That depends on the shape alone, so that a layer gives the same bits by itself and among others.
     const int share = batch ? std::max(1, (int)((long long)sms * pb.n_keys / total_keys)) : sms;
     const int pairs = (tiles + 1) / 2;
-    pb.t1 = clamp_tasks(l, share, (long long)l.units * pairs <= sms ? pairs : (pairs + 1) / 2);
-    // Pass 2 leaves no partial results, so the pass nothing follows is cut finer: its tasks end
-    // closer together.
+    pb.s1 = clamp_tasks(l, share, (long long)l.units * pairs <= sms ? pairs : (pairs + 1) / 2);
+    // A task by itself runs one segment; with other layers to fill the SMs it runs as many as make five pairs:
+    // the way from task to task costs as much as one (32 layers of 5003 keys: 302 us with two pairs a
+    // task, 253 with four or more).  The same in pass 2, which leaves no partial results.
+    const bool alone = batch || n == 1;
+    const long long work = (long long)l.units * pairs;
+    const int run = alone ? 1 : (int)std::max(1ll, (10ll * pb.s1 + work) / (2 * work));
+    pb.t1 = run == 1 ? pb.s1 : clamp_tasks(l, pb.s1 / run, pb.s1);
+    // The pass nothing follows is cut finer: its tasks end closer together.
     // (Not below eight tiles a task, each of which merges its unit's statistics first.)
     const bool last = batch || i == n - 1;
-    if (!last) pb.t2 = clamp_tasks(l, share, (tiles + 3) / 4);
+    if (!last) pb.t2 = clamp_tasks(l, share, run > 1 ? (tiles + 9) / 10 : (tiles + 3) / 4);
     else pb.t2 = clamp_tasks(l, (long long)l.units * tiles >= 16ll * share ? 2 * share : share, tiles);
     pb.part0 = part0;
-    part0 += pb.t1;
+    part0 += pb.s1;
   }
   // ticket order
   int n_ph = 0, tickets = 0;
@@ -131,9 +137,9 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
   } else {
     // Pass 1 runs `ahead` layers in front of pass 2, far enough to cover the way from a unit's last
     // pass-1 task to its merged statistics (10 to 15 us) with other work: one layer where a layer's
-    // pass 1 is at least eight pairs of key tiles (1.2 us each) per SM, more for shorter sequences.
+    // pass 1 is at least twelve pairs of key tiles (1.2 us each) per SM, more for shorter sequences.
     const long long pairs = (long long)l.units * ((p.prob[0].n_keys + 2 * kKeyTile - 1) / (2 * kKeyTile));
-    const int ahead = (int)std::min<long long>(std::min(n - 1, 12), std::max(1ll, (8ll * sms + pairs - 1) / pairs));
+    const int ahead = (int)std::min<long long>(std::min(n - 1, 20), std::max(1ll, (12ll * sms + pairs - 1) / pairs));
     for (int i = 0; i < n + ahead; ++i) {
       if (i < n) phase(i, 1);
       if (i >= ahead) phase(i - ahead, 2);

@@ -15,7 +15,8 @@
 // pass is drawn, no SM idles while the slowest CTA of a pass finishes, and nothing of a CTA's set-up
 // (launch, tensor-memory allocation, first copies) is paid per layer: with two launches per layer
 // that set-up and the uneven last wave were 12 % of a layer of 131072 keys and a third at 32768.
-// Which keys a pass-1 task covers depends on the shape alone, so results do not depend on timing.
+// Which keys a partial of pass 1 covers (a segment) depends on the shape alone, so results depend neither on
+// timing nor on how many segments a task runs.
 //
 // Two layouts of the score rows:
 //   wide    (more than 64 rows per KV group) pass 1 D[rows, keys] = Q K^T, lane = row; pass 2
@@ -74,7 +75,7 @@ struct TcProblem {
   int map, head0;                      // tensor maps; first head in the Q tensor
   float c2, inv_c2, v_min;             // |scale| * log2(e), at least 1e-30; 1 / c2; -125 / c2
   int negate;                          // the scale is negative: the MMA negates its A operand
-  int t1, t2, part0;                   // tasks of the two passes; first partial of pass 1
+  int s1, t1, t2, part0;               // key segments of pass 1, tasks of the two passes; first partial of pass 1
 };
 // A run of consecutive tickets: tasks [task0, ...) of one pass of one problem.
 struct TcPhase { int first; unsigned short task0; unsigned char prob, pass; };
@@ -420,7 +421,8 @@ struct alignas(16) TcTask {
   int negate;
   float* cols;                         // pass 2: output of the KV group's first head
   int prob, group;
-  int part, part0, n_part, pad;        // pass 1: where its statistics go; the unit's partials
+  int part, part0, n_part, n_arrive;   // pass 1: where its statistics go; the unit's partials and pass-1 tasks
+  int seg, n_seg, n_pairs, pad;        // pass 1: segments [seg, seg + n_seg) of the unit's n_part over n_pairs tile pairs
 };
 constexpr int kTaskBytes = 96;
 static_assert(sizeof(TcTask) <= kTaskBytes && sizeof(TcTask) % 16 == 0, "task slot");
@@ -621,7 +623,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
 
   // A consumer warp takes its next task: lane 0 polls (bounded), every lane reads the descriptor.
   // (With the suspending wait: helper warps sit here for a whole task and must not take issue slots.)
-  auto next_task = [&](int n, TcTask& t) {
+  auto next_task = [&](int n, TcTask& t, bool keep = false) {
     const int k = n % kTaskRing;
     int ok = 1;
     if (lane == 0)
@@ -630,6 +632,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     asm volatile("" ::: "memory");
     t = *task_slot(k);
     asm volatile("" ::: "memory");
+    if (keep) return t.pass != 0;                          // the slot is given back by task_done
     __syncwarp();
     if (lane == 0) mbar_arrive(bar(kBarTaskEmpty + k));
     return t.pass != 0;
@@ -648,6 +651,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     *reinterpret_cast<__nv_bfloat16*>(bx + k16_offset(r, 2)) = lo;
   };
   auto is_row = [&](int row) { return row < p.rows_pg && (row & (p.w_pad - 1)) < p.window; };   // row of the KV group, padding excluded
+  // First key tile of segment k of a pass-1 task (which holds n_seg of them).
+  auto segment_lo = [](const volatile TcTask& t, int k) { return 2 * (int)((unsigned)(t.seg + k) * (unsigned)t.n_pairs / (unsigned)t.n_part); };
   // The n-th Q block: wide ones come in halves with a barrier each, narrow ones alternate between two buffers.
   auto q_bar = [](int n, int half) { return S::kQBufs == 2 ? n & 1 : half; };
   auto q_parity = [](int n) { return (uint32_t)(S::kQBufs == 2 ? n >> 1 : n) & 1u; };
@@ -686,22 +691,26 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
           const int w0 = g * p.w_group + rb * kFullWeight;
           const int i0 = tc_deal(w0, tasks, p.w_total);
           const int w_unit = rb == p.n_rb - 1 ? p.w_last : kFullWeight;
-          const int n_seg = tc_deal(w0 + w_unit, tasks, p.w_total) - i0;
-          const int seg = i - i0, n_tiles = (pb.n_keys + kKeyTile - 1) / kKeyTile;
+          const int n_here = tc_deal(w0 + w_unit, tasks, p.w_total) - i0;
+          const int at = i - i0, n_tiles = (pb.n_keys + kKeyTile - 1) / kKeyTile;
+          // the unit's segments: one partial each
+          const int s0 = tc_deal(w0, pb.s1, p.w_total);
+          t.n_part = tc_deal(w0 + w_unit, pb.s1, p.w_total) - s0;
+          t.part0 = pb.part0 + s0;
           if (t.pass == 1) {
-            const int n_pairs = (n_tiles + 1) / 2;
-            t.lo = 2 * (int)((long long)seg * n_pairs / n_seg);
-            t.hi = 2 * (int)((long long)(seg + 1) * n_pairs / n_seg);
+            t.n_arrive = n_here;
+            t.seg = at * t.n_part / n_here;
+            t.n_seg = (at + 1) * t.n_part / n_here - t.seg;
+            t.part = t.part0 + t.seg;
+            t.n_pairs = (n_tiles + 1) / 2;
+            t.lo = segment_lo(t, 0);
+            t.hi = segment_lo(t, t.n_seg);
             if (S::kNarrow) t.hi = min(t.hi, n_tiles);     // a wide accumulator takes a pair: the odd tile's partner is masked
           } else {
-            t.lo = (int)((long long)seg * n_tiles / n_seg);
-            t.hi = (int)((long long)(seg + 1) * n_tiles / n_seg);
+            t.n_arrive = tc_deal(w0 + w_unit, pb.t1, p.w_total) - tc_deal(w0, pb.t1, p.w_total);
+            t.lo = (int)((long long)at * n_tiles / n_here);
+            t.hi = (int)((long long)(at + 1) * n_tiles / n_here);
           }
-          t.part = pb.part0 + i;
-          // the unit's partials: pass 1 deals its own number of tasks
-          const int p0 = tc_deal(w0, pb.t1, p.w_total);
-          t.n_part = tc_deal(w0 + w_unit, pb.t1, p.w_total) - p0;
-          t.part0 = pb.part0 + p0;
           t.unit = g * p.n_rb + rb;
           t.slot = t.prob * p.n_units + t.unit;
           t.n_keys = pb.n_keys;
@@ -907,7 +916,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         if (ok) {
           mbar_arrive(bar(kBarPartEmpty));
           __threadfence();
-          last = atomicAdd(p.ctl + kCtlArrive + t.prob * kQueueUnits + t.unit, 1) == t.n_part - 1;
+          last = atomicAdd(p.ctl + kCtlArrive + t.prob * kQueueUnits + t.unit, 1) == t.n_arrive - 1;
         }
       }
       if (!__shfl_sync(0xffffffffu, ok, 0)) break;
@@ -933,7 +942,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     const int sub = (warp - kHelperWarps) >> 2;   // which quarter of an accumulator's columns (or of the tiles) it takes
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
     float2* part_s = reinterpret_cast<float2*>(sm + L::kPartOff);
-    int u = 0, n_p1 = 0, n_ext = 0;
+    int u = 0, n_p1 = 0, n_fold = 0, n_ext = 0;
     // Every lane polls: a barrier that has already flipped costs one test, no divergence, no broadcast
     // (with four chunks of arithmetic per accumulator and scheduler each instruction here shows).
     auto acc_full_at = [&](int u) {
@@ -956,14 +965,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     // column groups; narrow: one set of rows, four lane quarters) leave them in shared memory, meet, and one or
     // two of them fold and store them.  Two buffers: whoever writes one again has met the readers of
     // the other since.  The helper that counts the task's arrival works beside the next task.
-    auto part_buf = [&](int k) { return part_s + ((n_p1 & 1) * 3 + k) * R; };
+    auto part_buf = [&](int k) { return part_s + ((n_fold & 1) * 3 + k) * R; };
     auto fold_meet = [&](int set) {
       __syncwarp();
       if (lane == 0) mbar_arrive(bar(kBarFold + set));
-      const bool ok = mbar_wait(bar(kBarFold + set), (uint32_t)n_p1 & 1u, abort_flag);
+      const bool ok = mbar_wait(bar(kBarFold + set), (uint32_t)n_fold & 1u, abort_flag);
       return __all_sync(0xffffffffu, ok) != 0;
     };
-    auto part_stored = [&](const TcTask& t) {
+    auto part_stored = [&](const volatile TcTask& t) {
       __syncwarp();
       bool ok = true;
       if (lane == 0) {
@@ -988,7 +997,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         while (ok) {
           int seen;
           asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
-          if (seen >= t.n_part * S::kFoldWarps) break;
+          if (seen >= t.n_arrive * S::kFoldWarps) break;
           if (*abort_flag) ok = false;
           else if ((unsigned long long)(clock64() - t0) > kWaitCycles) { *abort_flag = 1; ok = false; }
         }
@@ -1026,8 +1035,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     };
     TcTask t;
     bool live = true;
-    for (int n = 0; live && next_task(n, t); ++n) {
-      const int n_keys = t.n_keys, items = items_of(t);
+    // What a task needs between its segments stays in its slot, not in registers.
+    auto task_done = [&](int n) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(kBarTaskEmpty + n % kTaskRing));
+    };
+    for (int n = 0; live && next_task(n, t, true); task_done(n), ++n) {
+      const volatile TcTask& slot = *task_slot(n % kTaskRing);
+      const int n_keys = t.n_keys;
       const float c2 = t.c2;
       const uint64_t c22 = pack2(c2, c2);
       const int last_open_key = n_keys - p.window;         // the last key every window row sees
@@ -1039,13 +1054,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         // row (quarter * 32 + lane) of BOTH halves (accumulators alternate between them) and the 64
         // keys [sub * 64, sub * 64 + 64) of every pair.
         float v[32] = {};
-        RowStat rs[2] = {{-INFINITY, 0.f, 0.f}, {-INFINITY, 0.f, 0.f}};
         const int row_lo = quarter * 32 + lane;
         const int rows_here = min(R, t.rows), n_half = rows_here > 128 ? 2 : 1;
         auto chunk = [&](RowStat& r, int jb, bool first, int hf) {
           // of the last pair only the chunks that hold window keys (or lie beyond the sequence) are masked
           bool careful = jb + 31 > last_open_key;
-          if (first && !careful) {                          // a task's first chunk gives the rows their reference
+          if (first && !careful) {                          // a segment's first chunk gives the rows their reference
             float mx = v[0];
 #pragma unroll
             for (int e = 1; e < 32; ++e) mx = fmaxf(mx, v[e]);
@@ -1061,37 +1075,41 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         // One copy of the body for both halves (instruction cache): the statistics of the two rows swap
         // places after every accumulator.  The two 32-key chunks stay unrolled, so that the second
         // load travels under the first chunk's arithmetic.
-        const int n_acc = items * n_half;
-        for (int k = 0; k < n_acc; ++k) {
-          if (!acc_full()) { live = false; break; }
-          const int it = n_half == 2 ? k >> 1 : k, hf = n_half == 2 ? k & 1 : 0;
-          const int jb = (t.lo + 2 * it) * kKeyTile + sub * 64;
-          const bool warp_active = hf * 128 + quarter * 32 < rows_here;
-          if (warp_active) {
-            tmem_ld(acc_addr() + sub * 64, v);
-            chunk(rs[0], jb, it == 0, hf);
-            tmem_ld(acc_addr() + sub * 64 + 32, v);
+        for (int sg = 0; sg < slot.n_seg && live; ++sg) {
+          const int lo = segment_lo(slot, sg), n_acc = (segment_lo(slot, sg + 1) - lo) / 2 * n_half;
+          RowStat rs[2] = {{-INFINITY, 0.f, 0.f}, {-INFINITY, 0.f, 0.f}};
+          for (int k = 0; k < n_acc; ++k) {
+            if (!acc_full()) { live = false; break; }
+            const int it = n_half == 2 ? k >> 1 : k, hf = n_half == 2 ? k & 1 : 0;
+            const int jb = (lo + 2 * it) * kKeyTile + sub * 64;
+            const bool warp_active = hf * 128 + quarter * 32 < rows_here;
+            if (warp_active) {
+              tmem_ld(acc_addr() + sub * 64, v);
+              chunk(rs[0], jb, it == 0, hf);
+              tmem_ld(acc_addr() + sub * 64 + 32, v);
+            }
+            acc_release();
+            if (warp_active) chunk(rs[0], jb + 32, false, hf);
+            if (n_half == 2) {
+              const RowStat o = rs[0];
+              rs[0] = rs[1];
+              rs[1] = o;
+            }
+            ++u;
           }
-          acc_release();
-          if (warp_active) chunk(rs[0], jb + 32, false, hf);
-          if (n_half == 2) {
-            const RowStat o = rs[0];
-            rs[0] = rs[1];
-            rs[1] = o;
+          if (!live) break;
+          // column group 0 folds the rows of the first half, column group 1 those of the second
+          const float2 part0 = stat_partial(rs[0]), part1 = stat_partial(rs[1]);
+          if (sub != 0) part_buf(sub - 1)[row_lo] = part0;
+          if (sub != 1) part_buf(sub == 0 ? 0 : sub - 1)[128 + row_lo] = part1;
+          if (!fold_meet(quarter)) { live = false; break; }
+          if (sub < 2) {
+            const int r = sub * 128 + row_lo;
+            __stcg(&p.part[(size_t)(slot.part + sg) * R + r], fold_row(part_buf(0) + r, R, sub == 0 ? part0 : part1, sub));
           }
-          ++u;
+          ++n_fold;
         }
-        if (!live) break;
-        // column group 0 folds the rows of the first half, column group 1 those of the second
-        const float2 part0 = stat_partial(rs[0]), part1 = stat_partial(rs[1]);
-        if (sub != 0) part_buf(sub - 1)[row_lo] = part0;
-        if (sub != 1) part_buf(sub == 0 ? 0 : sub - 1)[128 + row_lo] = part1;
-        if (!fold_meet(quarter)) break;
-        if (sub < 2) {
-          const int r = sub * 128 + row_lo;
-          __stcg(&p.part[(size_t)t.part * R + r], fold_row(part_buf(0) + r, R, sub == 0 ? part0 : part1, sub));
-          if (!part_stored(t)) break;
-        }
+        if (!live || (sub < 2 && !part_stored(slot))) break;
         ++n_p1;
       } else if (t.pass == 1) {
         if constexpr (S::kNarrow) {
@@ -1103,104 +1121,107 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
           constexpr int RT = R / 4, T = RT == 8 ? 4 : 1, kLanes = 32 / RT;
           float v[T * RT];
           const float masked = fmaxf(kMasked * t.inv_c2, kMaskedAcc);   // times c2: finite, and 2^x flushes to 0
-          uint64_t nref2[RT / 2], Z2[RT / 2], U2[RT / 2];  // pairs of rows: -reference, Z, U
+          for (int sg = 0; sg < slot.n_seg && live; ++sg) {
+            const int lo = segment_lo(slot, sg), hi = min((int)slot.hi, segment_lo(slot, sg + 1));
+            uint64_t nref2[RT / 2], Z2[RT / 2], U2[RT / 2];  // pairs of rows: -reference, Z, U
 #pragma unroll
-          for (int e = 0; e < RT / 2; ++e) nref2[e] = Z2[e] = U2[e] = 0;
-          for (int tile0 = t.lo; tile0 < t.hi; tile0 += T) {
-            const int n_here = min(T, t.hi - tile0);
-            for (int k = 0; k < n_here; ++k) live = live && acc_full_at(u + k);
+            for (int e = 0; e < RT / 2; ++e) nref2[e] = Z2[e] = U2[e] = 0;
+            for (int tile0 = lo; tile0 < hi; tile0 += T) {
+              const int n_here = min(T, hi - tile0);
+              for (int k = 0; k < n_here; ++k) live = live && acc_full_at(u + k);
+              if (!live) break;
+#pragma unroll
+              for (int k = 0; k < T; ++k)
+                tmem_ld_issue<RT>(tmem + lane_base + (uint32_t)(((u + min(k, n_here - 1)) % S::kAcc) * S::kAccCols) + sub * RT, v + k * RT);
+              tmem_ld_wait(v);
+              tc_fence_before();
+              __syncwarp();
+              if (lane < n_here) mbar_arrive(bar(kBarAccEmpty + (u + lane) % S::kAcc));
+              u += n_here;
+              const bool plain = tile0 + n_here <= first_tail_tile && n_here == T;
+              if (!plain) {
+#pragma unroll
+                for (int k = 0; k < T; ++k) {
+                  const int over = k < n_here ? (tile0 + k) * kKeyTile + quarter * 32 + lane - last_open_key : 0x7fffffff;
+#pragma unroll
+                  for (int e = 0; e < RT; ++e)         // rows i < over do not see this key
+                    if (((sub * RT + e) & (p.w_pad - 1)) < over) v[k * RT + e] = masked;
+                }
+              }
+              // largest logit of rows 2 e and 2 e + 1 over the warp's keys of these tiles
+              auto row_max = [&](int e, float& m0, float& m1) {
+                m0 = v[2 * e];
+                m1 = v[2 * e + 1];
+#pragma unroll
+                for (int k = 1; k < T; ++k) {
+                  m0 = fmaxf(m0, v[k * RT + 2 * e]);
+                  m1 = fmaxf(m1, v[k * RT + 2 * e + 1]);
+                }
+                m0 = warp_max(m0) * c2;
+                m1 = warp_max(m1) * c2;
+              };
+              if (tile0 == lo) {                           // the references: where a task starts, unless masked
+#pragma unroll
+                for (int e = 0; e < RT / 2; ++e) {
+                  float m0, m1;
+                  row_max(e, m0, m1);
+                  nref2[e] = pack2(m0 > 0.5f * masked * c2 ? -m0 : 0.f, m1 > 0.5f * masked * c2 ? -m1 : 0.f);
+                }
+              }
+              float top = -INFINITY;
+#pragma unroll
+              for (int i = 0; i < T * RT / 2; ++i) {
+                const uint64_t x2 = fma2(pack2(v[2 * i], v[2 * i + 1]), c22, nref2[i % (RT / 2)]);
+                float x0, x1;
+                unpack2(x2, x0, x1);
+                top = fmaxf(top, fmaxf(x0, x1));
+              }
+              if (__any_sync(0xffffffffu, top > 60.f)) {     // far above the references: they move up
+#pragma unroll
+                for (int e = 0; e < RT / 2; ++e) {
+                  float m[2], r[2], z[2], w[2];
+                  row_max(e, m[0], m[1]);
+                  unpack2(nref2[e], r[0], r[1]);
+                  unpack2(Z2[e], z[0], z[1]);
+                  unpack2(U2[e], w[0], w[1]);
+#pragma unroll
+                  for (int h = 0; h < 2; ++h)
+                    if (m[h] > -r[h]) {
+                      const float dm = -r[h] - m[h], f = fast_exp2(dm);
+                      w[h] = f * fmaf(dm, z[h], w[h]);
+                      z[h] *= f;
+                      r[h] = -m[h];
+                    }
+                  nref2[e] = pack2(r[0], r[1]);
+                  Z2[e] = pack2(z[0], z[1]);
+                  U2[e] = pack2(w[0], w[1]);
+                }
+              }
+#pragma unroll
+              for (int i = 0; i < T * RT / 2; ++i) {
+                const uint64_t x2 = fma2(pack2(v[2 * i], v[2 * i + 1]), c22, nref2[i % (RT / 2)]), p2 = exp2_sfu2(x2);
+                Z2[i % (RT / 2)] = add2(Z2[i % (RT / 2)], p2);
+                U2[i % (RT / 2)] = fma2(p2, x2, U2[i % (RT / 2)]);
+              }
+            }
             if (!live) break;
+            float ref[RT], Z[RT], U[RT];
 #pragma unroll
-            for (int k = 0; k < T; ++k)
-              tmem_ld_issue<RT>(tmem + lane_base + (uint32_t)(((u + min(k, n_here - 1)) % S::kAcc) * S::kAccCols) + sub * RT, v + k * RT);
-            tmem_ld_wait(v);
-            tc_fence_before();
-            __syncwarp();
-            if (lane < n_here) mbar_arrive(bar(kBarAccEmpty + (u + lane) % S::kAcc));
-            u += n_here;
-            const bool plain = tile0 + n_here <= first_tail_tile && n_here == T;
-            if (!plain) {
-#pragma unroll
-              for (int k = 0; k < T; ++k) {
-                const int over = k < n_here ? (tile0 + k) * kKeyTile + quarter * 32 + lane - last_open_key : 0x7fffffff;
-#pragma unroll
-                for (int e = 0; e < RT; ++e)         // rows i < over do not see this key
-                  if (((sub * RT + e) & (p.w_pad - 1)) < over) v[k * RT + e] = masked;
-              }
+            for (int e = 0; e < RT / 2; ++e) {
+              unpack2(nref2[e], ref[2 * e], ref[2 * e + 1]);
+              unpack2(Z2[e], Z[2 * e], Z[2 * e + 1]);
+              unpack2(U2[e], U[2 * e], U[2 * e + 1]);
             }
-            // largest logit of rows 2 e and 2 e + 1 over the warp's keys of these tiles
-            auto row_max = [&](int e, float& m0, float& m1) {
-              m0 = v[2 * e];
-              m1 = v[2 * e + 1];
-#pragma unroll
-              for (int k = 1; k < T; ++k) {
-                m0 = fmaxf(m0, v[k * RT + 2 * e]);
-                m1 = fmaxf(m1, v[k * RT + 2 * e + 1]);
-              }
-              m0 = warp_max(m0) * c2;
-              m1 = warp_max(m1) * c2;
-            };
-            if (tile0 == t.lo) {                           // the references: where a task starts, unless masked
-#pragma unroll
-              for (int e = 0; e < RT / 2; ++e) {
-                float m0, m1;
-                row_max(e, m0, m1);
-                nref2[e] = pack2(m0 > 0.5f * masked * c2 ? -m0 : 0.f, m1 > 0.5f * masked * c2 ? -m1 : 0.f);
-              }
-            }
-            float top = -INFINITY;
-#pragma unroll
-            for (int i = 0; i < T * RT / 2; ++i) {
-              const uint64_t x2 = fma2(pack2(v[2 * i], v[2 * i + 1]), c22, nref2[i % (RT / 2)]);
-              float x0, x1;
-              unpack2(x2, x0, x1);
-              top = fmaxf(top, fmaxf(x0, x1));
-            }
-            if (__any_sync(0xffffffffu, top > 60.f)) {     // far above the references: they move up
-#pragma unroll
-              for (int e = 0; e < RT / 2; ++e) {
-                float m[2], r[2], z[2], w[2];
-                row_max(e, m[0], m[1]);
-                unpack2(nref2[e], r[0], r[1]);
-                unpack2(Z2[e], z[0], z[1]);
-                unpack2(U2[e], w[0], w[1]);
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                  if (m[h] > -r[h]) {
-                    const float dm = -r[h] - m[h], f = fast_exp2(dm);
-                    w[h] = f * fmaf(dm, z[h], w[h]);
-                    z[h] *= f;
-                    r[h] = -m[h];
-                  }
-                nref2[e] = pack2(r[0], r[1]);
-                Z2[e] = pack2(z[0], z[1]);
-                U2[e] = pack2(w[0], w[1]);
-              }
-            }
-#pragma unroll
-            for (int i = 0; i < T * RT / 2; ++i) {
-              const uint64_t x2 = fma2(pack2(v[2 * i], v[2 * i + 1]), c22, nref2[i % (RT / 2)]), p2 = exp2_sfu2(x2);
-              Z2[i % (RT / 2)] = add2(Z2[i % (RT / 2)], p2);
-              U2[i % (RT / 2)] = fma2(p2, x2, U2[i % (RT / 2)]);
-            }
+            const float ref_l = -lane_element(ref, lane), Z_l = warp_sum_scatter(Z, lane), U_l = warp_sum_scatter(U, lane);
+            const float2 part = stat_partial(RowStat{Z_l > 0.f ? ref_l : -INFINITY, Z_l, U_l});
+            const int r = sub * RT + lane / kLanes;
+            if (quarter != 0 && lane % kLanes == 0) part_buf(quarter - 1)[r] = part;
+            if (!fold_meet(sub)) { live = false; break; }
+            if (quarter == 0 && lane % kLanes == 0)
+              __stcg(&p.part[(size_t)(slot.part + sg) * R + r], fold_row(part_buf(0) + r, R, part, 0));
+            ++n_fold;
           }
-          if (!live) break;
-          float ref[RT], Z[RT], U[RT];
-#pragma unroll
-          for (int e = 0; e < RT / 2; ++e) {
-            unpack2(nref2[e], ref[2 * e], ref[2 * e + 1]);
-            unpack2(Z2[e], Z[2 * e], Z[2 * e + 1]);
-            unpack2(U2[e], U[2 * e], U[2 * e + 1]);
-          }
-          const float ref_l = -lane_element(ref, lane), Z_l = warp_sum_scatter(Z, lane), U_l = warp_sum_scatter(U, lane);
-          const float2 part = stat_partial(RowStat{Z_l > 0.f ? ref_l : -INFINITY, Z_l, U_l});
-          const int r = sub * RT + lane / kLanes;
-          if (quarter != 0 && lane % kLanes == 0) part_buf(quarter - 1)[r] = part;
-          if (!fold_meet(sub)) break;
-          if (quarter == 0) {
-            if (lane % kLanes == 0) __stcg(&p.part[(size_t)t.part * R + r], fold_row(part_buf(0) + r, R, part, 0));
-            if (!part_stored(t)) break;
-          }
+          if (!live || (quarter == 0 && !part_stored(slot))) break;
           ++n_p1;
         }
       } else {
