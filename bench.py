@@ -376,15 +376,19 @@ def compaction_figures(wl, kv_budget, compact_ms_per_step, peaks):
 
 def launches_per_step(wl, flags):
     from paper_2604_06746_b200 import binding
-    # layer by layer: scorer pass 1, pass 2, column reduce + metrics (the CUDA-core scorer adds a row
-    # finalisation); per step: batched head statistics (2), accumulate, 2 selections, one K/V gather
-    # over all layers, hidden states, positions
-    stats = 0 if (flags & binding.FLAG_NO_HEAD_STATS) else 2
-    if wl.dtype == "bf16" and not (flags & (binding.FLAG_NO_HEAD_STATS | binding.FLAG_FORCE_SIMT)):
-        scoring = 2 * wl.n_layers + 1          # one structkv_score_layers call: two passes per layer, one reduce over heads
+    # one call for all layers: the tensor-core scorer (one launch per 32 layers, both passes) or the two
+    # CUDA-core passes, then one launch for the sums over heads; layer by layer the same per layer.  Per
+    # step: head statistics of all layers, centrality at the pivot, all selections, one K/V gather over
+    # all layers, hidden states, positions
+    tc = wl.dtype == "bf16" and not flags & binding.FLAG_FORCE_SIMT
+    together = not flags & (binding.FLAG_NO_HEAD_STATS | binding.FLAG_FORCE_SIMT)
+    stats = 0 if flags & binding.FLAG_NO_HEAD_STATS else 1
+    scorer = 1 if tc else 2
+    if together:
+        scoring = (-(-wl.n_layers // 32) if tc else scorer) + 1
     else:
-        scoring = wl.n_layers * (3 if wl.dtype == "bf16" else 4)
-    return scoring + stats + 1 + 2 + 1 + 2
+        scoring = wl.n_layers * (scorer + 1)
+    return scoring + stats + 1 + 1 + 1 + 2
 
 
 # ------------------------------------------------------------------------------------------------

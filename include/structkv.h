@@ -12,7 +12,8 @@
  *     caller passes one workspace at context creation (structkv_workspace_bytes()).
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  All
  *     calls enqueue work on it and return without synchronising, except structkv_pivot and
- *     structkv_poll_device_status, which synchronise that stream.
+ *     structkv_poll_device_status, which synchronise that stream, and structkv_pivot_select and
+ *     structkv_prefill, which return once the device has found the pivot.
  *   - Every call returns a status; invalid arguments are rejected on the host before any
  *     launch.  There is no CPU fallback: an unsupported shape returns
  *     STRUCTKV_ERR_UNSUPPORTED.  Device-side waits are bounded; if one expires the kernel
@@ -51,10 +52,9 @@ typedef enum { STRUCTKV_BF16 = 0, STRUCTKV_FP32 = 1 } structkv_dtype;
 #define STRUCTKV_FLAG_FORCE_SIMT 2u    /* use the CUDA-core scorer even where the tensor-core one applies */
 /* The caller vouches that q_window and k are complete and visible to the device before the call
  * is enqueued: no kernel still in flight on `stream` writes them (they were written before an
- * earlier synchronisation, or on another stream joined through an event).  The first scorer
- * pass then starts reading them while the kernels enqueued before it (the previous layer's
- * column reduction) are still draining; results are identical.  Without the flag the pass
- * waits for everything enqueued before it, as any kernel on a stream does. */
+ * earlier synchronisation, or on another stream joined through an event).  A scorer may then read
+ * them while the kernels enqueued before it are still draining; results are identical.  (The
+ * present scorers set up early but read nothing before that: the flag changes nothing.) */
 #define STRUCTKV_FLAG_INPUTS_READY 4u
 
 typedef struct {
@@ -127,8 +127,8 @@ structkv_status structkv_score_layer(structkv_ctx* ctx, const void* q_window, co
  * (Section 4.1, implementation details: batches whose prompts reach their pivots at different
  * layers are served with a padded addressing mask; every prompt is an independent problem with
  * its own length, statistics, pivot and index sets).  The prompts' keys are packed back to back
- * along the token axis; one launch per scorer pass covers all prompts, each prompt receiving a
- * share of the grid in proportion to its length.  Per prompt the results equal those of
+ * along the token axis; one launch runs both scorer passes over all prompts, each prompt receiving
+ * a share of the tasks in proportion to its length.  Per prompt the results equal those of
  * structkv_score_layer on that prompt alone (same equations: Eq. 1, 2, 3, 4, 5, 6).
  *
  *   q_window      device, [batch, H, w, d] contiguous bf16.
@@ -144,7 +144,7 @@ structkv_status structkv_score_layer(structkv_ctx* ctx, const void* q_window, co
  *   batch_workspace  device, 256-byte aligned, at least
  *                 structkv_batch_workspace_bytes(cfg, batch, total) bytes, caller-owned; calls that
  *                 share it must be ordered by the caller.
- * Served by the tensor-core scorer only (bf16, window 32 / 64 / 128): other configurations
+ * Served by the tensor-core scorer only (bf16, head_dim 64 or 128): other configurations
  * return UNSUPPORTED.  Errors: INVALID_ARG, UNSUPPORTED, WORKSPACE, CUDA.  Asynchronous on `stream`.
  */
 size_t structkv_batch_workspace_bytes(const structkv_config* cfg, int max_batch, long long max_total_tokens);
@@ -174,10 +174,9 @@ structkv_status structkv_select_batch(structkv_ctx* ctx, const float* scores, co
  * Per layer the results are the very bits structkv_score_layer gives with
  * STRUCTKV_FLAG_NO_HEAD_STATS: S^(l), the pooled per-head attention, the layer's entropy; C is
  * carried through all layers (C <- lambda*C + S^(l), l ascending).  What differs is the order of
- * the work: the first scorer pass of layer l+1 is enqueued between the two passes of layer l, and
- * the second pass of layer l waits for a completion counter of its own first pass instead of for
- * the kernel enqueued before it, so no SM idles while the slowest CTA of a pass finishes; the
- * sums over heads of all layers are taken by one launch at the end.
+ * the work: one persistent launch (per 32 layers) runs both scorer passes of all layers, the first
+ * pass ahead of the second, so no SM idles while the slowest CTA of a pass finishes; the sums over
+ * heads of all layers are taken by one launch at the end.
  *
  *   q_windows, ks  HOST arrays [n_layers] of device pointers, laid out as for structkv_score_layer
  *                 (one stride pair serves all layers); every tensor must be complete and visible
