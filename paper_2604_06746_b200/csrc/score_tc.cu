@@ -70,6 +70,34 @@ int clamp_tasks(const Layout& l, int target, int items) {
   return std::min(std::max(target, lo), hi);
 }
 
+// Key segments of pass 1 for a sequence that is due `share` of the SMs: at least two pairs of tiles each, unless
+// all of them run at once anyway.
+int segments(const Layout& l, int share, int tiles, int sms) {
+  const int pairs = (tiles + 1) / 2;
+  return clamp_tasks(l, share, (long long)l.units * pairs <= sms ? pairs : (pairs + 1) / 2);
+}
+int batch_share(const ScoreCall& a, int i, int sms) {
+  return std::max(1, (int)((long long)sms * (a.cu_seqlens[i + 1] - a.cu_seqlens[i]) / a.cu_seqlens[a.n]));
+}
+// How finely a batch's pass 1 is cut: one segment per SM in all (1), or two (2).  A sequence's segments are whole
+// numbers per unit, so with one per SM the longest can be far above the average (40000 + 20000 + 50000
+// + 21072 keys: 39.5 pairs of tiles against 27.8); with two the SMs even out, for one more hand-over
+// (worth a pair) and part of a segment at the end.  Measured with one / two, us: those four 205 / 181, six
+// of 1001 to 12000 keys 84 / 79; but 50000 + 1000 94 / 98 and 30001 + 1500 65 / 71.
+int batch_cut(const Layout& l, const ScoreCall& a, int sms) {
+  if (a.n == 1) return 1;                                  // the bits of the plain call
+  float longest[2] = {0.f, 0.f}, all = 0.f;
+  for (int i = 0; i < a.n; ++i) {
+    const int tiles = (a.cu_seqlens[i + 1] - a.cu_seqlens[i] + kKeyTile - 1) / kKeyTile, pairs = (tiles + 1) / 2;
+    for (int c = 0; c < 2; ++c) {
+      const int per_unit = std::max(1, segments(l, (c + 1) * batch_share(a, i, sms), tiles, sms) * kFullWeight / l.w_total);
+      longest[c] = std::max(longest[c], (float)((pairs + per_unit - 1) / per_unit));
+    }
+    all += (float)pairs * l.w_total / kFullWeight / sms;
+  }
+  return longest[0] <= all + 0.25f * longest[1] + 1.f ? 1 : 2;
+}
+
 template <int MAXP>
 cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n, cudaStream_t st) {
   TcParams<MAXP> p;
@@ -90,6 +118,7 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
     if (!encode3(ctx, &p.map_k[i], a.k[first + i], total_keys, cfg.n_kv_heads, s_tok, s_head, kKeyTile, 1))
       return cudaErrorInvalidValue;
   }
+  const int cut = batch ? batch_cut(l, a, sms) : 1;
   int part0 = 0;
   for (int i = 0; i < n; ++i) {
     TcProblem& pb = p.prob[i];
@@ -104,12 +133,12 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
     pb.inv_c2 = 1.f / pb.c2;
     pb.v_min = -125.f / pb.c2;
     const int tiles = (pb.n_keys + kKeyTile - 1) / kKeyTile;
-    // Pass 1 leaves one partial per key segment: as many segments as SMs, shared out over the sequences of a
-    // batch by their lengths, of at least two pairs of tiles unless all of them run at once anyway.
-    // That depends on the shape alone, so that a layer gives the same bits by itself and among others.
-    const int share = batch ? std::max(1, (int)((long long)sms * pb.n_keys / total_keys)) : sms;
+    // Pass 1 leaves one partial per key segment: as many segments as SMs, or twice as many, shared out over the
+    // sequences of a batch by their lengths.  That depends on the shape alone, so that a layer gives the same
+    // bits by itself and among others.
+    const int share = batch ? batch_share(a, i, sms) : sms;
     const int pairs = (tiles + 1) / 2;
-    pb.s1 = clamp_tasks(l, share, (long long)l.units * pairs <= sms ? pairs : (pairs + 1) / 2);
+    pb.s1 = segments(l, cut * share, tiles, sms);
     // A task by itself runs one segment; with other layers to fill the SMs it runs as many as make five pairs:
     // the way from task to task costs as much as one (32 layers of 5003 keys: 302 us with two pairs a
     // task, 253 with four or more).  The same in pass 2, which leaves no partial results.
@@ -186,7 +215,7 @@ int tc_window_pad(int window) {
 size_t tc_part_tasks(const structkv_config& cfg, int n, bool batch) {
   const size_t units = (size_t)layout_of(cfg).units;
   const size_t m = (size_t)std::min(n, kMaxBatch);
-  return batch ? kMaxSms + 2 * units * m : (kMaxSms + 2 * units) * m;
+  return batch ? 2 * kMaxSms + 2 * units * m : (kMaxSms + 2 * units) * m;
 }
 
 bool tc_supported(const Ctx& ctx, long long k_stride_head, long long k_stride_token) {
