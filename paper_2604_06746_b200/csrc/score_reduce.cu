@@ -335,7 +335,8 @@ __global__ void __launch_bounds__(128) accumulate(const float* __restrict__ s_hi
 }
 
 // Eq. 7-9, then the same recursion.  Every block finds the pivot for itself (one warp, 2 us), so that no
-// launch and no host round trip comes between the metrics and the centrality.
+// launch and no host round trip comes between the metrics and the centrality.  The last block sums
+// nothing: it tells the host, beside the others' sums.
 template <int VEC>
 __global__ void __launch_bounds__(128)
 accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int n_layers, int n, float lambda,
@@ -343,6 +344,7 @@ accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int 
                     volatile int* host, int tag) {
   using T = typename Keys<VEC>::T;
   __shared__ int pivot_s;
+  const bool tells = blockIdx.x == gridDim.x - 1;
   pdl_trigger();
   pdl_wait();
   if (threadIdx.x < 32) {
@@ -351,7 +353,8 @@ accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int 
     double Tl[kPer];
 #pragma unroll
     for (int k = 0; k < kPer; ++k) Tl[k] = 0.0;
-    for (int col = 0; col < 3; ++col) {
+#pragma unroll
+    for (int col = 0; col < 3; ++col) {                    // unrolled: the three chains overlap
       const double sign = col == 0 ? -1.0 : 1.0, w = col == 0 ? weights.x : col == 1 ? weights.y : weights.z;
       double d[kPer], lo = INFINITY, hi = -INFINITY;
       int nan = 0;
@@ -371,11 +374,11 @@ accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int 
         lo = a < lo ? a : lo;
         hi = b > hi ? b : hi;
       }
-      if (__any_sync(0xffffffffu, nan) || !(hi > lo)) continue;
+      const bool usable = !__any_sync(0xffffffffu, nan) && hi > lo;
 #pragma unroll
       for (int k = 0; k < kPer; ++k) {
         const int l = lane + 32 * k;
-        if (l > 0 && l < n_layers)
+        if (usable && l > 0 && l < n_layers)
           Tl[k] = __dadd_rn(Tl[k], __ddiv_rn(__dmul_rn(w, __dsub_rn(d[k], lo)), __dsub_rn(hi, lo)));
       }
     }
@@ -385,7 +388,7 @@ accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int 
     for (int k = 0; k < kPer; ++k) {
       const int l = lane + 32 * k;
       if (l > 0 && l < n_layers && Tl[k] > best) { best = Tl[k]; at = l; }
-      if (blockIdx.x == 0 && l < n_layers) {
+      if (tells && l < n_layers) {
         host[1 + l] = __float_as_int((float)Tl[k]);
         __threadfence_system();
       }
@@ -401,18 +404,19 @@ accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int 
     __syncwarp();
     if (lane == 0) {
       pivot_s = at;
-      if (blockIdx.x == 0) {                           // last: the host polls this word
+      if (tells) {                                     // last: the host polls this word
         __threadfence_system();
         host[0] = tag | at;
       }
     }
   }
+  if (tells) return;
   __syncthreads();
   const int pivot = pivot_s;
   const int j = (blockIdx.x * blockDim.x + threadIdx.x) * VEC;
   if (j >= n) return;
   T c{};
-#pragma unroll 8
+#pragma unroll 16
   for (int l = 0; l <= pivot; ++l) c = decay(lambda, c, *reinterpret_cast<const T*>(s_hist + (size_t)l * row_stride + j));
   *reinterpret_cast<T*>(c_out + j) = c;
 }
@@ -491,9 +495,9 @@ cudaError_t launch_accumulate_at_pivot(const float* s_hist, long long row_stride
                                        int tag, cudaStream_t st) {
   const float3 w = make_float3(weights[0], weights[1], weights[2]);
   if (n % 4 == 0 && row_stride % 4 == 0 && (uintptr_t)s_hist % 16 == 0 && (uintptr_t)c_out % 16 == 0)
-    return launch_pdl(accumulate_at_pivot<4>, dim3((n / 4 + 127) / 128), dim3(128), 0, st, s_hist, row_stride, n_layers, n,
+    return launch_pdl(accumulate_at_pivot<4>, dim3((n / 4 + 127) / 128 + 1), dim3(128), 0, st, s_hist, row_stride, n_layers, n,
                       lambda, metrics, w, l_limit, c_out, (volatile int*)host, tag);
-  return launch_pdl(accumulate_at_pivot<1>, dim3((n + 127) / 128), dim3(128), 0, st, s_hist, row_stride, n_layers, n, lambda,
+  return launch_pdl(accumulate_at_pivot<1>, dim3((n + 127) / 128 + 1), dim3(128), 0, st, s_hist, row_stride, n_layers, n, lambda,
                     metrics, w, l_limit, c_out, (volatile int*)host, tag);
 }
 
