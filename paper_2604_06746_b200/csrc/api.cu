@@ -538,10 +538,21 @@ structkv_status structkv_prefill(structkv_ctx* ctx, const structkv_prefill_args*
     s = structkv_compact_layers(ctx, p->kv_srcs, p->n_layers, p->kv_slab_stride_bytes, p->kv_row_stride_bytes, p->kv_row_bytes,
                                 p->kv_slabs, p->kv_rows, p->i_kv, p->kv_budget, p->kv_budget, p->kv_dst,
                                 p->kv_dst_layer_stride_bytes, stream);
-  if (s == STRUCTKV_OK && p->hidden)
+  // hidden states and 4-byte positions share a launch
+  const bool together = p->hidden && p->positions && p->hidden_dst && p->positions_dst && p->hidden_row_bytes >= 1 &&
+                        p->hidden_row_stride_bytes >= p->hidden_row_bytes && p->position_row_bytes == 4 &&
+                        p->position_row_stride_bytes >= 4 && p->position_row_stride_bytes % 4 == 0 &&
+                        (uintptr_t)p->positions % 4 == 0 && (uintptr_t)p->positions_dst % 4 == 0;
+  if (s == STRUCTKV_OK && together) {
+    const CompactWords words = {p->positions, p->position_row_stride_bytes, p->positions_dst};
+    if (launch_compact(p->hidden, 0, p->hidden_row_stride_bytes, p->hidden_row_bytes, 1, p->n_keys, p->i_struct, 0,
+                       p->struct_budget, p->hidden_dst, ctx->c.ws.status, ctx->c.sm_count, st, &words) != cudaSuccess)
+      s = STRUCTKV_ERR_CUDA;
+  }
+  if (s == STRUCTKV_OK && p->hidden && !together)
     s = structkv_compact(ctx, p->hidden, 0, p->hidden_row_stride_bytes, p->hidden_row_bytes, 1, p->n_keys, p->i_struct,
                          p->struct_budget, p->hidden_dst, stream);
-  if (s == STRUCTKV_OK && p->positions)
+  if (s == STRUCTKV_OK && p->positions && !together)
     s = structkv_compact(ctx, p->positions, 0, p->position_row_stride_bytes, p->position_row_bytes, 1, p->n_keys, p->i_struct,
                          p->struct_budget, p->positions_dst, stream);
   if (on_device) {

@@ -127,10 +127,12 @@ cudaError_t launch_block_scores(const float* scores, long long row_stride, int b
 cudaError_t launch_mass_recovery(const float* scores, long long row_stride, int batch, int n, const int* idx,
                                  int n_idx, float* out, int* status, cudaStream_t st);
 
+// 4-byte rows (aligned) of a second source, gathered by the same list as a compaction of one slab.
+struct CompactWords { const void* src; long long row_stride; void* dst; };
 cudaError_t launch_compact(const void* src, long long slab_stride, long long row_stride,
                            int row_bytes, int n_slabs, int n_rows_src, const int* idx,
                            long long idx_slab_stride, int n_idx, void* dst, int* status, int sm_count,
-                           cudaStream_t st);
+                           cudaStream_t st, const CompactWords* words = nullptr);
 cudaError_t launch_compact_layers(const void* const* srcs, int n_layers, long long slab_stride, long long row_stride,
                                   int row_bytes, int n_slabs, int n_rows_src, const int* idx,
                                   long long idx_layer_stride, int n_idx, void* dst, long long dst_layer_stride,
