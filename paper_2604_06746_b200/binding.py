@@ -105,6 +105,15 @@ class PrefillArgs(ctypes.Structure):
                 ("hidden_row_bytes", _i), ("hidden_dst", _vp), ("positions", _vp), ("position_row_stride_bytes", _ll),
                 ("position_row_bytes", _i), ("positions_dst", _vp)]
 
+    @classmethod
+    def for_layers(cls, n_layers: int) -> "PrefillArgs":
+        """A block whose per-layer arrays exist (``arrays``: q_windows, ks, kv_srcs, scales), nothing filled in."""
+        a = cls()
+        a.n_layers = n_layers
+        a.arrays = (*((_vp * n_layers)() for _ in range(3)), (_f * n_layers)())
+        a.q_windows, a.ks, a.kv_srcs, a.scales = a.arrays
+        return a
+
 
 lib.structkv_prefill.restype = _i
 lib.structkv_prefill.argtypes = [_vp, ctypes.POINTER(PrefillArgs), ctypes.POINTER(_i), ctypes.POINTER(_f), _vp]

@@ -16,6 +16,10 @@ PAPER_LAMBDA = 0.9
 PAPER_WEIGHTS = (0.2, 0.3, 0.5)
 
 
+def _fits(t: torch.Tensor, shape, dtype: torch.dtype) -> bool:
+    return t.shape == shape and t.dtype == dtype and t.is_contiguous()
+
+
 class Prefill:
     def __init__(self, n_layers: int, n_q_heads: int, n_kv_heads: int, head_dim: int, window: int,
                  seq: int, kv_budget: int, struct_budget: int, dtype: torch.dtype,
@@ -193,62 +197,65 @@ class Prefill:
         return self.pivot
 
     def _prefill_args(self, layers, hidden, positions) -> Optional[binding.PrefillArgs]:
-        """The argument block of the one-call path, laid out once per set of tensors (None: not in that form).
-        A block is used again only for the very same tensors at the same addresses."""
-        plan = self._plan
-        if plan is not None and len(layers) == len(plan["layers"]) and hidden is plan["hidden"] and positions is plan["positions"]:
-            for t, (q, k, kv, scale, qp, kp, kvp) in zip(layers, plan["layers"]):
-                if not (t["q_win"] is q and t["k"] is k and t.get("kv") is kv and t["scale"] == scale and q.data_ptr() == qp
-                        and k.data_ptr() == kp and kv.data_ptr() == kvp):
-                    break
-            else:
-                if hidden is None or (hidden.data_ptr(), positions.data_ptr()) == plan["rows"]:
-                    return plan["args"]
-        L = len(layers)
-        if not (self.defer and self.keep_kv and L == self.L and L <= 128 and all("kv" in t for t in layers)
-                and self.flags in (0, binding.FLAG_INPUTS_READY)):
+        """The argument block of the one-call path (None: these tensors are not in that form).  Only the block's own
+        memory is kept: every field is checked and written for every call, so that new tensors, other
+        hyper-parameters and replaced output buffers are seen, and no tensor outlives its call here."""
+        L, N, Hkv, d, dt = len(layers), self.N, self.Hkv, self.d, self.dtype
+        if not (self.defer and self.keep_kv and L == self.L and L <= 128 and self.flags in (0, binding.FLAG_INPUTS_READY)):
             return None
-        k0, kv0 = layers[0]["k"], layers[0]["kv"]
-        if not all(t["k"].shape == k0.shape and t["k"].stride() == k0.stride() and t["kv"].shape == kv0.shape
-                   and t["kv"].stride() == kv0.stride() and t["k"].dtype == t["q_win"].dtype == t["kv"].dtype == self.dtype
-                   and t["q_win"].is_contiguous() for t in layers):
+        k0, kv0 = layers[0]["k"], layers[0].get("kv")
+        if kv0 is None or kv0.shape != (2, Hkv, N, d) or k0.stride(2) != 1 or k0.shape[1] != N:
             return None
-        if k0.stride(2) != 1 or k0.shape[1] != self.N or kv0.shape != (2, self.Hkv, self.N, self.d):
+        k_shape, k_stride, kv_shape, kv_stride = k0.shape, k0.stride(), kv0.shape, kv0.stride()
+        q_ptr, k_ptr, kv_ptr, scales = [], [], [], []
+        for t in layers:
+            q, k, kv = t["q_win"], t["k"], t.get("kv")
+            if (kv is None or k.shape != k_shape or k.stride() != k_stride or kv.shape != kv_shape or kv.stride() != kv_stride
+                    or not k.dtype == q.dtype == kv.dtype == dt or not q.is_contiguous()):
+                return None
+            q_ptr.append(q.data_ptr())
+            k_ptr.append(k.data_ptr())
+            kv_ptr.append(kv.data_ptr())
+            scales.append(t["scale"])
+        f32, i32, rows = torch.float32, torch.int32, self.struct_budget
+        if not (_fits(self.s_hist, (L, N), f32) and _fits(self.head_cols, (L, self.H, N), f32)
+                and _fits(self.metrics, (L, 3), f32) and _fits(self.c_running, (N,), f32) and _fits(self.c_star, (N,), f32)
+                and _fits(self.i_kv, (L, self.kv_budget), i32) and _fits(self.i_struct, (rows,), i32)
+                and _fits(self.kv_out, (L, 2, Hkv, self.kv_budget, d), dt)):
             return None
         if hidden is not None and not (self.hidden_out is not None and hidden.dim() == 2 and hidden.stride(1) == 1
-                                       and hidden.shape == (self.N, self.hidden_out.shape[1])
-                                       and hidden.dtype == self.hidden_out.dtype and positions.dim() == 1
-                                       and positions.shape[0] == self.N and positions.dtype == self.pos_out.dtype):
+                                       and hidden.shape[0] == N and hidden.dtype == self.hidden_out.dtype
+                                       and self.hidden_out.is_contiguous() and self.hidden_out.shape == (rows, hidden.shape[1])
+                                       and positions.dim() == 1 and positions.shape[0] == N and positions.dtype == i32
+                                       and _fits(self.pos_out, (rows,), i32)):
             return None
-        src = self.ctx.layer_sources([t["kv"].view(2 * self.Hkv, self.N, self.d) for t in layers])
+        if Hkv > 1 and kv_stride[0] != Hkv * kv_stride[1]:   # the 2 H_kv slabs have no common stride
+            return None
         if self._layers_ws is None:
-            self._layers_ws = self.ctx.layers_workspace(self.L)
-        vp, f = binding._vp, binding._f
-        a = binding.PrefillArgs()
-        a.n_layers, a.n_keys, a.lam, a.l_limit, a.window = L, self.N, self.lam, self.l_limit, self.w
-        a.q_windows = (vp * L)(*[t["q_win"].data_ptr() for t in layers])
-        a.ks = (vp * L)(*[t["k"].data_ptr() for t in layers])
-        a.scales = (f * L)(*[t["scale"] for t in layers])
-        a.k_stride_head, a.k_stride_token = k0.stride(0), k0.stride(1)
-        a.s_out, a.s_layer_stride, a.c_out = self.s_hist.data_ptr(), self.s_hist.stride(0), self.c_running.data_ptr()
-        a.head_cols, a.head_cols_layer_stride = self.head_cols.data_ptr(), self.head_cols.stride(0)
+            self._layers_ws = self.ctx.layers_workspace(L)
+        if self._plan is None or self._plan.n_layers != L:
+            self._plan = binding.PrefillArgs.for_layers(L)
+        a, es = self._plan, kv0.element_size()
+        for array, values in zip(a.arrays, (q_ptr, k_ptr, kv_ptr, scales)):
+            array[:] = values
+        a.n_keys, a.lam, a.l_limit, a.window = N, self.lam, self.l_limit, self.w
+        a.k_stride_head, a.k_stride_token = k_stride[0], k_stride[1]
+        a.s_out, a.s_layer_stride, a.c_out = self.s_hist.data_ptr(), N, self.c_running.data_ptr()
+        a.head_cols, a.head_cols_layer_stride = self.head_cols.data_ptr(), self.H * N
         a.metrics = self.metrics.data_ptr()
         a.layers_workspace, a.layers_workspace_bytes = self._layers_ws.data_ptr(), self._layers_ws.numel()
-        a.weights = (f * 3)(*self.weights)
-        a.kv_budget, a.struct_budget = self.kv_budget, self.struct_budget
+        a.weights = (binding._f * 3)(*self.weights)
+        a.kv_budget, a.struct_budget = self.kv_budget, rows
         a.i_kv, a.i_struct, a.c_star = self.i_kv.data_ptr(), self.i_struct.data_ptr(), self.c_star.data_ptr()
-        a.kv_srcs = src.ptrs
-        a.kv_slab_stride_bytes, a.kv_row_stride_bytes = src.slab_stride_bytes, src.row_stride_bytes
-        a.kv_row_bytes, a.kv_slabs, a.kv_rows = src.row_bytes, src.n_slabs, src.n_rows
-        a.kv_dst, a.kv_dst_layer_stride_bytes = self.kv_out.data_ptr(), self.kv_out.stride(0) * self.kv_out.element_size()
-        if hidden is not None:
+        a.kv_slab_stride_bytes, a.kv_row_stride_bytes = kv_stride[1 if Hkv > 1 else 0] * es, kv_stride[2] * es
+        a.kv_row_bytes, a.kv_slabs, a.kv_rows = d * es, 2 * Hkv, N
+        a.kv_dst, a.kv_dst_layer_stride_bytes = self.kv_out.data_ptr(), 2 * Hkv * self.kv_budget * d * es
+        if hidden is None:
+            a.hidden = a.hidden_dst = a.positions = a.positions_dst = None
+        else:
             es, ps = hidden.element_size(), positions.element_size()
             a.hidden, a.hidden_row_stride_bytes, a.hidden_row_bytes = hidden.data_ptr(), hidden.stride(0) * es, hidden.shape[1] * es
             a.hidden_dst = self.hidden_out.data_ptr()
             a.positions, a.position_row_stride_bytes, a.position_row_bytes = positions.data_ptr(), positions.stride(0) * ps, ps
             a.positions_dst = self.pos_out.data_ptr()
-        self._plan = {"args": a, "src": src, "hidden": hidden, "positions": positions,
-                      "rows": None if hidden is None else (hidden.data_ptr(), positions.data_ptr()),
-                      "layers": [(t["q_win"], t["k"], t["kv"], t["scale"], t["q_win"].data_ptr(), t["k"].data_ptr(),
-                                  t["kv"].data_ptr()) for t in layers]}
         return a

@@ -1,6 +1,9 @@
 """structkv_pivot_select and structkv_prefill against the separate calls they stand for: the same bits, the
 same pivot and transition scores, also with a cap, without hidden states, with one layer, and when the
 tensors change from call to call."""
+import gc
+import weakref
+
 import pytest
 import torch
 
@@ -80,3 +83,56 @@ def test_pivot_on_the_device_equals_the_host_rule(cuda_device):
                 ctx.accumulate(s, want[0], 0.9, c2)
                 assert torch.equal(c1, c2)
     ctx.close()
+
+
+def prompt(cuda_device, seq, n_layers, budget, shift=0, **more):
+    from paper_2604_06746_b200 import pipeline
+    wl = synth.WORKLOADS["llama32k"].scaled(seq, n_layers=n_layers, n_hubs=6, budgets=(budget,))
+    pl = synth.plan(wl)
+    layers = [synth.make_layer(wl, pl, (l + shift) % n_layers, device=cuda_device) for l in range(n_layers)]
+    hidden = torch.randn((seq, 96), device=cuda_device).to(torch.bfloat16)
+    positions = torch.arange(seq, device=cuda_device, dtype=torch.int32) + shift
+    pf = pipeline.Prefill(wl.n_layers, wl.n_q_heads, wl.n_kv_heads, wl.head_dim, wl.window, wl.seq, budget,
+                          wl.struct_budget(), torch.bfloat16, hidden_dim=96, device=cuda_device, **more)
+    return pf, (layers, hidden, positions)
+
+
+def test_every_run_reads_the_attributes(cuda_device):
+    """Hyper-parameters, flags and output buffers changed between two runs over the very same tensors count for
+    the second one, as they do for a Prefill made with them."""
+    from paper_2604_06746_b200 import binding
+    pf, args = prompt(cuda_device, 2001, 6, 300)
+    pf.run(*args)
+    changes = [dict(weights=(0.0, 0.0, 1.0)), dict(weights=(1.0, 0.0, 0.0)), dict(l_limit=1), dict(lam=0.25),
+               dict(flags=binding.FLAG_FORCE_SIMT), dict(flags=0, l_limit=-1)]
+    now = {}
+    for change in changes:
+        now.update(change)
+        for name, value in change.items():
+            setattr(pf, name, value)
+        fresh, _ = prompt(cuda_device, 2001, 6, 300, **now)
+        pf.run(*args)
+        fresh.run(*args)
+        assert (pf.pivot, pf.transition) == (fresh.pivot, fresh.transition), change
+        for key in OUT + ("hidden_out", "pos_out"):
+            assert torch.equal(getattr(pf, key), getattr(fresh, key)), (change, key)
+    for key in OUT + ("hidden_out", "pos_out"):
+        old = getattr(pf, key)
+        was = old.clone()
+        old.zero_()
+        setattr(pf, key, torch.empty_like(old))
+        pf.run(*args)
+        assert torch.equal(getattr(pf, key), was) and not old.any(), key
+    pf.i_kv = pf.i_kv.long()                              # a buffer that does not fit is refused, not written to
+    with pytest.raises(AssertionError):
+        pf.run(*args)
+
+
+def test_a_finished_run_keeps_no_tensor_of_its_prompt(cuda_device):
+    pf, args = prompt(cuda_device, 1501, 4, 200)
+    pf.run(*args)
+    gone = [weakref.ref(t) for d in args[0] for t in d.values() if torch.is_tensor(t)] + [weakref.ref(t) for t in args[1:]]
+    torch.cuda.synchronize()
+    del args
+    gc.collect()
+    assert not [r() for r in gone if r() is not None]
