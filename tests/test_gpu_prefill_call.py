@@ -136,3 +136,23 @@ def test_a_finished_run_keeps_no_tensor_of_its_prompt(cuda_device):
     del args
     gc.collect()
     assert not [r() for r in gone if r() is not None]
+
+
+def test_the_gather_reads_the_layout_of_every_call(cuda_device):
+    """Head-major and token-major K/V at the same addresses, another output buffer, nothing kept afterwards."""
+    from paper_2604_06746_b200 import pipeline
+    L, Hkv, N, d, budget = 3, 2, 300, 64, 40
+    pf = pipeline.Prefill(L, 4, Hkv, d, 8, N, budget, 80, torch.bfloat16, device=cuda_device)
+    pf.i_kv.copy_(torch.stack([torch.randperm(N, device=cuda_device)[:budget].sort().values for _ in range(L)]))
+    raw = [torch.randn(2 * Hkv * N * d, device=cuda_device).to(torch.bfloat16) for _ in range(L)]
+    views = (lambda x: x.view(2, Hkv, N, d), lambda x: x.view(N, 2, Hkv, d).permute(1, 2, 0, 3))
+    for view in (*views, views[0]):
+        layers = [{"kv": view(x)} for x in raw]
+        pf.kv_out = torch.zeros_like(pf.kv_out)
+        pf.compact_all_kv(layers)
+        for l, t in enumerate(layers):
+            assert torch.equal(pf.kv_out[l], t["kv"][:, :, pf.i_kv[l].long()])
+    gone = [weakref.ref(x) for x in raw]
+    del raw, layers, t, view
+    gc.collect()
+    assert not [r() for r in gone if r() is not None]
