@@ -136,8 +136,8 @@ cudaError_t launch_group_saliency(const float* head_cols, long long col_stride, 
 cudaError_t launch_mass_recovery(const float* scores, long long row_stride, int batch, int n, const int* idx,
                                  int n_idx, float* out, int* status, cudaStream_t st) {
   // a slice below 4096 scores is not worth the exchange
-  if (n <= 4096) return launch_cluster<1>(mass_recovery<1>, batch, 0, st, scores, row_stride, n, idx, n_idx, out, status);
-  return launch_cluster<8>(mass_recovery<8>, batch * 8, 0, st, scores, row_stride, n, idx, n_idx, out, status);
+  if (n <= 4096) return launch_cluster<1>(mass_recovery<1>, dim3(batch), dim3(kRxThreads), 0, st, scores, row_stride, n, idx, n_idx, out, status);
+  return launch_cluster<8>(mass_recovery<8>, dim3(batch * 8), dim3(kRxThreads), 0, st, scores, row_stride, n, idx, n_idx, out, status);
 }
 
 }  // namespace skv

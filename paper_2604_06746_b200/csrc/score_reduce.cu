@@ -1,9 +1,12 @@
 // Small deterministic reductions after the scorers: the sum
 // over heads with the centrality update, per-head sparsity / variance with the layer's metrics, and
 // the closed-form centrality re-accumulation.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
 
 namespace skv {
+namespace cg = cooperative_groups;
 namespace {
 
 // ---- what follows the scorer passes of a layer, of several layers or of a packed batch ----------
@@ -177,58 +180,96 @@ __device__ __forceinline__ void head_done(const FinishArgs& a, int vec, float me
 // L2 together, by reading them twice (1024 vectors of 131072 keys: 2 x 537 MB, 164 us).  One histogram,
 // without copies for the lanes: same-address hits cost less than clearing and summing copies, whether the
 // values concentrate or not (1024 vectors of 5003 / 32768 keys: 41 / 85 us with four, 20 / 59 with one).
-// Eight-bit rank searches over keys in registers, by one CTA or a cluster, took four barriers more and ran
-// in waves (32 vectors of 5003 / 32768 keys 11 / 17 us, now 8 / 12; 128 of 131072 89, now 28).
+//
+// Few long vectors are dealt out over clusters of CL CTAs, which count their own entries; the histograms are
+// read through distributed shared memory, and the first CTA adds up.  An SM's shared-memory atomics bound a CTA
+// (0.16 us per 1000 keys); three cluster barriers and two remote reads of the histogram come to 4 us.
+//
+// The bits of a vector's sums must depend neither on how many threads and CTAs work on it nor on its alignment:
+// entry j belongs to accumulator j mod 1024 ROWS, where ROWS follows from the length alone.  Rows of 1024 are
+// dealt out to the CTAs in turn, and a thread has kAccs of the accumulators.
 constexpr int kSwBins = 2048;
+constexpr int kLongRows = 8;                               // ROWS of a long vector; a short one has a single row
+constexpr int kLongFrom = 32768;                           // keys a short vector has at most
 struct SweepShared {
-  unsigned hist[2][kSwBins];
-  float red[3][33];
-  unsigned scan[33], bin, rem;
+  alignas(16) unsigned hist[2][kSwBins];
+  float red[2][kLongRows][32], red_bin[32];                // sums of the warps, row by row
+  unsigned scan[2][32], bin, rem;                          // [level] sums of the warps, or of 64 bins each
 };
-// The bits of a vector's sums must depend neither on how many threads work on it nor on its alignment: entry j
-// belongs to accumulator j mod 1024, and 512 threads have two each (k = 0 and 1).
-template <int T> constexpr int kStandFor = 1024 / T;
-// Applies f(entry, k) to a[0 .. n) once each, 48 or 64 KB of loads in flight on an SM.
-template <int T, class F>
-__device__ __forceinline__ void sweep_from_memory(const float* __restrict__ a, int n, F f) {
-  constexpr int kAt = T == 1024 ? 16 : 8, odd = kStandFor<T> - 1;
-  int j = threadIdx.x;
+template <int T, int CL, int ROWS> constexpr int kAccs = ROWS == 1 ? 1024 / T : ROWS * 1024 / (T * CL);
+// Applies f(entry, accumulator) to this CTA's entries of a[0 .. n) once each, 48 or 64 KB of loads in flight on an SM.
+template <int T, int CL, int ROWS, class F>
+__device__ __forceinline__ void sweep_from_memory(const float* __restrict__ a, int n, int rank, F f) {
+  constexpr int kAt = T == 1024 ? 16 : 8, kStep = ROWS == 1 ? T : T * CL, kMine = kAccs<T, CL, ROWS>;
+  constexpr int kChunk = kMine > kAt ? kMine : kAt;
+  if (ROWS == 1 && rank > 0) return;
+  int first = rank * T;
   float v[kAt];
-  for (; j - (int)threadIdx.x + kAt * T <= n; j += kAt * T) {
+  for (; first + (kChunk - 1) * kStep + T <= n; first += kChunk * kStep) {
 #pragma unroll
-    for (int u = 0; u < kAt; ++u) v[u] = a[j + u * T];
+    for (int h = 0; h < kChunk; h += kAt) {
 #pragma unroll
-    for (int u = 0; u < kAt; ++u) f(v[u], u & odd);
+      for (int u = 0; u < kAt; ++u) v[u] = a[first + threadIdx.x + (h + u) * kStep];
+#pragma unroll
+      for (int u = 0; u < kAt; ++u) f(v[u], (h + u) & (kMine - 1));
+    }
   }
+  const int j = first + threadIdx.x;
 #pragma unroll
-  for (int u = 0; u < kAt; ++u)
-    if (j + u * T < n) v[u] = a[j + u * T];
+  for (int h = 0; h < kChunk; h += kAt) {
 #pragma unroll
-  for (int u = 0; u < kAt; ++u)
-    if (j + u * T < n) f(v[u], u & odd);
+    for (int u = 0; u < kAt; ++u)
+      if (j + (h + u) * kStep < n) v[u] = a[j + (h + u) * kStep];
+#pragma unroll
+    for (int u = 0; u < kAt; ++u)
+      if (j + (h + u) * kStep < n) f(v[u], (h + u) & (kMine - 1));
+  }
 }
-// Sum of the accumulators over the block, in every thread of warp 0 (fixed order).
-template <int T>
-__device__ __forceinline__ float block_total(const float (&v)[kStandFor<T>], float* red) {
+// Sums of N accumulators over each warp, to the rows they belong to.
+template <int T, int CL, int N>
+__device__ __forceinline__ void warp_sums(const float (&v)[N], float* red, int rank) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int k = 0; k < kStandFor<T>; ++k) {
+  for (int k = 0; k < N; ++k) {
     float s = v[k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) red[k * (T / 32) + warp] = s;
+    if (lane == 0) red[T == 1024 ? (k * CL + rank) * 32 + warp : k * (T / 32) + warp] = s;
   }
-  __syncthreads();
-  float s = 0.f;
-  if (warp == 0) {
-    s = red[lane];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  }
-  return s;
 }
-// Walks the bins of a histogram from the top: s.bin holds the `remaining`-th largest candidate, s.rem is the
-// rank still wanted inside it.
+// `p` in CTA `rank` of the cluster.
+template <int CL, class P>
+__device__ __forceinline__ P* in_cta(P* p, int rank) {
+  return CL > 1 ? cg::this_cluster().map_shared_rank(p, rank) : p;
+}
+template <int CL>
+__device__ __forceinline__ void all_ctas() {
+  if (CL > 1) cg::this_cluster().sync();
+  else __syncthreads();
+}
+template <int CL>
+__device__ __forceinline__ unsigned count_of(unsigned* bin) {
+  unsigned c = 0;
+#pragma unroll
+  for (int r = 0; r < CL; ++r) c += *in_cta<CL>(bin, r);
+  return c;
+}
+// Total over the rows (one warp calls, after all_ctas; fixed order, all loads in flight together).
+template <int CL, int ROWS>
+__device__ __forceinline__ float total_of(float (*red)[32]) {
+  float s[ROWS], total = 0.f;
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r) s[r] = in_cta<CL>(red[r], r % CL)[threadIdx.x];
+#pragma unroll
+  for (int r = 0; r < ROWS; ++r) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s[r] += __shfl_xor_sync(0xffffffffu, s[r], o);
+    total += s[r];
+  }
+  return total;
+}
+// Once all warps have counted: walks the bins of a histogram from the top.  s.bin holds the
+// `remaining`-th largest candidate, s.rem is the rank still wanted inside it.
 template <int T>
 __device__ __forceinline__ void sweep_pick(SweepShared& s, const unsigned* hist, unsigned remaining) {
   constexpr int kPer = kSwBins / T;                        // bins of a thread, higher first
@@ -243,10 +284,10 @@ __device__ __forceinline__ void sweep_pick(SweepShared& s, const unsigned* hist,
     const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += t;
   }
-  if (lane == 31) s.scan[warp] = incl;
+  if (lane == 31) s.scan[0][warp] = incl;
   __syncthreads();
   unsigned before = incl - mine;
-  for (int w = 0; w < warp; ++w) before += s.scan[w];
+  for (int w = 0; w < warp; ++w) before += s.scan[0][w];
   if (before < remaining && remaining <= before + mine) {
 #pragma unroll
     for (int b = 0; b < kPer; ++b) {
@@ -259,41 +300,101 @@ __device__ __forceinline__ void sweep_pick(SweepShared& s, const unsigned* hist,
   }
   __syncthreads();
 }
-template <int T>
-__device__ __forceinline__ void sweep_cta(const FinishArgs& a, SweepShared& s, int vec) {
-  const int tid = threadIdx.x, p = vec / a.H;
-  const Problem pb = problem_of(a, p);
-  const float* x = pb.cols + (size_t)(vec - p * a.H) * a.col_stride;
-  const int n = pb.n;
+// The same for a cluster, in two steps of one warp: 32 groups of 64 bins, summed by their owners before the
+// barrier, then the bins of one group.
+template <int CL>
+__device__ __forceinline__ void cluster_pick(SweepShared& s, int level, unsigned remaining) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned* const hist = s.hist[level];
+  unsigned* const groups = s.scan[level];
+  __syncthreads();
+  const uint2 mine = reinterpret_cast<const uint2*>(hist)[warp * 32 + lane];
+  const unsigned sum = __reduce_add_sync(0xffffffffu, mine.x + mine.y);
+  if (lane == 0) groups[warp] = sum;
+  all_ctas<CL>();
+  if (warp == 0) {
+    // lane l: the l-th of 32 counts from the top; where the wanted rank falls, and the rank inside it
+    auto find = [&](unsigned count, unsigned& rest) {
+      unsigned incl = count;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const unsigned before = incl - count;
+      const int at = __ffs(__ballot_sync(0xffffffffu, before < rest && rest <= incl)) - 1;
+      rest -= __shfl_sync(0xffffffffu, before, at);
+      return at;
+    };
+    unsigned rest = remaining, lo = 0, hi = 0;
+    const int group = 31 - find(count_of<CL>(&groups[31 - lane]), rest);
+    const int pair = 32 * group + 31 - lane;
+#pragma unroll
+    for (int r = 0; r < CL; ++r) {
+      const uint2 c = *in_cta<CL>(reinterpret_cast<uint2*>(hist) + pair, r);
+      lo += c.x;
+      hi += c.y;
+    }
+    const int at = find(lo + hi, rest);
+    if (lane == at) {
+      s.bin = (unsigned)(2 * pair) + (rest <= hi ? 1u : 0u);
+      s.rem = rest <= hi ? rest : rest - hi;
+    }
+  }
+  __syncthreads();
+}
+template <int T, int CL, int ROWS>
+__device__ __forceinline__ void sweep_cta(const FinishArgs& a, SweepShared& s, const Problem& pb, int vec) {
+  const int tid = threadIdx.x, rank = CL > 1 ? (int)(blockIdx.x % CL) : 0, n = pb.n;
+  const float* x = pb.cols + (size_t)(vec % a.H) * a.col_stride;
   const float mean = 1.f / (float)n;
-  float sq[kStandFor<T>] = {}, mass[kStandFor<T>] = {}, in_bin[kStandFor<T>] = {};
-  sweep_from_memory<T>(x, n, [&](float v, int k) {
+  auto pick = [&](int level, unsigned remaining) {
+    if (CL > 1) cluster_pick<CL>(s, level, remaining);
+    else sweep_pick<T>(s, s.hist[level], remaining);
+  };
+  float acc[kAccs<T, CL, ROWS>] = {};
+  sweep_from_memory<T, CL, ROWS>(x, n, rank, [&](float v, int k) {
     const float dv = v - mean;
-    sq[k] = fmaf(dv, dv, sq[k]);
+    acc[k] = fmaf(dv, dv, acc[k]);
     atomicAdd(&s.hist[0][(__float_as_uint(v) >> 20) & 0x7ffu], 1u);
   });
-  sweep_pick<T>(s, s.hist[0], (unsigned)max(1, n / 10));
+  if (ROWS > 1 || rank == 0) warp_sums<T, CL>(acc, s.red[0][0], rank);
+  pick(0, (unsigned)max(1, n / 10));
   const unsigned b1 = s.bin, rem1 = s.rem;
-  sweep_from_memory<T>(x, n, [&](float v, int k) {
+#pragma unroll
+  for (float& m : acc) m = 0.f;
+  sweep_from_memory<T, CL, ROWS>(x, n, rank, [&](float v, int k) {
     const unsigned u = __float_as_uint(v), top = (u >> 20) & 0x7ffu;
-    if (top > b1) mass[k] += v;
+    if (top > b1) acc[k] += v;
     else if (top == b1) atomicAdd(&s.hist[1][(u >> 9) & 0x7ffu], 1u);
   });
-  sweep_pick<T>(s, s.hist[1], rem1);
-  // entries of the threshold bin above sub-bin b2, and rem2 entries of sub-bin b2 itself
-  const unsigned b2 = s.bin, rem2 = s.rem;
+  if (ROWS > 1 || rank == 0) warp_sums<T, CL>(acc, s.red[1][0], rank);
+  pick(1, rem1);
+  if (rank == 0) {
+    // entries of the threshold bin above sub-bin b2, and rem2 entries of sub-bin b2 itself
+    const unsigned b2 = s.bin, rem2 = s.rem;
+    constexpr int kAccsBin = 1024 / T;
+    float in_bin[kAccsBin] = {};
 #pragma unroll
-  for (int q = 0; q < kSwBins / T; ++q) {
-    const int b = q * T + tid;
-    const float mid = __uint_as_float((b1 << 20) | ((unsigned)b << 9) | 0x100u);
-    const unsigned cnt = (unsigned)b > b2 ? s.hist[1][b] : ((unsigned)b == b2 ? rem2 : 0u);
-    float& to = in_bin[q & (kStandFor<T> - 1)];
-    to = fmaf((float)cnt, mid, to);
+    for (int q = 0; q < kSwBins / T; ++q) {
+      const int b = q * T + tid;
+      const float mid = __uint_as_float((b1 << 20) | ((unsigned)b << 9) | 0x100u);
+      const unsigned cnt = (unsigned)b > b2 ? count_of<CL>(&s.hist[1][b]) : ((unsigned)b == b2 ? rem2 : 0u);
+      float& to = in_bin[q & (kAccsBin - 1)];
+      to = fmaf((float)cnt, mid, to);
+    }
+    warp_sums<T, 1>(in_bin, s.red_bin, 0);
+    __syncthreads();
+    if (tid < 32) {
+      const float sq = total_of<CL, ROWS>(s.red[0]), mass = total_of<CL, ROWS>(s.red[1]);
+      head_done(a, vec, mean, sq, mass + total_of<1, 1>(&s.red_bin));
+    }
   }
-  const float sq_t = block_total<T>(sq, s.red[0]), mass_t = block_total<T>(mass, s.red[1]), in_t = block_total<T>(in_bin, s.red[2]);
-  if (tid < 32) head_done(a, vec, mean, sq_t, mass_t + in_t);
+  if (CL > 1) all_ctas<CL>();                              // no CTA leaves while the first one reads its memory
 }
-template <int VEC, int T>
+// LONG: some vector has more than kLongFrom keys.  Short ones have a kernel of their own: with both forms in one
+// kernel a launch over 32 vectors of 4096 keys took a microsecond longer.
+template <int VEC, int T, int CL, bool LONG>
 __global__ void __launch_bounds__(T, T == 512 ? 3 : 1) finish(const __grid_constant__ FinishArgs a) {
   __shared__ union { SweepShared stats; SumShared<VEC> sum; } sh;
   const bool stats = (int)blockIdx.x < a.n_stat_ctas;
@@ -303,10 +404,13 @@ __global__ void __launch_bounds__(T, T == 512 ? 3 : 1) finish(const __grid_const
   pdl_wait();
   __syncthreads();
   if (stats) {
-    sweep_cta<T>(a, sh.stats, blockIdx.x);
+    const int vec = blockIdx.x / CL;
+    const Problem pb = problem_of(a, vec / a.H);
+    if (LONG && pb.n > kLongFrom) sweep_cta<T, CL, kLongRows>(a, sh.stats, pb, vec);
+    else sweep_cta<T, CL, 1>(a, sh.stats, pb, vec);
   } else {
     const int b = blockIdx.x - a.n_stat_ctas, p = b / a.chunks;
-    sum_block<VEC, T>(a, sh.sum, p, b - p * a.chunks);
+    if (p < a.n_prob) sum_block<VEC, T>(a, sh.sum, p, b - p * a.chunks);   // the grid is whole clusters
   }
 }
 constexpr int kSumThreads = 256;     // many short blocks: 16 loads in flight per thread
@@ -430,11 +534,22 @@ static cudaError_t launch_finish(FinishArgs& a, int longest, int sms, cudaStream
   if (!a.with_stats) return launch_pdl(sum_layers<VEC>, dim3(sums), dim3(kSumThreads), 0, st, a);
   // An SM per vector: as many threads as a CTA can have.  More vectors than SMs: three CTAs an SM fill each
   // other's gaps between barriers (512 vectors of 5003 / 32768 keys: 26 / 41 us with one of 1024 threads an
-  // SM, 15 / 31 with three of 512).
-  a.n_stat_ctas = a.n_prob * a.H;
-  const dim3 grid(a.n_stat_ctas + sums);
-  if (a.n_stat_ctas <= sms) return launch_pdl(finish<VEC, 1024>, grid, dim3(1024), 0, st, a);
-  return launch_pdl(finish<VEC, 512>, grid, dim3(512), 0, st, a);
+  // SM, 15 / 31 with three of 512).  Few long vectors: clusters, as large as leaves room for all of them at once.
+  // us with one CTA / with clusters: 32 vectors of 33000 / 65536 / 131072 / 262144 keys 12.5, 10.5 / 17.5, 12.5 / 27.2,
+  // 15.1 / 46.2, 20.1; 8 of 262144 46, 15; 64 of 262144 46, 29.  A cluster needs its SMs free in one GPC: of
+  // eight CTAs 15 run at once (16 vectors of 262144 keys: 27.6), of four 32, of two 64.
+  const int n_vec = a.n_prob * a.H, room = longest > kLongFrom ? sms * 7 / 8 / n_vec : 1;
+  const int cl = 8 * n_vec <= sms * 3 / 4 && room >= 8 ? 8 : room >= 4 ? 4 : room >= 2 ? 2 : 1;
+  a.n_stat_ctas = n_vec * cl;
+  const dim3 grid((a.n_stat_ctas + sums + cl - 1) / cl * cl), wide(1024), narrow(512);
+  if (cl == 8) return launch_cluster<8>(finish<VEC, 1024, 8, true>, grid, wide, 0, st, a);
+  if (cl == 4) return launch_cluster<4>(finish<VEC, 1024, 4, true>, grid, wide, 0, st, a);
+  if (cl == 2) return launch_cluster<2>(finish<VEC, 1024, 2, true>, grid, wide, 0, st, a);
+  if (longest > kLongFrom)
+    return n_vec <= sms ? launch_pdl(finish<VEC, 1024, 1, true>, grid, wide, 0, st, a)
+                        : launch_pdl(finish<VEC, 512, 1, true>, grid, narrow, 0, st, a);
+  return n_vec <= sms ? launch_pdl(finish<VEC, 1024, 1, false>, grid, wide, 0, st, a)
+                      : launch_pdl(finish<VEC, 512, 1, false>, grid, narrow, 0, st, a);
 }
 
 static FinishArgs finish_args(const Ctx& ctx, const float* cols, long long col_stride, int n, float* metrics) {

@@ -176,7 +176,8 @@ cudaError_t launch(const SelectArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     ready.fetch_or(bit, std::memory_order_release);
   }
-  return launch_cluster<CL>(select_topk<CL, ITEMS>, (a.batch + (a.extra.scores ? 1 : 0)) * CL, sizeof(RadixShared<CL>), st, a);
+  return launch_cluster<CL>(select_topk<CL, ITEMS>, dim3((a.batch + (a.extra.scores ? 1 : 0)) * CL), dim3(kRxThreads),
+                            sizeof(RadixShared<CL>), st, a);
 }
 
 // The smallest cluster and the fewest items per thread that hold a vector, as measured (us for 1 / 32
