@@ -201,6 +201,11 @@ __device__ __forceinline__ uint64_t l2_policy_evict_last() {
   asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
   return p;
 }
+__device__ __forceinline__ uint64_t l2_policy_evict_normal() {
+  uint64_t p;
+  asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
+  return p;
+}
 __device__ __forceinline__ uint64_t l2_policy_evict_first() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
@@ -374,11 +379,14 @@ __device__ __forceinline__ uint64_t exp2_sfu2(uint64_t x) {
 #endif
 __host__ __device__ constexpr bool poly1(int pr) { return (SKV_POLY1 >> (pr & 15)) & 1; }
 __host__ __device__ constexpr bool poly2(int pr) { return (SKV_POLY2 >> (pr & 15)) & 1; }
-// Percentage of a problem's keys (its end) that pass 1 asks L2 to keep for pass 2, which walks
-// backwards.
-#ifndef SKV_L2_KEEP_PCT
-#define SKV_L2_KEEP_PCT 20
-#endif
+// Percentage of a problem's keys (its end) that pass 1 asks L2 to keep for pass 2, which walks backwards; the
+// other keys make room first.  Whole prefills of 32768 keys, us, with nothing kept / with this: window 64
+// 1727 / 1714, window 8 1009 / 991.
+// Several row blocks of a KV group read the same keys one after the other, so among other layers none of
+// them makes room first.  us with the hints / without: 16 layers of 65536 keys in two blocks 1418 / 1386, in four
+// 2625 / 2545; 28 of 20001 1453 / 1428, of 5003 418 / 416; but 20 of 2048 105 / 108, and one layer of 131072
+// 326 / 331.
+constexpr int kL2KeepPct = 20, kL2PlainFrom = 4096;
 
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of 128 bytes, 8-row
 // groups 1024 bytes apart (the layout TMA writes with CU_TENSOR_MAP_SWIZZLE_128B).
@@ -665,7 +673,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
   if (warp == 0) {
     // ---------------- ticket taker and TMA producer ----------------
     if (lane == 0) {
-      const uint64_t pol_keep = l2_policy_evict_last(), pol_stream = l2_policy_evict_first();
+      const uint64_t pol_keep = l2_policy_evict_last(), pol_stream = l2_policy_evict_first(), pol_plain = l2_policy_evict_normal();
       int* const ticket = p.ctl + kCtlTicket;
       const int n_tickets = p.phase[p.n_phase].first;
       int tk = atomicAdd(ticket, 1), ph = 0;
@@ -727,7 +735,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         if (t.pass == 0) break;
         const TcProblem& pb = p.prob[t.prob];
         const int n_tiles = (pb.n_keys + kKeyTile - 1) / kKeyTile;
-        const int keep_from = t.pass == 1 ? n_tiles - (n_tiles * SKV_L2_KEEP_PCT) / 100 : n_tiles;
+        const bool plain = p.n_rb > 1 && !p.hurry && pb.n_keys >= kL2PlainFrom;
+        const int keep_from = t.pass == 1 && !plain ? n_tiles - (n_tiles * kL2KeepPct) / 100 : n_tiles;
         bool ok = true;
         for (int it = 0; it < items_of(t) && ok; ++it) {
           for (int half = 0; half < 2; ++half, ++st) {
@@ -745,7 +754,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
             // sequence of a packed batch): the causal mask discards those keys
             for (int c = 0; c < L::kSub; ++c)
               tma_load_3d_hint(base + L::kKOff + (c * kStages + sg) * L::kKSub, &p.map_k[pb.map], bar(kBarFull + sg),
-                               c * 64, pb.key0 + tile * kKeyTile, g, tile >= keep_from ? pol_keep : pol_stream);
+                               c * 64, pb.key0 + tile * kKeyTile, g, tile >= keep_from ? pol_keep : plain ? pol_plain : pol_stream);
           }
           if (it == 0 && ok) {
             // The Q block, behind the first keys, in halves: each waits for the previous task's MMAs on it,
