@@ -8,22 +8,11 @@
 namespace skv {
 namespace {
 
-#ifndef SKV_CP_THREADS
-#define SKV_CP_THREADS 256
-#endif
-#ifndef SKV_CP_UNROLL
-#define SKV_CP_UNROLL 2
-#endif
-#ifndef SKV_CP_BLOCKS_PER_SM
-#define SKV_CP_BLOCKS_PER_SM 64
-#endif
-constexpr int kCpThreads = SKV_CP_THREADS;
-constexpr int kCpUnroll = SKV_CP_UNROLL;
+constexpr int kCpThreads = 256, kCpUnroll = 2, kCpBlocksPerSm = 64;
 
 // Rows are read once and written once: loads bypass L1 allocation, stores are streaming.
 template <typename V> __device__ __forceinline__ V ld_stream(const V* p) { return *p; }
 template <typename V> __device__ __forceinline__ void st_stream(V* p, const V& v) { *p = v; }
-#ifndef SKV_CP_PLAIN
 template <> __device__ __forceinline__ uint4 ld_stream<uint4>(const uint4* p) {
   uint4 v;
   asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0, %1, %2, %3}, [%4];"
@@ -33,7 +22,6 @@ template <> __device__ __forceinline__ uint4 ld_stream<uint4>(const uint4* p) {
 template <> __device__ __forceinline__ void st_stream<uint4>(uint4* p, const uint4& v) {
   asm volatile("st.global.cs.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
-#endif
 
 // Block 0 .. blocks - 1 of a gather.
 template <typename V>
@@ -174,7 +162,7 @@ cudaError_t launch_compact_layers(const void* const* srcs, int n_layers, long lo
   const int upr = row_bytes / unit;
   const long long total = (long long)n_slabs * n_idx * upr;
   long long blocks = (total + (long long)kCpThreads * kCpUnroll - 1) / ((long long)kCpThreads * kCpUnroll);
-  const long long cap = ((long long)sm_count * SKV_CP_BLOCKS_PER_SM + n_layers - 1) / n_layers;
+  const long long cap = ((long long)sm_count * kCpBlocksPerSm + n_layers - 1) / n_layers;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
   const dim3 grid((unsigned)blocks, (unsigned)n_layers);
@@ -197,7 +185,7 @@ cudaError_t launch_compact(const void* src, long long slab_stride, long long row
   const int upr = row_bytes / unit;
   const long long total = (long long)n_slabs * n_idx * upr;
   long long blocks = (total + (long long)kCpThreads * kCpUnroll - 1) / ((long long)kCpThreads * kCpUnroll);
-  const long long cap = (long long)sm_count * SKV_CP_BLOCKS_PER_SM;
+  const long long cap = (long long)sm_count * kCpBlocksPerSm;
   if (blocks > cap) blocks = cap;
   if (blocks < 1) blocks = 1;
   const char* s = (const char*)src;

@@ -134,18 +134,16 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
       : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
   return ok != 0;
 }
-// Same test, letting the hardware suspend the thread for up to `ns` nanoseconds while the phase
+// Same test, letting the hardware suspend the thread for up to kSuspendNs while the phase
 // is incomplete: a waiting producer then issues (almost) no instructions on its scheduler.
-#ifndef SKV_WAIT_HINT_NS
-#define SKV_WAIT_HINT_NS 1000
-#endif
+constexpr uint32_t kSuspendNs = 1000;
 __device__ __forceinline__ bool mbar_try_suspend(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n.reg .pred p;\n"
       "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
       "selp.u32 %0, 1, 0, p;\n}"
-      : "=r"(ok) : "r"(bar), "r"(parity), "r"((uint32_t)SKV_WAIT_HINT_NS) : "memory");
+      : "=r"(ok) : "r"(bar), "r"(parity), "r"(kSuspendNs) : "memory");
   return ok != 0;
 }
 // Bounded wait of a producer (TMA / MMA warp): long, rarely latency critical.
@@ -156,7 +154,7 @@ __device__ __forceinline__ bool mbar_wait_producer(uint32_t bar, uint32_t parity
   for (;;) {
 #pragma unroll 1
     for (int i = 0; i < 16; ++i)
-      if (SKV_WAIT_HINT_NS > 0 ? mbar_try_suspend(bar, parity) : mbar_try(bar, parity)) return true;
+      if (mbar_try_suspend(bar, parity)) return true;
     if (*abort_flag) return false;
     if ((unsigned long long)(clock64() - t0) > limit) { *abort_flag = 1; return false; }
   }
@@ -371,14 +369,8 @@ __device__ __forceinline__ uint64_t exp2_sfu2(uint64_t x) {
 // inside the kernel, where every instruction beside the arithmetic takes issue slots from it, the
 // shares below are the best at the power cap (128K keys, us per pass-1 / pass-2 task: 80.6 / 71.2
 // with 2 and 4 pairs, 85.0 / 70.0 with 0 and 5, 81.1 / 73.4 with 3 and 6).
-#ifndef SKV_POLY1
-#define SKV_POLY1 0x0101
-#endif
-#ifndef SKV_POLY2
-#define SKV_POLY2 0x1111
-#endif
-__host__ __device__ constexpr bool poly1(int pr) { return (SKV_POLY1 >> (pr & 15)) & 1; }
-__host__ __device__ constexpr bool poly2(int pr) { return (SKV_POLY2 >> (pr & 15)) & 1; }
+__host__ __device__ constexpr bool poly1(int pr) { return pr % 8 == 0; }
+__host__ __device__ constexpr bool poly2(int pr) { return pr % 4 == 0; }
 // Percentage of a problem's keys (its end) that pass 1 asks L2 to keep for pass 2, which walks backwards; the
 // other keys make room first.  Whole prefills of 32768 keys, us, with nothing kept / with this: window 64
 // 1727 / 1714, window 8 1009 / 991.
