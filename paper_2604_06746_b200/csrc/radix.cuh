@@ -1,12 +1,10 @@
-// Rank search over fp32 keys held in registers, shared by the token selection and the head
-// statistics.  A cluster of CL CTAs of kRxThreads threads shares one vector; digits of eight bits from
-// the top.  Each level: every lane counts into histogram copies of its own (bank = lane, so a warp's
-// hits never collide, however concentrated the digit), a warp sums the copies of a bin with one
-// reduction instruction, the 256 counts go to every CTA of the cluster in coalesced copies, and every
-// warp walks them on its own.  Two block barriers and one exchange per level; one pass over memory in
-// all where the vector fits the registers.  (Before: 2048-bin histograms with eight copies merged in
-// CTA 0 by remote atomics, a serial walk over warp totals and a sweep of memory per level: 21 us
-// for any short vector, 35 us for a layer's head statistics.)
+// Rank search over fp32 keys held in registers (token selection).  A cluster of CL CTAs of kRxThreads threads
+// shares one vector; digits of eight bits from the top.  Each level: every lane counts into histogram copies
+// of its own (bank = lane, so a warp's hits never collide, however concentrated the digit), a warp sums the
+// copies of a bin with one reduction instruction, the 256 counts go to every CTA of the cluster in
+// coalesced copies, and every warp walks them on its own.  Two block barriers and one exchange per level; one
+// pass over memory in all where the vector fits the registers.  (2048-bin histograms with eight copies
+// merged in CTA 0 by remote atomics and a sweep of memory per level took 21 us for any short vector.)
 #pragma once
 
 #include <cooperative_groups.h>
@@ -26,7 +24,6 @@ struct RadixShared {
   unsigned cnt[2][CL][256];            // counts of every CTA of the cluster
   unsigned mine[256];                  // this CTA's, before the exchange
   unsigned scratch[2 * kRxThreads];    // block reductions, output offsets
-  float red[4][33];
 };
 
 template <int CL>

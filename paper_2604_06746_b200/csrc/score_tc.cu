@@ -157,7 +157,7 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
   // ticket order
   int n_ph = 0, tickets = 0;
   auto phase = [&](int i, int pass) {
-    p.phase[n_ph++] = TcPhase{tickets, 0, (unsigned char)i, (unsigned char)pass};
+    p.phase[n_ph++] = TcPhase{tickets, (unsigned char)i, (unsigned char)pass};
     tickets += pass == 1 ? p.prob[i].t1 : p.prob[i].t2;
   };
   if (batch) {
@@ -174,7 +174,7 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
       if (i >= ahead) phase(i - ahead, 2);
     }
   }
-  p.phase[n_ph] = TcPhase{tickets, 0, 0, 0};
+  p.phase[n_ph] = TcPhase{tickets, 0, 0};
   p.n_phase = n_ph;
   p.n_prob = n;
   p.window = cfg.window;

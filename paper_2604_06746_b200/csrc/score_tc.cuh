@@ -77,8 +77,8 @@ struct TcProblem {
   int negate;                          // the scale is negative: the MMA negates its A operand
   int s1, t1, t2, part0;               // key segments of pass 1, tasks of the two passes; first partial of pass 1
 };
-// A run of consecutive tickets: tasks [task0, ...) of one pass of one problem.
-struct TcPhase { int first; unsigned short task0; unsigned char prob, pass; };
+// A run of consecutive tickets, from `first` on: the tasks of one pass of one problem.
+struct TcPhase { int first; unsigned char prob, pass; };
 
 template <int MAXP>
 struct alignas(64) TcParams {
@@ -682,7 +682,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
           t.group = p.group;
           const TcProblem& pb = p.prob[t.prob];
           const int tasks = t.pass == 1 ? pb.t1 : pb.t2;
-          int i = p.phase[ph].task0 + tk - p.phase[ph].first;
+          int i = tk - p.phase[ph].first;
           if (t.pass == 2) i = tasks - 1 - i;              // pass 2 starts with the keys pass 1 touched last
           // the unit whose share [tc_deal(W), tc_deal(W + w)) holds task i
           const int w_at = ((i + 1) * p.w_total - 1) / tasks;
