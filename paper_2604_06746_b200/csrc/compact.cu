@@ -107,38 +107,8 @@ gather_rows_layers(const __grid_constant__ LayerPtrs srcs, long long slab_stride
   pdl_trigger();
   pdl_wait();
   const int layer = blockIdx.y;
-  const char* __restrict__ src = srcs.src[layer];
-  const int* __restrict__ my_idx = idx + (long long)layer * idx_layer_stride;
-  char* __restrict__ my_dst = dst + (long long)layer * dst_layer_stride;
-  const long long total = (long long)n_slabs * n_idx * units_per_row;
-  const long long stride = (long long)gridDim.x * kCpThreads;
-  for (long long u0 = (long long)blockIdx.x * kCpThreads + threadIdx.x; u0 < total; u0 += stride * kCpUnroll) {
-    V val[kCpUnroll];
-    bool ok[kCpUnroll];
-#pragma unroll
-    for (int e = 0; e < kCpUnroll; ++e) {
-      const long long u = u0 + e * stride;
-      ok[e] = false;
-      if (u < total) {
-        const long long row = u / units_per_row;           // s * n_idx + r
-        const int c = (int)(u - row * units_per_row);
-        const int s = (int)(row / n_idx), r = (int)(row - (long long)s * n_idx);
-        const int j = __ldg(my_idx + r);
-        if (j >= 0 && j < n_rows_src) {
-          val[e] = ld_stream(reinterpret_cast<const V*>(src + s * slab_stride + j * row_stride +
-                                                        (long long)c * sizeof(V)));
-          ok[e] = true;
-        } else if (c == 0) {
-          atomicCAS(status, 0, (int)STRUCTKV_ERR_INVALID_ARG);
-        }
-      }
-    }
-#pragma unroll
-    for (int e = 0; e < kCpUnroll; ++e) {
-      const long long u = u0 + e * stride;
-      if (ok[e]) st_stream(reinterpret_cast<V*>(my_dst + u * (long long)sizeof(V)), val[e]);
-    }
-  }
+  gather_blocks<V>(gridDim.x, srcs.src[layer], slab_stride, row_stride, units_per_row, n_slabs, n_rows_src,
+                   idx + (long long)layer * idx_layer_stride, 0, n_idx, dst + (long long)layer * dst_layer_stride, status);
 }
 
 }  // namespace
