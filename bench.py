@@ -36,13 +36,11 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 SM_COUNT = 148
 SFU_EXP_PER_CLK_PER_SM = 16      # special-function results per clock per SM (cc 10.0 arithmetic-throughput table)
 
-# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the scorer launches of one layer,
-# from an ncu capture of the current kernels; None = no capture of the current kernels exists.
-NCU_TRAFFIC_BYTES_PER_LAYER = 549.0e6
-NCU_TRAFFIC_NOTE = ("dram read + write of the two tc_score launches of one layer (llama128k shape), single-metric "
-                    "ncu captures with the caches left as the previous kernel leaves them: pass 1 reads 269 MB, "
-                    "pass 2 252 MB when the next layer's pass 1 ran in between (every layer but the last; 218 MB "
-                    "otherwise: it starts with the tiles pass 1 asked L2 to keep), 28 + 1 MB written")
+# DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the scorer for one layer, from an ncu
+# capture of the current kernel (profiles/tc_score_llama128k_ncu.md); None = there is none.
+NCU_TRAFFIC_BYTES_PER_LAYER = 505.9e6
+NCU_TRAFFIC_NOTE = ("half of the dram read + write of the tc_score launch over two layers (llama128k shape): 1007 MB read, "
+                    "4.6 MB written; each layer's K is 268 MB and is read by both passes")
 
 
 def load_peaks():
@@ -749,7 +747,7 @@ def main():
     roof = scorer_roofline(wl, phase_ms["score"] / n_timed, peaks, sm_mhz)
     roof["traffic"] = NCU_TRAFFIC_BYTES_PER_LAYER if wl.name.startswith("llama128k") else None
     roof["traffic_note"] = NCU_TRAFFIC_NOTE
-    roof["kernel"] = "structkv_score_layer (both scorer passes + reductions), per layer"
+    roof["kernel"] = "structkv_score_layers (both scorer passes + reductions), per layer"
     roof["peaks"] = peaks["source"]
     if sm_mhz:
         roof["us_per_layer_x_sm_mhz"] = roof["us_per_layer"] * sm_mhz

@@ -237,7 +237,7 @@ structkv_status structkv_head_stats(structkv_ctx* ctx, const float* head_cols, l
  *
  * Limit: the configuration must satisfy
  *     0 < structkv_workspace_bytes(cfg) <= STRUCTKV_STATIC_SCRATCH_BYTES
- * (a Llama-3-8B shape, 32 query heads, window 64, fits up to max_seq = 16384).  A larger
+ * (a Llama-3-8B shape, 32 query heads, window 64, fits up to max_seq = 56064).  A larger
  * configuration is refused with STRUCTKV_ERR_WORKSPACE before anything is launched.
  *
  * Set-up: the first call on each device (with that device current) resolves the device

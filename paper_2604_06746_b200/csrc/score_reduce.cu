@@ -10,7 +10,7 @@ namespace cg = cooperative_groups;
 namespace {
 
 // ---- what follows the scorer passes of a layer, of several layers or of a packed batch ----------
-// One launch: one CTA per (problem, head) vector first (Eq. 5-6), then blocks that sum 128 x VEC keys over
+// One launch: a CTA or a cluster per (problem, head) vector first (Eq. 5-6), then blocks that sum 128 x VEC keys over
 // the heads (Eq. 2) and carry the centrality (Eq. 3).  Every sum has a fixed order.
 struct FinishArgs {
   const float* cols;                   // problem p, head h, key j at cols + p * layer_stride + h * col_stride + j
@@ -166,7 +166,7 @@ __device__ __forceinline__ void head_done(const FinishArgs& a, int vec, float me
   }
 }
 
-// Eq. 5 and 6 of one (problem, head) vector by one CTA, in two sweeps over memory: the sum of squared
+// Eq. 5 and 6 of one (problem, head) vector by a CTA or a cluster, in two sweeps over memory: the sum of squared
 // deviations from 1/n (the pooled vector sums to 1, so 1/n is its mean; summing deviations instead of
 // squares keeps near-uniform attention from cancelling) and the mass of the floor(n / 10) largest entries.
 // Counting sweeps locate the k-th largest value to 22 bits (all entries are >= 0: the order of the bit
@@ -177,7 +177,7 @@ __device__ __forceinline__ void head_done(const FinishArgs& a, int vec, float me
 // level are 2^-14 wide relative to their value, far inside the metric's tolerance.
 //
 // Bound by latency up to some 100 vectors, then by the shared-memory atomics and, where the vectors exceed
-// L2 together, by reading them twice (1024 vectors of 131072 keys: 2 x 537 MB, 164 us).  One histogram,
+// L2 together, by reading them twice (1024 vectors of 131072 keys: 2 x 537 MB, 164 of 208 us).  One histogram,
 // without copies for the lanes: same-address hits cost less than clearing and summing copies, whether the
 // values concentrate or not (1024 vectors of 5003 / 32768 keys: 41 / 85 us with four, 20 / 59 with one).
 //
