@@ -8,7 +8,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libstructkv.so")
 SOURCES = ["api.cu", "score_simt.cu", "score_tc.cu", "score_tc_d64_one.cu",
-           "score_tc_d64_many.cu", "score_tc_d128_one.cu", "score_tc_d128_many.cu", "score_reduce.cu", "select.cu", "compact.cu", "aggregate.cu"]
+           "score_tc_d64_many.cu", "score_tc_d128_one.cu", "score_tc_d128_many.cu", "score_res.cu",
+           "score_res_d64.cu", "score_res_d128.cu", "score_reduce.cu", "select.cu", "compact.cu", "aggregate.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fno-gnu-unique", "-Wno-deprecated-gpu-targets"]
 

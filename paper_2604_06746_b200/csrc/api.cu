@@ -50,6 +50,7 @@ Workspace carve_workspace(const structkv_config& cfg, void* base) {
   w.ctl = (int*)take(kCtlInts * sizeof(int));
   w.stat_ctr = (int*)take(kMaxStatLayers * sizeof(int));
   w.chunk_ctr = (int*)take(n_pad / kKeyTile * sizeof(int));
+  w.xch = (unsigned long long*)take(kXchWords * sizeof(unsigned long long));
   w.zero_bytes = off;
   w.row_part = (float2*)take(std::max(simt_part_entries(cfg, 1), tc_part_tasks(cfg, 1, false) * kRowBlock) * sizeof(float2));
   w.row_lse2 = (float*)take(rows_pad * sizeof(float));

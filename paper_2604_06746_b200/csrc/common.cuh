@@ -18,6 +18,8 @@ constexpr int kMaxStatLayers = 128;   // layers one batched head-statistics call
 constexpr int kMaxGatherLayers = 128; // layers one multi-layer gather may cover (their pointers are a kernel argument)
 constexpr int kQueueUnits = 256;      // (KV group, row block) units of one problem the tensor-core scorer can hold
 constexpr int kCtlInts = 64 + 2 * kMaxBatch * kQueueUnits;   // its control block: tickets, arrivals, ready flags
+constexpr int kXchSlots = 16;          // units of an exchange ring of the resident scorer's teams
+constexpr int kXchWords = 2 * kMaxSms * kXchSlots * 64;   // their tagged 64-bit words
 constexpr int kMergeGroup = 6;         // partials of a row merged together
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -34,6 +36,7 @@ struct Workspace {
   float* head_part;     // [kMaxStatLayers][H][4] per-(layer, head) {sum of squared deviations from 1/n, top-k mass}
   int* stat_ctr;        // [kMaxStatLayers] and, behind it, chunk_ctr [n_pad / kKeyTile]: zero between launches
   int* chunk_ctr;
+  unsigned long long* xch;   // [kXchWords] tagged words the resident scorer's CTAs exchange; zero at first
   size_t zero_bytes;    // from `status` on: what starts from zero
   size_t bytes;
 };
@@ -84,6 +87,9 @@ size_t tc_part_tasks(const structkv_config& cfg, int n, bool batch);
 structkv_status tc_create(Ctx& ctx);
 void tc_destroy(Ctx& ctx);
 cudaError_t launch_score_tc(const Ctx& ctx, const ScoreCall& a, cudaStream_t st);
+// The form of it for sequences whose probabilities fit the chip's tensor memory (score_res.cu).
+bool res_supported(const Ctx& ctx, const ScoreCall& a);
+cudaError_t launch_score_res(const Ctx& ctx, const ScoreCall& a, int first, int n, cudaStream_t st);
 
 // One thread waits (bounded by limit_cycles) on a barrier nobody arrives on, then records
 // STRUCTKV_ERR_TIMEOUT in *status.

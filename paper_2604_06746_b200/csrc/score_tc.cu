@@ -27,16 +27,6 @@ __global__ void wait_expiry_probe(unsigned long long limit_cycles, int* status) 
   }
 }
 
-bool encode3(const Ctx& ctx, CUtensorMap* m, const void* base, cuuint64_t d1, cuuint64_t d2, cuuint64_t s1,
-             cuuint64_t s2, cuuint32_t b1, cuuint32_t b2) {
-  const cuuint64_t dims[3] = {(cuuint64_t)ctx.cfg.head_dim, d1, d2};
-  const cuuint64_t strides[2] = {s1, s2};
-  const cuuint32_t box[3] = {64, b1, b2}, estr[3] = {1, 1, 1};
-  return ((TcState*)ctx.tc)->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
-                                    estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // How a configuration's score rows are laid out and weighted.
 struct Layout {
   int group, rows_pg, n_rb, units, shape, unit_rows, w_last, w_group, w_total;
@@ -110,12 +100,12 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
   const cuuint64_t row = (cuuint64_t)cfg.head_dim * 2;
   const int n_maps = batch ? 1 : n;
   for (int i = 0; i < n_maps; ++i) {
-    if (!encode3(ctx, &p.map_q[i], a.q[first + i], cfg.window, (cuuint64_t)cfg.n_q_heads * (batch ? n : 1), row,
+    if (!tc_encode3(ctx, &p.map_q[i], a.q[first + i], cfg.window, (cuuint64_t)cfg.n_q_heads * (batch ? n : 1), row,
                  row * cfg.window, std::min(ctx.w_pad, box_rows), std::max(1, box_rows / ctx.w_pad)))
       return cudaErrorInvalidValue;
     const cuuint64_t s_tok = (cuuint64_t)a.k_stride_token * 2;
     const cuuint64_t s_head = cfg.n_kv_heads == 1 ? s_tok * (cuuint64_t)total_keys : (cuuint64_t)a.k_stride_head * 2;
-    if (!encode3(ctx, &p.map_k[i], a.k[first + i], total_keys, cfg.n_kv_heads, s_tok, s_head, kKeyTile, 1))
+    if (!tc_encode3(ctx, &p.map_k[i], a.k[first + i], total_keys, cfg.n_kv_heads, s_tok, s_head, kKeyTile, 1))
       return cudaErrorInvalidValue;
   }
   const int cut = batch ? batch_cut(l, a, sms) : 1;
@@ -206,6 +196,16 @@ cudaError_t launch_wait_probe(unsigned long long limit_cycles, int* status, cuda
   return cudaGetLastError();
 }
 
+bool tc_encode3(const Ctx& ctx, CUtensorMap* m, const void* base, cuuint64_t d1, cuuint64_t d2, cuuint64_t s1,
+                cuuint64_t s2, cuuint32_t b1, cuuint32_t b2) {
+  const cuuint64_t dims[3] = {(cuuint64_t)ctx.cfg.head_dim, d1, d2};
+  const cuuint64_t strides[2] = {s1, s2};
+  const cuuint32_t box[3] = {64, b1, b2}, estr[3] = {1, 1, 1};
+  return ((TcState*)ctx.tc)->encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
+                                    estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 int tc_window_pad(int window) {
   int w = 8;
   while (w < window) w *= 2;
@@ -245,6 +245,13 @@ void tc_destroy(Ctx& ctx) {
 }
 
 cudaError_t launch_score_tc(const Ctx& ctx, const ScoreCall& a, cudaStream_t st) {
+  if (res_supported(ctx, a)) {
+    cudaError_t e = cudaSuccess;
+    for (int l = 0; l < a.n && e == cudaSuccess; l += kMaxBatch) e = launch_score_res(ctx, a, l, std::min(kMaxBatch, a.n - l), st);
+    // where the device does not give this process all of its SMs at once, the general scorer does it
+    if (e != cudaErrorCooperativeLaunchTooLarge) return e;
+    cudaGetLastError();
+  }
   if (a.cu_seqlens) return a.n == 1 ? launch_problems<1>(ctx, a, 0, 1, st) : launch_problems<kMaxBatch>(ctx, a, 0, a.n, st);
   for (int l = 0; l < a.n; l += kMaxBatch) {
     const int n = std::min(kMaxBatch, a.n - l);

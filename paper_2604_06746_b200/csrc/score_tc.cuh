@@ -101,7 +101,7 @@ struct alignas(64) TcParams {
   // hidden and the compute warps' is not (32 layers of 5003 keys: 317 us in a hurry, 300 without).
   int hurry;
 };
-constexpr int kCtlTicket = 0, kCtlExit = 1, kCtlArrive = 64, kCtlReady = 64 + kMaxBatch * kQueueUnits;
+constexpr int kCtlTicket = 0, kCtlExit = 1, kCtlTag = 2, kCtlArrive = 64, kCtlReady = 64 + kMaxBatch * kQueueUnits;
 static_assert(kCtlInts == 64 + 2 * kMaxBatch * kQueueUnits, "control block");
 
 // Tasks of a problem are dealt out to its units in proportion to their weights: unit u owns tasks
@@ -1327,6 +1327,11 @@ cudaError_t tc_launch(const TcParams<MAXP>& p, int grid, int device, cudaStream_
   return cudaLaunchKernelExC(&cfg, (const void*)kern, args);
 }
 #endif  // __CUDACC__
+
+// A 3-D tensor map of bf16 rows of head_dim elements, 128-byte swizzle: extents d1 x d2 of strides s1, s2 (bytes),
+// boxes of b1 x b2 rows.
+bool tc_encode3(const Ctx& ctx, CUtensorMap* m, const void* base, cuuint64_t d1, cuuint64_t d2, cuuint64_t s1,
+                cuuint64_t s2, cuuint32_t b1, cuuint32_t b2);
 
 // One translation unit per head dimension and parameter size instantiates the kernels.
 cudaError_t tc_launch_64(int shape, const TcParams<1>& p, int grid, int device, cudaStream_t st);
