@@ -1,4 +1,5 @@
-"""Thin ctypes binding over the C-ABI library ``libstructkv.so``.
+"""Thin binding over the C-ABI library ``libstructkv.so``: the calls made per layer or per prompt go through the native
+module ``_native`` (argument checks, pointers and strides), the others through ctypes.
 
 Argument marshalling only: every step of the path runs in the library's CUDA
 kernels.  PyTorch tensors supply device memory and streams.  Importing this
@@ -16,12 +17,14 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libstructkv.so")
 
-if not os.path.exists(LIB_PATH):
+if not (os.path.exists(LIB_PATH) and os.path.exists(os.path.join(_HERE, "_native.so"))):
     raise ImportError(
-        f"{LIB_PATH} is missing: build it with `python -m paper_2604_06746_b200.build` "
+        f"{LIB_PATH} or _native.so is missing: build it with `python -m paper_2604_06746_b200.build` "
         "(the StructKV hot path has no non-CUDA fallback)")
 
 lib = ctypes.CDLL(LIB_PATH)
+
+from . import _native  # noqa: E402  (links against the library)
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT = range(6)
 BF16, FP32 = 0, 1
@@ -115,6 +118,18 @@ class PrefillArgs(ctypes.Structure):
         return a
 
 
+_CODES = {torch.bfloat16: BF16, torch.float32: FP32}
+
+
+def fill_prefill(args: PrefillArgs, layers, hidden, positions, s_hist, head_cols, metrics, c_running, c_star, i_kv, i_struct,
+                 kv_out, hidden_out, pos_out, layers_workspace, sizes, dtype, lam, weights) -> bool:
+    """Checks one prompt's tensors and fills the block in (``args.arrays`` exist).  False: they are not in the form that
+    ``structkv_prefill`` takes, and nothing of the block counts.  ``sizes``: query heads, KV heads, keys, head
+    dimension, window, K/V budget, structural budget, cap of the pivot."""
+    return _native.fill_prefill(ctypes.addressof(args), layers, hidden, positions, s_hist, head_cols, metrics, c_running, c_star,
+                                i_kv, i_struct, kv_out, hidden_out, pos_out, layers_workspace, sizes, _CODES[dtype], lam, weights)
+
+
 lib.structkv_prefill.restype = _i
 lib.structkv_prefill.argtypes = [_vp, ctypes.POINTER(PrefillArgs), ctypes.POINTER(_i), ctypes.POINTER(_f), _vp]
 lib.structkv_selftest_wait_expiry.restype = _i
@@ -165,7 +180,7 @@ def score_layer_static(n_q_heads: int, n_kv_heads: int, head_dim: int, window: i
     and must not overlap on the GPU, and the first call on a device does a one-time set-up that
     should precede any stream capture.  The current torch device must be the tensors' device.
     """
-    code = {torch.bfloat16: BF16, torch.float32: FP32}[q_window.dtype]
+    code = _CODES[q_window.dtype]
     assert q_window.is_contiguous() and k.stride(2) == 1 and k.dtype == q_window.dtype
     cfg = Config(n_q_heads, n_kv_heads, head_dim, window, max_seq, code)
     with torch.cuda.device(q_window.device):
@@ -200,7 +215,7 @@ class Context:
 
     def __init__(self, n_q_heads: int, n_kv_heads: int, head_dim: int, window: int, max_seq: int,
                  dtype: torch.dtype, device: str = "cuda:0"):
-        code = {torch.bfloat16: BF16, torch.float32: FP32}[dtype]
+        code = _CODES[dtype]
         self.cfg = Config(n_q_heads, n_kv_heads, head_dim, window, max_seq, code)
         self.device = torch.device(device)
         self.dtype = dtype
@@ -230,11 +245,8 @@ class Context:
                     lam: float = 0.9, head_cols_out: Optional[torch.Tensor] = None, flags: int = 0,
                     stream: Optional[torch.cuda.Stream] = None) -> None:
         """structkv_score_layer: ``k`` is ``[H_kv, N, d]`` with arbitrary head / token strides."""
-        assert q_window.is_contiguous() and k.stride(2) == 1 and k.dtype == self.dtype == q_window.dtype
-        _check(lib.structkv_score_layer(self._h, q_window.data_ptr(), k.data_ptr(), k.stride(0), k.stride(1),
-                                        k.shape[1], scale, lam, s_out.data_ptr(), _ptr(c_inout),
-                                        _ptr(head_cols_out), metrics_out.data_ptr(), flags,
-                                        _stream(stream)), "structkv_score_layer")
+        _check(_native.score_layer(self._h.value, self.cfg.dtype, q_window, k, scale, s_out, metrics_out, c_inout, lam,
+                                   head_cols_out, flags, stream), "structkv_score_layer")
 
     def score_layer_batch(self, q_window: torch.Tensor, k: torch.Tensor, cu_seqlens: Sequence[int], scale: float,
                           s_out: torch.Tensor, metrics_out: torch.Tensor, workspace: torch.Tensor,
@@ -338,37 +350,23 @@ class Context:
 
     def prefill(self, args: PrefillArgs, stream: Optional[torch.cuda.Stream] = None) -> Tuple[int, list]:
         """structkv_prefill on a prepared argument block; returns ``(L*, T)``."""
-        piv, T = _i(0), (_f * args.n_layers)()
-        _check(lib.structkv_prefill(self._h, ctypes.byref(args), ctypes.byref(piv), T, _stream(stream)), "structkv_prefill")
-        return piv.value, list(T)
+        status, pivot, transition = _native.prefill(self._h.value, ctypes.addressof(args), stream)
+        _check(status, "structkv_prefill")
+        return pivot, transition
 
     def accumulate(self, s_hist: torch.Tensor, pivot: int, lam: float, c_out: torch.Tensor,
                    stream: Optional[torch.cuda.Stream] = None) -> None:
-        _check(lib.structkv_accumulate(self._h, s_hist.data_ptr(), s_hist.stride(0), pivot, s_hist.shape[1],
-                                       lam, c_out.data_ptr(), _stream(stream)), "structkv_accumulate")
+        _check(_native.accumulate(self._h.value, s_hist, pivot, lam, c_out, stream), "structkv_accumulate")
 
     def select(self, scores: torch.Tensor, budget: int, window: int, idx_out: torch.Tensor,
                stream: Optional[torch.cuda.Stream] = None) -> None:
         """structkv_select over ``scores [batch, n]`` (or ``[n]``) into ``idx_out [batch, budget]`` int32."""
-        s2 = scores if scores.dim() == 2 else scores[None]
-        assert s2.stride(1) == 1 and s2.dtype == torch.float32 and idx_out.dtype == torch.int32
-        assert idx_out.is_contiguous() and idx_out.numel() == s2.shape[0] * budget
-        _check(lib.structkv_select(self._h, s2.data_ptr(), s2.stride(0), s2.shape[0], s2.shape[1], budget,
-                                   window, idx_out.data_ptr(), _stream(stream)), "structkv_select")
+        _check(_native.select(self._h.value, scores, budget, window, idx_out, stream), "structkv_select")
 
     def compact(self, src: torch.Tensor, idx: torch.Tensor, dst: torch.Tensor,
                 stream: Optional[torch.cuda.Stream] = None) -> None:
         """structkv_compact: ``src [n_slabs, n_rows, row...]`` (row contiguous) -> ``dst [n_slabs, n_idx, row...]``."""
-        assert idx.dtype == torch.int32 and idx.is_contiguous() and dst.is_contiguous()
-        row_elems = 1
-        for s in src.shape[2:]:
-            row_elems *= s
-        es = src.element_size()
-        if src.dim() > 2:
-            assert src[0, 0].is_contiguous()
-        _check(lib.structkv_compact(self._h, src.data_ptr(), src.stride(0) * es, src.stride(1) * es,
-                                    row_elems * es, src.shape[0], src.shape[1], idx.data_ptr(),
-                                    idx.numel(), dst.data_ptr(), _stream(stream)), "structkv_compact")
+        _check(_native.compact(self._h.value, src, idx, dst, stream), "structkv_compact")
 
     @staticmethod
     def layer_sources(srcs: Sequence[torch.Tensor]) -> "LayerSources":
@@ -395,43 +393,23 @@ class Context:
     def group_saliency(self, head_cols: torch.Tensor, out: torch.Tensor,
                        stream: Optional[torch.cuda.Stream] = None) -> None:
         """structkv_group_saliency: ``head_cols [H, n]`` -> ``out [H_kv, n]`` (sum over each GQA group)."""
-        assert head_cols.stride(1) == 1 and head_cols.dtype == torch.float32 and out.is_contiguous()
-        assert head_cols.shape[0] == self.cfg.n_q_heads and out.shape == (self.cfg.n_kv_heads, head_cols.shape[1])
-        _check(lib.structkv_group_saliency(self._h, head_cols.data_ptr(), head_cols.stride(0), head_cols.shape[1],
-                                           out.data_ptr(), _stream(stream)), "structkv_group_saliency")
+        _check(_native.group_saliency(self._h.value, self.cfg.n_q_heads, self.cfg.n_kv_heads, head_cols, out, stream),
+               "structkv_group_saliency")
 
     def compact_per_slab(self, src: torch.Tensor, idx: torch.Tensor, dst: torch.Tensor,
                          stream: Optional[torch.cuda.Stream] = None) -> None:
         """structkv_compact_per_slab: ``src [n_slabs, n_rows, row...]``, ``idx [n_slabs, n_idx]`` int32."""
-        assert idx.dtype == torch.int32 and idx.dim() == 2 and idx.stride(1) == 1 and dst.is_contiguous()
-        assert idx.shape[0] == src.shape[0]
-        row_elems = 1
-        for sdim in src.shape[2:]:
-            row_elems *= sdim
-        es = src.element_size()
-        _check(lib.structkv_compact_per_slab(self._h, src.data_ptr(), src.stride(0) * es, src.stride(1) * es,
-                                             row_elems * es, src.shape[0], src.shape[1], idx.data_ptr(),
-                                             idx.stride(0), idx.shape[1], dst.data_ptr(), _stream(stream)),
-               "structkv_compact_per_slab")
+        _check(_native.compact_per_slab(self._h.value, src, idx, dst, stream), "structkv_compact_per_slab")
 
     def block_scores(self, scores: torch.Tensor, block_size: int, out: torch.Tensor,
                      stream: Optional[torch.cuda.Stream] = None) -> None:
         """structkv_block_scores over ``scores [batch, n]`` (or ``[n]``) into ``out [batch, ceil(n / block_size)]``."""
-        s2 = scores if scores.dim() == 2 else scores[None]
-        assert s2.stride(1) == 1 and s2.dtype == torch.float32 and out.dtype == torch.float32 and out.is_contiguous()
-        assert out.numel() == s2.shape[0] * ((s2.shape[1] + block_size - 1) // block_size)
-        _check(lib.structkv_block_scores(self._h, s2.data_ptr(), s2.stride(0), s2.shape[0], s2.shape[1], block_size,
-                                         out.data_ptr(), _stream(stream)), "structkv_block_scores")
+        _check(_native.block_scores(self._h.value, scores, block_size, out, stream), "structkv_block_scores")
 
     def mass_recovery(self, scores: torch.Tensor, idx: torch.Tensor, out: torch.Tensor,
                       stream: Optional[torch.cuda.Stream] = None) -> None:
         """structkv_mass_recovery: share of each row of ``scores [batch, n]`` that lies at ``idx``."""
-        s2 = scores if scores.dim() == 2 else scores[None]
-        assert s2.stride(1) == 1 and s2.dtype == torch.float32 and idx.dtype == torch.int32 and idx.is_contiguous()
-        assert out.dtype == torch.float32 and out.numel() == s2.shape[0]
-        _check(lib.structkv_mass_recovery(self._h, s2.data_ptr(), s2.stride(0), s2.shape[0], s2.shape[1],
-                                          idx.data_ptr(), idx.numel(), out.data_ptr(), _stream(stream)),
-               "structkv_mass_recovery")
+        _check(_native.mass_recovery(self._h.value, scores, idx, out, stream), "structkv_mass_recovery")
 
     def selftest_wait_expiry(self, limit_cycles: int, stream: Optional[torch.cuda.Stream] = None) -> None:
         """structkv_selftest_wait_expiry: lets one bounded device wait run out (records TIMEOUT)."""

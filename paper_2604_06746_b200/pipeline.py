@@ -16,10 +16,6 @@ PAPER_LAMBDA = 0.9
 PAPER_WEIGHTS = (0.2, 0.3, 0.5)
 
 
-def _fits(t: torch.Tensor, shape, dtype: torch.dtype) -> bool:
-    return t.shape == shape and t.dtype == dtype and t.is_contiguous()
-
-
 class Prefill:
     def __init__(self, n_layers: int, n_q_heads: int, n_kv_heads: int, head_dim: int, window: int,
                  seq: int, kv_budget: int, struct_budget: int, dtype: torch.dtype,
@@ -197,59 +193,15 @@ class Prefill:
         L, N, Hkv, d, dt = len(layers), self.N, self.Hkv, self.d, self.dtype
         if not (self.defer and self.keep_kv and L == self.L and L <= 128 and self.flags in (0, binding.FLAG_INPUTS_READY)):
             return None
-        k0, kv0 = layers[0]["k"], layers[0].get("kv")
-        if kv0 is None or kv0.shape != (2, Hkv, N, d) or k0.stride(2) != 1 or k0.shape[1] != N:
-            return None
-        k_shape, k_stride, kv_shape, kv_stride = k0.shape, k0.stride(), kv0.shape, kv0.stride()
-        q_ptr, k_ptr, kv_ptr, scales = [], [], [], []
-        for t in layers:
-            q, k, kv = t["q_win"], t["k"], t.get("kv")
-            if (kv is None or k.shape != k_shape or k.stride() != k_stride or kv.shape != kv_shape or kv.stride() != kv_stride
-                    or not k.dtype == q.dtype == kv.dtype == dt or not q.is_contiguous()):
-                return None
-            q_ptr.append(q.data_ptr())
-            k_ptr.append(k.data_ptr())
-            kv_ptr.append(kv.data_ptr())
-            scales.append(t["scale"])
-        f32, i32, rows = torch.float32, torch.int32, self.struct_budget
-        if not (_fits(self.s_hist, (L, N), f32) and _fits(self.head_cols, (L, self.H, N), f32)
-                and _fits(self.metrics, (L, 3), f32) and _fits(self.c_running, (N,), f32) and _fits(self.c_star, (N,), f32)
-                and _fits(self.i_kv, (L, self.kv_budget), i32) and _fits(self.i_struct, (rows,), i32)
-                and _fits(self.kv_out, (L, 2, Hkv, self.kv_budget, d), dt)):
-            return None
-        if hidden is not None and not (self.hidden_out is not None and hidden.dim() == 2 and hidden.stride(1) == 1
-                                       and hidden.shape[0] == N and hidden.dtype == self.hidden_out.dtype
-                                       and self.hidden_out.is_contiguous() and self.hidden_out.shape == (rows, hidden.shape[1])
-                                       and positions.dim() == 1 and positions.shape[0] == N and positions.dtype == i32
-                                       and _fits(self.pos_out, (rows,), i32)):
-            return None
-        if Hkv > 1 and kv_stride[0] != Hkv * kv_stride[1]:   # the 2 H_kv slabs have no common stride
+        if self._plan is None or self._plan.n_layers != L:
+            self._plan = binding.PrefillArgs.for_layers(L)
+        a = self._plan
+        sizes = (self.H, Hkv, N, d, self.w, self.kv_budget, self.struct_budget, self.l_limit)
+        if not binding.fill_prefill(a, layers, hidden, positions, self.s_hist, self.head_cols, self.metrics, self.c_running,
+                                    self.c_star, self.i_kv, self.i_struct, self.kv_out, self.hidden_out, self.pos_out,
+                                    self._layers_ws, sizes, dt, self.lam, self.weights):
             return None
         if self._layers_ws is None:
             self._layers_ws = self.ctx.layers_workspace(L)
-        if self._plan is None or self._plan.n_layers != L:
-            self._plan = binding.PrefillArgs.for_layers(L)
-        a, es = self._plan, kv0.element_size()
-        for array, values in zip(a.arrays, (q_ptr, k_ptr, kv_ptr, scales)):
-            array[:] = values
-        a.n_keys, a.lam, a.l_limit, a.window = N, self.lam, self.l_limit, self.w
-        a.k_stride_head, a.k_stride_token = k_stride[0], k_stride[1]
-        a.s_out, a.s_layer_stride, a.c_out = self.s_hist.data_ptr(), N, self.c_running.data_ptr()
-        a.head_cols, a.head_cols_layer_stride = self.head_cols.data_ptr(), self.H * N
-        a.metrics = self.metrics.data_ptr()
-        a.layers_workspace, a.layers_workspace_bytes = self._layers_ws.data_ptr(), self._layers_ws.numel()
-        a.weights = (binding._f * 3)(*self.weights)
-        a.kv_budget, a.struct_budget = self.kv_budget, rows
-        a.i_kv, a.i_struct, a.c_star = self.i_kv.data_ptr(), self.i_struct.data_ptr(), self.c_star.data_ptr()
-        a.kv_slab_stride_bytes, a.kv_row_stride_bytes = kv_stride[1 if Hkv > 1 else 0] * es, kv_stride[2] * es
-        a.kv_row_bytes, a.kv_slabs, a.kv_rows = d * es, 2 * Hkv, N
-        a.kv_dst, a.kv_dst_layer_stride_bytes = self.kv_out.data_ptr(), 2 * Hkv * self.kv_budget * d * es
-        if hidden is None:
-            a.hidden = a.hidden_dst = a.positions = a.positions_dst = None
-        else:
-            es, ps = hidden.element_size(), positions.element_size()
-            a.hidden, a.hidden_row_stride_bytes, a.hidden_row_bytes = hidden.data_ptr(), hidden.stride(0) * es, hidden.shape[1] * es
-            a.hidden_dst = self.hidden_out.data_ptr()
-            a.positions, a.position_row_stride_bytes, a.position_row_bytes = positions.data_ptr(), positions.stride(0) * ps, ps
-            a.positions_dst = self.pos_out.data_ptr()
+            a.layers_workspace, a.layers_workspace_bytes = self._layers_ws.data_ptr(), self._layers_ws.numel()
         return a
