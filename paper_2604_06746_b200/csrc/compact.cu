@@ -1,9 +1,12 @@
 // Row gather / compaction: dst[s, r, :] = src[s, idx[r], :], byte exact.  Rows are split into
 // 16-byte (or 4-byte / 1-byte) units; consecutive threads take consecutive units of a row, so
-// writes are fully coalesced and reads are coalesced within each gathered row.  Two loads in
-// flight per thread and up to 64 resident blocks per SM measured best on B200 (more unrolling
-// or fewer, fatter blocks lose 10-25 % of the copy bandwidth).
+// writes are fully coalesced and reads are coalesced within each gathered row.
+// Bound by DRAM: 32 layers x 16 slabs x 16384 rows of 256 bytes 690 us, 6.22 TB/s (a plain copy: 6.46); 2048 rows a
+// slab 93 us.  With a 64-bit division per unit and blocks striding over the whole output these took 745 and 107: the
+// divisions used more issue slots than the loads.  Two, four and eight loads in flight per thread: 690 / 696 / 687 us.
 #include "common.cuh"
+
+#include <algorithm>
 
 namespace skv {
 namespace {
@@ -23,93 +26,119 @@ template <> __device__ __forceinline__ void st_stream<uint4>(uint4* p, const uin
   asm volatile("st.global.cs.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-// Block 0 .. blocks - 1 of a gather.
+// u / d for u < 2^31 by one multiplication (a 64-bit division took some 100 instructions, two of them per 16 bytes).
+struct Divisor { unsigned mul; int shift; };               // mul 0: d is 1
+inline Divisor divisor(unsigned d) {
+  int l = 0;
+  while ((1ull << l) < d) ++l;
+  return d == 1 ? Divisor{0, 0} : Divisor{(unsigned)((1ull << (31 + l)) / d + 1), l - 1};
+}
+__device__ __forceinline__ unsigned operator/(unsigned u, const Divisor& d) {
+  return d.mul == 0 ? u : __umulhi(u, d.mul) >> d.shift;
+}
+
+// One list's rows out of one slab after the other: blocks 0 .. blocks - 1 of blockIdx.x, every gridDim.y-th slab.  A block
+// takes kCpUnroll * kCpThreads consecutive units.
+struct Gather {
+  long long slab_stride, row_stride, idx_slab_stride;
+  Divisor per_row;                     // units of a row
+  unsigned row_units, units;           // units this launch writes in a slab
+  unsigned long long slab_units;       // from slab to slab of the output
+  int n_slabs, n_rows_src;
+};
 template <typename V>
-__device__ __forceinline__ void
-gather_blocks(int blocks, const char* __restrict__ src, long long slab_stride, long long row_stride,
-              int units_per_row, int n_slabs, int n_rows_src, const int* __restrict__ idx,
-              long long idx_slab_stride, int n_idx,
-              char* __restrict__ dst, int* __restrict__ status) {
-  const long long total = (long long)n_slabs * n_idx * units_per_row;
-  const long long stride = (long long)blocks * kCpThreads;
-  for (long long u0 = (long long)blockIdx.x * kCpThreads + threadIdx.x; u0 < total;
-       u0 += stride * kCpUnroll) {
-    V val[kCpUnroll];
-    bool ok[kCpUnroll];
+__device__ __forceinline__ void gather_blocks(const Gather& g, unsigned blocks, const char* __restrict__ src,
+                                              const int* __restrict__ idx, char* __restrict__ dst, int* __restrict__ status) {
+  for (int s = blockIdx.y; s < g.n_slabs; s += gridDim.y) {
+    const char* const from = src + s * g.slab_stride;
+    const int* const list = idx + s * g.idx_slab_stride;   // stride 0: one list for every slab
+    V* const to = reinterpret_cast<V*>(dst) + s * g.slab_units;
+    for (unsigned u0 = blockIdx.x * (kCpThreads * kCpUnroll) + threadIdx.x; u0 < g.units; u0 += blocks * (kCpThreads * kCpUnroll)) {
+      V val[kCpUnroll];
+      int j[kCpUnroll];
 #pragma unroll
-    for (int e = 0; e < kCpUnroll; ++e) {
-      const long long u = u0 + e * stride;
-      ok[e] = false;
-      if (u < total) {
-        const long long row = u / units_per_row;           // s * n_idx + r
-        const int c = (int)(u - row * units_per_row);
-        const int s = (int)(row / n_idx), r = (int)(row - (long long)s * n_idx);
-        const int j = __ldg(idx + s * idx_slab_stride + r);   // stride 0: one list for every slab
-        if (j >= 0 && j < n_rows_src) {
-          val[e] = ld_stream(reinterpret_cast<const V*>(src + s * slab_stride + j * row_stride +
-                                                        (long long)c * sizeof(V)));
-          ok[e] = true;
-        } else if (c == 0) {
-          atomicCAS(status, 0, (int)STRUCTKV_ERR_INVALID_ARG);
-        }
+      for (int e = 0; e < kCpUnroll; ++e) {
+        const unsigned u = u0 + e * kCpThreads;
+        j[e] = u < g.units ? __ldg(list + u / g.per_row) : -1;
       }
-    }
 #pragma unroll
-    for (int e = 0; e < kCpUnroll; ++e) {
-      const long long u = u0 + e * stride;
-      if (ok[e]) st_stream(reinterpret_cast<V*>(dst + u * (long long)sizeof(V)), val[e]);
+      for (int e = 0; e < kCpUnroll; ++e) {
+        const unsigned u = u0 + e * kCpThreads, c = u - u / g.per_row * g.row_units;
+        if (j[e] >= 0 && j[e] < g.n_rows_src)
+          val[e] = ld_stream(reinterpret_cast<const V*>(from + j[e] * g.row_stride) + c);
+        else if (u < g.units && c == 0)
+          atomicCAS(status, 0, (int)STRUCTKV_ERR_INVALID_ARG);
+      }
+#pragma unroll
+      for (int e = 0; e < kCpUnroll; ++e)
+        if (j[e] >= 0 && j[e] < g.n_rows_src) st_stream(to + u0 + e * kCpThreads, val[e]);
     }
   }
 }
 
 template <typename V>
 __global__ void __launch_bounds__(kCpThreads)
-gather_rows(const char* __restrict__ src, long long slab_stride, long long row_stride,
-            int units_per_row, int n_slabs, int n_rows_src, const int* __restrict__ idx,
-            long long idx_slab_stride, int n_idx,
-            char* __restrict__ dst, int* __restrict__ status) {
+gather_rows(const Gather g, const char* __restrict__ src, const int* __restrict__ idx, char* __restrict__ dst,
+            int* __restrict__ status) {
   pdl_trigger();
   pdl_wait();
-  gather_blocks<V>(gridDim.x, src, slab_stride, row_stride, units_per_row, n_slabs, n_rows_src, idx, idx_slab_stride, n_idx,
-                   dst, status);
+  gather_blocks<V>(g, gridDim.x, src, idx, dst, status);
 }
 // The last `words` blocks gather one word per row of a second source by the same list (a launch of its own for
 // 4 bytes a row took 2 to 3 us after the gather it follows: the smallest whole prefill 66.8 -> 65.0 us).
 template <typename V>
 __global__ void __launch_bounds__(kCpThreads)
-gather_rows_words(const char* __restrict__ src, long long row_stride, int units_per_row, int n_rows_src,
-                  const int* __restrict__ idx, int n_idx, char* __restrict__ dst, int* __restrict__ status,
-                  const CompactWords w, int words) {
+gather_rows_words(const Gather g, const char* __restrict__ src, const int* __restrict__ idx, int n_idx,
+                  char* __restrict__ dst, int* __restrict__ status, const CompactWords w, int words) {
   pdl_trigger();
   pdl_wait();
   if ((int)blockIdx.x >= (int)gridDim.x - words) {
     const int r = ((int)blockIdx.x - (int)gridDim.x + words) * kCpThreads + (int)threadIdx.x;
     if (r < n_idx) {
       const int j = __ldg(idx + r);
-      if (j >= 0 && j < n_rows_src)
+      if (j >= 0 && j < g.n_rows_src)
         reinterpret_cast<unsigned*>(w.dst)[r] = *reinterpret_cast<const unsigned*>((const char*)w.src + j * w.row_stride);
     }
     return;
   }
-  gather_blocks<V>(gridDim.x - words, src, 0, row_stride, units_per_row, 1, n_rows_src, idx, 0, n_idx, dst, status);
+  gather_blocks<V>(g, gridDim.x - words, src, idx, dst, status);
 }
 
-// The same gather for several layers in one launch: layer blockIdx.y reads its own source (the
-// pointers travel as a kernel argument), its own index list and writes its own slab of dst.
+// The same gather for several layers in one launch: layer blockIdx.z reads its own source (the
+// pointers travel as a kernel argument), its own index list and writes its own slabs of dst.
 struct LayerPtrs { const char* src[kMaxGatherLayers]; };
 
 template <typename V>
 __global__ void __launch_bounds__(kCpThreads)
-gather_rows_layers(const __grid_constant__ LayerPtrs srcs, long long slab_stride, long long row_stride,
-                   int units_per_row, int n_slabs, int n_rows_src, const int* __restrict__ idx,
-                   long long idx_layer_stride, int n_idx, char* __restrict__ dst, long long dst_layer_stride,
-                   int* __restrict__ status) {
+gather_rows_layers(const Gather g, const __grid_constant__ LayerPtrs srcs, const int* __restrict__ idx,
+                   long long idx_layer_stride, char* __restrict__ dst, long long dst_layer_stride, int* __restrict__ status) {
   pdl_trigger();
   pdl_wait();
-  const int layer = blockIdx.y;
-  gather_blocks<V>(gridDim.x, srcs.src[layer], slab_stride, row_stride, units_per_row, n_slabs, n_rows_src,
-                   idx + (long long)layer * idx_layer_stride, 0, n_idx, dst + (long long)layer * dst_layer_stride, status);
+  const int layer = blockIdx.z;
+  gather_blocks<V>(g, gridDim.x, srcs.src[layer], idx + (long long)layer * idx_layer_stride,
+                   dst + (long long)layer * dst_layer_stride, status);
 }
+
+// The unit of a copy whose pointers, strides and row size have the low bits `low` between them, and the launch over it: at
+// most kCpBlocksPerSm blocks an SM.  A launch counts its units of a slab in 31 bits: longer lists go `rows` at a time.
+struct Plan {
+  Gather g;
+  int unit, rows;
+  dim3 grid;
+  Plan(unsigned long long low, long long slab_stride, long long row_stride, int row_bytes, int n_slabs, int n_rows_src,
+       long long idx_slab_stride, int n_idx)
+      : unit(low % 16 == 0 ? 16 : low % 4 == 0 ? 4 : 1) {
+    const unsigned per_row = (unsigned)(row_bytes / unit);
+    g = Gather{slab_stride, row_stride, idx_slab_stride, divisor(per_row), per_row, 0, (unsigned long long)per_row * n_idx, n_slabs, n_rows_src};
+    rows = (int)std::min((long long)n_idx, 0x7fffffffll / per_row);
+  }
+  void take(int n, int n_layers, int sm_count) {           // the next n indices
+    g.units = (unsigned)n * g.row_units;
+    const long long want = ((long long)g.units + kCpThreads * kCpUnroll - 1) / (kCpThreads * kCpUnroll);
+    const long long slabs = std::min(g.n_slabs, 32768), cap = (long long)sm_count * kCpBlocksPerSm / (slabs * n_layers);
+    grid = dim3((unsigned)std::max(1ll, std::min(want, cap)), (unsigned)slabs, (unsigned)n_layers);
+  }
+};
 
 }  // namespace
 
@@ -119,27 +148,20 @@ cudaError_t launch_compact_layers(const void* const* srcs, int n_layers, long lo
                                   int* status, int sm_count, cudaStream_t st) {
   if (n_idx == 0 || n_slabs == 0 || n_layers == 0) return cudaSuccess;
   LayerPtrs lp;
-  bool a16 = ((uintptr_t)dst % 16 == 0) && slab_stride % 16 == 0 && row_stride % 16 == 0 && row_bytes % 16 == 0 &&
-             dst_layer_stride % 16 == 0;
-  bool a4 = ((uintptr_t)dst % 4 == 0) && slab_stride % 4 == 0 && row_stride % 4 == 0 && row_bytes % 4 == 0 &&
-            dst_layer_stride % 4 == 0;
+  unsigned long long low = (uintptr_t)dst | slab_stride | row_stride | row_bytes | dst_layer_stride;
   for (int l = 0; l < n_layers; ++l) {
     lp.src[l] = (const char*)srcs[l];
-    a16 = a16 && ((uintptr_t)srcs[l] % 16 == 0);
-    a4 = a4 && ((uintptr_t)srcs[l] % 4 == 0);
+    low |= (uintptr_t)srcs[l];
   }
-  const int unit = a16 ? 16 : (a4 ? 4 : 1);
-  const int upr = row_bytes / unit;
-  const long long total = (long long)n_slabs * n_idx * upr;
-  long long blocks = (total + (long long)kCpThreads * kCpUnroll - 1) / ((long long)kCpThreads * kCpUnroll);
-  const long long cap = ((long long)sm_count * kCpBlocksPerSm + n_layers - 1) / n_layers;
-  if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
-  const dim3 grid((unsigned)blocks, (unsigned)n_layers);
-  char* d = (char*)dst;
-  const auto kernel = unit == 16 ? gather_rows_layers<uint4> : unit == 4 ? gather_rows_layers<unsigned> : gather_rows_layers<unsigned char>;
-  return launch_pdl(kernel, grid, dim3(kCpThreads), 0, st, lp, slab_stride, row_stride, upr, n_slabs, n_rows_src, idx,
-                    idx_layer_stride, n_idx, d, dst_layer_stride, status);
+  Plan p(low, slab_stride, row_stride, row_bytes, n_slabs, n_rows_src, 0, n_idx);
+  const auto kernel = p.unit == 16 ? gather_rows_layers<uint4> : p.unit == 4 ? gather_rows_layers<unsigned> : gather_rows_layers<unsigned char>;
+  for (int r = 0; r < n_idx; r += p.rows) {
+    p.take(std::min(p.rows, n_idx - r), n_layers, sm_count);
+    const cudaError_t e = launch_pdl(kernel, p.grid, dim3(kCpThreads), 0, st, p.g, lp, idx + r, idx_layer_stride,
+                                     (char*)dst + (long long)r * row_bytes, dst_layer_stride, status);
+    if (e != cudaSuccess || n_idx - r <= p.rows) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_compact(const void* src, long long slab_stride, long long row_stride,
@@ -147,28 +169,24 @@ cudaError_t launch_compact(const void* src, long long slab_stride, long long row
                            long long idx_slab_stride, int n_idx, void* dst, int* status, int sm_count,
                            cudaStream_t st, const CompactWords* words) {
   if (n_idx == 0 || n_slabs == 0) return cudaSuccess;
-  const bool a16 = ((uintptr_t)src % 16 == 0) && ((uintptr_t)dst % 16 == 0) && slab_stride % 16 == 0 &&
-                   row_stride % 16 == 0 && row_bytes % 16 == 0;
-  const bool a4 = ((uintptr_t)src % 4 == 0) && ((uintptr_t)dst % 4 == 0) && slab_stride % 4 == 0 &&
-                  row_stride % 4 == 0 && row_bytes % 4 == 0;
-  const int unit = a16 ? 16 : (a4 ? 4 : 1);
-  const int upr = row_bytes / unit;
-  const long long total = (long long)n_slabs * n_idx * upr;
-  long long blocks = (total + (long long)kCpThreads * kCpUnroll - 1) / ((long long)kCpThreads * kCpUnroll);
-  const long long cap = (long long)sm_count * kCpBlocksPerSm;
-  if (blocks > cap) blocks = cap;
-  if (blocks < 1) blocks = 1;
-  const char* s = (const char*)src;
-  char* d = (char*)dst;
-  if (words) {
-    const auto both = unit == 16 ? gather_rows_words<uint4> : unit == 4 ? gather_rows_words<unsigned> : gather_rows_words<unsigned char>;
-    const int extra = (n_idx + kCpThreads - 1) / kCpThreads;
-    return launch_pdl(both, dim3((unsigned)(blocks + extra)), dim3(kCpThreads), 0, st, s, row_stride, upr, n_rows_src, idx, n_idx,
-                      d, status, *words, extra);
+  Plan p((uintptr_t)src | (uintptr_t)dst | slab_stride | row_stride | row_bytes, slab_stride, row_stride, row_bytes, n_slabs, n_rows_src,
+         idx_slab_stride, n_idx);
+  const auto both = p.unit == 16 ? gather_rows_words<uint4> : p.unit == 4 ? gather_rows_words<unsigned> : gather_rows_words<unsigned char>;
+  const auto kernel = p.unit == 16 ? gather_rows<uint4> : p.unit == 4 ? gather_rows<unsigned> : gather_rows<unsigned char>;
+  for (int r = 0; r < n_idx; r += p.rows) {
+    p.take(std::min(p.rows, n_idx - r), 1, sm_count);
+    char* const to = (char*)dst + (long long)r * row_bytes;
+    cudaError_t e;
+    if (words && r == 0) {
+      const unsigned extra = ((unsigned)n_idx + kCpThreads - 1) / kCpThreads;
+      e = launch_pdl(both, dim3(p.grid.x + extra), dim3(kCpThreads), 0, st, p.g, (const char*)src, idx, n_idx, to, status, *words,
+                     (int)extra);
+    } else {
+      e = launch_pdl(kernel, p.grid, dim3(kCpThreads), 0, st, p.g, (const char*)src, idx + r, to, status);
+    }
+    if (e != cudaSuccess || n_idx - r <= p.rows) return e;
   }
-  const auto kernel = unit == 16 ? gather_rows<uint4> : unit == 4 ? gather_rows<unsigned> : gather_rows<unsigned char>;
-  return launch_pdl(kernel, dim3((unsigned)blocks), dim3(kCpThreads), 0, st, s, slab_stride, row_stride, upr, n_slabs,
-                    n_rows_src, idx, idx_slab_stride, n_idx, d, status);
+  return cudaSuccess;
 }
 
 }  // namespace skv
