@@ -1,10 +1,10 @@
 // Budgeted token selection (top-k of the prefix, ties to the lower index, output in position
-// order, window appended), exact: four eight-bit levels find the k-th largest key (radix.cuh), then every
+// order, window appended), exact: three levels of 11, 11 and 10 bits find the k-th largest key (radix.cuh), then every
 // kept token's place in the output follows from ballots and one scan of the counts per (group of
 // 1024 tokens, warp).  A cluster of CL CTAs shares one vector, each CTA a contiguous slice that it
 // holds in registers (up to ITEMS tokens a thread; a longer slice is read again per level).
 //
-// Bound by the chain of barriers, not by memory: one CTA up to 16384 tokens (no exchange between CTAs).
+// Bound by the chain of barriers, not by memory.
 #include <atomic>
 
 #include "radix.cuh"
@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(kRxThreads, ITEMS <= 8 ? 2 : 1) select_topk(co
   const int rank = CL > 1 ? (int)cg::this_cluster().block_rank() : 0;
   const int vec = blockIdx.x / CL;
   pdl_trigger();
-  radix_clear(s, 0);
+  radix_clear(s);
   cluster_barrier<CL>();                             // all CTAs of the cluster run before any remote access
   pdl_wait();
   const bool own = !a.packed && vec == a.batch;      // the extra vector
@@ -74,17 +74,16 @@ __global__ void __launch_bounds__(kRxThreads, ITEMS <= 8 ? 2 : 1) select_topk(co
     int level = 0;
 #pragma unroll 1
     for (; level < kRxLevels; ++level) {
-      const int shift = 24 - 8 * level;
-      const unsigned mask = level == 0 ? 0u : 0xffffffffu << (shift + 8);
+      const unsigned mask = level == 0 ? 0u : 0xffffffffu << radix_shift(level - 1);
       for (int c = 0; c < chunks; ++c) {
         if (chunks > 1) load(c);
 #pragma unroll
         for (int e = 0; e < ITEMS; ++e)
-          if (valid(c, e) && (key[e] & mask) == thr) radix_count(s, level & 1, (key[e] >> shift) & 255u);
+          if (valid(c, e) && (key[e] & mask) == thr) radix_count(s, level, radix_digit(key[e], level));
       }
       unsigned digit, in;
-      radix_pick(s, level & 1, remaining, digit, in);
-      thr |= digit << shift;
+      radix_pick(s, level, remaining, digit, in);
+      thr |= digit << radix_shift(level);
       if (in == remaining) break;                    // all keys of the digit are kept: no need to look inside
     }
     ge = level < kRxLevels ? thr : thr + 1;
@@ -180,18 +179,19 @@ cudaError_t launch(const SelectArgs& a, cudaStream_t st) {
                             sizeof(RadixShared<CL>), st, a);
 }
 
-// The smallest cluster and the fewest items per thread that hold a vector, as measured (us for 1 / 32
-// vectors): 1777 tokens 5.8 / 7.7 with 1 x 4 items, 5003 9.6 / 11.5 with 1 x 8, 12000 12.6 / 15.0 with
-// 1 x 16 (14.0 / 19.6 with a cluster of 2), 32768 17.3 / 20.3 with 2 x 16 (20.6 / 23.5 with 1 x 32, 19.3 /
-// 41.9 with 8 x 8), 65536 19.2 / 22.8 with 4 x 16.  At 131072 eight CTAs of 16 items take 23.1 us for one
-// vector but 69.1 for 32, whose 256 CTAs no longer run side by side; four of 32 take 28.6 / 33.0.
+// One CTA while that is a matter of three barriers a level; beyond, few vectors get more CTAs with fewer items each, and
+// many (whose CTAs would not run side by side) the smallest cluster that holds one.  us for 1 / 8 / 33 vectors, chained
+// launches: 1777 tokens 5.1 / 5.2 / 5.6 with 1 x 4 items (a cluster of two 6.9 / 7.0 / 7.2), 8192 7.0 / 7.2 / 8.4 with
+// 1 x 8 (2 x 4: 7.2 / 7.3 / 9.0), 16384 9.9 / 10.0 / 11.7 with 1 x 16 and 8.1 / 8.3 / 11.9 with 4 x 4, 32768 12.0 /
+// 12.2 / 14.1 with 2 x 16 and 10.6 / 11.0 / 16.0 with 4 x 8, 65536 13.1 / 13.3 / 16.2 with 4 x 16 and 12.5 /
+// 13.2 / 26.0 with 8 x 8, 131072 18.6 with 8 x 16 and 24.1 for 33 with 4 x 32.
 cudaError_t dispatch(const SelectArgs& a, int longest, cudaStream_t st) {
   if (longest <= 4 * kRxThreads) return launch<1, 4>(a, st);
   if (longest <= 8 * kRxThreads) return launch<1, 8>(a, st);
-  if (longest <= 16 * kRxThreads) return launch<1, 16>(a, st);
-  if (longest <= 32 * kRxThreads) return launch<2, 16>(a, st);
+  const bool room = a.batch <= 16;                   // up to eight CTAs a vector, one per SM
+  if (longest <= 16 * kRxThreads) return room ? launch<4, 4>(a, st) : launch<1, 16>(a, st);
+  if (longest <= 32 * kRxThreads) return room ? launch<4, 8>(a, st) : launch<2, 16>(a, st);
   if (longest <= 64 * kRxThreads) return launch<4, 16>(a, st);
-  const bool room = a.batch <= 16;                   // eight CTAs a vector, one per SM
   if (!room) return launch<4, 32>(a, st);
   if (longest <= 128 * kRxThreads) return launch<8, 16>(a, st);
   return launch<8, 32>(a, st);                       // beyond 262144 tokens the slices are read again per level
