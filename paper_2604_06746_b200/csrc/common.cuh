@@ -20,6 +20,8 @@ constexpr int kQueueUnits = 256;      // (KV group, row block) units of one prob
 constexpr int kCtlInts = 64 + 2 * kMaxBatch * kQueueUnits;   // its control block: tickets, arrivals, ready flags
 constexpr int kXchSlots = 16;          // units of an exchange ring of the resident scorer's teams
 constexpr int kXchWords = 2 * kMaxSms * kXchSlots * 64;   // their tagged 64-bit words
+constexpr int kCtlExit = 1, kCtlTag = 2;   // in the control block: CTAs that are done; last tag of the exchange words
+constexpr unsigned long long kWaitCycles = 1000000000ull;   // bound of a device wait, about 0.5 s at the maximum SM clock
 constexpr int kMergeGroup = 6;         // partials of a row merged together
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
@@ -186,6 +188,24 @@ inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = CL > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
+// The same for a kernel whose blocks wait for one another: all of them run at once, or the launch is refused.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_cooperative(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeCooperative;
+  attr[1].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 

@@ -31,6 +31,7 @@
 #pragma once
 
 #include "score_tc.cuh"
+#include "tagged.cuh"
 
 namespace skv {
 
@@ -74,21 +75,6 @@ struct alignas(64) ResParams {
 };
 
 #ifdef __CUDACC__
-
-// A value and the tag that says whose it is, in one 64-bit word: whoever sees the tag sees the value.
-__device__ __forceinline__ unsigned long long tagged(float v, unsigned tag) {
-  return (unsigned long long)tag << 32 | __float_as_uint(v);
-}
-__device__ __forceinline__ float word_value(unsigned long long w) { return __uint_as_float((unsigned)w); }
-__device__ __forceinline__ bool word_has(unsigned long long w, unsigned tag) { return (unsigned)(w >> 32) == tag; }
-__device__ __forceinline__ void put_word(unsigned long long* p, unsigned long long w) {
-  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
-}
-__device__ __forceinline__ unsigned long long get_word(const unsigned long long* p) {
-  unsigned long long w;
-  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
-  return w;
-}
 
 template <int D, int MAXP>
 struct ResSmem {
@@ -624,19 +610,9 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
   }
-  // the last CTA moves the tags on (and, long before they wrap, starts them over with clean words)
   if (threadIdx.x == 0) fl->last = atomicAdd(p.ctl + kCtlExit, 1) == (int)gridDim.x - 1;
   __syncthreads();
-  if (fl->last) {
-    const unsigned next = tag0 - 1u + (unsigned)((n_prob * n_kv + teams - 1) / teams);
-    const bool over = next > 0x7f000000u;
-    if (over)
-      for (size_t i = threadIdx.x; i < kXchWords; i += kResThreads) p.xch[i] = 0;
-    if (threadIdx.x == 0) {
-      p.ctl[kCtlTag] = over ? 0 : (int)next;
-      p.ctl[kCtlExit] = 0;
-    }
-  }
+  if (fl->last) pass_tags_on(p.xch, p.ctl, tag0 - 1u + (unsigned)((n_prob * n_kv + teams - 1) / teams));
 }
 
 template <int D, int MAXP>

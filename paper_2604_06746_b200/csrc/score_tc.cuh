@@ -60,7 +60,6 @@ constexpr int kTaskRing = 4;           // task descriptors in flight inside a CT
 constexpr int kHelperWarps = 4;
 constexpr int kComputeWarps = 16;
 constexpr int kTcThreads = (kHelperWarps + kComputeWarps) * 32;   // 20 warps: the most that fit at 96 registers a thread
-constexpr unsigned long long kWaitCycles = 1000000000ull;   // about 0.5 s at the maximum SM clock
 constexpr float kMasked = -1.0e30f;    // exponent standing for -inf: 2^x flushes to 0 and 0 * x stays finite
 constexpr float kMaskedAcc = -3.0e38f; // the same for an accumulator, before the scaling by c2 >= 1e-30
 constexpr int kFullWeight = 20;        // weight of a full row block when key ranges are dealt out (see tc_deal)
@@ -101,7 +100,7 @@ struct alignas(64) TcParams {
   // hidden and the compute warps' is not (32 layers of 5003 keys: 317 us in a hurry, 300 without).
   int hurry;
 };
-constexpr int kCtlTicket = 0, kCtlExit = 1, kCtlTag = 2, kCtlArrive = 64, kCtlReady = 64 + kMaxBatch * kQueueUnits;
+constexpr int kCtlTicket = 0, kCtlArrive = 64, kCtlReady = 64 + kMaxBatch * kQueueUnits;
 static_assert(kCtlInts == 64 + 2 * kMaxBatch * kQueueUnits, "control block");
 
 // Tasks of a problem are dealt out to its units in proportion to their weights: unit u owns tasks
