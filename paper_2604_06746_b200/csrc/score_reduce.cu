@@ -25,7 +25,8 @@ struct FinishArgs {
   int rows_pad, n_valid;
   float* metrics;                      // [n_prob][3]
   float* head_part;                    // [n_prob][H][4]
-  int with_stats, n_stat_ctas, chunks; // chunks: key ranges a problem's sum is cut into
+  int with_stats, chunks;              // chunks: key ranges a problem's sum is cut into
+  int stat_ctas;                       // CTAs of a problem's statistics
   int* stat_ctr;                       // [n_prob] heads done; zero between launches
   int* chunk_ctr;                      // [chunks] layers done; zero between launches
   int packed;                          // sequences of one layer: problem p owns columns [cu[p], cu[p + 1])
@@ -277,37 +278,41 @@ __device__ __forceinline__ float total_of(float (*red)[32]) {
   }
   return total;
 }
-// Once all warps have counted: walks the bins of a histogram from the top.  s.bin holds the
-// `remaining`-th largest candidate, s.rem is the rank still wanted inside it.
-template <int T>
-__device__ __forceinline__ void sweep_pick(SweepShared& s, const unsigned* hist, unsigned remaining) {
-  constexpr int kPer = kSwBins / T;                        // bins of a thread, higher first
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, top = kSwBins - 1 - kPer * tid;
-  unsigned c[kPer], mine = 0;
-  __syncthreads();
-#pragma unroll
-  for (int b = 0; b < kPer; ++b) mine += c[b] = hist[top - b];
-  unsigned incl = mine;
+// Lane l: the l-th of 32 counts from the top.  Where the wanted rank falls; `rest` becomes the rank inside it.
+__device__ __forceinline__ int find_rank(unsigned count, unsigned& rest) {
+  const int lane = threadIdx.x & 31;
+  unsigned incl = count;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += t;
   }
-  if (lane == 31) s.scan[0][warp] = incl;
+  const unsigned before = incl - count;
+  const int at = __ffs(__ballot_sync(0xffffffffu, before < rest && rest <= incl)) - 1;
+  rest -= __shfl_sync(0xffffffffu, before, at);
+  return at;
+}
+// Once all warps have counted: walks the bins of a histogram from the top.  `bin` holds the
+// `remaining`-th largest candidate, `rem` is the rank still wanted inside it.  32 groups of 64 bins first, summed by
+// their warps, then, in every warp alike, the groups and the bins of one of them.
+template <int T>
+__device__ __forceinline__ void sweep_pick(SweepShared& s, int level, unsigned remaining, unsigned& bin, unsigned& rem) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint2* const pairs = reinterpret_cast<const uint2*>(s.hist[level]);
   __syncthreads();
-  unsigned before = incl - mine;
-  for (int w = 0; w < warp; ++w) before += s.scan[0][w];
-  if (before < remaining && remaining <= before + mine) {
 #pragma unroll
-    for (int b = 0; b < kPer; ++b) {
-      if (before < remaining && remaining <= before + c[b]) {
-        s.bin = (unsigned)(top - b);
-        s.rem = remaining - before;
-      }
-      before += c[b];
-    }
+  for (int g = warp; g < 32; g += T / 32) {
+    const uint2 c = pairs[g * 32 + lane];
+    const unsigned sum = __reduce_add_sync(0xffffffffu, c.x + c.y);
+    if (lane == 0) s.scan[level][g] = sum;
   }
   __syncthreads();
+  unsigned rest = remaining;
+  const int group = 31 - find_rank(s.scan[level][31 - lane], rest), pair = 32 * group + 31 - lane;
+  const uint2 c = pairs[pair];
+  const int at = find_rank(c.x + c.y, rest);
+  bin = __shfl_sync(0xffffffffu, (unsigned)(2 * pair) + (rest <= c.y ? 1u : 0u), at);
+  rem = __shfl_sync(0xffffffffu, rest <= c.y ? rest : rest - c.y, at);
 }
 // The same for a cluster, in two steps of one warp: 32 groups of 64 bins, summed by their owners before the
 // barrier, then the bins of one group.
@@ -322,21 +327,8 @@ __device__ __forceinline__ void cluster_pick(SweepShared& s, int level, unsigned
   if (lane == 0) groups[warp] = sum;
   all_ctas<CL>();
   if (warp == 0) {
-    // lane l: the l-th of 32 counts from the top; where the wanted rank falls, and the rank inside it
-    auto find = [&](unsigned count, unsigned& rest) {
-      unsigned incl = count;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      const unsigned before = incl - count;
-      const int at = __ffs(__ballot_sync(0xffffffffu, before < rest && rest <= incl)) - 1;
-      rest -= __shfl_sync(0xffffffffu, before, at);
-      return at;
-    };
     unsigned rest = remaining, lo = 0, hi = 0;
-    const int group = 31 - find(count_of<CL>(&groups[31 - lane]), rest);
+    const int group = 31 - find_rank(count_of<CL>(&groups[31 - lane]), rest);
     const int pair = 32 * group + 31 - lane;
 #pragma unroll
     for (int r = 0; r < CL; ++r) {
@@ -344,7 +336,7 @@ __device__ __forceinline__ void cluster_pick(SweepShared& s, int level, unsigned
       lo += c.x;
       hi += c.y;
     }
-    const int at = find(lo + hi, rest);
+    const int at = find_rank(lo + hi, rest);
     if (lane == at) {
       s.bin = (unsigned)(2 * pair) + (rest <= hi ? 1u : 0u);
       s.rem = rest <= hi ? rest : rest - hi;
@@ -357,9 +349,14 @@ __device__ __forceinline__ void sweep_cta(const FinishArgs& a, SweepShared& s, c
   const int tid = threadIdx.x, rank = CL > 1 ? (int)(blockIdx.x % CL) : 0, n = pb.n;
   const float* x = pb.cols + (size_t)(vec % a.H) * a.col_stride;
   const float mean = 1.f / (float)n;
-  auto pick = [&](int level, unsigned remaining) {
-    if (CL > 1) cluster_pick<CL>(s, level, remaining);
-    else sweep_pick<T>(s, s.hist[level], remaining);
+  auto pick = [&](int level, unsigned remaining, unsigned& bin, unsigned& rem) {
+    if (CL > 1) {
+      cluster_pick<CL>(s, level, remaining);
+      bin = s.bin;
+      rem = s.rem;
+    } else {
+      sweep_pick<T>(s, level, remaining, bin, rem);
+    }
   };
   float acc[kAccs<T, CL, ROWS>] = {};
   sweep_from_memory<T, CL, ROWS>(x, n, rank, [&](float v, int k) {
@@ -368,8 +365,8 @@ __device__ __forceinline__ void sweep_cta(const FinishArgs& a, SweepShared& s, c
     atomicAdd(&s.hist[0][(__float_as_uint(v) >> 20) & 0x7ffu], 1u);
   });
   if (ROWS > 1 || rank == 0) warp_sums<T, CL>(acc, s.red[0][0], rank);
-  pick(0, (unsigned)max(1, n / 10));
-  const unsigned b1 = s.bin, rem1 = s.rem;
+  unsigned b1, rem1, b2, rem2;
+  pick(0, (unsigned)max(1, n / 10), b1, rem1);
 #pragma unroll
   for (float& m : acc) m = 0.f;
   sweep_from_memory<T, CL, ROWS>(x, n, rank, [&](float v, int k) {
@@ -378,10 +375,9 @@ __device__ __forceinline__ void sweep_cta(const FinishArgs& a, SweepShared& s, c
     else if (top == b1) atomicAdd(&s.hist[1][(u >> 9) & 0x7ffu], 1u);
   });
   if (ROWS > 1 || rank == 0) warp_sums<T, CL>(acc, s.red[1][0], rank);
-  pick(1, rem1);
+  pick(1, rem1, b2, rem2);
   if (rank == 0) {
     // entries of the threshold bin above sub-bin b2, and rem2 entries of sub-bin b2 itself
-    const unsigned b2 = s.bin, rem2 = s.rem;
     constexpr int kAccsBin = 1024 / T;
     float in_bin[kAccsBin] = {};
 #pragma unroll
@@ -404,22 +400,41 @@ __device__ __forceinline__ void sweep_cta(const FinishArgs& a, SweepShared& s, c
 // LONG: some vector has more than kLongFrom keys.  Short ones have a kernel of their own: with both forms in one
 // kernel a launch over 32 vectors of 4096 keys took a microsecond longer.
 template <int VEC, int T, int CL, bool LONG>
-__global__ void __launch_bounds__(T, T == 512 ? 3 : 1) finish(const __grid_constant__ FinishArgs a) {
+__global__ void __launch_bounds__(T, T == 256 ? 6 : T == 512 ? 3 : 1) finish(const __grid_constant__ FinishArgs a) {
   __shared__ union { SweepShared stats; SumShared<VEC> sum; } sh;
-  const bool stats = (int)blockIdx.x < a.n_stat_ctas;
+  // Few vectors (an SM each): all statistics, then all sums.  Many: problem after problem, its sums right behind its
+  // statistics, so that they find in L2 what these have read, and the last problem first: of the columns the scorer has just
+  // written L2 still holds the last ones.  (us after the scorer, all statistics before all sums / so: 32 layers of
+  // 32768 keys 93 / 82, 28 of 65536 141 / 126, 32 of 131072 343 / 329.  Clusters of four CTAs for many long vectors, fewer of
+  // them at a time, did not help: 140 and 351.  A batch of four prompts, 128 vectors, lost 2 us a layer by it.)
+  constexpr bool kFront = T == 1024;
+  int p, b = blockIdx.x;
+  bool stats;
+  if (kFront) {
+    stats = b < a.n_prob * a.stat_ctas;
+    const int per = stats ? a.stat_ctas : a.chunks;
+    if (!stats) b -= a.n_prob * a.stat_ctas;
+    p = b / per;
+    b -= p * per;
+  } else {
+    const int per = a.stat_ctas + a.chunks, at = b / per;
+    p = a.n_prob - 1 - at;
+    b -= at * per;
+    stats = b < a.stat_ctas;
+    if (!stats) b -= a.stat_ctas;
+  }
   pdl_trigger();
   if (stats)
-    for (int b = threadIdx.x; b < 2 * kSwBins; b += T) sh.stats.hist[0][b] = 0;
+    for (int i = threadIdx.x; i < 2 * kSwBins; i += T) sh.stats.hist[0][i] = 0;
   pdl_wait();
   __syncthreads();
   if (stats) {
-    const int vec = blockIdx.x / CL;
-    const Problem pb = problem_of(a, vec / a.H);
+    const int vec = p * a.H + b / CL;
+    const Problem pb = problem_of(a, p);
     if (LONG && pb.n > kLongFrom) sweep_cta<T, CL, kLongRows>(a, sh.stats, pb, vec);
     else sweep_cta<T, CL, 1>(a, sh.stats, pb, vec);
-  } else {
-    const int b = blockIdx.x - a.n_stat_ctas, p = b / a.chunks;
-    if (p < a.n_prob) sum_block<VEC, T>(a, sh.sum, p, b - p * a.chunks);   // the grid is whole clusters
+  } else if (p < a.n_prob) {                               // the grid is whole clusters
+    sum_block<VEC, T>(a, sh.sum, p, b);
   }
 }
 constexpr int kSumThreads = 256;     // many short blocks: 16 loads in flight per thread
@@ -538,19 +553,20 @@ accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int 
 
 template <int VEC>
 static cudaError_t launch_finish(FinishArgs& a, int longest, int sms, cudaStream_t st) {
-  a.chunks = (longest + kSumLanes * VEC - 1) / (kSumLanes * VEC);
-  const int sums = a.row_ent ? a.n_prob * a.chunks : 0;
+  a.chunks = a.row_ent ? (longest + kSumLanes * VEC - 1) / (kSumLanes * VEC) : 0;
+  const int sums = a.n_prob * a.chunks;
   if (!a.with_stats) return launch_pdl(sum_layers<VEC>, dim3(sums), dim3(kSumThreads), 0, st, a);
-  // An SM per vector: as many threads as a CTA can have.  More vectors than SMs: three CTAs an SM fill each
-  // other's gaps between barriers (512 vectors of 5003 / 32768 keys: 26 / 41 us with one of 1024 threads an
-  // SM, 15 / 31 with three of 512).  Few long vectors: clusters, as large as leaves room for all of them at once.
+  // An SM per vector: as many threads as a CTA can have.  More vectors than SMs: several CTAs an SM fill each
+  // other's gaps between barriers, six of 256 for short vectors, three of 512 for long ones.  us after the scorer, 32 layers of
+  // 32 heads with their sums, three of 512 / six of 256: 5003 keys 30 / 23.5, 20001 (28 layers) 70 / 58, 32768 82 / 70 to
+  // 80 (five of 256: 26, 63, 71 to 78).  Few long vectors: clusters, as large as leaves room for all of them at once.
   // us with one CTA / with clusters: 32 vectors of 33000 / 65536 / 131072 / 262144 keys 12.5, 10.5 / 17.5, 12.5 / 27.2,
   // 15.1 / 46.2, 20.1; 8 of 262144 46, 15; 64 of 262144 46, 29.  A cluster needs its SMs free in one GPC: of
   // eight CTAs 15 run at once (16 vectors of 262144 keys: 27.6), of four 32, of two 64.
   const int n_vec = a.n_prob * a.H, room = longest > kLongFrom ? sms * 7 / 8 / n_vec : 1;
   const int cl = 8 * n_vec <= sms * 3 / 4 && room >= 8 ? 8 : room >= 4 ? 4 : room >= 2 ? 2 : 1;
-  a.n_stat_ctas = n_vec * cl;
-  const dim3 grid((a.n_stat_ctas + sums + cl - 1) / cl * cl), wide(1024), narrow(512);
+  a.stat_ctas = a.H * cl;
+  const dim3 grid((n_vec * cl + sums + cl - 1) / cl * cl), wide(1024), narrow(512);
   if (cl == 8) return launch_cluster<8>(finish<VEC, 1024, 8, true>, grid, wide, 0, st, a);
   if (cl == 4) return launch_cluster<4>(finish<VEC, 1024, 4, true>, grid, wide, 0, st, a);
   if (cl == 2) return launch_cluster<2>(finish<VEC, 1024, 2, true>, grid, wide, 0, st, a);
@@ -558,7 +574,7 @@ static cudaError_t launch_finish(FinishArgs& a, int longest, int sms, cudaStream
     return n_vec <= sms ? launch_pdl(finish<VEC, 1024, 1, true>, grid, wide, 0, st, a)
                         : launch_pdl(finish<VEC, 512, 1, true>, grid, narrow, 0, st, a);
   return n_vec <= sms ? launch_pdl(finish<VEC, 1024, 1, false>, grid, wide, 0, st, a)
-                      : launch_pdl(finish<VEC, 512, 1, false>, grid, narrow, 0, st, a);
+                      : launch_pdl(finish<VEC, 256, 1, false>, grid, dim3(256), 0, st, a);
 }
 
 static FinishArgs finish_args(const Ctx& ctx, const float* cols, long long col_stride, int n, float* metrics) {
