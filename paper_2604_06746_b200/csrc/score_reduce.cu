@@ -399,42 +399,32 @@ __device__ __forceinline__ void sweep_cta(const FinishArgs& a, SweepShared& s, c
 }
 // LONG: some vector has more than kLongFrom keys.  Short ones have a kernel of their own: with both forms in one
 // kernel a launch over 32 vectors of 4096 keys took a microsecond longer.
-template <int VEC, int T, int CL, bool LONG>
+// FRONT: all statistics, then all sums: where every vector has an SM, and where there are no sums (a vector that follows
+// from the block's index alone leaves the sweeps the registers for another load: 1024 vectors of 131072 keys 219 us, 234 in the other order).
+// Else problem after problem, its sums right behind its statistics, so that they find in L2 what these have
+// read, and the last problem first: of the columns the scorer has just written L2 still holds the last ones.  (us after the
+// scorer, in front / so: 32 layers of 32768 keys 93 / 82, 28 of 65536 141 / 126, 32 of 131072 343 / 329.  A
+// batch of four prompts, 128 vectors, lost 2 us a layer by it.  Clusters of four for many long vectors, fewer of them at
+// a time, did not help: 140 and 351.)
+template <int VEC, int T, int CL, bool LONG, bool FRONT>
 __global__ void __launch_bounds__(T, T == 256 ? 6 : T == 512 ? 3 : 1) finish(const __grid_constant__ FinishArgs a) {
   __shared__ union { SweepShared stats; SumShared<VEC> sum; } sh;
-  // Few vectors (an SM each): all statistics, then all sums.  Many: problem after problem, its sums right behind its
-  // statistics, so that they find in L2 what these have read, and the last problem first: of the columns the scorer has just
-  // written L2 still holds the last ones.  (us after the scorer, all statistics before all sums / so: 32 layers of
-  // 32768 keys 93 / 82, 28 of 65536 141 / 126, 32 of 131072 343 / 329.  Clusters of four CTAs for many long vectors, fewer of
-  // them at a time, did not help: 140 and 351.  A batch of four prompts, 128 vectors, lost 2 us a layer by it.)
-  constexpr bool kFront = T == 1024;
-  int p, b = blockIdx.x;
-  bool stats;
-  if (kFront) {
-    stats = b < a.n_prob * a.stat_ctas;
-    const int per = stats ? a.stat_ctas : a.chunks;
-    if (!stats) b -= a.n_prob * a.stat_ctas;
-    p = b / per;
-    b -= p * per;
-  } else {
-    const int per = a.stat_ctas + a.chunks, at = b / per;
-    p = a.n_prob - 1 - at;
-    b -= at * per;
-    stats = b < a.stat_ctas;
-    if (!stats) b -= a.stat_ctas;
-  }
+  const int per = a.stat_ctas + a.chunks, at = FRONT ? 0 : blockIdx.x / per, in_front = FRONT ? a.n_prob * a.stat_ctas : a.stat_ctas;
+  const int b = blockIdx.x - at * per;                     // FRONT: of the launch; else of its problem
+  const bool stats = b < in_front;
   pdl_trigger();
   if (stats)
     for (int i = threadIdx.x; i < 2 * kSwBins; i += T) sh.stats.hist[0][i] = 0;
   pdl_wait();
   __syncthreads();
   if (stats) {
-    const int vec = p * a.H + b / CL;
-    const Problem pb = problem_of(a, p);
+    const int vec = FRONT ? blockIdx.x / CL : (a.n_prob - 1 - at) * a.H + b / CL;
+    const Problem pb = problem_of(a, vec / a.H);
     if (LONG && pb.n > kLongFrom) sweep_cta<T, CL, kLongRows>(a, sh.stats, pb, vec);
     else sweep_cta<T, CL, 1>(a, sh.stats, pb, vec);
-  } else if (p < a.n_prob) {                               // the grid is whole clusters
-    sum_block<VEC, T>(a, sh.sum, p, b);
+  } else {
+    const int c = b - in_front, p = FRONT ? c / a.chunks : a.n_prob - 1 - at;
+    if (p < a.n_prob) sum_block<VEC, T>(a, sh.sum, p, FRONT ? c - p * a.chunks : c);   // the grid is whole clusters
   }
 }
 constexpr int kSumThreads = 256;     // many short blocks: 16 loads in flight per thread
@@ -551,30 +541,39 @@ accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int 
 
 }  // namespace
 
+constexpr int kNarrowMany = 8192;    // keys up to which six CTAs of 256 are the better ones for many vectors, sums or not
+
 template <int VEC>
 static cudaError_t launch_finish(FinishArgs& a, int longest, int sms, cudaStream_t st) {
   a.chunks = a.row_ent ? (longest + kSumLanes * VEC - 1) / (kSumLanes * VEC) : 0;
   const int sums = a.n_prob * a.chunks;
   if (!a.with_stats) return launch_pdl(sum_layers<VEC>, dim3(sums), dim3(kSumThreads), 0, st, a);
   // An SM per vector: as many threads as a CTA can have.  More vectors than SMs: several CTAs an SM fill each
-  // other's gaps between barriers, six of 256 for short vectors, three of 512 for long ones.  us after the scorer, 32 layers of
-  // 32 heads with their sums, three of 512 / six of 256: 5003 keys 30 / 23.5, 20001 (28 layers) 70 / 58, 32768 82 / 70 to
-  // 80 (five of 256: 26, 63, 71 to 78).  Few long vectors: clusters, as large as leaves room for all of them at once.
-  // us with one CTA / with clusters: 32 vectors of 33000 / 65536 / 131072 / 262144 keys 12.5, 10.5 / 17.5, 12.5 / 27.2,
-  // 15.1 / 46.2, 20.1; 8 of 262144 46, 15; 64 of 262144 46, 29.  A cluster needs its SMs free in one GPC: of
-  // eight CTAs 15 run at once (16 vectors of 262144 keys: 27.6), of four 32, of two 64.
+  // other's gaps between barriers, six of 256 for short vectors, three of 512 for long ones.  us after the scorer, 32
+  // layers of 32 heads with their sums, three of 512 / six of 256: 5003 keys 30 / 23.5, 20001 (28 layers) 70 / 58, 32768 81 /
+  // 80 (window 8: 76 / 69; five of 256: 26, 63, 71 to 78); without sums 5003 keys 20 / 17, 8192 22.7 / 21.0, 16384 31.3 /
+  // 31.9, 32768 58 / 71, and of 8 layers, which three of 512 take in one go, 9.4 / 10.0.
+  // Few long vectors: clusters, as large as leaves room for all of them at once.
   const int n_vec = a.n_prob * a.H, room = longest > kLongFrom ? sms * 7 / 8 / n_vec : 1;
   const int cl = 8 * n_vec <= sms * 3 / 4 && room >= 8 ? 8 : room >= 4 ? 4 : room >= 2 ? 2 : 1;
   a.stat_ctas = a.H * cl;
   const dim3 grid((n_vec * cl + sums + cl - 1) / cl * cl), wide(1024), narrow(512);
-  if (cl == 8) return launch_cluster<8>(finish<VEC, 1024, 8, true>, grid, wide, 0, st, a);
-  if (cl == 4) return launch_cluster<4>(finish<VEC, 1024, 4, true>, grid, wide, 0, st, a);
-  if (cl == 2) return launch_cluster<2>(finish<VEC, 1024, 2, true>, grid, wide, 0, st, a);
-  if (longest > kLongFrom)
-    return n_vec <= sms ? launch_pdl(finish<VEC, 1024, 1, true>, grid, wide, 0, st, a)
-                        : launch_pdl(finish<VEC, 512, 1, true>, grid, narrow, 0, st, a);
-  return n_vec <= sms ? launch_pdl(finish<VEC, 1024, 1, false>, grid, wide, 0, st, a)
-                      : launch_pdl(finish<VEC, 256, 1, false>, grid, dim3(256), 0, st, a);
+  if (cl == 8) return launch_cluster<8>(finish<VEC, 1024, 8, true, true>, grid, wide, 0, st, a);
+  if (cl == 4) return launch_cluster<4>(finish<VEC, 1024, 4, true, true>, grid, wide, 0, st, a);
+  if (cl == 2) return launch_cluster<2>(finish<VEC, 1024, 2, true, true>, grid, wide, 0, st, a);
+  if (n_vec <= sms)
+    return longest > kLongFrom ? launch_pdl(finish<VEC, 1024, 1, true, true>, grid, wide, 0, st, a)
+                               : launch_pdl(finish<VEC, 1024, 1, false, true>, grid, wide, 0, st, a);
+  // Sums behind their statistics only where the statistics take several goes of three CTAs an SM.  us after the
+  // scorer, in front / behind: 5003 keys, 6 layers of 32 heads 9.5 / 12.5, 14 layers 17 / 14; 32768 keys, 10 layers 28 / 47,
+  // 20 58 / 63, 24 71 / 65; 65536 keys, 14 82 / 86, 20 119 / 111, 24 141 / 128; 131072 keys, 10 109 / 131, 20 220 / 219.
+  const bool several = n_vec > (longest > kNarrowMany ? 5 : 3) * sms;
+  if (!sums || !several)
+    return longest > kLongFrom ? launch_pdl(finish<VEC, 512, 1, true, true>, grid, narrow, 0, st, a)
+           : longest > kNarrowMany || n_vec <= 3 * sms ? launch_pdl(finish<VEC, 512, 1, false, true>, grid, narrow, 0, st, a)
+                                                        : launch_pdl(finish<VEC, 256, 1, false, true>, grid, dim3(256), 0, st, a);
+  return longest > kLongFrom ? launch_pdl(finish<VEC, 512, 1, true, false>, grid, narrow, 0, st, a)
+                             : launch_pdl(finish<VEC, 256, 1, false, false>, grid, dim3(256), 0, st, a);
 }
 
 static FinishArgs finish_args(const Ctx& ctx, const float* cols, long long col_stride, int n, float* metrics) {

@@ -1,5 +1,6 @@
 """Sums and head statistics of more (layer, head) vectors than SMs in one launch, at the edges of its forms (blocks of
-512 keys, six CTAs an SM up to 32768 keys, three beyond): the bits of the separate calls."""
+512 keys; all statistics first, or each layer's sums behind its own; three or six CTAs an SM): the bits of the
+separate calls."""
 import pytest
 import torch
 
@@ -8,7 +9,8 @@ from tests.test_gpu_prefill_call import OUT, prompt, step_by_step
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("seq,n_layers", [(130, 5), (512, 33), (516, 9), (4097, 6), (32768, 5), (32769, 5), (33000, 7)])
+@pytest.mark.parametrize("seq,n_layers", [(130, 5), (512, 33), (513, 14), (4097, 13), (8193, 24), (32768, 7),
+                                          (33000, 24)])
 def test_one_launch_equals_the_separate_calls(cuda_device, seq, n_layers):
     one, args = prompt(cuda_device, seq, n_layers, 100)
     ref, _ = prompt(cuda_device, seq, n_layers, 100)
