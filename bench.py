@@ -374,14 +374,14 @@ def compaction_figures(wl, kv_budget, compact_ms_per_step, peaks):
 
 def launches_per_step(wl, flags):
     from paper_2604_06746_b200 import binding
-    # one call for all layers: the tensor-core scorer (one launch per 32 layers, both passes) or the two
-    # CUDA-core passes, then one launch for the sums over heads; layer by layer the same per layer.  Per
+    # one call for all layers: the tensor-core scorer (one launch per 32 layers, both passes) or the
+    # CUDA-core one (one launch up to 4096 keys, else one per pass), then one launch for the sums over heads; layer by layer the same per layer.  Per
     # step: head statistics of all layers, centrality at the pivot, all selections, one K/V gather over
     # all layers, hidden states, positions
     tc = wl.dtype == "bf16" and not flags & binding.FLAG_FORCE_SIMT
     together = not flags & (binding.FLAG_NO_HEAD_STATS | binding.FLAG_FORCE_SIMT)
     stats = 0 if flags & binding.FLAG_NO_HEAD_STATS else 1
-    scorer = 1 if tc else 2
+    scorer = 1 if tc or wl.seq <= 4096 else 2
     if together:
         scoring = (-(-wl.n_layers // 32) if tc else scorer) + 1
     else:
