@@ -38,7 +38,7 @@ struct Workspace {
   float* head_part;     // [kMaxStatLayers][H][4] per-(layer, head) {sum of squared deviations from 1/n, top-k mass}
   int* stat_ctr;        // [kMaxStatLayers] and, behind it, chunk_ctr [n_pad / kKeyTile]: zero between launches
   int* chunk_ctr;
-  unsigned long long* xch;   // [kXchWords] tagged words the resident scorer's CTAs exchange; zero at first
+  unsigned long long* xch;   // [kXchWords] tagged words the CTAs of the one-pass scorers exchange; zero at first
   size_t zero_bytes;    // from `status` on: what starts from zero
   size_t bytes;
 };

@@ -10,8 +10,8 @@ namespace cg = cooperative_groups;
 namespace {
 
 // ---- what follows the scorer passes of a layer, of several layers or of a packed batch ----------
-// One launch: a CTA or a cluster per (problem, head) vector first (Eq. 5-6), then blocks that sum 128 x VEC keys over
-// the heads (Eq. 2) and carry the centrality (Eq. 3).  Every sum has a fixed order.
+// One launch: a CTA or a cluster per (problem, head) vector (Eq. 5-6), and blocks that sum 128 x VEC keys over the
+// heads (Eq. 2) and carry the centrality (Eq. 3); which come first is the launch's choice.  Every sum has a fixed order.
 struct FinishArgs {
   const float* cols;                   // problem p, head h, key j at cols + p * layer_stride + h * col_stride + j
   long long layer_stride, col_stride;
@@ -180,7 +180,8 @@ __device__ __forceinline__ void head_done(const FinishArgs& a, int vec, float me
 // Bound by latency up to some 100 vectors, then by the shared-memory atomics and, where the vectors exceed
 // L2 together, by reading them twice (1024 vectors of 131072 keys: 2 x 537 MB, 164 of 208 us).  One histogram,
 // without copies for the lanes: same-address hits cost less than clearing and summing copies, whether the
-// values concentrate or not (1024 vectors of 5003 / 32768 keys: 41 / 85 us with four, 20 / 59 with one).
+// values concentrate or not (1024 vectors of 5003 / 32768 keys: 41 / 85 us with four, 20 / 59 with one,
+// both with three CTAs of 512 an SM).
 //
 // Few long vectors are dealt out over clusters of CL CTAs, which count their own entries; the histograms are
 // read through distributed shared memory, and the first CTA adds up.  A CTA takes 0.15 us per 1000 keys, mostly
