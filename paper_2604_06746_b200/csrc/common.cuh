@@ -18,8 +18,8 @@ constexpr int kMaxStatLayers = 128;   // layers one batched head-statistics call
 constexpr int kMaxGatherLayers = 128; // layers one multi-layer gather may cover (their pointers are a kernel argument)
 constexpr int kQueueUnits = 256;      // (KV group, row block) units of one problem the tensor-core scorer can hold
 constexpr int kCtlInts = 64 + 2 * kMaxBatch * kQueueUnits;   // its control block: tickets, arrivals, ready flags
-constexpr int kXchSlots = 16;          // units of an exchange ring of the resident scorer's teams
-constexpr int kXchWords = 2 * kMaxSms * kXchSlots * 64;   // their tagged 64-bit words
+constexpr int kXchSlots = 17;          // units of an exchange ring of the resident scorer's teams
+constexpr int kXchWords = 2 * kMaxSms * 16 * 64;          // their tagged 64-bit words, and room
 constexpr int kCtlExit = 1, kCtlTag = 2;   // in the control block: CTAs that are done; last tag of the exchange words
 constexpr unsigned long long kWaitCycles = 1000000000ull;   // bound of a device wait, about 0.5 s at the maximum SM clock
 constexpr int kMergeGroup = 6;         // partials of a row merged together

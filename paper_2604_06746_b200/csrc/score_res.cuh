@@ -48,7 +48,7 @@ constexpr int kRefKeys = 8;            // keys a row's common reference looks at
 constexpr float kSumUnit = 67108864.f, kSumLimit = 2097152.f;
 constexpr unsigned long long kSumCount = 1ull << 56, kSumOver = 1ull << 55, kSumBias = 1ull << 47;
 static_assert(kMaxSms * 2097152ull * 67108864ull < kSumOver && kMaxSms * 2 * kSumBias < kSumCount, "summed words");
-static_assert(kXchSlots == 2 * kResRing, "a slot of tagged words is free again after two rings");
+static_assert(kXchSlots > 2 * kResRing && 2 * kMaxSms * kXchSlots * kResRows <= kXchWords, "slots of tagged words");
 
 struct ResProblem {
   float* cols;                         // output of head 0, key 0
@@ -165,9 +165,11 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
     if ((unsigned long long)(now - t0) > kWaitCycles) { *abort_flag = 1; return false; }
     return true;
   };
-  // Tagged words of unit u: [team][slot][rank][row], log-sum-exps, then entropies.  A slot is used again two rings
-  // later: whoever gets there has its column sums of a ring before behind it, so that every CTA has
-  // published those, and is itself done with the unit a ring before them.
+  // Tagged words of unit u: [team][slot][rank][row], log-sum-exps, then entropies.  Who publishes unit v has summed, so
+  // known, unit v - kResRing; so every CTA had published that one, hence summed and known unit v - 2 kResRing.  Knowing
+  // a unit means that its log-sum-exps have been read.  The CTA that leaves its entropies reads those afterwards, before it
+  // looks at the next unit: all words are read of units before v - 2 kResRing, so that a slot must
+  // last one unit longer than two rings.
   constexpr size_t kEntWords = kXchWords / 2;
   auto tagged_word = [&](unsigned u, int from, int row) {
     return p.xch + ((size_t)((team * kXchSlots + (int)(u % kXchSlots)) * G + from) * R + row);

@@ -29,12 +29,16 @@ def test_logits_far_above_the_references(cuda_device, H, Hkv, N, scale):
     score(cuda_device, H, Hkv, 128, 8, N, scale)
 
 
-@pytest.mark.parametrize("Hkv", [8, 1])
-def test_layers_repetition_and_replay(cuda_device, Hkv):
+@pytest.mark.parametrize("Hkv,N", [
+    (8, 4200), (1, 4200),
+    (4, 4200), (4, 9400),                                                    # teams of 37, one and two tiles a CTA
+    (1, 70000), (2, 40000),                                                  # summed, four and five tiles a CTA
+])
+def test_layers_repetition_and_replay(cuda_device, Hkv, N):
     """Layers of one call, the same call again, and a captured call replayed on other inputs: the bits of single
     layers (more layers than a launch holds; the CTAs' tagged words pass from call to call)."""
     from paper_2604_06746_b200 import binding
-    L, H, d, w, N = 34, 4 * Hkv, 64, 8, 4200
+    L, H, d, w = 34, 4 * Hkv, 64, 8
     g = torch.Generator(device=cuda_device)
     g.manual_seed(11)
     qs = [torch.randn((H, w, d), generator=g, device=cuda_device).bfloat16() for _ in range(L)]
