@@ -50,6 +50,7 @@ Workspace carve_workspace(const structkv_config& cfg, void* base) {
   w.ctl = (int*)take(kCtlInts * sizeof(int));
   w.stat_ctr = (int*)take(kMaxStatLayers * sizeof(int));
   w.chunk_ctr = (int*)take(n_pad / kKeyTile * sizeof(int));
+  w.ctr_bytes = off;
   w.xch = (unsigned long long*)take(kXchWords * sizeof(unsigned long long));
   w.zero_bytes = off;
   w.row_part = (float2*)take(std::max(simt_part_entries(cfg, 1), tc_part_tasks(cfg, 1, false) * kRowBlock) * sizeof(float2));
@@ -144,6 +145,7 @@ structkv_status structkv_create(structkv_ctx** ctx_out, const structkv_config* c
   c.rows_pad = rows_pad_of(*cfg);
   c.n_pad = (int)align_up((size_t)cfg->max_seq, kKeyTile);
   c.tc = nullptr;
+  c.old_words = false;
   if (cudaGetDevice(&c.device) != cudaSuccess ||
       cudaDeviceGetAttribute(&c.sm_count, cudaDevAttrMultiProcessorCount, c.device) != cudaSuccess ||
       cudaMemset(c.ws.status, 0, c.ws.zero_bytes) != cudaSuccess ||
@@ -730,8 +732,10 @@ extern "C" structkv_status structkv_score_layer_static(
   c.rows_pad = rows_pad_of(*cfg);
   c.n_pad = (int)align_up((size_t)cfg->max_seq, kKeyTile);
   c.tc = cfg->dtype == STRUCTKV_BF16 ? slot->tc : nullptr;
-  // The scratch keeps the previous call's contents; the status word and the scorer's counters start from zero.
-  if (cudaMemsetAsync(c.ws.status, 0, c.ws.zero_bytes, (cudaStream_t)stream) != cudaSuccess) return STRUCTKV_ERR_CUDA;
+  // The scratch keeps the previous call's contents: the status word and the scorer's counters start from zero, and so do
+  // the exchange words where a scorer uses them (1.4 MB, most calls' clearing would be nothing else).
+  c.old_words = true;
+  if (cudaMemsetAsync(c.ws.status, 0, c.ws.ctr_bytes, (cudaStream_t)stream) != cudaSuccess) return STRUCTKV_ERR_CUDA;
   return structkv_score_layer(&tmp, q_window, k, k_stride_head, k_stride_token, n_keys, scale, lambda,
                               s_out, c_inout, head_cols_out, metrics_out, flags, stream);
 }

@@ -19,7 +19,8 @@ constexpr int kMaxGatherLayers = 128; // layers one multi-layer gather may cover
 constexpr int kQueueUnits = 256;      // (KV group, row block) units of one problem the tensor-core scorer can hold
 constexpr int kCtlInts = 64 + 2 * kMaxBatch * kQueueUnits;   // its control block: tickets, arrivals, ready flags
 constexpr int kXchSlots = 17;          // units of an exchange ring of the resident scorer's teams
-constexpr int kXchWords = 2 * kMaxSms * 16 * 64;          // their tagged 64-bit words, and room
+constexpr int kResRows = 32;           // score rows of one of its units, at most
+constexpr int kXchWords = 2 * kMaxSms * kXchSlots * kResRows;   // the teams' tagged 64-bit words; the CUDA-core scorer needs fewer
 constexpr int kCtlExit = 1, kCtlTag = 2;   // in the control block: CTAs that are done; last tag of the exchange words
 constexpr unsigned long long kWaitCycles = 1000000000ull;   // bound of a device wait, about 0.5 s at the maximum SM clock
 constexpr int kMergeGroup = 6;         // partials of a row merged together
@@ -38,6 +39,7 @@ struct Workspace {
   float* head_part;     // [kMaxStatLayers][H][4] per-(layer, head) {sum of squared deviations from 1/n, top-k mass}
   int* stat_ctr;        // [kMaxStatLayers] and, behind it, chunk_ctr [n_pad / kKeyTile]: zero between launches
   int* chunk_ctr;
+  size_t ctr_bytes;     // from `status` to here: counters
   unsigned long long* xch;   // [kXchWords] tagged words the CTAs of the one-pass scorers exchange; zero at first
   size_t zero_bytes;    // from `status` on: what starts from zero
   size_t bytes;
@@ -52,6 +54,7 @@ struct Ctx {
   int w_pad;            // rows a head occupies in a scorer's row blocks: w up to a power of two, at least 8
   int rows_pad;         // rows per KV group (heads at w_pad rows) padded to kRowBlock, times H_kv
   int n_pad;            // max_seq rounded up to kKeyTile
+  bool old_words;       // the exchange words hold anything (a call's own context): who uses them clears them first
   void* tc;             // tensor-core scorer state (tensor-map encoder), owned by score_tc.cu
   struct HostSlot* slot = nullptr;   // where the device leaves the pivot for the host (api.cu), taken at first use
 };
@@ -60,6 +63,11 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // Carves the workspace; with base == nullptr only the size is computed.
 Workspace carve_workspace(const structkv_config& cfg, void* base);
+
+// What a launch that uses the exchange words does first.
+inline cudaError_t clean_words(const Ctx& ctx, cudaStream_t st) {
+  return ctx.old_words ? cudaMemsetAsync(ctx.ws.xch, 0, kXchWords * sizeof(unsigned long long), st) : cudaSuccess;
+}
 
 // ---- launchers (each returns cudaGetLastError() of its launches) -------------------------
 // Both scorer passes over `n` problems: layers of one shape, or (tensor cores only) the sequences of a

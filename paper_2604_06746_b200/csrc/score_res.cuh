@@ -38,7 +38,6 @@ namespace skv {
 constexpr int kResSubs = 4;            // compute warps of a lane quarter
 constexpr int kResWarps = 4 * kResSubs;
 constexpr int kResThreads = (kResWarps + 4) * 32;   // 20 warps: the most that fit at 96 registers a thread
-constexpr int kResRows = 32;           // score rows of a unit, at most
 constexpr int kResChunk = 32;          // keys are dealt out to a team's CTAs in chunks of 32
 constexpr int kResRing = 8;            // units a CTA may have between its statistics and its last column sum
 constexpr int kDirectTeam = 40;        // CTAs of a team that merges partials directly
@@ -48,7 +47,7 @@ constexpr int kRefKeys = 8;            // keys a row's common reference looks at
 constexpr float kSumUnit = 67108864.f, kSumLimit = 2097152.f;
 constexpr unsigned long long kSumCount = 1ull << 56, kSumOver = 1ull << 55, kSumBias = 1ull << 47;
 static_assert(kMaxSms * 2097152ull * 67108864ull < kSumOver && kMaxSms * 2 * kSumBias < kSumCount, "summed words");
-static_assert(kXchSlots > 2 * kResRing && 2 * kMaxSms * kXchSlots * kResRows <= kXchWords, "slots of tagged words");
+static_assert(kXchSlots > 2 * kResRing, "slots of tagged words");
 
 struct ResProblem {
   float* cols;                         // output of head 0, key 0

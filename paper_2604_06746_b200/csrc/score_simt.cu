@@ -367,7 +367,7 @@ cudaError_t launch_typed(const Ctx& ctx, const SimtArgs& a, int layers, cudaStre
   const int room = (int)(std::min((long long)per_sm[dev].load(std::memory_order_relaxed) * ctx.sm_count, kXchWords / (2ll * kSmRows)) / per_layer);
   if (span == 1 && a.n_keys_tiles == a.parts && room >= 1) {
     const int launches = (layers + room - 1) / room;
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = clean_words(ctx, st);
     for (int i = 0; i < launches && e == cudaSuccess; ++i) {
       const int lo = i * layers / launches, n = (i + 1) * layers / launches - lo;
       SimtArgs b = a;

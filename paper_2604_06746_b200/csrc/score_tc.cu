@@ -246,7 +246,7 @@ void tc_destroy(Ctx& ctx) {
 
 cudaError_t launch_score_tc(const Ctx& ctx, const ScoreCall& a, cudaStream_t st) {
   if (res_supported(ctx, a)) {
-    cudaError_t e = cudaSuccess;
+    cudaError_t e = clean_words(ctx, st);
     for (int l = 0; l < a.n && e == cudaSuccess; l += kMaxBatch) e = launch_score_res(ctx, a, l, std::min(kMaxBatch, a.n - l), st);
     // where the device does not give this process all of its SMs at once, the general scorer does it
     if (e != cudaErrorCooperativeLaunchTooLarge) return e;

@@ -50,6 +50,13 @@ def test_workspace_bytes(B):
         assert B.workspace_bytes(bad) == 0
 
 
+@pytest.mark.parametrize("shape,longest", [((32, 8, 128, 64), 56064), ((32, 8, 128, 8), 56064)])
+def test_what_the_static_scratch_takes(B, shape, longest):
+    """The scratch grows and shrinks with the workspace: the documented longest sequence, and the next is refused."""
+    assert B.workspace_bytes(B.Config(*shape, longest, B.BF16)) <= B.STATIC_SCRATCH_BYTES
+    assert B.workspace_bytes(B.Config(*shape, longest + 1, B.BF16)) > B.STATIC_SCRATCH_BYTES
+
+
 def test_create_rejects_bad_arguments_on_the_host(B):
     h = ctypes.c_void_p()
     cfg = B.Config(8, 2, 64, 32, 2048, B.FP32)

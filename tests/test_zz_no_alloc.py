@@ -91,3 +91,53 @@ def test_static_scratch_scoring_refuses_configurations_beyond_its_scratch(cuda_d
     assert rc == binding.ERR_WORKSPACE
     assert binding.lib.structkv_score_layer_static(None, None, None, 0, 0, 0, 1.0, 0.9, None, None, None, None,
                                                    0, None) == binding.ERR_INVALID_ARG
+
+
+def test_static_scratch_serves_every_scorer_in_any_order(cuda_device):
+    """Calls of different scorers and lengths in a row, each on what the one before left in the scratch: the bits a context
+    gives.  (Window 8 from 4096 keys on and short fp32 layers exchange words whose place depends on max_seq.)"""
+    from paper_2604_06746_b200 import binding
+    g = torch.Generator(device=cuda_device)
+    g.manual_seed(3)
+    forms = [(32, 8, 128, 8, 5000, torch.bfloat16, 0), (8, 2, 64, 32, 2048, torch.float32, 0),
+             (32, 8, 128, 64, 9000, torch.bfloat16, 0), (4, 1, 128, 8, 30000, torch.bfloat16, 0),
+             (32, 8, 128, 8, 20000, torch.bfloat16, 0), (32, 8, 128, 8, 700, torch.bfloat16, binding.FLAG_FORCE_SIMT)]
+    for H, Hkv, d, w, n, dt, flags in forms + forms[::-1] + forms:
+        q = torch.randn((H, w, d), generator=g, device=cuda_device).to(dt)
+        k = torch.randn((Hkv, n, d), generator=g, device=cuda_device).to(dt)
+        ctx = binding.Context(H, Hkv, d, w, n, dt, cuda_device)
+        out = [(torch.zeros(n, device=cuda_device), torch.zeros(3, device=cuda_device)) for _ in range(2)]
+        ctx.score_layer(q, k, 0.1, *out[0], flags=flags)
+        binding.score_layer_static(H, Hkv, d, w, n, q, k, 0.1, *out[1], flags=flags)
+        assert ctx.poll_device_status() == binding.OK
+        assert all(torch.equal(a, b) for a, b in zip(*out)), (H, Hkv, d, w, n, dt)
+        ctx.close()
+
+
+@pytest.mark.parametrize("w,n,most", [(64, 5000, 96 << 10), (8, 4000, 96 << 10), (8, 5000, 3 << 19)])
+def test_static_scratch_clears_what_the_scorer_uses(cuda_device, w, n, most):
+    """Bytes a captured call clears: its counters, and the exchange words only where its scorer has CTAs exchange them."""
+    from cuda.bindings import runtime as rt
+
+    from paper_2604_06746_b200 import binding
+    q = torch.zeros((32, w, 128), device=cuda_device, dtype=torch.bfloat16)
+    k = torch.zeros((8, n, 128), device=cuda_device, dtype=torch.bfloat16)
+    s, m = torch.zeros(n, device=cuda_device), torch.zeros(3, device=cuda_device)
+    args = (32, 8, 128, w, n, q, k, 0.1, s, m)
+    binding.score_layer_static(*args)                      # one-time set-up
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        binding.score_layer_static(*args)
+    raw = rt.cudaGraph_t(init_value=int(graph.raw_cuda_graph()))
+    err, _, count = rt.cudaGraphGetNodes(raw)
+    assert err == rt.cudaError_t.cudaSuccess
+    err, nodes, _ = rt.cudaGraphGetNodes(raw, count)
+    assert err == rt.cudaError_t.cudaSuccess
+    cleared = 0
+    for node in nodes:
+        if rt.cudaGraphNodeGetType(node)[1] == rt.cudaGraphNodeType.cudaGraphNodeTypeMemset:
+            p = rt.cudaGraphMemsetNodeGetParams(node)[1]
+            cleared += p.width * p.elementSize * p.height
+    del graph
+    assert 0 < cleared <= most
