@@ -199,9 +199,9 @@ inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 bloc
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
-// The same for a kernel whose blocks wait for one another: all of them run at once, or the launch is refused.
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_cooperative(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+// The same for a kernel of one argument whose blocks wait for one another: all of them run at once, or the launch is refused.
+template <typename Arg>
+inline cudaError_t launch_cooperative(void (*kernel)(Arg), dim3 grid, dim3 block, size_t smem, cudaStream_t st, const Arg& arg) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -214,7 +214,8 @@ inline cudaError_t launch_cooperative(void (*kernel)(KArgs...), dim3 grid, dim3 
   attr[1].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+  void* args[1] = {const_cast<Arg*>(&arg)};              // no copies of a parameter block of kilobytes
+  return cudaLaunchKernelExC(&cfg, (const void*)kernel, args);
 }
 
 __device__ __forceinline__ void add_to(float4& s, const float4& v) { s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }

@@ -93,10 +93,7 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
         !tc_encode3(ctx, &p.map_k[i], a.k[first + i], a.n_keys, cfg.n_kv_heads, s_tok, s_head, kResChunk, 1))
       return cudaErrorInvalidValue;
     ResProblem& pb = p.prob[i];
-    pb.key0 = 0;
     pb.n_keys = a.n_keys;
-    pb.map = i;
-    pb.head0 = 0;
     pb.cols = a.cols + (size_t)(first + i) * a.cols_layer_stride;
     const float c2 = a.scale[first + i] * kLog2e;
     pb.negate = c2 < 0.f;

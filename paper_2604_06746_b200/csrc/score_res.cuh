@@ -51,8 +51,7 @@ static_assert(kXchSlots > 2 * kResRing, "slots of tagged words");
 
 struct ResProblem {
   float* cols;                         // output of head 0, key 0
-  int key0, n_keys;                    // rows of the K tensor
-  int map, head0;                      // tensor maps; first head in the Q tensor
+  int n_keys;
   float c2;                            // |scale| * log2(e), at least 1e-30
   int negate;
 };
@@ -202,7 +201,7 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
       bool ok = true;
       for (Walk w = walk_from(); w.pi < n_prob && ok; walk_on(w)) {
         const ResShare s = prob_s[w.pi];
-        const CUtensorMap* map_k = &p.map_k[s.p.map];
+        const CUtensorMap* map_k = &p.map_k[w.pi];
         for (int a = 0; a < s.c && ok; a += 4) {
           const int sg = kt % kStages, n = min(4, s.c - a);
           ok = mbar_wait_producer(bar(L::kKEmpty + sg), ((kt / kStages) & 1u) ^ 1u, abort_flag, kWaitCycles);
@@ -212,15 +211,15 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
           for (int q = 0; q < n; ++q)
             for (int c = 0; c < L::kSub; ++c)
               tma_load_3d_hint(base + sg * L::kTile + c * L::kTileSub + q * (kResChunk * 128), map_k, bar(L::kKFull + sg),
-                               c * 64, s.p.key0 + (s.lo + a + q) * kResChunk, w.g, pol_stream);
+                               c * 64, (s.lo + a + q) * kResChunk, w.g, pol_stream);
           ++kt;
           if (a > 0) continue;
           ok = mbar_wait_producer(bar(L::kQEmpty + (qn & 1)), ((qn >> 1) & 1u) ^ 1u, abort_flag, kWaitCycles);
           if (!ok) break;
           mbar_expect_tx(bar(L::kQFull + (qn & 1)), L::kQ);
           for (int c = 0; c < L::kSub; ++c)
-            tma_load_3d_hint(base + L::kQOff + (qn & 1) * L::kQ + c * L::kQSub, &p.map_q[s.p.map], bar(L::kQFull + (qn & 1)),
-                             c * 64, 0, s.p.head0 + w.g * p.group, pol_keep);
+            tma_load_3d_hint(base + L::kQOff + (qn & 1) * L::kQ + c * L::kQSub, &p.map_q[w.pi], bar(L::kQFull + (qn & 1)),
+                             c * 64, 0, w.g * p.group, pol_keep);
           ++qn;
         }
       }
@@ -627,20 +626,7 @@ cudaError_t res_launch(const ResParams<MAXP>& p, int device, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     ready.fetch_or(bit, std::memory_order_release);
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(p.team * p.teams);
-  cfg.blockDim = dim3(kResThreads);
-  cfg.dynamicSmemBytes = kAlloc;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeCooperative;
-  attr[1].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  void* args[1] = {const_cast<ResParams<MAXP>*>(&p)};
-  return cudaLaunchKernelExC(&cfg, (const void*)kern, args);
+  return launch_cooperative(kern, dim3(p.team * p.teams), dim3(kResThreads), kAlloc, st, p);
 }
 #endif  // __CUDACC__
 
