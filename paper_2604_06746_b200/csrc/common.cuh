@@ -20,7 +20,10 @@ constexpr int kQueueUnits = 256;      // (KV group, row block) units of one prob
 constexpr int kCtlInts = 64 + 2 * kMaxBatch * kQueueUnits;   // its control block: tickets, arrivals, ready flags
 constexpr int kXchSlots = 17;          // units of an exchange ring of the resident scorer's teams
 constexpr int kResRows = 32;           // score rows of one of its units, at most
-constexpr int kXchWords = 2 * kMaxSms * kXchSlots * kResRows;   // the teams' tagged 64-bit words; the CUDA-core scorer needs fewer
+constexpr int kRefSlots = 32;          // units of a ring of common references
+// Tagged 64-bit words: two for every row and CTA of the teams' rings (the CUDA-core scorer needs fewer), then the rings of
+// references, of three teams at most.
+constexpr int kXchPairs = kMaxSms * kXchSlots * kResRows, kXchWords = 2 * kXchPairs + 3 * kRefSlots * kResRows;
 constexpr int kCtlExit = 1, kCtlTag = 2;   // in the control block: CTAs that are done; last tag of the exchange words
 constexpr unsigned long long kWaitCycles = 1000000000ull;   // bound of a device wait, about 0.5 s at the maximum SM clock
 constexpr int kMergeGroup = 6;         // partials of a row merged together

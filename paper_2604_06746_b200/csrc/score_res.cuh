@@ -14,11 +14,14 @@
 //   direct (teams of up to kDirectTeam)  every CTA leaves its partials as words that carry a tag, reads
 //           all of its mates' and merges them in order
 //   summed (larger teams)                a row has one reference for the whole team (its largest logit over a few
-//           sampled keys, res_refs), so that sums of 2^(x - ref) add up; they do as fixed-point integers, in
-//           any order the same bits, in words whose top byte counts the CTAs.  Where a CTA's sum leaves the range
+//           sampled keys; one CTA finds a unit's, some units ahead, and leaves them as tagged words), so that sums of
+//           2^(x - ref) add up; they do as fixed-point integers, in any order the same bits, in words whose
+//           top byte counts the CTAs.  Where a CTA's sum leaves the range
 //           (a logit 2^20 above the reference) it marks the word, and the team takes the direct way for that unit.
-// Direct teams of 74 read too many words: 65536 keys 506 us for 16 layers, summed 427; of 37 (20011 keys, 32
-// layers) 307 and 279, but a layer by itself then waits for res_refs: 32768 keys 32.8 direct, 41.7 summed.
+// Direct teams of 74 read too many words: 65536 keys 506 us for 16 layers, summed 427.  The references came from a launch of
+// their own at first, which a layer by itself waited for; us with it / with them found inside, one layer: 8 KV heads
+// 40000 keys 43.0 / 36.6, 98304 64.6 / 60.1, 262144 150 / 135; 4 KV heads 40000 32.9 / 26.7, 131072 49.5 / 44.4;
+// one KV head 32768 24.4 / 18.5; a layer of 32 with 8 KV heads of 262144 keys 135 / 121.
 // Which keys a CTA holds depends on the sequence length, the KV heads and the SM count alone: results depend
 // neither on timing nor on how many layers a call has.
 //
@@ -41,16 +44,19 @@ constexpr int kResThreads = (kResWarps + 4) * 32;   // 20 warps: the most that f
 constexpr int kResChunk = 32;          // keys are dealt out to a team's CTAs in chunks of 32
 constexpr int kResRing = 8;            // units a CTA may have between its statistics and its last column sum
 constexpr int kDirectTeam = 40;        // CTAs of a team that merges partials directly
-constexpr int kRefKeys = 8;            // keys a row's common reference looks at: the first and the last before the window
+constexpr int kRefAhead = 2 * kResRing;   // a unit's common references are found so many units before
 // A row's summed words: [63:56] CTAs so far, [55] somebody's sum is out of range, below it sum Z in units of
 // 2^-26; [63:56] CTAs, below it sum (U + 2^21) in units of 2^-26.
 constexpr float kSumUnit = 67108864.f, kSumLimit = 2097152.f;
 constexpr unsigned long long kSumCount = 1ull << 56, kSumOver = 1ull << 55, kSumBias = 1ull << 47;
 static_assert(kMaxSms * 2097152ull * 67108864ull < kSumOver && kMaxSms * 2 * kSumBias < kSumCount, "summed words");
 static_assert(kXchSlots > 2 * kResRing, "slots of tagged words");
+static_assert(kRefSlots >= kRefAhead + 2 * kResRing && kRefAhead <= kDirectTeam && 4 * (kDirectTeam + 1) > kMaxSms,
+              "rings of references");
 
 struct ResProblem {
   float* cols;                         // output of head 0, key 0
+  const __nv_bfloat16 *q, *k;
   int n_keys;
   float c2;                            // |scale| * log2(e), at least 1e-30
   int negate;
@@ -66,9 +72,8 @@ struct alignas(64) ResParams {
   int* ctl;
   unsigned long long* xch;             // tagged words, kXchWords
   unsigned long long* sums;            // summed: [unit of the launch][kResRows] x {Z, U}; NULL: direct
-  const float* refs;                   // [unit][kResRows] common references
   float* row_ent;                      // [problem][KV group][kRowBlock] entropy of a row, nats (0: no row)
-  long long col_stride;
+  long long col_stride, k_stride_head, k_stride_token;   // elements
   int* status;
 };
 
@@ -168,7 +173,7 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
   // a unit means that its log-sum-exps have been read.  The CTA that leaves its entropies reads those afterwards, before it
   // looks at the next unit: all words are read of units before v - 2 kResRing, so that a slot must
   // last one unit longer than two rings.
-  constexpr size_t kEntWords = kXchWords / 2;
+  constexpr size_t kEntWords = kXchPairs;
   auto tagged_word = [&](unsigned u, int from, int row) {
     return p.xch + ((size_t)((team * kXchSlots + (int)(u % kXchSlots)) * G + from) * R + row);
   };
@@ -191,6 +196,21 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
     const float2 pt = stat_partial(fold(u, row, top));
     put_word(tagged_word(u, rank, row), tagged(pt.x, tag0 + u));
     put_word(tagged_word(u, rank, row) + kEntWords, tagged(pt.y, tag0 + u));
+  };
+
+  // Summed: the row's common reference in unit u of this team.  A slot is used again kRefSlots units later: who
+  // finds the references of unit v has published unit v - kRefAhead, so every CTA is done with the
+  // units before v - kRefAhead - 2 kResRing + 1.
+  auto ref_word = [&](unsigned u, int row) {
+    return p.xch + 2 * (size_t)kXchPairs + (size_t)(team * kRefSlots + (int)(u % kRefSlots)) * R + row;
+  };
+  // Waits for it; `word` was read before.  Whoever has it finds the row's summed words clean.
+  auto have_ref = [&](unsigned u, int row, unsigned long long& word) {
+    for (long long t0 = 0; !__all_sync(0xffffffffu, word_has(word, tag0 + u));) {
+      if (!__all_sync(0xffffffffu, keep_polling(t0))) return false;
+      word = get_word_acquire(ref_word(u, row));
+    }
+    return true;
   };
 
   if (warp == kResWarps) {
@@ -269,20 +289,72 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
   } else if (warp == kResWarps + 3) {
     // ---------------- this CTA's statistics ----------------
     const int row = lane;
+    // Common references of a unit (a row's largest logit over the first four keys and the last four that all of its rows
+    // see) and clean summed words: 32 rows by 8 keys, two m16n8 products.  Which of a thread's eight consecutive elements
+    // stands for which k of the instruction does not matter as long as both operands agree.
+    auto find_refs = [&](unsigned v) {
+      const int gu = team + (int)v * teams, pi = gu / n_kv, g = gu - pi * n_kv;
+      if (pi >= n_prob) return;
+      const ResProblem& pb = prob_s[pi].p;
+      const int open = pb.n_keys - p.window, t = lane & 3, n = lane >> 2;
+      const int key = n < 4 ? min(n, open) : max(0, open - (n - 4));
+      const __nv_bfloat16* const k = pb.k + g * p.k_stride_head + key * p.k_stride_token + t * 8;
+      float top[4];                                        // of rows n, n + 8, n + 16, n + 24
+#pragma unroll
+      for (int m = 0; m < 2; ++m) {
+        const __nv_bfloat16* q[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = m * 16 + h * 8 + n, at = is_row(r) ? r / p.w_pad * p.window + (r & (p.w_pad - 1)) : 0;
+          q[h] = pb.q + ((size_t)g * p.group * p.window + at) * D + t * 8;
+        }
+        float acc[4] = {};
+#pragma unroll
+        for (int c = 0; c < D; c += 32) {
+          const uint4 a = __ldg(reinterpret_cast<const uint4*>(q[0] + c)), b = __ldg(reinterpret_cast<const uint4*>(q[1] + c));
+          const uint4 x = __ldg(reinterpret_cast<const uint4*>(k + c));
+          mma_16x8x16(acc, a.x, b.x, a.y, b.y, x.x, x.y);
+          mma_16x8x16(acc, a.z, b.z, a.w, b.w, x.z, x.w);
+        }
+        const float c2 = pb.negate ? -pb.c2 : pb.c2;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float x = fmaxf(acc[2 * h] * c2, acc[2 * h + 1] * c2);
+          x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 1));
+          top[2 * m + h] = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 2));
+        }
+      }
+      float ref = 0.f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float x = __shfl_sync(0xffffffffu, top[i], (row & 7) * 4);
+        if (row >> 3 == i) ref = x;
+      }
+      if (!is_row(row) || !(fabsf(ref) < 3.0e38f)) ref = 0.f;
+      reinterpret_cast<ulonglong2*>(p.sums)[(size_t)gu * R + row] = make_ulonglong2(0, 0);
+      __threadfence();
+      put_word(ref_word(v, row), tagged(ref, tag0 + v));
+    };
     unsigned u = 0;
+    unsigned long long ref = 0;
+    if (p.sums && rank < kRefAhead) find_refs(rank);
     for (Walk w = walk_from(); w.pi < n_prob; walk_on(w), ++u) {
       const size_t at = (size_t)unit_of(w) * R + row;
-      const float ref = p.sums ? __ldg(p.refs + at) : 0.f;
+      if (p.sums && !have_ref(u, row, ref)) break;
       if (!__all_sync(0xffffffffu, mbar_wait(bar(L::kStats + (int)(u % kResRing)), (u / kResRing) & 1u, abort_flag))) break;
       if (!p.sums) {
         publish(u, row);
       } else if (is_row(row)) {
-        const RowStat f = fold(u, row, ref);
+        const RowStat f = fold(u, row, word_value(ref));
         unsigned long long* const to = p.sums + 2 * at;
         const bool fits = f.Z < kSumLimit && fabsf(f.U) < kSumLimit;
         if (!fits) atomicOr(to, kSumOver);
         atomicAdd(to, kSumCount + (fits ? (unsigned long long)__float2ll_rn(f.Z * kSumUnit) : 0ull));
         atomicAdd(to + 1, kSumCount + kSumBias + (fits ? (unsigned long long)__float2ll_rn(f.U * kSumUnit) : 0ull));
+      }
+      if (p.sums) {
+        if ((u + kRefAhead) % (unsigned)G == (unsigned)rank) find_refs(u + kRefAhead);
+        ref = get_word_acquire(ref_word(u + 1, row));
       }
     }
   } else if (warp == kResWarps + 2) {
@@ -290,6 +362,7 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
     const int row = lane;
     const bool valid = is_row(row);
     unsigned u = 0;
+    unsigned long long ref = 0;
     bool live = true;
     // A row's word once all CTAs are in it (rows that exist), or the CTA gives up.
     auto summed = [&](const unsigned long long* at) {
@@ -308,11 +381,12 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
       float lse = -INFINITY, Z = 0.f;
       bool direct = p.sums == nullptr;
       if (!direct) {
-        const float ref = __ldg(p.refs + at);
+        if (!have_ref(u, row, ref)) break;
         const unsigned long long x = summed(p.sums + 2 * at);
         if (!live) break;
         Z = (float)(x & (kSumOver - 1)) * (1.f / kSumUnit);
-        lse = ref + __log2f(Z);
+        lse = word_value(ref) + __log2f(Z);
+        ref = get_word_acquire(ref_word(u + 1, row));
         if (__any_sync(0xffffffffu, (x & kSumOver) != 0)) {   // the same answer in every CTA
           direct = true;
           __threadfence_block();
@@ -412,12 +486,15 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
       walk_on(a.w);
     };
     At e{walk_from(), 0, 0}, s = e;
-    // The common references of this warp's rows in the next unit (summed; lane l holds that of row l % RT), loaded
+    // The common references of this warp's rows in unit e (summed; lane l holds that of row l % RT), first looked for
     // a unit ahead.
-    auto load_refs = [&](const Walk& w) {
-      return p.sums && w.pi < n_prob ? __ldg(p.refs + (size_t)unit_of(w) * R + set0 + lane % RT) : 0.f;
+    auto look_for_refs = [&](unsigned u) { return p.sums ? get_word(ref_word(u, set0 + lane % RT)) : 0ull; };
+    unsigned long long refs = look_for_refs(0);
+    auto have_refs = [&]() {
+      if (!p.sums || __all_sync(0xffffffffu, word_has(refs, tag0 + e.u))) return true;
+      refs = look_for_refs(e.u);
+      return __all_sync(0xffffffffu, word_has(refs, tag0 + e.u)) != 0;
     };
-    float next_refs = load_refs(e.w);
     long long t0 = 0;
     while (s.w.pi < n_prob) {
       if (__all_sync(0xffffffffu, fl->known > (int)s.u)) {
@@ -477,8 +554,8 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
         next_unit(s);
         continue;
       }
-      // ---- statistics of the next unit: all of its tiles are there, and a place for its statistics is ----
-      if (e.w.pi < n_prob && __all_sync(0xffffffffu, fl->summed + kResRing > (int)e.u) && full(e.tile + tiles_of(e) - 1)) {
+      // ---- statistics of the next unit: all of its tiles and references are there, and a place for its statistics is ----
+      if (e.w.pi < n_prob && __all_sync(0xffffffffu, fl->summed + kResRing > (int)e.u) && full(e.tile + tiles_of(e) - 1) && have_refs()) {
         t0 = 0;
         tc_fence_after();
         const ResShare& sh = prob_s[e.w.pi];
@@ -486,10 +563,8 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
         const uint64_t c22 = pack2(c2, c2);
         const int last_open_key = sh.p.n_keys - p.window, hi = (sh.lo + sh.c) * kResChunk;
         const float masked = fmaxf(__fdividef(kMasked, c2), kMaskedAcc);   // times c2: finite, and 2^x flushes to 0
-        const float common = next_refs;
-        Walk n = e.w;
-        walk_on(n);
-        next_refs = load_refs(n);
+        const float common = word_value(refs);
+        refs = look_for_refs(e.u + 1);
         const int tiles = tiles_of(e), j0 = sh.lo * kResChunk + quarter * 32 + lane;
         float v[T * RT];
         // The logits of tiles [i0, i0 + n_here), where a row does not see a key: masked.

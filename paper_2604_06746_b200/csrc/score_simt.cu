@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kSmThreads, 3) simt_once(const __grid_constant
   const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;
   const float c2 = a.c2[layer];
   const unsigned tag = (unsigned)__ldcg(a.ctl + kCtlTag) + 1u;
-  constexpr size_t kEntWords = kXchWords / 2;
+  constexpr size_t kEntWords = kXchPairs;
   unsigned long long* const words = a.xch + (size_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x * kSmRows;   // of these rows: [part][row]
   stage_rows<T, D>(a, (const T*)a.q[layer], g, rt, s.q);
   stage_keys<T, D>(a, (const T*)a.k[layer] + (size_t)g * a.sh, j0, s.k);
@@ -364,7 +364,7 @@ cudaError_t launch_typed(const Ctx& ctx, const SimtArgs& a, int layers, cudaStre
   // The layers whose blocks all run at once, as even as it goes (8 layers of 4096 keys: 110 us in two passes, 89
   // three layers at a time; 32 of 2048 keys 187 / 160).
   const long long per_layer = (long long)a.n_keys_tiles * a.n_rt * G;
-  const int room = (int)(std::min((long long)per_sm[dev].load(std::memory_order_relaxed) * ctx.sm_count, kXchWords / (2ll * kSmRows)) / per_layer);
+  const int room = (int)(std::min((long long)per_sm[dev].load(std::memory_order_relaxed) * ctx.sm_count, (long long)kXchPairs / kSmRows) / per_layer);
   if (span == 1 && a.n_keys_tiles == a.parts && room >= 1) {
     const int launches = (layers + room - 1) / room;
     cudaError_t e = clean_words(ctx, st);

@@ -185,6 +185,11 @@ __device__ __forceinline__ bool mbar_drain(uint32_t bar, uint32_t parity, volati
     if ((unsigned long long)(clock64() - t0) > limit) { *abort_flag = 1; return false; }
   }
 }
+// d[16 x 8] += a[16 x 16] b[16 x 8], for products too small for a tcgen05 tile.
+__device__ __forceinline__ void mma_16x8x16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
 // 3-D tile copy with an L2 eviction-priority hint for the lines it brings in.
 __device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0,
                                                  int c1, int c2, uint64_t policy) {

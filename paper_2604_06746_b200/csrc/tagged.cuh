@@ -21,6 +21,12 @@ __device__ __forceinline__ unsigned long long get_word(const unsigned long long*
   asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
   return w;
 }
+// The same for a value that says that others are ready.
+__device__ __forceinline__ unsigned long long get_word_acquire(const unsigned long long* p) {
+  unsigned long long w;
+  asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+  return w;
+}
 // What the last CTA of a launch does (all of its threads call): the tags move on to `next`, or, long before they wrap,
 // start over with clean words.
 __device__ __forceinline__ void pass_tags_on(unsigned long long* xch, int* ctl, unsigned next) {

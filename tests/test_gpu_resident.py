@@ -106,3 +106,24 @@ def test_two_streams(cuda_device):
         torch.testing.assert_close(s[b][0].double(), cols.sum(0), rtol=2e-4, atol=1e-7 * H / N)
         assert abs(m[b][0, 0].item() - ent.item()) < 1e-4 * abs(ent.item()) + 1e-5
         ctx[b].close()
+
+
+def test_a_layer_takes_two_launches(cuda_device):
+    """The scorer and the sums over heads; large teams find their rows' references inside the scorer."""
+    from cuda.bindings import runtime as rt
+
+    from paper_2604_06746_b200 import binding
+    H, Hkv, d, w, N = 4, 1, 128, 8, 50000
+    q = torch.zeros((H, w, d), device=cuda_device, dtype=torch.bfloat16)
+    k = torch.zeros((Hkv, N, d), device=cuda_device, dtype=torch.bfloat16)
+    s, m = torch.zeros(N, device=cuda_device), torch.zeros(3, device=cuda_device)
+    ctx = binding.Context(H, Hkv, d, w, N, torch.bfloat16, cuda_device)
+    ctx.score_layer(q, k, 0.1, s, m, flags=binding.FLAG_NO_HEAD_STATS)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        ctx.score_layer(q, k, 0.1, s, m, flags=binding.FLAG_NO_HEAD_STATS)
+    err, _, count = rt.cudaGraphGetNodes(rt.cudaGraph_t(init_value=int(graph.raw_cuda_graph())))
+    assert err == rt.cudaError_t.cudaSuccess and count == 2
+    del graph
+    ctx.close()
