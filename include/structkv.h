@@ -254,7 +254,7 @@ structkv_status structkv_head_stats(structkv_ctx* ctx, const float* head_cols, l
  * Arguments: `cfg` host pointer; everything else exactly as structkv_score_layer, with
  * cfg->max_seq >= n_keys.  Errors: INVALID_ARG, UNSUPPORTED, WORKSPACE, CUDA.
  */
-#define STRUCTKV_STATIC_SCRATCH_BYTES ((8u << 20) + 1417216u)
+#define STRUCTKV_STATIC_SCRATCH_BYTES ((8u << 20) + 1449984u)
 structkv_status structkv_score_layer_static(const structkv_config* cfg, const void* q_window,
                                             const void* k, long long k_stride_head,
                                             long long k_stride_token, int n_keys, float scale,

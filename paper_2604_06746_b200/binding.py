@@ -55,7 +55,7 @@ lib.structkv_score_layer.argtypes = [_vp, _vp, _vp, _ll, _ll, _i, _f, _f, _vp, _
 lib.structkv_score_layer_static.restype = _i
 lib.structkv_score_layer_static.argtypes = [ctypes.POINTER(Config), _vp, _vp, _ll, _ll, _i, _f, _f, _vp, _vp,
                                             _vp, _vp, _u, _vp]
-STATIC_SCRATCH_BYTES = (8 << 20) + 1417216
+STATIC_SCRATCH_BYTES = (8 << 20) + 1449984
 lib.structkv_batch_workspace_bytes.restype = ctypes.c_size_t
 lib.structkv_batch_workspace_bytes.argtypes = [ctypes.POINTER(Config), _i, _ll]
 lib.structkv_score_layer_batch.restype = _i

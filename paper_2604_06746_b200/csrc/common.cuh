@@ -20,10 +20,12 @@ constexpr int kQueueUnits = 256;      // (KV group, row block) units of one prob
 constexpr int kCtlInts = 64 + 2 * kMaxBatch * kQueueUnits;   // its control block: tickets, arrivals, ready flags
 constexpr int kXchSlots = 17;          // units of an exchange ring of the resident scorer's teams
 constexpr int kResRows = 32;           // score rows of one of its units, at most
-constexpr int kRefSlots = 32;          // units of a ring of common references
+constexpr int kDirectTeam = 20;        // CTAs of a team that merges partials directly (score_res.cuh)
+constexpr int kRefSlots = 32;          // units of a ring of common references, which larger teams have
 // Tagged 64-bit words: two for every row and CTA of the teams' rings (the CUDA-core scorer needs fewer), then the rings of
-// references, of three teams at most.
-constexpr int kXchPairs = kMaxSms * kXchSlots * kResRows, kXchWords = 2 * kXchPairs + 3 * kRefSlots * kResRows;
+// references.
+constexpr int kXchPairs = kMaxSms * kXchSlots * kResRows;
+constexpr int kXchWords = 2 * kXchPairs + kMaxSms / (kDirectTeam + 1) * kRefSlots * kResRows;
 constexpr int kCtlExit = 1, kCtlTag = 2;   // in the control block: CTAs that are done; last tag of the exchange words
 constexpr unsigned long long kWaitCycles = 1000000000ull;   // bound of a device wait, about 0.5 s at the maximum SM clock
 constexpr int kMergeGroup = 6;         // partials of a row merged together

@@ -24,8 +24,13 @@ Plan plan_of(int n_keys, int n_kv, int sms) {
   }
   return best;
 }
-// Shorter sequences stay with the general scorer, which has less to do per unit (see score_res.cuh).
-constexpr int kResFrom = 4096;
+// Shorter sequences stay with the general scorer: however short, a team takes 2.6 us for a unit among many and has its way
+// through the exchange in one by itself, and as many units follow one another as a team has KV groups.  us per layer,
+// general / this one, one layer | one of 32: one KV head 4096 keys 14.7 / 17.7 | 1.8 / 2.6, 9001 keys 15.0 / 18.6 | 2.4 / 2.6,
+// 16000 keys 17.1 / 18.5 | 2.9 / 2.6, 20000 keys 19.3 / 18.5 | 3.4 / 3.0; two 4096 keys 15.8 / 18.5 | 2.0 / 2.6, 7500
+// keys 17.4 / 18.5 | 2.7 / 2.6, 9001 keys 18.6 / 18.5 | 3.2 / 2.7; four 4096 keys 18.5 / 18.5 | 2.9 / 2.7; eight 2500
+// keys 21.4 / 18.9 | 3.2 / 3.5, 4096 keys 21.3 / 20.3 | 4.5 / 3.4.
+constexpr int kResFrom = 4096, kResKeys = 16384;           // keys; keys of all KV heads
 
 template <int MAXP>
 cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n, cudaStream_t st) {
@@ -72,8 +77,8 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
 }  // namespace
 
 bool res_supported(const Ctx& ctx, const ScoreCall& a) {
-  return !a.cu_seqlens && a.n_keys >= kResFrom && ctx.cfg.n_q_heads / ctx.cfg.n_kv_heads * ctx.w_pad <= kResRows &&
-         plan_of(a.n_keys, ctx.cfg.n_kv_heads, std::min(ctx.sm_count, kMaxSms)).team > 0;
+  return !a.cu_seqlens && a.n_keys >= kResFrom && (long long)a.n_keys * ctx.cfg.n_kv_heads >= kResKeys &&
+         ctx.cfg.n_q_heads / ctx.cfg.n_kv_heads * ctx.w_pad <= kResRows && plan_of(a.n_keys, ctx.cfg.n_kv_heads, std::min(ctx.sm_count, kMaxSms)).team > 0;
 }
 
 cudaError_t launch_score_res(const Ctx& ctx, const ScoreCall& a, int first, int n, cudaStream_t st) {

@@ -18,7 +18,12 @@
 //           2^(x - ref) add up; they do as fixed-point integers, in any order the same bits, in words whose
 //           top byte counts the CTAs.  Where a CTA's sum leaves the range
 //           (a logit 2^20 above the reference) it marks the word, and the team takes the direct way for that unit.
-// Direct teams of 74 read too many words: 65536 keys 506 us for 16 layers, summed 427.  The references came from a launch of
+// The more mates, the more words a direct team reads.  us per layer, direct / summed, one layer | one of 32: 74 CTAs (65536
+// keys) - | 31.6 / 26.7; 37 CTAs (8 KV heads, 20011 keys) 28.8 / 26.7 | 9.8 / 8.4, (32768 keys) 33.1 / 30.8 | 13.9 /
+// 12.7, (4 KV heads, 4096 keys) 20.6 / 18.5 | 3.8 / 2.7; 24 CTAs (6 KV heads, 5003 keys) 21.0 / 19.9 | 4.0 / 3.1.  The
+// general scorer takes 18.5 | 2.9 for those 4096 keys and 20.4 | 4.3 for those 5003, so direct teams of 24 and more lost.
+// Those of 18 do not (8 KV heads, 4096 keys 20.3 | 3.4, general 21.3 | 4.5, summed 18.8 | 3.0) and keep
+// their form.  The references came from a launch of
 // their own at first, which a layer by itself waited for; us with it / with them found inside, one layer: 8 KV heads
 // 40000 keys 43.0 / 36.6, 98304 64.6 / 60.1, 262144 150 / 135; 4 KV heads 40000 32.9 / 26.7, 131072 49.5 / 44.4;
 // one KV head 32768 24.4 / 18.5; a layer of 32 with 8 KV heads of 262144 keys 135 / 121.
@@ -43,7 +48,6 @@ constexpr int kResWarps = 4 * kResSubs;
 constexpr int kResThreads = (kResWarps + 4) * 32;   // 20 warps: the most that fit at 96 registers a thread
 constexpr int kResChunk = 32;          // keys are dealt out to a team's CTAs in chunks of 32
 constexpr int kResRing = 8;            // units a CTA may have between its statistics and its last column sum
-constexpr int kDirectTeam = 40;        // CTAs of a team that merges partials directly
 constexpr int kRefAhead = 2 * kResRing;   // a unit's common references are found so many units before
 // A row's summed words: [63:56] CTAs so far, [55] somebody's sum is out of range, below it sum Z in units of
 // 2^-26; [63:56] CTAs, below it sum (U + 2^21) in units of 2^-26.
@@ -51,8 +55,7 @@ constexpr float kSumUnit = 67108864.f, kSumLimit = 2097152.f;
 constexpr unsigned long long kSumCount = 1ull << 56, kSumOver = 1ull << 55, kSumBias = 1ull << 47;
 static_assert(kMaxSms * 2097152ull * 67108864ull < kSumOver && kMaxSms * 2 * kSumBias < kSumCount, "summed words");
 static_assert(kXchSlots > 2 * kResRing, "slots of tagged words");
-static_assert(kRefSlots >= kRefAhead + 2 * kResRing && kRefAhead <= kDirectTeam && 4 * (kDirectTeam + 1) > kMaxSms,
-              "rings of references");
+static_assert(kRefSlots >= kRefAhead + 2 * kResRing && kRefAhead <= kDirectTeam, "rings of references");
 
 struct ResProblem {
   float* cols;                         // output of head 0, key 0

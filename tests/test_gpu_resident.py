@@ -1,5 +1,5 @@
-"""The scorer of short windows that reads K once (at most 32 score rows per KV group, sequences from 4096 keys on): the
-edges of its chunks, tiles and teams, both ways its CTAs add up their rows (small teams and large ones),
+"""The scorer of short windows that reads K once (at most 32 score rows per KV group, sequences from 4096 keys on, from 16384
+keys of all KV heads on): the edges of its chunks, tiles and teams, both ways its CTAs add up their rows (small teams and large ones),
 logits far above the sampled references, repetition on one workspace, and streams side by side."""
 import math
 
@@ -16,12 +16,14 @@ pytestmark = pytest.mark.gpu
     (32, 8, 128, 7, 9215), (32, 8, 128, 8, 18433),                           # eight teams of 18, four of 37
     (8, 2, 128, 3, 4161), (8, 2, 64, 8, 20000), (4, 4, 64, 32, 6001),        # teams of 74; of 37; one head of 32 rows
     (4, 1, 128, 8, 4737), (1, 1, 64, 1, 5000), (3, 1, 128, 8, 70001),        # one team of all SMs, its rows summed
+    (4, 1, 128, 8, 16383), (4, 1, 128, 8, 16384), (8, 2, 64, 3, 8192),       # few KV heads: the last length, the first ones
+    (7, 7, 128, 8, 4100), (24, 6, 128, 8, 4800), (20, 5, 64, 7, 37889),      # teams of 21, 24 and 29, summed
 ])
 def test_edges(cuda_device, H, Hkv, d, w, N):
     score(cuda_device, H, Hkv, d, w, N, 1 / math.sqrt(d))
 
 
-@pytest.mark.parametrize("H,Hkv,N", [(32, 8, 5000), (4, 1, 5000)])
+@pytest.mark.parametrize("H,Hkv,N", [(32, 8, 5000), (4, 1, 5000), (4, 1, 20000), (16, 4, 9000)])
 @pytest.mark.parametrize("scale", [-0.3, 0.0, 1.0, 3.0])
 def test_logits_far_above_the_references(cuda_device, H, Hkv, N, scale):
     """Unit-variance keys give logits of 11 |scale| nats' deviation: at 1 a CTA's sums leave the range of the summed
@@ -32,6 +34,7 @@ def test_logits_far_above_the_references(cuda_device, H, Hkv, N, scale):
 @pytest.mark.parametrize("Hkv,N", [
     (8, 4200), (1, 4200),
     (4, 4200), (4, 9400),                                                    # teams of 37, one and two tiles a CTA
+    (7, 4200), (1, 16500),                                                   # teams of 21, seven of them; one of 148
     (1, 70000), (2, 40000),                                                  # summed, four and five tiles a CTA
 ])
 def test_layers_repetition_and_replay(cuda_device, Hkv, N):

@@ -114,16 +114,16 @@ def test_static_scratch_serves_every_scorer_in_any_order(cuda_device):
         ctx.close()
 
 
-@pytest.mark.parametrize("w,n,most", [(64, 5000, 96 << 10), (8, 4000, 96 << 10), (8, 5000, 3 << 19)])
-def test_static_scratch_clears_what_the_scorer_uses(cuda_device, w, n, most):
+@pytest.mark.parametrize("w,Hkv,n,most", [(64, 8, 5000, 96 << 10), (8, 8, 4000, 96 << 10), (8, 1, 16383, 96 << 10), (8, 8, 5000, 3 << 19)])
+def test_static_scratch_clears_what_the_scorer_uses(cuda_device, w, Hkv, n, most):
     """Bytes a captured call clears: its counters, and the exchange words only where its scorer has CTAs exchange them."""
     from cuda.bindings import runtime as rt
 
     from paper_2604_06746_b200 import binding
-    q = torch.zeros((32, w, 128), device=cuda_device, dtype=torch.bfloat16)
-    k = torch.zeros((8, n, 128), device=cuda_device, dtype=torch.bfloat16)
+    q = torch.zeros((4 * Hkv, w, 128), device=cuda_device, dtype=torch.bfloat16)
+    k = torch.zeros((Hkv, n, 128), device=cuda_device, dtype=torch.bfloat16)
     s, m = torch.zeros(n, device=cuda_device), torch.zeros(3, device=cuda_device)
-    args = (32, 8, 128, w, n, q, k, 0.1, s, m)
+    args = (4 * Hkv, Hkv, 128, w, n, q, k, 0.1, s, m)
     binding.score_layer_static(*args)                      # one-time set-up
     torch.cuda.synchronize()
     graph = torch.cuda.CUDAGraph(keep_graph=True)
