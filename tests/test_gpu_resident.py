@@ -130,3 +130,41 @@ def test_a_layer_takes_two_launches(cuda_device):
     assert err == rt.cudaError_t.cudaSuccess and count == 2
     del graph
     ctx.close()
+
+
+@pytest.mark.parametrize("H,Hkv,d,w,N", [
+    (32, 8, 128, 8, 5000), (8, 8, 64, 32, 4200),                             # small teams
+    (16, 4, 64, 7, 9001), (6, 2, 128, 5, 40000), (4, 1, 128, 8, 20000),      # teams with common references
+])
+def test_layouts_of_k(cuda_device, H, Hkv, d, w, N):
+    """Token-major K, and rows and heads with room between them: the bits of contiguous K, for a layer by itself, for several,
+    and on the static scratch."""
+    from paper_2604_06746_b200 import binding
+    g = torch.Generator(device=cuda_device)
+    g.manual_seed(N)
+    q = [torch.randn((H, w, d), generator=g, device=cuda_device).bfloat16() for _ in range(2)]
+    k = [torch.randn((Hkv, N, d), generator=g, device=cuda_device).bfloat16() for _ in range(2)]
+    ctx = binding.Context(H, Hkv, d, w, N, torch.bfloat16, cuda_device)
+    ws = ctx.layers_workspace(2)
+
+    def run(ks):
+        s, m, h = (torch.zeros(x, device=cuda_device) for x in ((4, N), (4, 3), (4, H, N)))
+        ctx.score_layer(q[0], ks[0], 0.1, s[0], m[0], head_cols_out=h[0], flags=binding.FLAG_NO_HEAD_STATS)
+        binding.score_layer_static(H, Hkv, d, w, N, q[0], ks[0], 0.1, s[1], m[1], head_cols_out=h[1], flags=binding.FLAG_NO_HEAD_STATS)
+        ctx.score_layers(q, ks, [0.1, 0.1], s[2:], m[2:], h[2:], ws)
+        assert ctx.poll_device_status() == binding.OK
+        return s, m[:, 0], h
+
+    first = run(k)
+    for a in first:
+        assert torch.equal(a[0], a[1]) and torch.equal(a[0], a[2])
+    cols, ent = reference(q[1], k[1], 0.1)
+    torch.testing.assert_close(first[2][3].double(), cols, rtol=2e-4, atol=1e-7 / N)
+    assert abs(first[1][3].item() - ent.item()) < 1e-4 * ent.item()
+    for lay in (lambda x: x.transpose(0, 1).contiguous().transpose(0, 1),                        # [N, H_kv, d]
+                lambda x: torch.nn.functional.pad(x, (0, 8, 0, 3))[:, :N, :d]):                  # room after rows and heads
+        views = [lay(x) for x in k]
+        assert not views[0].is_contiguous() or Hkv == 1
+        for a, b in zip(run(views), first):
+            assert torch.equal(a, b)
+    ctx.close()
