@@ -5,7 +5,7 @@
 // where these come through distributed shared memory, one warp does it for its CTA (all 32 of them: 131072 keys 103 us).
 // Two or three block barriers a level; one pass over memory in all where the vector fits the registers.
 // Bound by the chain of barriers and shared-memory round trips.  Four levels of eight bits with a copy of every bin
-// per lane took 7.5 us for 1000 keys (now 5.1), 9.7 for 5003 (6.7), 16.8 for 32768 (10.6), 22.3 for 131072 (18.6).
+// per lane took 7.5 us for 1000 keys (now 5.1), 9.7 for 5003 (6.7), 16.8 for 32768 (9.3), 22.3 for 131072 (18.6).
 #pragma once
 
 #include <cooperative_groups.h>

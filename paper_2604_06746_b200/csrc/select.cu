@@ -23,8 +23,11 @@ struct SelectArgs {
   SelectExtra extra;                   // vector `batch` of a uniform call, if it has scores
 };
 
+// Two CTAs an SM for the many short vectors that need them.  Clusters of up to eight items a thread serve at most 17 vectors,
+// 68 CTAs: bound to 32 registers they spilled (8 / 16 vectors of 32768 tokens 13.0 / 14.8 us, now 11.2 / 11.3; of 12000
+// 8.1 / 8.3, now 7.7 / 7.7).
 template <int CL, int ITEMS>
-__global__ void __launch_bounds__(kRxThreads, ITEMS <= 8 ? 2 : 1) select_topk(const __grid_constant__ SelectArgs a) {
+__global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) select_topk(const __grid_constant__ SelectArgs a) {
   extern __shared__ __align__(16) unsigned char sel_smem[];
   RadixShared<CL>& s = *reinterpret_cast<RadixShared<CL>*>(sel_smem);
   __shared__ unsigned cta_tot[2][CL];
@@ -182,8 +185,8 @@ cudaError_t launch(const SelectArgs& a, cudaStream_t st) {
 // One CTA while that is a matter of three barriers a level; beyond, few vectors get more CTAs with fewer items each, and
 // many (whose CTAs would not run side by side) the smallest cluster that holds one.  us for 1 / 8 / 33 vectors, chained
 // launches: 1777 tokens 5.1 / 5.2 / 5.6 with 1 x 4 items (a cluster of two 6.9 / 7.0 / 7.2), 8192 7.0 / 7.2 / 8.4 with
-// 1 x 8 (2 x 4: 7.2 / 7.3 / 9.0), 16384 9.9 / 10.0 / 11.7 with 1 x 16 and 8.1 / 8.3 / 11.9 with 4 x 4, 32768 12.0 /
-// 12.2 / 14.1 with 2 x 16 and 10.6 / 11.0 / 16.0 with 4 x 8, 65536 13.1 / 13.3 / 16.2 with 4 x 16 and 12.5 /
+// 1 x 8 (2 x 4: 7.2 / 7.3 / 9.0), 16384 9.9 / 10.0 / 11.7 with 1 x 16 and 7.7 / 7.8 with 4 x 4, 32768 12.0 / 12.2 /
+// 14.1 with 2 x 16 and 9.3 / 11.2 with 4 x 8, 65536 13.1 / 13.3 / 16.2 with 4 x 16 and 12.5 /
 // 13.2 / 26.0 with 8 x 8, 131072 18.6 with 8 x 16 and 24.1 for 33 with 4 x 32.
 cudaError_t dispatch(const SelectArgs& a, int longest, cudaStream_t st) {
   if (longest <= 4 * kRxThreads) return launch<1, 4>(a, st);
