@@ -372,20 +372,32 @@ def compaction_figures(wl, kv_budget, compact_ms_per_step, peaks):
             "frac": nbytes / s / 1e9 / peaks["hbm_gbs"], "bytes_per_step": nbytes}
 
 
+def cuda_core_launches(wl, layers):
+    """Launches of the CUDA-core scorer for `layers` layers: up to 64 tiles of 64 keys as many layers as run at once (three
+    blocks an SM with head_dim 64, two with 128), where one does; else one launch per pass."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w_pad = max(8, 1 << (wl.window - 1).bit_length())
+    tiles = -(-wl.seq // 64)
+    per_layer = tiles * -(-(wl.n_q_heads // wl.n_kv_heads) * w_pad // 128) * wl.n_kv_heads
+    room = (3 if wl.head_dim == 64 else 2) * sms // per_layer
+    if tiles > 64 or w_pad > 128 or room < 1:
+        return 2 * -(-layers // 32)
+    return sum(-(-min(32, layers - l) // room) for l in range(0, layers, 32))
+
+
 def launches_per_step(wl, flags):
     from paper_2604_06746_b200 import binding
     # one call for all layers: the tensor-core scorer (one launch per 32 layers, both passes) or the
-    # CUDA-core one (one launch up to 4096 keys, else one per pass), then one launch for the sums over heads; layer by layer the same per layer.  Per
+    # CUDA-core one, then one launch for the sums over heads; layer by layer the same per layer.  Per
     # step: head statistics of all layers, centrality at the pivot, all selections, one K/V gather over
     # all layers, hidden states, positions
     tc = wl.dtype == "bf16" and not flags & binding.FLAG_FORCE_SIMT
     together = not flags & (binding.FLAG_NO_HEAD_STATS | binding.FLAG_FORCE_SIMT)
     stats = 0 if flags & binding.FLAG_NO_HEAD_STATS else 1
-    scorer = 1 if tc or wl.seq <= 4096 else 2
     if together:
-        scoring = (-(-wl.n_layers // 32) if tc else scorer) + 1
+        scoring = (-(-wl.n_layers // 32) if tc else cuda_core_launches(wl, wl.n_layers)) + 1
     else:
-        scoring = wl.n_layers * (scorer + 1)
+        scoring = wl.n_layers * ((1 if tc else cuda_core_launches(wl, 1)) + 1)
     return scoring + stats + 1 + 1 + 1 + 2
 
 

@@ -22,6 +22,12 @@
  *   - A context serialises its calls through its workspace: calls on one context must be
  *     issued on one stream (or be ordered by the caller).  Distinct contexts are independent.
  *   - Results are deterministic: the same inputs give the same bits.
+ *   - Work on other streams: kernels whose blocks exchange values are launched so that all of their
+ *     blocks run at once (cooperative launches): the scorer of short windows (at most 32 score rows
+ *     per KV group; lengths in score_res.cu), which takes up to every SM, and the CUDA-core scorer of
+ *     up to 4096 keys.  Beside a kernel of another stream that holds SMs they start when that one
+ *     has made room; the other kernels take the SMs that are free.  So nothing may hold SMs until
+ *     such a call has finished (a resident kernel that waits for its result, say).
  *
  * Index conventions: N = n_keys prompt tokens, w = window (the last w positions are the
  * observation-window queries, row i sits at position t = N-w+i and attends to keys j <= t),

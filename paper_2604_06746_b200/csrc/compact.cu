@@ -26,7 +26,8 @@ template <> __device__ __forceinline__ void st_stream<uint4>(uint4* p, const uin
   asm volatile("st.global.cs.v4.u32 [%0], {%1, %2, %3, %4};" ::"l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
-// u / d for u < 2^31 by one multiplication (a 64-bit division took some 100 instructions, two of them per 16 bytes).
+// u / d for u < 2^31 by one multiplication and a shift, after Granlund and Montgomery (Division by Invariant Integers using
+// Multiplication, 1994); a 64-bit division took some 100 instructions, two of them per 16 bytes.
 struct Divisor { unsigned mul; int shift; };               // mul 0: d is 1
 inline Divisor divisor(unsigned d) {
   int l = 0;

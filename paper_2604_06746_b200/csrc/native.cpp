@@ -1,6 +1,6 @@
 // CPython side of the binding's calls: checks the tensors, reads their pointers and strides, calls the C ABI.  (Through
 // ctypes and tensor attributes a call cost 6 us beside its launches, and the argument block of a prefill of 32
-// layers 42 us; here 1 us and 4 us.)  Every function returns the library's status, checks raise AssertionError, and
+// layers 42 us; here 1 us and 3 us.)  Every function returns the library's status, checks raise AssertionError, and
 // the interpreter lock is released while the library runs.
 #include <Python.h>
 
