@@ -1,6 +1,8 @@
 """Builds libstructkv.so (sm_100a, nvcc) and _native.so (the binding's calls, g++ against torch's headers) in-tree.
 Run: python -m paper_2604_06746_b200.build"""
+import importlib.metadata
 import os
+import platform
 import subprocess
 import sys
 import sysconfig
@@ -17,9 +19,17 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fno-gnu-unique", "-Wno-deprecated-gpu-targets"]
 
 
+def native_for():
+    """What _native.so is compiled against; it carries the text."""
+    return f"structkv binding for torch {importlib.metadata.version('torch')}, python {platform.python_version()}"
+
+
 def needs_build():
     if not (os.path.exists(LIB) and os.path.exists(NATIVE)):
         return True
+    with open(NATIVE, "rb") as f:
+        if native_for().encode() + b"\0" not in f.read():
+            return True
     t = min(os.path.getmtime(LIB), os.path.getmtime(NATIVE))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "structkv.h")]
     return any(os.path.getmtime(d) > t for d in deps)
@@ -33,7 +43,8 @@ def native_commands():
     inc = cpp_extension.include_paths() + ["/usr/local/cuda/include", sysconfig.get_paths()["include"], os.path.join(ROOT, "include")]
     abi = int(torch._C._GLIBCXX_USE_CXX11_ABI)
     libs = [f"-L{p}" for p in cpp_extension.library_paths()] + ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
-    return ([cxx, "-O2", "-std=c++17", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={abi}", *[f"-isystem{i}" for i in inc], "-c",
+    return ([cxx, "-O2", "-std=c++17", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={abi}",
+             f'-DSTRUCTKV_NATIVE_FOR="{native_for()}"', *[f"-isystem{i}" for i in inc], "-c",
              os.path.join(CSRC, "native.cpp"), "-o", obj],
             [cxx, "-shared", "-o", NATIVE, obj, f"-L{HERE}", "-lstructkv", "-Wl,-rpath,$ORIGIN", *libs])
 

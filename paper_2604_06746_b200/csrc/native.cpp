@@ -371,4 +371,7 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_native", nullptr, -1, methods, nu
 
 }  // namespace
 
+// Read from the file by the build, which compiles this again for another torch or python.
+extern "C" __attribute__((used)) const char structkv_native_for[] = STRUCTKV_NATIVE_FOR;
+
 PyMODINIT_FUNC PyInit__native() { return PyModule_Create(&module); }

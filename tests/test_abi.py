@@ -17,6 +17,14 @@ def B():
     return binding
 
 
+def test_another_torch_is_built_for_again(B, monkeypatch):
+    """_native.so is compiled against torch's headers: the same sources need a build once torch changes."""
+    from paper_2604_06746_b200 import build
+    assert not build.needs_build()
+    monkeypatch.setattr(build.importlib.metadata, "version", lambda name: "0.0")
+    assert build.needs_build()
+
+
 def declared_functions():
     text = open(os.path.join(ROOT, "include", "structkv.h")).read()
     text = re.sub(r"/\*.*?\*/", "", text, flags=re.S)
