@@ -5,9 +5,9 @@
 // rows of one KV group) by keys, and a CTA holds the unit's logits over its own keys in tensor memory, 32 columns for
 // 128 keys, from the first pass over them until the team knows the rows' normalisers: at 32768 keys 7 of 16
 // tiles a unit, two units in flight and the keys of the next ones on their way.
-// us per layer, general scorer / this one, 32 query heads, 8 KV heads, window 8, 32 layers: 2500 keys 3.0 / 3.3, 5003 3.9 / 3.7,
-// 9001 6.7 / 4.1, 20011 13.9 / 9.6, 32768 21.4 / 13.7 (reading K once takes 10.4), 98304 66 / 41, 131072 91 / 57; one layer
-// of 32768 37.8 / 32.8.  What is left above the reading is the way from tile to tile of a warp, at 60 % of the
+// us per layer with the sums over heads, general scorer / this one, 32 query heads, 8 KV heads, window 8, 32 layers: 2500 keys
+// 3.2 / 3.5, 5003 4.1 / 3.9, 9001 6.8 / 4.3, 20011 13.8 / 8.4, 32768 21 / 12.6 (reading K once takes 10.4), 98304 67 / 39,
+// 131072 93 / 53, 262144 183 / 121; one layer of 32768 37.4 / 30.9, of 98304 76.7 / 60.4.  What is left above the reading is the way from tile to tile of a warp, at 60 % of the
 // special-function unit's rate.  With 64 rows (window 16) both forms take as long: there the exponentials bound it.
 //
 // How a team adds up its rows' statistics, without fences, flags or a second trip:
@@ -298,6 +298,7 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
     auto find_refs = [&](unsigned v) {
       const int gu = team + (int)v * teams, pi = gu / n_kv, g = gu - pi * n_kv;
       if (pi >= n_prob) return;
+      __syncwarp();                                        // the products want the whole warp
       const ResProblem& pb = prob_s[pi].p;
       const int open = pb.n_keys - p.window, t = lane & 3, n = lane >> 2;
       const int key = n < 4 ? min(n, open) : max(0, open - (n - 4));
