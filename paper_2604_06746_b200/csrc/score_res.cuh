@@ -177,9 +177,9 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
   // looks at the next unit: all words are read of units before v - 2 kResRing, so that a slot must
   // last one unit longer than two rings.
   constexpr size_t kEntWords = kXchPairs;
-  auto tagged_word = [&](unsigned u, int from, int row) {
-    return p.xch + ((size_t)((team * kXchSlots + (int)(u % kXchSlots)) * G + from) * R + row);
-  };
+  // (Who walks the units counts the slots along: 17 is no power of two.)
+  auto tagged_words = [&](int slot, int row) { return p.xch + ((size_t)(team * kXchSlots + slot) * G * R + row); };
+  auto next_slot = [](int slot) { return slot + 1 < kXchSlots ? slot + 1 : 0; };
   // This CTA's statistics of a row, its lane quarters' in order, relative to `ref`.
   auto fold = [&](unsigned u, int row, float ref) {
     RowStat f{ref, 0.f, 0.f};
@@ -192,13 +192,14 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
     }
     return f;
   };
-  auto publish = [&](unsigned u, int row) {
+  auto publish = [&](unsigned u, int slot, int row) {
     float top = -INFINITY;
 #pragma unroll
     for (int k = 0; k < 4; ++k) top = fmaxf(top, stat_at(u, k, row)[0]);
     const float2 pt = stat_partial(fold(u, row, top));
-    put_word(tagged_word(u, rank, row), tagged(pt.x, tag0 + u));
-    put_word(tagged_word(u, rank, row) + kEntWords, tagged(pt.y, tag0 + u));
+    unsigned long long* const to = tagged_words(slot, row) + rank * R;
+    put_word(to, tagged(pt.x, tag0 + u));
+    put_word(to + kEntWords, tagged(pt.y, tag0 + u));
   };
 
   // Summed: the row's common reference in unit u of this team.  A slot is used again kRefSlots units later: who
@@ -340,6 +341,7 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
       put_word(ref_word(v, row), tagged(ref, tag0 + v));
     };
     unsigned u = 0;
+    int slot = 0;
     unsigned long long ref = 0;
     if (p.sums && rank < kRefAhead) find_refs(rank);
     for (Walk w = walk_from(); w.pi < n_prob; walk_on(w), ++u) {
@@ -347,7 +349,8 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
       if (p.sums && !have_ref(u, row, ref)) break;
       if (!__all_sync(0xffffffffu, mbar_wait(bar(L::kStats + (int)(u % kResRing)), (u / kResRing) & 1u, abort_flag))) break;
       if (!p.sums) {
-        publish(u, row);
+        publish(u, slot, row);
+        slot = next_slot(slot);
       } else if (is_row(row)) {
         const RowStat f = fold(u, row, word_value(ref));
         unsigned long long* const to = p.sums + 2 * at;
@@ -366,6 +369,7 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
     const int row = lane;
     const bool valid = is_row(row);
     unsigned u = 0;
+    int slot = 0;
     unsigned long long ref = 0;
     bool live = true;
     // A row's word once all CTAs are in it (rows that exist), or the CTA gives up.
@@ -378,8 +382,9 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
       }
       return x;
     };
-    for (Walk w = walk_from(); w.pi < n_prob; walk_on(w), ++u) {
+    for (Walk w = walk_from(); w.pi < n_prob; walk_on(w), ++u, slot = next_slot(slot)) {
       const bool leaves = (int)(u % (unsigned)G) == rank;  // one CTA of the team leaves the rows' entropies
+      const unsigned long long* const words = tagged_words(slot, row);
       const size_t at = (size_t)unit_of(w) * R + row;
       const unsigned tag = tag0 + u;
       float lse = -INFINITY, Z = 0.f;
@@ -394,7 +399,7 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
         if (__any_sync(0xffffffffu, (x & kSumOver) != 0)) {   // the same answer in every CTA
           direct = true;
           __threadfence_block();
-          publish(u, row);
+          publish(u, slot, row);
         }
       }
       if (direct) {
@@ -408,7 +413,7 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
 #pragma unroll
             for (int i = 0; i < kAt; ++i) {
               unsigned long long x = 0;
-              if (s0 + i < G) x = get_word(tagged_word(u, s0 + i, row));
+              if (s0 + i < G) x = get_word(words + (s0 + i) * R);
               l[i] = s0 + i < G ? word_value(x) : -INFINITY;
               all = all && (s0 + i >= G || word_has(x, tag));
             }
@@ -448,8 +453,8 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
 #pragma unroll
             for (int i = 0; i < kAt; ++i) {
               const int from = min(s0 + i, G - 1);
-              l[i] = get_word(tagged_word(u, from, row));
-              h[i] = get_word(tagged_word(u, from, row) + kEntWords);
+              l[i] = get_word(words + from * R);
+              h[i] = get_word(words + from * R + kEntWords);
             }
 #pragma unroll
             for (int i = 0; i < kAt; ++i) all = all && word_has(h[i], tag);
