@@ -22,8 +22,9 @@
 // keys) - | 31.6 / 26.7; 37 CTAs (8 KV heads, 20011 keys) 28.8 / 26.7 | 9.8 / 8.4, (32768 keys) 33.1 / 30.8 | 13.9 /
 // 12.7, (4 KV heads, 4096 keys) 20.6 / 18.5 | 3.8 / 2.7; 24 CTAs (6 KV heads, 5003 keys) 21.0 / 19.9 | 4.0 / 3.1.  The
 // general scorer takes 18.5 | 2.9 for those 4096 keys and 20.4 | 4.3 for those 5003, so direct teams of 24 and more lost.
-// Those of 18 do not (8 KV heads, 4096 keys 20.3 | 3.4, general 21.3 | 4.5, summed 18.8 | 3.0) and keep
-// their form.  The references came from a launch of
+// Those of 18 do not (8 KV heads, 4096 keys 20.3 | 3.4, general 21.3 | 4.5) and keep their form: summed they take 18.8 | 3.0,
+// but their columns' errors against float64 are 3 to 8 % larger (3.9e-7 instead of 3.7e-7; of teams of 37 4.2e-7
+// instead of 4.5e-7).  The references came from a launch of
 // their own at first, which a layer by itself waited for; us with it / with them found inside, one layer: 8 KV heads
 // 40000 keys 43.0 / 36.6, 98304 64.6 / 60.1, 262144 150 / 135; 4 KV heads 40000 32.9 / 26.7, 131072 49.5 / 44.4;
 // one KV head 32768 24.4 / 18.5; a layer of 32 with 8 KV heads of 262144 keys 135 / 121.
@@ -295,7 +296,9 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
     const int row = lane;
     // Common references of a unit (a row's largest logit over the first four keys and the last four that all of its rows
     // see) and clean summed words: 32 rows by 8 keys, two m16n8 products.  Which of a thread's eight consecutive elements
-    // stands for which k of the instruction does not matter as long as both operands agree.
+    // stands for which k of the instruction does not matter as long as both operands agree.  (Unrolled over both halves of the
+    // rows it cost every form: 28 layers of 5003 keys, direct, 3.83 us a layer, so 3.74; rolled up altogether, with one load
+    // in flight, a layer of one KV head and 40000 keys 18.8 -> 20.9.)
     auto find_refs = [&](unsigned v) {
       const int gu = team + (int)v * teams, pi = gu / n_kv, g = gu - pi * n_kv;
       if (pi >= n_prob) return;
@@ -304,8 +307,8 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
       const int open = pb.n_keys - p.window, t = lane & 3, n = lane >> 2;
       const int key = n < 4 ? min(n, open) : max(0, open - (n - 4));
       const __nv_bfloat16* const k = pb.k + g * p.k_stride_head + key * p.k_stride_token + t * 8;
-      float top[4];                                        // of rows n, n + 8, n + 16, n + 24
-#pragma unroll
+      float ref = 0.f;
+#pragma unroll 1
       for (int m = 0; m < 2; ++m) {
         const __nv_bfloat16* q[2];
 #pragma unroll
@@ -326,14 +329,10 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
         for (int h = 0; h < 2; ++h) {
           float x = fmaxf(acc[2 * h] * c2, acc[2 * h + 1] * c2);
           x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 1));
-          top[2 * m + h] = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 2));
+          x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, 2));
+          x = __shfl_sync(0xffffffffu, x, (row & 7) * 4);
+          if (row >> 3 == 2 * m + h) ref = x;
         }
-      }
-      float ref = 0.f;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float x = __shfl_sync(0xffffffffu, top[i], (row & 7) * 4);
-        if (row >> 3 == i) ref = x;
       }
       if (!is_row(row) || !(fabsf(ref) < 3.0e38f)) ref = 0.f;
       reinterpret_cast<ulonglong2*>(p.sums)[(size_t)gu * R + row] = make_ulonglong2(0, 0);

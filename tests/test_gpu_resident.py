@@ -13,6 +13,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("H,Hkv,d,w,N", [
     (32, 8, 128, 8, 4095), (32, 8, 128, 8, 4096), (32, 8, 128, 8, 4097),     # the general scorer's last length, this one's first
+    (16, 16, 64, 8, 4096), (18, 9, 128, 8, 7001),                            # direct teams of 9 and 16
     (32, 8, 128, 7, 9215), (32, 8, 128, 8, 18433),                           # eight teams of 18, four of 37
     (8, 2, 128, 3, 4161), (8, 2, 64, 8, 20000), (4, 4, 64, 32, 6001),        # teams of 74; of 37; one head of 32 rows
     (4, 1, 128, 8, 4737), (1, 1, 64, 1, 5000), (3, 1, 128, 8, 70001),        # one team of all SMs, its rows summed
@@ -23,7 +24,7 @@ def test_edges(cuda_device, H, Hkv, d, w, N):
     score(cuda_device, H, Hkv, d, w, N, 1 / math.sqrt(d))
 
 
-@pytest.mark.parametrize("H,Hkv,N", [(32, 8, 5000), (4, 1, 5000), (4, 1, 20000), (16, 4, 9000)])
+@pytest.mark.parametrize("H,Hkv,N", [(32, 8, 5000), (4, 1, 5000), (4, 1, 20000), (16, 4, 9000), (32, 16, 5000)])
 @pytest.mark.parametrize("scale", [-0.3, 0.0, 1.0, 3.0])
 def test_logits_far_above_the_references(cuda_device, H, Hkv, N, scale):
     """Unit-variance keys give logits of 11 |scale| nats' deviation: at 1 a CTA's sums leave the range of the summed
@@ -34,6 +35,7 @@ def test_logits_far_above_the_references(cuda_device, H, Hkv, N, scale):
 @pytest.mark.parametrize("Hkv,N", [
     (8, 4200), (1, 4200),
     (4, 4200), (4, 9400),                                                    # teams of 37, one and two tiles a CTA
+    (16, 4200), (12, 9400),                                                  # direct teams of 9 and 12
     (7, 4200), (1, 16500),                                                   # teams of 21, seven of them; one of 148
     (1, 70000), (2, 40000),                                                  # summed, four and five tiles a CTA
 ])
@@ -133,7 +135,8 @@ def test_a_layer_takes_two_launches(cuda_device):
 
 
 @pytest.mark.parametrize("H,Hkv,d,w,N", [
-    (32, 8, 128, 8, 5000), (8, 8, 64, 32, 4200),                             # small teams
+    (32, 16, 128, 8, 5000), (9, 9, 64, 32, 4200),                            # small teams
+    (32, 8, 128, 8, 5000), (8, 8, 64, 32, 4200),
     (16, 4, 64, 7, 9001), (6, 2, 128, 5, 40000), (4, 1, 128, 8, 20000),      # teams with common references
 ])
 def test_layouts_of_k(cuda_device, H, Hkv, d, w, N):
