@@ -386,14 +386,15 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
       const unsigned long long* const words = tagged_words(slot, row);
       const size_t at = (size_t)unit_of(w) * R + row;
       const unsigned tag = tag0 + u;
-      float lse = -INFINITY, Z = 0.f;
+      float lse = -INFINITY, Z = 0.f, log_z = 0.f;
       bool direct = p.sums == nullptr;
       if (!direct) {
         if (!have_ref(u, row, ref)) break;
         const unsigned long long x = summed(p.sums + 2 * at);
         if (!live) break;
         Z = (float)(x & (kSumOver - 1)) * (1.f / kSumUnit);
-        lse = word_value(ref) + __log2f(Z);
+        log_z = log2f(Z);                                  // Z is some tens: the fast one errs as much as lse's last bit
+        lse = word_value(ref) + log_z;
         ref = get_word_acquire(ref_word(u + 1, row));
         if (__any_sync(0xffffffffu, (x & kSumOver) != 0)) {   // the same answer in every CTA
           direct = true;
@@ -441,7 +442,7 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
         const unsigned long long x = summed(p.sums + 2 * at + 1);
         if (!live) break;
         const long long us = (long long)(x & (kSumCount - 1)) - (long long)(kSumBias * (unsigned long long)G);
-        ent = kLn2 * (__log2f(Z) - (float)us * (1.f / kSumUnit) / Z);
+        ent = kLn2 * (log_z - (float)us * (1.f / kSumUnit) / Z);
       } else {
         constexpr int kAt = 10;
         long long t0 = 0;
