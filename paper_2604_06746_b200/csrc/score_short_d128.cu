@@ -1,0 +1,8 @@
+// Scorer of one layer of few keys, head dimension 128.
+#include "score_short.cuh"
+
+namespace skv {
+cudaError_t short_launch_128(int shape, const ShortParams& p, int device, cudaStream_t st) {
+  return short_dispatch<128>(shape, p, device, st);
+}
+}  // namespace skv

@@ -1,0 +1,8 @@
+// Scorer of one layer of few keys, head dimension 64.
+#include "score_short.cuh"
+
+namespace skv {
+cudaError_t short_launch_64(int shape, const ShortParams& p, int device, cudaStream_t st) {
+  return short_dispatch<64>(shape, p, device, st);
+}
+}  // namespace skv

@@ -1,6 +1,6 @@
 // Host side of the tensor-core scorer (score_tc.cuh): tensor maps, how a call's work is cut into
 // tasks and in which order they are drawn.
-#include "score_tc.cuh"
+#include "score_short.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -86,6 +86,51 @@ int batch_cut(const Layout& l, const ScoreCall& a, int sms) {
     all += (float)pairs * l.w_total / kFullWeight / sms;
   }
   return longest[0] <= all + 0.25f * longest[1] + 1.f ? 1 : 2;
+}
+
+// The form for one layer whose segments all run at once, two pairs of tiles each at most (score_short.cuh).  False: not this call.
+bool launch_short(const Ctx& ctx, const ScoreCall& a, int first, cudaStream_t st, cudaError_t* e) {
+  const structkv_config& cfg = ctx.cfg;
+  const Layout l = layout_of(cfg);
+  const int sms = std::min(ctx.sm_count, kMaxSms);
+  const int n_keys = a.cu_seqlens ? a.cu_seqlens[1] : a.n_keys;
+  const int tiles = (n_keys + kKeyTile - 1) / kKeyTile, pairs = (tiles + 1) / 2, s1 = segments(l, sms, tiles, sms);
+  // (units of equal weight have equally many segments; the exchange words of a context of one call hold anything)
+  if (l.shape >= kNarrow32 || l.w_last != kFullWeight || s1 % l.units != 0 || s1 > sms || ctx.old_words) return false;
+  ShortParams p;
+  p.n_seg = s1 / l.units;
+  if (2 * ((pairs + p.n_seg - 1) / p.n_seg) > kShortTiles) return false;
+  p.n_pairs = pairs;
+  p.split = p.n_seg == pairs && 2 * s1 <= sms && l.rows_pg - (l.n_rb - 1) * kRowBlock > kRowBlock / 2;
+  p.n_tasks = s1 << p.split;
+  const cuuint64_t row = (cuuint64_t)cfg.head_dim * 2, s_tok = (cuuint64_t)a.k_stride_token * 2;
+  const cuuint64_t s_head = cfg.n_kv_heads == 1 ? s_tok * (cuuint64_t)n_keys : (cuuint64_t)a.k_stride_head * 2;
+  *e = cudaErrorInvalidValue;
+  if (!tc_encode3(ctx, &p.map_q, a.q[first], cfg.window, (cuuint64_t)cfg.n_q_heads, row, row * cfg.window,
+                  std::min(ctx.w_pad, kRowBlock / 2), std::max(1, kRowBlock / 2 / ctx.w_pad)) ||
+      !tc_encode3(ctx, &p.map_k, a.k[first], n_keys, cfg.n_kv_heads, s_tok, s_head, kKeyTile, 1))
+    return true;
+  p.cols = a.cols + (size_t)first * a.cols_layer_stride;
+  p.row_ent = a.row_ent + (size_t)first * ctx.rows_pad;
+  p.xch = ctx.ws.xch;
+  p.ctl = ctx.ws.ctl;
+  p.status = ctx.ws.status;
+  p.col_stride = a.col_stride;
+  const float c2 = a.scale[first] * kLog2e;
+  p.negate = c2 < 0.f;
+  p.c2 = std::max(std::fabs(c2), 1e-30f);
+  p.inv_c2 = 1.f / p.c2;
+  p.v_min = -125.f / p.c2;
+  p.n_keys = n_keys;
+  p.window = cfg.window;
+  p.w_pad = ctx.w_pad;
+  p.w_shift = 0;
+  while ((1 << p.w_shift) < ctx.w_pad) ++p.w_shift;
+  p.group = l.group;
+  p.rows_pg = l.rows_pg;
+  p.n_rb = l.n_rb;
+  *e = cfg.head_dim == 128 ? short_launch_128(l.shape, p, ctx.device, st) : short_launch_64(l.shape, p, ctx.device, st);
+  return true;
 }
 
 template <int MAXP>
@@ -252,10 +297,12 @@ cudaError_t launch_score_tc(const Ctx& ctx, const ScoreCall& a, cudaStream_t st)
     if (e != cudaErrorCooperativeLaunchTooLarge) return e;
     cudaGetLastError();
   }
+  cudaError_t e = cudaSuccess;
+  if (a.n == 1 && launch_short(ctx, a, 0, st, &e)) return e;
   if (a.cu_seqlens) return a.n == 1 ? launch_problems<1>(ctx, a, 0, 1, st) : launch_problems<kMaxBatch>(ctx, a, 0, a.n, st);
   for (int l = 0; l < a.n; l += kMaxBatch) {
     const int n = std::min(kMaxBatch, a.n - l);
-    const cudaError_t e = n == 1 ? launch_problems<1>(ctx, a, l, 1, st) : launch_problems<kMaxBatch>(ctx, a, l, n, st);
+    e = n == 1 ? launch_problems<1>(ctx, a, l, 1, st) : launch_problems<kMaxBatch>(ctx, a, l, n, st);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
