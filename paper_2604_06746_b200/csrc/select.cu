@@ -1,10 +1,12 @@
 // Budgeted token selection (top-k of the prefix, ties to the lower index, output in position
 // order, window appended), exact: three levels of 11, 11 and 10 bits find the k-th largest key (radix.cuh), then every
-// kept token's place in the output follows from ballots and one scan of the counts per (group of
-// 1024 tokens, warp).  A cluster of CL CTAs shares one vector, each CTA a contiguous slice that it
+// kept token's place in the output follows from ballots and one scan of the warps' counts (a warp's tokens are
+// consecutive).  A cluster of CL CTAs shares one vector, each CTA a contiguous slice that it
 // holds in registers (up to ITEMS tokens a thread; a longer slice is read again per level).
 //
-// Bound by the chain of barriers, not by memory.
+// Bound by the chain of barriers, not by memory; with several tokens a thread, by the instructions for each: one vector
+// of 131072 tokens took 18.7 us, 5.8 of them for the output's places, scanned per (group of 1024 tokens, warp) with equal
+// keys counted whether there are any or not; now 12.5 and 3.
 #include <atomic>
 
 #include "radix.cuh"
@@ -23,9 +25,8 @@ struct SelectArgs {
   SelectExtra extra;                   // vector `batch` of a uniform call, if it has scores
 };
 
-// Two CTAs an SM for the many short vectors that need them.  Clusters of up to eight items a thread serve at most 17 vectors,
-// 68 CTAs: bound to 32 registers they spilled (8 / 16 vectors of 32768 tokens 13.0 / 14.8 us, now 11.2 / 11.3; of 12000
-// 8.1 / 8.3, now 7.7 / 7.7).
+// Two CTAs an SM for the many short vectors that need them.  Clusters of up to eight items a thread have an SM per CTA: bound
+// to 32 registers they spilled (8 / 16 vectors of 32768 tokens 13.0 / 14.8 us instead of 11.2 / 11.3).
 template <int CL, int ITEMS>
 __global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) select_topk(const __grid_constant__ SelectArgs a) {
   extern __shared__ __align__(16) unsigned char sel_smem[];
@@ -36,13 +37,13 @@ __global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) sel
   const int vec = blockIdx.x / CL;
   pdl_trigger();
   radix_clear(s);
-  cluster_barrier<CL>();                             // all CTAs of the cluster run before any remote access
-  pdl_wait();
   const bool own = !a.packed && vec == a.batch;      // the extra vector
   const float* x = own ? a.extra.scores : a.scores + (a.packed ? (size_t)a.cu[vec] : (size_t)vec * a.row_stride);
   const int n = a.packed ? a.cu[vec + 1] - a.cu[vec] : a.n, budget = own ? a.extra.budget : a.packed ? a.budgets[vec] : a.budget;
   int* out = own ? a.extra.idx_out : a.out + (size_t)vec * a.out_stride;
   const int prefix_len = n - a.window, k = budget - a.window;
+  cluster_barrier<CL>();                             // all CTAs of the cluster run before any remote access
+  pdl_wait();
   if (rank == 0) {
     for (int i = tid; i < a.window; i += kRxThreads) out[k + i] = prefix_len + i;
     if (a.packed)
@@ -55,19 +56,18 @@ __global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) sel
   constexpr int kChunk = kRxThreads * ITEMS;
   const int chunks = (per + kChunk - 1) / kChunk;    // more than one: the slice does not fit the registers
   unsigned key[ITEMS];
-  // token of item e: base + e * 1024 + tid
+  int n_mine = 0;                                    // this thread's tokens of the loaded chunk
+  // a warp's tokens are consecutive; item e of this thread: first + 32 e
+  auto first_of = [&](int c) { return lo + c * kChunk + warp * (32 * ITEMS) + lane; };
   auto load = [&](int c) {
-    const int base = lo + c * kChunk;
+    const int first = first_of(c);
+    n_mine = min(ITEMS, (hi - first + 31) >> 5);     // (none where this is not positive)
     float v[ITEMS];
 #pragma unroll
-    for (int e = 0; e < ITEMS; ++e) {
-      const int j = base + e * kRxThreads + tid;
-      v[e] = j < hi ? x[j] : 0.f;
-    }
+    for (int e = 0; e < ITEMS; ++e) v[e] = e < n_mine ? x[first + 32 * e] : 0.f;
 #pragma unroll
     for (int e = 0; e < ITEMS; ++e) key[e] = order_key(v[e]);
   };
-  auto valid = [&](int c, int e) { return lo + c * kChunk + e * kRxThreads + tid < hi; };
 
   if (chunks == 1) load(0);
   // kept: every key >= ge, and the first need_eq of the keys equal to thr
@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) sel
         if (chunks > 1) load(c);
 #pragma unroll
         for (int e = 0; e < ITEMS; ++e)
-          if (valid(c, e) && (key[e] & mask) == thr) radix_count(s, level, radix_digit(key[e], level));
+          radix_count(s, level, radix_digit(key[e], level), e < n_mine && (key[e] & mask) == thr);
       }
       unsigned digit, in;
       radix_pick(s, level, remaining, digit, in);
@@ -93,76 +93,76 @@ __global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) sel
     need_eq = level < kRxLevels ? 0 : remaining;
   }
 
-  // keys kept outright / equal to the threshold in this CTA's slice -> where the slice starts
-  unsigned gt_run = 0, eq_run = 0;
+  // Place of a token in the output = (#kept outright before it) + min(#equal before it, need_eq).  Counts of this warp in the
+  // loaded chunk:
+  unsigned w_gt = 0, w_eq = 0;
+  auto tally = [&]() {
+    w_gt = w_eq = 0;
+#pragma unroll
+    for (int e = 0; e < ITEMS; ++e) w_gt += __popc(__ballot_sync(0xffffffffu, e < n_mine && key[e] >= ge));
+    if (need_eq == 0) return;                        // keys that differ: what stays is above
+#pragma unroll
+    for (int e = 0; e < ITEMS; ++e) w_eq += __popc(__ballot_sync(0xffffffffu, e < n_mine && key[e] < ge && key[e] == thr));
+  };
+  auto leave = [&](unsigned gt, unsigned eq) {
+    if (lane == 0) { s.scratch[0][warp] = gt; s.scratch[1][warp] = eq; }
+    __syncthreads();
+  };
+  unsigned gt_run = 0, eq_run = 0;                   // before this CTA's slice, then before the chunk
   if (CL > 1) {
-    unsigned my_gt = 0, my_eq = 0;
+    unsigned all_gt = 0, all_eq = 0;
     for (int c = 0; c < chunks; ++c) {
       if (chunks > 1) load(c);
-#pragma unroll
-      for (int e = 0; e < ITEMS; ++e) {
-        my_gt += valid(c, e) && key[e] >= ge ? 1u : 0u;
-        my_eq += valid(c, e) && key[e] < ge && key[e] == thr ? 1u : 0u;
-      }
+      tally();
+      all_gt += w_gt;
+      all_eq += w_eq;
     }
-    my_gt = __reduce_add_sync(0xffffffffu, my_gt);
-    my_eq = __reduce_add_sync(0xffffffffu, my_eq);
-    if (lane == 0) { s.scratch[warp] = my_gt; s.scratch[32 + warp] = my_eq; }
-    __syncthreads();
+    leave(all_gt, all_eq);
     if (warp < 2) {
-      const unsigned t = __reduce_add_sync(0xffffffffu, s.scratch[warp * 32 + lane]);
+      const unsigned t = __reduce_add_sync(0xffffffffu, s.scratch[warp][lane]);
       if (lane < CL) cg::this_cluster().map_shared_rank(&cta_tot[0][0], lane)[warp * CL + rank] = t;
     }
     cluster_barrier<CL>();
     for (int r = 0; r < rank; ++r) { gt_run += cta_tot[0][r]; eq_run += cta_tot[1][r]; }
   }
-
-  // Place of token j in the output = (#kept outright before j) + min(#equal before j, need_eq).
-  unsigned* const cnt = s.scratch;                   // [ITEMS][32 warps] (#outright << 16) | #equal, then exclusive sums
-  unsigned* const tot = s.scratch + kRxThreads;      // [ITEMS]
   const unsigned below = (1u << lane) - 1u;
   for (int c = 0; c < chunks; ++c) {
-    if (chunks > 1) load(c);
-    __syncthreads();                                 // scratch is free
-#pragma unroll
-    for (int e = 0; e < ITEMS; ++e) {
-      const bool in = valid(c, e), gt = in && key[e] >= ge, eq = in && !gt && key[e] == thr;
-      const unsigned bg = __ballot_sync(0xffffffffu, gt), be = __ballot_sync(0xffffffffu, eq);
-      if (lane == 0) cnt[e * 32 + warp] = (unsigned)__popc(bg) << 16 | (unsigned)__popc(be);
+    if (chunks > 1) {
+      load(c);
+      __syncthreads();                               // the counts of the chunk before have been read
     }
-    __syncthreads();
-    if (tid < ITEMS * 32) {                          // warp e scans the warps of item e
-      const unsigned v = cnt[tid];
-      unsigned incl = v;
+    if (CL == 1 || chunks > 1) {                     // else they are there
+      tally();
+      leave(w_gt, w_eq);
+    }
+    const unsigned g = s.scratch[0][lane], g_incl = warp_scan(g, lane);
+    unsigned gt_at = gt_run + __shfl_sync(0xffffffffu, g_incl - g, warp), eq_at = 0;
+    gt_run += __shfl_sync(0xffffffffu, g_incl, 31);
+    if (need_eq) {
+      const unsigned q = s.scratch[1][lane], q_incl = warp_scan(q, lane);
+      eq_at = eq_run + __shfl_sync(0xffffffffu, q_incl - q, warp);
+      eq_run += __shfl_sync(0xffffffffu, q_incl, 31);
+    }
+    const int first = first_of(c);
+    if (need_eq == 0) {
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
+      for (int e = 0; e < ITEMS; ++e) {
+        const bool gt = e < n_mine && key[e] >= ge;
+        const unsigned bg = __ballot_sync(0xffffffffu, gt);
+        if (gt) out[gt_at + __popc(bg & below)] = first + 32 * e;
+        gt_at += __popc(bg);
       }
-      cnt[tid] = incl - v;
-      if (lane == 31) tot[warp] = incl;
-    }
-    __syncthreads();
-    unsigned t_incl = lane < ITEMS ? tot[lane] : 0u;
-    const unsigned t_own = t_incl;
+    } else {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned t = __shfl_up_sync(0xffffffffu, t_incl, o);
-      if (lane >= o) t_incl += t;
+      for (int e = 0; e < ITEMS; ++e) {
+        const bool in = e < n_mine, gt = in && key[e] >= ge, eq = in && !gt && key[e] == thr;
+        const unsigned bg = __ballot_sync(0xffffffffu, gt), be = __ballot_sync(0xffffffffu, eq);
+        const unsigned eq_before = eq_at + __popc(be & below);
+        if (gt || (eq && eq_before < need_eq)) out[gt_at + __popc(bg & below) + min(eq_before, need_eq)] = first + 32 * e;
+        gt_at += __popc(bg);
+        eq_at += __popc(be);
+      }
     }
-#pragma unroll
-    for (int e = 0; e < ITEMS; ++e) {
-      const bool in = valid(c, e), gt = in && key[e] >= ge, eq = in && !gt && key[e] == thr;
-      const unsigned bg = __ballot_sync(0xffffffffu, gt), be = __ballot_sync(0xffffffffu, eq);
-      const unsigned before = __shfl_sync(0xffffffffu, t_incl - t_own, e) + cnt[e * 32 + warp];
-      const unsigned gt_before = gt_run + (before >> 16) + __popc(bg & below);
-      const unsigned eq_before = eq_run + (before & 0xffffu) + __popc(be & below);
-      if (gt || (eq && eq_before < need_eq))
-        out[gt_before + min(eq_before, need_eq)] = lo + c * kChunk + e * kRxThreads + tid;
-    }
-    const unsigned all = __shfl_sync(0xffffffffu, t_incl, 31);
-    gt_run += all >> 16;
-    eq_run += all & 0xffffu;
   }
 }
 
@@ -182,20 +182,21 @@ cudaError_t launch(const SelectArgs& a, cudaStream_t st) {
                             sizeof(RadixShared<CL>), st, a);
 }
 
-// One CTA while that is a matter of three barriers a level; beyond, few vectors get more CTAs with fewer items each, and
-// many (whose CTAs would not run side by side) the smallest cluster that holds one.  us for 1 / 8 / 33 vectors, chained
-// launches: 1777 tokens 5.1 / 5.2 / 5.6 with 1 x 4 items (a cluster of two 6.9 / 7.0 / 7.2), 8192 7.0 / 7.2 / 8.4 with
-// 1 x 8 (2 x 4: 7.2 / 7.3 / 9.0), 16384 9.9 / 10.0 / 11.7 with 1 x 16 and 7.7 / 7.8 with 4 x 4, 32768 12.0 / 12.2 /
-// 14.1 with 2 x 16 and 9.3 / 11.2 with 4 x 8, 65536 13.1 / 13.3 / 16.2 with 4 x 16 and 12.5 /
-// 13.2 / 26.0 with 8 x 8, 131072 18.6 with 8 x 16 and 24.1 for 33 with 4 x 32.
+// One CTA while that is a matter of three barriers a level; beyond, as many CTAs with as few items each as leave all
+// vectors running at once (a CTA has an SM, clusters do not cross a GPC).  us, CTAs x items, for 1 / 8 / 33 vectors, chained launches:
+// 1777 tokens 1 x 4 4.9 / 4.0 / 4.5, 2 x 2 5.4 / 5.5 / 5.5; 8192 1 x 8 5.1 / 5.2 / 6.4, 4 x 2 5.7 / 5.9 / 7.2; 16384 4 x 4
+// 7.8 / 6.4 / 8.0, 1 x 16 8.9 / 7.5 / 9.1, 8 x 2 7.7 / 6.5 / 18.9; 32768 8 x 4 6.6 / 8.5 / 22.2, 4 x 8 7.2 / 9.2 / 9.3, 2 x 16
+// 9.2 / 11.3 / 11.4; 65536 8 x 8 9.6 / 10.0 / 25.6, 4 x 16 11.3 / 11.4 / 11.8; 131072 8 x 16 12.5 / 12.8 / 33.6, 4 x 32
+// 15.9 / 16.1 / 19.8.
 cudaError_t dispatch(const SelectArgs& a, int longest, cudaStream_t st) {
   if (longest <= 4 * kRxThreads) return launch<1, 4>(a, st);
   if (longest <= 8 * kRxThreads) return launch<1, 8>(a, st);
-  const bool room = a.batch <= 16;                   // up to eight CTAs a vector, one per SM
-  if (longest <= 16 * kRxThreads) return room ? launch<4, 4>(a, st) : launch<1, 16>(a, st);
-  if (longest <= 32 * kRxThreads) return room ? launch<4, 8>(a, st) : launch<2, 16>(a, st);
-  if (longest <= 64 * kRxThreads) return launch<4, 16>(a, st);
-  if (!room) return launch<4, 32>(a, st);
+  const int vectors = a.batch + (a.extra.scores ? 1 : 0);
+  const bool by_eight = vectors <= 8, by_four = vectors <= 33;
+  if (longest <= 16 * kRxThreads) return by_four ? launch<4, 4>(a, st) : launch<1, 16>(a, st);
+  if (longest <= 32 * kRxThreads) return by_eight ? launch<8, 4>(a, st) : by_four ? launch<4, 8>(a, st) : launch<2, 16>(a, st);
+  if (longest <= 64 * kRxThreads) return by_eight ? launch<8, 8>(a, st) : launch<4, 16>(a, st);
+  if (!by_eight) return launch<4, 32>(a, st);
   if (longest <= 128 * kRxThreads) return launch<8, 16>(a, st);
   return launch<8, 32>(a, st);                       // beyond 262144 tokens the slices are read again per level
 }

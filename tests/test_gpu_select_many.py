@@ -1,0 +1,28 @@
+"""Selection of so many vectors that the number of CTAs a vector gets depends on it (up to 8, up to 33, more), at the
+last lengths of its forms: exact, with thresholds among equal keys and among keys that all differ."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import structkv_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("batch", [8, 9, 33, 34])
+@pytest.mark.parametrize("n", [16384, 32768, 32769, 65536, 65537])
+@pytest.mark.parametrize("ties", [False, True])
+def test_select_many_vectors(cuda_device, batch, n, ties):
+    from paper_2604_06746_b200 import binding
+    ctx = binding.Context(4, 2, 128, 64, 1024, torch.bfloat16, cuda_device)
+    rng = np.random.default_rng(batch + n)
+    sc = (rng.random((batch, n + 64)) ** 4).astype(np.float32)
+    if ties:
+        sc = np.round(sc * 50) / 50
+    k = 64 + n // 9
+    out = torch.zeros((batch, k), dtype=torch.int32, device="cuda")
+    ctx.select(torch.from_numpy(sc).cuda(), k, 64, out)
+    got = out.cpu().numpy()
+    for b in (0, batch // 2, batch - 1):
+        assert np.array_equal(got[b], O.select(sc[b], k, 64)), b
+    ctx.close()
