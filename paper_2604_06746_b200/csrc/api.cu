@@ -64,31 +64,31 @@ Workspace carve_workspace(const structkv_config& cfg, void* base) {
 
 // ---- host words the device writes for the host: one page-locked block per process, a slot per context --
 struct HostSlot {
-  int* mem;                              // [kSlotInts], mapped
+  unsigned long long* mem;               // [kSlotWords], mapped
   unsigned seq;                          // calls so far: tags the answers
 };
 namespace {
-constexpr int kSlots = 64, kSlotInts = 256;
-static_assert(kSlotInts > kMaxStatLayers, "a slot holds the pivot and every T_l");
+constexpr int kSlots = 64, kSlotWords = 144;
+static_assert(kSlotWords > kMaxStatLayers, "a slot holds the pivot and every T_l");
 std::mutex g_slot_mutex;
-int* g_slot_mem = nullptr;
+unsigned long long* g_slot_mem = nullptr;
 bool g_slot_used[kSlots];
 
 // A slot for the context, or NULL: none left, or no page-locked memory (the caller then copies).
 HostSlot* take_slot() {
   std::lock_guard<std::mutex> lock(g_slot_mutex);
   if (!g_slot_mem &&
-      cudaHostAlloc((void**)&g_slot_mem, sizeof(int) * kSlots * kSlotInts, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      cudaHostAlloc((void**)&g_slot_mem, sizeof(*g_slot_mem) * kSlots * kSlotWords, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
     g_slot_mem = nullptr;
     cudaGetLastError();
     return nullptr;
   }
   for (int i = 0; i < kSlots; ++i)
     if (!g_slot_used[i]) {
-      HostSlot* s = new (std::nothrow) HostSlot{g_slot_mem + i * kSlotInts, 0};
+      HostSlot* s = new (std::nothrow) HostSlot{g_slot_mem + i * kSlotWords, 0};
       if (!s) return nullptr;
       g_slot_used[i] = true;
-      s->mem[0] = 0;
+      std::fill(s->mem, s->mem + kSlotWords, 0ull);
       return s;
     }
   return nullptr;
@@ -96,7 +96,7 @@ HostSlot* take_slot() {
 void give_back(HostSlot* s) {
   if (!s) return;
   std::lock_guard<std::mutex> lock(g_slot_mutex);
-  g_slot_used[(s->mem - g_slot_mem) / kSlotInts] = false;
+  g_slot_used[(s->mem - g_slot_mem) / kSlotWords] = false;
   delete s;
 }
 }  // namespace
@@ -463,7 +463,7 @@ static structkv_status enqueue_pivot_select(Ctx& c, const float* s_hist, long lo
                                             const float* metrics, const float* weights, int l_limit, float lambda, int window,
                                             int kv_budget, int* i_kv, int struct_budget, float* c_star, int* i_struct,
                                             cudaStream_t st) {
-  const int tag = (int)(++c.slot->seq << 8);
+  const unsigned tag = ++c.slot->seq == 0 ? ++c.slot->seq : c.slot->seq;   // never that of clean words
   if (launch_accumulate_at_pivot(s_hist, row_stride, n_layers, n, lambda, metrics, weights, l_limit, c_star, c.slot->mem,
                                  tag, st) != cudaSuccess)
     return STRUCTKV_ERR_CUDA;
@@ -471,23 +471,23 @@ static structkv_status enqueue_pivot_select(Ctx& c, const float* s_hist, long lo
   return launch_select(s_hist, row_stride, n_layers, n, kv_budget, window, i_kv, st, &extra) == cudaSuccess ? STRUCTKV_OK
                                                                                                             : STRUCTKV_ERR_CUDA;
 }
-// Waits for the word enqueue_pivot_select asked for.
+// Waits for the words enqueue_pivot_select asked for.
 static structkv_status await_pivot(Ctx& c, int n_layers, int* pivot_out, float* t_out, cudaStream_t st) {
-  volatile int* mem = c.slot->mem;
-  const unsigned tag = c.slot->seq << 8;
-  for (unsigned spins = 1; ((unsigned)mem[0] & ~255u) != tag; ++spins) {
-    if (spins % 100000 != 0) continue;                 // tens of microseconds
-    const cudaError_t e = cudaStreamQuery(st);
-    if (e == cudaErrorNotReady) continue;
-    if (e != cudaSuccess || ((unsigned)mem[0] & ~255u) != tag) return STRUCTKV_ERR_CUDA;   // done, and no word
-  }
-  std::atomic_thread_fence(std::memory_order_acquire);
-  *pivot_out = mem[0] & 255;
-  if (t_out)
-    for (int l = 0; l < n_layers; ++l) {
-      const int bits = mem[1 + l];
-      std::memcpy(&t_out[l], &bits, sizeof(float));
+  const volatile unsigned long long* mem = c.slot->mem;
+  const unsigned tag = c.slot->seq;
+  unsigned spins = 0;
+  for (int i = 0; i <= (t_out ? n_layers : 0); ++i) {
+    unsigned long long word;
+    while ((unsigned)((word = mem[i]) >> 32) != tag) {
+      if (++spins % 100000 != 0) continue;               // tens of microseconds
+      const cudaError_t e = cudaStreamQuery(st);
+      if (e == cudaErrorNotReady) continue;
+      if (e != cudaSuccess || (unsigned)(mem[i] >> 32) != tag) return STRUCTKV_ERR_CUDA;   // done, and no word
     }
+    const unsigned value = (unsigned)word;
+    if (i == 0) *pivot_out = (int)value;
+    else std::memcpy(&t_out[i - 1], &value, sizeof(float));
+  }
   return STRUCTKV_OK;
 }
 static bool pivot_select_args_ok(const float* s_hist, long long row_stride, int n_layers, int n, const float* metrics,

@@ -129,11 +129,11 @@ cudaError_t launch_head_stats_batch(const Ctx& ctx, const float* cols, long long
 cudaError_t launch_accumulate(const float* s_hist, long long row_stride, int pivot, int n,
                               float lambda, float* c_out, cudaStream_t st);
 
-// Eq. 7-9 on the device (n_layers <= kMaxStatLayers), then launch_accumulate at that pivot.  `host` (mapped
-// memory) receives T_l [n_layers] from word 1 on and then, in word 0, tag | pivot (the tag's low byte is 0).
+// Eq. 7-9 on the device (n_layers <= kMaxStatLayers), then launch_accumulate at that pivot.  `host` (mapped memory)
+// receives the pivot in word 0 and T_l [n_layers] from word 1 on, each below the tag in the upper half, in any order.
 cudaError_t launch_accumulate_at_pivot(const float* s_hist, long long row_stride, int n_layers, int n, float lambda,
-                                       const float* metrics, const float* weights, int l_limit, float* c_out, int* host,
-                                       int tag, cudaStream_t st);
+                                       const float* metrics, const float* weights, int l_limit, float* c_out,
+                                       unsigned long long* host, unsigned tag, cudaStream_t st);
 
 // One more vector of a selection, with its own budget and output.
 struct SelectExtra { const float* scores; int budget; int* idx_out; };

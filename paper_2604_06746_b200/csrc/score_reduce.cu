@@ -453,66 +453,74 @@ __global__ void __launch_bounds__(128) accumulate(const float* __restrict__ s_hi
   *reinterpret_cast<T*>(c_out + j) = c;
 }
 
-// Eq. 7-9, then the same recursion.  Every block finds the pivot for itself (one warp, 2 us), so that no
-// launch and no host round trip comes between the metrics and the centrality.  The last block sums
-// nothing: it tells the host, beside the others' sums.
+// Eq. 7-9, then the same recursion.  Every block finds the pivot for itself, so that no launch and no host round trip comes
+// between the metrics and the centrality, while its first kEarly layers are on their way.  The last block sums nothing: it
+// tells the host, beside the others' sums, in words that carry the call's tag, so that none waits for another.
+// Bound by latency, above all by fetching instructions that nothing has run before: with one warp for the three columns
+// and four rounds of layers, all unrolled, a dozen double divisions written out, the smallest launches took 8.8 to 10 us by
+// themselves; with a warp per column and rolled loops 5.2 to 5.4 (whole prefills 3.5 to 4.3 us less).
+constexpr int kPivotThreads = 128, kEarly = 8;
 template <int VEC>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kPivotThreads)
 accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int n_layers, int n, float lambda,
                     const float* __restrict__ metrics, float3 weights, int l_limit, float* __restrict__ c_out,
-                    volatile int* host, int tag) {
+                    volatile unsigned long long* host, unsigned tag) {
   using T = typename Keys<VEC>::T;
+  __shared__ float m_s[3 * kMaxStatLayers];
+  __shared__ double t_s[3][kMaxStatLayers];
   __shared__ int pivot_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool tells = blockIdx.x == gridDim.x - 1;
+  const int j = (blockIdx.x * kPivotThreads + tid) * VEC;
+  const bool sums = !tells && j < n;
   pdl_trigger();
   pdl_wait();
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    constexpr int kPer = kMaxStatLayers / 32;
-    double Tl[kPer];
+  for (int i = tid; i < 3 * n_layers; i += kPivotThreads) m_s[i] = metrics[i];
+  T early[kEarly] = {};
+  if (sums) {
 #pragma unroll
-    for (int k = 0; k < kPer; ++k) Tl[k] = 0.0;
-#pragma unroll
-    for (int col = 0; col < 3; ++col) {                    // unrolled: the three chains overlap
-      const double sign = col == 0 ? -1.0 : 1.0, w = col == 0 ? weights.x : col == 1 ? weights.y : weights.z;
-      double d[kPer], lo = INFINITY, hi = -INFINITY;
-      int nan = 0;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        const int l = lane + 32 * k;
-        if (l < n_layers) {
-          const float m = metrics[l * 3 + col], before = l > 0 ? metrics[(l - 1) * 3 + col] : 0.f;
-          nan |= isnan(m);
-          d[k] = sign * ((double)m - (double)before);
-          if (l > 0) { lo = d[k] < lo ? d[k] : lo; hi = d[k] > hi ? d[k] : hi; }
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const double a = __shfl_xor_sync(0xffffffffu, lo, o), b = __shfl_xor_sync(0xffffffffu, hi, o);
-        lo = a < lo ? a : lo;
-        hi = b > hi ? b : hi;
-      }
-      const bool usable = !__any_sync(0xffffffffu, nan) && hi > lo;
-#pragma unroll
-      for (int k = 0; k < kPer; ++k) {
-        const int l = lane + 32 * k;
-        if (usable && l > 0 && l < n_layers)
-          Tl[k] = __dadd_rn(Tl[k], __ddiv_rn(__dmul_rn(w, __dsub_rn(d[k], lo)), __dsub_rn(hi, lo)));
-      }
+    for (int l = 0; l < kEarly; ++l)
+      if (l < n_layers) early[l] = *reinterpret_cast<const T*>(s_hist + (size_t)l * row_stride + j);
+  }
+  __syncthreads();
+  if (warp < 3) {                                          // a column each
+    const double w = warp == 0 ? weights.x : warp == 1 ? weights.y : weights.z;
+    auto step = [&](int l) {                               // Eq. 8 takes the gradient of -entropy
+      const double d = (double)m_s[3 * l + warp] - (double)m_s[3 * l - 3 + warp];
+      return warp == 0 ? -d : d;
+    };
+    double lo = INFINITY, hi = -INFINITY;
+    int nan = 0;
+#pragma unroll 1
+    for (int l = lane; l < n_layers; l += 32) {
+      nan |= isnan(m_s[3 * l + warp]);
+      if (l == 0) continue;
+      const double d = step(l);
+      lo = d < lo ? d : lo;
+      hi = d > hi ? d : hi;
     }
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) {
+      const double a = __shfl_xor_sync(0xffffffffu, lo, o), b = __shfl_xor_sync(0xffffffffu, hi, o);
+      lo = a < lo ? a : lo;
+      hi = b > hi ? b : hi;
+    }
+    const bool usable = !__any_sync(0xffffffffu, nan) && hi > lo;
+#pragma unroll 1
+    for (int l = lane; l < n_layers; l += 32)
+      t_s[warp][l] = usable && l > 0 ? __ddiv_rn(__dmul_rn(w, __dsub_rn(step(l), lo)), __dsub_rn(hi, lo)) : 0.0;
+  }
+  __syncthreads();
+  if (warp == 0) {
     double best = -INFINITY;
     int at = kMaxStatLayers;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-      const int l = lane + 32 * k;
-      if (l > 0 && l < n_layers && Tl[k] > best) { best = Tl[k]; at = l; }
-      if (tells && l < n_layers) {
-        host[1 + l] = __float_as_int((float)Tl[k]);
-        __threadfence_system();
-      }
+#pragma unroll 1
+    for (int l = lane; l < n_layers; l += 32) {
+      const double t = __dadd_rn(__dadd_rn(t_s[0][l], t_s[1][l]), t_s[2][l]);
+      if (l > 0 && t > best) { best = t; at = l; }
+      if (tells) host[1 + l] = (unsigned long long)tag << 32 | (unsigned)__float_as_int((float)t);
     }
-#pragma unroll
+#pragma unroll 1
     for (int o = 16; o > 0; o >>= 1) {
       const double b = __shfl_xor_sync(0xffffffffu, best, o);
       const int i = __shfl_xor_sync(0xffffffffu, at, o);
@@ -520,23 +528,21 @@ accumulate_at_pivot(const float* __restrict__ s_hist, long long row_stride, int 
     }
     if (at == kMaxStatLayers) at = n_layers >= 2 ? 1 : 0;   // one layer, or nothing compares
     if (n_layers >= 2 && l_limit >= 0 && at > l_limit) at = l_limit;
-    __syncwarp();
     if (lane == 0) {
       pivot_s = at;
-      if (tells) {                                     // last: the host polls this word
-        __threadfence_system();
-        host[0] = tag | at;
-      }
+      if (tells) host[0] = (unsigned long long)tag << 32 | (unsigned)at;
     }
   }
   if (tells) return;
   __syncthreads();
+  if (!sums) return;
   const int pivot = pivot_s;
-  const int j = (blockIdx.x * blockDim.x + threadIdx.x) * VEC;
-  if (j >= n) return;
   T c{};
-#pragma unroll 16
-  for (int l = 0; l <= pivot; ++l) c = decay(lambda, c, *reinterpret_cast<const T*>(s_hist + (size_t)l * row_stride + j));
+#pragma unroll
+  for (int l = 0; l < kEarly; ++l)
+    if (l <= pivot) c = decay(lambda, c, early[l]);
+#pragma unroll 8
+  for (int l = kEarly; l <= pivot; ++l) c = decay(lambda, c, *reinterpret_cast<const T*>(s_hist + (size_t)l * row_stride + j));
   *reinterpret_cast<T*>(c_out + j) = c;
 }
 
@@ -631,14 +637,14 @@ cudaError_t launch_accumulate(const float* s_hist, long long row_stride, int piv
 }
 
 cudaError_t launch_accumulate_at_pivot(const float* s_hist, long long row_stride, int n_layers, int n, float lambda,
-                                       const float* metrics, const float* weights, int l_limit, float* c_out, int* host,
-                                       int tag, cudaStream_t st) {
+                                       const float* metrics, const float* weights, int l_limit, float* c_out,
+                                       unsigned long long* host, unsigned tag, cudaStream_t st) {
   const float3 w = make_float3(weights[0], weights[1], weights[2]);
   if (n % 4 == 0 && row_stride % 4 == 0 && (uintptr_t)s_hist % 16 == 0 && (uintptr_t)c_out % 16 == 0)
-    return launch_pdl(accumulate_at_pivot<4>, dim3((n / 4 + 127) / 128 + 1), dim3(128), 0, st, s_hist, row_stride, n_layers, n,
-                      lambda, metrics, w, l_limit, c_out, (volatile int*)host, tag);
-  return launch_pdl(accumulate_at_pivot<1>, dim3((n + 127) / 128 + 1), dim3(128), 0, st, s_hist, row_stride, n_layers, n, lambda,
-                    metrics, w, l_limit, c_out, (volatile int*)host, tag);
+    return launch_pdl(accumulate_at_pivot<4>, dim3((n / 4 + kPivotThreads - 1) / kPivotThreads + 1), dim3(kPivotThreads), 0, st, s_hist, row_stride, n_layers, n,
+                      lambda, metrics, w, l_limit, c_out, (volatile unsigned long long*)host, tag);
+  return launch_pdl(accumulate_at_pivot<1>, dim3((n + kPivotThreads - 1) / kPivotThreads + 1), dim3(kPivotThreads), 0, st, s_hist, row_stride, n_layers, n, lambda,
+                    metrics, w, l_limit, c_out, (volatile unsigned long long*)host, tag);
 }
 
 }  // namespace skv
