@@ -223,6 +223,12 @@ inline cudaError_t launch_cooperative(void (*kernel)(Arg), dim3 grid, dim3 block
   return cudaLaunchKernelExC(&cfg, (const void*)kernel, args);
 }
 
+// Adds one to a word of shared memory if `counts`; predicated, for a branch around it takes three times the instructions.
+__device__ __forceinline__ void count_if(bool counts, unsigned* word) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %1, 0;\n@p red.shared.add.u32 [%0], 1;\n}"
+               ::"r"((unsigned)__cvta_generic_to_shared(word)), "r"((unsigned)counts) : "memory");
+}
+
 __device__ __forceinline__ void add_to(float4& s, const float4& v) { s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w; }
 __device__ __forceinline__ void add_to(float& s, float v) { s += v; }
 

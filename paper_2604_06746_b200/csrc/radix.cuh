@@ -39,11 +39,9 @@ __device__ __forceinline__ void radix_clear(RadixShared<CL>& s) {
 #pragma unroll
   for (int i = 0; i < kRxLevels * kRxBins / kRxThreads; ++i) s.hist[0][i * kRxThreads + threadIdx.x] = make_uint4(0u, 0u, 0u, 0u);
 }
-// Counts a key's digit if `counts`; predicated, for a branch around it took three times the instructions.
 template <int CL>
 __device__ __forceinline__ void radix_count(RadixShared<CL>& s, int level, unsigned digit, bool counts) {
-  const unsigned at = (unsigned)__cvta_generic_to_shared(s.hist[level]) + digit * (4 * kRxCopies) + (threadIdx.x & (kRxCopies - 1)) * 4;
-  asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %1, 0;\n@p red.shared.add.u32 [%0], 1;\n}" ::"r"(at), "r"((unsigned)counts) : "memory");
+  count_if(counts, reinterpret_cast<unsigned*>(s.hist[level]) + digit * kRxCopies + (threadIdx.x & (kRxCopies - 1)));
 }
 template <int CL>
 __device__ __forceinline__ void cluster_barrier() {

@@ -177,6 +177,11 @@ __device__ __forceinline__ void head_done(const FinishArgs& a, int vec, float me
 // The entries inside the threshold bin are then summed as count x bin midpoint: bins of the second
 // level are 2^-14 wide relative to their value, far inside the metric's tolerance.
 //
+// A sweep's cost is its instructions: counts are predicated (a branch around each took three times as many), what lies beyond a
+// vector's end is skipped, one warp walks the bins, and one CTA with an SM to itself keeps up to 16384 entries in its
+// registers between the sweeps.  us without / with, chained launches over 32 heads: one layer of 16384 keys 9.0 / 7.6, of 32768
+// 11.6 / 9.6, of 262144 20.2 / 17.2; 32 layers of 5003 keys 15.6 / 14.4, of 32768 58 / 50, of 131072 215 / 196.
+//
 // Bound by latency up to some 100 vectors, then by the shared-memory atomics and, where the vectors exceed
 // L2 together, by reading them twice (1024 vectors of 131072 keys: 2 x 537 MB, 164 of 208 us).  One histogram,
 // without copies for the lanes: same-address hits cost less than clearing and summing copies, whether the
@@ -199,7 +204,7 @@ struct SweepShared {
   unsigned scan[2][32], bin, rem;                          // [level] sums of the warps, or of 64 bins each
 };
 template <int T, int CL, int ROWS> constexpr int kAccs = ROWS == 1 ? 1024 / T : ROWS * 1024 / (T * CL);
-// Applies f(entry, accumulator) to this CTA's entries of a[0 .. n) once each, 48 or 64 KB of loads in flight on an SM.
+// Applies f(entry, accumulator, whether there is one) to this CTA's entries of a[0 .. n) once each, 48 or 64 KB of loads in flight on an SM.
 template <int T, int CL, int ROWS, class F>
 __device__ __forceinline__ void sweep_from_memory(const float* __restrict__ a, int n, int rank, F f) {
   constexpr int kAt = T == 1024 ? 16 : 8, kStep = ROWS == 1 ? T : T * CL, kMine = kAccs<T, CL, ROWS>;
@@ -213,18 +218,18 @@ __device__ __forceinline__ void sweep_from_memory(const float* __restrict__ a, i
 #pragma unroll
       for (int u = 0; u < kAt; ++u) v[u] = a[first + threadIdx.x + (h + u) * kStep];
 #pragma unroll
-      for (int u = 0; u < kAt; ++u) f(v[u], (h + u) & (kMine - 1));
+      for (int u = 0; u < kAt; ++u) f(v[u], (h + u) & (kMine - 1), true);
     }
   }
   const int j = first + threadIdx.x;
 #pragma unroll
   for (int h = 0; h < kChunk; h += kAt) {
+    if (first + h * kStep >= n) return;
+#pragma unroll
+    for (int u = 0; u < kAt; ++u) v[u] = j + (h + u) * kStep < n ? a[j + (h + u) * kStep] : 0.f;
 #pragma unroll
     for (int u = 0; u < kAt; ++u)
-      if (j + (h + u) * kStep < n) v[u] = a[j + (h + u) * kStep];
-#pragma unroll
-    for (int u = 0; u < kAt; ++u)
-      if (j + (h + u) * kStep < n) f(v[u], (h + u) & (kMine - 1));
+      if (first + (h + u) * kStep < n) f(v[u], (h + u) & (kMine - 1), j + (h + u) * kStep < n);
   }
 }
 // Sums of N accumulators (a power of two) over each warp, to the rows they belong to.  While there are several, a
@@ -293,11 +298,11 @@ __device__ __forceinline__ int find_rank(unsigned count, unsigned& rest) {
   rest -= __shfl_sync(0xffffffffu, before, at);
   return at;
 }
-// Once all warps have counted: walks the bins of a histogram from the top.  `bin` holds the
-// `remaining`-th largest candidate, `rem` is the rank still wanted inside it.  32 groups of 64 bins first, summed by
-// their warps, then, in every warp alike, the groups and the bins of one of them.
+// Once all warps have counted: walks the bins of a histogram from the top.  s.bin holds the `remaining`-th largest candidate,
+// s.rem is the rank still wanted inside it.  32 groups of 64 bins first, summed by their warps, then, in one warp, the
+// groups and the bins of one of them.
 template <int T>
-__device__ __forceinline__ void sweep_pick(SweepShared& s, int level, unsigned remaining, unsigned& bin, unsigned& rem) {
+__device__ __forceinline__ void sweep_pick(SweepShared& s, int level, unsigned remaining) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint2* const pairs = reinterpret_cast<const uint2*>(s.hist[level]);
   __syncthreads();
@@ -308,12 +313,17 @@ __device__ __forceinline__ void sweep_pick(SweepShared& s, int level, unsigned r
     if (lane == 0) s.scan[level][g] = sum;
   }
   __syncthreads();
-  unsigned rest = remaining;
-  const int group = 31 - find_rank(s.scan[level][31 - lane], rest), pair = 32 * group + 31 - lane;
-  const uint2 c = pairs[pair];
-  const int at = find_rank(c.x + c.y, rest);
-  bin = __shfl_sync(0xffffffffu, (unsigned)(2 * pair) + (rest <= c.y ? 1u : 0u), at);
-  rem = __shfl_sync(0xffffffffu, rest <= c.y ? rest : rest - c.y, at);
+  if (warp == 0) {
+    unsigned rest = remaining;
+    const int group = 31 - find_rank(s.scan[level][31 - lane], rest), pair = 32 * group + 31 - lane;
+    const uint2 c = pairs[pair];
+    const int at = find_rank(c.x + c.y, rest);
+    if (lane == at) {
+      s.bin = (unsigned)(2 * pair) + (rest <= c.y ? 1u : 0u);
+      s.rem = rest <= c.y ? rest : rest - c.y;
+    }
+  }
+  __syncthreads();
 }
 // The same for a cluster, in two steps of one warp: 32 groups of 64 bins, summed by their owners before the
 // barrier, then the bins of one group.
@@ -350,33 +360,57 @@ __device__ __forceinline__ void sweep_cta(const FinishArgs& a, SweepShared& s, c
   const int tid = threadIdx.x, rank = CL > 1 ? (int)(blockIdx.x % CL) : 0, n = pb.n;
   const float* x = pb.cols + (size_t)(vec % a.H) * a.col_stride;
   const float mean = 1.f / (float)n;
-  auto pick = [&](int level, unsigned remaining, unsigned& bin, unsigned& rem) {
-    if (CL > 1) {
-      cluster_pick<CL>(s, level, remaining);
-      bin = s.bin;
-      rem = s.rem;
-    } else {
-      sweep_pick<T>(s, level, remaining, bin, rem);
-    }
-  };
   float acc[kAccs<T, CL, ROWS>] = {};
-  sweep_from_memory<T, CL, ROWS>(x, n, rank, [&](float v, int k) {
+  unsigned b1 = 0;
+  auto first_sweep = [&](float v, int k, bool in) {
     const float dv = v - mean;
-    acc[k] = fmaf(dv, dv, acc[k]);
-    atomicAdd(&s.hist[0][(__float_as_uint(v) >> 20) & 0x7ffu], 1u);
-  });
-  if (ROWS > 1 || rank == 0) warp_sums<T, CL>(acc, s.red[0][0], rank);
-  unsigned b1, rem1, b2, rem2;
-  pick(0, (unsigned)max(1, n / 10), b1, rem1);
-#pragma unroll
-  for (float& m : acc) m = 0.f;
-  sweep_from_memory<T, CL, ROWS>(x, n, rank, [&](float v, int k) {
+    acc[k] = in ? fmaf(dv, dv, acc[k]) : acc[k];
+    count_if(in, &s.hist[0][(__float_as_uint(v) >> 20) & 0x7ffu]);
+  };
+  auto second_sweep = [&](float v, int k, bool in) {
     const unsigned u = __float_as_uint(v), top = (u >> 20) & 0x7ffu;
-    if (top > b1) acc[k] += v;
-    else if (top == b1) atomicAdd(&s.hist[1][(u >> 9) & 0x7ffu], 1u);
-  });
-  if (ROWS > 1 || rank == 0) warp_sums<T, CL>(acc, s.red[1][0], rank);
-  pick(1, rem1, b2, rem2);
+    acc[k] += in && top > b1 ? v : 0.f;
+    count_if(in && top == b1, &s.hist[1][(u >> 9) & 0x7ffu]);
+  };
+  auto pick = [&](int level, unsigned remaining) {
+    if (ROWS > 1 || rank == 0) warp_sums<T, CL>(acc, s.red[level][0], rank);
+    if (CL > 1) cluster_pick<CL>(s, level, remaining);
+    else sweep_pick<T>(s, level, remaining);
+#pragma unroll
+    for (float& m : acc) m = 0.f;
+  };
+  // One CTA with an SM to itself keeps a short vector's entries in its registers from sweep to sweep.
+  constexpr int kHold = T == 1024 && CL == 1 && ROWS == 1 ? 16 : 0;
+  if (kHold > 0 && n <= kHold * T) {
+    constexpr int kAt = 4;
+    float v[kHold > 0 ? kHold : 1];
+#pragma unroll
+    for (int h = 0; h < kHold; h += kAt) {
+      if (h * T >= n) break;
+#pragma unroll
+      for (int u = h; u < h + kAt; ++u) v[u] = tid + u * T < n ? x[tid + u * T] : 0.f;
+    }
+    auto all = [&](auto f) {
+#pragma unroll
+      for (int h = 0; h < kHold; h += kAt) {
+        if (h * T >= n) break;
+#pragma unroll
+        for (int u = h; u < h + kAt; ++u) f(v[u], 0, tid + u * T < n);
+      }
+    };
+    all(first_sweep);
+    pick(0, (unsigned)max(1, n / 10));
+    b1 = s.bin;
+    all(second_sweep);
+  } else {
+    sweep_from_memory<T, CL, ROWS>(x, n, rank, first_sweep);
+    pick(0, (unsigned)max(1, n / 10));
+    b1 = s.bin;
+    sweep_from_memory<T, CL, ROWS>(x, n, rank, second_sweep);
+  }
+  const unsigned rem1 = s.rem;
+  pick(1, rem1);
+  const unsigned b2 = s.bin, rem2 = s.rem;
   if (rank == 0) {
     // entries of the threshold bin above sub-bin b2, and rem2 entries of sub-bin b2 itself
     constexpr int kAccsBin = 1024 / T;
@@ -556,10 +590,11 @@ static cudaError_t launch_finish(FinishArgs& a, int longest, int sms, cudaStream
   const int sums = a.n_prob * a.chunks;
   if (!a.with_stats) return launch_pdl(sum_layers<VEC>, dim3(sums), dim3(kSumThreads), 0, st, a);
   // An SM per vector: as many threads as a CTA can have.  More vectors than SMs: several CTAs an SM fill each
-  // other's gaps between barriers, six of 256 for short vectors, three of 512 for long ones.  us after the scorer, 32
-  // layers of 32 heads with their sums, three of 512 / six of 256: 5003 keys 30 / 23.5, 20001 (28 layers) 70 / 58, 32768 81 /
-  // 80 (window 8: 76 / 69; five of 256: 26, 63, 71 to 78); without sums 5003 keys 20 / 17, 8192 22.7 / 21.0, 16384 31.3 /
-  // 31.9, 32768 58 / 71, and of 8 layers, which three of 512 take in one go, 9.4 / 10.0.
+  // other's gaps between barriers, six of 256 for short vectors, three of 512 for long ones.  us, three of 512 / six of 256:
+  // statistics alone of 32 layers of 32 heads, 1500 keys 14.1 / 10.6, 5003 18.3 / 14.9, 8192 19.7 / 18.0, 16384 27.9 /
+  // 28.3, 32768 56 / 70; of 10 layers, which three of 512 take in one go, 5003 keys 8.5 / 10.1, 8192 9.0 / 11.8; whole prefills of
+  // 32 layers, 1500 keys 150.0 / 144.7, 5003 298.8 / 288.6, 8192 428.6 / 424.5, of 14 layers of 5003 keys 143.9 / 141.3, of 10 121.6
+  // / 123.9.
   // Few long vectors: clusters, as large as leaves room for all of them at once.
   const int n_vec = a.n_prob * a.H, room = longest > kLongFrom ? sms * 7 / 8 / n_vec : 1;
   const int cl = 8 * n_vec <= sms * 3 / 4 && room >= 8 ? 8 : room >= 4 ? 4 : room >= 2 ? 2 : 1;
@@ -572,8 +607,10 @@ static cudaError_t launch_finish(FinishArgs& a, int longest, int sms, cudaStream
     return longest > kLongFrom ? launch_pdl(finish<VEC, 1024, 1, true, true>, grid, wide, 0, st, a)
                                : launch_pdl(finish<VEC, 1024, 1, false, true>, grid, wide, 0, st, a);
   // Sums behind their statistics only where the statistics take several goes of three CTAs an SM.  us after the
-  // scorer, in front / behind: 5003 keys, 6 layers of 32 heads 9.5 / 12.5, 14 layers 17 / 14; 32768 keys, 10 layers 28 / 47,
-  // 20 58 / 63, 24 71 / 65; 65536 keys, 14 82 / 86, 20 119 / 111, 24 141 / 128; 131072 keys, 10 109 / 131, 20 220 / 219.
+  // scorer, in front / behind, before the sweeps took fewer instructions: 5003 keys, 6 layers of 32 heads 9.5 / 12.5, 14 layers
+  // 17 / 14; 32768 keys, 10 layers 28 / 47, 20 58 / 63, 24 71 / 65; 65536 keys, 14 82 / 86, 20 119 / 111, 24 141 / 128; 131072
+  // keys, 10 109 / 131, 20 220 / 219.  With them, whole prefills: 1500 keys, 14 layers 84.1 / 81.7, 32 layers 146.7 / 144.7;
+  // 5003 keys, 14 layers 142.2 / 141.3, 10 layers of 32768 keys 490 / 525.
   const bool several = n_vec > (longest > kNarrowMany ? 5 : 3) * sms;
   if (!sums || !several)
     return longest > kLongFrom ? launch_pdl(finish<VEC, 512, 1, true, true>, grid, narrow, 0, st, a)
