@@ -696,7 +696,7 @@ __global__ void __launch_bounds__(kResThreads, 1) tc_resident(const __grid_const
   }
   if (threadIdx.x == 0) fl->last = atomicAdd(p.ctl + kCtlExit, 1) == (int)gridDim.x - 1;
   __syncthreads();
-  if (fl->last) pass_tags_on(p.xch, p.ctl, tag0 - 1u + (unsigned)((n_prob * n_kv + teams - 1) / teams));
+  if (fl->last) pass_tags_on(p.xch, p.ctl, tag0 - 1u + (unsigned)((n_prob * n_kv + teams - 1) / teams), (int)threadIdx.x, (int)blockDim.x);
 }
 
 template <int D, int MAXP>

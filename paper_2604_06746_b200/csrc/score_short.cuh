@@ -9,8 +9,8 @@
 // twice as many CTAs fit the GPU a segment's row halves and tiles go to two of them.
 //
 // us per call with the sums over heads, general scorer / this one, 32 query heads, 8 KV heads, window 64: 1000 keys 20.5 /
-// 16.9, 1777 22.8 / 17.3, 2304 (the last by halves) 24.3 / 18.7, 3000 25.9 / 21.5, 4608 (the last with one pair a segment) 25.7 /
-// 21.1, 5003 31.5 / 27.0, 9216 30.0 / 26.3.  Bound by latency: at 4096 keys the first copy goes out 2 us after the kernel
+// 16.5, 2304 (the last by halves) 24.0 / 18.2, 3000 25.9 / 20.9, 4608 (the last with one pair a segment) 25.7 / 20.8, 5003
+// 31.0 / 26.2, 9216 30.0 / 25.8.  Bound by latency: at 4096 keys the first copy goes out 2 us after the kernel
 // before, its products are there 1.5 us later, then 2.7 us of exponentials, 2.5 us until the last CTA's partials are
 // merged, 3 us of exponentials, and the way to the next kernel.
 //
@@ -60,7 +60,7 @@ struct ShortSmem {
   struct Task { int pass, task, fresh; };                  // pass 0: none left; fresh: its tiles come anew
   struct Work { int unit, g, head, row0, rows, seg, lo, hi, half_lo, half_hi, t_lo, t_hi; };   // head: the unit's first
   struct Flags {
-    int abort, mma_in_flight, last;
+    int abort, mma_in_flight;
     uint32_t tmem;
     unsigned tag;                      // of this launch's words
     Task ring[2];
@@ -328,9 +328,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
   } else if (warp == 2) {
     // ---------------- entropies, beside the second pass: a unit's rows are dealt out to its segments' CTAs ----------------
     typename L::Task t;
+    unsigned n_ext = 0;
     for (int n = 0; next_task(n, t); ++n) {
       const typename L::Work w = flags->work[t.task];
-      if (t.pass != 2 || (p.split && w.half_lo != 0)) continue;
+      if (t.pass != 2) continue;
+      n_ext += w.t_lo < w.t_hi;
+      if (p.split && w.half_lo != 0) continue;
       const unsigned tag = flags->tag;
       long long t0 = 0;
       for (int r = w.seg * R / p.n_seg + lane; r < (w.seg + 1) * R / p.n_seg; r += 32) {
@@ -348,6 +351,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
         p.row_ent[(size_t)w.unit * R + r] = ent;
       }
     }
+    // No task is left and, once the last log-sum-exps are there, no word is read any more: the CTA signs off beside its last
+    // exponentials (by all of its warps after them: 0.4 us later).  The last one leaves the counters as it found them, and
+    // the tags one further.
+    int last = 0;
+    if (lane == 0) {
+      if (n_ext > 0) mbar_wait(bar(L::kExtFull), (n_ext - 1u) & 1u, abort_flag);
+      last = atomicAdd(p.ctl + kCtlExit, 1) == (int)gridDim.x - 1;
+      if (last) p.ctl[kCtlTicket] = 0;
+    }
+    if (__shfl_sync(0xffffffffu, last, 0)) pass_tags_on(p.xch, p.ctl, flags->tag, lane, 32);
   } else if (warp >= kHelperWarps) {
     // ---------------- compute warps ----------------
     const int quarter = warp & 3;            // tensor-memory lane quarter this warp may read
@@ -535,13 +548,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
   if (warp == 1 && !fl->mma_in_flight) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
-  }
-  // the last CTA leaves the counters as it found them, and the tags one further
-  if (threadIdx.x == 0) fl->last = atomicAdd(p.ctl + kCtlExit, 1) == (int)gridDim.x - 1;
-  __syncthreads();
-  if (fl->last) {
-    if (threadIdx.x == 0) p.ctl[kCtlTicket] = 0;
-    pass_tags_on(p.xch, p.ctl, flags->tag);
   }
 }
 

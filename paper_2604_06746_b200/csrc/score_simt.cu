@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kSmThreads, 3) simt_once(const __grid_constant
   }
   if (threadIdx.x == 0) last = atomicAdd(a.ctl + kCtlExit, 1) == (int)(gridDim.x * gridDim.y * gridDim.z) - 1;
   __syncthreads();
-  if (last) pass_tags_on(a.xch, a.ctl, tag);
+  if (last) pass_tags_on(a.xch, a.ctl, tag, (int)threadIdx.x, (int)blockDim.x);
 }
 
 template <typename T, int D>

@@ -27,13 +27,13 @@ __device__ __forceinline__ unsigned long long get_word_acquire(const unsigned lo
   asm volatile("ld.acquire.gpu.global.b64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
   return w;
 }
-// What the last CTA of a launch does (all of its threads call): the tags move on to `next`, or, long before they wrap,
-// start over with clean words.
-__device__ __forceinline__ void pass_tags_on(unsigned long long* xch, int* ctl, unsigned next) {
+// What the last CTA of a launch does, `threads` of its threads: the tags move on to `next`, or, long before they wrap, start
+// over with clean words.
+__device__ __forceinline__ void pass_tags_on(unsigned long long* xch, int* ctl, unsigned next, int thread, int threads) {
   const bool over = next > 0x7f000000u;
   if (over)
-    for (size_t i = threadIdx.x; i < (size_t)kXchWords; i += blockDim.x) xch[i] = 0;
-  if (threadIdx.x == 0) {
+    for (size_t i = thread; i < (size_t)kXchWords; i += threads) xch[i] = 0;
+  if (thread == 0) {
     ctl[kCtlTag] = over ? 0 : (int)next;
     ctl[kCtlExit] = 0;
   }
