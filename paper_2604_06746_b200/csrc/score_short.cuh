@@ -428,13 +428,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
           const int it = n_half == 2 ? k >> 1 : k, hf = n_half == 2 ? k & 1 : w.half_lo;
           const int jb = (w.lo + 2 * it) * kKeyTile + sub * 64;
           const bool warp_active = hf * 128 + quarter * 32 < w.rows;
-          if (warp_active) {
-            tmem_ld(acc_addr() + sub * 64, v);
-            chunk(rs[0], jb, it == 0, hf);
-            tmem_ld(acc_addr() + sub * 64 + 32, v);
+          // (one copy of the body: with two, 2304 keys with all statistics take 17.8 us instead of 16.9, 4096 20.4 instead of 19.9)
+#pragma unroll 1
+          for (int c = 0; c < 2; ++c) {
+            if (warp_active) tmem_ld(acc_addr() + sub * 64 + 32 * c, v);
+            if (c == 1) acc_release();
+            if (warp_active) chunk(rs[0], jb + 32 * c, it == 0 && c == 0, hf);
           }
-          acc_release();
-          if (warp_active) chunk(rs[0], jb + 32, false, hf);
           if (n_half == 2) {
             const RowStat o = rs[0];
             rs[0] = rs[1];

@@ -229,7 +229,8 @@ cudaError_t launch_problems(const Ctx& ctx, const ScoreCall& a, int first, int n
   p.row_ent = a.row_ent + (size_t)first * ctx.rows_pad;
   p.col_stride = a.col_stride;
   p.status = ctx.ws.status;
-  p.hurry = n == 1 || batch;
+  const long long pairs0 = (long long)l.units * ((p.prob[0].n_keys + 2 * kKeyTile - 1) / (2 * kKeyTile));
+  p.form = n == 1 || batch ? kHurry : pairs0 <= kBriefPairs ? kBrief : kAmong;
   const int grid = std::min(sms, tickets);
   return cfg.head_dim == 128 ? tc_launch_128(l.shape, p, grid, ctx.device, st) : tc_launch_64(l.shape, p, grid, ctx.device, st);
 }

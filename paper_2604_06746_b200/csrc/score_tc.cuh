@@ -64,6 +64,20 @@ constexpr float kMasked = -1.0e30f;    // exponent standing for -inf: 2^x flushe
 constexpr float kMaskedAcc = -3.0e38f; // the same for an accumulator, before the scaling by c2 >= 1e-30
 constexpr int kFullWeight = 20;        // weight of a full row block when key ranges are dealt out (see tc_deal)
 
+// What the kernel is compiled for.  kHurry: pass 2 has nothing to do but wait for pass 1 (one layer, a batch), so the compute
+// warps count their arrivals and merge the row statistics themselves, a thread per row, instead of leaving it to one helper
+// warp beside them (at 8192 keys 2 us instead of 6).  With layers to interleave the helpers' time is hidden and the compute
+// warps' is not (32 layers of 5003 keys: 317 us in a hurry, 300 without).  With both ways in one kernel 32 layers of 1500
+// keys took 117.7 us instead of 115.5, one layer of 9300 33.9 instead of 33.6.
+// kBrief: pass 2's arithmetic in one copy instead of two.  Short tasks alternate with pass 1 and are as long as it takes to fetch
+// them; long ones gain by a second load under way earlier.  us, two copies / one: window 64, 32 layers of 1500 keys 115.5 /
+// 109.6, of 5003 262 / 246, of 8192 387 / 370, 16 of 16384 366 / 356, of 24000 491 / 491, of 32768 657 / 657, 8 of 65536 656 /
+// 690; window 128, 28 query heads over 4 KV heads, 16 of 5000 278 / 267, 12 of 10000 372 / 355, 8 of 20000 398 / 408; a layer
+// by itself, 9300 keys 33.6 / 35.2, 131072 164 / 170.
+enum TcForm { kAmong = 0, kBrief, kHurry };
+// (KV group, row block, pair of key tiles) triples of a layer up to which its tasks count as short.
+constexpr int kBriefPairs = 768;
+
 // Layout classes of the kernel (template argument).
 enum TcShape { kWide16 = 0, kWide32, kWide64, kWide128, kWide256, kNarrow32, kNarrow64 };
 
@@ -94,11 +108,7 @@ struct alignas(64) TcParams {
   float* row_ent;                      // [problem][unit][256] entropy of a row, nats (0: no row)
   long long col_stride;
   int* status;
-  // Pass 2 has nothing to do but wait for pass 1 (one layer, a batch): the compute warps count their arrivals
-  // and merge the row statistics themselves, a thread per row, instead of leaving it to one helper
-  // warp beside them (at 8192 keys 2 us instead of 6).  With layers to interleave the helpers' time is
-  // hidden and the compute warps' is not (32 layers of 5003 keys: 317 us in a hurry, 300 without).
-  int hurry;
+  int form;                            // TcForm
 };
 constexpr int kCtlTicket = 0, kCtlArrive = 64, kCtlReady = 64 + kMaxBatch * kQueueUnits;
 static_assert(kCtlInts == 64 + 2 * kMaxBatch * kQueueUnits, "control block");
@@ -577,10 +587,11 @@ __device__ __forceinline__ float sum_exp(const float* v, uint64_t c22, float v_m
   return a + b;
 }
 
-template <int D, int SH, int MAXP>
+template <int D, int SH, int MAXP, int FORM>
 __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant__ TcParams<MAXP> p) {
   using L = Smem<D, SH>;
   using S = Shape<SH>;
+  constexpr bool HURRY = FORM == kHurry;
   constexpr int R = S::kRows, kQHalves = S::kQHalves;
   extern __shared__ unsigned char smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
@@ -599,7 +610,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     for (int s = 0; s < kStages; ++s) { mbar_init(bar(kBarFull + s), 1); mbar_init(bar(kBarEmpty + s), 1); }
     for (int s = 0; s < kTaskRing; ++s) { mbar_init(bar(kBarTaskFull + s), 1); mbar_init(bar(kBarTaskEmpty + s), kTaskConsumers); }
     for (int b = kBarQFull; b < kBarFold; ++b)
-      mbar_init(bar(b), p.hurry && b >= kBarExtFull && b < kBarExtEmpty ? R / 32 : 1);
+      mbar_init(bar(b), HURRY && b >= kBarExtFull && b < kBarExtEmpty ? R / 32 : 1);
     for (int b = 0; b < 4; ++b) mbar_init(bar(kBarFold + b), 4);
     mbar_init(bar(kBarPartFull), S::kFoldWarps);
     mbar_init(bar(kBarPartEmpty), 1);
@@ -731,7 +742,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         if (t.pass == 0) break;
         const TcProblem& pb = p.prob[t.prob];
         const int n_tiles = (pb.n_keys + kKeyTile - 1) / kKeyTile;
-        const bool plain = p.n_rb > 1 && !p.hurry && pb.n_keys >= kL2PlainFrom;
+        const bool plain = p.n_rb > 1 && !HURRY && pb.n_keys >= kL2PlainFrom;
         const int keep_from = t.pass == 1 && !plain ? n_tiles - (n_tiles * kL2KeepPct) / 100 : n_tiles;
         bool ok = true;
         for (int it = 0; it < items_of(t) && ok; ++it) {
@@ -883,7 +894,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     int n_ext = 0;
     TcTask t;
     for (int n = 0; next_task(n, t); ++n) {
-      if (p.hurry || t.pass != 2 || t.lo == t.hi) continue;
+      if (HURRY || t.pass != 2 || t.lo == t.hi) continue;
       int ok = 1;
       if (lane == 0) {
         // the MMAs of the last task but one have read the operand; this unit's statistics are merged
@@ -913,7 +924,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
     int n_p1 = 0;
     TcTask t;
     for (int n = 0; next_task(n, t); ++n) {
-      if (p.hurry || t.pass != 1) continue;
+      if (HURRY || t.pass != 1) continue;
       int last = 0, ok = 1;
       if (lane == 0) {
         // the compute warps have stored the task's statistics
@@ -981,7 +992,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
       __syncwarp();
       bool ok = true;
       if (lane == 0) {
-        if (p.hurry) {                                     // each storing warp counts for itself
+        if (HURRY) {                                     // each storing warp counts for itself
           __threadfence();
           atomicAdd(p.ctl + kCtlArrive + t.prob * kQueueUnits + t.unit, 1);
         } else {                                           // the helper has seen the previous task's
@@ -1231,7 +1242,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         }
       } else {
         // Pass 2: this thread owns key (tile * 128 + quarter * 32 + lane); x = c2 * accumulator.
-        if (p.hurry && t.hi > t.lo && !merge_now(t)) break;
+        if (HURRY && t.hi > t.lo && !merge_now(t)) break;
         const float v_min = t.v_min, inv_w = 1.0f / (float)p.window;
         // Columns (rows of the block) this warp sums: a quarter of them on every tile, or, where a
         // head spans more, the head's rows on every second or fourth tile, so that a head's column
@@ -1244,6 +1255,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
         const int my_turn = kW == 128 && !S::kNarrow ? sub >> 1 : sub;
         const bool warp_active = col0 < t.rows;
         const int h0 = (t.row0 + col0) >> p.w_shift, h_end = t.group;   // heads within the KV group
+        constexpr int kCopies = FORM == kBrief ? 1 : 2;
         for (int i = 0; i < t.hi - t.lo; ++i) {
           if (!acc_full()) { live = false; break; }
           const int tile = t.hi - 1 - i;
@@ -1254,7 +1266,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
           const uint32_t taddr = acc_addr() + col0;
           float tot = 0.f;
           int head = h0;
-#pragma unroll 2
+#pragma unroll kCopies
           for (int c = 0; c < kCols; c += 32) {
             float v[32] = {};
             if (mine) tmem_ld(taddr + c, v);
@@ -1309,8 +1321,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_score(const __grid_constant_
 
 template <int D, int SH, int MAXP>
 cudaError_t tc_launch(const TcParams<MAXP>& p, int grid, int device, cudaStream_t st) {
-  auto kern = tc_score<D, SH, MAXP>;
-  static std::atomic<unsigned long long> ready{0};        // devices whose shared-memory limit has been raised
+  // (one problem is in a hurry)
+  const auto kern = MAXP == 1 || p.form == kHurry ? tc_score<D, SH, MAXP, kHurry>
+                    : p.form == kBrief            ? tc_score<D, SH, MAXP, MAXP == 1 ? kHurry : kBrief>
+                                                  : tc_score<D, SH, MAXP, MAXP == 1 ? kHurry : kAmong>;
+  static std::atomic<unsigned long long> ready_for[3];    // devices whose shared-memory limit has been raised
+  std::atomic<unsigned long long>& ready = ready_for[p.form];
   const unsigned long long bit = 1ull << (device & 63);
   if (!(ready.load(std::memory_order_acquire) & bit)) {
     const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<D, SH>::kAlloc);
