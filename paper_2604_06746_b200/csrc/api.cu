@@ -518,6 +518,18 @@ structkv_status structkv_pivot_select(structkv_ctx* ctx, const float* s_hist, lo
   return s == STRUCTKV_OK ? await_pivot(ctx->c, n_layers, pivot_out, t_out, st) : s;
 }
 
+static bool compact_layers_args_ok(const void* const* srcs, int n_layers, long long slab_stride_bytes, long long row_stride_bytes,
+                                   int row_bytes, int n_slabs, int n_rows_src, const int* idx, long long idx_layer_stride, int n_idx,
+                                   const void* dst, long long dst_layer_stride_bytes) {
+  if (!srcs || !dst || !idx || n_layers < 1 || n_layers > kMaxGatherLayers) return false;
+  if (row_bytes < 1 || n_slabs < 0 || n_rows_src < 1 || n_idx < 0) return false;
+  if (row_stride_bytes < row_bytes || slab_stride_bytes < 0 || idx_layer_stride < n_idx) return false;
+  if (dst_layer_stride_bytes < (long long)n_slabs * n_idx * row_bytes) return false;
+  for (int l = 0; l < n_layers; ++l)
+    if (!srcs[l]) return false;
+  return true;
+}
+
 structkv_status structkv_prefill(structkv_ctx* ctx, const structkv_prefill_args* p, int* pivot_out, float* t_out,
                                  void* stream) {
   if (!ctx || !p || !p->c_out || p->n_layers < 1 || p->n_layers > kMaxStatLayers ||
@@ -537,16 +549,34 @@ structkv_status structkv_prefill(structkv_ctx* ctx, const structkv_prefill_args*
                 : structkv_pivot_select(ctx, p->s_out, p->s_layer_stride, p->n_layers, p->n_keys, p->metrics, p->weights,
                                         p->l_limit, p->lambda, p->window, p->kv_budget, p->i_kv, p->struct_budget, p->c_star,
                                         p->i_struct, pivot_out, t_out, stream);
-  if (s == STRUCTKV_OK && p->kv_srcs)
-    s = structkv_compact_layers(ctx, p->kv_srcs, p->n_layers, p->kv_slab_stride_bytes, p->kv_row_stride_bytes, p->kv_row_bytes,
-                                p->kv_slabs, p->kv_rows, p->i_kv, p->kv_budget, p->kv_budget, p->kv_dst,
-                                p->kv_dst_layer_stride_bytes, stream);
-  // hidden states and 4-byte positions share a launch
+  // hidden states and 4-byte positions share a launch, with the layers' K and V where these are copied in 16-byte units
   const bool together = p->hidden && p->positions && p->hidden_dst && p->positions_dst && p->hidden_row_bytes >= 1 &&
                         p->hidden_row_stride_bytes >= p->hidden_row_bytes && p->position_row_bytes == 4 &&
                         p->position_row_stride_bytes >= 4 && p->position_row_stride_bytes % 4 == 0 &&
                         (uintptr_t)p->positions % 4 == 0 && (uintptr_t)p->positions_dst % 4 == 0;
-  if (s == STRUCTKV_OK && together) {
+  bool all_together = false;
+  if (s == STRUCTKV_OK && p->kv_srcs) {
+    s = compact_layers_args_ok(p->kv_srcs, p->n_layers, p->kv_slab_stride_bytes, p->kv_row_stride_bytes, p->kv_row_bytes, p->kv_slabs,
+                               p->kv_rows, p->i_kv, p->kv_budget, p->kv_budget, p->kv_dst, p->kv_dst_layer_stride_bytes)
+            ? STRUCTKV_OK
+            : STRUCTKV_ERR_INVALID_ARG;
+    if (s == STRUCTKV_OK && together) {
+      const CompactRows kv = {nullptr, p->kv_slab_stride_bytes, p->kv_row_stride_bytes, p->kv_row_bytes, p->kv_slabs, p->kv_rows,
+                              p->i_kv, p->kv_budget, p->kv_dst};
+      const CompactRows other = {p->hidden, 0, p->hidden_row_stride_bytes, p->hidden_row_bytes, 1, p->n_keys, p->i_struct,
+                                 p->struct_budget, p->hidden_dst};
+      const CompactWords words = {p->positions, p->position_row_stride_bytes, p->positions_dst};
+      cudaError_t e = cudaSuccess;
+      all_together = launch_compact_prefill(kv, p->kv_srcs, p->n_layers, p->kv_budget, p->kv_dst_layer_stride_bytes, other, words,
+                                            ctx->c.ws.status, ctx->c.sm_count, st, &e);
+      if (e != cudaSuccess) s = STRUCTKV_ERR_CUDA;
+    }
+    if (s == STRUCTKV_OK && !all_together)
+      s = structkv_compact_layers(ctx, p->kv_srcs, p->n_layers, p->kv_slab_stride_bytes, p->kv_row_stride_bytes, p->kv_row_bytes,
+                                  p->kv_slabs, p->kv_rows, p->i_kv, p->kv_budget, p->kv_budget, p->kv_dst,
+                                  p->kv_dst_layer_stride_bytes, stream);
+  }
+  if (s == STRUCTKV_OK && together && !all_together) {
     const CompactWords words = {p->positions, p->position_row_stride_bytes, p->positions_dst};
     if (launch_compact(p->hidden, 0, p->hidden_row_stride_bytes, p->hidden_row_bytes, 1, p->n_keys, p->i_struct, 0,
                        p->struct_budget, p->hidden_dst, ctx->c.ws.status, ctx->c.sm_count, st, &words) != cudaSuccess)
@@ -583,13 +613,9 @@ structkv_status structkv_compact_layers(structkv_ctx* ctx, const void* const* sr
                                         long long slab_stride_bytes, long long row_stride_bytes, int row_bytes,
                                         int n_slabs, int n_rows_src, const int* idx, long long idx_layer_stride,
                                         int n_idx, void* dst, long long dst_layer_stride_bytes, void* stream) {
-  if (!ctx || !srcs || !dst || !idx) return STRUCTKV_ERR_INVALID_ARG;
-  if (n_layers < 1 || n_layers > kMaxGatherLayers) return STRUCTKV_ERR_INVALID_ARG;
-  if (row_bytes < 1 || n_slabs < 0 || n_rows_src < 1 || n_idx < 0) return STRUCTKV_ERR_INVALID_ARG;
-  if (row_stride_bytes < row_bytes || slab_stride_bytes < 0 || idx_layer_stride < n_idx) return STRUCTKV_ERR_INVALID_ARG;
-  if (dst_layer_stride_bytes < (long long)n_slabs * n_idx * row_bytes) return STRUCTKV_ERR_INVALID_ARG;
-  for (int l = 0; l < n_layers; ++l)
-    if (!srcs[l]) return STRUCTKV_ERR_INVALID_ARG;
+  if (!ctx || !compact_layers_args_ok(srcs, n_layers, slab_stride_bytes, row_stride_bytes, row_bytes, n_slabs, n_rows_src, idx,
+                                      idx_layer_stride, n_idx, dst, dst_layer_stride_bytes))
+    return STRUCTKV_ERR_INVALID_ARG;
   const Ctx& c = ctx->c;
   return launch_compact_layers(srcs, n_layers, slab_stride_bytes, row_stride_bytes, row_bytes, n_slabs, n_rows_src,
                                idx, idx_layer_stride, n_idx, dst, dst_layer_stride_bytes, c.ws.status, c.sm_count,

@@ -158,6 +158,20 @@ cudaError_t launch_compact_layers(const void* const* srcs, int n_layers, long lo
                                   int row_bytes, int n_slabs, int n_rows_src, const int* idx,
                                   long long idx_layer_stride, int n_idx, void* dst, long long dst_layer_stride,
                                   int* status, int sm_count, cudaStream_t st);
+// Rows of n_slabs slabs by one list.
+struct CompactRows {
+  const void* src;
+  long long slab_stride, row_stride;
+  int row_bytes, n_slabs, n_rows_src;
+  const int* idx;
+  int n_idx;
+  void* dst;
+};
+// A gather of several layers (sources srcs), one of a single slab and the words that go with it in one launch.  False: not in
+// that form (16-byte units, one launch each).
+bool launch_compact_prefill(const CompactRows& kv, const void* const* srcs, int n_layers, long long idx_layer_stride,
+                            long long dst_layer_stride, const CompactRows& other, const CompactWords& words, int* status, int sm_count,
+                            cudaStream_t st, cudaError_t* e);
 cudaError_t launch_group_saliency(const float* head_cols, long long col_stride, int n_heads, int group, int n,
                                   float* out, cudaStream_t st);
 

@@ -38,7 +38,7 @@ __device__ __forceinline__ unsigned operator/(unsigned u, const Divisor& d) {
   return d.mul == 0 ? u : __umulhi(u, d.mul) >> d.shift;
 }
 
-// One list's rows out of one slab after the other: blocks 0 .. blocks - 1 of blockIdx.x, every gridDim.y-th slab.  A block
+// One list's rows out of one slab after the other: block `block` of `blocks`, every `slab_step`-th slab from `slab` on.  A block
 // takes kCpUnroll * kCpThreads consecutive units.
 struct Gather {
   long long slab_stride, row_stride, idx_slab_stride;
@@ -48,13 +48,14 @@ struct Gather {
   int n_slabs, n_rows_src;
 };
 template <typename V>
-__device__ __forceinline__ void gather_blocks(const Gather& g, unsigned blocks, const char* __restrict__ src,
-                                              const int* __restrict__ idx, char* __restrict__ dst, int* __restrict__ status) {
-  for (int s = blockIdx.y; s < g.n_slabs; s += gridDim.y) {
+__device__ __forceinline__ void gather_blocks(const Gather& g, unsigned block, unsigned blocks, int slab, int slab_step,
+                                              const char* __restrict__ src, const int* __restrict__ idx, char* __restrict__ dst,
+                                              int* __restrict__ status) {
+  for (int s = slab; s < g.n_slabs; s += slab_step) {
     const char* const from = src + s * g.slab_stride;
     const int* const list = idx + s * g.idx_slab_stride;   // stride 0: one list for every slab
     V* const to = reinterpret_cast<V*>(dst) + s * g.slab_units;
-    for (unsigned u0 = blockIdx.x * (kCpThreads * kCpUnroll) + threadIdx.x; u0 < g.units; u0 += blocks * (kCpThreads * kCpUnroll)) {
+    for (unsigned u0 = block * (kCpThreads * kCpUnroll) + threadIdx.x; u0 < g.units; u0 += blocks * (kCpThreads * kCpUnroll)) {
       V val[kCpUnroll];
       int j[kCpUnroll];
 #pragma unroll
@@ -83,26 +84,27 @@ gather_rows(const Gather g, const char* __restrict__ src, const int* __restrict_
             int* __restrict__ status) {
   pdl_trigger();
   pdl_wait();
-  gather_blocks<V>(g, gridDim.x, src, idx, dst, status);
+  gather_blocks<V>(g, blockIdx.x, gridDim.x, blockIdx.y, gridDim.y, src, idx, dst, status);
 }
-// The last `words` blocks gather one word per row of a second source by the same list (a launch of its own for
-// 4 bytes a row took 2 to 3 us after the gather it follows: the smallest whole prefill 66.8 -> 65.0 us).
+// Block `block` of one word per row of a second source, by the same list.
+__device__ __forceinline__ void gather_words(const CompactWords& w, int block, const int* __restrict__ idx, int n_idx, int n_rows_src) {
+  const int r = block * kCpThreads + (int)threadIdx.x;
+  if (r >= n_idx) return;
+  const int j = __ldg(idx + r);
+  if (j >= 0 && j < n_rows_src)
+    reinterpret_cast<unsigned*>(w.dst)[r] = *reinterpret_cast<const unsigned*>((const char*)w.src + j * w.row_stride);
+}
+// The last `words` blocks do that (a launch of its own for 4 bytes a row took 2 to 3 us after the gather it follows: the
+// smallest whole prefill 66.8 -> 65.0 us).
 template <typename V>
 __global__ void __launch_bounds__(kCpThreads)
 gather_rows_words(const Gather g, const char* __restrict__ src, const int* __restrict__ idx, int n_idx,
                   char* __restrict__ dst, int* __restrict__ status, const CompactWords w, int words) {
   pdl_trigger();
   pdl_wait();
-  if ((int)blockIdx.x >= (int)gridDim.x - words) {
-    const int r = ((int)blockIdx.x - (int)gridDim.x + words) * kCpThreads + (int)threadIdx.x;
-    if (r < n_idx) {
-      const int j = __ldg(idx + r);
-      if (j >= 0 && j < g.n_rows_src)
-        reinterpret_cast<unsigned*>(w.dst)[r] = *reinterpret_cast<const unsigned*>((const char*)w.src + j * w.row_stride);
-    }
-    return;
-  }
-  gather_blocks<V>(g, gridDim.x - words, src, idx, dst, status);
+  const int rows = (int)gridDim.x - words;
+  if ((int)blockIdx.x >= rows) gather_words(w, (int)blockIdx.x - rows, idx, n_idx, g.n_rows_src);
+  else gather_blocks<V>(g, blockIdx.x, rows, blockIdx.y, gridDim.y, src, idx, dst, status);
 }
 
 // The same gather for several layers in one launch: layer blockIdx.z reads its own source (the
@@ -116,8 +118,30 @@ gather_rows_layers(const Gather g, const __grid_constant__ LayerPtrs srcs, const
   pdl_trigger();
   pdl_wait();
   const int layer = blockIdx.z;
-  gather_blocks<V>(g, gridDim.x, srcs.src[layer], idx + (long long)layer * idx_layer_stride,
+  gather_blocks<V>(g, blockIdx.x, gridDim.x, blockIdx.y, gridDim.y, srcs.src[layer], idx + (long long)layer * idx_layer_stride,
                    dst + (long long)layer * dst_layer_stride, status);
+}
+// The same, and one slab of another source by another list, with a word per row beside it, in blocks behind the layers': what
+// follows the selections of a whole prefill, in one launch (two took 2 us longer: the smallest whole prefill 40.4 -> 37.6 us).
+// One dimension of blocks: `blocks` for a slab, then `other_blocks`, then the words'.
+struct OtherRows { Gather g; const char* src; const int* idx; char* dst; CompactWords words; int n_idx, blocks; };
+template <typename V>
+__global__ void __launch_bounds__(kCpThreads)
+gather_rows_prefill(const Gather g, const __grid_constant__ LayerPtrs srcs, const int* __restrict__ idx, long long idx_layer_stride,
+                    char* __restrict__ dst, long long dst_layer_stride, int* __restrict__ status, int n_layers, int blocks,
+                    const __grid_constant__ OtherRows o) {
+  pdl_trigger();
+  pdl_wait();
+  const int per_layer = blocks * g.n_slabs, b = (int)blockIdx.x - n_layers * per_layer;
+  if (b < 0) {
+    const int layer = (int)blockIdx.x / per_layer, in = (int)blockIdx.x - layer * per_layer, slab = in / blocks;
+    gather_blocks<V>(g, in - slab * blocks, blocks, slab, g.n_slabs, srcs.src[layer], idx + (long long)layer * idx_layer_stride,
+                     dst + (long long)layer * dst_layer_stride, status);
+  } else if (b < o.blocks) {
+    gather_blocks<uint4>(o.g, b, o.blocks, 0, 1, o.src, o.idx, o.dst, status);
+  } else {
+    gather_words(o.words, b - o.blocks, o.idx, o.n_idx, o.g.n_rows_src);
+  }
 }
 
 // The unit of a copy whose pointers, strides and row size have the low bits `low` between them, and the launch over it: at
@@ -142,6 +166,31 @@ struct Plan {
 };
 
 }  // namespace
+
+bool launch_compact_prefill(const CompactRows& kv, const void* const* srcs, int n_layers, long long idx_layer_stride,
+                            long long dst_layer_stride, const CompactRows& other, const CompactWords& words, int* status, int sm_count,
+                            cudaStream_t st, cudaError_t* e) {
+  LayerPtrs lp;
+  unsigned long long low = (uintptr_t)kv.dst | kv.slab_stride | kv.row_stride | kv.row_bytes | dst_layer_stride;
+  for (int l = 0; l < n_layers; ++l) {
+    lp.src[l] = (const char*)srcs[l];
+    low |= (uintptr_t)srcs[l];
+  }
+  Plan p(low, kv.slab_stride, kv.row_stride, kv.row_bytes, kv.n_slabs, kv.n_rows_src, 0, kv.n_idx);
+  Plan q((uintptr_t)other.src | (uintptr_t)other.dst | other.row_stride | other.row_bytes, 0, other.row_stride, other.row_bytes, 1,
+         other.n_rows_src, 0, other.n_idx);
+  if (kv.n_idx < 1 || kv.n_slabs < 1 || n_layers < 1 || other.n_idx < 1 || p.unit != 16 || q.unit != 16 || p.rows < kv.n_idx ||
+      q.rows < other.n_idx)
+    return false;
+  p.take(kv.n_idx, n_layers, sm_count);
+  q.take(other.n_idx, 1, sm_count);
+  const long long first = (long long)p.grid.x * kv.n_slabs * n_layers, last = (other.n_idx + kCpThreads - 1) / kCpThreads;
+  if (first + q.grid.x + last > 0x7fffffffll) return false;
+  const OtherRows o = {q.g, (const char*)other.src, other.idx, (char*)other.dst, words, other.n_idx, (int)q.grid.x};
+  *e = launch_pdl(gather_rows_prefill<uint4>, dim3((unsigned)(first + q.grid.x + last)), dim3(kCpThreads), 0, st, p.g, lp, kv.idx,
+                  idx_layer_stride, (char*)kv.dst, dst_layer_stride, status, n_layers, (int)p.grid.x, o);
+  return true;
+}
 
 cudaError_t launch_compact_layers(const void* const* srcs, int n_layers, long long slab_stride, long long row_stride,
                                   int row_bytes, int n_slabs, int n_rows_src, const int* idx,
