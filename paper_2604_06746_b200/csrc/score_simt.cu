@@ -5,10 +5,13 @@
 //
 // Score rows are numbered as in the tensor-core scorer: row (h, i) of KV group g = h / G lives at
 // g * rows_pg_pad + (h % G) * w_pad + i.  A block multiplies 128 rows with 64 keys, 8 x 4 per thread,
-// both operands in shared memory with the head dimension outermost: 32 multiply-adds for three
+// both operands in shared memory with the head dimension outermost: 32 multiply-adds, two an instruction, for three
 // 16-byte loads.  Bound by the FMA pipe on long sequences and by latency on short ones (8 heads,
 // window 32, head dim 64, 2048 keys: a layer took 15 + 21 + 18 us with one dot product per lane, a
-// pass that merged the partials and one key per thread; four layers now take 30 us with their sums).
+// pass that merged the partials and one key per thread; four layers now take 25 us with their sums).
+// Instructions count on both: divisions by the rows a head occupies (a power of two), one multiply-add at a time, 96
+// shuffles and eight logarithms a thread to fold eight rows over 16 threads took 4 layers of 5000 keys 76.8 us, now 69.0;
+// 8 layers of 4096 92.5, now 84.1; 2 of 700 20.7, now 18.2; the whole prefill of 4 layers of 2048 keys 37.6, now 34.0.
 #include <algorithm>
 #include <atomic>
 
@@ -24,7 +27,8 @@ struct SimtArgs {
   const void *q[kSmLayers], *k[kSmLayers];
   float c2[kSmLayers];
   long long sh, st;
-  int N, w, w_pad, group, rows_pg, rows_pg_pad, rows_pad, n_rt, parts, n_keys_tiles;
+  int N, w, w_pad, w_shift, group, rows_pg,   // w_pad = 1 << w_shift: rows a head occupies
+      rows_pg_pad, rows_pad, n_rt, parts, n_keys_tiles;
   float2* part;                            // [layer][parts][rows_pad]
   float* row_ent;                          // [layer][rows_pad]
   float* cols;
@@ -55,9 +59,9 @@ struct SimtShared {
 template <typename T, int D>
 __device__ __forceinline__ void stage_rows(const SimtArgs& a, const T* q, int g, int rt, float (*dst)[kSmRows + 4]) {
   for (int x = threadIdx.x; x < kSmRows * (D / 4); x += kSmThreads) {
-    const int r = x % kSmRows, c = x / kSmRows * 4, row = rt * kSmRows + r, i = row % a.w_pad;
+    const int r = x % kSmRows, c = x / kSmRows * 4, row = rt * kSmRows + r, i = row & (a.w_pad - 1);
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (row < a.rows_pg && i < a.w) v = load4(q + ((size_t)(g * a.group + row / a.w_pad) * a.w + i) * D + c);
+    if (row < a.rows_pg && i < a.w) v = load4(q + ((size_t)(g * a.group + (row >> a.w_shift)) * a.w + i) * D + c);
     dst[c][r] = v.x; dst[c + 1][r] = v.y; dst[c + 2][r] = v.z; dst[c + 3][r] = v.w;
   }
 }
@@ -73,19 +77,24 @@ __device__ __forceinline__ void stage_keys(const SimtArgs& a, const T* k, int j0
 // acc[r][c] = q(row tr * 8 + r) . k(key tc * 4 + c)
 template <int D>
 __device__ __forceinline__ void multiply(const SimtShared<D>& s, int tr, int tc, float (&acc)[8][4]) {
-#pragma unroll
-  for (int r = 0; r < 8; ++r)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-#pragma unroll 8
+  unsigned long long sum[8][2] = {};                       // pairs of keys
+  auto both = [](float v) { unsigned long long x; asm("mov.b64 %0, {%1, %1};" : "=l"(x) : "f"(v)); return x; };
+#pragma unroll 4
   for (int d = 0; d < D; ++d) {
     const float4 q0 = *reinterpret_cast<const float4*>(&s.q[d][tr * 8]), q1 = *reinterpret_cast<const float4*>(&s.q[d][tr * 8 + 4]);
-    const float4 kv = *reinterpret_cast<const float4*>(&s.k[d][tc * 4]);
-    const float qr[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w}, kc[4] = {kv.x, kv.y, kv.z, kv.w};
+    const ulonglong2 kv = *reinterpret_cast<const ulonglong2*>(&s.k[d][tc * 4]);
+    const float qr[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < 8; ++r) {
+      const unsigned long long qq = both(qr[r]);
+      asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(sum[r][0]) : "l"(qq), "l"(kv.x));
+      asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(sum[r][1]) : "l"(qq), "l"(kv.y));
+    }
+  }
 #pragma unroll
-      for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(qr[r], kc[c], acc[r][c]);
+  for (int r = 0; r < 8; ++r) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[r][0]), "=f"(acc[r][1]) : "l"(sum[r][0]));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[r][2]), "=f"(acc[r][3]) : "l"(sum[r][1]));
   }
 }
 
@@ -94,7 +103,7 @@ __device__ __forceinline__ void add_tile(const SimtArgs& a, const float (&acc)[8
   const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    const int t_pos = a.N - a.w + (rt * kSmRows + tr * 8 + r) % a.w_pad;      // the row's position: it sees keys <= t_pos
+    const int t_pos = a.N - a.w + ((rt * kSmRows + tr * 8 + r) & (a.w_pad - 1));      // the row's position: it sees keys <= t_pos
     float x[4], mx = -INFINITY;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
@@ -118,23 +127,36 @@ __device__ __forceinline__ void add_tile(const SimtArgs& a, const float (&acc)[8
       }
   }
 }
+// op over the 16 threads of each of eight rows; thread t of the 16 ends with row t / 2.  Each halving leaves a thread half as
+// many rows (8 shuffles instead of 32), in the order of a butterfly.
+template <typename F>
+__device__ __forceinline__ float over_row(const float (&x)[8], F op) {
+  const bool u8 = threadIdx.x & 8, u4 = threadIdx.x & 4, u2 = threadIdx.x & 2;
+  float y[4], z[2];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) y[i] = op(u8 ? x[i + 4] : x[i], __shfl_xor_sync(0xffffffffu, u8 ? x[i] : x[i + 4], 8));
+#pragma unroll
+  for (int i = 0; i < 2; ++i) z[i] = op(u4 ? y[i + 2] : y[i], __shfl_xor_sync(0xffffffffu, u4 ? y[i] : y[i + 2], 4));
+  const float v = op(u2 ? z[1] : z[0], __shfl_xor_sync(0xffffffffu, u2 ? z[0] : z[1], 2));
+  return op(v, __shfl_xor_sync(0xffffffffu, v, 1));
+}
 // The 16 threads of a row fold into one partial; done(r, partial) in one of them, row r of the thread's eight.
 template <typename F>
 __device__ __forceinline__ void fold_rows(const RowStat (&st)[8], F done) {
+  auto sum = [](float a, float b) { return a + b; };
+  float x[8], u[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) x[r] = st[r].ref;
+  const float M = over_row(x, [](float a, float b) { return fmaxf(a, b); });
 #pragma unroll
   for (int r = 0; r < 8; ++r) {
-    float M = st[r].ref;
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
-    const float dm = st[r].ref == -INFINITY ? 0.f : st[r].ref - M, f = fast_exp2(dm);
-    float Z = f * st[r].Z, U = f * fmaf(dm, st[r].Z, st[r].U);
-#pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
-      Z += __shfl_xor_sync(0xffffffffu, Z, o);
-      U += __shfl_xor_sync(0xffffffffu, U, o);
-    }
-    if ((int)(threadIdx.x & 15) == r) done(r, stat_partial(RowStat{M, Z, U}));
+    const float Mr = __shfl_sync(0xffffffffu, M, (threadIdx.x & 16) | 2 * r);
+    const float dm = st[r].ref == -INFINITY ? 0.f : st[r].ref - Mr, f = fast_exp2(dm);
+    x[r] = f * st[r].Z;
+    u[r] = f * fmaf(dm, st[r].Z, st[r].U);
   }
+  const float Z = over_row(x, sum), U = over_row(u, sum);
+  if ((threadIdx.x & 1) == 0) done((int)(threadIdx.x & 15) >> 1, stat_partial(RowStat{M, Z, U}));
 }
 // Merges the partials [lo, hi) of a row, get(p): in batches of eight.
 template <typename F>
@@ -173,7 +195,7 @@ __device__ __forceinline__ void sum_columns(const SimtArgs& a, SimtShared<D>& s,
   float sum[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const int i = (rt * kSmRows + tr * 8 + q) % a.w_pad, t_pos = a.N - a.w + i;
+    const int i = (rt * kSmRows + tr * 8 + q) & (a.w_pad - 1), t_pos = a.N - a.w + i;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const float pe = fast_exp2(fmaf(acc[q][c], c2, -s.lse[tr * 8 + q]));
@@ -239,7 +261,7 @@ __global__ void __launch_bounds__(kSmThreads) simt_pass2(const __grid_constant__
     const int r = threadIdx.x & (kSmRows - 1), hp = threadIdx.x / kSmRows, row = rt * kSmRows + r;
     const int p_lo = hp * a.parts / 2, p_hi = (hp + 1) * a.parts / 2;
     float M = -INFINITY, W = 0.f, X = 0.f;
-    const bool valid = row < a.rows_pg && row % a.w_pad < a.w;
+    const bool valid = row < a.rows_pg && (row & (a.w_pad - 1)) < a.w;
     if (valid)
       merge_range(p_lo, p_hi, M, W, X, [&](int p) {
         return __ldcg(a.part + ((size_t)layer * a.parts + p) * a.rows_pad + g * a.rows_pg_pad + row);
@@ -275,17 +297,20 @@ __global__ void __launch_bounds__(kSmThreads, 3) simt_once(const __grid_constant
   extern __shared__ __align__(16) unsigned char simt_smem[];
   SimtShared<D>& s = *reinterpret_cast<SimtShared<D>*>(simt_smem);
   __shared__ int last;
+  __shared__ unsigned tag_s;
   pdl_trigger();
   pdl_wait();
+  // (one thread reads it: the line is every block's)
+  if (threadIdx.x == 0) tag_s = (unsigned)__ldcg(a.ctl + kCtlTag) + 1u;
   const int part = blockIdx.x, g = blockIdx.y / a.n_rt, rt = blockIdx.y - g * a.n_rt, layer = blockIdx.z, j0 = part * kSmKeys;
   const int tr = threadIdx.x >> 4, tc = threadIdx.x & 15;
   const float c2 = a.c2[layer];
-  const unsigned tag = (unsigned)__ldcg(a.ctl + kCtlTag) + 1u;
   constexpr size_t kEntWords = kXchPairs;
   unsigned long long* const words = a.xch + (size_t)(blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x * kSmRows;   // of these rows: [part][row]
   stage_rows<T, D>(a, (const T*)a.q[layer], g, rt, s.q);
   stage_keys<T, D>(a, (const T*)a.k[layer] + (size_t)g * a.sh, j0, s.k);
   __syncthreads();
+  const unsigned tag = tag_s;
   float acc[8][4];
   multiply<D>(s, tr, tc, acc);
   {
@@ -305,7 +330,7 @@ __global__ void __launch_bounds__(kSmThreads, 3) simt_once(const __grid_constant
   const int r = threadIdx.x & (kSmRows - 1), hp = threadIdx.x / kSmRows, row = rt * kSmRows + r;
   const int p_lo = hp * a.parts / 2, p_hi = (hp + 1) * a.parts / 2;
   float M = -INFINITY, W = 0.f, X = 0.f;
-  const bool valid = row < a.rows_pg && row % a.w_pad < a.w;
+  const bool valid = row < a.rows_pg && (row & (a.w_pad - 1)) < a.w;
   if (valid) {
     // all of the row's words are there, or the wait's bound expires
     long long t0 = 0;
@@ -396,6 +421,7 @@ cudaError_t launch_score_simt(const Ctx& ctx, const ScoreCall& c, cudaStream_t s
   SimtArgs a = {};
   a.sh = c.k_stride_head; a.st = c.k_stride_token;
   a.N = c.n_keys; a.w = ctx.cfg.window; a.w_pad = ctx.w_pad;
+  while (1 << a.w_shift < a.w_pad) ++a.w_shift;
   a.group = ctx.cfg.n_q_heads / ctx.cfg.n_kv_heads;
   a.rows_pg = a.group * a.w_pad; a.rows_pg_pad = ctx.rows_pad / ctx.cfg.n_kv_heads; a.rows_pad = ctx.rows_pad;
   // row tiles that hold rows, an even number where a head takes two
