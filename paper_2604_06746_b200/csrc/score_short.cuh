@@ -63,6 +63,7 @@ struct ShortSmem {
     int abort, mma_in_flight;
     uint32_t tmem;
     unsigned tag;                      // of this launch's words
+    unsigned ext_seen;                 // second passes whose log-sum-exps are there
     Task ring[2];
     unsigned short own[kMaxSms];       // tasks whose first pass this CTA has drawn
     Work work[kMaxSms];                // what the tasks are
@@ -95,6 +96,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
                         : b >= L::kFold && b < L::kAccFull ? 4 : b >= L::kAccEmpty && b < L::kDrain ? kComputeWarps : 1);
     fl->abort = 0;
     fl->mma_in_flight = 0;
+    fl->ext_seen = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.map_k) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&p.map_q) : "memory");
@@ -306,6 +308,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
             if (i == 0) {
               if (tiles > 1) products(1);
               if (!ok || !(ok = mbar_wait(bar(L::kExtFull), n_ext & 1u, abort_flag))) break;
+              fl->ext_seen = n_ext + 1;
             } else if (i > 1) {
               products(i);
               if (!ok) break;
@@ -356,7 +359,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
     // the tags one further.
     int last = 0;
     if (lane == 0) {
-      if (n_ext > 0) mbar_wait(bar(L::kExtFull), (n_ext - 1u) & 1u, abort_flag);
+      long long t0 = 0;
+      while (fl->ext_seen != n_ext && keep_polling(t0)) {}
       last = atomicAdd(p.ctl + kCtlExit, 1) == (int)gridDim.x - 1;
       if (last) p.ctl[kCtlTicket] = 0;
     }
