@@ -483,6 +483,13 @@ structkv_status structkv_mass_recovery(structkv_ctx* ctx, const float* scores, l
 structkv_status structkv_selftest_wait_expiry(structkv_ctx* ctx, unsigned long long limit_cycles,
                                               void* stream);
 
+/*
+ * Self-test of the scorer of one short layer, whose CTAs draw tasks: with fewer CTAs than tasks, as on a GPU that
+ * other work fills, a CTA runs several.  Bounds the CTAs of the launches to come (0: one per task, as at first).
+ * Results do not depend on it.  Errors: INVALID_ARG.
+ */
+structkv_status structkv_selftest_ctas(structkv_ctx* ctx, int ctas);
+
 /* Reads and clears the device status word (bounded-wait expiry, bad gather index).
  * Synchronises `stream`.  Returns STRUCTKV_OK if nothing was recorded. */
 structkv_status structkv_poll_device_status(structkv_ctx* ctx, void* stream);

@@ -134,6 +134,8 @@ lib.structkv_prefill.restype = _i
 lib.structkv_prefill.argtypes = [_vp, ctypes.POINTER(PrefillArgs), ctypes.POINTER(_i), ctypes.POINTER(_f), _vp]
 lib.structkv_selftest_wait_expiry.restype = _i
 lib.structkv_selftest_wait_expiry.argtypes = [_vp, ctypes.c_ulonglong, _vp]
+lib.structkv_selftest_ctas.restype = _i
+lib.structkv_selftest_ctas.argtypes = [_vp, _i]
 lib.structkv_poll_device_status.restype = _i
 lib.structkv_poll_device_status.argtypes = [_vp, _vp]
 
@@ -415,6 +417,10 @@ class Context:
         """structkv_selftest_wait_expiry: lets one bounded device wait run out (records TIMEOUT)."""
         _check(lib.structkv_selftest_wait_expiry(self._h, limit_cycles, _stream(stream)),
                "structkv_selftest_wait_expiry")
+
+    def selftest_ctas(self, ctas: int) -> None:
+        """structkv_selftest_ctas: bounds the CTAs of the scorer of one short layer (0: one per task)."""
+        _check(lib.structkv_selftest_ctas(self._h, ctas), "structkv_selftest_ctas")
 
     def poll_device_status(self, stream: Optional[torch.cuda.Stream] = None) -> int:
         return lib.structkv_poll_device_status(self._h, _stream(stream))

@@ -672,6 +672,12 @@ structkv_status structkv_selftest_wait_expiry(structkv_ctx* ctx, unsigned long l
              : STRUCTKV_ERR_CUDA;
 }
 
+structkv_status structkv_selftest_ctas(structkv_ctx* ctx, int ctas) {
+  if (!ctx || ctas < 0) return STRUCTKV_ERR_INVALID_ARG;
+  ctx->c.short_ctas = ctas;
+  return STRUCTKV_OK;
+}
+
 structkv_status structkv_poll_device_status(structkv_ctx* ctx, void* stream) {
   if (!ctx) return STRUCTKV_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;

@@ -59,6 +59,7 @@ struct Ctx {
   int w_pad;            // rows a head occupies in a scorer's row blocks: w up to a power of two, at least 8
   int rows_pad;         // rows per KV group (heads at w_pad rows) padded to kRowBlock, times H_kv
   int n_pad;            // max_seq rounded up to kKeyTile
+  int short_ctas = 0;   // CTAs of score_short.cuh's launches, at most; 0: one per task
   bool old_words;       // the exchange words hold anything (a call's own context): who uses them clears them first
   void* tc;             // tensor-core scorer state (tensor-map encoder), owned by score_tc.cu
   struct HostSlot* slot = nullptr;   // where the device leaves the pivot for the host (api.cu), taken at first use

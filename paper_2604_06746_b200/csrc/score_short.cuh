@@ -18,6 +18,8 @@
 // those that it drew, the last one first, whose keys it still holds.  A CTA thus waits for first passes that
 // running CTAs have drawn and that wait for nothing: the waits end whatever the number of resident CTAs.  (A cooperative
 // launch could do without the counter, but would start only when the kernel before it has left every SM.)
+// With halves and an odd number of tiles, the second half of a unit's last segment has no tile in pass 2: that second pass is
+// not posted.  So every posted task has products, before which the MMA warp waits for the task's copies.
 #pragma once
 
 #include "score_tc.cuh"
@@ -126,7 +128,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
     w.hi = 2 * (int)((unsigned)(w.seg + 1) * (unsigned)p.n_pairs / (unsigned)p.n_seg);
     w.half_lo = at & p.split;                              // row halves of pass 1
     w.half_hi = p.split ? w.half_lo + 1 : w.rows > 128 ? 2 : 1;
-    w.t_lo = w.lo + w.half_lo;                             // tiles of pass 2
+    w.t_lo = w.lo + w.half_lo;                             // tiles of pass 2, possibly none
     w.t_hi = min(n_tiles, p.split ? w.t_lo + 1 : w.hi);
     flags->work[task] = w;
   }
@@ -200,9 +202,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
           t.pass = 1;
           t.task = tk;
           flags->own[n_own++] = (unsigned short)tk;
-        } else if (n_own > 0) {
-          t.pass = 2;
-          t.task = flags->own[--n_own];
+        } else {
+          while (t.pass == 0 && n_own > 0) {
+            t.task = flags->own[--n_own];
+            if (flags->work[t.task].t_lo < flags->work[t.task].t_hi) t.pass = 2;
+          }
         }
         t.fresh = t.pass != 0 && t.task != loaded;
         if (!mbar_wait(bar(L::kTaskEmpty + (n & 1)), ((uint32_t)(n >> 1) & 1u) ^ 1u, abort_flag)) break;
@@ -210,7 +214,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
         mbar_arrive(bar(L::kTaskFull + (n & 1)));
         if (t.pass == 0) break;
         if (t.fresh) {
-          // the copies before have landed, and the MMAs of the task before have read what they wanted
+          // The copies before have landed, and the MMAs of the task before have read what they wanted.  (No wait here or in
+          // the MMA warp can be two phases behind, whose parity would let it through: a task's first products wait for its
+          // copies' first pair of tiles, and those copies for the products of the task before and for all copies before.)
           bool ok = n == 0 || mbar_wait(bar(L::kDone), (uint32_t)(n - 1) & 1u, abort_flag);
           for (int b = L::kKFull; b < L::kDone && ok && loads > 0; ++b)
             ok = mbar_wait(bar(b), (loads - 1u) & 1u, abort_flag);
@@ -303,7 +309,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
             fl->mma_in_flight = 1;
             ++u;
           };
-          if (tiles > 0) products(0);
+          products(0);
           for (int i = 0; i < tiles && ok; ++i) {
             if (i == 0) {
               if (tiles > 1) products(1);
@@ -317,7 +323,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
             tc_mma_bf16(tmem + (at & 1) * 256, ones_desc, ext_desc, idesc_ext, 1);
             tc_commit(bar(L::kAccFull + (at & 1)));
           }
-          n_ext += tiles > 0;
+          ++n_ext;
         }
         if (!ok) break;
         tc_commit(bar(L::kDone));
@@ -335,7 +341,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
     for (int n = 0; next_task(n, t); ++n) {
       const typename L::Work w = flags->work[t.task];
       if (t.pass != 2) continue;
-      n_ext += w.t_lo < w.t_hi;
+      ++n_ext;
       if (p.split && w.half_lo != 0) continue;
       const unsigned tag = flags->tag;
       long long t0 = 0;
@@ -468,7 +474,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
       // Pass 2: the unit's log-sum-exps, a thread per row, all partials of a row in one round of loads, merged in the
       // groups of score_tc.cuh.  At first one word alone is polled: with all threads reading all of their words over and over
       // the words themselves were late.
-      if (w.t_lo >= w.t_hi) continue;
       if (ct < R) {
         bool ok = true;
         float nlse = -INFINITY;
@@ -556,7 +561,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) tc_short(const __grid_constant_
 }
 
 template <int D, int SH>
-cudaError_t short_launch(const ShortParams& p, int device, cudaStream_t st) {
+cudaError_t short_launch(const ShortParams& p, int grid, int device, cudaStream_t st) {
   auto kern = tc_short<D, SH>;
   constexpr int kAlloc = ShortSmem<D>::kAlloc;
   static std::atomic<unsigned long long> ready{0};        // devices whose shared-memory limit has been raised
@@ -566,23 +571,23 @@ cudaError_t short_launch(const ShortParams& p, int device, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     ready.fetch_or(bit, std::memory_order_release);
   }
-  return launch_pdl(kern, dim3(p.n_tasks), dim3(kTcThreads), kAlloc, st, p);
+  return launch_pdl(kern, dim3(grid), dim3(kTcThreads), kAlloc, st, p);
 }
 template <int D>
-cudaError_t short_dispatch(int shape, const ShortParams& p, int device, cudaStream_t st) {
+cudaError_t short_dispatch(int shape, const ShortParams& p, int grid, int device, cudaStream_t st) {
   switch (shape) {
-    case kWide16: return short_launch<D, kWide16>(p, device, st);
-    case kWide32: return short_launch<D, kWide32>(p, device, st);
-    case kWide64: return short_launch<D, kWide64>(p, device, st);
-    case kWide128: return short_launch<D, kWide128>(p, device, st);
-    case kWide256: return short_launch<D, kWide256>(p, device, st);
+    case kWide16: return short_launch<D, kWide16>(p, grid, device, st);
+    case kWide32: return short_launch<D, kWide32>(p, grid, device, st);
+    case kWide64: return short_launch<D, kWide64>(p, grid, device, st);
+    case kWide128: return short_launch<D, kWide128>(p, grid, device, st);
+    case kWide256: return short_launch<D, kWide256>(p, grid, device, st);
   }
   return cudaErrorInvalidValue;
 }
 #endif  // __CUDACC__
 
 // One translation unit per head dimension instantiates the kernels.
-cudaError_t short_launch_64(int shape, const ShortParams& p, int device, cudaStream_t st);
-cudaError_t short_launch_128(int shape, const ShortParams& p, int device, cudaStream_t st);
+cudaError_t short_launch_64(int shape, const ShortParams& p, int grid, int device, cudaStream_t st);
+cudaError_t short_launch_128(int shape, const ShortParams& p, int grid, int device, cudaStream_t st);
 
 }  // namespace skv

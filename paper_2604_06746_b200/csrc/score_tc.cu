@@ -129,7 +129,8 @@ bool launch_short(const Ctx& ctx, const ScoreCall& a, int first, cudaStream_t st
   p.group = l.group;
   p.rows_pg = l.rows_pg;
   p.n_rb = l.n_rb;
-  *e = cfg.head_dim == 128 ? short_launch_128(l.shape, p, ctx.device, st) : short_launch_64(l.shape, p, ctx.device, st);
+  const int grid = ctx.short_ctas > 0 ? std::min(ctx.short_ctas, p.n_tasks) : p.n_tasks;
+  *e = cfg.head_dim == 128 ? short_launch_128(l.shape, p, grid, ctx.device, st) : short_launch_64(l.shape, p, grid, ctx.device, st);
   return true;
 }
 

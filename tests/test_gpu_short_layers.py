@@ -62,3 +62,39 @@ def test_bits_of_a_layer_among_others(cuda_device, H, Hkv, d, w, N):
     check()
     del graph
     ctx.close()
+
+
+@pytest.mark.parametrize("H,Hkv,d,w,N", [
+    (32, 8, 128, 64, 64), (32, 8, 128, 64, 300), (32, 8, 128, 64, 1900),     # halves, an odd number of tiles: 1, 3, 15
+    (32, 8, 128, 64, 256), (32, 8, 128, 64, 2304),                           # an even one
+    (32, 8, 128, 64, 2500), (32, 8, 128, 64, 9000),                          # whole segments of one pair and of one or two
+    (16, 1, 64, 16, 777), (12, 4, 128, 33, 4097), (3, 1, 128, 24, 3000),     # other windows and head dimensions
+    (4, 1, 128, 256, 1300), (2, 1, 64, 200, 5003), (16, 2, 64, 128, 300),    # several row blocks
+    (8, 8, 64, 100, 1001),
+])
+def test_several_tasks_a_cta(cuda_device, H, Hkv, d, w, N):
+    """Fewer CTAs than tasks, whatever else runs: the bits of one task a CTA, which are those of a layer among others."""
+    from paper_2604_06746_b200 import binding
+    g = torch.Generator(device=cuda_device)
+    g.manual_seed(N + w)
+    q = torch.randn((2, H, w, d), generator=g, device=cuda_device).bfloat16()
+    k = torch.randn((2, Hkv, N, d), generator=g, device=cuda_device).bfloat16()
+    ctx = binding.Context(H, Hkv, d, w, N, torch.bfloat16, cuda_device)
+
+    def layer(l, ctas):
+        s, m, cols = (torch.zeros(x, device=cuda_device) for x in ((N,), (3,), (H, N)))
+        ctx.selftest_ctas(ctas)
+        ctx.score_layer(q[l], k[l], 1 / math.sqrt(d), s, m, head_cols_out=cols)
+        return s, m, cols
+
+    s, m, cols = (torch.zeros(x, device=cuda_device) for x in ((2, N), (2, 3), (2, H, N)))
+    ctx.score_layers(list(q), list(k), [1 / math.sqrt(d)] * 2, s, m, cols, ctx.layers_workspace(2))
+    whole = [layer(l, 0) for l in range(2)]
+    for l in range(2):
+        assert torch.equal(whole[l][0], s[l]) and torch.equal(whole[l][1][0], m[l, 0]) and torch.equal(whole[l][2], cols[l])
+    for ctas in (1, 2, 3, 5, 11, 0):
+        got = [layer(l, ctas) for l in (0, 1, 0)]            # the words of one launch are there in the next
+        assert ctx.poll_device_status() == binding.OK, ctas
+        for l, r in zip((0, 1, 0), got):
+            assert all(torch.equal(a, b) for a, b in zip(r, whole[l])), ctas
+    ctx.close()
