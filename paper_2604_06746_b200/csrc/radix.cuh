@@ -115,9 +115,9 @@ __device__ __forceinline__ void radix_pick(RadixShared<CL>& s, int level, unsign
   remaining = s.found[level][2];
 }
 
-// Larger float -> larger unsigned; -0 is folded onto +0.
+// Larger float -> larger unsigned; -0 is folded onto +0, and any NaN onto infinity, 0xff800000: a threshold has a key above it.
 __device__ __forceinline__ unsigned order_key(float v) {
-  const unsigned b = __float_as_uint(v + 0.0f);
+  const unsigned b = __float_as_uint(fminf(v + 0.0f, INFINITY));   // (of a number and a NaN, fminf takes the number)
   return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 

@@ -1,0 +1,43 @@
+"""Selection among NaN scores: they come first, as infinity would, ties to the lower index, and nothing is written
+beyond a row of the output, however many of them there are.  Vectors of every form (CTAs, items a thread, slices that do not
+fit the registers)."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import structkv_oracle as O
+
+pytestmark = pytest.mark.gpu
+GUARD, W = 4096, 16
+
+
+def expected(sc, k):
+    return O.select(np.where(np.isnan(sc), np.inf, sc), k, W)
+
+
+@pytest.mark.parametrize("batch,n", [(1, 700), (3, 8000), (2, 16000), (40, 16000), (2, 32768), (20, 32000), (40, 32000), (1, 65000),
+                                     (9, 60000), (1, 131072), (17, 100000), (1, 300000), (17, 150000)])
+@pytest.mark.parametrize("nans", ["all", "one more than kept", "as many as kept", "few"])
+def test_nan_scores_stay_in_their_row(cuda_device, batch, n, nans):
+    from paper_2604_06746_b200 import binding
+    ctx = binding.Context(4, 2, 128, 64, 1024, torch.bfloat16, cuda_device)
+    k = W + n // 11
+    rng = np.random.default_rng(n + batch)
+    sc = rng.random((batch, n), dtype=np.float32)
+    count = {"all": n, "one more than kept": k - W + 1, "as many as kept": k - W, "few": 5}[nans]
+    for row in sc:                                           # bits and signs of all kinds
+        row[rng.permutation(n - W)[:count] if nans != "all" else slice(None)] = np.nan
+    bits = sc.view(np.uint32)
+    bits[np.isnan(sc)] ^= rng.integers(0, 2, np.isnan(sc).sum(), dtype=np.uint32) << np.uint32(31)
+    got = torch.full((GUARD + batch * k + GUARD,), -7, dtype=torch.int32, device=cuda_device)
+    scores, cu = torch.from_numpy(sc).cuda(), [n * b for b in range(batch + 1)]
+    ctx.select(scores, k, W, got[GUARD:-GUARD].view(batch, k))
+    packed = torch.full_like(got, -7)
+    many = min(batch, 32)
+    ctx.select_batch(scores.view(-1)[:many * n], cu[:many + 1], [k] * many, W, packed[GUARD:GUARD + many * k].view(many, k))
+    got, packed = got.cpu().numpy(), packed.cpu().numpy()
+    for out, rows in ((got, batch), (packed, many)):
+        assert (out[:GUARD] == -7).all() and (out[GUARD + rows * k:] == -7).all()
+        for b in range(rows):
+            assert np.array_equal(out[GUARD + b * k:GUARD + (b + 1) * k], expected(sc[b], k)), b
+    ctx.close()
