@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "host_slots.h"
 
 struct structkv_ctx {
   skv::Ctx c;
@@ -63,41 +64,30 @@ Workspace carve_workspace(const structkv_config& cfg, void* base) {
 }
 
 // ---- host words the device writes for the host: one page-locked block per process, a slot per context --
-struct HostSlot {
-  unsigned long long* mem;               // [kSlotWords], mapped
-  unsigned seq;                          // calls so far: tags the answers
-};
 namespace {
-constexpr int kSlots = 64, kSlotWords = 144;
 static_assert(kSlotWords > kMaxStatLayers, "a slot holds the pivot and every T_l");
 std::mutex g_slot_mutex;
 unsigned long long* g_slot_mem = nullptr;
-bool g_slot_used[kSlots];
+HostSlot g_slots[kSlots];
 
 // A slot for the context, or NULL: none left, or no page-locked memory (the caller then copies).
 HostSlot* take_slot() {
   std::lock_guard<std::mutex> lock(g_slot_mutex);
-  if (!g_slot_mem &&
-      cudaHostAlloc((void**)&g_slot_mem, sizeof(*g_slot_mem) * kSlots * kSlotWords, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-    g_slot_mem = nullptr;
-    cudaGetLastError();
-    return nullptr;
-  }
-  for (int i = 0; i < kSlots; ++i)
-    if (!g_slot_used[i]) {
-      HostSlot* s = new (std::nothrow) HostSlot{g_slot_mem + i * kSlotWords, 0};
-      if (!s) return nullptr;
-      g_slot_used[i] = true;
-      std::fill(s->mem, s->mem + kSlotWords, 0ull);
-      return s;
+  if (!g_slot_mem) {
+    constexpr size_t kBytes = sizeof(*g_slot_mem) * kSlots * kSlotWords;
+    if (cudaHostAlloc((void**)&g_slot_mem, kBytes, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+      g_slot_mem = nullptr;
+      cudaGetLastError();
+      return nullptr;
     }
-  return nullptr;
+    std::memset(g_slot_mem, 0, kBytes);
+  }
+  return take_slot(g_slots, g_slot_mem);
 }
 void give_back(HostSlot* s) {
   if (!s) return;
   std::lock_guard<std::mutex> lock(g_slot_mutex);
-  g_slot_used[(s->mem - g_slot_mem) / kSlotWords] = false;
-  delete s;
+  give_back_slot(s);
 }
 }  // namespace
 
@@ -463,7 +453,7 @@ static structkv_status enqueue_pivot_select(Ctx& c, const float* s_hist, long lo
                                             const float* metrics, const float* weights, int l_limit, float lambda, int window,
                                             int kv_budget, int* i_kv, int struct_budget, float* c_star, int* i_struct,
                                             cudaStream_t st) {
-  const unsigned tag = ++c.slot->seq == 0 ? ++c.slot->seq : c.slot->seq;   // never that of clean words
+  const unsigned tag = next_tag(*c.slot);
   if (launch_accumulate_at_pivot(s_hist, row_stride, n_layers, n, lambda, metrics, weights, l_limit, c_star, c.slot->mem,
                                  tag, st) != cudaSuccess)
     return STRUCTKV_ERR_CUDA;
@@ -473,22 +463,11 @@ static structkv_status enqueue_pivot_select(Ctx& c, const float* s_hist, long lo
 }
 // Waits for the words enqueue_pivot_select asked for.
 static structkv_status await_pivot(Ctx& c, int n_layers, int* pivot_out, float* t_out, cudaStream_t st) {
-  const volatile unsigned long long* mem = c.slot->mem;
-  const unsigned tag = c.slot->seq;
-  unsigned spins = 0;
-  for (int i = 0; i <= (t_out ? n_layers : 0); ++i) {
-    unsigned long long word;
-    while ((unsigned)((word = mem[i]) >> 32) != tag) {
-      if (++spins % 100000 != 0) continue;               // tens of microseconds
-      const cudaError_t e = cudaStreamQuery(st);
-      if (e == cudaErrorNotReady) continue;
-      if (e != cudaSuccess || (unsigned)(mem[i] >> 32) != tag) return STRUCTKV_ERR_CUDA;   // done, and no word
-    }
-    const unsigned value = (unsigned)word;
-    if (i == 0) *pivot_out = (int)value;
-    else std::memcpy(&t_out[i - 1], &value, sizeof(float));
-  }
-  return STRUCTKV_OK;
+  const bool ok = await_words(*c.slot, n_layers, pivot_out, t_out, [st]() {
+    const cudaError_t e = cudaStreamQuery(st);
+    return e == cudaErrorNotReady ? 0 : e == cudaSuccess ? 1 : -1;
+  });
+  return ok ? STRUCTKV_OK : STRUCTKV_ERR_CUDA;
 }
 static bool pivot_select_args_ok(const float* s_hist, long long row_stride, int n_layers, int n, const float* metrics,
                                  const float* weights, float lambda, int window, int kv_budget, const int* i_kv,
@@ -589,7 +568,7 @@ structkv_status structkv_prefill(structkv_ctx* ctx, const structkv_prefill_args*
     s = structkv_compact(ctx, p->positions, 0, p->position_row_stride_bytes, p->position_row_bytes, 1, p->n_keys, p->i_struct,
                          p->struct_budget, p->positions_dst, stream);
   if (on_device) {
-    const structkv_status w = await_pivot(ctx->c, p->n_layers, pivot_out, t_out, st);   // also after an error: the word is on its way
+    const structkv_status w = await_pivot(ctx->c, p->n_layers, pivot_out, t_out, st);   // also after an error: the words are on their way
     if (s == STRUCTKV_OK) s = w;
   }
   return s;
