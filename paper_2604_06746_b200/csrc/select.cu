@@ -183,16 +183,22 @@ cudaError_t launch(const SelectArgs& a, cudaStream_t st) {
 }
 
 // One CTA while that is a matter of three barriers a level; beyond, as many CTAs with as few items each as leave all
-// vectors running at once (a CTA has an SM, clusters do not cross a GPC).  us, CTAs x items, for 1 / 8 / 33 vectors, chained launches:
-// 1777 tokens 1 x 4 4.9 / 4.0 / 4.5, 2 x 2 5.4 / 5.5 / 5.5; 8192 1 x 8 5.1 / 5.2 / 6.4, 4 x 2 5.7 / 5.9 / 7.2; 16384 4 x 4
-// 7.8 / 6.4 / 8.0, 1 x 16 8.9 / 7.5 / 9.1, 8 x 2 7.7 / 6.5 / 18.9; 32768 8 x 4 6.6 / 8.5 / 22.2, 4 x 8 7.2 / 9.2 / 9.3, 2 x 16
-// 9.2 / 11.3 / 11.4; 65536 8 x 8 9.6 / 10.0 / 25.6, 4 x 16 11.3 / 11.4 / 11.8; 131072 8 x 16 12.5 / 12.8 / 33.6, 4 x 32
-// 15.9 / 16.1 / 19.8.
+// vectors running at once (a CTA has an SM, clusters do not cross a GPC: 148 SMs run 15 clusters of eight or 33 of four, and the
+// lines are theirs).  us, CTAs x items, for 1 / 8 / 33 vectors, chained launches (of which some take 1.2 to 2 us more
+// than others with the same work): 1777 tokens 1 x 4 4.9 / 4.0 / 4.5, 2 x 2 5.4 / 5.5 / 5.5; 8192 1 x 8 5.1 / 5.2 / 6.4, 4 x 2 5.7 /
+// 5.9 / 7.2; 16384 4 x 4 7.8 / 6.4 / 8.0, 1 x 16 8.9 / 7.5 / 9.1, 8 x 2 7.7 / 6.5 / 18.9; 32768 8 x 4 6.6 / 8.5 / 22.2, 4 x 8
+// 7.2 / 9.2 / 9.3, 2 x 16 9.2 / 11.3 / 11.4; 65536 8 x 8 9.6 / 10.0 / 25.6, 4 x 16 11.3 / 11.4 / 11.8; 131072 8 x 16 12.5 /
+// 12.8 / 33.6, 4 x 32 15.9 / 16.1 / 19.8.  15 / 16 vectors by eight, by four: 32768 tokens 8.8 / 13.5, 9.0 / 9.0; 65536 10.1 /
+// 15.5, 11.4 / 11.4; 131072 12.5 / 19.7, 16.3 / 16.3.
+// Where eight CTAs hold a vector in registers and four would read it again for every digit, two goes of eight are still the
+// faster ones: 200000 tokens, 16 / 30 / 31 vectors 30 / 33 / 44, by four 41; 262144 31 / 34 / 42, by four 43.  Where both
+// read again they are not: 400000 tokens, 15 / 16 / 30 vectors 42 / 75 / 83, by four 75.
 cudaError_t dispatch(const SelectArgs& a, int longest, cudaStream_t st) {
   if (longest <= 4 * kRxThreads) return launch<1, 4>(a, st);
   if (longest <= 8 * kRxThreads) return launch<1, 8>(a, st);
   const int vectors = a.batch + (a.extra.scores ? 1 : 0);
-  const bool by_eight = vectors <= 8, by_four = vectors <= 33;
+  const bool again = longest > 4 * 32 * kRxThreads && longest <= 8 * 32 * kRxThreads;
+  const bool by_eight = vectors <= (again ? 30 : 15), by_four = vectors <= 33;
   if (longest <= 16 * kRxThreads) return by_four ? launch<4, 4>(a, st) : launch<1, 16>(a, st);
   if (longest <= 32 * kRxThreads) return by_eight ? launch<8, 4>(a, st) : by_four ? launch<4, 8>(a, st) : launch<2, 16>(a, st);
   if (longest <= 64 * kRxThreads) return by_eight ? launch<8, 8>(a, st) : launch<4, 16>(a, st);
