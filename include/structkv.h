@@ -304,7 +304,7 @@ structkv_status structkv_accumulate(structkv_ctx* ctx, const float* s_hist, long
  * (I_KV = top-k(S^(l)) union I_win), Algorithm 1 lines 10 and 16.  For each of `batch` score
  * vectors: the (budget - window) highest-scoring tokens of the prefix [0, n - window), ties
  * to the lower index, written in ascending position order, followed by the window positions
- * n-window .. n-1.  A NaN counts as infinity.
+ * n-window .. n-1.  A NaN counts as larger than any number.
  *
  *   scores  device, fp32, vector b starts at scores + b*row_stride (elements).
  *   idx_out device, [batch, budget] int32.

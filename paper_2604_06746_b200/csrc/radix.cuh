@@ -115,10 +115,13 @@ __device__ __forceinline__ void radix_pick(RadixShared<CL>& s, int level, unsign
   remaining = s.found[level][2];
 }
 
-// Larger float -> larger unsigned; -0 is folded onto +0, and any NaN onto infinity, 0xff800000: a threshold has a key above it.
+// Larger float -> larger unsigned, NaN of either sign above all; -0 and +0 are the same.  (The comparison does what an
+// addition of zero, for -0, and a minimum with infinity, for NaN, do in two instructions more: 33 vectors of 200000 tokens
+// 39.7 us, with these 41.6, with the addition alone, which leaves a NaN its sign, 39.6.)
 __device__ __forceinline__ unsigned order_key(float v) {
-  const unsigned b = __float_as_uint(fminf(v + 0.0f, INFINITY));   // (of a number and a NaN, fminf takes the number)
-  return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+  unsigned negative, b = __float_as_uint(v);
+  asm("set.lt.u32.f32 %0, %1, 0f00000000;" : "=r"(negative) : "f"(v));   // all bits or none; none for -0 and NaN
+  return (b ^ negative) | (~negative & 0x80000000u);
 }
 
 }  // namespace skv

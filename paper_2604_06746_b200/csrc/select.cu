@@ -70,8 +70,9 @@ __global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) sel
   };
 
   if (chunks == 1) load(0);
-  // kept: every key >= ge, and the first need_eq of the keys equal to thr
-  unsigned ge = 0, thr = 0, need_eq = 0;
+  // kept: every key > above, and the first need_eq of the keys equal to thr.  (Keys start at 0x007fffff, minus infinity, so that
+  // thr - 1 does not wrap.  They end at 0xffffffff, a NaN: where that is the threshold, nothing is above it.)
+  unsigned above = 0, thr = 0, need_eq = 0;
   if (k < prefix_len) {
     unsigned remaining = (unsigned)k;
     int level = 0;
@@ -89,7 +90,7 @@ __global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) sel
       thr |= digit << radix_shift(level);
       if (in == remaining) break;                    // all keys of the digit are kept: no need to look inside
     }
-    ge = level < kRxLevels ? thr : thr + 1;
+    above = level < kRxLevels ? thr - 1 : thr;
     need_eq = level < kRxLevels ? 0 : remaining;
   }
 
@@ -99,10 +100,10 @@ __global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) sel
   auto tally = [&]() {
     w_gt = w_eq = 0;
 #pragma unroll
-    for (int e = 0; e < ITEMS; ++e) w_gt += __popc(__ballot_sync(0xffffffffu, e < n_mine && key[e] >= ge));
+    for (int e = 0; e < ITEMS; ++e) w_gt += __popc(__ballot_sync(0xffffffffu, e < n_mine && key[e] > above));
     if (need_eq == 0) return;                        // keys that differ: what stays is above
 #pragma unroll
-    for (int e = 0; e < ITEMS; ++e) w_eq += __popc(__ballot_sync(0xffffffffu, e < n_mine && key[e] < ge && key[e] == thr));
+    for (int e = 0; e < ITEMS; ++e) w_eq += __popc(__ballot_sync(0xffffffffu, e < n_mine && key[e] == thr));
   };
   auto leave = [&](unsigned gt, unsigned eq) {
     if (lane == 0) { s.scratch[0][warp] = gt; s.scratch[1][warp] = eq; }
@@ -147,7 +148,7 @@ __global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) sel
     if (need_eq == 0) {
 #pragma unroll
       for (int e = 0; e < ITEMS; ++e) {
-        const bool gt = e < n_mine && key[e] >= ge;
+        const bool gt = e < n_mine && key[e] > above;
         const unsigned bg = __ballot_sync(0xffffffffu, gt);
         if (gt) out[gt_at + __popc(bg & below)] = first + 32 * e;
         gt_at += __popc(bg);
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(kRxThreads, CL == 1 && ITEMS <= 8 ? 2 : 1) sel
     } else {
 #pragma unroll
       for (int e = 0; e < ITEMS; ++e) {
-        const bool in = e < n_mine, gt = in && key[e] >= ge, eq = in && !gt && key[e] == thr;
+        const bool in = e < n_mine, gt = in && key[e] > above, eq = in && key[e] == thr;
         const unsigned bg = __ballot_sync(0xffffffffu, gt), be = __ballot_sync(0xffffffffu, eq);
         const unsigned eq_before = eq_at + __popc(be & below);
         if (gt || (eq && eq_before < need_eq)) out[gt_at + __popc(bg & below) + min(eq_before, need_eq)] = first + 32 * e;

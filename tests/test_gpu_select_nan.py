@@ -1,4 +1,4 @@
-"""Selection among NaN scores: they come first, as infinity would, ties to the lower index, and nothing is written
+"""Selection among NaN scores: they come first, ties to the lower index, and nothing is written
 beyond a row of the output, however many of them there are.  Vectors of every form (CTAs, items a thread, slices that do not
 fit the registers)."""
 import numpy as np
@@ -40,4 +40,24 @@ def test_nan_scores_stay_in_their_row(cuda_device, batch, n, nans):
         assert (out[:GUARD] == -7).all() and (out[GUARD + rows * k:] == -7).all()
         for b in range(rows):
             assert np.array_equal(out[GUARD + b * k:GUARD + (b + 1) * k], expected(sc[b], k)), b
+    ctx.close()
+
+
+@pytest.mark.parametrize("n", [700, 8000, 16000, 32768, 65000, 131072, 300000])
+@pytest.mark.parametrize("more", [1, 40, None])
+def test_the_largest_key_is_the_threshold(cuda_device, n, more):
+    """NaN with all of their bits set: no key lies above them."""
+    from paper_2604_06746_b200 import binding
+    ctx = binding.Context(4, 2, 128, 64, 1024, torch.bfloat16, cuda_device)
+    k, rng = W + n // 13, np.random.default_rng(n)
+    sc = rng.random((2, n), dtype=np.float32)
+    for row in sc.view(np.uint32):
+        at = slice(None) if more is None else rng.permutation(n - W)[:k - W + more]
+        row[at] = rng.integers(0, 2, len(row[at]), dtype=np.uint32) << np.uint32(31) | np.uint32(0x7fffffff)
+    got = torch.full((GUARD + 2 * k + GUARD,), -7, dtype=torch.int32, device=cuda_device)
+    ctx.select(torch.from_numpy(sc).cuda(), k, W, got[GUARD:-GUARD].view(2, k))
+    got = got.cpu().numpy()
+    assert (got[:GUARD] == -7).all() and (got[-GUARD:] == -7).all()
+    for b in range(2):
+        assert np.array_equal(got[GUARD + b * k:GUARD + (b + 1) * k], expected(sc[b], k)), b
     ctx.close()
