@@ -14,7 +14,8 @@ LIB = os.path.join(HERE, "libstructkv.so")
 NATIVE = os.path.join(HERE, "_native.so")
 SOURCES = ["api.cu", "score_simt.cu", "score_tc.cu", "score_tc_d64_one.cu",
            "score_tc_d64_many.cu", "score_tc_d128_one.cu", "score_tc_d128_many.cu", "score_res.cu",
-           "score_res_d64.cu", "score_res_d128.cu", "score_short_d64.cu", "score_short_d128.cu", "score_reduce.cu", "select.cu", "compact.cu", "aggregate.cu"]
+           "score_res_d64.cu", "score_res_d128.cu", "score_short_d64.cu", "score_short_d128.cu", "score_reduce.cu",
+           "select.cu", "compact.cu", "aggregate.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-Xcompiler", "-fno-gnu-unique", "-Wno-deprecated-gpu-targets"]
 

@@ -183,10 +183,10 @@ __device__ __forceinline__ void head_done(const FinishArgs& a, int vec, float me
 // 11.6 / 9.6, of 262144 20.2 / 17.2; 32 layers of 5003 keys 15.6 / 14.4, of 32768 58 / 50, of 131072 215 / 196.
 //
 // Bound by latency up to some 100 vectors, then by the shared-memory atomics and, where the vectors exceed
-// L2 together, by reading them twice (1024 vectors of 131072 keys: 2 x 537 MB, 164 of 208 us).  One histogram,
+// L2 together, by reading them twice (1024 vectors of 131072 keys: 2 x 537 MB, 164 of 196 us).  One histogram,
 // without copies for the lanes: same-address hits cost less than clearing and summing copies, whether the
-// values concentrate or not (1024 vectors of 5003 / 32768 keys: 41 / 85 us with four, 20 / 59 with one,
-// both with three CTAs of 512 an SM).
+// values concentrate or not (1024 vectors of 5003 / 32768 keys, before counts were predicated: 41 / 85 us with four, 20 / 59 with
+// one, both with three CTAs of 512 an SM).
 //
 // Few long vectors are dealt out over clusters of CL CTAs, which count their own entries; the histograms are
 // read through distributed shared memory, and the first CTA adds up.  A CTA takes 0.15 us per 1000 keys, mostly
@@ -204,7 +204,8 @@ struct SweepShared {
   unsigned scan[2][32], bin, rem;                          // [level] sums of the warps, or of 64 bins each
 };
 template <int T, int CL, int ROWS> constexpr int kAccs = ROWS == 1 ? 1024 / T : ROWS * 1024 / (T * CL);
-// Applies f(entry, accumulator, whether there is one) to this CTA's entries of a[0 .. n) once each, 48 or 64 KB of loads in flight on an SM.
+// Applies f(entry, accumulator, whether there is one) to this CTA's entries of a[0 .. n) once each, 48 or 64 KB of loads in
+// flight on an SM.
 template <int T, int CL, int ROWS, class F>
 __device__ __forceinline__ void sweep_from_memory(const float* __restrict__ a, int n, int rank, F f) {
   constexpr int kAt = T == 1024 ? 16 : 8, kStep = ROWS == 1 ? T : T * CL, kMine = kAccs<T, CL, ROWS>;
@@ -435,12 +436,12 @@ __device__ __forceinline__ void sweep_cta(const FinishArgs& a, SweepShared& s, c
 // LONG: some vector has more than kLongFrom keys.  Short ones have a kernel of their own: with both forms in one
 // kernel a launch over 32 vectors of 4096 keys took a microsecond longer.
 // FRONT: all statistics, then all sums: where every vector has an SM, and where there are no sums (a vector that follows
-// from the block's index alone leaves the sweeps the registers for another load: 1024 vectors of 131072 keys 219 us, 234 in the other order).
+// from the block's index alone leaves the sweeps the registers for another load: 1024 vectors of 131072 keys took 219 us, 234 in
+// the other order, before counts were predicated).
 // Else problem after problem, its sums right behind its statistics, so that they find in L2 what these have
-// read, and the last problem first: of the columns the scorer has just written L2 still holds the last ones.  (us after the
-// scorer, in front / so: 32 layers of 32768 keys 93 / 82, 28 of 65536 141 / 126, 32 of 131072 343 / 329.  A
-// batch of four prompts, 128 vectors, lost 2 us a layer by it.  Clusters of four for many long vectors, fewer of them at
-// a time, did not help: 140 and 351.)
+// read, and the last problem first: of the columns the scorer has just written L2 still holds the last ones.  (The lines between
+// the two are at launch_finish.  A batch of four prompts, 128 vectors, lost 2 us a layer by it.  Clusters of four for many
+// long vectors, fewer of them at a time, took 11 to 22 us more than this order for 28 layers of 65536 keys and 32 of 131072.)
 template <int VEC, int T, int CL, bool LONG, bool FRONT>
 __global__ void __launch_bounds__(T, T == 256 ? 6 : T == 512 ? 3 : 1) finish(const __grid_constant__ FinishArgs a) {
   __shared__ union { SweepShared stats; SumShared<VEC> sum; } sh;
@@ -606,11 +607,11 @@ static cudaError_t launch_finish(FinishArgs& a, int longest, int sms, cudaStream
   if (n_vec <= sms)
     return longest > kLongFrom ? launch_pdl(finish<VEC, 1024, 1, true, true>, grid, wide, 0, st, a)
                                : launch_pdl(finish<VEC, 1024, 1, false, true>, grid, wide, 0, st, a);
-  // Sums behind their statistics only where the statistics take several goes of three CTAs an SM.  us after the
-  // scorer, in front / behind, before the sweeps took fewer instructions: 5003 keys, 6 layers of 32 heads 9.5 / 12.5, 14 layers
-  // 17 / 14; 32768 keys, 10 layers 28 / 47, 20 58 / 63, 24 71 / 65; 65536 keys, 14 82 / 86, 20 119 / 111, 24 141 / 128; 131072
-  // keys, 10 109 / 131, 20 220 / 219.  With them, whole prefills: 1500 keys, 14 layers 84.1 / 81.7, 32 layers 146.7 / 144.7;
-  // 5003 keys, 14 layers 142.2 / 141.3, 10 layers of 32768 keys 490 / 525.
+  // Sums behind their statistics only where the statistics take several goes of three CTAs an SM.  Whole prefills, 32 heads, us
+  // in front / behind: 1500 keys, 6 layers 74.6 / 77.6, 14 layers 86.5 / 83.5; 5003 keys, 6 layers 97.6 / 100.5, 10 122.4 /
+  // 124.4, 14 141.4 / 141.0; 20000 keys, 10 layers 333 / 339; 24 of 32768 1315 / 1288; 65536 keys, 14 layers 1492 / 1465, 20 2125 /
+  // 2053, 24 2516 / 2478.  No more apart than the runs of one: 20 and 32 layers of 5003, 14 to 24 of 8193, 20 to 28 of 20000, 20
+  // and 32 of 32768, 20 and 24 of 131072.
   const bool several = n_vec > (longest > kNarrowMany ? 5 : 3) * sms;
   if (!sums || !several)
     return longest > kLongFrom ? launch_pdl(finish<VEC, 512, 1, true, true>, grid, narrow, 0, st, a)
@@ -677,11 +678,12 @@ cudaError_t launch_accumulate_at_pivot(const float* s_hist, long long row_stride
                                        const float* metrics, const float* weights, int l_limit, float* c_out,
                                        unsigned long long* host, unsigned tag, cudaStream_t st) {
   const float3 w = make_float3(weights[0], weights[1], weights[2]);
+  const auto blocks = [](int threads) { return dim3((threads + kPivotThreads - 1) / kPivotThreads + 1); };
   if (n % 4 == 0 && row_stride % 4 == 0 && (uintptr_t)s_hist % 16 == 0 && (uintptr_t)c_out % 16 == 0)
-    return launch_pdl(accumulate_at_pivot<4>, dim3((n / 4 + kPivotThreads - 1) / kPivotThreads + 1), dim3(kPivotThreads), 0, st, s_hist, row_stride, n_layers, n,
-                      lambda, metrics, w, l_limit, c_out, (volatile unsigned long long*)host, tag);
-  return launch_pdl(accumulate_at_pivot<1>, dim3((n + kPivotThreads - 1) / kPivotThreads + 1), dim3(kPivotThreads), 0, st, s_hist, row_stride, n_layers, n, lambda,
-                    metrics, w, l_limit, c_out, (volatile unsigned long long*)host, tag);
+    return launch_pdl(accumulate_at_pivot<4>, blocks(n / 4), dim3(kPivotThreads), 0, st, s_hist, row_stride, n_layers, n, lambda,
+                      metrics, w, l_limit, c_out, (volatile unsigned long long*)host, tag);
+  return launch_pdl(accumulate_at_pivot<1>, blocks(n), dim3(kPivotThreads), 0, st, s_hist, row_stride, n_layers, n, lambda, metrics,
+                    w, l_limit, c_out, (volatile unsigned long long*)host, tag);
 }
 
 }  // namespace skv

@@ -67,8 +67,8 @@ constexpr int kFullWeight = 20;        // weight of a full row block when key ra
 // What the kernel is compiled for.  kHurry: pass 2 has nothing to do but wait for pass 1 (one layer, a batch), so the compute
 // warps count their arrivals and merge the row statistics themselves, a thread per row, instead of leaving it to one helper
 // warp beside them (at 8192 keys 2 us instead of 6).  With layers to interleave the helpers' time is hidden and the compute
-// warps' is not (32 layers of 5003 keys: 317 us in a hurry, 300 without).  With both ways in one kernel 32 layers of 1500
-// keys took 117.7 us instead of 115.5, one layer of 9300 33.9 instead of 33.6.
+// warps' is not (32 layers of 5003 keys, when both were one kernel and a pass slower than now: 317 us in a hurry, 300
+// without).  Then 32 layers of 1500 keys took 117.7 us instead of 115.5, one layer of 9300 33.9 instead of 33.6.
 // kBrief: pass 2's arithmetic in one copy instead of two.  Short tasks alternate with pass 1 and are as long as it takes to fetch
 // them; long ones gain by a second load under way earlier.  us, two copies / one: window 64, 32 layers of 1500 keys 115.5 /
 // 109.6, of 5003 262 / 246, of 8192 387 / 370, 16 of 16384 366 / 356, of 24000 491 / 491, of 32768 657 / 657, 8 of 65536 656 /
