@@ -61,3 +61,25 @@ def test_the_largest_key_is_the_threshold(cuda_device, n, more):
     for b in range(2):
         assert np.array_equal(got[GUARD + b * k:GUARD + (b + 1) * k], expected(sc[b], k)), b
     ctx.close()
+
+
+@pytest.mark.parametrize("H,Hkv,d,w,N,dtype", [(32, 8, 128, 64, 3000, torch.bfloat16), (8, 2, 64, 32, 1500, torch.float32)])
+def test_nan_queries_keep_lists_whole(cuda_device, H, Hkv, d, w, N, dtype):
+    """A whole prefill with a head of them: every list is ascending, within the prompt and ends with the window."""
+    from paper_2604_06746_b200 import binding, pipeline
+    L, budget = 3, N // 10
+    g = torch.Generator(device=cuda_device)
+    g.manual_seed(N)
+    layers = []
+    for _ in range(L):
+        kv = torch.randn((2, Hkv, N, d), generator=g, device=cuda_device).to(dtype)
+        q = torch.randn((H, w, d), generator=g, device=cuda_device).to(dtype)
+        layers.append({"q_win": q, "k": kv[0], "v": kv[1], "kv": kv, "scale": d ** -0.5})
+    layers[1]["q_win"][H // 2] = float("nan")
+    pf = pipeline.Prefill(L, H, Hkv, d, w, N, budget, 2 * budget, dtype, device=cuda_device)
+    pf.run(layers)
+    assert pf.ctx.poll_device_status() == binding.OK and pf.s_hist[1, :N - w].isnan().all() and not pf.s_hist[0].isnan().any()
+    for ids in (*pf.i_kv, pf.i_struct):
+        assert ids[0] >= 0 and (ids.diff() > 0).all() and torch.equal(ids[-w:], torch.arange(N - w, N, device=cuda_device, dtype=ids.dtype))
+    for l in range(L):
+        assert torch.equal(pf.kv_out[l], layers[l]["kv"][:, :, pf.i_kv[l].long()])
